@@ -417,7 +417,7 @@ namespace {
 // gradient buffers and the transposed weights.
 struct BwdLayout {
   size_t HZs, D32, dOp, dYgu, dYg, rowscale, dgate, dU1, ddelta, dBm, dCm, dpre, dxdbl, dU2, dHZs, dHZp, dxp, dlogit;
-  size_t WoT, WiT, WdtT, WxT, ckpt, Xt, Yt, total;
+  size_t WoT, WiT, WdtT, WxT, ckpt, total;
 };
 BwdLayout make_bwd_layout(const rom_config& c, const WsLayout& l) {
   BwdLayout b{};
@@ -442,15 +442,13 @@ BwdLayout make_bwd_layout(const rom_config& c, const WsLayout& l) {
   b.dHZp = take(esz * rows * 2 * De);
   b.dxp = take(esz * rows * Dm);
   b.dlogit = take(4 * T * c.E);
-  b.WoT = take(esz * (size_t)c.E * De * Dm);
-  b.WiT = take(esz * (size_t)c.E * Dm * 2 * De);
-  b.WdtT = take(esz * R * De);
-  b.WxT = take(esz * De * (R + 2 * N));
+  // transposed weights of the data gradients: plain-FMA path only (the tensor path reads the weights as they are)
+  const bool tr = c.dtype != ROM_BF16 || (c.flags & ROM_FLAG_SIMT_GEMM);
+  b.WoT = take(tr ? esz * (size_t)c.E * De * Dm : 0);
+  b.WiT = take(tr ? esz * (size_t)c.E * Dm * 2 * De : 0);
+  b.WdtT = take(tr ? esz * R * De : 0);
+  b.WxT = take(tr ? esz * De * (R + 2 * N) : 0);
   b.ckpt = take(scan_bwd_ws_bytes(c.B, c.d_inner, c.L));
-  // tensor path: the activations of the two grouped weight gradients, transposed (token rows contiguous)
-  const bool tcw = c.dtype == ROM_BF16 && !(c.flags & ROM_FLAG_SIMT_GEMM);
-  b.Xt = take(tcw ? esz * 2 * De * rows : 0);
-  b.Yt = take(tcw ? esz * (De > Dm ? De : Dm) * rows : 0);
   b.total = o;
   return b;
 }
@@ -507,12 +505,27 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
     return launch_gemm_simt(c.dtype, A_, lda, B_, ldb, bstride, M_max, Nn, Kd, te, nmt, ep, st);
   };
   auto store_to = [&](void* C_, int ldc) { return Epilogue{EPI_STORE, C_, ldc, nullptr, nullptr, nullptr, 0, 0, nullptr, nullptr}; };
+  // data gradient C[M, Nn] = A[M, Kd] W[e], W [n_experts, Kd, Nn] as the layer holds it: the tensor path reads it MN-major, the
+  // plain-FMA kernels take a transposed copy
+  auto gemm_dgrad = [&](const void* A_, int lda, const void* Wt, int n_experts, int M_max, int Nn, int Kd, const int32_t* te, const int32_t* nmt,
+                        void* scratch, const Epilogue& ep) -> cudaError_t {
+    if (tc) return launch_gemm_tc(A_, lda, Wt, Nn, n_experts, M_max, Nn, Kd, te, nmt, ep, status, st, false, true);
+    const cudaError_t e = launch_transpose(c.dtype, Wt, scratch, n_experts, Kd, Nn, st);
+    if (e != cudaSuccess) return e;
+    return launch_gemm_simt(c.dtype, A_, lda, scratch, Kd, (int64_t)Nn * Kd, M_max, Nn, Kd, te, nmt, ep, st);
+  };
 
   // ---- forward, recomputed with the raw Gate Proj rows kept (the forward proper stores them activated at top-1)
   ROM_CUDA(cudaMemsetAsync(status, 0, sizeof(int32_t) * kStatusInts, st));
   ROM_CUDA(launch_route_gather(c, x, w->W_r, w->b_r, nullptr, gates, nullptr, W, lay, st));
-  ROM_CUDA(gemm(W + lay.x_perm, Dm, w->W_inz, Dm, c.E, (int64_t)2 * De * Dm, rows, 2 * De, Dm, tile_expert, num_m_tiles, store_to(W + lay.XZp, 2 * De)));
-  ROM_CUDA(launch_slot_sum(c.dtype, W + lay.XZp, row_of_assign, W + bl.HZs, T, 2 * De, c.K, st));       // H_t, Z_t: sums over the selected experts
+  if (tc && c.K == 1) {
+    // one expert per token: the output op writes every row at its token's position (no activation: R = width)
+    Epilogue e_in{EPI_INPROJ, W + bl.HZs, 2 * De, nullptr, nullptr, nullptr, 2 * De, 0, reinterpret_cast<const int32_t*>(W + lay.assign_of_row), nullptr};
+    ROM_CUDA(gemm(W + lay.x_perm, Dm, w->W_inz, Dm, c.E, (int64_t)2 * De * Dm, rows, 2 * De, Dm, tile_expert, num_m_tiles, e_in));
+  } else {
+    ROM_CUDA(gemm(W + lay.x_perm, Dm, w->W_inz, Dm, c.E, (int64_t)2 * De * Dm, rows, 2 * De, Dm, tile_expert, num_m_tiles, store_to(W + lay.XZp, 2 * De)));
+    ROM_CUDA(launch_slot_sum(c.dtype, W + lay.XZp, row_of_assign, W + bl.HZs, T, 2 * De, c.K, st));       // H_t, Z_t: sums over the selected experts
+  }
   rom_config c1 = c;
   c1.K = 1;
   ROM_CUDA(launch_conv(c1, W + bl.HZs, nullptr, w->w_conv, w->b_conv, W + lay.U, nullptr, st));
@@ -523,29 +536,26 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
   float* D32 = reinterpret_cast<float*>(W + bl.D32);
   ROM_CUDA(launch_cast_f32(c.dtype, W + lay.Delta, D32, (long long)T * De, st));
   // gated scan output in expert order (operand of the Out Proj weight gradient); padding rows must be zero
-  ROM_CUDA(cudaMemsetAsync(W + lay.Ygp, 0, esz * (size_t)rows * De, st));
+  ROM_CUDA(launch_zero_padding(c, W + lay.Ygp, De, W, lay, st));
   const char* zraw = W + bl.HZs + (size_t)De * esz;
   ROM_CUDA(launch_scan(c, W + lay.U, W + lay.Delta, false, w->A, Bm, Cm, w->D, zraw, 2 * De, nullptr, nullptr, W + lay.Ygp, nullptr,
                        row_of_assign, c.K, reinterpret_cast<float*>(W + lay.scan_ws), false, st));
 
   // ---- Out Proj and combine, reversed: back_k = dO_t W_out,k; dYg, dgate; dW_out
   ROM_CUDA(launch_gather_rows_to(c, dout, W + bl.dOp, Dm, W, lay, st));
-  ROM_CUDA(launch_transpose(c.dtype, w->W_out, W + bl.WoT, c.E, Dm, De, st));
-  ROM_CUDA(gemm(W + bl.dOp, Dm, W + bl.WoT, Dm, c.E, (int64_t)De * Dm, rows, De, Dm, tile_expert, num_m_tiles, store_to(W + bl.dYgu, De)));
-  float* rowscale = reinterpret_cast<float*>(W + bl.rowscale);
+  ROM_CUDA(gemm_dgrad(W + bl.dOp, Dm, w->W_out, c.E, rows, De, Dm, tile_expert, num_m_tiles, W + bl.WoT, store_to(W + bl.dYgu, De)));
+  // the weight gradient takes gate * Yg: scaled in place on the tensor path, a per-row factor of the plain-FMA kernel otherwise
+  float* rowscale = tc ? nullptr : reinterpret_cast<float*>(W + bl.rowscale);
   float* dgate = reinterpret_cast<float*>(W + bl.dgate);
-  ROM_CUDA(cudaMemsetAsync(rowscale, 0, sizeof(float) * rows, st));
+  if (rowscale) ROM_CUDA(cudaMemsetAsync(rowscale, 0, sizeof(float) * rows, st));
   ROM_CUDA(launch_combine_bwd(c.dtype, W + bl.dYgu, W + lay.Ygp, row_of_assign, gates, W + bl.dYg, dgate, rowscale, T, De, c.K, st));
-  // grouped weight gradient (a sum over each expert's row segment): tensor path = the grouped GEMM over transposed
-  // activations with per-expert K ranges; otherwise the plain fp32-FMA kernel
-  auto grouped_wgrad = [&](const void* X, int P, const void* Y, int Q, const float* scale, float* C) -> cudaError_t {
-    if (!tc) return launch_wgrad(c.dtype, X, P, Y, Q, scale, pad_offsets, c.E, rows, P, Q, C, st);
-    cudaError_t e = launch_transpose_scaled(c.dtype, X, W + bl.Xt, rows, P, rows, scale, st);
-    if (e == cudaSuccess) e = launch_transpose_scaled(c.dtype, Y, W + bl.Yt, rows, Q, rows, nullptr, st);
-    if (e == cudaSuccess) e = launch_gemm_tc_wgrad(W + bl.Xt, W + bl.Yt, rows, pad_offsets, c.E, P, Q, C, status, st);
-    return e;
+  // weight gradients: sums over each expert's row segment (seg) or over all rows
+  auto wgrad = [&](const void* X, int P, const void* Y, int Q, const float* scale, const int32_t* seg, int n_rows, float* C) -> cudaError_t {
+    const int n_seg = seg ? c.E : 1;
+    if (!tc) return launch_wgrad(c.dtype, X, P, Y, Q, scale, seg, n_seg, n_rows, P, Q, C, st);
+    return launch_gemm_tc_wgrad(X, Y, n_rows, seg, n_seg, P, Q, C, status, st);
   };
-  ROM_CUDA(grouped_wgrad(W + bl.dOp, Dm, W + lay.Ygp, De, rowscale, g->dW_out));
+  ROM_CUDA(wgrad(W + bl.dOp, Dm, W + lay.Ygp, De, rowscale, pad_offsets, rows, g->dW_out));
 
   // ---- gate and scan, reversed
   float* ddelta = reinterpret_cast<float*>(W + bl.ddelta);
@@ -557,24 +567,11 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
   // ---- dt Proj and x Proj, reversed
   ROM_CUDA(cudaMemsetAsync(g->db_dt, 0, sizeof(float) * De, st));
   ROM_CUDA(launch_softplus_bwd(c.dtype, ddelta, D32, W + bl.dpre, g->db_dt, T, De, st));
-  ROM_CUDA(launch_transpose(c.dtype, w->W_dt, W + bl.WdtT, 1, De, R, st));
-  ROM_CUDA(gemm(W + bl.dpre, De, W + bl.WdtT, De, 1, 0, T, R, De, nullptr, nullptr, store_to(W + bl.dxdbl, R + 2 * N)));      // d(delta) into columns [0, R)
-  // weight gradient of a shared projection (a sum over all tokens): tensor path = the plain GEMM over transposed
-  // activations (row pitch padded to 64 tokens; the tail of the last K block is filled with zeros by the tensor map)
-  const int Tp = (int)align_up((size_t)T, 64);
-  auto shared_wgrad = [&](const void* X, int P, const void* Y, int Q, float* C) -> cudaError_t {
-    if (!tc) return launch_wgrad(c.dtype, X, P, Y, Q, nullptr, nullptr, 1, T, P, Q, C, st);
-    cudaError_t e = launch_transpose_scaled(c.dtype, X, W + bl.Xt, T, P, Tp, nullptr, st);
-    if (e == cudaSuccess) e = launch_transpose_scaled(c.dtype, Y, W + bl.Yt, T, Q, Tp, nullptr, st);
-    if (e == cudaSuccess) e = launch_gemm_tc(W + bl.Xt, Tp, W + bl.Yt, Tp, 1, P, Q, T, nullptr, nullptr,
-                                             Epilogue{EPI_F32, C, Q, nullptr, nullptr, nullptr, 0, 0, nullptr, nullptr}, status, st);
-    return e;
-  };
-  ROM_CUDA(shared_wgrad(W + bl.dpre, De, W + lay.delta_r, R, g->dW_dt));
+  ROM_CUDA(gemm_dgrad(W + bl.dpre, De, w->W_dt, 1, T, R, De, nullptr, nullptr, W + bl.WdtT, store_to(W + bl.dxdbl, R + 2 * N)));      // d(delta) into columns [0, R)
+  ROM_CUDA(wgrad(W + bl.dpre, De, W + lay.delta_r, R, nullptr, nullptr, T, g->dW_dt));
   ROM_CUDA(launch_pack_bc(c.dtype, dBm, dCm, W + bl.dxdbl, T, R, N, st));
-  ROM_CUDA(launch_transpose(c.dtype, w->W_x, W + bl.WxT, 1, R + 2 * N, De, st));
-  ROM_CUDA(gemm(W + bl.dxdbl, R + 2 * N, W + bl.WxT, R + 2 * N, 1, 0, T, De, R + 2 * N, nullptr, nullptr, store_to(W + bl.dU2, De)));
-  ROM_CUDA(shared_wgrad(W + bl.dxdbl, R + 2 * N, W + lay.U, De, g->dW_x));
+  ROM_CUDA(gemm_dgrad(W + bl.dxdbl, R + 2 * N, w->W_x, 1, T, De, R + 2 * N, nullptr, nullptr, W + bl.WxT, store_to(W + bl.dU2, De)));
+  ROM_CUDA(wgrad(W + bl.dxdbl, R + 2 * N, W + lay.U, De, nullptr, nullptr, T, g->dW_x));
 
   // ---- conv, reversed (dU = scan part + x Proj part)
   ROM_CUDA(cudaMemsetAsync(g->dw_conv, 0, sizeof(float) * (size_t)c.d_conv * De, st));
@@ -583,9 +580,8 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
 
   // ---- Conv Proj | Gate Proj, reversed: every selected expert of a token receives the token's (dH, dZ)
   ROM_CUDA(launch_gather_rows_to(c, W + bl.dHZs, W + bl.dHZp, 2 * De, W, lay, st));
-  ROM_CUDA(launch_transpose(c.dtype, w->W_inz, W + bl.WiT, c.E, 2 * De, Dm, st));
-  ROM_CUDA(gemm(W + bl.dHZp, 2 * De, W + bl.WiT, 2 * De, c.E, (int64_t)Dm * 2 * De, rows, Dm, 2 * De, tile_expert, num_m_tiles, store_to(W + bl.dxp, Dm)));
-  ROM_CUDA(grouped_wgrad(W + bl.dHZp, 2 * De, W + lay.x_perm, Dm, nullptr, g->dW_inz));
+  ROM_CUDA(gemm_dgrad(W + bl.dHZp, 2 * De, w->W_inz, c.E, rows, Dm, 2 * De, tile_expert, num_m_tiles, W + bl.WiT, store_to(W + bl.dxp, Dm)));
+  ROM_CUDA(wgrad(W + bl.dHZp, 2 * De, W + lay.x_perm, Dm, nullptr, pad_offsets, rows, g->dW_inz));
 
   // ---- router, reversed (through the gate values only), and dx
   float* dlogit = reinterpret_cast<float*>(W + bl.dlogit);

@@ -50,23 +50,6 @@ transpose_kernel(const T* __restrict__ in, T* __restrict__ out, int R, int C) {
   }
 }
 
-// out[c][r] = scale[r] * in[r][c] (activations transposed for the tensor-core weight gradient; scale = the row's gate)
-template <typename T>
-__global__ void __launch_bounds__(256)
-transpose_scaled_kernel(const T* __restrict__ in, T* __restrict__ out, int R, int C, int ldo, const float* __restrict__ scale) {
-  __shared__ float tile[32][33];
-  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-  for (int i = threadIdx.y; i < 32; i += 8) {
-    const int r = r0 + i, c = c0 + threadIdx.x;
-    if (r < R && c < C) tile[i][threadIdx.x] = to_f32(in[(size_t)r * C + c]) * (scale ? scale[r] : 1.0f);
-  }
-  __syncthreads();
-  for (int i = threadIdx.y; i < 32; i += 8) {
-    const int c = c0 + i, r = r0 + threadIdx.x;
-    if (r < R && c < C) out[(size_t)c * ldo + r] = from_f32<T>(tile[threadIdx.x][i]);
-  }
-}
-
 // dst[t, :] = sum_k src[row_of_assign[t*K + k], :]  (ascending k, fp32 accumulation), rows `width` wide
 template <typename T>
 __global__ void __launch_bounds__(256)
@@ -97,10 +80,11 @@ cast_f32_kernel(const T* __restrict__ in, float* __restrict__ out, long long n) 
 }
 
 // Reverse of O_t = sum_k gate_k * (Yg_t W_out,k): with back_k = dO_t W_out,k (rows of dYgu, expert order),
-//   dYg_t = sum_k gate_k back_k,  dgate_k = <back_k, Yg_t>;  also the gate of every padded row (scale of the weight gradient).
+//   dYg_t = sum_k gate_k back_k,  dgate_k = <back_k, Yg_t>;  and the operand of the Out Proj weight gradient, gate_k Yg_t: written
+// over the token's rows of Ygp, or (rowscale != nullptr) left as it is with the gate of every padded row in rowscale.
 template <typename T>
 __global__ void __launch_bounds__(128)
-combine_bwd_kernel(const T* __restrict__ dYgu, const T* __restrict__ Ygp, const int32_t* __restrict__ row_of_assign,
+combine_bwd_kernel(const T* __restrict__ dYgu, T* Ygp, const int32_t* __restrict__ row_of_assign,
                    const float* __restrict__ gates, T* __restrict__ dYg, float* __restrict__ dgate, float* __restrict__ rowscale,
                    int De, int K) {
   __shared__ float red[kMaxK][4];
@@ -109,11 +93,11 @@ combine_bwd_kernel(const T* __restrict__ dYgu, const T* __restrict__ Ygp, const 
   for (int k = 0; k < K; ++k) { rows[k] = row_of_assign[t * K + k]; g[k] = gates[t * K + k]; part[k] = 0.0f; }
   const T* yg = Ygp + (size_t)rows[0] * De;          // the K rows of a token hold the same gated scan output
   constexpr int V = V16<T>::N;
-  if (De % V == 0) {                                   // 16-byte accesses
+  {
     for (int i = threadIdx.x; i < De / V; i += blockDim.x) {
       V16<T> q;
       float y[V], acc[V];
-      q.load(yg + (size_t)i * V); q.get(y);
+      ldv(yg + (size_t)i * V, y);
 #pragma unroll
       for (int j = 0; j < V; ++j) acc[j] = 0.0f;
       for (int k = 0; k < K; ++k) {
@@ -123,17 +107,14 @@ combine_bwd_kernel(const T* __restrict__ dYgu, const T* __restrict__ Ygp, const 
         for (int j = 0; j < V; ++j) { acc[j] = fmaf(g[k], bv[j], acc[j]); part[k] = fmaf(bv[j], y[j], part[k]); }
       }
       V16<T>::store(dYg + t * De + (size_t)i * V, acc);
-    }
-  } else {
-    for (int c = threadIdx.x; c < De; c += blockDim.x) {
-      const float y = to_f32(yg[c]);
-      float acc = 0.0f;
-      for (int k = 0; k < K; ++k) {
-        const float b = to_f32(dYgu[(size_t)rows[k] * De + c]);
-        acc = fmaf(g[k], b, acc);
-        part[k] = fmaf(b, y, part[k]);
+      if (!rowscale) {
+        for (int k = 0; k < K; ++k) {
+          float sv[V];
+#pragma unroll
+          for (int j = 0; j < V; ++j) sv[j] = g[k] * y[j];
+          V16<T>::store(Ygp + (size_t)rows[k] * De + (size_t)i * V, sv);
+        }
       }
-      dYg[t * De + c] = from_f32<T>(acc);
     }
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -147,7 +128,7 @@ combine_bwd_kernel(const T* __restrict__ dYgu, const T* __restrict__ Ygp, const 
   if (threadIdx.x < K) {
     const int k = threadIdx.x;
     dgate[t * K + k] = (red[k][0] + red[k][1]) + (red[k][2] + red[k][3]);
-    rowscale[rows[k]] = g[k];
+    if (rowscale) rowscale[rows[k]] = g[k];
   }
 }
 
@@ -406,14 +387,6 @@ cudaError_t launch_transpose(int dtype, const void* in, void* out, int batch, in
   return cudaGetLastError();
 }
 
-cudaError_t launch_transpose_scaled(int dtype, const void* in, void* out, int R, int C, int ldo, const float* scale, cudaStream_t st) {
-  const dim3 grid((C + 31) / 32, (R + 31) / 32), block(32, 8);
-  if (dtype == ROM_BF16) transpose_scaled_kernel<__nv_bfloat16><<<grid, block, 0, st>>>((const __nv_bfloat16*)in, (__nv_bfloat16*)out, R, C, ldo, scale);
-  else transpose_scaled_kernel<float><<<grid, block, 0, st>>>((const float*)in, (float*)out, R, C, ldo, scale);
-  count_launch();
-  return cudaGetLastError();
-}
-
 cudaError_t launch_slot_sum(int dtype, const void* src, const int32_t* row_of_assign, void* dst, long long Tn, int width, int K, cudaStream_t st) {
   const long long total = Tn * (width / (dtype == ROM_BF16 ? 8 : 4));
   const unsigned blocks = (unsigned)((total + 255) / 256);
@@ -431,13 +404,13 @@ cudaError_t launch_cast_f32(int dtype, const void* in, float* out, long long n, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_combine_bwd(int dtype, const void* dYgu, const void* Ygp, const int32_t* row_of_assign, const float* gates, void* dYg,
+cudaError_t launch_combine_bwd(int dtype, const void* dYgu, void* Ygp, const int32_t* row_of_assign, const float* gates, void* dYg,
                                float* dgate, float* rowscale, long long Tn, int De, int K, cudaStream_t st) {
   if (dtype == ROM_BF16)
-    combine_bwd_kernel<__nv_bfloat16><<<(unsigned)Tn, 128, 0, st>>>((const __nv_bfloat16*)dYgu, (const __nv_bfloat16*)Ygp, row_of_assign, gates,
+    combine_bwd_kernel<__nv_bfloat16><<<(unsigned)Tn, 128, 0, st>>>((const __nv_bfloat16*)dYgu, (__nv_bfloat16*)Ygp, row_of_assign, gates,
                                                                   (__nv_bfloat16*)dYg, dgate, rowscale, De, K);
   else
-    combine_bwd_kernel<float><<<(unsigned)Tn, 128, 0, st>>>((const float*)dYgu, (const float*)Ygp, row_of_assign, gates, (float*)dYg, dgate,
+    combine_bwd_kernel<float><<<(unsigned)Tn, 128, 0, st>>>((const float*)dYgu, (float*)Ygp, row_of_assign, gates, (float*)dYg, dgate,
                                                           rowscale, De, K);
   count_launch();
   return cudaGetLastError();

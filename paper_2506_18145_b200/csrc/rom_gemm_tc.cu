@@ -132,7 +132,11 @@ __device__ __forceinline__ void epi_softplus32(const Epilogue& ep, float* sw, in
     for (int r4 = 0; r4 < 8; ++r4) {
       const int R = r4 * 4 + (lane >> 3);
       const float4 v = *reinterpret_cast<const float4*>(sw + R * 32 + ((c ^ (R & 7)) << 2));
-      if (row0 + R < M_valid && n < N) *reinterpret_cast<float4*>(reinterpret_cast<float*>(ep.C) + (size_t)(row0 + R) * ep.ldc + n) = v;
+      if (row0 + R < M_valid && n < N) {
+        float4* dst = reinterpret_cast<float4*>(reinterpret_cast<float*>(ep.C) + (size_t)(row0 + R) * ep.ldc + n);
+        if (ep.accumulate) atomicAdd(dst, v);      // split K: the partial sums of a tile meet in C (zeroed by the launcher)
+        else *dst = v;
+      }
     }
   } else {
     // rounded to bf16: a lane takes 8 columns (two staged float4), 4 lanes one 64-byte row segment, 8 rows per store
@@ -164,7 +168,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
                int M_max, int N, int Kd, int block_n, uint32_t idesc,
                const int32_t* __restrict__ tile_expert, const int32_t* __restrict__ num_m_tiles_dev,
                Epilogue ep, int32_t* __restrict__ status, uint32_t wait_limit, int withhold_kb,
-               const int32_t* __restrict__ k_seg, int n_seg) {
+               const int32_t* __restrict__ k_seg, int n_seg, int a_mn, int b_mn) {
   constexpr int STAGES = stages_of(MODE);
   constexpr int SB = stage_bytes_of(MODE);          // bytes per operand stage (multiple of 1024)
   extern __shared__ unsigned char smem_raw[];
@@ -190,22 +194,30 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   const int n_tiles = MODE == EPI_SWIGLU ? N / 128 : (N + block_n - 1) / block_n;
   // Weight-gradient mode (k_seg != nullptr): n_seg independent problems share A and B; problem s contracts the K range
   // [k_seg[s], k_seg[s+1]) (multiples of BLOCK_K; an expert's padded row segment) and writes rows [s M_max, (s+1) M_max) of C.
+  // Split-K mode (k_seg == nullptr, n_seg > 1): the K range is cut into n_seg equal pieces whose partial sums add up in C.
   const int seg_tiles = num_m_tiles * n_tiles;
-  const int total_tiles = k_seg ? n_seg * seg_tiles : seg_tiles;
+  const int total_tiles = n_seg * seg_tiles;
   const int num_kb = (Kd + BLOCK_K - 1) / BLOCK_K;
+  const int split_kb = (num_kb + n_seg - 1) / n_seg;
   auto decode = [&](int tile, int& m_tile, int& n_tile, int& seg, int& kb0, int& nkb) {
     seg = 0; kb0 = 0; nkb = num_kb;
     int lt = tile;
-    if (k_seg) {
+    if (n_seg > 1 || k_seg) {
       seg = tile / seg_tiles;
       lt = tile - seg * seg_tiles;
-      kb0 = k_seg[seg] / BLOCK_K;
-      nkb = (k_seg[seg + 1] - k_seg[seg]) / BLOCK_K;
+      if (k_seg) {
+        kb0 = k_seg[seg] / BLOCK_K;
+        nkb = (k_seg[seg + 1] - k_seg[seg]) / BLOCK_K;
+      } else {
+        kb0 = seg * split_kb;
+        nkb = min(split_kb, num_kb - kb0);
+      }
     }
     m_tile = lt / n_tiles;
     n_tile = lt - m_tile * n_tiles;
   };
-  const uint32_t stage_tx = A_STAGE_BYTES + (uint32_t)block_n * BLOCK_K * 2;
+  const int b_boxes = b_mn ? (block_n + 63) / 64 : 1;
+  const uint32_t stage_tx = A_STAGE_BYTES + (b_mn ? (uint32_t)b_boxes * MN_BOX_BYTES : (uint32_t)block_n * BLOCK_K * 2);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
@@ -243,8 +255,18 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
           // fault injection (tests only): the copies of K block `withhold_kb` of this CTA's first tile are never issued,
           // so the stage never fills and the waits downstream run out
           if (!(withhold_kb >= 0 && tile == (int)blockIdx.x && kq == withhold_kb)) {
-            tma_load_2d(sa, &tmap_a, full_bar(stage), kb * BLOCK_K, m_tile * BLOCK_M);
-            tma_load_2d(sa + A_STAGE_BYTES, &tmap_b, full_bar(stage), kb * BLOCK_K, b_row);
+            if (a_mn) {
+              tma_load_2d(sa, &tmap_a, full_bar(stage), m_tile * BLOCK_M, kb * BLOCK_K);
+              tma_load_2d(sa + MN_BOX_BYTES, &tmap_a, full_bar(stage), m_tile * BLOCK_M + 64, kb * BLOCK_K);
+            } else {
+              tma_load_2d(sa, &tmap_a, full_bar(stage), kb * BLOCK_K, m_tile * BLOCK_M);
+            }
+            if (b_mn) {      // B is [n_experts * Kd, N]: the expert's rows are its K range
+              for (int i = 0; i < b_boxes; ++i)
+                tma_load_2d(sa + A_STAGE_BYTES + i * MN_BOX_BYTES, &tmap_b, full_bar(stage), n_tile * block_n + 64 * i, e * Kd + kb * BLOCK_K);
+            } else {
+              tma_load_2d(sa + A_STAGE_BYTES, &tmap_b, full_bar(stage), kb * BLOCK_K, b_row);
+            }
             if (MODE == EPI_SWIGLU)     // second half of the B tile: the up rows of the same 128 hidden units (box = 128 rows)
               tma_load_2d(sa + A_STAGE_BYTES + 128 * BLOCK_K * 2, &tmap_b, full_bar(stage), kb * BLOCK_K, b_row + N);
           }
@@ -282,13 +304,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
           if (!mbar_wait(full_bar(stage), phase, abort_flag, wait_limit)) { ok = false; break; }
           tc_fence_after();
           const uint32_t sa = base + stage * SB;
-          const uint64_t adesc = make_smem_desc(sa);
-          const uint64_t bdesc = make_smem_desc(sa + A_STAGE_BYTES);
+          const uint64_t adesc = a_mn ? make_smem_desc_mn(sa) : make_smem_desc(sa);
+          const uint64_t bdesc = b_mn ? make_smem_desc_mn(sa + A_STAGE_BYTES) : make_smem_desc(sa + A_STAGE_BYTES);
+          // K-major: 16 elements = 32 bytes along K inside the swizzled row, +2 in the address field
+          const uint32_t astep = a_mn ? MN_KSTEP : 2u, bstep = b_mn ? MN_KSTEP : 2u;
 #pragma unroll
-          for (int k = 0; k < BLOCK_K / UMMA_K; ++k) {
-            // advance 16 elements = 32 bytes along K inside the swizzled row: +2 in the address field
-            umma_bf16(tmem_d, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc, (kb | k) != 0 ? 1u : 0u);
-          }
+          for (int k = 0; k < BLOCK_K / UMMA_K; ++k)
+            umma_bf16(tmem_d, adesc + (uint64_t)(astep * k), bdesc + (uint64_t)(bstep * k), idesc, (kb | k) != 0 ? 1u : 0u);
           umma_commit(empty_bar(stage));
           issued_any = true;
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
@@ -392,7 +414,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       // weight-gradient mode: problem `seg` owns its own rows of C; an empty K range leaves zeros
       Epilogue epl = ep;
       if (MODE == EPI_F32 && k_seg) epl.C = reinterpret_cast<float*>(ep.C) + (size_t)seg * M_max * ep.ldc;
-      const bool zero_acc = MODE == EPI_F32 && k_seg && nkb == 0;
+      const bool zero_acc = MODE == EPI_F32 && nkb <= 0;
       int ch = (MODE == EPI_SWIGLU || EWQ == 4) ? n_chunks : half;
       if (ch < n_chunks) tmem_ld32_issue(taddr + ch * 32, ra);
       // two register buffers: while one chunk is processed the next chunk's tensor-memory load is in flight
@@ -440,20 +462,29 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
 
 }  // namespace
 
+namespace {
+// instruction descriptor: D = f32, A = B = bf16, operand majorness (1 = MN-major) at bits 15 / 16, N >> 3 at bit 17, M >> 4 at bit 24
+uint32_t make_idesc(int block_n, bool a_mn, bool b_mn) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a_mn << 15) | ((uint32_t)b_mn << 16) | ((uint32_t)(block_n >> 3) << 17) |
+         ((uint32_t)(BLOCK_M >> 4) << 24);
+}
+}  // namespace
+
 cudaError_t launch_gemm_tc(const void* A, int lda, const void* Bw, int ldb, int n_experts, int M_max, int N, int Kd,
                            const int32_t* tile_expert, const int32_t* num_m_tiles_dev, const Epilogue& epi,
-                           int32_t* status, cudaStream_t st, bool test_stall) {
+                           int32_t* status, cudaStream_t st, bool test_stall, bool b_mn) {
   // N tile: a multiple of 32 (epilogue column groups) and of 16 (UMMA N for M = 128), at most 256
   const bool swiglu = epi.mode == EPI_SWIGLU;      // N output columns from 2N rows of B per expert, loaded as two boxes of 128 rows
-  if (swiglu && (N % 128 != 0 || MAX_BLOCK_N != 256)) return cudaErrorInvalidValue;
+  if (swiglu && (N % 128 != 0 || MAX_BLOCK_N != 256 || b_mn)) return cudaErrorInvalidValue;
+  if (b_mn && n_experts > 1 && Kd % BLOCK_K != 0) return cudaErrorInvalidValue;      // a K block must not run into the next expert
   int block_n = (swiglu || N >= MAX_BLOCK_N) ? MAX_BLOCK_N : (N + 31) / 32 * 32;
   if (epi.mode == EPI_XPROJ && block_n > XPROJ_BLOCK_N) block_n = XPROJ_BLOCK_N;
   CUtensorMap ta, tb;
   if (!make_tmap(&ta, A, (uint64_t)M_max, (uint64_t)Kd, (uint64_t)lda, BLOCK_M)) return cudaErrorInvalidValue;
-  if (!make_tmap(&tb, Bw, (uint64_t)n_experts * (swiglu ? 2 * N : N), (uint64_t)Kd, (uint64_t)ldb, swiglu ? 128u : (uint32_t)block_n))
-    return cudaErrorInvalidValue;
-  // instruction descriptor: D = f32, A = B = bf16, both K-major, N >> 3 at bit 17, M >> 4 at bit 24
-  const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(block_n >> 3) << 17) | ((uint32_t)(BLOCK_M >> 4) << 24);
+  const bool ok = b_mn ? make_tmap(&tb, Bw, (uint64_t)n_experts * Kd, (uint64_t)N, (uint64_t)ldb, BLOCK_K)
+                       : make_tmap(&tb, Bw, (uint64_t)n_experts * (swiglu ? 2 * N : N), (uint64_t)Kd, (uint64_t)ldb, swiglu ? 128u : (uint32_t)block_n);
+  if (!ok) return cudaErrorInvalidValue;
+  const uint32_t idesc = make_idesc(block_n, false, b_mn);
   int num_sms = 0;
   cudaError_t e = current_device_sm_count(&num_sms);
   if (e != cudaSuccess) return e;
@@ -469,33 +500,46 @@ cudaError_t launch_gemm_tc(const void* A, int lda, const void* Bw, int ldb, int 
   const long long max_tiles = (long long)((M_max + BLOCK_M - 1) / BLOCK_M) * n_tiles;
   const int grid = (int)(max_tiles < num_sms ? max_tiles : num_sms);
   kern<<<grid, threads_of(epi.mode), smem_bytes, st>>>(ta, tb, M_max, N, Kd, block_n, idesc, tile_expert, num_m_tiles_dev, epi, status,
-                                                            test_stall ? WAIT_LIMIT_TEST : WAIT_LIMIT, test_stall ? 1 : -1, nullptr, 0);
+                                                            test_stall ? WAIT_LIMIT_TEST : WAIT_LIMIT, test_stall ? 1 : -1, nullptr, 1, 0, b_mn ? 1 : 0);
   count_launch();
   return cudaGetLastError();
 }
 
-// Grouped weight gradient on the tensor cores: C[s][P, Q] (fp32) = sum over the rows r in [seg[s], seg[s+1]) of Xt[p, r] Yt[q, r].
-// Xt [P, ld], Yt [Q, ld]: the activations transposed, so the contracted token rows are contiguous; seg: n_seg + 1 device offsets,
-// multiples of 64 (the padded expert segments); rows outside every segment are never read.
-cudaError_t launch_gemm_tc_wgrad(const void* Xt, const void* Yt, int ld, const int32_t* seg, int n_seg, int P, int Q, float* C,
+// Weight gradient on the tensor cores: C[s][P, Q] (fp32) = sum over the rows r of segment s of X[r, p] Y[r, q], X [rows, P] and
+// Y [rows, Q] bf16 as the layer holds them (token rows outermost): both operands are MN-major tiles, nothing is transposed in
+// memory.  seg: n_seg + 1 device offsets, multiples of 64 (the padded expert segments; rows outside are never read).
+// seg == nullptr: one sum over all rows; with too few output tiles to fill the GPU (the shared x Proj / dt Proj: 32 tiles
+// against 16384 rows) the rows are cut into pieces that add into C.
+cudaError_t launch_gemm_tc_wgrad(const void* X, const void* Y, int rows, const int32_t* seg, int n_seg, int P, int Q, float* C,
                                  int32_t* status, cudaStream_t st) {
   const int block_n = Q >= MAX_BLOCK_N ? MAX_BLOCK_N : (Q + 31) / 32 * 32;
   CUtensorMap ta, tb;
-  if (!make_tmap(&ta, Xt, (uint64_t)P, (uint64_t)ld, (uint64_t)ld, BLOCK_M)) return cudaErrorInvalidValue;
-  if (!make_tmap(&tb, Yt, (uint64_t)Q, (uint64_t)ld, (uint64_t)ld, (uint32_t)block_n)) return cudaErrorInvalidValue;
-  const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(block_n >> 3) << 17) | ((uint32_t)(BLOCK_M >> 4) << 24);
+  if (!make_tmap(&ta, X, (uint64_t)rows, (uint64_t)P, (uint64_t)P, BLOCK_K)) return cudaErrorInvalidValue;
+  if (!make_tmap(&tb, Y, (uint64_t)rows, (uint64_t)Q, (uint64_t)Q, BLOCK_K)) return cudaErrorInvalidValue;
   int num_sms = 0;
   cudaError_t e = current_device_sm_count(&num_sms);
   if (e != cudaSuccess) return e;
   const int smem_bytes = smem_bytes_of(EPI_F32);
   e = cudaFuncSetAttribute(gemm_tc_kernel<EPI_F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   if (e != cudaSuccess) return e;
-  const int n_tiles = (Q + block_n - 1) / block_n;
-  const long long max_tiles = (long long)n_seg * ((P + BLOCK_M - 1) / BLOCK_M) * n_tiles;
+  const long long tiles = (long long)((P + BLOCK_M - 1) / BLOCK_M) * ((Q + block_n - 1) / block_n);
+  Epilogue epi{EPI_F32, C, Q, nullptr, nullptr, nullptr, 0, 0, nullptr, nullptr};
+  if (!seg) {
+    // pieces of at least eight K blocks, as many as keep one tile per SM
+    const int num_kb = (rows + BLOCK_K - 1) / BLOCK_K;
+    n_seg = 1;
+    while ((n_seg + 1) * tiles <= num_sms && num_kb / (n_seg + 1) >= 8) ++n_seg;
+    if (n_seg > 1) {
+      const int per = (num_kb + n_seg - 1) / n_seg;
+      n_seg = (num_kb + per - 1) / per;            // no empty piece
+      epi.accumulate = 1;
+      if ((e = cudaMemsetAsync(C, 0, sizeof(float) * (size_t)P * Q, st)) != cudaSuccess) return e;
+    }
+  }
+  const long long max_tiles = (long long)n_seg * tiles;
   const int grid = (int)(max_tiles < num_sms ? max_tiles : num_sms);
-  const Epilogue epi{EPI_F32, C, Q, nullptr, nullptr, nullptr, 0, 0, nullptr, nullptr};
-  gemm_tc_kernel<EPI_F32><<<grid, threads_of(EPI_F32), smem_bytes, st>>>(ta, tb, P, Q, ld, block_n, idesc, nullptr, nullptr, epi, status,
-                                                                        WAIT_LIMIT, -1, seg, n_seg);
+  gemm_tc_kernel<EPI_F32><<<grid, threads_of(EPI_F32), smem_bytes, st>>>(ta, tb, P, Q, rows, block_n, make_idesc(block_n, true, true), nullptr, nullptr, epi,
+                                                                        status, WAIT_LIMIT, -1, seg, n_seg, 1, 1);
   count_launch();
   return cudaGetLastError();
 }

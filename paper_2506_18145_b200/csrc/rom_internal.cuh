@@ -100,6 +100,7 @@ struct Epilogue {
   int R, N;
   const int32_t* row_token;   // EPI_OUTPROJ, EPI_INPROJ: token of each (padded) row, -1 in padding
   const float* row_scale;     // EPI_OUTPROJ: gate of each token
+  int accumulate;             // EPI_F32 (tensor path): add into C instead of storing (split K)
 };
 
 // ---------------------------------------------------------------- launchers (each returns a cudaError_t)
@@ -130,6 +131,8 @@ cudaError_t launch_gather_rows(const rom_config& c, const void* x, char* ws, con
 // dst[row, :] = src[token of row, :] for rows of `width` dtype elements (zero rows in the padding); dst has rows_max rows.
 cudaError_t launch_gather_rows_to(const rom_config& c, const void* src, void* dst, int width, char* ws, const WsLayout& lay,
                                   cudaStream_t st);
+// Zero the padding rows of every expert segment of buf [rows_max, width] (dtype).
+cudaError_t launch_zero_padding(const rom_config& c, void* buf, int width, char* ws, const WsLayout& lay, cudaStream_t st);
 // Per-expert x Proj / dt Proj: sums over the K slots of a token, in ascending slot order (fp32):
 //   Bm[t, :] = sum_k Bp[row(t,k), :],  Cm likewise,  Delta[t, c] = softplus(b_dt[c] + sum_k Dpre[row(t,k), c]).
 cudaError_t launch_small_combine(const rom_config& c, const float* Bp, const float* Cp, const float* Dpre,
@@ -147,16 +150,16 @@ cudaError_t launch_gemm_simt(int dtype, const void* A, int lda, const void* Bw, 
 cudaError_t launch_gemm_skinny(int dtype, const void* A, int lda, const void* Bw, int ldb, int M, int N, int Kd,
                                const Epilogue& epi, cudaStream_t st);
 
+// b_mn: B is [n_experts * Kd, N] with N contiguous (ldb its row pitch), i.e. C = A * B[e] instead of A * B[e]^T (a data gradient
+// on the weights as stored).
 cudaError_t launch_gemm_tc(const void* A, int lda, const void* Bw, int ldb, int n_experts,
                            int M_max, int N, int Kd, const int32_t* tile_expert, const int32_t* num_m_tiles_dev,
-                           const Epilogue& epi, int32_t* status, cudaStream_t st, bool test_stall = false);
+                           const Epilogue& epi, int32_t* status, cudaStream_t st, bool test_stall = false, bool b_mn = false);
 
-// Grouped weight gradient on the tensor cores (bf16): C[s][P, Q] fp32 = sum over rows r of segment s of Xt[p, r] Yt[q, r];
-// Xt [P, ld], Yt [Q, ld] bf16 (activations transposed); seg: n_seg + 1 device row offsets, multiples of 64.
-cudaError_t launch_gemm_tc_wgrad(const void* Xt, const void* Yt, int ld, const int32_t* seg, int n_seg, int P, int Q, float* C,
+// Weight gradient on the tensor cores (bf16): C[s][P, Q] fp32 = sum over rows r of segment s of X[r, p] Y[r, q]; X [rows, P],
+// Y [rows, Q]; seg: n_seg + 1 device row offsets, multiples of 64, or nullptr = one sum over all rows.
+cudaError_t launch_gemm_tc_wgrad(const void* X, const void* Y, int rows, const int32_t* seg, int n_seg, int P, int Q, float* C,
                                  int32_t* status, cudaStream_t st);
-// out[c][r] = scale[r] * in[r][c] for in [R, C] (scale may be nullptr); out has row pitch ldo >= R.
-cudaError_t launch_transpose_scaled(int dtype, const void* in, void* out, int R, int C, int ldo, const float* scale, cudaStream_t st);
 
 // Conv + SiLU, x Proj and dt Proj + softplus as one tcgen05 kernel (bf16, rows of HZ in token order, shared small layers):
 // U, delta_r, Bm, Cm, Delta as the three separate launches leave them.  fused_conv_xdt_supported says whether the sizes fit.
@@ -209,7 +212,7 @@ cudaError_t launch_scan_backward(const rom_config& c, const void* dy, const void
 cudaError_t launch_transpose(int dtype, const void* in, void* out, int batch, int R, int C, cudaStream_t st);      // out[b][c][r] = in[b][r][c]
 cudaError_t launch_slot_sum(int dtype, const void* src, const int32_t* row_of_assign, void* dst, long long Tn, int width, int K, cudaStream_t st);
 cudaError_t launch_cast_f32(int dtype, const void* in, float* out, long long n, cudaStream_t st);
-cudaError_t launch_combine_bwd(int dtype, const void* dYgu, const void* Ygp, const int32_t* row_of_assign, const float* gates, void* dYg,
+cudaError_t launch_combine_bwd(int dtype, const void* dYgu, void* Ygp, const int32_t* row_of_assign, const float* gates, void* dYg,
                                float* dgate, float* rowscale, long long Tn, int De, int K, cudaStream_t st);
 cudaError_t launch_softplus_bwd(int dtype, const float* ddelta, const float* Delta32, void* dpre, float* db_dt, long long Tn, int De, cudaStream_t st);
 cudaError_t launch_pack_bc(int dtype, const float* dBm, const float* dCm, void* dxdbl, long long Tn, int R, int N, cudaStream_t st);

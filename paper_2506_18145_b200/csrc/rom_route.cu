@@ -446,7 +446,23 @@ gather_rows(const uint4* __restrict__ x, uint4* __restrict__ x_perm, const int32
   }
 }
 
+// Padding rows of every expert segment set to zero (sixteen blocks share an expert's at most kTileM - 1 rows).
+__global__ void __launch_bounds__(256)
+zero_padding(uint4* __restrict__ buf, const int32_t* __restrict__ offsets, const int32_t* __restrict__ pad_offsets, int vec_per_row) {
+  const int e = blockIdx.x;
+  const int first = pad_offsets[e] + (offsets[e + 1] - offsets[e]), last = pad_offsets[e + 1];
+  for (int r = first + blockIdx.y; r < last; r += gridDim.y)
+    for (int v = threadIdx.x; v < vec_per_row; v += blockDim.x) buf[(size_t)r * vec_per_row + v] = make_uint4(0, 0, 0, 0);
+}
+
 }  // namespace
+
+cudaError_t launch_zero_padding(const rom_config& c, void* buf, int width, char* ws, const WsLayout& lay, cudaStream_t st) {
+  zero_padding<<<dim3(c.E, 16), 256, 0, st>>>(reinterpret_cast<uint4*>(buf), reinterpret_cast<const int32_t*>(ws + lay.offsets),
+                                             reinterpret_cast<const int32_t*>(ws + lay.pad_offsets), (int)((size_t)width * lay.esz / 16));
+  count_launch();
+  return cudaGetLastError();
+}
 
 cudaError_t launch_route(const rom_config& c, const void* x, const void* W_r, const float* b_r,
                          int32_t* topk_idx, float* gates, int32_t* counts, int32_t* offsets,

@@ -96,6 +96,21 @@ __device__ __forceinline__ uint64_t make_smem_desc(uint32_t saddr) {
   return d;
 }
 
+// The same for an MN-major tile (the M or N index contiguous in memory, so the contracted index walks rows): TMA boxes of
+// 64 MN elements (one 128-byte swizzle row) x 64 K rows, 8 KB each.  8-row groups along K are 1024 bytes apart (stride byte
+// offset), the next 64 MN elements one box further (leading byte offset).  16 K elements = two 8-row groups = 2048 bytes.
+constexpr int MN_BOX_BYTES = 64 * BLOCK_K * 2;
+constexpr uint32_t MN_KSTEP = 2048 >> 4;           // descriptor address units per UMMA_K
+__device__ __forceinline__ uint64_t make_smem_desc_mn(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr & 0x3ffffu) >> 4);
+  d |= (uint64_t)(MN_BOX_BYTES >> 4) << 16;          // leading byte offset
+  d |= (uint64_t)(1024 >> 4) << 32;                  // stride byte offset
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)2 << 61;
+  return d;
+}
+
 // Softplus output op for sixteen epilogue warps: a warp owns two adjacent 32-column chunks of its 32 rows.  Every lane
 // activates and rounds its row of a chunk to bf16 and stages it (swizzled 16-byte pieces, 128 bytes per row for the two
 // chunks); after the second chunk the warp writes whole 128-byte row segments, four rows per store instruction.
