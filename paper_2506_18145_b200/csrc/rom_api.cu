@@ -246,8 +246,8 @@ int rom_scan_backward(const rom_config* cfg, const void* dy, const void* u, cons
   if (ws_bytes < scan_bwd_ws_bytes(cfg->B, cfg->d_inner, cfg->L)) return ROM_ERR_WORKSPACE;
   if ((rc = check_device()) != ROM_OK) return rc;
   LaunchCounter::count = 0;
-  ROM_CUDA(launch_scan_backward(*cfg, dy, u, delta, A, Bm, Cm, D, z, h0, dh_last, du, ddelta, dA, dBm, dCm, dD, dz, dh0,
-                                static_cast<float*>(ws), cfg->d_inner, static_cast<cudaStream_t>(stream)));
+  ROM_CUDA(launch_scan_backward(*cfg, ScanBwd{dy, u, delta, true, A, Bm, Cm, D, z, h0, dh_last, du, ddelta, dA, dBm, dCm, dD, dz, dh0, nullptr, nullptr,
+                                              static_cast<float*>(ws), false, cfg->d_inner}, static_cast<cudaStream_t>(stream)));
   return ROM_OK;
 }
 
@@ -416,7 +416,7 @@ namespace {
 // Scratch of rom_layer_backward: the forward workspace (routing tables and recomputed activations) followed by the
 // gradient buffers and the transposed weights.
 struct BwdLayout {
-  size_t HZs, D32, dOp, dYgu, dYg, rowscale, dgate, dU1, ddelta, dBm, dCm, dpre, dxdbl, dU2, dHZs, dHZp, dxp, dlogit;
+  size_t HZs, dOp, dYgu, dYg, rowscale, dgate, dU1, dBm, dCm, dpre, dxdbl, dU2, dHZs, dHZp, dxp, dlogit;
   size_t WoT, WiT, WdtT, WxT, ckpt, total;
 };
 BwdLayout make_bwd_layout(const rom_config& c, const WsLayout& l) {
@@ -425,14 +425,12 @@ BwdLayout make_bwd_layout(const rom_config& c, const WsLayout& l) {
   auto take = [&](size_t bytes) { size_t at = o; o = align_up(o + bytes, 256); return at; };
   const size_t T = (size_t)l.T, rows = (size_t)l.rows_max, De = c.d_inner, Dm = c.d_model, N = c.d_state, R = c.dt_rank, esz = l.esz;
   b.HZs = take(esz * T * 2 * De);
-  b.D32 = take(4 * T * De);
   b.dOp = take(esz * rows * Dm);
   b.dYgu = take(esz * rows * De);
   b.dYg = take(esz * T * De);
   b.rowscale = take(4 * rows);
   b.dgate = take(4 * T * c.K);
   b.dU1 = take(esz * T * De);
-  b.ddelta = take(4 * T * De);
   b.dBm = take(4 * T * N);
   b.dCm = take(4 * T * N);
   b.dpre = take(esz * T * De);
@@ -533,13 +531,11 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
   ROM_CUDA(gemm(W + lay.U, De, w->W_x, De, 1, 0, T, R + 2 * N, De, nullptr, nullptr, e_x));
   Epilogue e_dt{EPI_SOFTPLUS, W + lay.Delta, De, nullptr, nullptr, w->b_dt, 0, 0, nullptr, nullptr};
   ROM_CUDA(gemm(W + lay.delta_r, R, w->W_dt, R, 1, 0, T, De, R, nullptr, nullptr, e_dt));
-  float* D32 = reinterpret_cast<float*>(W + bl.D32);
-  ROM_CUDA(launch_cast_f32(c.dtype, W + lay.Delta, D32, (long long)T * De, st));
   // gated scan output in expert order (operand of the Out Proj weight gradient); padding rows must be zero
   ROM_CUDA(launch_zero_padding(c, W + lay.Ygp, De, W, lay, st));
   const char* zraw = W + bl.HZs + (size_t)De * esz;
   ROM_CUDA(launch_scan(c, W + lay.U, W + lay.Delta, false, w->A, Bm, Cm, w->D, zraw, 2 * De, nullptr, nullptr, W + lay.Ygp, nullptr,
-                       row_of_assign, c.K, reinterpret_cast<float*>(W + lay.scan_ws), false, st));
+                       row_of_assign, c.K, reinterpret_cast<float*>(W + lay.scan_ws), false, st, false, reinterpret_cast<float*>(W + bl.ckpt)));
 
   // ---- Out Proj and combine, reversed: back_k = dO_t W_out,k; dYg, dgate; dW_out
   ROM_CUDA(launch_gather_rows_to(c, dout, W + bl.dOp, Dm, W, lay, st));
@@ -557,16 +553,14 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
   };
   ROM_CUDA(wgrad(W + bl.dOp, Dm, W + lay.Ygp, De, rowscale, pad_offsets, rows, g->dW_out));
 
-  // ---- gate and scan, reversed
-  float* ddelta = reinterpret_cast<float*>(W + bl.ddelta);
+  // ---- gate, scan and softplus, reversed
   float* dBm = reinterpret_cast<float*>(W + bl.dBm);
   float* dCm = reinterpret_cast<float*>(W + bl.dCm);
-  ROM_CUDA(launch_scan_backward(c, W + bl.dYg, W + lay.U, D32, w->A, Bm, Cm, w->D, zraw, nullptr, nullptr, W + bl.dU1, ddelta, g->dA, dBm, dCm,
-                                g->dD, W + bl.dHZs + (size_t)De * esz, nullptr, reinterpret_cast<float*>(W + bl.ckpt), 2 * De, st));
+  ROM_CUDA(launch_scan_backward(c, ScanBwd{W + bl.dYg, W + lay.U, W + lay.Delta, c.dtype != ROM_BF16, w->A, Bm, Cm, w->D, zraw, nullptr, nullptr, W + bl.dU1,
+                                           nullptr, g->dA, dBm, dCm, g->dD, W + bl.dHZs + (size_t)De * esz, nullptr, W + bl.dpre, g->db_dt,
+                                           reinterpret_cast<float*>(W + bl.ckpt), true, 2 * De}, st));
 
   // ---- dt Proj and x Proj, reversed
-  ROM_CUDA(cudaMemsetAsync(g->db_dt, 0, sizeof(float) * De, st));
-  ROM_CUDA(launch_softplus_bwd(c.dtype, ddelta, D32, W + bl.dpre, g->db_dt, T, De, st));
   ROM_CUDA(gemm_dgrad(W + bl.dpre, De, w->W_dt, 1, T, R, De, nullptr, nullptr, W + bl.WdtT, store_to(W + bl.dxdbl, R + 2 * N)));      // d(delta) into columns [0, R)
   ROM_CUDA(wgrad(W + bl.dpre, De, W + lay.delta_r, R, nullptr, nullptr, T, g->dW_dt));
   ROM_CUDA(launch_pack_bc(c.dtype, dBm, dCm, W + bl.dxdbl, T, R, N, st));

@@ -72,13 +72,6 @@ slot_sum_kernel(const T* __restrict__ src, const int32_t* __restrict__ row_of_as
   stv(dst + t * width + c0, acc);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256)
-cast_f32_kernel(const T* __restrict__ in, float* __restrict__ out, long long n) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) out[i] = to_f32(in[i]);
-}
-
 // Reverse of O_t = sum_k gate_k * (Yg_t W_out,k): with back_k = dO_t W_out,k (rows of dYgu, expert order),
 //   dYg_t = sum_k gate_k back_k,  dgate_k = <back_k, Yg_t>;  and the operand of the Out Proj weight gradient, gate_k Yg_t: written
 // over the token's rows of Ygp, or (rowscale != nullptr) left as it is with the gate of every padded row in rowscale.
@@ -130,23 +123,6 @@ combine_bwd_kernel(const T* __restrict__ dYgu, T* Ygp, const int32_t* __restrict
     dgate[t * K + k] = (red[k][0] + red[k][1]) + (red[k][2] + red[k][3]);
     if (rowscale) rowscale[rows[k]] = g[k];
   }
-}
-
-// Reverse of Delta = softplus(pre): dpre = dDelta * sigmoid(pre) = dDelta * (1 - exp(-Delta)); db_dt[c] = sum_t dpre.
-template <typename T>
-__global__ void __launch_bounds__(256)
-softplus_bwd_kernel(const float* __restrict__ ddelta, const float* __restrict__ Delta32, T* __restrict__ dpre, float* __restrict__ db_dt,
-                    long long Tn, int De) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= De) return;
-  const long long t0 = (long long)blockIdx.y * 64, t1 = min(t0 + 64, Tn);
-  float s = 0.0f;
-  for (long long t = t0; t < t1; ++t) {
-    const float v = ddelta[t * De + c] * (-expm1f(-Delta32[t * De + c]));
-    dpre[t * De + c] = from_f32<T>(v);
-    s += v;
-  }
-  atomicAdd(db_dt + c, s);
 }
 
 // dxdbl[t, R + j] = dB[t, j] (j < N) or dC[t, j - N]: the B | C part of the gradient of (delta, B, C) = U W_x
@@ -396,14 +372,6 @@ cudaError_t launch_slot_sum(int dtype, const void* src, const int32_t* row_of_as
   return cudaGetLastError();
 }
 
-cudaError_t launch_cast_f32(int dtype, const void* in, float* out, long long n, cudaStream_t st) {
-  const unsigned blocks = (unsigned)((n + 255) / 256);
-  if (dtype == ROM_BF16) cast_f32_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>((const __nv_bfloat16*)in, out, n);
-  else cast_f32_kernel<float><<<blocks, 256, 0, st>>>((const float*)in, out, n);
-  count_launch();
-  return cudaGetLastError();
-}
-
 cudaError_t launch_combine_bwd(int dtype, const void* dYgu, void* Ygp, const int32_t* row_of_assign, const float* gates, void* dYg,
                                float* dgate, float* rowscale, long long Tn, int De, int K, cudaStream_t st) {
   if (dtype == ROM_BF16)
@@ -412,14 +380,6 @@ cudaError_t launch_combine_bwd(int dtype, const void* dYgu, void* Ygp, const int
   else
     combine_bwd_kernel<float><<<(unsigned)Tn, 128, 0, st>>>((const float*)dYgu, (float*)Ygp, row_of_assign, gates, (float*)dYg, dgate,
                                                           rowscale, De, K);
-  count_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t launch_softplus_bwd(int dtype, const float* ddelta, const float* Delta32, void* dpre, float* db_dt, long long Tn, int De, cudaStream_t st) {
-  const dim3 grid((De + 255) / 256, (unsigned)((Tn + 63) / 64));
-  if (dtype == ROM_BF16) softplus_bwd_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(ddelta, Delta32, (__nv_bfloat16*)dpre, db_dt, Tn, De);
-  else softplus_bwd_kernel<float><<<grid, 256, 0, st>>>(ddelta, Delta32, (float*)dpre, db_dt, Tn, De);
   count_launch();
   return cudaGetLastError();
 }

@@ -13,6 +13,7 @@ constexpr int kTileM = 128;        // expert segments are padded to this many ro
 constexpr int kChunkTokens = 32;   // tokens per routing chunk (one warp)
 constexpr int kMaxE = 64;
 constexpr int kMaxK = 8;
+constexpr int kScanCkpt = 8;         // steps between the state checkpoints of the scan's backward pass
 constexpr int kStatusInts = 64;    // status block at the head of the workspace
 
 // status word slots
@@ -187,7 +188,8 @@ cudaError_t launch_conv_step(const rom_config& c, const void* XZp, const int32_t
 cudaError_t launch_scan(const rom_config& c, const void* u, const void* delta, bool delta_fp32, const float* A, const float* Bm,
                         const float* Cm, const float* D, const void* z, int ldz, const int32_t* z_row, const float* h0,
                         void* y, float* h_last, const int32_t* y_rows, int K, float* chunk_ws, bool gate_activated, cudaStream_t st,
-                        bool scalar_A = false /* A[c, :] constant per channel and disc_mode 1: one exponential per channel and step */);
+                        bool scalar_A = false /* A[c, :] constant per channel and disc_mode 1: one exponential per channel and step */,
+                        float* ckpt = nullptr /* also store the state at the start of every kScanCkpt steps, [B, ceil(L / kScanCkpt), De, 16] */);
 
 // One-pass scan for few long sequences (rom_scan_seq.cu): every exponential evaluated once, no workspace.  bf16 storage only.
 bool scan_seq_applicable(const rom_config& c, const void* u, const void* delta, bool delta_fp32, const float* Bm, const float* Cm,
@@ -200,21 +202,26 @@ cudaError_t launch_scan_seq(const rom_config& c, const void* u, const void* delt
 cudaError_t launch_scan_states(const rom_config& c, const void* u, const float* delta, const float* A, const float* Bm, int Lc, int ncc,
                                const float* h_in, float* h_end, float* sum_delta, float* ckpt, int nck, cudaStream_t st);
 
-// Backward of the scan (gradients of every input); ckpt: scan_bwd_ws_bytes() bytes of scratch.  dA, dBm, dCm, dD are
+// Backward of the scan (gradients of every input); ckpt: scan_bwd_ws_bytes() bytes of scratch.  dA, dBm, dCm, dD, db_dt are
 // zeroed here and accumulated with atomics.  z / dz, h0, dh_last, dD, dh0 may be null.
+struct ScanBwd {
+  const void* dy; const void* u; const void* delta; bool delta_fp32; const float* A; const float* Bm; const float* Cm; const float* D;
+  const void* z; const float* h0; const float* dh_last;
+  void* du; float* ddelta; float* dA; float* dBm; float* dCm; float* dD; void* dz; float* dh0;
+  void* dpre; float* db_dt;      // both or neither: Delta = softplus(pre); d(pre) leaves in the storage type and its sum over tokens
+                                 // in db_dt, instead of ddelta
+  float* ckpt; bool ckpt_ready;  // ckpt_ready: the head of ckpt already holds launch_scan's checkpoints
+  int ldz;                       // row pitch of z and dz
+};
+size_t scan_bwd_ckpt_floats(int B, int De, int L);
 size_t scan_bwd_ws_bytes(int B, int De, int L);
-cudaError_t launch_scan_backward(const rom_config& c, const void* dy, const void* u, const float* delta, const float* A,
-                                 const float* Bm, const float* Cm, const float* D, const void* z, const float* h0,
-                                 const float* dh_last, void* du, float* ddelta, float* dA, float* dBm, float* dCm, float* dD,
-                                 void* dz, float* dh0, float* ckpt, int ldz /* row pitch of z and dz */, cudaStream_t st);
+cudaError_t launch_scan_backward(const rom_config& c, const ScanBwd& s, cudaStream_t st);
 
 // Pieces of the layer's backward pass (rom_backward.cu); dtype tensors per the config, sums in fp32.
 cudaError_t launch_transpose(int dtype, const void* in, void* out, int batch, int R, int C, cudaStream_t st);      // out[b][c][r] = in[b][r][c]
 cudaError_t launch_slot_sum(int dtype, const void* src, const int32_t* row_of_assign, void* dst, long long Tn, int width, int K, cudaStream_t st);
-cudaError_t launch_cast_f32(int dtype, const void* in, float* out, long long n, cudaStream_t st);
 cudaError_t launch_combine_bwd(int dtype, const void* dYgu, void* Ygp, const int32_t* row_of_assign, const float* gates, void* dYg,
                                float* dgate, float* rowscale, long long Tn, int De, int K, cudaStream_t st);
-cudaError_t launch_softplus_bwd(int dtype, const float* ddelta, const float* Delta32, void* dpre, float* db_dt, long long Tn, int De, cudaStream_t st);
 cudaError_t launch_pack_bc(int dtype, const float* dBm, const float* dCm, void* dxdbl, long long Tn, int R, int N, cudaStream_t st);
 cudaError_t launch_conv_bwd(const rom_config& c, const void* HZ, const void* w_conv, const float* b_conv, const void* dU1, const void* dU2,
                             void* dHZ, float* dw, float* db, cudaStream_t st);

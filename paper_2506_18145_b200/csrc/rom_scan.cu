@@ -125,7 +125,7 @@ struct ScanArgs {
   float* sum_delta;     // state-only blocks: [B*nch, De] sum of Delta over the chunk
   int gate_activated;   // z already holds SiLU(gate pre-activation): multiply only
   int chunk_off;        // chunk of blockIdx.z == 0
-  float* ckpt;          // MODE 3: [B, nck, De, 16] state at the start of every 16 steps (nck per sequence)
+  float* ckpt;          // MODE 3..5: [B, nck, De, 16] state at the start of every kScanCkpt steps (nck per sequence)
   int nck;
   int scalar_a;         // A[c, :] is one value per channel (scalar-per-head decay of a Mamba2-style block): one exponential
                         // per channel and step instead of one per state (only with B-bar = Delta B)
@@ -136,7 +136,8 @@ struct ScanArgs {
 // state update (bf16 configurations, 2e-2 tolerance).
 // ZOH: zero-order-hold B-bar (disc_mode 0); otherwise B-bar = Delta B.
 // MODE 0: full scan.  MODE 1: state only (no outputs, only h_last and sum_delta of every chunk).  MODE 3: state only
-// from the given chunk-start states, storing the state at the start of every 16 steps (backward pass).  MODE 2: first
+// from the given chunk-start states, storing the state at the start of every kScanCkpt steps (backward pass).  MODE 4 and 5:
+// MODE 0 and 2 with those stores beside the outputs (the layer backward's recomputed forward).  MODE 2: first
 // launch of the chunked scan: chunk 0 runs the full scan from the caller's initial state (h0 indexed by
 // sequence), the other chunks run state-only from a zero state.
 template <typename T, typename TD, int NC, int NS, bool PRECISE, bool ZOH, int MODE>
@@ -156,7 +157,8 @@ scan_kernel(const ScanArgs p) {
   const int De = p.De, K = p.K;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int chunk = blockIdx.z + p.chunk_off;
-  const bool so = MODE == 1 || MODE == 3 || (MODE == 2 && chunk != 0);  // this block only produces states
+  constexpr bool FIRST = MODE == 2 || MODE == 5;
+  const bool so = MODE == 1 || MODE == 3 || (FIRST && chunk != 0);  // this block only produces states
   const T* __restrict__ z = so ? nullptr : static_cast<const T*>(p.z);
   const int t_first = chunk == 0 ? 0 : p.L0 + (chunk - 1) * p.Lc;
   const int L = min(chunk == 0 ? p.L0 : p.Lc, p.L - t_first);   // steps of this chunk (<= 0: an empty chunk)
@@ -178,8 +180,8 @@ scan_kernel(const ScanArgs p) {
       const float a0 = p.A[(size_t)c * NST + n], a1 = p.A[(size_t)c * NST + n + 1];
       a2[i][q] = PRECISE ? make_float2(a0, a1) : make_float2(a0 * kLog2e, a1 * kLog2e);
       kin[i][q] = make_float2(-1.0f / a0, -1.0f / a1);
-      const size_t hb = MODE == 2 ? (size_t)blockIdx.y : (size_t)b;
-      h[i][q] = (p.h0 && !(MODE == 2 && so)) ? make_float2(p.h0[(hb * De + c) * NST + n], p.h0[(hb * De + c) * NST + n + 1])
+      const size_t hb = FIRST ? (size_t)blockIdx.y : (size_t)b;
+      h[i][q] = (p.h0 && !(FIRST && so)) ? make_float2(p.h0[(hb * De + c) * NST + n], p.h0[(hb * De + c) * NST + n + 1])
                                              : make_float2(0.0f, 0.0f);
     }
   }
@@ -274,16 +276,6 @@ scan_kernel(const ScanArgs p) {
   for (int t0 = 0; t0 < L; t0 += TS, buf ^= 1) {
     const bool more = t0 + TS < L;
     if (more) fetch(t0 + TS);
-    if constexpr (MODE == 3) {
-      static_assert(MODE != 3 || (TS == 16 && NC == 1), "one checkpoint per tile");
-      const int c = c_base + cl;
-      if (c < De) {
-        float* dst = p.ckpt + (((size_t)blockIdx.y * p.nck + (size_t)((t_first + t0) >> 4)) * De + c) * NST + g * NS;
-#pragma unroll
-        for (int q = 0; q < NP; q += 2)
-          *reinterpret_cast<float4*>(dst + 2 * q) = make_float4(h[0][q].x, h[0][q].y, h[0][q + 1].x, h[0][q + 1].y);
-      }
-    }
     const TileT& tl = tiles[buf];
     float* ys = ysum + buf * TS * YP;
 
@@ -294,14 +286,28 @@ scan_kernel(const ScanArgs p) {
     const float4* __restrict__ bcp = &tl.bc[0][g * NP];
     float* __restrict__ ysp = ys + cl;
     float* __restrict__ psp = ps;
-    constexpr int UF = S > 4 ? S : (NC * NS >= 16 ? 2 : 4);
+    constexpr int UF = S > 4 ? S : (MODE >= 3 ? kScanCkpt : (NC * NS >= 16 ? 2 : 4));
     float held = 0.0f;      // the even step's partial sum, kept for the paired exchange (S == 2)
     float pend_keep = 0.0f, pend_recv = 0.0f;   // the exchange of the previous pair, finished one pair later (S == 2)
     auto tile_steps = [&](auto so_tag, auto sc_tag) {
     constexpr bool STATE_ONLY = decltype(so_tag)::value;
     constexpr bool SCALAR_A = decltype(sc_tag)::value && !ZOH;
+    constexpr bool CKPT = MODE == 3 || MODE == 4 || (MODE == 5 && !STATE_ONLY);
+    static_assert(MODE < 3 || (NC == 1 && TS % kScanCkpt == 0), "checkpoints fall on tile steps");
 #pragma unroll UF
     for (int tt = 0; tt < TS; ++tt) {
+      if constexpr (CKPT) {
+        if (tt % kScanCkpt == 0 && t0 + tt < L && c_base + cl < De) {
+          float* dst = p.ckpt + (((size_t)blockIdx.y * p.nck + (size_t)((t_first + t0 + tt) / kScanCkpt)) * De + c_base + cl) * NST + g * NS;
+          if constexpr (NP == 1) {
+            *reinterpret_cast<float2*>(dst) = h[0][0];
+          } else {
+#pragma unroll
+            for (int q = 0; q < NP; q += 2)
+              *reinterpret_cast<float4*>(dst + 2 * q) = make_float4(h[0][q].x, h[0][q].y, h[0][(q + 1) % NP].x, h[0][(q + 1) % NP].y);
+          }
+        }
+      }
       float4 bc[NP];
 #pragma unroll
       for (int q = 0; q < NP; ++q) bc[q] = bcp[tt * (NST / 2) + q];
@@ -403,10 +409,10 @@ scan_kernel(const ScanArgs p) {
     if (MODE == 1 || MODE == 3) {
       tile_steps(std::true_type{}, std::false_type{});
     } else if (p.scalar_a) {
-      if (MODE == 2 && so) tile_steps(std::true_type{}, std::true_type{});
+      if (FIRST && so) tile_steps(std::true_type{}, std::true_type{});
       else tile_steps(std::false_type{}, std::true_type{});
     } else {
-      if (MODE == 2 && so) tile_steps(std::true_type{}, std::false_type{});
+      if (FIRST && so) tile_steps(std::true_type{}, std::false_type{});
       else tile_steps(std::false_type{}, std::false_type{});
     }
 
@@ -541,21 +547,23 @@ int pick_thread_shape(int B, int De, int num_sms) {
   return 102;
 }
 
-template <typename T, typename TD, bool PRECISE, bool ZOH>
+template <typename T, typename TD, bool PRECISE, bool ZOH, int MODE>
 cudaError_t launch_shape(int shape, const ScanArgs& a, int B, cudaStream_t st) {
   switch (shape) {
-    case 108: return launch_one<T, TD, 1, 8, PRECISE, ZOH, 0>(a, B, a.nch, st);
-    case 104: return launch_one<T, TD, 1, 4, PRECISE, ZOH, 0>(a, B, a.nch, st);
-    case 102: return launch_one<T, TD, 1, 2, PRECISE, ZOH, 0>(a, B, a.nch, st);
+    case 108: return launch_one<T, TD, 1, 8, PRECISE, ZOH, MODE>(a, B, a.nch, st);
+    case 104: return launch_one<T, TD, 1, 4, PRECISE, ZOH, MODE>(a, B, a.nch, st);
+    case 102: return launch_one<T, TD, 1, 2, PRECISE, ZOH, MODE>(a, B, a.nch, st);
     default: return cudaErrorInvalidValue;
   }
 }
 
-template <typename T, typename TD, bool PRECISE>
+// CKPT: also store the checkpoints of the backward pass (MODE 4 / 5 instead of 0 / 2).
+template <typename T, typename TD, bool PRECISE, bool CKPT = false>
 cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const float* h0, float* h_last,
                           float* chunk_ws, int num_sms, cudaStream_t st) {
+  constexpr int FULL = CKPT ? 4 : 0, FIRST = CKPT ? 5 : 2;
   const bool zoh = c.disc_mode == 0;
-  if (c.L == 1) {
+  if (!CKPT && c.L == 1) {
     a.h0 = h0; a.h_last = h_last;
     dim3 grid((c.d_inner + BLOCK - 1) / BLOCK, c.B);
     if (zoh) scan_step_kernel<T, TD, PRECISE, true><<<grid, BLOCK, 0, st>>>(a);
@@ -567,7 +575,7 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
   if (nch == 1) {
     a.Lc = c.L; a.L0 = c.L; a.nch = 1;
     const int shape = pick_thread_shape(c.B, c.d_inner, num_sms);
-    return zoh ? launch_shape<T, TD, PRECISE, true>(shape, a, c.B, st) : launch_shape<T, TD, PRECISE, false>(shape, a, c.B, st);
+    return zoh ? launch_shape<T, TD, PRECISE, true, FULL>(shape, a, c.B, st) : launch_shape<T, TD, PRECISE, false, FULL>(shape, a, c.B, st);
   }
   // chunked, two launches, 8 states per thread.  Launch A: chunk 0 in full from the caller's state, chunks
   // 1..n_end-1 state-only from zero; chain; launch B: chunks 1..nch-1 in full from their true initial states.
@@ -584,7 +592,7 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
   const int n_end = h_last ? nch : nch - 1;       // the last chunk's end state is only needed for h_last
   ScanArgs pa = a;
   pa.h_last = h_end; pa.sum_delta = sum_delta; pa.chunk_off = 0;
-  cudaError_t e = zoh ? launch_one<T, TD, 1, 8, PRECISE, true, 2>(pa, c.B, n_end, st) : launch_one<T, TD, 1, 8, PRECISE, false, 2>(pa, c.B, n_end, st);
+  cudaError_t e = zoh ? launch_one<T, TD, 1, 8, PRECISE, true, FIRST>(pa, c.B, n_end, st) : launch_one<T, TD, 1, 8, PRECISE, false, FIRST>(pa, c.B, n_end, st);
   if (e != cudaSuccess) return e;
   const long long n_thr = (long long)c.B * c.d_inner * NST;
   chain_chunk_states<<<(unsigned)((n_thr + 255) / 256), 256, 0, st>>>(A, h_end, sum_delta, h_in, h_last, c.B, c.d_inner, nch, n_end);
@@ -592,7 +600,7 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   a.h0 = h_in; a.h_last = nullptr; a.chunk_off = 1;
-  return zoh ? launch_one<T, TD, 1, 8, PRECISE, true, 0>(a, c.B, nch - 1, st) : launch_one<T, TD, 1, 8, PRECISE, false, 0>(a, c.B, nch - 1, st);
+  return zoh ? launch_one<T, TD, 1, 8, PRECISE, true, FULL>(a, c.B, nch - 1, st) : launch_one<T, TD, 1, 8, PRECISE, false, FULL>(a, c.B, nch - 1, st);
 }
 
 }  // namespace
@@ -600,16 +608,21 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
 cudaError_t launch_scan(const rom_config& c, const void* u, const void* delta, bool delta_fp32, const float* A, const float* Bm,
                         const float* Cm, const float* D, const void* z, int ldz, const int32_t* z_row, const float* h0,
                         void* y, float* h_last, const int32_t* y_rows, int K, float* chunk_ws, bool gate_activated, cudaStream_t st,
-                        bool scalar_A) {
+                        bool scalar_A, float* ckpt) {
   int num_sms = 0;
   const cudaError_t e = current_device_sm_count(&num_sms);
   if (e != cudaSuccess) return e;
   // Few long sequences and no workspace for the chunked scan: the one-pass low-occupancy kernel (every exponential once;
   // 0.74 ms against 1.04 ms for one 16384-step sequence of 4096 channels).  With a workspace the two chunked launches
   // below are faster (0.67 ms), so they stay the path of the layer.
-  if (chunk_ws == nullptr && !scalar_A && scan_seq_applicable(c, u, delta, delta_fp32, Bm, Cm, z, ldz, z_row, y_rows, gate_activated, num_sms))
+  if (chunk_ws == nullptr && !scalar_A && ckpt == nullptr && scan_seq_applicable(c, u, delta, delta_fp32, Bm, Cm, z, ldz, z_row, y_rows, gate_activated, num_sms))
     return launch_scan_seq(c, u, delta, delta_fp32, A, Bm, Cm, D, z, ldz, h0, y, h_last, y_rows, K, gate_activated, st);
-  const ScanArgs a{u, delta, A, Bm, Cm, D, z, ldz, z_row, h0, y, h_last, y_rows, K, c.L, c.d_inner, c.L, 1, c.L, nullptr, gate_activated ? 1 : 0, 0, nullptr, 0, (scalar_A && c.disc_mode == 1) ? 1 : 0};
+  const ScanArgs a{u, delta, A, Bm, Cm, D, z, ldz, z_row, h0, y, h_last, y_rows, K, c.L, c.d_inner, c.L, 1, c.L, nullptr, gate_activated ? 1 : 0, 0,
+                   ckpt, (c.L + kScanCkpt - 1) / kScanCkpt, (scalar_A && c.disc_mode == 1) ? 1 : 0};
+  if (ckpt != nullptr) {      // the layer backward's recomputed forward: Delta in the storage type
+    if (c.dtype != ROM_BF16) return launch_scan_t<float, float, true, true>(c, a, A, h0, h_last, chunk_ws, num_sms, st);
+    return delta_fp32 ? cudaErrorInvalidValue : launch_scan_t<__nv_bfloat16, __nv_bfloat16, false, true>(c, a, A, h0, h_last, chunk_ws, num_sms, st);
+  }
   if (c.dtype != ROM_BF16) return launch_scan_t<float, float, true>(c, a, A, h0, h_last, chunk_ws, num_sms, st);
   return delta_fp32 ? launch_scan_t<__nv_bfloat16, float, false>(c, a, A, h0, h_last, chunk_ws, num_sms, st)
                     : launch_scan_t<__nv_bfloat16, __nv_bfloat16, false>(c, a, A, h0, h_last, chunk_ws, num_sms, st);
@@ -618,7 +631,7 @@ cudaError_t launch_scan(const rom_config& c, const void* u, const void* delta, b
 // State recurrence alone over uniform chunks of Lc steps (Lc a multiple of 16; ncc chunks per sequence), for the backward pass.
 // ckpt == nullptr: every chunk from a zero state; h_end [B, ncc, De, 16] and sum_delta [B, ncc, De] leave.
 // ckpt != nullptr: every chunk from its true start state h_in [B, ncc, De, 16] (null: zero); the state at the start of every
-// 16 steps is stored to ckpt [B, nck, De, 16].
+// kScanCkpt steps is stored to ckpt [B, nck, De, 16].
 cudaError_t launch_scan_states(const rom_config& c, const void* u, const float* delta, const float* A, const float* Bm, int Lc, int ncc,
                                const float* h_in, float* h_end, float* sum_delta, float* ckpt, int nck, cudaStream_t st) {
   ScanArgs a{u, delta, A, Bm, /* C is fetched with B but not used */ Bm, nullptr, nullptr, 0, nullptr, h_in, nullptr, h_end, nullptr, 1, c.L, c.d_inner, Lc, ncc, Lc, sum_delta,

@@ -4,19 +4,24 @@
 //           a = exp(Delta A);  b = expm1(Delta A)/A * B (zero-order hold)  or  Delta B.
 // Reverse, with g = dLoss/dh_t carried from later steps and e_t = dout_t * SiLU(z_t):
 //           g += C_t e_t;  dC_t = sum_c e_t h_t;  dA-bar = g h_{t-1};  db = g u_t;  du_t = sum_n g b + D e_t;  g <- a_t g.
+// With w = -u B / A the zero-order-hold step is h_t = a (h_{t-1} - w) + w, and everything that passes through the exponent is
+// g p with p = a (h_{t-1} - w):  dDelta = sum_n A g p,  dA = Delta g p + r w  with  r = g (a - 1) / A,  dB = r u,  du = sum_n r B.
 //
-// The reverse sweep needs h_{t-1} and h_t at every step.  First the forward scan kernel runs the recurrence in its
-// state-only mode and keeps the state at the start of every chunk of 16 steps (checkpoints in the workspace).  The second kernel walks the chunks
-// backwards: it recomputes the chunk's states from its checkpoint into shared memory, then sweeps the chunk in
-// reverse.  A thread owns 4 of the 16 states of one channel of one sequence (4 adjacent lanes per channel): sums over
-// the states (dDelta, du, the forward y for the gate's derivative) are shuffles over those lanes; sums over channels
-// (dB, dC) are shuffles over the 8 channels of a warp, shared-memory atomics over the block and one global atomic per
-// (step, state) and block; dA and dD accumulate in registers over the sequence and leave with one atomic per thread.
-// A long sequence with few channels is cut into coarse chunks that run in parallel, as in the forward scan: both
-// recurrences are linear, the states' forward in time and the state gradients' backward in time.  A pre-pass runs, per
-// coarse chunk, the state recurrence from a zero state (end state, sum of Delta) and the gradient recurrence from a
-// zero gradient (the gradient leaving the chunk's start); a chain kernel composes them into the true state at the start
-// and the true gradient at the end of every coarse chunk; the two kernels above then run once per coarse chunk.
+// The reverse sweep needs h_{t-1} and h_t at every step.  The state at the start of every CK = 8 steps is kept in the workspace
+// (checkpoints, written by a forward scan: the layer's recomputed forward, or the state-only passes of rom_scan_backward); the
+// reverse kernel walks the checkpoints backwards, recomputes eight states into shared memory and sweeps them in reverse.
+//
+// A long sequence with few channels is cut into coarse chunks that run in parallel, as in the forward scan: the gradient
+// recurrence is linear in g.  A pre-pass runs it per chunk from a zero gradient (the gradient that leaves the chunk's start, and
+// the sum of Delta), a chain kernel composes the true gradient at the end of every chunk.
+//
+// What bounds the reverse kernel: the fp32 pipe.  Per state and step it needs about 23 fp32 lane operations (6 recomputed
+// forward, 17 reverse) and two exponentials, so the layout is chosen to add as little as possible: a thread owns 4 states of 4
+// adjacent channels (packed pairs along the states), so that the sums over channels (dB, dC) start as accumulation in
+// registers and the sums over states (dDelta, du, y) need four lanes only; the former finish with a transposed 7-shuffle
+// reduction per step, the latter are left in the shared-memory slot of the state just consumed and added by the lane that owns
+// the output.  A warp owns 32 channels and everything it touches: no block barrier.  Shared memory (81 KB per block of four
+// warps) allows two blocks per SM, and the 16 independent updates per thread and step hide the latencies.
 // All arithmetic is fp32; the fp32 configuration uses the accurate exp / expm1, the bf16 one a single ex2.approx per state
 // and step (exp(x) - 1 by subtraction: with Delta A down to -5e-4 that is still good to a few 1e-4 relative).
 #include "rom_internal.cuh"
@@ -25,177 +30,245 @@ namespace rom {
 namespace {
 
 constexpr int NST = 16;
-constexpr int CK = 16;            // steps per chunk (16: four blocks fit an SM's shared memory)
-constexpr int BCH = 32;           // channels per block
-constexpr int BT = BCH * 4;       // threads per block
-constexpr size_t BWD_SMEM = sizeof(float4) * CK * BT + sizeof(float) * CK * (8 * BCH + 4 * NST);
+constexpr int CK = kScanCkpt;     // steps per checkpoint
+constexpr int WCH = 32;           // channels per warp
+constexpr int WPB = 4;            // warps per block
+constexpr int BT = WPB * 32;
+constexpr int BCH = WPB * WCH;    // channels per block
+constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
+
+struct WarpSmem {
+  float4 h[CK][4][32];            // [step][channel of the thread][lane]: state before the step; later the step's partial sums
+  float4 dl[CK][8], u[CK][8], e[CK][8];     // Delta, u, e of 4 channels; group g of step r sits at g ^ r
+  float4 bc[2][CK][4];            // B, C
+};
+constexpr int BWD_SMEM = WPB * (int)sizeof(WarpSmem);
+constexpr int BLOCKS_PER_SM = 2;
 
 struct BwdArgs {
-  const void* dy; const void* u; const float* delta; const float* A; const float* Bm; const float* Cm; const float* D;
-  const void* z; const float* h0; const float* dh_last;
+  const void* dy; const void* u; const void* delta; const float* A; const float* Bm; const float* Cm; const float* D;
+  const void* z; const float* dh_last;
   void* du; float* ddelta; float* dA; float* dBm; float* dCm; float* dD; void* dz; float* dh0;
-  float* ckpt;        // [B, nck, De, 16]
+  void* dpre; float* db_dt;       // dpre != nullptr: the gradient goes through Delta = softplus(pre) and leaves as dpre (ddelta unused)
+  const float* ckpt;              // [B, nck, De, 16]
   int L, De, nck;
-  int ldz;            // row pitch (elements) of z and dz
-  // coarse chunks (blockIdx.z): chunk j covers steps [j Lc, (j+1) Lc); Lc is a multiple of CK.  ncc == 1: the whole sequence.
-  int Lc, ncc;
-  const float* h_in;  // [B, ncc, De, 16] state at the start of every coarse chunk (ncc > 1)
-  const float* g_in;  // [B, ncc, De, 16] state gradient at the end of every coarse chunk (ncc > 1)
-  float* h_end; float* q_start; float* sum_delta;     // pre-pass outputs: [B, ncc, De, 16] x 2 and [B, ncc, De]
+  int ldz;                        // row pitch (elements) of z and dz
+  int Lc, ncc;                    // coarse chunks (blockIdx.z): chunk j covers steps [j Lc, (j+1) Lc); Lc is a multiple of 16
+  float* g_in;                    // [B, ncc, De, 16] state gradient at the end of every coarse chunk (ncc > 1)
+  float* q_start; float* sum_delta;         // pre-pass outputs: [B, ncc, De, 16] and [B, ncc, De]
 };
 
-__device__ __forceinline__ float sigmoid_f(float v) { return 1.0f / (1.0f + expf(-v)); }
-
-// exp(x) and exp(x) - 1
-template <bool PRECISE>
-__device__ __forceinline__ void exp_and_expm1(float x, float& ex, float& em1) {
-  if (PRECISE) { ex = expf(x); em1 = expm1f(x); }
-  else { ex = ex2_ftz(1.4426950408889634f * x); em1 = ex - 1.0f; }
+// 8 consecutive elements of a row, as loaded
+template <typename T> struct Raw8;
+template <> struct Raw8<__nv_bfloat16> {
+  V16<__nv_bfloat16> q;
+  __device__ __forceinline__ void load(const __nv_bfloat16* p) { q.load(p); }
+  __device__ __forceinline__ void zero() { q.zero(); }
+  __device__ __forceinline__ void get(float (&v)[8]) const { q.get(v); }
+};
+template <> struct Raw8<float> {
+  float4 a, b;
+  __device__ __forceinline__ void load(const float* p) { a = __ldg(reinterpret_cast<const float4*>(p)); b = __ldg(reinterpret_cast<const float4*>(p) + 1); }
+  __device__ __forceinline__ void zero() { a = make_float4(0.0f, 0.0f, 0.0f, 0.0f); b = a; }
+  __device__ __forceinline__ void get(float (&v)[8]) const { v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w; }
+};
+__device__ __forceinline__ void store8(__nv_bfloat16* p, const float (&v)[8]) { V16<__nv_bfloat16>::store(p, v); }
+__device__ __forceinline__ void store8(float* p, const float (&v)[8]) {
+  reinterpret_cast<float4*>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
+  reinterpret_cast<float4*>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
 }
-template <bool PRECISE>
-__device__ __forceinline__ float exp_only(float x) { return PRECISE ? expf(x) : ex2_ftz(1.4426950408889634f * x); }
 
-template <typename T, bool ZOH>
-__global__ void __launch_bounds__(BT)
+template <bool PRECISE> __device__ __forceinline__ float sigmoid_f(float v) {
+  return PRECISE ? 1.0f / (1.0f + expf(-v)) : rcp_ftz(1.0f + ex2_ftz(-kLog2e * v));
+}
+// 1 - exp(-x), x >= 0 (the derivative of softplus expressed in its result)
+template <bool PRECISE> __device__ __forceinline__ float one_minus_exp(float x) {
+  if (PRECISE) return -expm1f(-x);
+  // series below 1/4 (next term x^5/720, 1.4e-6 relative), subtraction above
+  const float s = x * fmaf(x, -fmaf(x, -fmaf(x, -fmaf(x, -1.0f / 120.0f, 1.0f / 24.0f), 1.0f / 6.0f), 0.5f), 1.0f);
+  return x < 0.25f ? s : 1.0f - ex2_ftz(-kLog2e * x);
+}
+__device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 neg2(float2 v) { return make_float2(-v.x, -v.y); }
+// exp(Delta A) of a pair of states, and exp - 1; a2 holds A log2(e) (A itself when PRECISE)
+template <bool PRECISE> __device__ __forceinline__ float2 exp_pair(float2 x) {
+  return PRECISE ? make_float2(expf(x.x), expf(x.y)) : make_float2(ex2_ftz(x.x), ex2_ftz(x.y));
+}
+
+template <typename T, typename TD, bool ZOH>
+__global__ void __launch_bounds__(BT, BLOCKS_PER_SM)
 scan_bwd_kernel(const BwdArgs p) {
+  constexpr bool PRECISE = sizeof(T) == 4;
   extern __shared__ __align__(16) unsigned char bwd_smem[];
-  float4 (*hbuf)[BT] = reinterpret_cast<float4 (*)[BT]>(bwd_smem);                    // states after each step of the chunk (this thread's 4)
-  float (*s_dl)[BCH] = reinterpret_cast<float (*)[BCH]>(bwd_smem + sizeof(float4) * CK * BT);
-  float (*s_u)[BCH] = s_dl + CK;
-  float (*s_e)[BCH] = s_u + CK;
-  float (*s_z)[BCH] = s_e + CK;
-  float (*s_dy)[BCH] = s_z + CK;
-  float (*s_dd)[BCH] = s_dy + CK;
-  float (*s_du)[BCH] = s_dd + CK;
-  float (*s_y)[BCH] = s_du + CK;
-  float (*s_B)[NST] = reinterpret_cast<float (*)[NST]>(s_y + CK);
-  float (*s_C)[NST] = s_B + CK;
-  float (*s_dB)[NST] = s_C + CK;
-  float (*s_dC)[NST] = s_dB + CK;
-
-  const int tid = threadIdx.x, cl = tid >> 2, q = tid & 3, lane = tid & 31;
-  const int c_base = blockIdx.x * BCH;
-  const int c = c_base + cl;
-  const bool c_ok = c < p.De;
-  const int cc = c_ok ? c : p.De - 1;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  WarpSmem& s = reinterpret_cast<WarpSmem*>(bwd_smem)[warp];
+  const int De = p.De, L = p.L;
+  const int c_warp = blockIdx.x * BCH + warp * WCH;
+  if (c_warp >= De) return;                      // d_inner is a multiple of 64: a warp's 32 channels are all in or all out
   const size_t b = blockIdx.y;
-  const T* __restrict__ u = static_cast<const T*>(p.u);
-  const T* __restrict__ dy = static_cast<const T*>(p.dy);
-  const T* __restrict__ z = static_cast<const T*>(p.z);
-  T* __restrict__ du = static_cast<T*>(p.du);
-  T* __restrict__ dz = static_cast<T*>(p.dz);
-
   const int cj = blockIdx.z;
   const int k_lo = cj * (p.Lc / CK), k_hi = min(k_lo + p.Lc / CK, p.nck);
-  float a[4], g[4], dAacc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+
+  // ---- compute role: channels c0 .. c0+3, states 4q .. 4q+3
+  const int q = lane & 3, cg = lane >> 2;
+  const int c0 = c_warp + 4 * cg;
+  float2 a2[4][2], ik[4][2], g[4][2], dA[4][2];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    a[i] = p.A[(size_t)cc * NST + 4 * q + i];
-    if (p.ncc > 1) g[i] = p.g_in[((b * p.ncc + cj) * p.De + cc) * NST + 4 * q + i];
-    else g[i] = p.dh_last ? p.dh_last[(b * p.De + cc) * NST + 4 * q + i] : 0.0f;
+    const float4 av = *reinterpret_cast<const float4*>(p.A + (size_t)(c0 + i) * NST + 4 * q);
+    const float sc = PRECISE ? 1.0f : kLog2e;
+    a2[i][0] = make_float2(av.x * sc, av.y * sc); a2[i][1] = make_float2(av.z * sc, av.w * sc);
+    ik[i][0] = make_float2(1.0f / av.x, 1.0f / av.y); ik[i][1] = make_float2(1.0f / av.z, 1.0f / av.w);
+    float4 gv = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (p.ncc > 1) gv = *reinterpret_cast<const float4*>(p.g_in + ((b * p.ncc + cj) * De + c0 + i) * NST + 4 * q);
+    else if (p.dh_last) gv = *reinterpret_cast<const float4*>(p.dh_last + (b * De + c0 + i) * NST + 4 * q);
+    g[i][0] = make_float2(gv.x, gv.y); g[i][1] = make_float2(gv.z, gv.w);
+    dA[i][0] = make_float2(0.0f, 0.0f); dA[i][1] = dA[i][0];
   }
-  const float Dc = p.D ? p.D[cc] : 0.0f;
-  float dDacc = 0.0f;
-  constexpr bool PRECISE = sizeof(T) == 4;
-  float ia[4];
+  // ---- loader / output role: step lt of every checkpoint interval, channels lc .. lc+7
+  const int lt = lane & 7, l8 = lane >> 3, lc = c_warp + 8 * l8;
+  float Dv[8], dDacc[8], dbacc[8];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) ia[i] = 1.0f / a[i];
+  for (int i = 0; i < 8; ++i) { Dv[i] = p.D ? p.D[lc + i] : 0.0f; dDacc[i] = 0.0f; dbacc[i] = 0.0f; }
+  const T* __restrict__ up = static_cast<const T*>(p.u);
+  const T* __restrict__ dyp = static_cast<const T*>(p.dy);
+  const T* __restrict__ zp = static_cast<const T*>(p.z);
+  const TD* __restrict__ dlp = static_cast<const TD*>(p.delta);
+
+  Raw8<TD> r_dl; Raw8<T> r_u, r_dy, r_z, cur_dy, cur_z;
+  float4 r_b, r_c, r_h[4];
+  auto fetch = [&](int k) {
+    const int t = k * CK + lt;
+    if (t < L) {
+      const size_t row = b * L + t;
+      r_dl.load(dlp + row * De + lc); r_u.load(up + row * De + lc); r_dy.load(dyp + row * De + lc);
+      if (zp) r_z.load(zp + row * p.ldz + lc);
+    } else {
+      r_dl.zero(); r_u.zero(); r_dy.zero(); r_z.zero();
+    }
+    // eight steps of B and C: 128 consecutive floats each, four per lane
+    const int tb = k * CK + (lane >> 2);
+    const float4 zero4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    r_b = tb < L ? __ldg(reinterpret_cast<const float4*>(p.Bm + (b * L + k * CK) * NST) + lane) : zero4;
+    r_c = tb < L ? __ldg(reinterpret_cast<const float4*>(p.Cm + (b * L + k * CK) * NST) + lane) : zero4;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) r_h[i] = __ldg(reinterpret_cast<const float4*>(p.ckpt + ((b * p.nck + k) * De + c0 + i) * NST) + q);
+  };
+  fetch(k_hi - 1);
 
   for (int k = k_hi - 1; k >= k_lo; --k) {
-    const int t0 = k * CK;
-    const int nt = min(CK, p.L - t0);
-    // ---- stage the chunk's inputs; e = dout * SiLU(z) is the gradient arriving at y
-    for (int i = tid; i < CK * BCH; i += BT) {
-      const int r = i / BCH, j = i % BCH;
-      float dl = 0.0f, uu = 0.0f, dyv = 0.0f, zz = 0.0f;
-      if (r < nt && c_base + j < p.De) {
-        const size_t e = (b * p.L + t0 + r) * p.De + c_base + j;
-        dl = p.delta[e]; uu = to_f32(u[e]); dyv = to_f32(dy[e]);
-        if (z) zz = to_f32(z[(b * p.L + t0 + r) * p.ldz + c_base + j]);
+    // ---- stage the interval: e = dout * SiLU(z) is the gradient arriving at y; steps past the end are all zero (they change nothing)
+    float2 h[4][2];
+    {
+      float dl[8], uu[8], dy[8];
+      r_dl.get(dl); r_u.get(uu); r_dy.get(dy);
+      s.dl[lt][(2 * l8) ^ lt] = make_float4(dl[0], dl[1], dl[2], dl[3]);
+      s.dl[lt][(2 * l8 + 1) ^ lt] = make_float4(dl[4], dl[5], dl[6], dl[7]);
+      s.u[lt][(2 * l8) ^ lt] = make_float4(uu[0], uu[1], uu[2], uu[3]);
+      s.u[lt][(2 * l8 + 1) ^ lt] = make_float4(uu[4], uu[5], uu[6], uu[7]);
+      if (zp) {
+        float zz[8];
+        r_z.get(zz);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) dy[i] *= zz[i] * sigmoid_f<PRECISE>(zz[i]);
       }
-      s_dl[r][j] = dl; s_u[r][j] = uu; s_dy[r][j] = dyv; s_z[r][j] = zz;
-      s_e[r][j] = z ? dyv * zz * sigmoid_f(zz) : dyv;
+      s.e[lt][(2 * l8) ^ lt] = make_float4(dy[0], dy[1], dy[2], dy[3]);
+      s.e[lt][(2 * l8 + 1) ^ lt] = make_float4(dy[4], dy[5], dy[6], dy[7]);
+      reinterpret_cast<float4*>(s.bc[0])[lane] = r_b;
+      reinterpret_cast<float4*>(s.bc[1])[lane] = r_c;
+      cur_dy = r_dy; cur_z = r_z;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) { h[i][0] = make_float2(r_h[i].x, r_h[i].y); h[i][1] = make_float2(r_h[i].z, r_h[i].w); }
     }
-    for (int i = tid; i < CK * NST; i += BT) {
-      const int r = i / NST, n = i % NST;
-      const bool in = r < nt;
-      s_B[r][n] = in ? p.Bm[(b * p.L + t0 + r) * NST + n] : 0.0f;
-      s_C[r][n] = in ? p.Cm[(b * p.L + t0 + r) * NST + n] : 0.0f;
-      s_dB[r][n] = 0.0f; s_dC[r][n] = 0.0f;
-    }
-    __syncthreads();
+    __syncwarp();
+    if (k > k_lo) fetch(k - 1);
 
-    // ---- recompute the chunk's states from its checkpoint
-    const float4 h4 = *reinterpret_cast<const float4*>(p.ckpt + ((b * p.nck + k) * p.De + cc) * NST + 4 * q);
-    const float hstart[4] = {h4.x, h4.y, h4.z, h4.w};
-    float h[4] = {h4.x, h4.y, h4.z, h4.w};
-    for (int r = 0; r < nt; ++r) {
-      const float dl = s_dl[r][cl], uu = s_u[r][cl];
-      float ys = 0.0f;
+    // ---- the interval's states, from its checkpoint
+#pragma unroll 4
+    for (int r = 0; r < CK; ++r) {
+      const float4 dl4 = s.dl[r][cg ^ r], u4 = s.u[r][cg ^ r], B4 = s.bc[0][r][q];
+      const float dlv[4] = {dl4.x, dl4.y, dl4.z, dl4.w}, uv[4] = {u4.x, u4.y, u4.z, u4.w};
+      const float2 Bv[2] = {make_float2(B4.x, B4.y), make_float2(B4.z, B4.w)};
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        float ex, em1;
-        exp_and_expm1<PRECISE>(dl * a[i], ex, em1);
-        const float bb = ZOH ? em1 * ia[i] * s_B[r][4 * q + i] : dl * s_B[r][4 * q + i];
-        h[i] = fmaf(ex, h[i], bb * uu);
-        ys = fmaf(s_C[r][4 * q + i], h[i], ys);
-      }
-      hbuf[r][tid] = make_float4(h[0], h[1], h[2], h[3]);
-      if (z) {                                     // forward y (before the gate) for the gate's derivative
-        ys += __shfl_xor_sync(0xffffffffu, ys, 1);
-        ys += __shfl_xor_sync(0xffffffffu, ys, 2);
-        if (q == 0) s_y[r][cl] = fmaf(Dc, uu, ys);
-      }
-    }
-
-    // ---- reverse sweep over the chunk
-    for (int r = nt - 1; r >= 0; --r) {
-      const float dl = s_dl[r][cl], uu = s_u[r][cl], ev = c_ok ? s_e[r][cl] : 0.0f;
-      const float4 hc4 = hbuf[r][tid];
-      const float hc[4] = {hc4.x, hc4.y, hc4.z, hc4.w};
-      float hp[4];
-      if (r > 0) { const float4 v = hbuf[r - 1][tid]; hp[0] = v.x; hp[1] = v.y; hp[2] = v.z; hp[3] = v.w; }
-      else { hp[0] = hstart[0]; hp[1] = hstart[1]; hp[2] = hstart[2]; hp[3] = hstart[3]; }
-      float dd = 0.0f, duv = 0.0f, dBp[4], dCp[4];
+        s.h[r][i][lane] = make_float4(h[i][0].x, h[i][0].y, h[i][1].x, h[i][1].y);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float Bv = s_B[r][4 * q + i], Cv = s_C[r][4 * q + i];
-        g[i] = fmaf(Cv, ev, g[i]);
-        dCp[i] = ev * hc[i];
-        float ex, em1;
-        exp_and_expm1<PRECISE>(dl * a[i], ex, em1);
-        float dx = g[i] * hp[i] * ex;              // through A-bar = exp(x)
-        if (ZOH) {
-          const float gub = g[i] * uu * Bv * ia[i], ge = g[i] * em1 * ia[i];
-          dx = fmaf(gub, ex, dx);                  // through expm1(x)
-          dAacc[i] = fmaf(gub, -em1 * ia[i], dAacc[i]);
-          dBp[i] = ge * uu;
-          duv = fmaf(ge, Bv, duv);
-          dd = fmaf(dx, a[i], dd);
-        } else {
-          dBp[i] = g[i] * uu * dl;
-          duv = fmaf(g[i] * dl, Bv, duv);
-          dd = fmaf(dx, a[i], dd);
-          dd = fmaf(g[i] * uu, Bv, dd);
+        for (int j = 0; j < 2; ++j) {
+          const float2 x = __fmul2_rn(dup(dlv[i]), a2[i][j]);
+          const float2 a = exp_pair<PRECISE>(x);
+          const float2 uB = __fmul2_rn(dup(ZOH ? uv[i] : uv[i] * dlv[i]), Bv[j]);
+          if (!ZOH) {
+            h[i][j] = __ffma2_rn(a, h[i][j], uB);
+          } else if (PRECISE) {
+            const float2 em1 = make_float2(expm1f(x.x), expm1f(x.y));
+            h[i][j] = __ffma2_rn(a, h[i][j], __fmul2_rn(__fmul2_rn(em1, ik[i][j]), uB));
+          } else {
+            const float2 w = __fmul2_rn(neg2(ik[i][j]), uB);
+            h[i][j] = __ffma2_rn(a, __fadd2_rn(h[i][j], neg2(w)), w);
+          }
         }
-        dAacc[i] = fmaf(dx, dl, dAacc[i]);
-        g[i] *= ex;
       }
-      // sums over the 16 states: the 4 lanes of the channel
-      dd += __shfl_xor_sync(0xffffffffu, dd, 1);  dd += __shfl_xor_sync(0xffffffffu, dd, 2);
-      duv += __shfl_xor_sync(0xffffffffu, duv, 1); duv += __shfl_xor_sync(0xffffffffu, duv, 2);
-      if (q == 0) {
-        s_dd[r][cl] = dd;
-        s_du[r][cl] = fmaf(Dc, ev, duv);
-        dDacc = fmaf(ev, uu, dDacc);
-      }
-      // sums over channels: the 8 channels of a warp hold 8 values each (4 dB, 4 dC of the lane's states); three exchange
-      // steps halve the values a lane keeps while adding its partner's, so every lane ends with ONE fully reduced value
-      // (7 shuffles instead of 24), then the block's warps meet in shared-memory atomics
-      {
-        float v[8];
+    }
+
+    // ---- reverse sweep
+#pragma unroll 2
+    for (int r = CK - 1; r >= 0; --r) {
+      const float4 dl4 = s.dl[r][cg ^ r], u4 = s.u[r][cg ^ r], e4 = s.e[r][cg ^ r], B4 = s.bc[0][r][q], C4 = s.bc[1][r][q];
+      const float dlv[4] = {dl4.x, dl4.y, dl4.z, dl4.w}, uv[4] = {u4.x, u4.y, u4.z, u4.w}, ev[4] = {e4.x, e4.y, e4.z, e4.w};
+      const float2 Bv[2] = {make_float2(B4.x, B4.y), make_float2(B4.z, B4.w)}, Cv[2] = {make_float2(C4.x, C4.y), make_float2(C4.z, C4.w)};
+      float2 dB[2], dC[2];
+      float ddv[4], duv[4], yv[4];
+      float4 hp4[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) { v[i] = c_ok ? dBp[i] : 0.0f; v[4 + i] = dCp[i]; }
+      for (int i = 0; i < 4; ++i) hp4[i] = s.h[r][i][lane];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 hp[2] = {make_float2(hp4[i].x, hp4[i].y), make_float2(hp4[i].z, hp4[i].w)};
+        const float2 dl = dup(dlv[i]), uu = dup(uv[i]), ee = dup(ev[i]);
+        float2 dd, du, yy;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const float2 x = __fmul2_rn(dl, a2[i][j]);
+          const float2 a = exp_pair<PRECISE>(x);
+          yy = j == 0 ? __fmul2_rn(Cv[j], h[i][j]) : __ffma2_rn(Cv[j], h[i][j], yy);
+          dC[j] = i == 0 ? __fmul2_rn(ee, h[i][j]) : __ffma2_rn(ee, h[i][j], dC[j]);
+          const float2 gg = __ffma2_rn(Cv[j], ee, g[i][j]);
+          if (ZOH) {
+            const float2 w = __fmul2_rn(neg2(ik[i][j]), __fmul2_rn(uu, Bv[j]));
+            const float2 gp = __fmul2_rn(gg, __fmul2_rn(a, __fadd2_rn(hp[j], neg2(w))));
+            const float2 am1 = PRECISE ? make_float2(expm1f(x.x), expm1f(x.y)) : __fadd2_rn(a, dup(-1.0f));
+            const float2 rr = __fmul2_rn(__fmul2_rn(gg, am1), ik[i][j]);
+            dd = j == 0 ? __fmul2_rn(a2[i][j], gp) : __ffma2_rn(a2[i][j], gp, dd);
+            du = j == 0 ? __fmul2_rn(rr, Bv[j]) : __ffma2_rn(rr, Bv[j], du);
+            dB[j] = i == 0 ? __fmul2_rn(rr, uu) : __ffma2_rn(rr, uu, dB[j]);
+            dA[i][j] = __ffma2_rn(dl, gp, dA[i][j]);
+            dA[i][j] = __ffma2_rn(rr, w, dA[i][j]);
+          } else {
+            const float2 gp = __fmul2_rn(gg, __fmul2_rn(a, hp[j]));
+            const float2 gB = __fmul2_rn(gg, Bv[j]);
+            dd = j == 0 ? __fmul2_rn(a2[i][j], gp) : __ffma2_rn(a2[i][j], gp, dd);
+            du = j == 0 ? gB : __fadd2_rn(du, gB);
+            const float2 ud = dup(uv[i] * dlv[i]);
+            dB[j] = i == 0 ? __fmul2_rn(gg, ud) : __ffma2_rn(gg, ud, dB[j]);
+            dA[i][j] = __ffma2_rn(dl, gp, dA[i][j]);
+          }
+          g[i][j] = __fmul2_rn(gg, a);
+          h[i][j] = hp[j];
+        }
+        yv[i] = yy.x + yy.y;
+        const float dsum = (dd.x + dd.y) * (PRECISE ? 1.0f : kLn2), usum = du.x + du.y;
+        if (ZOH) { ddv[i] = dsum; duv[i] = usum; }
+        else { ddv[i] = fmaf(usum, uv[i], dsum); duv[i] = usum * dlv[i]; }        // b = Delta B: du = Delta sum g B, dDelta += u sum g B
+      }
+      // partial sums over this lane's states, into the slot of the state that every lane has now consumed
+      __syncwarp();
+      s.h[r][0][lane ^ r] = make_float4(ddv[0], ddv[1], ddv[2], ddv[3]);
+      s.h[r][1][lane ^ r] = make_float4(duv[0], duv[1], duv[2], duv[3]);
+      s.h[r][2][lane ^ r] = make_float4(yv[0], yv[1], yv[2], yv[3]);
+      // sums over the warp's channels: 8 values (4 dB, 4 dC of the lane's states) over the 8 channel groups; three exchange
+      // steps halve the values a lane keeps while adding its partner's, so every lane ends with ONE fully reduced value
+      {
+        const float v[8] = {dB[0].x, dB[0].y, dB[1].x, dB[1].y, dC[0].x, dC[0].y, dC[1].x, dC[1].y};
         const bool b2 = lane & 4, b3 = lane & 8, b4 = lane & 16;
         float w4[4], w2[2];
 #pragma unroll
@@ -210,97 +283,187 @@ scan_bwd_kernel(const BwdArgs p) {
         }
         const float send = b4 ? w2[0] : w2[1], keep = b4 ? w2[1] : w2[0];
         const float tot = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-        const int idx = (b2 ? 4 : 0) + (b3 ? 2 : 0) + (b4 ? 1 : 0);      // which of the 8 values this lane ended with
-        float* dst = idx < 4 ? &s_dB[r][4 * q + idx] : &s_dC[r][4 * q + (idx - 4)];
-        atomicAdd(dst, tot);
+        const int t = k * CK + r;
+        float* dst = (b2 ? p.dCm : p.dBm) + (b * L + t) * NST + 4 * q + (b3 ? 2 : 0) + (b4 ? 1 : 0);
+        if (t < L) atomicAdd(dst, tot);
       }
     }
-    __syncthreads();
+    __syncwarp();
 
-    // ---- write the chunk's outputs
-    for (int i = tid; i < CK * BCH; i += BT) {
-      const int r = i / BCH, j = i % BCH;
-      if (r < nt && c_base + j < p.De) {
-        const size_t e = (b * p.L + t0 + r) * p.De + c_base + j;
-        p.ddelta[e] = s_dd[r][j];
-        du[e] = from_f32<T>(s_du[r][j]);
-        if (z) {
-          const float zz = s_z[r][j], sg = sigmoid_f(zz);
-          dz[(b * p.L + t0 + r) * p.ldz + c_base + j] = from_f32<T>(s_dy[r][j] * s_y[r][j] * sg * (1.0f + zz * (1.0f - sg)));
+    // ---- outputs of step lt, channels lc .. lc+7: the four lanes' partial sums of each value
+    {
+      float dd[8], du[8], yy[8], dl[8], uu[8], ee[8];
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        const int grp = 2 * l8 + hf;
+        float4 acc[3];
+#pragma unroll
+        for (int v = 0; v < 3; ++v) {
+          const float4 x0 = s.h[lt][v][(grp * 4) ^ lt], x1 = s.h[lt][v][(grp * 4 + 1) ^ lt], x2 = s.h[lt][v][(grp * 4 + 2) ^ lt], x3 = s.h[lt][v][(grp * 4 + 3) ^ lt];
+          acc[v] = make_float4((x0.x + x1.x) + (x2.x + x3.x), (x0.y + x1.y) + (x2.y + x3.y), (x0.z + x1.z) + (x2.z + x3.z), (x0.w + x1.w) + (x2.w + x3.w));
+        }
+        dd[4 * hf] = acc[0].x; dd[4 * hf + 1] = acc[0].y; dd[4 * hf + 2] = acc[0].z; dd[4 * hf + 3] = acc[0].w;
+        du[4 * hf] = acc[1].x; du[4 * hf + 1] = acc[1].y; du[4 * hf + 2] = acc[1].z; du[4 * hf + 3] = acc[1].w;
+        yy[4 * hf] = acc[2].x; yy[4 * hf + 1] = acc[2].y; yy[4 * hf + 2] = acc[2].z; yy[4 * hf + 3] = acc[2].w;
+        const float4 d4 = s.dl[lt][grp ^ lt], u4 = s.u[lt][grp ^ lt], e4 = s.e[lt][grp ^ lt];
+        dl[4 * hf] = d4.x; dl[4 * hf + 1] = d4.y; dl[4 * hf + 2] = d4.z; dl[4 * hf + 3] = d4.w;
+        uu[4 * hf] = u4.x; uu[4 * hf + 1] = u4.y; uu[4 * hf + 2] = u4.z; uu[4 * hf + 3] = u4.w;
+        ee[4 * hf] = e4.x; ee[4 * hf + 1] = e4.y; ee[4 * hf + 2] = e4.z; ee[4 * hf + 3] = e4.w;
+      }
+      const int t = k * CK + lt;
+      if (t < L) {
+        const size_t row = b * L + t;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) { du[i] = fmaf(Dv[i], ee[i], du[i]); dDacc[i] = fmaf(ee[i], uu[i], dDacc[i]); }
+        store8(static_cast<T*>(p.du) + row * De + lc, du);
+        if (zp) {
+          float zz[8], dy[8], o[8];
+          cur_z.get(zz); cur_dy.get(dy);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const float sg = sigmoid_f<PRECISE>(zz[i]);
+            o[i] = dy[i] * fmaf(Dv[i], uu[i], yy[i]) * sg * (1.0f + zz[i] * (1.0f - sg));
+          }
+          store8(static_cast<T*>(p.dz) + row * p.ldz + lc, o);
+        }
+        if (p.dpre) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) { dd[i] *= one_minus_exp<PRECISE>(dl[i]); dbacc[i] += dd[i]; }
+          store8(static_cast<T*>(p.dpre) + row * De + lc, dd);
+        } else {
+          store8(p.ddelta + row * De + lc, dd);
         }
       }
     }
-    for (int i = tid; i < CK * NST; i += BT) {
-      const int r = i / NST, n = i % NST;
-      if (r < nt) {
-        atomicAdd(p.dBm + (b * p.L + t0 + r) * NST + n, s_dB[r][n]);
-        atomicAdd(p.dCm + (b * p.L + t0 + r) * NST + n, s_dC[r][n]);
-      }
-    }
-    __syncthreads();
+    __syncwarp();
   }
 
-  if (c_ok) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      atomicAdd(p.dA + (size_t)c * NST + 4 * q + i, dAacc[i]);
-      if (p.dh0 && cj == 0) p.dh0[(b * p.De + c) * NST + 4 * q + i] = g[i];
+  for (int i = 0; i < 4; ++i) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      atomicAdd(p.dA + (size_t)(c0 + i) * NST + 4 * q + 2 * j, dA[i][j].x);
+      atomicAdd(p.dA + (size_t)(c0 + i) * NST + 4 * q + 2 * j + 1, dA[i][j].y);
     }
-    if (q == 0 && p.dD) atomicAdd(p.dD + c, dDacc);
+    if (p.dh0 && cj == 0)
+      *reinterpret_cast<float4*>(p.dh0 + (b * De + c0 + i) * NST + 4 * q) = make_float4(g[i][0].x, g[i][0].y, g[i][1].x, g[i][1].y);
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) { dDacc[i] += __shfl_xor_sync(0xffffffffu, dDacc[i], o); dbacc[i] += __shfl_xor_sync(0xffffffffu, dbacc[i], o); }
+    if (lt == 0 && p.dD) atomicAdd(p.dD + lc + i, dDacc[i]);
+    if (lt == 0 && p.dpre) atomicAdd(p.db_dt + lc + i, dbacc[i]);
   }
 }
-
 
 // Pre-pass of the chunk-parallel form, one coarse chunk per blockIdx.z: from a zero gradient, the gradient that leaves the
-// chunk's start (g <- a_t (g + C_t e_t), t descending).  (The chunk's end state and sum of Delta from a zero state come
-// from the forward scan kernel's state-only mode.)
-template <typename T>
+// chunk's start (g <- a_t (g + C_t e_t), t descending) and the sum of Delta over the chunk.  A lane owns all 16 states of one
+// channel, a warp 32 channels; eight steps are staged at a time, the next eight in flight.  Bound by the special-function unit
+// (one exponential per state and step against three fp32 operations).
+struct PreSmem { float2 de[CK][32]; float4 c[CK][4]; };
+template <typename T, typename TD>
 __global__ void __launch_bounds__(BT)
 scan_bwd_prepass_kernel(const BwdArgs p) {
-  const int tid = threadIdx.x, cl = tid >> 2, q = tid & 3;
-  const int c = blockIdx.x * BCH + cl;
-  const size_t b = blockIdx.y;
-  if (c >= p.De) return;
-  const int cj = blockIdx.z;
-  const int t_lo = cj * p.Lc, t_hi = min(t_lo + p.Lc, p.L);
-  const T* __restrict__ dy = static_cast<const T*>(p.dy);
-  const T* __restrict__ z = static_cast<const T*>(p.z);
-  float a[4], g[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-  for (int i = 0; i < 4; ++i) a[i] = p.A[(size_t)c * NST + 4 * q + i];
   constexpr bool PRECISE = sizeof(T) == 4;
-  constexpr int G = 8;                            // steps whose loads are in flight together
-  for (int t4 = t_hi - 1; t4 >= t_lo; t4 -= G) {
-    float dl[G], ev[G], zz[G];
-    float4 C4[G];
+  __shared__ PreSmem sm[WPB];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  PreSmem& s = sm[warp];
+  const int De = p.De;
+  const int c_warp = blockIdx.x * BCH + warp * WCH;
+  if (c_warp >= De) return;
+  const size_t b = blockIdx.y;
+  const int cj = blockIdx.z + 1;                  // chunk 0's start gradient is nobody's input
+  const int t_lo = cj * p.Lc, t_hi = min(t_lo + p.Lc, p.L);
+  const int c = c_warp + lane;
+  const int lt = lane & 7, l8 = lane >> 3, lc = c_warp + 8 * l8;
+  float2 a2[8], g[8];
 #pragma unroll
-    for (int j = 0; j < G; ++j) {
-      const int t = max(t4 - j, t_lo);
-      const size_t e = (b * p.L + t) * p.De + c;
-      dl[j] = p.delta[e];
-      ev[j] = to_f32(dy[e]);
-      zz[j] = z ? to_f32(z[(b * p.L + t) * p.ldz + c]) : 0.0f;
-      C4[j] = *reinterpret_cast<const float4*>(p.Cm + (b * p.L + t) * NST + 4 * q);
-    }
-#pragma unroll
-    for (int j = 0; j < G; ++j) {
-      if (t4 - j < t_lo) break;
-      if (z) ev[j] *= zz[j] * sigmoid_f(zz[j]);
-      const float cv[4] = {C4[j].x, C4[j].y, C4[j].z, C4[j].w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i) g[i] = fmaf(cv[i], ev[j], g[i]) * exp_only<PRECISE>(dl[j] * a[i]);
-    }
+  for (int i = 0; i < 4; ++i) {
+    const float4 av = *reinterpret_cast<const float4*>(p.A + (size_t)c * NST + 4 * i);
+    const float sc = PRECISE ? 1.0f : kLog2e;
+    a2[2 * i] = make_float2(av.x * sc, av.y * sc); a2[2 * i + 1] = make_float2(av.z * sc, av.w * sc);
+    g[2 * i] = make_float2(0.0f, 0.0f); g[2 * i + 1] = g[2 * i];
   }
-  const size_t o = ((b * p.ncc + cj) * p.De + c) * NST + 4 * q;
-  *reinterpret_cast<float4*>(p.q_start + o) = make_float4(g[0], g[1], g[2], g[3]);
+  float sd = 0.0f;
+  const T* __restrict__ dyp = static_cast<const T*>(p.dy);
+  const T* __restrict__ zp = static_cast<const T*>(p.z);
+  const TD* __restrict__ dlp = static_cast<const TD*>(p.delta);
+  Raw8<TD> r_dl; Raw8<T> r_dy, r_z; float4 r_c;
+  auto fetch = [&](int t0) {
+    const int t = t0 + lt;
+    if (t < t_hi) {
+      const size_t row = b * p.L + t;
+      r_dl.load(dlp + row * De + lc); r_dy.load(dyp + row * De + lc);
+      if (zp) r_z.load(zp + row * p.ldz + lc);
+    } else {
+      r_dl.zero(); r_dy.zero(); r_z.zero();
+    }
+    r_c = t0 + (lane >> 2) < t_hi ? __ldg(reinterpret_cast<const float4*>(p.Cm + (b * p.L + t0) * NST) + lane) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  };
+  int t0 = t_lo + (t_hi - t_lo - 1) / CK * CK;
+  fetch(t0);
+  for (; t0 >= t_lo; t0 -= CK) {
+    {
+      float dl[8], dy[8];
+      r_dl.get(dl); r_dy.get(dy);
+      if (zp) {
+        float zz[8];
+        r_z.get(zz);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) dy[i] *= zz[i] * sigmoid_f<PRECISE>(zz[i]);
+      }
+      // channel pairs of an 8-channel group rotated by the step: the eight lanes of a store fall into different banks
+      float4* row = reinterpret_cast<float4*>(&s.de[lt][0]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) row[(4 * l8 + i) ^ lt] = make_float4(dl[2 * i], dy[2 * i], dl[2 * i + 1], dy[2 * i + 1]);
+      reinterpret_cast<float4*>(s.c)[lane] = r_c;
+    }
+    __syncwarp();
+    if (t0 > t_lo) fetch(t0 - CK);
+#pragma unroll
+    for (int r = CK - 1; r >= 0; --r) {
+      const float2 de = s.de[r][((((lane >> 1) ^ r)) << 1) | (lane & 1)];
+      sd += de.x;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float4 C4 = s.c[r][i];
+        const float2 x0 = __fmul2_rn(dup(de.x), a2[2 * i]), x1 = __fmul2_rn(dup(de.x), a2[2 * i + 1]);
+        g[2 * i] = __fmul2_rn(__ffma2_rn(make_float2(C4.x, C4.y), dup(de.y), g[2 * i]), exp_pair<PRECISE>(x0));
+        g[2 * i + 1] = __fmul2_rn(__ffma2_rn(make_float2(C4.z, C4.w), dup(de.y), g[2 * i + 1]), exp_pair<PRECISE>(x1));
+      }
+    }
+    __syncwarp();
+  }
+  const size_t o = (b * p.ncc + cj) * De + c;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    *reinterpret_cast<float4*>(p.q_start + o * NST + 4 * i) = make_float4(g[2 * i].x, g[2 * i].y, g[2 * i + 1].x, g[2 * i + 1].y);
+  p.sum_delta[o] = sd;
 }
 
-// Composes the coarse chunks (both recurrences are linear): with P_j = exp(A sum_delta_j),
-//   h_in[0] = h0,  h_in[j+1] = P_j h_in[j] + h_end[j];   g_in[ncc-1] = dh_last,  g_in[j-1] = P_j g_in[j] + q_start[j].
+// Composes the gradient over the coarse chunks (the recurrence is linear): with P_j = exp(A sum_delta_j),
+//   g_in[ncc-1] = dh_last,  g_in[j-1] = P_j g_in[j] + q_start[j].
 __global__ void __launch_bounds__(256)
-scan_bwd_chain_kernel(const float* __restrict__ A, const float* __restrict__ h0, const float* __restrict__ dh_last,
-                      const float* __restrict__ h_end, const float* __restrict__ q_start, const float* __restrict__ sum_delta,
-                      float* __restrict__ h_in, float* __restrict__ g_in, int B, int De, int ncc) {
+scan_bwd_chain_kernel(const float* __restrict__ A, const float* __restrict__ dh_last, const float* __restrict__ q_start,
+                      const float* __restrict__ sum_delta, float* __restrict__ g_in, int B, int De, int ncc) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (long long)B * De * NST) return;
+  const int n = (int)(i % NST);
+  const int c = (int)((i / NST) % De);
+  const size_t b = (size_t)(i / ((long long)NST * De));
+  const float a = A[(size_t)c * NST + n];
+  float g = dh_last ? dh_last[i] : 0.0f;
+  for (int j = ncc - 1; j >= 0; --j) {
+    const size_t sq = b * ncc + j;
+    g_in[(sq * De + c) * NST + n] = g;
+    if (j > 0) g = fmaf(expf(a * sum_delta[sq * De + c]), g, q_start[(sq * De + c) * NST + n]);
+  }
+}
+// The same for the states (rom_scan_backward, where no forward scan has left checkpoints): h_in[0] = h0, h_in[j+1] = P_j h_in[j] + h_end[j].
+__global__ void __launch_bounds__(256)
+scan_bwd_chain_states_kernel(const float* __restrict__ A, const float* __restrict__ h0, const float* __restrict__ h_end,
+                             const float* __restrict__ sum_delta, float* __restrict__ h_in, int B, int De, int ncc) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (long long)B * De * NST) return;
   const int n = (int)(i % NST);
@@ -313,81 +476,92 @@ scan_bwd_chain_kernel(const float* __restrict__ A, const float* __restrict__ h0,
     h_in[(sq * De + c) * NST + n] = h;
     h = fmaf(expf(a * sum_delta[sq * De + c]), h, h_end[(sq * De + c) * NST + n]);
   }
-  float g = dh_last ? dh_last[i] : 0.0f;
-  for (int j = ncc - 1; j >= 0; --j) {
-    const size_t sq = b * ncc + j;
-    g_in[(sq * De + c) * NST + n] = g;
-    g = fmaf(expf(a * sum_delta[sq * De + c]), g, q_start[(sq * De + c) * NST + n]);
-  }
 }
 
-// Coarse chunks per sequence: 1 when batch x channels already give about 2048 blocks' worth of work, else enough chunks
-// (each a multiple of CK steps, at least 4 CK) to get there.  A function of the sizes only (workspace sizing = launch).
+// Coarse chunks per sequence: the count (at most 32, chunks of at least 64 steps) for which the reverse kernel's blocks best
+// fill whole waves of two blocks per SM (148 SMs assumed); the pre-pass costs about a fifth of the reverse kernel, so one chunk
+// (no pre-pass) is kept when it already fills 80 % of its waves.  A function of the sizes only (workspace sizing = launch).
 int coarse_chunks(int B, int De, int L, int* Lc_out) {
-  const long long blocks1 = (long long)B * ((De + BCH - 1) / BCH);
+  const long long blocks1 = (long long)B * ((De + BCH - 1) / BCH), slots = 148 * BLOCKS_PER_SM;
   int ncc = 1;
-  if (blocks1 < 1024) {
-    ncc = (int)((2048 + blocks1 - 1) / blocks1);
-    const int max_ncc = (L + 4 * CK - 1) / (4 * CK);
-    if (ncc > max_ncc) ncc = max_ncc;
-    if (ncc < 1) ncc = 1;
+  double best = 0.0;
+  for (int n = 1; n <= 32 && (n == 1 || (L + n - 1) / n >= 64); ++n) {
+    const long long blocks = blocks1 * n;
+    double fill = (double)blocks / (double)((blocks + slots - 1) / slots * slots);
+    if (n == 1) fill *= 1.2;
+    if (fill > best + 0.02) { best = fill; ncc = n; }
+    if (blocks > 2 * slots) break;
   }
   int Lc = (L + ncc - 1) / ncc;
-  Lc = (Lc + CK - 1) / CK * CK;
-  ncc = (L + Lc - 1) / Lc;
+  Lc = (Lc + 15) / 16 * 16;
   *Lc_out = Lc;
-  return ncc;
+  return (L + Lc - 1) / Lc;
 }
 
 }  // namespace
 
+size_t scan_bwd_ckpt_floats(int B, int De, int L) { return (size_t)B * ((L + CK - 1) / CK) * De * NST; }
+
 size_t scan_bwd_ws_bytes(int B, int De, int L) {
-  const size_t nck = (size_t)(L + CK - 1) / CK;
   int Lc = 0;
   const int ncc = coarse_chunks(B, De, L, &Lc);
-  size_t floats = (size_t)B * nck * De * NST;
-  if (ncc > 1) floats += (size_t)B * ncc * De * (4 * NST + 1);
+  size_t floats = scan_bwd_ckpt_floats(B, De, L);
+  if (ncc > 1) floats += (size_t)B * ncc * De * (4 * NST + 2);
   return align_up(sizeof(float) * floats, 256);
 }
 
-cudaError_t launch_scan_backward(const rom_config& c, const void* dy, const void* u, const float* delta, const float* A,
-                                 const float* Bm, const float* Cm, const float* D, const void* z, const float* h0,
-                                 const float* dh_last, void* du, float* ddelta, float* dA, float* dBm, float* dCm, float* dD,
-                                 void* dz, float* dh0, float* ckpt, int ldz, cudaStream_t st) {
+cudaError_t launch_scan_backward(const rom_config& c, const ScanBwd& s, cudaStream_t st) {
   const int nck = (c.L + CK - 1) / CK;
   int Lc = 0;
   const int ncc = coarse_chunks(c.B, c.d_inner, c.L, &Lc);
-  const size_t n_fine = (size_t)c.B * nck * c.d_inner * NST, n_coarse = (size_t)c.B * ncc * c.d_inner * NST;
-  float* h_end = ckpt + n_fine;
-  float* q_start = h_end + n_coarse;
-  float* h_in = q_start + n_coarse;
-  float* g_in = h_in + n_coarse;
-  float* sum_delta = g_in + n_coarse;
-  const BwdArgs a{dy, u, delta, A, Bm, Cm, D, z, h0, dh_last, du, ddelta, dA, dBm, dCm, dD, dz, dh0, ckpt, c.L, c.d_inner, nck, ldz,
-                  Lc, ncc, h_in, g_in, h_end, q_start, sum_delta};
-  cudaError_t e = cudaMemsetAsync(dA, 0, sizeof(float) * (size_t)c.d_inner * NST, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(dBm, 0, sizeof(float) * (size_t)c.B * c.L * NST, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(dCm, 0, sizeof(float) * (size_t)c.B * c.L * NST, st);
-  if (e == cudaSuccess && dD) e = cudaMemsetAsync(dD, 0, sizeof(float) * (size_t)c.d_inner, st);
+  const size_t n_fine = scan_bwd_ckpt_floats(c.B, c.d_inner, c.L), n_coarse = (size_t)c.B * ncc * c.d_inner * NST;
+  float* q_start = s.ckpt + n_fine;
+  float* g_in = q_start + n_coarse;
+  float* h_end = g_in + n_coarse;
+  float* h_in = h_end + n_coarse;
+  float* sum_delta = h_in + n_coarse;
+  float* sum_delta_h = sum_delta + (size_t)c.B * ncc * c.d_inner;
+  const BwdArgs a{s.dy, s.u, s.delta, s.A, s.Bm, s.Cm, s.D, s.z, s.dh_last, s.du, s.ddelta, s.dA, s.dBm, s.dCm, s.dD, s.dz, s.dh0, s.dpre, s.db_dt,
+                  s.ckpt, c.L, c.d_inner, nck, s.ldz, Lc, ncc, g_in, q_start, sum_delta};
+  cudaError_t e = cudaMemsetAsync(s.dA, 0, sizeof(float) * (size_t)c.d_inner * NST, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(s.dBm, 0, sizeof(float) * (size_t)c.B * c.L * NST, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(s.dCm, 0, sizeof(float) * (size_t)c.B * c.L * NST, st);
+  if (e == cudaSuccess && s.dD) e = cudaMemsetAsync(s.dD, 0, sizeof(float) * (size_t)c.d_inner, st);
+  if (e == cudaSuccess && s.dpre) e = cudaMemsetAsync(s.db_dt, 0, sizeof(float) * (size_t)c.d_inner, st);
   if (e != cudaSuccess) return e;
-  const dim3 grid((c.d_inner + BCH - 1) / BCH, c.B, ncc);
   const bool zoh = c.disc_mode == 0, bf = c.dtype == ROM_BF16;
+  const long long n_thr = (long long)c.B * c.d_inner * NST;
+  const unsigned chain_blocks = (unsigned)((n_thr + 255) / 256);
+  if (!s.ckpt_ready) {
+    // no forward scan has left checkpoints: state-only passes of the forward kernel (chunk end states, chain, checkpoints)
+    if (!s.delta_fp32) return cudaErrorInvalidValue;
+    const float* delta = static_cast<const float*>(s.delta);
+    const float* h_start = s.h0;
+    if (ncc > 1) {
+      if ((e = launch_scan_states(c, s.u, delta, s.A, s.Bm, Lc, ncc, nullptr, h_end, sum_delta_h, nullptr, 0, st)) != cudaSuccess) return e;
+      scan_bwd_chain_states_kernel<<<chain_blocks, 256, 0, st>>>(s.A, s.h0, h_end, sum_delta_h, h_in, c.B, c.d_inner, ncc);
+      count_launch();
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      h_start = h_in;
+    }
+    if ((e = launch_scan_states(c, s.u, delta, s.A, s.Bm, Lc, ncc, h_start, nullptr, nullptr, s.ckpt, nck, st)) != cudaSuccess) return e;
+  }
+  const dim3 grid((c.d_inner + BCH - 1) / BCH, c.B, ncc);
   if (ncc > 1) {
-    // chunk end states and sums of Delta from a zero state (forward scan kernel, state-only), chunk-start gradients from zero
-    if ((e = launch_scan_states(c, u, delta, A, Bm, Lc, ncc, nullptr, h_end, sum_delta, nullptr, 0, st)) != cudaSuccess) return e;
-    if (bf) scan_bwd_prepass_kernel<__nv_bfloat16><<<grid, BT, 0, st>>>(a); else scan_bwd_prepass_kernel<float><<<grid, BT, 0, st>>>(a);
+    const dim3 pgrid(grid.x, grid.y, ncc - 1);
+    if (!bf) scan_bwd_prepass_kernel<float, float><<<pgrid, BT, 0, st>>>(a);
+    else if (s.delta_fp32) scan_bwd_prepass_kernel<__nv_bfloat16, float><<<pgrid, BT, 0, st>>>(a);
+    else scan_bwd_prepass_kernel<__nv_bfloat16, __nv_bfloat16><<<pgrid, BT, 0, st>>>(a);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const long long n_thr = (long long)c.B * c.d_inner * NST;
-    scan_bwd_chain_kernel<<<(unsigned)((n_thr + 255) / 256), 256, 0, st>>>(A, h0, dh_last, h_end, q_start, sum_delta, h_in, g_in, c.B, c.d_inner, ncc);
+    scan_bwd_chain_kernel<<<chain_blocks, 256, 0, st>>>(s.A, s.dh_last, q_start, sum_delta, g_in, c.B, c.d_inner, ncc);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  // the state at the start of every 16 steps, from the true chunk-start states (forward scan kernel, state-only)
-  if ((e = launch_scan_states(c, u, delta, A, Bm, Lc, ncc, ncc > 1 ? h_in : h0, nullptr, nullptr, ckpt, nck, st)) != cudaSuccess) return e;
-  auto kern = bf ? (zoh ? scan_bwd_kernel<__nv_bfloat16, true> : scan_bwd_kernel<__nv_bfloat16, false>)
-                 : (zoh ? scan_bwd_kernel<float, true> : scan_bwd_kernel<float, false>);
-  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BWD_SMEM)) != cudaSuccess) return e;
+  auto kern = !bf ? (zoh ? scan_bwd_kernel<float, float, true> : scan_bwd_kernel<float, float, false>)
+              : s.delta_fp32 ? (zoh ? scan_bwd_kernel<__nv_bfloat16, float, true> : scan_bwd_kernel<__nv_bfloat16, float, false>)
+                             : (zoh ? scan_bwd_kernel<__nv_bfloat16, __nv_bfloat16, true> : scan_bwd_kernel<__nv_bfloat16, __nv_bfloat16, false>);
+  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, BWD_SMEM)) != cudaSuccess) return e;
   kern<<<grid, BT, BWD_SMEM, st>>>(a);
   count_launch();
   return cudaGetLastError();
