@@ -246,7 +246,7 @@ int rom_scan_backward(const rom_config* cfg, const void* dy, const void* u, cons
   if (ws_bytes < scan_bwd_ws_bytes(cfg->B, cfg->d_inner, cfg->L)) return ROM_ERR_WORKSPACE;
   if ((rc = check_device()) != ROM_OK) return rc;
   LaunchCounter::count = 0;
-  ROM_CUDA(launch_scan_backward(*cfg, ScanBwd{dy, u, delta, true, A, Bm, Cm, D, z, h0, dh_last, du, ddelta, dA, dBm, dCm, dD, dz, dh0, nullptr, nullptr,
+  ROM_CUDA(launch_scan_backward(*cfg, ScanBwd{dy, u, delta, true, A, Bm, Cm, D, z, h0, dh_last, nullptr, 1, du, ddelta, dA, dBm, dCm, dD, dz, dh0, nullptr, nullptr,
                                               static_cast<float*>(ws), false, cfg->d_inner}, static_cast<cudaStream_t>(stream)));
   return ROM_OK;
 }
@@ -416,7 +416,7 @@ namespace {
 // Scratch of rom_layer_backward: the forward workspace (routing tables and recomputed activations) followed by the
 // gradient buffers and the transposed weights.
 struct BwdLayout {
-  size_t HZs, dOp, dYgu, dYg, rowscale, dgate, dU1, dBm, dCm, dpre, dxdbl, dU2, dHZs, dHZp, dxp, dlogit;
+  size_t HZs, dOp, dYgu, dYg, rowscale, dgate, dU1, dBm, dCm, dpre, dxdbl, dU2, probs, dHZp, dxp, dlogit;
   size_t WoT, WiT, WdtT, WxT, ckpt, total;
 };
 BwdLayout make_bwd_layout(const rom_config& c, const WsLayout& l) {
@@ -436,7 +436,7 @@ BwdLayout make_bwd_layout(const rom_config& c, const WsLayout& l) {
   b.dpre = take(esz * T * De);
   b.dxdbl = take(esz * T * (R + 2 * N));
   b.dU2 = take(esz * T * De);
-  b.dHZs = take(esz * T * 2 * De);
+  b.probs = take(4 * T * c.E);
   b.dHZp = take(esz * rows * 2 * De);
   b.dxp = take(esz * rows * Dm);
   b.dlogit = take(4 * T * c.E);
@@ -515,7 +515,8 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
 
   // ---- forward, recomputed with the raw Gate Proj rows kept (the forward proper stores them activated at top-1)
   ROM_CUDA(cudaMemsetAsync(status, 0, sizeof(int32_t) * kStatusInts, st));
-  ROM_CUDA(launch_route_gather(c, x, w->W_r, w->b_r, nullptr, gates, nullptr, W, lay, st));
+  float* probs = reinterpret_cast<float*>(W + bl.probs);
+  ROM_CUDA(launch_route_gather(c, x, w->W_r, w->b_r, nullptr, gates, nullptr, W, lay, st, probs));
   if (tc && c.K == 1) {
     // one expert per token: the output op writes every row at its token's position (no activation: R = width)
     Epilogue e_in{EPI_INPROJ, W + bl.HZs, 2 * De, nullptr, nullptr, nullptr, 2 * De, 0, reinterpret_cast<const int32_t*>(W + lay.assign_of_row), nullptr};
@@ -554,10 +555,11 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
   ROM_CUDA(wgrad(W + bl.dOp, Dm, W + lay.Ygp, De, rowscale, pad_offsets, rows, g->dW_out));
 
   // ---- gate, scan and softplus, reversed
+  ROM_CUDA(launch_zero_padding(c, W + bl.dHZp, 2 * De, W, lay, st));
   float* dBm = reinterpret_cast<float*>(W + bl.dBm);
   float* dCm = reinterpret_cast<float*>(W + bl.dCm);
-  ROM_CUDA(launch_scan_backward(c, ScanBwd{W + bl.dYg, W + lay.U, W + lay.Delta, c.dtype != ROM_BF16, w->A, Bm, Cm, w->D, zraw, nullptr, nullptr, W + bl.dU1,
-                                           nullptr, g->dA, dBm, dCm, g->dD, W + bl.dHZs + (size_t)De * esz, nullptr, W + bl.dpre, g->db_dt,
+  ROM_CUDA(launch_scan_backward(c, ScanBwd{W + bl.dYg, W + lay.U, W + lay.Delta, c.dtype != ROM_BF16, w->A, Bm, Cm, w->D, zraw, nullptr, nullptr, row_of_assign, c.K,
+                                           W + bl.dU1, nullptr, g->dA, dBm, dCm, g->dD, W + bl.dHZp + (size_t)De * esz, nullptr, W + bl.dpre, g->db_dt,
                                            reinterpret_cast<float*>(W + bl.ckpt), true, 2 * De}, st));
 
   // ---- dt Proj and x Proj, reversed
@@ -570,10 +572,9 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
   // ---- conv, reversed (dU = scan part + x Proj part)
   ROM_CUDA(cudaMemsetAsync(g->dw_conv, 0, sizeof(float) * (size_t)c.d_conv * De, st));
   ROM_CUDA(cudaMemsetAsync(g->db_conv, 0, sizeof(float) * De, st));
-  ROM_CUDA(launch_conv_bwd(c, W + bl.HZs, w->w_conv, w->b_conv, W + bl.dU1, W + bl.dU2, W + bl.dHZs, g->dw_conv, g->db_conv, st));
+  ROM_CUDA(launch_conv_bwd(c, W + bl.HZs, w->w_conv, w->b_conv, W + bl.dU1, W + bl.dU2, W + bl.dHZp, row_of_assign, g->dw_conv, g->db_conv, st));
 
-  // ---- Conv Proj | Gate Proj, reversed: every selected expert of a token receives the token's (dH, dZ)
-  ROM_CUDA(launch_gather_rows_to(c, W + bl.dHZs, W + bl.dHZp, 2 * De, W, lay, st));
+  // ---- Conv Proj | Gate Proj, reversed: every selected expert of a token receives the token's (dH, dZ), written above to its rows
   ROM_CUDA(gemm_dgrad(W + bl.dHZp, 2 * De, w->W_inz, c.E, rows, Dm, 2 * De, tile_expert, num_m_tiles, W + bl.WiT, store_to(W + bl.dxp, Dm)));
   ROM_CUDA(wgrad(W + bl.dHZp, 2 * De, W + lay.x_perm, Dm, nullptr, pad_offsets, rows, g->dW_inz));
 
@@ -581,7 +582,7 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
   float* dlogit = reinterpret_cast<float*>(W + bl.dlogit);
   ROM_CUDA(cudaMemsetAsync(g->dW_r, 0, sizeof(float) * (size_t)c.E * Dm, st));
   if (g->db_r) ROM_CUDA(cudaMemsetAsync(g->db_r, 0, sizeof(float) * c.E, st));
-  ROM_CUDA(launch_router_bwd(c, x, w->W_r, w->b_r, reinterpret_cast<const int32_t*>(W + lay.topk_idx), gates, dgate, dlogit, g->db_r, g->dW_r, st));
+  ROM_CUDA(launch_router_bwd(c, x, probs, reinterpret_cast<const int32_t*>(W + lay.topk_idx), gates, dgate, dlogit, g->db_r, g->dW_r, st));
   ROM_CUDA(launch_dx(c, W + bl.dxp, row_of_assign, dlogit, w->W_r, dx, st));
   return ROM_OK;
 }

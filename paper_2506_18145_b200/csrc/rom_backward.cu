@@ -3,9 +3,9 @@
 // gate-weighted combine, softplus / conv / router reverses and the weight gradients (sums over tokens).
 //
 // Section 5.1 trains the layer end to end and Appendix A.3 trains the router through the gate values; the equations
-// differentiated are those of Sections 3.1 and 4.2 (forward: rom_api.cu).  This is the first, plain version: every
-// kernel is a straightforward fp32-accumulating loop, weight gradients leave in fp32, and sums that cross thread
-// blocks use floating-point atomics (their last bits vary from run to run).
+// differentiated are those of Sections 3.1 and 4.2 (forward: rom_api.cu).  All
+// sums are fp32, weight gradients leave in fp32, and sums that cross thread blocks use floating-point atomics (their last bits
+// vary from run to run).
 #include "rom_internal.cuh"
 
 namespace rom {
@@ -136,124 +136,158 @@ pack_bc_kernel(const float* __restrict__ dBm, const float* __restrict__ dCm, T* 
   dxdbl[t * (R + 2 * N) + R + j] = from_f32<T>(j < N ? dBm[t * N + j] : dCm[t * N + (j - N)]);
 }
 
-// Reverse of U = SiLU(b + sum_j w[j] H[t - (k-1-j)]) for a segment of 64 steps of one channel per thread:
+// Reverse of U = SiLU(b + sum_j w[j] H[t - (k-1-j)]):
 //   g_t = dU_t SiLU'(pre_t);  dH_tau = sum_j w[j] g_{tau + (k-1-j)};  dw[j] = sum_t g_t H[t - (k-1-j)];  db = sum_t g_t.
-// H is the left half of HZ ([T, 2 De]); dU = dU1 + dU2 (scan part + x Proj part); dH goes to the left half of dHZ.
-constexpr int CSEG = 64;
-template <typename T>
+// H is the left half of HZ ([T, 2 De]); dU = dU1 + dU2 (scan part + x Proj part); dH of token t goes to the left half of the K
+// rows of dHZ that row_of_assign names (the operand of the grouped Conv/Gate gradients).
+// A thread walks `seg` steps of four channels (two packed pairs) with a window of the last k-1 rows of H and of the k-1 rows of
+// dH still being collected; three rows of four steps are in flight while four are used.  Bound by HBM (24 bytes per token and
+// four channels at bf16) at one walk per element: one channel per thread with two-byte loads took 0.96 ms at 16384 x 4096
+// channels (0.56 TB/s), bound by its load and exponential instructions.
+template <typename T> struct Raw4;
+template <> struct Raw4<__nv_bfloat16> {
+  uint2 q;
+  __device__ __forceinline__ void load(const __nv_bfloat16* p) { q = __ldg(reinterpret_cast<const uint2*>(p)); }
+  __device__ __forceinline__ void zero() { q = make_uint2(0, 0); }
+  __device__ __forceinline__ void get(float2 (&v)[2]) const {
+    v[0] = make_float2(__uint_as_float(q.x << 16), __uint_as_float(q.x & 0xffff0000u));
+    v[1] = make_float2(__uint_as_float(q.y << 16), __uint_as_float(q.y & 0xffff0000u));
+  }
+  static __device__ __forceinline__ void store(__nv_bfloat16* p, const float2 (&v)[2]) {
+    const __nv_bfloat162 a = __floats2bfloat162_rn(v[0].x, v[0].y), b = __floats2bfloat162_rn(v[1].x, v[1].y);
+    *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+  }
+};
+template <> struct Raw4<float> {
+  float4 q;
+  __device__ __forceinline__ void load(const float* p) { q = __ldg(reinterpret_cast<const float4*>(p)); }
+  __device__ __forceinline__ void zero() { q = make_float4(0.0f, 0.0f, 0.0f, 0.0f); }
+  __device__ __forceinline__ void get(float2 (&v)[2]) const { v[0] = make_float2(q.x, q.y); v[1] = make_float2(q.z, q.w); }
+  static __device__ __forceinline__ void store(float* p, const float2 (&v)[2]) { *reinterpret_cast<float4*>(p) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y); }
+};
+// SiLU'(v) = s (1 + v (1 - s)), s = sigmoid(v)
+template <bool PRECISE> __device__ __forceinline__ float dsilu(float v) {
+  const float s = PRECISE ? 1.0f / (1.0f + expf(-v)) : rcp_ftz(1.0f + ex2_ftz(-1.4426950408889634f * v));
+  return s * fmaf(v, 1.0f - s, 1.0f);
+}
+
+template <typename T, int KC>
 __global__ void __launch_bounds__(128)
 conv_bwd_kernel(const T* __restrict__ HZ, const T* __restrict__ w_conv, const float* __restrict__ b_conv, const T* __restrict__ dU1,
-                const T* __restrict__ dU2, T* __restrict__ dHZ, float* __restrict__ dw, float* __restrict__ db, int L, int De, int k) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+                const T* __restrict__ dU2, T* __restrict__ dHZ, const int32_t* __restrict__ row_of_assign, float* __restrict__ dw,
+                float* __restrict__ db, int L, int De, int K, int seg) {
+  constexpr bool PRECISE = sizeof(T) == 4;
+  constexpr int G = 4;
+  const int c = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
   if (c >= De) return;
   const size_t tok0 = (size_t)blockIdx.z * L;
-  const int t0 = blockIdx.y * CSEG, t1 = min(t0 + CSEG, L), t_end = min(t1 + k - 1, L);
+  const int t0 = blockIdx.y * seg, t1 = min(t0 + seg, L), t_end = min(t1 + KC - 1, L);
   const int ld = 2 * De;
-  float w[4] = {0.0f, 0.0f, 0.0f, 0.0f}, hw[4] = {0.0f, 0.0f, 0.0f, 0.0f}, dacc[4] = {0.0f, 0.0f, 0.0f, 0.0f}, dwl[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-  for (int j = 0; j < k; ++j) w[j] = to_f32(w_conv[(size_t)j * De + c]);
-  const float bias = b_conv ? b_conv[c] : 0.0f;
-  float dbl = 0.0f;
-  // hw[j] = H[t - (k-1-j)]: before step t0 the window holds H[t0-k+1 .. t0-1] in hw[1 .. k-1]
-  for (int j = 1; j < k; ++j) {
-    const int t = t0 - k + j;
-    hw[j] = t >= 0 ? to_f32(HZ[(tok0 + t) * ld + c]) : 0.0f;
+  float2 w[KC][2], dwl[KC][2], hw[KC - 1][2], dacc[KC - 1][2], bias[2], dbl[2];
+  const float2 zero2 = make_float2(0.0f, 0.0f);
+#pragma unroll
+  for (int j = 0; j < KC; ++j) {
+    Raw4<T> r;
+    r.load(w_conv + (size_t)j * De + c); r.get(w[j]);
+    dwl[j][0] = zero2; dwl[j][1] = zero2;
   }
-  constexpr int G = 8;                      // steps whose loads are in flight together
-  for (int tg = t0; tg < t_end; tg += G) {
-    float hz[G], d1[G], d2[G];
+  bias[0] = b_conv ? make_float2(b_conv[c], b_conv[c + 1]) : zero2;
+  bias[1] = b_conv ? make_float2(b_conv[c + 2], b_conv[c + 3]) : zero2;
+  dbl[0] = zero2; dbl[1] = zero2;
+#pragma unroll
+  for (int j = 0; j < KC - 1; ++j) {      // hw[j] = H[t - (KC-1) + j] before step t
+    Raw4<T> r;
+    const int t = t0 - (KC - 1) + j;
+    if (t >= 0) r.load(HZ + (tok0 + t) * ld + c); else r.zero();
+    r.get(hw[j]);
+    dacc[j][0] = zero2; dacc[j][1] = zero2;
+  }
+  auto put = [&](int tau, const float2 (&v)[2]) {
+    for (int k = 0; k < K; ++k) Raw4<T>::store(dHZ + (size_t)__ldg(row_of_assign + (tok0 + tau) * K + k) * ld + c, v);
+  };
+  Raw4<T> rh[G], r1[G], r2[G];
+  auto fetch = [&](int tg) {
 #pragma unroll
     for (int i = 0; i < G; ++i) {
-      const int t = min(tg + i, t_end - 1);
-      hz[i] = to_f32(HZ[(tok0 + t) * ld + c]);
-      d1[i] = to_f32(dU1[(tok0 + t) * De + c]);
-      d2[i] = to_f32(dU2[(tok0 + t) * De + c]);
+      const size_t t = tok0 + min(tg + i, t_end - 1);
+      rh[i].load(HZ + t * ld + c); r1[i].load(dU1 + t * De + c); r2[i].load(dU2 + t * De + c);
     }
+  };
+  fetch(t0);
+  for (int tg = t0; tg < t_end; tg += G) {
+    Raw4<T> ch[G], c1[G], c2[G];
+#pragma unroll
+    for (int i = 0; i < G; ++i) { ch[i] = rh[i]; c1[i] = r1[i]; c2[i] = r2[i]; }
+    if (tg + G < t_end) fetch(tg + G);
 #pragma unroll
     for (int i = 0; i < G; ++i) {
       const int t = tg + i;
       if (t >= t_end) break;
-      for (int j = 0; j + 1 < k; ++j) hw[j] = hw[j + 1];
-      hw[k - 1] = hz[i];
-      float pre = bias;
-      for (int j = 0; j < k; ++j) pre = fmaf(w[j], hw[j], pre);
-      const float sg = 1.0f / (1.0f + expf(-pre));
-      const float g = (d1[i] + d2[i]) * sg * (1.0f + pre * (1.0f - sg));
-      if (t < t1) {
-        dbl += g;
-        for (int j = 0; j < k; ++j) dwl[j] = fmaf(g, hw[j], dwl[j]);
+      float2 hz[2], d1[2], d2[2], g[2], o[2];
+      ch[i].get(hz); c1[i].get(d1); c2[i].get(d2);
+      const bool own = t < t1;
+#pragma unroll
+      for (int v = 0; v < 2; ++v) {
+        float2 pre = __ffma2_rn(w[KC - 1][v], hz[v], bias[v]);
+#pragma unroll
+        for (int j = 0; j < KC - 1; ++j) pre = __ffma2_rn(w[j][v], hw[j][v], pre);
+        g[v] = __fmul2_rn(__fadd2_rn(d1[v], d2[v]), make_float2(dsilu<PRECISE>(pre.x), dsilu<PRECISE>(pre.y)));
+        if (own) {
+          dbl[v] = __fadd2_rn(dbl[v], g[v]);
+#pragma unroll
+          for (int j = 0; j < KC - 1; ++j) dwl[j][v] = __ffma2_rn(g[v], hw[j][v], dwl[j][v]);
+          dwl[KC - 1][v] = __ffma2_rn(g[v], hz[v], dwl[KC - 1][v]);
+        }
+        // dacc[i] collects dH of step t - (KC-1) + i; with this step's term, index 0 is complete
+        o[v] = __ffma2_rn(w[0][v], g[v], dacc[0][v]);
+#pragma unroll
+        for (int j = 0; j + 1 < KC - 1; ++j) dacc[j][v] = __ffma2_rn(w[j + 1][v], g[v], dacc[j + 1][v]);
+        dacc[KC - 2][v] = __fmul2_rn(w[KC - 1][v], g[v]);
+#pragma unroll
+        for (int j = 0; j + 1 < KC - 1; ++j) hw[j][v] = hw[j + 1][v];
+        hw[KC - 2][v] = hz[v];
       }
-      // dacc[i] collects dH of step t - (k-1) + i; after this step's terms, index 0 is complete
-      for (int j = 0; j < k; ++j) dacc[j] = fmaf(w[j], g, dacc[j]);
-      const int tau = t - (k - 1);
-      if (tau >= t0) dHZ[(tok0 + tau) * ld + c] = from_f32<T>(dacc[0]);
-      for (int j = 0; j + 1 < k; ++j) dacc[j] = dacc[j + 1];
-      dacc[k - 1] = 0.0f;
+      if (t - (KC - 1) >= t0) put(t - (KC - 1), o);
     }
   }
   // steps whose later neighbours do not exist (end of the sequence): what has been collected is final
-  for (int i = 0; i + 1 < k; ++i) {
-    const int tau = t_end - (k - 1) + i;
-    if (tau >= t0 && tau < t1) dHZ[(tok0 + tau) * ld + c] = from_f32<T>(dacc[i]);
+#pragma unroll
+  for (int i = 0; i < KC - 1; ++i) {
+    const int tau = t_end - (KC - 1) + i;
+    if (tau >= t0 && tau < t1) put(tau, dacc[i]);
   }
-  for (int j = 0; j < k; ++j) atomicAdd(dw + (size_t)j * De + c, dwl[j]);
-  atomicAdd(db + c, dbl);
+#pragma unroll
+  for (int j = 0; j < KC; ++j) atomicAdd(reinterpret_cast<float4*>(dw + (size_t)j * De + c), make_float4(dwl[j][0].x, dwl[j][0].y, dwl[j][1].x, dwl[j][1].y));
+  atomicAdd(reinterpret_cast<float4*>(db + c), make_float4(dbl[0].x, dbl[0].y, dbl[1].x, dbl[1].y));
 }
 
-// Reverse of the gate values with the selected set held fixed (one warp per token): logits and softmax are recomputed,
-// dP[idx_k] = dgate_k (gate_mode 0) or (dgate_k - sum_j dgate_j gate_j) / sum_j P[idx_j] (gate_mode 1),
+// Reverse of the gate values with the selected set held fixed, one thread per token: with P = Softmax(X W_r) as the router left
+// it, dP[idx_k] = dgate_k (gate_mode 0) or (dgate_k - sum_j dgate_j gate_j) / sum_j P[idx_j] (gate_mode 1),
 // dlogit = P (dP - sum_e dP_e P_e).  Writes dlogit [T, E] (fp32) and adds db_r.
-template <typename T>
-__global__ void __launch_bounds__(256)
-router_bwd_kernel(const T* __restrict__ x, const T* __restrict__ W_r, const float* __restrict__ b_r, const int32_t* __restrict__ idx,
-                  const float* __restrict__ gates, const float* __restrict__ dgate, float* __restrict__ dlogit, float* __restrict__ db_r,
-                  long long Tn, int Dm, int E, int K, int gate_mode) {
-  const int lane = threadIdx.x & 31;
-  const long long t = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (t >= Tn) return;
-  float lg[2] = {0.0f, 0.0f};              // lane e & 31 holds logit[e] in lg[e >> 5]
-  for (int e = 0; e < E; ++e) {
-    float s = 0.0f;
-    for (int d = lane; d < Dm; d += 32) s = fmaf(to_f32(x[t * Dm + d]), to_f32(W_r[(size_t)e * Dm + d]), s);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    s += b_r ? b_r[e] : 0.0f;
-    if ((e & 31) == lane) lg[e >> 5] = s;
-  }
-  // softmax over E (two values per lane at most)
-  float m = -INFINITY;
-  for (int h = 0; h < 2; ++h) if (lane + 32 * h < E) m = fmaxf(m, lg[h]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  float p[2] = {0.0f, 0.0f}, den = 0.0f;
-  for (int h = 0; h < 2; ++h) if (lane + 32 * h < E) { p[h] = expf(lg[h] - m); den += p[h]; }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) den += __shfl_xor_sync(0xffffffffu, den, o);
-  p[0] /= den; p[1] /= den;
-  // dP on the selected experts
-  float S = 1.0f, dot = 0.0f;
+__global__ void __launch_bounds__(128)
+router_bwd_kernel(const float* __restrict__ P, const int32_t* __restrict__ idx, const float* __restrict__ gates, const float* __restrict__ dgate,
+                  float* __restrict__ dlogit, float* __restrict__ db_r, long long Tn, int E, int K, int gate_mode) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool in = t < Tn;
+  const float* p = P + (in ? t : 0) * E;
+  int sel[kMaxK]; float ds[kMaxK];
+  float S = 1.0f, dot = 0.0f, mean = 0.0f;
+  for (int k = 0; k < K; ++k) { sel[k] = in ? idx[t * K + k] : 0; ds[k] = in ? dgate[t * K + k] : 0.0f; }
   if (gate_mode == 1) {
     S = 0.0f;
-    for (int k = 0; k < K; ++k) {
-      const int e = idx[t * K + k];
-      S += __shfl_sync(0xffffffffu, p[e >> 5], e & 31);
-      dot = fmaf(dgate[t * K + k], gates[t * K + k], dot);
-    }
+    for (int k = 0; k < K; ++k) { S += p[sel[k]]; dot = fmaf(ds[k], in ? gates[t * K + k] : 0.0f, dot); }
+    for (int k = 0; k < K; ++k) ds[k] = (ds[k] - dot) / S;
   }
-  float dP[2] = {0.0f, 0.0f};
-  for (int k = 0; k < K; ++k) {
-    const int e = idx[t * K + k];
-    const float ds = gate_mode == 1 ? (dgate[t * K + k] - dot) / S : dgate[t * K + k];
-    if ((e & 31) == lane) dP[e >> 5] += ds;
-  }
-  float mean = dP[0] * p[0] + dP[1] * p[1];
+  for (int k = 0; k < K; ++k) mean = fmaf(ds[k], p[sel[k]], mean);
+  for (int e = 0; e < E; ++e) {
+    float dP = 0.0f;
+    for (int k = 0; k < K; ++k) dP += sel[k] == e ? ds[k] : 0.0f;
+    float dl = in ? p[e] * (dP - mean) : 0.0f;
+    if (in) dlogit[t * E + e] = dl;
+    if (db_r) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mean += __shfl_xor_sync(0xffffffffu, mean, o);
-  for (int h = 0; h < 2; ++h) {
-    const int e = lane + 32 * h;
-    if (e < E) {
-      const float dl = p[h] * (dP[h] - mean);
-      dlogit[t * E + e] = dl;
-      if (db_r) atomicAdd(db_r + e, dl);
+      for (int o = 16; o > 0; o >>= 1) dl += __shfl_xor_sync(0xffffffffu, dl, o);
+      if ((threadIdx.x & 31) == 0) atomicAdd(db_r + e, dl);
     }
   }
 }
@@ -288,17 +322,47 @@ dx_kernel(const T* __restrict__ dxp, const int32_t* __restrict__ row_of_assign, 
   stv(dx + t * Dm + c0, acc);
 }
 
-// dW_r[e, d] = sum_t dlogit[t, e] x[t, d]: the tokens are cut into slabs of 1024, one atomic per slab and element
+// dW_r[e, d] = sum_t dlogit[t, e] x[t, d]: a thread owns four columns of x and eight experts over a slab of tokens (x is read
+// once per eight experts; the slab's dlogit values sit in shared memory), one 16-byte atomic per slab, expert and four columns.
+constexpr int RSLAB = 64;
 template <typename T>
 __global__ void __launch_bounds__(128)
 router_wgrad_kernel(const float* __restrict__ dlogit, const T* __restrict__ x, float* __restrict__ dW_r, long long Tn, int Dm, int E) {
-  const int d = blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ float dl[RSLAB][8];
+  const int e0 = blockIdx.y * 8;
+  const long long t0 = (long long)blockIdx.z * RSLAB;
+  const int nt = (int)min((long long)RSLAB, Tn - t0);
+  for (int i = threadIdx.x; i < RSLAB * 8; i += blockDim.x) {
+    const int r = i >> 3, e = e0 + (i & 7);
+    dl[r][i & 7] = (r < nt && e < E) ? dlogit[(t0 + r) * E + e] : 0.0f;
+  }
+  __syncthreads();
+  const int d = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
   if (d >= Dm) return;
-  const int e = blockIdx.y;
-  const long long t0 = (long long)blockIdx.z * 1024, t1 = min(t0 + 1024, Tn);
-  float s = 0.0f;
-  for (long long t = t0; t < t1; ++t) s = fmaf(dlogit[t * E + e], to_f32(x[t * Dm + d]), s);
-  atomicAdd(dW_r + (size_t)e * Dm + d, s);
+  float2 acc[8][2];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) { acc[e][0] = make_float2(0.0f, 0.0f); acc[e][1] = acc[e][0]; }
+  constexpr int G = 8;
+  for (int r0 = 0; r0 < nt; r0 += G) {
+    Raw4<T> raw[G];
+#pragma unroll
+    for (int i = 0; i < G; ++i) raw[i].load(x + (t0 + min(r0 + i, nt - 1)) * Dm + d);
+#pragma unroll
+    for (int i = 0; i < G; ++i) {      // rows past the slab's end repeat its last token with a zero factor
+      float2 v[2];
+      raw[i].get(v);
+      const float4 f0 = *reinterpret_cast<const float4*>(&dl[r0 + i][0]), f1 = *reinterpret_cast<const float4*>(&dl[r0 + i][4]);
+      const float f[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        acc[e][0] = __ffma2_rn(make_float2(f[e], f[e]), v[0], acc[e][0]);
+        acc[e][1] = __ffma2_rn(make_float2(f[e], f[e]), v[1], acc[e][1]);
+      }
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < 8; ++e)
+    if (e0 + e < E) atomicAdd(reinterpret_cast<float4*>(dW_r + (size_t)(e0 + e) * Dm + d), make_float4(acc[e][0].x, acc[e][0].y, acc[e][1].x, acc[e][1].y));
 }
 
 // Weight gradient of a (grouped) projection: C[s][p, q] = sum over the rows r of segment s of scale[r] X[r, p] Y[r, q]
@@ -392,35 +456,36 @@ cudaError_t launch_pack_bc(int dtype, const float* dBm, const float* dCm, void* 
   return cudaGetLastError();
 }
 
+template <typename T>
+static void launch_conv_bwd_t(const rom_config& c, const void* HZ, const void* w_conv, const float* b_conv, const void* dU1, const void* dU2, void* dHZ,
+                              const int32_t* row_of_assign, float* dw, float* db, cudaStream_t st) {
+  // 64 steps per thread (three of them walked twice), 32 when that leaves SMs idle
+  const unsigned gx = (c.d_inner / 4 + 127) / 128;
+  const int seg = (long long)gx * c.B * ((c.L + 63) / 64) >= 4 * 148 ? 64 : 32;
+  const dim3 grid(gx, (c.L + seg - 1) / seg, c.B);
+  auto go = [&](auto kern) {
+    kern<<<grid, 128, 0, st>>>((const T*)HZ, (const T*)w_conv, b_conv, (const T*)dU1, (const T*)dU2, (T*)dHZ, row_of_assign, dw, db, c.L, c.d_inner, c.K, seg);
+  };
+  if (c.d_conv == 4) go(conv_bwd_kernel<T, 4>);
+  else if (c.d_conv == 3) go(conv_bwd_kernel<T, 3>);
+  else go(conv_bwd_kernel<T, 2>);
+}
 cudaError_t launch_conv_bwd(const rom_config& c, const void* HZ, const void* w_conv, const float* b_conv, const void* dU1, const void* dU2,
-                            void* dHZ, float* dw, float* db, cudaStream_t st) {
-  const dim3 grid((c.d_inner + 127) / 128, (c.L + CSEG - 1) / CSEG, c.B);
-  if (c.dtype == ROM_BF16)
-    conv_bwd_kernel<__nv_bfloat16><<<grid, 128, 0, st>>>((const __nv_bfloat16*)HZ, (const __nv_bfloat16*)w_conv, b_conv, (const __nv_bfloat16*)dU1,
-                                                       (const __nv_bfloat16*)dU2, (__nv_bfloat16*)dHZ, dw, db, c.L, c.d_inner, c.d_conv);
-  else
-    conv_bwd_kernel<float><<<grid, 128, 0, st>>>((const float*)HZ, (const float*)w_conv, b_conv, (const float*)dU1, (const float*)dU2, (float*)dHZ,
-                                               dw, db, c.L, c.d_inner, c.d_conv);
+                            void* dHZ, const int32_t* row_of_assign, float* dw, float* db, cudaStream_t st) {
+  if (c.dtype == ROM_BF16) launch_conv_bwd_t<__nv_bfloat16>(c, HZ, w_conv, b_conv, dU1, dU2, dHZ, row_of_assign, dw, db, st);
+  else launch_conv_bwd_t<float>(c, HZ, w_conv, b_conv, dU1, dU2, dHZ, row_of_assign, dw, db, st);
   count_launch();
   return cudaGetLastError();
 }
 
-cudaError_t launch_router_bwd(const rom_config& c, const void* x, const void* W_r, const float* b_r, const int32_t* idx, const float* gates,
-                              const float* dgate, float* dlogit, float* db_r, float* dW_r, cudaStream_t st) {
+cudaError_t launch_router_bwd(const rom_config& c, const void* x, const float* probs, const int32_t* idx, const float* gates, const float* dgate,
+                              float* dlogit, float* db_r, float* dW_r, cudaStream_t st) {
   const long long Tn = (long long)c.B * c.L;
-  const unsigned blocks = (unsigned)((Tn + 7) / 8);
-  const dim3 wgrid((c.d_model + 127) / 128, c.E, (unsigned)((Tn + 1023) / 1024));
-  if (c.dtype == ROM_BF16) {
-    router_bwd_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>((const __nv_bfloat16*)x, (const __nv_bfloat16*)W_r, b_r, idx, gates, dgate, dlogit, db_r,
-                                                           Tn, c.d_model, c.E, c.K, c.gate_mode);
-    count_launch();
-    router_wgrad_kernel<__nv_bfloat16><<<wgrid, 128, 0, st>>>(dlogit, (const __nv_bfloat16*)x, dW_r, Tn, c.d_model, c.E);
-  } else {
-    router_bwd_kernel<float><<<blocks, 256, 0, st>>>((const float*)x, (const float*)W_r, b_r, idx, gates, dgate, dlogit, db_r, Tn, c.d_model, c.E,
-                                                   c.K, c.gate_mode);
-    count_launch();
-    router_wgrad_kernel<float><<<wgrid, 128, 0, st>>>(dlogit, (const float*)x, dW_r, Tn, c.d_model, c.E);
-  }
+  router_bwd_kernel<<<(unsigned)((Tn + 127) / 128), 128, 0, st>>>(probs, idx, gates, dgate, dlogit, db_r, Tn, c.E, c.K, c.gate_mode);
+  count_launch();
+  const dim3 wgrid((c.d_model / 4 + 127) / 128, (c.E + 7) / 8, (unsigned)((Tn + RSLAB - 1) / RSLAB));
+  if (c.dtype == ROM_BF16) router_wgrad_kernel<__nv_bfloat16><<<wgrid, 128, 0, st>>>(dlogit, (const __nv_bfloat16*)x, dW_r, Tn, c.d_model, c.E);
+  else router_wgrad_kernel<float><<<wgrid, 128, 0, st>>>(dlogit, (const float*)x, dW_r, Tn, c.d_model, c.E);
   count_launch();
   return cudaGetLastError();
 }

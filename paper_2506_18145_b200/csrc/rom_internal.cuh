@@ -115,10 +115,11 @@ cudaError_t launch_route(const rom_config& c, const void* x, const void* W_r, co
 cudaError_t launch_route_stats(const rom_config& c, const void* x, const void* W_r, const float* b_r,
                                int32_t* topk_idx, float* gates, int32_t* counts, int32_t* offsets,
                                int32_t* perm, int32_t* inv_perm, char* ws, const WsLayout& lay, double* chunk_prob, cudaStream_t st,
-                               bool gather_x);
+                               bool gather_x, float* probs = nullptr /* [T, E] Softmax(X W_r) */);
 // Router + tables + x_perm in two launches (the layer's path).
 cudaError_t launch_route_gather(const rom_config& c, const void* x, const void* W_r, const float* b_r,
-                                int32_t* topk_idx, float* gates, int32_t* counts, char* ws, const WsLayout& lay, cudaStream_t st);
+                                int32_t* topk_idx, float* gates, int32_t* counts, char* ws, const WsLayout& lay, cudaStream_t st,
+                                float* probs = nullptr);
 // Router + load-balance statistic: F[E], Pbar[E], loss[1] (device fp32, each may be null).
 cudaError_t launch_balance(const rom_config& c, const void* x, const void* W_r, const float* b_r, float alpha,
                            float* F, float* Pbar, float* loss, char* ws, const WsLayout& lay, cudaStream_t st);
@@ -207,6 +208,7 @@ cudaError_t launch_scan_states(const rom_config& c, const void* u, const float* 
 struct ScanBwd {
   const void* dy; const void* u; const void* delta; bool delta_fp32; const float* A; const float* Bm; const float* Cm; const float* D;
   const void* z; const float* h0; const float* dh_last;
+  const int32_t* dz_rows; int K;  // dz_rows != nullptr: dz of token t goes to its K rows dz_rows[t K + k]
   void* du; float* ddelta; float* dA; float* dBm; float* dCm; float* dD; void* dz; float* dh0;
   void* dpre; float* db_dt;      // both or neither: Delta = softplus(pre); d(pre) leaves in the storage type and its sum over tokens
                                  // in db_dt, instead of ddelta
@@ -224,9 +226,9 @@ cudaError_t launch_combine_bwd(int dtype, const void* dYgu, void* Ygp, const int
                                float* dgate, float* rowscale, long long Tn, int De, int K, cudaStream_t st);
 cudaError_t launch_pack_bc(int dtype, const float* dBm, const float* dCm, void* dxdbl, long long Tn, int R, int N, cudaStream_t st);
 cudaError_t launch_conv_bwd(const rom_config& c, const void* HZ, const void* w_conv, const float* b_conv, const void* dU1, const void* dU2,
-                            void* dHZ, float* dw, float* db, cudaStream_t st);
-cudaError_t launch_router_bwd(const rom_config& c, const void* x, const void* W_r, const float* b_r, const int32_t* idx, const float* gates,
-                              const float* dgate, float* dlogit, float* db_r, float* dW_r, cudaStream_t st);
+                            void* dHZ, const int32_t* row_of_assign, float* dw, float* db, cudaStream_t st);
+cudaError_t launch_router_bwd(const rom_config& c, const void* x, const float* probs, const int32_t* idx, const float* gates, const float* dgate,
+                              float* dlogit, float* db_r, float* dW_r, cudaStream_t st);
 cudaError_t launch_dx(const rom_config& c, const void* dxp, const int32_t* row_of_assign, const float* dlogit, const void* W_r, void* dx,
                       cudaStream_t st);
 // C[s][P, Q] = sum over rows r of segment s of scale[r] X[r, :P]^T Y[r, :Q]; seg: n_seg + 1 row offsets (device) or nullptr = one

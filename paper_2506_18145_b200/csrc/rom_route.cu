@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(512)
 route_logits_topk(const T* __restrict__ x, const T* __restrict__ W_r, const float* __restrict__ b_r,
                   int T_tokens, int Dm, int E, int K, int gate_mode,
                   int32_t* __restrict__ topk_idx, float* __restrict__ gates,
-                  int32_t* __restrict__ chunk_counts, double* __restrict__ chunk_prob, int n_chunks, const OffsetsArgs oa) {
+                  int32_t* __restrict__ chunk_counts, double* __restrict__ chunk_prob, float* __restrict__ probs, int n_chunks, const OffsetsArgs oa) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int Epad = (E + NT8 - 1) / NT8 * NT8;
   const int n_wtiles = Epad / NT8;
@@ -262,6 +262,8 @@ route_logits_topk(const T* __restrict__ x, const T* __restrict__ W_r, const floa
         if (topk_idx) topk_idx[(size_t)t * K + k] = isel[k];
         if (gates) gates[(size_t)t * K + k] = (float)gk;
       }
+      if (probs)
+        for (int e = 0; e < E; ++e) probs[(size_t)t * E + e] = (float)(pe_row[e] / denom);
     } else {
       for (int k = 0; k < K; ++k) idx_s[tid * K + k] = -1;
     }
@@ -471,8 +473,9 @@ cudaError_t launch_route(const rom_config& c, const void* x, const void* W_r, co
 }
 
 cudaError_t launch_route_gather(const rom_config& c, const void* x, const void* W_r, const float* b_r,
-                                int32_t* topk_idx, float* gates, int32_t* counts, char* ws, const WsLayout& lay, cudaStream_t st) {
-  return launch_route_stats(c, x, W_r, b_r, topk_idx, gates, counts, nullptr, nullptr, nullptr, ws, lay, nullptr, st, true);
+                                int32_t* topk_idx, float* gates, int32_t* counts, char* ws, const WsLayout& lay, cudaStream_t st,
+                                float* probs) {
+  return launch_route_stats(c, x, W_r, b_r, topk_idx, gates, counts, nullptr, nullptr, nullptr, ws, lay, nullptr, st, true, probs);
 }
 
 // Load-balance statistic (Appendix A.3): F_i = assignments of expert i / tokens, Pbar_i = mean over tokens of
@@ -517,7 +520,7 @@ static cudaError_t launch_scatter(const rom_config& c, const int32_t* idx_ws, in
 cudaError_t launch_route_stats(const rom_config& c, const void* x, const void* W_r, const float* b_r,
                                int32_t* topk_idx, float* gates, int32_t* counts, int32_t* offsets,
                                int32_t* perm, int32_t* inv_perm, char* ws, const WsLayout& lay, double* chunk_prob, cudaStream_t st,
-                               bool gather_x) {
+                               bool gather_x, float* probs) {
   const int T = (int)lay.T;
   int32_t* idx_ws = topk_idx ? topk_idx : reinterpret_cast<int32_t*>(ws + lay.topk_idx);
   int32_t* chunk_counts = reinterpret_cast<int32_t*>(ws + lay.chunk_counts);
@@ -541,10 +544,10 @@ cudaError_t launch_route_stats(const rom_config& c, const void* x, const void* W
   if (bf)
     route_logits_topk<__nv_bfloat16><<<blocks, threads, smem, st>>>(
         (const __nv_bfloat16*)x, (const __nv_bfloat16*)W_r, b_r, T, c.d_model, c.E, c.K, c.gate_mode, idx_ws, gates, chunk_counts,
-        chunk_prob, (int)lay.n_chunks, oa);
+        chunk_prob, probs, (int)lay.n_chunks, oa);
   else
     route_logits_topk<float><<<blocks, threads, smem, st>>>(
-        (const float*)x, (const float*)W_r, b_r, T, c.d_model, c.E, c.K, c.gate_mode, idx_ws, gates, chunk_counts, chunk_prob,
+        (const float*)x, (const float*)W_r, b_r, T, c.d_model, c.E, c.K, c.gate_mode, idx_ws, gates, chunk_counts, chunk_prob, probs,
         (int)lay.n_chunks, oa);
   count_launch();
   cudaError_t err = cudaGetLastError();

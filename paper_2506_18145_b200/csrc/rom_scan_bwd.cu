@@ -53,6 +53,7 @@ struct BwdArgs {
   const float* ckpt;              // [B, nck, De, 16]
   int L, De, nck;
   int ldz;                        // row pitch (elements) of z and dz
+  const int32_t* dz_rows; int K;  // rows of dz that take token t: dz_rows[t K + k]; nullptr: row t
   int Lc, ncc;                    // coarse chunks (blockIdx.z): chunk j covers steps [j Lc, (j+1) Lc); Lc is a multiple of 16
   float* g_in;                    // [B, ncc, De, 16] state gradient at the end of every coarse chunk (ncc > 1)
   float* q_start; float* sum_delta;         // pre-pass outputs: [B, ncc, De, 16] and [B, ncc, De]
@@ -137,9 +138,11 @@ scan_bwd_kernel(const BwdArgs p) {
 
   Raw8<TD> r_dl; Raw8<T> r_u, r_dy, r_z, cur_dy, cur_z;
   float4 r_b, r_c, r_h[4];
+  int r_row = 0, cur_row = 0;      // first output row of dz of this lane's step
   auto fetch = [&](int k) {
     const int t = k * CK + lt;
     if (t < L) {
+      r_row = p.dz_rows ? __ldg(p.dz_rows + (b * L + t) * p.K) : (int)(b * L + t);
       const size_t row = b * L + t;
       r_dl.load(dlp + row * De + lc); r_u.load(up + row * De + lc); r_dy.load(dyp + row * De + lc);
       if (zp) r_z.load(zp + row * p.ldz + lc);
@@ -176,7 +179,7 @@ scan_bwd_kernel(const BwdArgs p) {
       s.e[lt][(2 * l8 + 1) ^ lt] = make_float4(dy[4], dy[5], dy[6], dy[7]);
       reinterpret_cast<float4*>(s.bc[0])[lane] = r_b;
       reinterpret_cast<float4*>(s.bc[1])[lane] = r_c;
-      cur_dy = r_dy; cur_z = r_z;
+      cur_dy = r_dy; cur_z = r_z; cur_row = r_row;
 #pragma unroll
       for (int i = 0; i < 4; ++i) { h[i][0] = make_float2(r_h[i].x, r_h[i].y); h[i][1] = make_float2(r_h[i].z, r_h[i].w); }
     }
@@ -324,7 +327,9 @@ scan_bwd_kernel(const BwdArgs p) {
             const float sg = sigmoid_f<PRECISE>(zz[i]);
             o[i] = dy[i] * fmaf(Dv[i], uu[i], yy[i]) * sg * (1.0f + zz[i] * (1.0f - sg));
           }
-          store8(static_cast<T*>(p.dz) + row * p.ldz + lc, o);
+          store8(static_cast<T*>(p.dz) + (size_t)cur_row * p.ldz + lc, o);
+          if (p.dz_rows)
+            for (int kk = 1; kk < p.K; ++kk) store8(static_cast<T*>(p.dz) + (size_t)__ldg(p.dz_rows + row * p.K + kk) * p.ldz + lc, o);
         }
         if (p.dpre) {
 #pragma unroll
@@ -522,7 +527,7 @@ cudaError_t launch_scan_backward(const rom_config& c, const ScanBwd& s, cudaStre
   float* sum_delta = h_in + n_coarse;
   float* sum_delta_h = sum_delta + (size_t)c.B * ncc * c.d_inner;
   const BwdArgs a{s.dy, s.u, s.delta, s.A, s.Bm, s.Cm, s.D, s.z, s.dh_last, s.du, s.ddelta, s.dA, s.dBm, s.dCm, s.dD, s.dz, s.dh0, s.dpre, s.db_dt,
-                  s.ckpt, c.L, c.d_inner, nck, s.ldz, Lc, ncc, g_in, q_start, sum_delta};
+                  s.ckpt, c.L, c.d_inner, nck, s.ldz, s.dz_rows, s.K, Lc, ncc, g_in, q_start, sum_delta};
   cudaError_t e = cudaMemsetAsync(s.dA, 0, sizeof(float) * (size_t)c.d_inner * NST, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(s.dBm, 0, sizeof(float) * (size_t)c.B * c.L * NST, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(s.dCm, 0, sizeof(float) * (size_t)c.B * c.L * NST, st);
