@@ -290,6 +290,12 @@ int layer_forward_impl(const rom_config* cfg, const rom_weights* w, const void* 
   int32_t* row_of_assign = reinterpret_cast<int32_t*>(W + lay.row_of_assign);
   float* gates = gates_out ? gates_out : reinterpret_cast<float*>(W + lay.gates);
 
+  // single-token step with few tokens per expert: its own short launch sequence
+  if (conv_state && !ev && step_small_applicable(c)) {
+    ROM_CUDA(launch_step_small(c, *w, x, conv_state, ssm_state, out, topk_idx_out, gates, W, lay, st));
+    return ROM_OK;
+  }
+
   int stage = 0;
 #define ROM_STAGE_DONE()                                       \
   do {                                                         \

@@ -179,6 +179,11 @@ cudaError_t launch_conv(const rom_config& c, const void* XZp, const int32_t* row
 cudaError_t launch_conv_step(const rom_config& c, const void* XZp, const int32_t* row_of_assign, const void* w_conv,
                              const float* b_conv, float* conv_state, void* U, void* Zs, cudaStream_t st);
 
+// Single-token step for a few tokens per expert (rom_step.cu): the whole launch sequence.
+bool step_small_applicable(const rom_config& c);
+cudaError_t launch_step_small(const rom_config& c, const rom_weights& w, const void* x, float* conv_state, float* ssm_state, void* out,
+                              int32_t* topk_idx_out, float* gates, char* W, const WsLayout& lay, cudaStream_t st);
+
 // Scan.  z is a [rows, ldz] matrix; the gate row of token t is z_row[t] (z_row == nullptr: row t).
 // y_rows == nullptr: y is [T, d_inner]; otherwise the output row of token t is written K times, to rows
 // y_rows[t*K + k].

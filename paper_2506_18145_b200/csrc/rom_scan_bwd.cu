@@ -90,7 +90,7 @@ template <bool PRECISE> __device__ __forceinline__ float one_minus_exp(float x) 
   return x < 0.25f ? s : 1.0f - ex2_ftz(-kLog2e * x);
 }
 __device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
-__device__ __forceinline__ float2 neg2(float2 v) { return make_float2(-v.x, -v.y); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }      // a - b
 // exp(Delta A) of a pair of states, and exp - 1; a2 holds A log2(e) (A itself when PRECISE)
 template <bool PRECISE> __device__ __forceinline__ float2 exp_pair(float2 x) {
   return PRECISE ? make_float2(expf(x.x), expf(x.y)) : make_float2(ex2_ftz(x.x), ex2_ftz(x.y));
@@ -113,13 +113,13 @@ scan_bwd_kernel(const BwdArgs p) {
   // ---- compute role: channels c0 .. c0+3, states 4q .. 4q+3
   const int q = lane & 3, cg = lane >> 2;
   const int c0 = c_warp + 4 * cg;
-  float2 a2[4][2], ik[4][2], g[4][2], dA[4][2];
+  float2 a2[4][2], nik[4][2], g[4][2], dA[4][2];      // A (log2 e), -1/A, gradient carried, dA
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const float4 av = *reinterpret_cast<const float4*>(p.A + (size_t)(c0 + i) * NST + 4 * q);
     const float sc = PRECISE ? 1.0f : kLog2e;
     a2[i][0] = make_float2(av.x * sc, av.y * sc); a2[i][1] = make_float2(av.z * sc, av.w * sc);
-    ik[i][0] = make_float2(1.0f / av.x, 1.0f / av.y); ik[i][1] = make_float2(1.0f / av.z, 1.0f / av.w);
+    nik[i][0] = make_float2(-1.0f / av.x, -1.0f / av.y); nik[i][1] = make_float2(-1.0f / av.z, -1.0f / av.w);
     float4 gv = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (p.ncc > 1) gv = *reinterpret_cast<const float4*>(p.g_in + ((b * p.ncc + cj) * De + c0 + i) * NST + 4 * q);
     else if (p.dh_last) gv = *reinterpret_cast<const float4*>(p.dh_last + (b * De + c0 + i) * NST + 4 * q);
@@ -203,11 +203,11 @@ scan_bwd_kernel(const BwdArgs p) {
           if (!ZOH) {
             h[i][j] = __ffma2_rn(a, h[i][j], uB);
           } else if (PRECISE) {
-            const float2 em1 = make_float2(expm1f(x.x), expm1f(x.y));
-            h[i][j] = __ffma2_rn(a, h[i][j], __fmul2_rn(__fmul2_rn(em1, ik[i][j]), uB));
+            const float2 nem1 = make_float2(-expm1f(x.x), -expm1f(x.y));
+            h[i][j] = __ffma2_rn(a, h[i][j], __fmul2_rn(__fmul2_rn(nem1, nik[i][j]), uB));
           } else {
-            const float2 w = __fmul2_rn(neg2(ik[i][j]), uB);
-            h[i][j] = __ffma2_rn(a, __fadd2_rn(h[i][j], neg2(w)), w);
+            const float2 w = __fmul2_rn(nik[i][j], uB);
+            h[i][j] = __ffma2_rn(a, sub2(h[i][j], w), w);
           }
         }
       }
@@ -237,10 +237,10 @@ scan_bwd_kernel(const BwdArgs p) {
           dC[j] = i == 0 ? __fmul2_rn(ee, h[i][j]) : __ffma2_rn(ee, h[i][j], dC[j]);
           const float2 gg = __ffma2_rn(Cv[j], ee, g[i][j]);
           if (ZOH) {
-            const float2 w = __fmul2_rn(neg2(ik[i][j]), __fmul2_rn(uu, Bv[j]));
-            const float2 gp = __fmul2_rn(gg, __fmul2_rn(a, __fadd2_rn(hp[j], neg2(w))));
-            const float2 am1 = PRECISE ? make_float2(expm1f(x.x), expm1f(x.y)) : __fadd2_rn(a, dup(-1.0f));
-            const float2 rr = __fmul2_rn(__fmul2_rn(gg, am1), ik[i][j]);
+            const float2 w = __fmul2_rn(nik[i][j], __fmul2_rn(uu, Bv[j]));
+            const float2 gp = __fmul2_rn(gg, __fmul2_rn(a, sub2(hp[j], w)));
+            const float2 oma = PRECISE ? make_float2(-expm1f(x.x), -expm1f(x.y)) : sub2(dup(1.0f), a);      // 1 - a
+            const float2 rr = __fmul2_rn(__fmul2_rn(gg, oma), nik[i][j]);
             dd = j == 0 ? __fmul2_rn(a2[i][j], gp) : __ffma2_rn(a2[i][j], gp, dd);
             du = j == 0 ? __fmul2_rn(rr, Bv[j]) : __ffma2_rn(rr, Bv[j], du);
             dB[j] = i == 0 ? __fmul2_rn(rr, uu) : __ffma2_rn(rr, uu, dB[j]);

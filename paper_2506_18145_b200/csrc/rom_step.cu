@@ -1,0 +1,803 @@
+// Single-token step of the layer (recurrent inference) for a few tokens per expert, bf16: five launches, chained by programmatic
+// dependent launch, against the eight of the general sequence.
+//
+//   step_route    : one block per token: logits in fp64 (exact products, the same order for every expert), softmax, top-K
+//   step_gemm<IN> : grouped [Conv Proj | Gate Proj] of the selected experts; at top-1 its output op also runs the short conv
+//                   on the caller's window of H (step_conv does both for K > 1, where H is a sum over experts)
+//   step_gemm<X>  : x Proj -> delta_r | B | C
+//   step_dt_scan  : dt Proj + softplus, one step of the recurrence on the caller's state, skip, gate
+//   step_gemm<OUT>: grouped Out Proj, times the gate (K > 1: rows summed by step_combine)
+//
+// What bounds it: the weights of the selected experts, read once (HBM), and below that latency -- every stage waits for the one
+// before.  With a handful of tokens per expert a 128-row tensor tile is nearly all padding and one CTA per 256 columns leaves
+// most SMs idle (out_proj of one token: 8 CTAs, 26 us for 16 MB).  Here the weights are the M operand of mma.m16n8k16 and the
+// tokens its N = 8 columns: a block owns 16 or 32 weight rows and splits the contracted index over its warps, so that one token
+// already spreads over 128 to 256 blocks; lanes read 16 consecutive bytes of a weight row straight into fragments (the
+// contracted index is permuted inside a 32-wide block, alike for both operands).  Every kernel requests what does not depend on
+// its predecessor (states, small weights, and for the Out Proj its first weight tiles) before it waits.
+// The predecessor's predecessors are complete by then: every kernel triggers its successor only after its own wait.
+#include "rom_tc_ptx.cuh"
+
+namespace rom {
+namespace {
+
+constexpr int NST = 16;
+constexpr int kStepMaxTokens = 512, kStepMaxAssign = 2048;
+constexpr int kStreamMin = 4;          // assignments from which the weights are streamed (step_tc)
+constexpr float kLog2e = 1.4426950408889634f;
+typedef __nv_bfloat16 bf16;
+
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+__device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+               : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// One 32-wide block of the contracted index: q0 / q1 = rows g / g + 8 of the weights, xq = token g, each 8 consecutive elements
+// at 8 t.  The pairs (0,1), (2,3) feed the first MMA, (4,5), (6,7) the second.
+__device__ __forceinline__ void mma_block(float (&d)[4], const uint4& q0, const uint4& q1, const uint4& xq) {
+  mma_bf16(d, q0.x, q1.x, q0.y, q1.y, xq.x, xq.y);
+  mma_bf16(d, q0.z, q1.z, q0.w, q1.w, xq.z, xq.w);
+}
+// weights are read once per step: keep them out of the way of the activations in L1
+__device__ __forceinline__ uint4 ld_stream(const bf16* p) {
+  uint4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+// activations of an earlier kernel of the chain
+__device__ __forceinline__ uint4 ld_act(const bf16* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  return v;
+}
+
+// ---------------------------------------------------------------------------------------------- router
+__global__ void __launch_bounds__(256)
+step_route(const bf16* __restrict__ x, const bf16* __restrict__ W_r, const float* __restrict__ b_r, int Dm, int E, int K, int gate_mode,
+           int32_t* __restrict__ idx_ws, float* __restrict__ gates_ws, int32_t* __restrict__ idx_out, int32_t* __restrict__ status) {
+  __shared__ double part[8][kMaxE];
+  __shared__ double lg[kMaxE], pr[kMaxE];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int t = blockIdx.x;
+  pdl_trigger();                        // the first kernel of the chain: nothing before it is pending
+  if (t == 0 && threadIdx.x < kStatusInts) status[threadIdx.x] = 0;
+  // warp w takes the 8-element groups w * 32 + lane, ...: every expert sums in the same order
+  for (int e0 = 0; e0 < E; e0 += 8) {
+    double acc[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[e] = 0.0;
+    for (int d = (warp * 32 + lane) * 8; d < Dm; d += 2048) {
+      V16<bf16> q;
+      float xv[8];
+      q.load(x + (size_t)t * Dm + d); q.get(xv);
+      V16<bf16> wq[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) wq[e].load(W_r + (size_t)min(e0 + e, E - 1) * Dm + d);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        float wv[8];
+        wq[e].get(wv);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) acc[e] += (double)(xv[i] * wv[i]);      // bf16 products are exact in fp32
+      }
+    }
+    // transposed sums over the lanes: 8 values -> lane keeps value (lane & 7) after three exchanges, then two plain ones
+    {
+      double a4[4], a2[2], a1;
+      const bool s0 = lane & 1, s1 = lane & 2, s2 = lane & 4;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const double send = s2 ? acc[i] : acc[4 + i], keep = s2 ? acc[4 + i] : acc[i];
+        a4[i] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const double send = s1 ? a4[i] : a4[2 + i], keep = s1 ? a4[2 + i] : a4[i];
+        a2[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
+      }
+      const double send = s0 ? a2[0] : a2[1], keep = s0 ? a2[1] : a2[0];
+      a1 = keep + __shfl_xor_sync(0xffffffffu, send, 1);
+      a1 += __shfl_xor_sync(0xffffffffu, a1, 8);
+      a1 += __shfl_xor_sync(0xffffffffu, a1, 16);
+      if (lane < 8 && e0 + lane < kMaxE) part[warp][e0 + lane] = a1;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < E) {
+    const int e = threadIdx.x;
+    double v = b_r ? (double)b_r[e] : 0.0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) v += part[w][e];
+    lg[e] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x < E) {
+    double m = -INFINITY;
+    for (int j = 0; j < E; ++j) { const double v = lg[j]; if (v > m) m = v; }      // NaN never raises m
+    pr[threadIdx.x] = exp(lg[threadIdx.x] - m);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double denom = 0.0, gsum = 0.0, gsel[kMaxK];
+    for (int e = 0; e < E; ++e) denom += pr[e];
+    unsigned long long taken = 0ull;
+    int isel[kMaxK];
+    for (int k = 0; k < K; ++k) {
+      int best = -1; double bestv = -INFINITY;
+      for (int e = 0; e < E; ++e) {
+        if ((taken >> e) & 1ull) continue;
+        double v = lg[e];
+        if (v != v) v = -INFINITY;
+        if (best < 0 || v > bestv) { best = e; bestv = v; }
+      }
+      taken |= 1ull << best;
+      isel[k] = best;
+      gsel[k] = pr[best] / denom;
+      gsum += gsel[k];
+    }
+    for (int k = 0; k < K; ++k) {
+      idx_ws[t * K + k] = isel[k];
+      if (idx_out) idx_out[t * K + k] = isel[k];
+      gates_ws[t * K + k] = (float)(gate_mode == 1 ? gsel[k] / gsum : gsel[k]);
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------------------------- projections
+enum StepGemm { STEP_IN = 0, STEP_X = 1, STEP_OUT = 2 };
+struct StepGemmArgs {
+  const bf16* x; int ldx;               // activation rows: IN: x [B, Dm]; X: U [B, De]; OUT: Yg [B, De]
+  const bf16* W; int Kd, n_rows;        // weights [E or 1, n_rows, Kd]
+  const int32_t* idx; const float* gates; int B, K, E;
+  bf16* C; int ldc;                     // IN: XZ [B K, 2 De]; X: delta_r [B, R]; OUT: out [B, Dm] (K == 1) or Op [B K, Dm]
+  // IN at top-1: the short conv
+  int De; const bf16* w_conv; const float* b_conv; float* conv_state; int dconv; bf16* U;
+  // X
+  float* Bm; float* Cm; int R;
+};
+
+template <int MODE, int RT, int NT, int WARPS>
+__global__ void __launch_bounds__(WARPS * 32)
+step_gemm(const StepGemmArgs p) {
+  constexpr int ROWS = RT * 16, COLS = NT * 8, PITCH = ROWS + 4;
+  constexpr int U = RT == 2 ? 4 : 8;                 // 32-wide blocks in flight per warp
+  __shared__ __align__(16) float red[WARPS][COLS][PITCH];
+  __shared__ int list[kStepMaxTokens];               // assignments of this block's expert
+  __shared__ unsigned long long mask;
+  __shared__ int count;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t4 = lane & 3;
+  const int row0 = blockIdx.x * ROWS;
+  const int nkb = p.Kd / 32;
+
+  int e = 0;
+  int m;                                             // tokens of this block
+  if (MODE == STEP_IN) { pdl_wait(); pdl_trigger(); }      // (OUT: the routing tables are two kernels back, complete already)
+  if (MODE != STEP_X) {
+    // the blockIdx.y-th selected expert and its assignments (in whatever order: a token's column does not matter)
+    if (threadIdx.x == 0) { mask = 0ull; count = 0; }
+    __syncthreads();
+    const int A = p.B * p.K;
+    for (int a = threadIdx.x; a < A; a += WARPS * 32) atomicOr(&mask, 1ull << p.idx[a]);
+    __syncthreads();
+    unsigned long long mk = mask;
+    for (int i = 0; i < (int)blockIdx.y && mk; ++i) mk &= mk - 1;
+    if (!mk) {
+      if (MODE == STEP_OUT) { pdl_wait(); pdl_trigger(); }
+      return;
+    }
+    e = __ffsll(mk) - 1;
+    for (int a = threadIdx.x; a < A; a += WARPS * 32)
+      if (p.idx[a] == e) list[atomicAdd(&count, 1)] = a;
+    __syncthreads();
+    m = count;
+  } else {
+    m = min(COLS, p.B - (int)blockIdx.y * COLS);
+  }
+  const bf16* wrow[RT][2];
+#pragma unroll
+  for (int r = 0; r < RT; ++r)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) wrow[r][h] = p.W + ((size_t)e * p.n_rows + row0 + r * 16 + h * 8 + g) * p.Kd + 8 * t4;
+
+  bool waited = MODE == STEP_IN;
+  for (int n0 = 0; n0 < m; n0 += COLS) {
+    const int nt_used = (min(m - n0, COLS) + 7) / 8;
+    const bf16* xrow[NT];
+#pragma unroll
+    for (int n = 0; n < NT; ++n) {
+      const int j = n0 + n * 8 + g;
+      const int tok = j < m ? (MODE == STEP_X ? (int)blockIdx.y * COLS + j : list[j] / p.K) : -1;
+      xrow[n] = tok >= 0 ? p.x + (size_t)tok * p.ldx + 8 * t4 : nullptr;
+    }
+    float acc[RT][NT][4] = {};
+    for (int kb0 = warp; kb0 < nkb; kb0 += WARPS * U) {
+      uint4 wq[U][RT][2];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int kb = min(kb0 + u * WARPS, nkb - 1);      // past the end: the last block again, against zero activations
+#pragma unroll
+        for (int r = 0; r < RT; ++r) { wq[u][r][0] = ld_stream(wrow[r][0] + kb * 32); wq[u][r][1] = ld_stream(wrow[r][1] + kb * 32); }
+      }
+      if (!waited) { pdl_wait(); pdl_trigger(); waited = true; }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int kb = kb0 + u * WARPS;
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+          if (n >= nt_used) break;
+          const uint4 xq = (xrow[n] && kb < nkb) ? ld_act(xrow[n] + kb * 32) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+          for (int r = 0; r < RT; ++r) mma_block(acc[r][n], wq[u][r][0], wq[u][r][1], xq);
+        }
+      }
+    }
+    if (!waited) { pdl_wait(); pdl_trigger(); waited = true; }
+    if (n0 > 0) __syncthreads();                     // the previous group's sums have been read
+#pragma unroll
+    for (int r = 0; r < RT; ++r)
+#pragma unroll
+      for (int n = 0; n < NT; ++n) {
+        if (n >= nt_used) break;
+        red[warp][n * 8 + 2 * t4][r * 16 + g] = acc[r][n][0];
+        red[warp][n * 8 + 2 * t4 + 1][r * 16 + g] = acc[r][n][1];
+        red[warp][n * 8 + 2 * t4][r * 16 + g + 8] = acc[r][n][2];
+        red[warp][n * 8 + 2 * t4 + 1][r * 16 + g + 8] = acc[r][n][3];
+      }
+    __syncthreads();
+    // sums over the warps, output op on two adjacent rows of one token
+    constexpr int PAIRS = ROWS / 2;
+    for (int i = threadIdx.x; i < min(m - n0, COLS) * PAIRS; i += WARPS * 32) {
+      const int j = i / PAIRS, r = (i % PAIRS) * 2;
+      float2 v = make_float2(0.0f, 0.0f);
+#pragma unroll
+      for (int w = 0; w < WARPS; ++w) {
+        const float2 q = *reinterpret_cast<const float2*>(&red[w][j][r]);
+        v.x += q.x; v.y += q.y;
+      }
+      const int row = row0 + r;
+      if (MODE == STEP_X) {
+        const size_t tok = blockIdx.y * COLS + j;
+        if (row < p.R) *reinterpret_cast<__nv_bfloat162*>(p.C + tok * p.R + row) = __floats2bfloat162_rn(v.x, v.y);
+        else if (row < p.R + NST) *reinterpret_cast<float2*>(p.Bm + tok * NST + row - p.R) = v;
+        else *reinterpret_cast<float2*>(p.Cm + tok * NST + row - p.R - NST) = v;
+      } else if (MODE == STEP_OUT) {
+        const int a = list[n0 + j];
+        const float gt = p.K == 1 ? p.gates[a] : 1.0f;
+        *reinterpret_cast<__nv_bfloat162*>(p.C + (size_t)a * p.ldc + row) = __floats2bfloat162_rn(v.x * gt, v.y * gt);
+      } else {
+        const int a = list[n0 + j];
+        if (p.U == nullptr) {                        // K > 1: rows of the assignment, summed over the slots by step_conv
+          *reinterpret_cast<__nv_bfloat162*>(p.C + (size_t)a * p.ldc + row) = __floats2bfloat162_rn(v.x, v.y);
+        } else if (row >= p.De) {                    // Gate Proj row, activated
+          *reinterpret_cast<__nv_bfloat162*>(p.C + (size_t)a * p.ldc + row) = __floats2bfloat162_rn(silu_fast(v.x), silu_fast(v.y));
+        } else {
+          // Conv Proj row: H (rounded to the storage type), the conv over the caller's window, and the window moved on
+          const __nv_bfloat162 hb = __floats2bfloat162_rn(v.x, v.y);
+          const float2 h = __bfloat1622float2(hb);
+          float* st = p.conv_state + (size_t)a * (p.dconv - 1) * p.De + row;
+          float2 u = p.b_conv ? *reinterpret_cast<const float2*>(p.b_conv + row) : make_float2(0.0f, 0.0f);
+          float2 win[3];
+          for (int q = 0; q < p.dconv - 1; ++q) win[q] = *reinterpret_cast<const float2*>(st + (size_t)q * p.De);
+          for (int q = 0; q < p.dconv; ++q) {
+            const float2 w = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p.w_conv + (size_t)q * p.De + row));
+            const float2 hv = q < p.dconv - 1 ? win[q] : h;
+            u.x = fmaf(w.x, hv.x, u.x); u.y = fmaf(w.y, hv.y, u.y);
+          }
+          *reinterpret_cast<__nv_bfloat162*>(p.U + (size_t)a * p.De + row) = __floats2bfloat162_rn(silu_fast(u.x), silu_fast(u.y));
+          for (int q = 0; q + 1 < p.dconv - 1; ++q) *reinterpret_cast<float2*>(st + (size_t)q * p.De) = win[q + 1];
+          *reinterpret_cast<float2*>(st + (size_t)(p.dconv - 2) * p.De) = h;
+        }
+      }
+    }
+  }
+  if (!waited) { pdl_wait(); pdl_trigger(); }
+}
+
+// The same for more assignments, where the weights of most experts are walked and streaming them is all that counts: tcgen05 with
+// the weights as the M = 128 operand and an expert's tokens (16, 32 or 64 columns, at most TC_N per pass) as N.  One persistent CTA
+// per SM takes (expert, 128 weight rows) tiles; warp 0 keeps a ring of operand stages full of weights (128 x 64 by one TMA load),
+// warps 6..9 put the tokens' rows beside them (16-byte loads on their indices into the swizzled layout: nothing is permuted in
+// memory, and the TMA unit is left to the weights -- gather4 loads cost it about 28 ns a row, more than the weights of the stage),
+// warp 1 issues the MMAs, warps 2..5 drain the accumulator (lane = weight row, column = token; double-buffered) while the next tile
+// streams.  The register-fed kernel above reached 3.6 TB/s at 64 tokens (268 MB in 74 us), waiting on its own sums and output ops.
+constexpr int TC_N = 64;                             // token columns per pass
+constexpr int TC_A_BYTES = 128 * BLOCK_K * 2, TC_STAGE = TC_A_BYTES + TC_N * BLOCK_K * 2;
+constexpr int TC_STAGES = 8;
+constexpr int TC_SMEM = TC_STAGES * TC_STAGE + 1024;
+constexpr int TC_THREADS = 320;
+
+template <int MODE>
+__global__ void __launch_bounds__(TC_THREADS, 1)
+step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_t* __restrict__ status) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  __shared__ int cnt[kMaxE], off[kMaxE + 1], fill[kMaxE], act[kMaxE], n_act_s;
+  __shared__ short list[kStepMaxAssign], tok[kStepMaxAssign];      // assignments by expert, and their tokens
+  __shared__ __align__(8) unsigned long long bars[2 * TC_STAGES + 5];
+  __shared__ uint32_t tmem_s;
+  __shared__ int abort_s;
+  volatile int* abort_flag = &abort_s;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  auto full_bar = [&](int s) { return smem_u32(&bars[s]); };
+  auto empty_bar = [&](int s) { return smem_u32(&bars[TC_STAGES + s]); };
+  auto tfull_bar = [&](int a) { return smem_u32(&bars[2 * TC_STAGES + a]); };
+  auto tempty_bar = [&](int a) { return smem_u32(&bars[2 * TC_STAGES + 2 + a]); };
+  const uint32_t drain_bar = smem_u32(&bars[2 * TC_STAGES + 4]);
+
+  if (MODE == STEP_IN) { pdl_wait(); pdl_trigger(); }      // OUT: the routing is two kernels back; the wait comes before the activations
+  if (tid == 0) {
+    for (int s = 0; s < TC_STAGES; ++s) { mbar_init(full_bar(s), 1 + 4); mbar_init(empty_bar(s), 1); }
+    for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), 4); }
+    mbar_init(drain_bar, 1);
+    abort_s = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (tid < kMaxE) { cnt[tid] = 0; fill[tid] = 0; }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_s)), "r"(2 * TC_N) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = tmem_s;
+  // assignments of every expert (in whatever order: a token's column does not matter)
+  const int A = p.B * p.K;
+  for (int a = tid; a < A; a += TC_THREADS) atomicAdd(&cnt[p.idx[a]], 1);
+  __syncthreads();
+  auto cols = [](int m) { return m > 32 ? 64 : m > 16 ? 32 : 16; };      // N of a pass over m tokens
+  if (tid == 0) {
+    int o = 0, n = 0;
+    for (int e = 0; e < p.E; ++e) { off[e] = o; o += cnt[e]; if (cnt[e]) act[n++] = e; }
+    n_act_s = n;
+  }
+  __syncthreads();
+  for (int a = tid; a < A; a += TC_THREADS) {
+    const int e = p.idx[a], at = off[e] + atomicAdd(&fill[e], 1);
+    list[at] = (short)a; tok[at] = (short)(a / p.K);
+  }
+  __syncthreads();
+  const int tpe = (p.n_rows + 127) / 128;            // weight tiles per expert
+  const int total = n_act_s * tpe;
+  const int num_kb = p.Kd / BLOCK_K;
+
+  if (warp == 0) {
+    // ---------------------------------------------------------------- TMA producer of the weights (nothing here depends on the launch before)
+    if (lane == 0) {
+    int stage = 0, issued = 0; uint32_t phase = 0;
+    bool ok = true;
+    for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
+      const int e = act[w / tpe], tile = w % tpe;
+      for (int n0 = 0; n0 < cnt[e] && ok; n0 += TC_N)
+        for (int kb = 0; kb < num_kb; ++kb) {
+          if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, WAIT_LIMIT)) { ok = false; break; }
+          mbar_expect_tx(full_bar(stage), TC_A_BYTES);
+          tma_load_2d(base + stage * TC_STAGE, &tmap_w, full_bar(stage), kb * BLOCK_K, e * p.n_rows + tile * 128);
+          ++issued;
+          if (++stage == TC_STAGES) { stage = 0; phase ^= 1u; }
+        }
+    }
+    if (!ok) {
+      if (!*abort_flag) { atomicExch(status + kStatCode, ROM_ERR_DEVICE_TIMEOUT); atomicExch(status + kStatWhere, 4); }
+      *abort_flag = 1;
+    }
+    if (*abort_flag) {                               // give the copies still in flight a bounded time to land before the CTA exits
+      for (int i = 0; i < min(issued, TC_STAGES); ++i) {
+        if (--stage < 0) { stage = TC_STAGES - 1; phase ^= 1u; }
+        for (uint32_t it = 0; it < (WAIT_LIMIT >> 2); ++it)
+          if (mbar_try_wait(full_bar(stage), phase)) break;
+      }
+    }
+    }
+  } else if (warp == 1) {
+    // ---------------------------------------------------------------- MMA issuer
+    if (lane == 0) {
+      int stage = 0; uint32_t phase = 0;
+      int acc = 0; uint32_t acc_phase = 0;
+      bool ok = true, issued_any = false;
+      for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
+        const int e = act[w / tpe];
+        for (int n0 = 0; n0 < cnt[e] && ok; n0 += TC_N) {
+          const int n16 = cols(min(cnt[e] - n0, TC_N));
+          const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n16 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+          if (!mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag, WAIT_LIMIT)) { ok = false; break; }
+          tc_fence_after();
+          for (int kb = 0; kb < num_kb; ++kb) {
+            if (!mbar_wait(full_bar(stage), phase, abort_flag, WAIT_LIMIT)) { ok = false; break; }
+            tc_fence_after();
+            const uint64_t adesc = make_smem_desc(base + stage * TC_STAGE), bdesc = make_smem_desc(base + stage * TC_STAGE + TC_A_BYTES);
+#pragma unroll
+            for (int k = 0; k < BLOCK_K / UMMA_K; ++k)
+              umma_bf16(tmem_base + acc * TC_N, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc, (kb | k) != 0 ? 1u : 0u);
+            umma_commit(empty_bar(stage));
+            issued_any = true;
+            if (++stage == TC_STAGES) { stage = 0; phase ^= 1u; }
+          }
+          if (!ok) break;
+          umma_commit(tfull_bar(acc));
+          if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+        }
+      }
+      if (!ok) {
+        if (!*abort_flag) { atomicExch(status + kStatCode, ROM_ERR_DEVICE_TIMEOUT); atomicExch(status + kStatWhere, 5); }
+        *abort_flag = 1;
+      }
+      if (*abort_flag && issued_any) {
+        umma_commit(drain_bar);
+        for (uint32_t it = 0; it < (WAIT_LIMIT >> 2); ++it)
+          if (mbar_try_wait(drain_bar, 0)) break;
+      }
+    }
+  } else if (warp >= 6) {
+    // ---------------------------------------------------------------- token rows of every stage: 128 threads, 16-byte pieces
+    const int l = tid - 6 * 32, lrow = l >> 3, chunk = l & 7;
+    if (MODE == STEP_OUT) { pdl_wait(); pdl_trigger(); }
+    int stage = 0; uint32_t phase = 0;
+    bool ok = true;
+    for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
+      const int e = act[w / tpe];
+      for (int n0 = 0; n0 < cnt[e] && ok; n0 += TC_N) {
+        const int m = min(cnt[e] - n0, TC_N), nq = cols(m) >> 4;      // 16-row groups: 1, 2 or 4 pieces per thread and stage
+        const bf16* src[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) src[q] = p.x + (size_t)tok[off[e] + n0 + min(lrow + 16 * q, m - 1)] * p.ldx + chunk * 8;      // (rows past the last token repeat it)
+        const int kpc = 4 / nq, n_ch = (num_kb + kpc - 1) / kpc;      // four pieces in flight per thread while four are stored
+        uint4 cur[4], nxt[4];
+        auto fetch = [&](int ch, uint4 (&d)[4]) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int kb = min(ch * kpc + i / nq, num_kb - 1);
+            const bf16* sp = nq == 1 ? src[0] : nq == 2 ? src[i & 1] : src[i];
+            d[i] = ld_act(sp + kb * BLOCK_K);
+          }
+        };
+        fetch(0, cur);
+        for (int ch = 0; ch < n_ch && ok; ++ch) {
+          if (ch + 1 < n_ch) fetch(ch + 1, nxt);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int kb = ch * kpc + i / nq, q = nq == 1 ? 0 : nq == 2 ? (i & 1) : i;
+            if (kb >= num_kb) break;
+            if (q == 0) {
+              ok = __all_sync(0xffffffffu, mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, WAIT_LIMIT));
+              if (!ok) break;
+            }
+            const int r = lrow + 16 * q;
+            *reinterpret_cast<uint4*>(smem_raw + (base - smem_u32(smem_raw)) + stage * TC_STAGE + TC_A_BYTES + r * 128 + ((chunk ^ (r & 7)) << 4)) = cur[i];
+            if (q == nq - 1) {
+              asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+              __syncwarp();
+              if (lane == 0) mbar_arrive(full_bar(stage));
+              if (++stage == TC_STAGES) { stage = 0; phase ^= 1u; }
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < 4; ++i) cur[i] = nxt[i];
+        }
+      }
+    }
+    if (!ok && lane == 0) {
+      if (!*abort_flag) { atomicExch(status + kStatCode, ROM_ERR_DEVICE_TIMEOUT); atomicExch(status + kStatWhere, 7); }
+      *abort_flag = 1;
+    }
+  } else {
+    // ---------------------------------------------------------------- output: lane = weight row, column = token
+    const int quarter = warp & 3;
+    int acc = 0; uint32_t acc_phase = 0;
+    bool ok = true;
+    for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
+      const int e = act[w / tpe], row = (w % tpe) * 128 + quarter * 32 + lane;
+      const bool row_ok = row < p.n_rows;
+      const bool conv = MODE == STEP_IN && p.U != nullptr && row < p.De;      // warp-uniform: De is a multiple of 32
+      float wv[4], bias = 0.0f;
+      if (conv) {
+        if (p.b_conv) bias = p.b_conv[row];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) wv[q] = q < p.dconv ? to_f32(p.w_conv[(size_t)q * p.De + row]) : 0.0f;
+      }
+      for (int n0 = 0; n0 < cnt[e] && ok; n0 += TC_N) {
+        const int m = min(cnt[e] - n0, TC_N);
+        const short* mine = list + off[e] + n0;
+        if (!__all_sync(0xffffffffu, mbar_wait(tfull_bar(acc), acc_phase, abort_flag, WAIT_LIMIT))) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)acc * TC_N;
+        for (int c0 = 0; c0 < m; c0 += 32) {
+          uint32_t r[32];
+          tmem_ld32_issue(taddr + c0, r);
+          tmem_ld_wait(r);
+          const int mm = m - c0;
+#pragma unroll
+          for (int jb = 0; jb < 32; jb += 8) {
+            if (jb >= mm) break;
+            if (conv) {
+              float win[8][3];
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                const float* st = p.conv_state + (size_t)mine[c0 + min(jb + j, mm - 1)] * (p.dconv - 1) * p.De + row;
+#pragma unroll
+                for (int q = 0; q < 3; ++q) win[j][q] = q < p.dconv - 1 ? st[(size_t)q * p.De] : 0.0f;
+              }
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                if (jb + j >= mm) break;
+                const size_t a = mine[c0 + jb + j];
+                // Conv Proj row: H (rounded to the storage type), the conv over the caller's window, and the window moved on
+                const float h = to_f32(__float2bfloat16_rn(__uint_as_float(r[jb + j])));
+                float u = bias;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                  if (q >= p.dconv) break;
+                  u = fmaf(wv[q], q < p.dconv - 1 ? win[j][q < 3 ? q : 2] : h, u);
+                }
+                p.U[a * p.De + row] = __float2bfloat16_rn(silu_fast(u));
+                float* st = p.conv_state + a * (p.dconv - 1) * p.De + row;
+#pragma unroll
+                for (int q = 0; q < 2; ++q)
+                  if (q + 1 < p.dconv - 1) st[(size_t)q * p.De] = win[j][q + 1];
+                st[(size_t)(p.dconv - 2) * p.De] = h;
+              }
+            } else if (row_ok) {
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                if (jb + j >= mm) break;
+                const size_t a = mine[c0 + jb + j];
+                float v = __uint_as_float(r[jb + j]);
+                if (MODE == STEP_IN && p.U != nullptr) v = silu_fast(v);      // Gate Proj row
+                if (MODE == STEP_OUT && p.K == 1) v *= p.gates[a];
+                p.C[a * p.ldc + row] = __float2bfloat16_rn(v);
+              }
+            }
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(tempty_bar(acc));
+        if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+      }
+    }
+    if (!ok && lane == 0) {
+      if (!*abort_flag) { atomicExch(status + kStatCode, ROM_ERR_DEVICE_TIMEOUT); atomicExch(status + kStatWhere, 6); }
+      *abort_flag = 1;
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(2 * TC_N) : "memory");
+  }
+}
+
+// K > 1: H and Z of a token are sums over its slots (ascending), then the conv as above and G = SiLU(Z).  Two channels per thread.
+__global__ void __launch_bounds__(128)
+step_conv(const bf16* __restrict__ XZ, int K, int De, const bf16* __restrict__ w_conv, const float* __restrict__ b_conv,
+          float* __restrict__ conv_state, int dconv, bf16* __restrict__ U, bf16* __restrict__ Zs) {
+  const int c = (blockIdx.x * blockDim.x + threadIdx.x) * 2;
+  const size_t b = blockIdx.y;
+  const bool in = c < De;
+  float* st = conv_state + b * (size_t)(dconv - 1) * De + c;
+  float2 win[3], w[4], u = make_float2(0.0f, 0.0f);
+  if (in) {                                          // the window and the taps do not depend on the launch before
+    if (b_conv) u = *reinterpret_cast<const float2*>(b_conv + c);
+    for (int q = 0; q < dconv - 1; ++q) win[q] = *reinterpret_cast<const float2*>(st + (size_t)q * De);
+    for (int q = 0; q < dconv; ++q) w[q] = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(w_conv + (size_t)q * De + c));
+  }
+  pdl_wait();
+  pdl_trigger();
+  if (!in) return;
+  float2 h = make_float2(0.0f, 0.0f), z = h;
+  for (int k = 0; k < K; ++k) {
+    const bf16* r = XZ + (b * K + k) * (size_t)(2 * De) + c;
+    const float2 hv = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(r)), zv = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(r + De));
+    h.x += hv.x; h.y += hv.y; z.x += zv.x; z.y += zv.y;
+  }
+  for (int q = 0; q < dconv; ++q) {
+    const float2 hv = q < dconv - 1 ? win[q] : h;
+    u.x = fmaf(w[q].x, hv.x, u.x); u.y = fmaf(w[q].y, hv.y, u.y);
+  }
+  *reinterpret_cast<__nv_bfloat162*>(U + b * De + c) = __floats2bfloat162_rn(silu_fast(u.x), silu_fast(u.y));
+  *reinterpret_cast<__nv_bfloat162*>(Zs + b * De + c) = __floats2bfloat162_rn(silu_fast(z.x), silu_fast(z.y));
+  for (int q = 0; q + 1 < dconv - 1; ++q) *reinterpret_cast<float2*>(st + (size_t)q * De) = win[q + 1];
+  *reinterpret_cast<float2*>(st + (size_t)(dconv - 2) * De) = h;
+}
+
+// ---------------------------------------------------------------------------------------------- dt Proj + recurrence
+// A warp takes 16 channels x 8 tokens: Delta by MMA, then one (channel half, token) at a time with four lanes per channel (four
+// states each), so that states move as whole 512-byte rows.  The states (the traffic that counts: 8 KB in and out per warp), A and
+// the dt weights are requested before the wait.
+template <bool ZOH>
+__global__ void __launch_bounds__(128)
+step_dt_scan(const bf16* __restrict__ delta_r, const bf16* __restrict__ W_dt, const float* __restrict__ b_dt, int R,
+             const float* __restrict__ A, const float* __restrict__ Bm, const float* __restrict__ Cm, const float* __restrict__ D,
+             const bf16* __restrict__ U, const bf16* __restrict__ Z, int ldz, float* __restrict__ ssm_state, bf16* __restrict__ Yg, int B, int De) {
+  __shared__ float dls[4][8][17], ys[4][8][17];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t4 = lane & 3;
+  const int c0 = (blockIdx.x * 4 + warp) * 16;
+  const int tb = blockIdx.y * 8, nt = min(8, B - tb);
+  const uint4 zero4 = make_uint4(0, 0, 0, 0);
+  float4* hp = reinterpret_cast<float4*>(ssm_state) + ((size_t)tb * De + c0 + g) * 4 + t4;      // token tl, half hf: + (tl De + 8 hf) 4
+  float4 h[8][2];
+#pragma unroll
+  for (int tl = 0; tl < 8; ++tl)
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) h[tl][hf] = tl < nt ? hp[((size_t)tl * De + 8 * hf) * 4] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  uint4 wq[4][2];                                    // the first 128 columns of the dt weights
+#pragma unroll
+  for (int kb = 0; kb < 4; ++kb) {
+    const bool in = kb * 32 + 8 * t4 < R;
+    wq[kb][0] = in ? ld_stream(W_dt + (size_t)(c0 + g) * R + kb * 32 + 8 * t4) : zero4;
+    wq[kb][1] = in ? ld_stream(W_dt + (size_t)(c0 + g + 8) * R + kb * 32 + 8 * t4) : zero4;
+  }
+  const float4 a0 = __ldg(reinterpret_cast<const float4*>(A + (size_t)(c0 + g) * NST) + t4), a1 = __ldg(reinterpret_cast<const float4*>(A + (size_t)(c0 + 8 + g) * NST) + t4);
+  const float av[2][4] = {{a0.x, a0.y, a0.z, a0.w}, {a1.x, a1.y, a1.z, a1.w}};
+  const float bias[2] = {b_dt ? b_dt[c0 + g] : 0.0f, b_dt ? b_dt[c0 + 8 + g] : 0.0f}, Dc[2] = {D ? D[c0 + g] : 0.0f, D ? D[c0 + 8 + g] : 0.0f};
+  pdl_wait();
+  pdl_trigger();
+  float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  const bool tok_ok = g < nt;
+  const bf16* dr = delta_r + (size_t)(tb + g) * R + 8 * t4;
+#pragma unroll
+  for (int kb = 0; kb < 4; ++kb) {
+    if (kb * 32 >= R) break;
+    mma_block(acc, wq[kb][0], wq[kb][1], (tok_ok && kb * 32 + 8 * t4 < R) ? ld_act(dr + kb * 32) : zero4);
+  }
+  for (int kb = 4; kb * 32 < R; ++kb) {
+    const bool in = kb * 32 + 8 * t4 < R;
+    const uint4 q0 = in ? ld_stream(W_dt + (size_t)(c0 + g) * R + kb * 32 + 8 * t4) : zero4;
+    const uint4 q1 = in ? ld_stream(W_dt + (size_t)(c0 + g + 8) * R + kb * 32 + 8 * t4) : zero4;
+    mma_block(acc, q0, q1, (tok_ok && in) ? ld_act(dr + kb * 32) : zero4);
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) dls[warp][2 * t4 + (j & 1)][g + 8 * (j >> 1)] = softplus_fast(acc[j] + bias[j >> 1]);
+  __syncwarp();
+  float a2[2][4], nk[2][4];
+#pragma unroll
+  for (int hf = 0; hf < 2; ++hf)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { a2[hf][i] = av[hf][i] * kLog2e; nk[hf][i] = -1.0f / av[hf][i]; }
+#pragma unroll
+  for (int tl = 0; tl < 8; ++tl) {
+    if (tl >= nt) break;
+    const size_t t = tb + tl;
+    const float4 b4 = reinterpret_cast<const float4*>(Bm + t * NST)[t4], c4 = reinterpret_cast<const float4*>(Cm + t * NST)[t4];
+    const float bb[4] = {b4.x, b4.y, b4.z, b4.w}, cc[4] = {c4.x, c4.y, c4.z, c4.w};
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+      const int c = c0 + 8 * hf + g;
+      const float uu = to_f32(U[t * De + c]), dl = dls[warp][tl][8 * hf + g];
+      float hv[4] = {h[tl][hf].x, h[tl][hf].y, h[tl][hf].z, h[tl][hf].w};
+      float y = 0.0f;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float a = ex2_ftz(dl * a2[hf][i]);
+        if (ZOH) {
+          const float w = (uu * nk[hf][i]) * bb[i];
+          hv[i] = fmaf(a, hv[i] - w, w);
+        } else {
+          hv[i] = fmaf(a, hv[i], (dl * uu) * bb[i]);
+        }
+        y = fmaf(cc[i], hv[i], y);
+      }
+      hp[((size_t)tl * De + 8 * hf) * 4] = make_float4(hv[0], hv[1], hv[2], hv[3]);
+      y += __shfl_xor_sync(0xffffffffu, y, 1);
+      y += __shfl_xor_sync(0xffffffffu, y, 2);
+      if (t4 == 0) ys[warp][tl][8 * hf + g] = fmaf(Dc[hf], uu, y) * to_f32(Z[t * ldz + c]);
+    }
+  }
+  __syncwarp();
+  if (g < nt) {                                      // lane (token g, channels 4 t4 ..)
+    const float* y4 = &ys[warp][g][4 * t4];
+    __nv_bfloat162 lo = __floats2bfloat162_rn(y4[0], y4[1]), hi = __floats2bfloat162_rn(y4[2], y4[3]);
+    *reinterpret_cast<uint2*>(Yg + (size_t)(tb + g) * De + c0 + 4 * t4) = make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
+  }
+}
+
+// out[t, :] = sum_k gate_k Op[t K + k, :]
+__global__ void __launch_bounds__(128)
+step_combine(const bf16* __restrict__ Op, const float* __restrict__ gates, bf16* __restrict__ out, int Dm, int K) {
+  const int c = (blockIdx.x * blockDim.x + threadIdx.x) * 2;
+  const size_t t = blockIdx.y;
+  pdl_wait();
+  if (c >= Dm) return;
+  float2 acc = make_float2(0.0f, 0.0f);
+  for (int k = 0; k < K; ++k) {
+    const float gk = gates[t * K + k];
+    const float2 v = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(Op + (t * K + k) * (size_t)Dm + c));
+    acc.x = fmaf(gk, v.x, acc.x); acc.y = fmaf(gk, v.y, acc.y);
+  }
+  *reinterpret_cast<__nv_bfloat162*>(out + t * Dm + c) = __floats2bfloat162_rn(acc.x, acc.y);
+}
+
+// Launch that may begin while the kernel before it on the stream drains (it waits in griddepcontrol.wait).
+template <typename... P, typename... Args>
+cudaError_t launch_chained_smem(void (*kern)(P...), dim3 grid, int threads, int smem, cudaStream_t st, bool chained, Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.dynamicSmemBytes = smem;
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = chained ? 1 : 0;
+  count_launch();
+  return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
+template <typename... P, typename... Args>
+cudaError_t launch_chained(void (*kern)(P...), dim3 grid, int threads, cudaStream_t st, bool chained, Args... args) {
+  return launch_chained_smem(kern, grid, threads, 0, st, chained, args...);
+}
+
+template <int MODE>
+cudaError_t launch_step_tc(const StepGemmArgs& a, int num_sms, int32_t* status, cudaStream_t st) {
+  CUtensorMap tw;
+  if (!make_tmap(&tw, a.W, (uint64_t)a.E * a.n_rows, (uint64_t)a.Kd, (uint64_t)a.Kd, 128)) return cudaErrorInvalidValue;
+  cudaError_t e = cudaFuncSetAttribute(step_tc<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
+  if (e != cudaSuccess) return e;
+  return launch_chained_smem(step_tc<MODE>, dim3(num_sms), TC_THREADS, TC_SMEM, st, true, tw, a, status);
+}
+
+template <int MODE, int RT, int WARPS>
+cudaError_t launch_step_gemm(const StepGemmArgs& a, dim3 grid, cudaStream_t st) {
+  return launch_chained(step_gemm<MODE, RT, 1, WARPS>, grid, WARPS * 32, st, true, a);
+}
+
+}  // namespace
+
+bool step_small_applicable(const rom_config& c) {
+  return c.dtype == ROM_BF16 && c.flags == 0 && c.small_proj_experts <= 1 && c.L == 1 && c.B <= kStepMaxTokens && c.B * c.K <= kStepMaxAssign &&
+         c.dt_rank % 16 == 0;
+}
+
+cudaError_t launch_step_small(const rom_config& c, const rom_weights& w, const void* x, float* conv_state, float* ssm_state, void* out,
+                              int32_t* topk_idx_out, float* gates, char* W, const WsLayout& lay, cudaStream_t st) {
+  const int B = c.B, De = c.d_inner, Dm = c.d_model, R = c.dt_rank, K = c.K;
+  int32_t* idx = reinterpret_cast<int32_t*>(W + lay.topk_idx);
+  bf16* XZ = reinterpret_cast<bf16*>(W + lay.XZp);
+  bf16* U = reinterpret_cast<bf16*>(W + lay.U);
+  bf16* Zs = reinterpret_cast<bf16*>(W + lay.Zs);
+  bf16* dr = reinterpret_cast<bf16*>(W + lay.delta_r);
+  bf16* Yg = reinterpret_cast<bf16*>(W + lay.Ygp);
+  bf16* Op = reinterpret_cast<bf16*>(W + lay.Op);
+  float* Bm = reinterpret_cast<float*>(W + lay.Bm);
+  float* Cm = reinterpret_cast<float*>(W + lay.Cm);
+  cudaError_t e = launch_chained(step_route, dim3(B), 256, st, false, (const bf16*)x, (const bf16*)w.W_r, w.b_r, Dm, c.E, K, c.gate_mode, idx, gates,
+                                 topk_idx_out, reinterpret_cast<int32_t*>(W + lay.status));
+  if (e != cudaSuccess) return e;
+  const int slots = B * K < c.E ? B * K : c.E;      // selected experts at most
+  StepGemmArgs a{};
+  a.x = (const bf16*)x; a.ldx = Dm; a.W = (const bf16*)w.W_inz; a.Kd = Dm; a.n_rows = 2 * De;
+  a.idx = idx; a.gates = gates; a.B = B; a.K = K; a.E = c.E; a.C = XZ; a.ldc = 2 * De; a.De = De;
+  if (K == 1) { a.w_conv = (const bf16*)w.w_conv; a.b_conv = w.b_conv; a.conv_state = conv_state; a.dconv = c.d_conv; a.U = U; }
+  // few assignments: latency counts, the register-fed kernel spreads them over more blocks; more: stream the weights
+  int num_sms = 0;
+  if ((e = current_device_sm_count(&num_sms)) != cudaSuccess) return e;
+  int32_t* status = reinterpret_cast<int32_t*>(W + lay.status);
+  const bool stream = B * K >= kStreamMin;
+  if (stream) e = launch_step_tc<STEP_IN>(a, num_sms, status, st);
+  else e = launch_step_gemm<STEP_IN, 2, 8>(a, dim3(2 * De / 32, slots), st);
+  if (e != cudaSuccess) return e;
+  if (K > 1 && (e = launch_chained(step_conv, dim3((De / 2 + 127) / 128, B), 128, st, true, (const bf16*)XZ, K, De, (const bf16*)w.w_conv, w.b_conv, conv_state,
+                                   c.d_conv, U, Zs)) != cudaSuccess) return e;
+  StepGemmArgs ax{};
+  ax.x = U; ax.ldx = De; ax.W = (const bf16*)w.W_x; ax.Kd = De; ax.n_rows = R + 2 * NST; ax.B = B; ax.K = 1; ax.C = dr; ax.ldc = R; ax.Bm = Bm; ax.Cm = Cm; ax.R = R;
+  if ((e = launch_step_gemm<STEP_X, 1, 16>(ax, dim3((R + 2 * NST) / 16, (B + 7) / 8), st)) != cudaSuccess) return e;
+  auto scan = c.disc_mode == 0 ? step_dt_scan<true> : step_dt_scan<false>;
+  if ((e = launch_chained(scan, dim3(De / 64, (B + 7) / 8), 128, st, true, (const bf16*)dr, (const bf16*)w.W_dt, w.b_dt, R, w.A, (const float*)Bm, (const float*)Cm, w.D,
+                          (const bf16*)U, (const bf16*)(K == 1 ? XZ + De : Zs), K == 1 ? 2 * De : De, ssm_state, Yg, B, De)) != cudaSuccess) return e;
+  StepGemmArgs ao{};
+  ao.x = Yg; ao.ldx = De; ao.W = (const bf16*)w.W_out; ao.Kd = De; ao.n_rows = Dm; ao.idx = idx; ao.gates = gates; ao.B = B; ao.K = K; ao.E = c.E;
+  ao.C = K == 1 ? (bf16*)out : Op; ao.ldc = Dm;
+  if (stream) e = launch_step_tc<STEP_OUT>(ao, num_sms, status, st);
+  else e = launch_step_gemm<STEP_OUT, 1, 16>(ao, dim3(Dm / 16, slots), st);
+  if (e != cudaSuccess) return e;
+  if (K > 1) return launch_chained(step_combine, dim3((Dm / 2 + 127) / 128, B), 128, st, true, (const bf16*)Op, (const float*)gates, (bf16*)out, Dm, K);
+  return cudaSuccess;
+}
+
+}  // namespace rom
