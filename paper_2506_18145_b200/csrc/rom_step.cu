@@ -156,6 +156,7 @@ struct StepGemmArgs {
   int De; const bf16* w_conv; const float* b_conv; float* conv_state; int dconv; bf16* U;
   // X
   float* Bm; float* Cm; int R;
+  int tile_rows;                        // step_tc: rows per weight tile
 };
 
 template <int MODE, int RT, int NT, int WARPS>
@@ -297,14 +298,16 @@ step_gemm(const StepGemmArgs p) {
 
 // The same for more assignments, where the weights of most experts are walked and streaming them is all that counts: tcgen05 with
 // the weights as the M = 128 operand and an expert's tokens (16, 32 or 64 columns, at most TC_N per pass) as N.  One persistent CTA
-// per SM takes (expert, 128 weight rows) tiles; warp 0 keeps a ring of operand stages full of weights (128 x 64 by one TMA load),
+// per SM takes (expert, 128 weight rows) tiles; warp 0 keeps a ring of operand stages full of weights (128 x 128 by two TMA loads),
 // warps 6..9 put the tokens' rows beside them (16-byte loads on their indices into the swizzled layout: nothing is permuted in
 // memory, and the TMA unit is left to the weights -- gather4 loads cost it about 28 ns a row, more than the weights of the stage),
 // warp 1 issues the MMAs, warps 2..5 drain the accumulator (lane = weight row, column = token; double-buffered) while the next tile
 // streams.  The register-fed kernel above reached 3.6 TB/s at 64 tokens (268 MB in 74 us), waiting on its own sums and output ops.
 constexpr int TC_N = 64;                             // token columns per pass
-constexpr int TC_A_BYTES = 128 * BLOCK_K * 2, TC_STAGE = TC_A_BYTES + TC_N * BLOCK_K * 2;
-constexpr int TC_STAGES = 8;
+constexpr int TC_W_HALF = 128 * BLOCK_K * 2, TC_X_HALF = TC_N * BLOCK_K * 2;      // a stage: two 64-wide K blocks of both operands
+constexpr int TC_A_BYTES = 2 * TC_W_HALF, TC_STAGE = TC_A_BYTES + 2 * TC_X_HALF;
+constexpr int TC_STAGES = 4;
+constexpr int TC_X_FLIGHT = 2;                       // stages of token rows in flight (at most TC_STAGES - 2)
 constexpr int TC_SMEM = TC_STAGES * TC_STAGE + 1024;
 constexpr int TC_THREADS = 320;
 
@@ -360,9 +363,12 @@ step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_
     list[at] = (short)a; tok[at] = (short)(a / p.K);
   }
   __syncthreads();
-  const int tpe = (p.n_rows + 127) / 128;            // weight tiles per expert
+  const int tpe = (p.n_rows + p.tile_rows - 1) / p.tile_rows;      // weight tiles per expert
   const int total = n_act_s * tpe;
-  const int num_kb = p.Kd / BLOCK_K;
+  const int num_kb = (p.Kd + 2 * BLOCK_K - 1) / (2 * BLOCK_K);      // stages of 128; d_model may leave half of the last one
+  // every CTA starts at its own K block: in step they would all read the same 128-byte column of rows that are a power of two apart
+  const int rot = (blockIdx.x * 5) % num_kb;
+  auto k_of = [&](int kb) { return (kb + rot < num_kb ? kb + rot : kb + rot - num_kb) * 2 * BLOCK_K; };
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer of the weights (nothing here depends on the launch before)
@@ -370,12 +376,14 @@ step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_
     int stage = 0, issued = 0; uint32_t phase = 0;
     bool ok = true;
     for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
-      const int e = act[w / tpe], tile = w % tpe;
+      const int e = act[w / tpe], row = e * p.n_rows + (w % tpe) * p.tile_rows;
       for (int n0 = 0; n0 < cnt[e] && ok; n0 += TC_N)
         for (int kb = 0; kb < num_kb; ++kb) {
           if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, WAIT_LIMIT)) { ok = false; break; }
-          mbar_expect_tx(full_bar(stage), TC_A_BYTES);
-          tma_load_2d(base + stage * TC_STAGE, &tmap_w, full_bar(stage), kb * BLOCK_K, e * p.n_rows + tile * 128);
+          const int k0 = k_of(kb);
+          mbar_expect_tx(full_bar(stage), 2 * p.tile_rows * BLOCK_K * 2);
+          tma_load_2d(base + stage * TC_STAGE, &tmap_w, full_bar(stage), k0, row);
+          tma_load_2d(base + stage * TC_STAGE + TC_W_HALF, &tmap_w, full_bar(stage), k0 + BLOCK_K, row);
           ++issued;
           if (++stage == TC_STAGES) { stage = 0; phase ^= 1u; }
         }
@@ -408,10 +416,14 @@ step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_
           for (int kb = 0; kb < num_kb; ++kb) {
             if (!mbar_wait(full_bar(stage), phase, abort_flag, WAIT_LIMIT)) { ok = false; break; }
             tc_fence_after();
-            const uint64_t adesc = make_smem_desc(base + stage * TC_STAGE), bdesc = make_smem_desc(base + stage * TC_STAGE + TC_A_BYTES);
+            const int halves = k_of(kb) + BLOCK_K < p.Kd ? 2 : 1;
+            for (int hf = 0; hf < halves; ++hf) {
+              const uint64_t adesc = make_smem_desc(base + stage * TC_STAGE + hf * TC_W_HALF);
+              const uint64_t bdesc = make_smem_desc(base + stage * TC_STAGE + TC_A_BYTES + hf * TC_X_HALF);
 #pragma unroll
-            for (int k = 0; k < BLOCK_K / UMMA_K; ++k)
-              umma_bf16(tmem_base + acc * TC_N, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc, (kb | k) != 0 ? 1u : 0u);
+              for (int k = 0; k < BLOCK_K / UMMA_K; ++k)
+                umma_bf16(tmem_base + acc * TC_N, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc, (kb | hf | k) != 0 ? 1u : 0u);
+            }
             umma_commit(empty_bar(stage));
             issued_any = true;
             if (++stage == TC_STAGES) { stage = 0; phase ^= 1u; }
@@ -435,8 +447,15 @@ step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_
     // ---------------------------------------------------------------- token rows of every stage: 128 threads, 16-byte pieces
     const int l = tid - 6 * 32, lrow = l >> 3, chunk = l & 7;
     if (MODE == STEP_OUT) { pdl_wait(); pdl_trigger(); }
-    int stage = 0; uint32_t phase = 0;
+    int stage = 0, pub = 0, pending = 0; uint32_t phase = 0;
     bool ok = true;
+    auto publish = [&]() {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(full_bar(pub));
+      if (++pub == TC_STAGES) pub = 0;
+      --pending;
+    };
     for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
       const int e = act[w / tpe];
       for (int n0 = 0; n0 < cnt[e] && ok; n0 += TC_N) {
@@ -444,41 +463,30 @@ step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_
         const bf16* src[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) src[q] = p.x + (size_t)tok[off[e] + n0 + min(lrow + 16 * q, m - 1)] * p.ldx + chunk * 8;      // (rows past the last token repeat it)
-        const int kpc = 4 / nq, n_ch = (num_kb + kpc - 1) / kpc;      // four pieces in flight per thread while four are stored
-        uint4 cur[4], nxt[4];
-        auto fetch = [&](int ch, uint4 (&d)[4]) {
+        for (int kb = 0; kb < num_kb; ++kb) {
+          ok = __all_sync(0xffffffffu, mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, WAIT_LIMIT));
+          if (!ok) break;
+          const uint32_t dst = base + stage * TC_STAGE + TC_A_BYTES + lrow * 128 + ((chunk ^ (lrow & 7)) << 4);
+          const int k0 = k_of(kb);
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int kb = min(ch * kpc + i / nq, num_kb - 1);
-            const bf16* sp = nq == 1 ? src[0] : nq == 2 ? src[i & 1] : src[i];
-            d[i] = ld_act(sp + kb * BLOCK_K);
-          }
-        };
-        fetch(0, cur);
-        for (int ch = 0; ch < n_ch && ok; ++ch) {
-          if (ch + 1 < n_ch) fetch(ch + 1, nxt);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int kb = ch * kpc + i / nq, q = nq == 1 ? 0 : nq == 2 ? (i & 1) : i;
-            if (kb >= num_kb) break;
-            if (q == 0) {
-              ok = __all_sync(0xffffffffu, mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, WAIT_LIMIT));
-              if (!ok) break;
+          for (int q = 0; q < 4; ++q)
+            if (q < nq) {
+              asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + q * 16 * 128), "l"(src[q] + k0) : "memory");
+              if (k0 + BLOCK_K < p.Kd)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + TC_X_HALF + q * 16 * 128), "l"(src[q] + k0 + BLOCK_K) : "memory");
             }
-            const int r = lrow + 16 * q;
-            *reinterpret_cast<uint4*>(smem_raw + (base - smem_u32(smem_raw)) + stage * TC_STAGE + TC_A_BYTES + r * 128 + ((chunk ^ (r & 7)) << 4)) = cur[i];
-            if (q == nq - 1) {
-              asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-              __syncwarp();
-              if (lane == 0) mbar_arrive(full_bar(stage));
-              if (++stage == TC_STAGES) { stage = 0; phase ^= 1u; }
-            }
+          asm volatile("cp.async.commit_group;" ::: "memory");
+          if (++stage == TC_STAGES) { stage = 0; phase ^= 1u; }
+          // the stage of TC_X_FLIGHT copies ago has landed: publish it to the tensor cores
+          if (++pending > TC_X_FLIGHT) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(TC_X_FLIGHT) : "memory");
+            publish();
           }
-#pragma unroll
-          for (int i = 0; i < 4; ++i) cur[i] = nxt[i];
         }
       }
     }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    while (pending > 0) publish();
     if (!ok && lane == 0) {
       if (!*abort_flag) { atomicExch(status + kStatCode, ROM_ERR_DEVICE_TIMEOUT); atomicExch(status + kStatWhere, 7); }
       *abort_flag = 1;
@@ -489,9 +497,9 @@ step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_
     int acc = 0; uint32_t acc_phase = 0;
     bool ok = true;
     for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
-      const int e = act[w / tpe], row = (w % tpe) * 128 + quarter * 32 + lane;
-      const bool row_ok = row < p.n_rows;
-      const bool conv = MODE == STEP_IN && p.U != nullptr && row < p.De;      // warp-uniform: De is a multiple of 32
+      const int e = act[w / tpe], r = quarter * 32 + lane, row = (w % tpe) * p.tile_rows + r;
+      const bool row_ok = r < p.tile_rows && row < p.n_rows;      // (rows of the stage beyond the tile keep what they hold)
+      const bool conv = MODE == STEP_IN && p.U != nullptr && row < p.De && row_ok;
       float wv[4], bias = 0.0f;
       if (conv) {
         if (p.b_conv) bias = p.b_conv[row];
@@ -609,7 +617,7 @@ step_conv(const bf16* __restrict__ XZ, int K, int De, const bf16* __restrict__ w
 // states each), so that states move as whole 512-byte rows.  The states (the traffic that counts: 8 KB in and out per warp), A and
 // the dt weights are requested before the wait.
 template <bool ZOH>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, 4)
 step_dt_scan(const bf16* __restrict__ delta_r, const bf16* __restrict__ W_dt, const float* __restrict__ b_dt, int R,
              const float* __restrict__ A, const float* __restrict__ Bm, const float* __restrict__ Cm, const float* __restrict__ D,
              const bf16* __restrict__ U, const bf16* __restrict__ Z, int ldz, float* __restrict__ ssm_state, bf16* __restrict__ Yg, int B, int De) {
@@ -736,10 +744,22 @@ cudaError_t launch_chained(void (*kern)(P...), dim3 grid, int threads, cudaStrea
 template <int MODE>
 cudaError_t launch_step_tc(const StepGemmArgs& a, int num_sms, int32_t* status, cudaStream_t st) {
   CUtensorMap tw;
-  if (!make_tmap(&tw, a.W, (uint64_t)a.E * a.n_rows, (uint64_t)a.Kd, (uint64_t)a.Kd, 128)) return cudaErrorInvalidValue;
+  if (!make_tmap(&tw, a.W, (uint64_t)a.E * a.n_rows, (uint64_t)a.Kd, (uint64_t)a.Kd, a.tile_rows)) return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(step_tc<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
   if (e != cudaSuccess) return e;
   return launch_chained_smem(step_tc<MODE>, dim3(num_sms), TC_THREADS, TC_SMEM, st, true, tw, a, status);
+}
+
+// Rows per weight tile: the multiple of 16 in 96 .. 128 for which the CTAs' rounds x rows is smallest when every expert that can be
+// selected is (d_model 2048, 8 experts: 112 rows make the in_proj 4.0 rounds of tiles, where 128 need 4 rounds for 3.46).
+int pick_tile_rows(int slots, int n_rows, int num_sms) {
+  int best = 128;
+  long long cost = -1;
+  for (int h = 128; h >= 96; h -= 16) {
+    const long long tiles = (long long)slots * ((n_rows + h - 1) / h), c = (tiles + num_sms - 1) / num_sms * h;
+    if (cost < 0 || c < cost) { cost = c; best = h; }
+  }
+  return best;
 }
 
 template <int MODE, int RT, int WARPS>
@@ -779,13 +799,14 @@ cudaError_t launch_step_small(const rom_config& c, const rom_weights& w, const v
   if ((e = current_device_sm_count(&num_sms)) != cudaSuccess) return e;
   int32_t* status = reinterpret_cast<int32_t*>(W + lay.status);
   const bool stream = B * K >= kStreamMin;
+  a.tile_rows = pick_tile_rows(slots, 2 * De, num_sms);
   if (stream) e = launch_step_tc<STEP_IN>(a, num_sms, status, st);
   else e = launch_step_gemm<STEP_IN, 2, 8>(a, dim3(2 * De / 32, slots), st);
   if (e != cudaSuccess) return e;
   if (K > 1 && (e = launch_chained(step_conv, dim3((De / 2 + 127) / 128, B), 128, st, true, (const bf16*)XZ, K, De, (const bf16*)w.w_conv, w.b_conv, conv_state,
                                    c.d_conv, U, Zs)) != cudaSuccess) return e;
   StepGemmArgs ax{};
-  ax.x = U; ax.ldx = De; ax.W = (const bf16*)w.W_x; ax.Kd = De; ax.n_rows = R + 2 * NST; ax.B = B; ax.K = 1; ax.C = dr; ax.ldc = R; ax.Bm = Bm; ax.Cm = Cm; ax.R = R;
+  ax.x = U; ax.ldx = De; ax.W = (const bf16*)w.W_x; ax.Kd = De; ax.n_rows = R + 2 * NST; ax.B = B; ax.K = K; ax.C = dr; ax.ldc = R; ax.Bm = Bm; ax.Cm = Cm; ax.R = R;
   if ((e = launch_step_gemm<STEP_X, 1, 16>(ax, dim3((R + 2 * NST) / 16, (B + 7) / 8), st)) != cudaSuccess) return e;
   auto scan = c.disc_mode == 0 ? step_dt_scan<true> : step_dt_scan<false>;
   if ((e = launch_chained(scan, dim3(De / 64, (B + 7) / 8), 128, st, true, (const bf16*)dr, (const bf16*)w.W_dt, w.b_dt, R, w.A, (const float*)Bm, (const float*)Cm, w.D,
@@ -793,6 +814,7 @@ cudaError_t launch_step_small(const rom_config& c, const rom_weights& w, const v
   StepGemmArgs ao{};
   ao.x = Yg; ao.ldx = De; ao.W = (const bf16*)w.W_out; ao.Kd = De; ao.n_rows = Dm; ao.idx = idx; ao.gates = gates; ao.B = B; ao.K = K; ao.E = c.E;
   ao.C = K == 1 ? (bf16*)out : Op; ao.ldc = Dm;
+  ao.tile_rows = pick_tile_rows(slots, Dm, num_sms);
   if (stream) e = launch_step_tc<STEP_OUT>(ao, num_sms, status, st);
   else e = launch_step_gemm<STEP_OUT, 1, 16>(ao, dim3(Dm / 16, slots), st);
   if (e != cudaSuccess) return e;
