@@ -197,6 +197,13 @@ cudaError_t launch_scan(const rom_config& c, const void* u, const void* delta, b
                         bool scalar_A = false /* A[c, :] constant per channel and disc_mode 1: one exponential per channel and step */,
                         float* ckpt = nullptr /* also store the state at the start of every kScanCkpt steps, [B, ceil(L / kScanCkpt), De, 16] */);
 
+// Scalar-decay recurrence of the Mamba2-style block as chunked matrix products (rom_ssd.cu): bf16, 64 channels per head.  zx: the
+// projection rows [T, W] (gate pre-activation in column 0.., dt pre-activation of head h in column dt_col + h); y: gated rows [T, De].
+bool ssd_applicable(const rom_config& c, int headdim);
+size_t ssd_ws_floats(const rom_config& c);
+cudaError_t launch_ssd(const rom_config& c, const void* xc, const float* Bm, const float* Cm, const void* zx, int W, int dt_col, const float* dt_bias,
+                       const float* A, const float* D, void* y, float* ws, cudaStream_t st);
+
 // One-pass scan for few long sequences (rom_scan_seq.cu): every exponential evaluated once, no workspace.  bf16 storage only.
 bool scan_seq_applicable(const rom_config& c, const void* u, const void* delta, bool delta_fp32, const float* Bm, const float* Cm,
                          const void* z, int ldz, const int32_t* z_row, const int32_t* y_rows, bool gate_activated, int num_sms);

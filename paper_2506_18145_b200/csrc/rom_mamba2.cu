@@ -53,13 +53,14 @@ M2Layout make_m2_layout(const rom_config& c, int headdim) {
   m.xc = take(esz * T * De);
   m.Bm = take(4 * T * N);
   m.Cm = take(4 * T * N);
-  m.D32 = take(4 * T * De);
-  m.A_exp = take(4 * De * N);
-  m.D_exp = take(4 * De);
+  const bool ssd = ssd_applicable(c, headdim);      // no per-channel expansion of dt, A, D
+  m.D32 = take(ssd ? 0 : 4 * T * De);
+  m.A_exp = take(ssd ? 0 : 4 * De * N);
+  m.D_exp = take(ssd ? 0 : 4 * De);
   m.Yt = take(esz * T * De);
   m.Ygp = take(esz * rows * De);
   m.Op = take(esz * rows * c.d_model);
-  m.scan_ws = take(sizeof(float) * scan_ws_floats(c.B, c.d_inner, c.L));
+  m.scan_ws = take(sizeof(float) * (ssd ? ssd_ws_floats(c) : scan_ws_floats(c.B, c.d_inner, c.L)));
   m.total = o;
   l.total = o;
   return m;
@@ -159,11 +160,65 @@ m2_dt_kernel(const T* __restrict__ ZXs, const float* __restrict__ dt_bias, const
   *reinterpret_cast<float4*>(D32 + tok * De + c) = make_float4(v, v, v, v);
 }
 
-// y^ = g / sqrt(mean g^2 + eps) * w_norm with g = the gated scan output of the token (one block per token, 16-byte
-// accesses), written to the K expert-order rows of the token.
-template <typename T>
+// y^ = g / sqrt(mean g^2 + eps) * w_norm with g = the gated scan output of the token, written to the K expert-order rows of the
+// token.  A block takes M2_NT tokens in turn with the row and the norm weight in registers (NV 16-byte vectors per thread): one
+// read and K writes of a row, the weight (16 KB at 4096 channels, more than the row) once per M2_NT rows.
+constexpr int M2_NT = 8;
+template <typename T, int NV>
 __global__ void __launch_bounds__(256)
 m2_norm_kernel(const T* __restrict__ Yt, const float* __restrict__ w_norm, const int32_t* __restrict__ row_of_assign, T* __restrict__ Ygp,
+               int De, int K, float eps, long long Tn) {
+  constexpr int V = V16<T>::N;
+  __shared__ float red[2][8];
+  const int nvec = De / V, tid = threadIdx.x;
+  const long long t0 = (long long)blockIdx.x * M2_NT, t1 = min(t0 + M2_NT, Tn);
+  float w[NV][V];
+#pragma unroll
+  for (int j = 0; j < NV; ++j)
+#pragma unroll
+    for (int i = 0; i < V; ++i) w[j][i] = j * 256 + tid < nvec ? w_norm[(size_t)(j * 256 + tid) * V + i] : 0.0f;
+  V16<T> q[NV], nx[NV];
+  auto fetch = [&](long long t) {
+#pragma unroll
+    for (int j = 0; j < NV; ++j)
+      if (j * 256 + tid < nvec) nx[j].load(Yt + t * De + (size_t)(j * 256 + tid) * V); else nx[j].zero();
+  };
+  fetch(t0);
+  for (long long t = t0; t < t1; ++t) {
+    const int buf = (int)(t & 1);
+    float ss = 0.0f;
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      q[j] = nx[j];
+      float v[V];
+      q[j].get(v);
+#pragma unroll
+      for (int i = 0; i < V; ++i) ss = fmaf(v[i], v[i], ss);
+    }
+    if (t + 1 < t1) fetch(t + 1);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    if ((tid & 31) == 0) red[buf][tid >> 5] = ss;
+    __syncthreads();                                 // (two buffers: a warp is never more than one token ahead)
+    float tot = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) tot += red[buf][i];
+    const float r = rsqrtf(tot / (float)De + eps);
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      if (j * 256 + tid >= nvec) continue;
+      float v[V];
+      q[j].get(v);
+#pragma unroll
+      for (int i = 0; i < V; ++i) v[i] = v[i] * r * w[j][i];
+      for (int k = 0; k < K; ++k) V16<T>::store(Ygp + (size_t)row_of_assign[t * K + k] * De + (size_t)(j * 256 + tid) * V, v);
+    }
+  }
+}
+// Rows too wide for the registers of a block: one token per block, the row read twice.
+template <typename T>
+__global__ void __launch_bounds__(256)
+m2_norm_wide_kernel(const T* __restrict__ Yt, const float* __restrict__ w_norm, const int32_t* __restrict__ row_of_assign, T* __restrict__ Ygp,
                int De, int K, float eps) {
   constexpr int V = V16<T>::N;
   __shared__ float red[8];
@@ -191,6 +246,20 @@ m2_norm_kernel(const T* __restrict__ Yt, const float* __restrict__ w_norm, const
     for (int j = 0; j < V; ++j) v[j] = to_f32(from_f32<T>(v[j] * r * w_norm[(size_t)i * V + j]));
     for (int k = 0; k < K; ++k) V16<T>::store(Ygp + (size_t)row_of_assign[t * K + k] * De + (size_t)i * V, v);
   }
+}
+
+template <typename T>
+cudaError_t launch_norm(const void* Yt, const float* w_norm, const int32_t* rows, void* Ygp, int De, int K, long long Tn, cudaStream_t st) {
+  const int nv = (De / V16<T>::N + 255) / 256;
+  auto go = [&](auto kern) { kern<<<(unsigned)((Tn + M2_NT - 1) / M2_NT), 256, 0, st>>>((const T*)Yt, w_norm, rows, (T*)Ygp, De, K, 1e-5f, Tn); };
+  if (nv <= 1) go(m2_norm_kernel<T, 1>);
+  else if (nv <= 2) go(m2_norm_kernel<T, 2>);
+  else if (nv <= 4) go(m2_norm_kernel<T, 4>);
+  else if (nv <= 8) go(m2_norm_kernel<T, 8>);
+  else if (nv <= 16) go(m2_norm_kernel<T, 16>);
+  else m2_norm_wide_kernel<T><<<(unsigned)Tn, 256, 0, st>>>((const T*)Yt, w_norm, rows, (T*)Ygp, De, K, 1e-5f);
+  count_launch();
+  return cudaGetLastError();
 }
 
 #define ROM_CUDA(expr)                            \
@@ -273,6 +342,9 @@ int rom_mamba2_layer_forward(const rom_config* cfg, int32_t headdim, const rom_m
                                                     c.L, De, N, Wd, c.d_conv);
     count_launch();
     ROM_CUDA(cudaGetLastError());
+    if (ssd_applicable(c, headdim)) {
+      ROM_CUDA(launch_ssd(c, W + m.xc, Bm, Cm, W + m.ZXs, Wd, 2 * De + 2 * N, w->dt_bias, w->A, w->D, W + m.Yt, reinterpret_cast<float*>(W + m.scan_ws), st));
+    } else {
     const long long total2 = max((long long)T * (De / 4), (long long)De);
     const unsigned blocks2 = (unsigned)((total2 + 255) / 256);
     float* D32 = reinterpret_cast<float*>(W + m.D32);
@@ -288,12 +360,11 @@ int rom_mamba2_layer_forward(const rom_config* cfg, int32_t headdim, const rom_m
     cs.disc_mode = 1;
     ROM_CUDA(launch_scan(cs, W + m.xc, D32, true, A_exp, Bm, Cm, w->D ? D_exp : nullptr, W + m.ZXs, Wd, nullptr, nullptr, W + m.Yt, nullptr,
                          nullptr, 1, reinterpret_cast<float*>(W + m.scan_ws), false, st, true));
+    }
   }
   // gated RMS norm, rows written in expert order
-  if (bf) m2_norm_kernel<__nv_bfloat16><<<T, 256, 0, st>>>((const __nv_bfloat16*)(W + m.Yt), w->w_norm, row_of_assign, (__nv_bfloat16*)(W + m.Ygp), De, c.K, 1e-5f);
-  else m2_norm_kernel<float><<<T, 256, 0, st>>>((const float*)(W + m.Yt), w->w_norm, row_of_assign, (float*)(W + m.Ygp), De, c.K, 1e-5f);
-  count_launch();
-  ROM_CUDA(cudaGetLastError());
+  ROM_CUDA(bf ? launch_norm<__nv_bfloat16>(W + m.Yt, w->w_norm, row_of_assign, W + m.Ygp, De, c.K, T, st)
+              : launch_norm<float>(W + m.Yt, w->w_norm, row_of_assign, W + m.Ygp, De, c.K, T, st));
   // output projection of the selected experts and the gate-weighted sum
   if (tc && c.K == 1) {
     Epilogue e_out{EPI_OUTPROJ, out, Dm, nullptr, nullptr, nullptr, 0, 0, reinterpret_cast<const int32_t*>(W + lay.assign_of_row), gates};
