@@ -319,7 +319,8 @@ int layer_forward_impl(const rom_config* cfg, const rom_weights* w, const void* 
     if (!te && M_max <= 128 && Kd >= 1024 && Kd % 2048 == 0 && ep.mode == EPI_XPROJ)
       return launch_gemm_skinny(c.dtype, A_, lda, B_, ldb, M_max, Nn, Kd, ep, st);
     if (tc) return launch_gemm_tc(A_, lda, B_, ldb, n_experts, M_max, Nn, Kd, te, nmt, ep, status, st,
-                                  (c.flags & ROM_FLAG_TEST_STALL) != 0 && (ep.mode == EPI_INPROJ || (ep.mode == EPI_STORE && Nn == 2 * De)));
+                                  (c.flags & ROM_FLAG_TEST_STALL) != 0 && (ep.mode == EPI_INPROJ || (ep.mode == EPI_STORE && Nn == 2 * De)), false,
+                                  te ? reinterpret_cast<const int32_t*>(W + lay.pad_offsets) : nullptr);
     return launch_gemm_simt(c.dtype, A_, lda, B_, ldb, bstride, M_max, Nn, Kd, te, nmt, ep, st);
   };
 
@@ -505,7 +506,7 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
   float* Cm = reinterpret_cast<float*>(W + lay.Cm);
   auto gemm = [&](const void* A_, int lda, const void* B_, int ldb, int n_experts, int64_t bstride, int M_max, int Nn, int Kd,
                   const int32_t* te, const int32_t* nmt, const Epilogue& ep) -> cudaError_t {
-    if (tc) return launch_gemm_tc(A_, lda, B_, ldb, n_experts, M_max, Nn, Kd, te, nmt, ep, status, st);
+    if (tc) return launch_gemm_tc(A_, lda, B_, ldb, n_experts, M_max, Nn, Kd, te, nmt, ep, status, st, false, false, te ? pad_offsets : nullptr);
     return launch_gemm_simt(c.dtype, A_, lda, B_, ldb, bstride, M_max, Nn, Kd, te, nmt, ep, st);
   };
   auto store_to = [&](void* C_, int ldc) { return Epilogue{EPI_STORE, C_, ldc, nullptr, nullptr, nullptr, 0, 0, nullptr, nullptr}; };
@@ -513,7 +514,7 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
   // plain-FMA kernels take a transposed copy
   auto gemm_dgrad = [&](const void* A_, int lda, const void* Wt, int n_experts, int M_max, int Nn, int Kd, const int32_t* te, const int32_t* nmt,
                         void* scratch, const Epilogue& ep) -> cudaError_t {
-    if (tc) return launch_gemm_tc(A_, lda, Wt, Nn, n_experts, M_max, Nn, Kd, te, nmt, ep, status, st, false, true);
+    if (tc) return launch_gemm_tc(A_, lda, Wt, Nn, n_experts, M_max, Nn, Kd, te, nmt, ep, status, st, false, true, te ? pad_offsets : nullptr);
     const cudaError_t e = launch_transpose(c.dtype, Wt, scratch, n_experts, Kd, Nn, st);
     if (e != cudaSuccess) return e;
     return launch_gemm_simt(c.dtype, A_, lda, scratch, Kd, (int64_t)Nn * Kd, M_max, Nn, Kd, te, nmt, ep, st);

@@ -112,6 +112,7 @@ int rom_ffn_moe_forward(const rom_config* cfg, int32_t d_ff, const void* W_gu, c
   int32_t* status = reinterpret_cast<int32_t*>(W + lay.status);
   const int32_t* tile_expert = reinterpret_cast<const int32_t*>(W + lay.tile_expert);
   const int32_t* num_m_tiles = reinterpret_cast<const int32_t*>(W + lay.num_m_tiles);
+  const int32_t* pad_offsets = reinterpret_cast<const int32_t*>(W + lay.pad_offsets);
   const int32_t* row_of_assign = reinterpret_cast<const int32_t*>(W + lay.row_of_assign);
   const int32_t* assign_of_row = reinterpret_cast<const int32_t*>(W + lay.assign_of_row);
 
@@ -122,15 +123,15 @@ int rom_ffn_moe_forward(const rom_config* cfg, int32_t d_ff, const void* W_gu, c
   if (tc) {
     // [gate | up] projection; the output op forms SiLU(gate) * up from the accumulator, nothing wider is stored
     Epilogue e_up{EPI_SWIGLU, W + lay.Ygp, d_ff, nullptr, nullptr, nullptr, d_ff, 0, nullptr, nullptr};
-    ROM_CUDA(launch_gemm_tc(W + lay.x_perm, Dm, W_gu, Dm, c.E, (int)lay.rows_max, d_ff, Dm, tile_expert, num_m_tiles, e_up, status, st));
+    ROM_CUDA(launch_gemm_tc(W + lay.x_perm, Dm, W_gu, Dm, c.E, (int)lay.rows_max, d_ff, Dm, tile_expert, num_m_tiles, e_up, status, st, false, false, pad_offsets));
     if (c.K == 1) {
       // down projection: rows scaled by their gate and written at their token's position
       Epilogue e_dn{EPI_OUTPROJ, out, Dm, nullptr, nullptr, nullptr, 0, 0, assign_of_row, gates};
-      ROM_CUDA(launch_gemm_tc(W + lay.Ygp, d_ff, W_down, d_ff, c.E, (int)lay.rows_max, Dm, d_ff, tile_expert, num_m_tiles, e_dn, status, st));
+      ROM_CUDA(launch_gemm_tc(W + lay.Ygp, d_ff, W_down, d_ff, c.E, (int)lay.rows_max, Dm, d_ff, tile_expert, num_m_tiles, e_dn, status, st, false, false, pad_offsets));
       return ROM_OK;
     }
     Epilogue e_dn{EPI_STORE, W + lay.Op, Dm, nullptr, nullptr, nullptr, 0, 0, nullptr, nullptr};
-    ROM_CUDA(launch_gemm_tc(W + lay.Ygp, d_ff, W_down, d_ff, c.E, (int)lay.rows_max, Dm, d_ff, tile_expert, num_m_tiles, e_dn, status, st));
+    ROM_CUDA(launch_gemm_tc(W + lay.Ygp, d_ff, W_down, d_ff, c.E, (int)lay.rows_max, Dm, d_ff, tile_expert, num_m_tiles, e_dn, status, st, false, false, pad_offsets));
   } else {
     Epilogue e_up{EPI_STORE, W + lay.XZp, 2 * d_ff, nullptr, nullptr, nullptr, 0, 0, nullptr, nullptr};
     ROM_CUDA(launch_gemm_simt(c.dtype, W + lay.x_perm, Dm, W_gu, Dm, (int64_t)2 * d_ff * Dm, (int)lay.rows_max, 2 * d_ff, Dm,

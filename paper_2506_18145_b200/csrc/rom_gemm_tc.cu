@@ -34,7 +34,6 @@ constexpr int STAGE_BYTES = A_STAGE_BYTES + B_STAGE_BYTES;
 constexpr int ACC_STAGES = 2;
 constexpr int TMEM_COLS = 512;
 constexpr int NUM_EPI_WARPS = NUM_EPI_WARPS_C;
-constexpr int NUM_THREADS = 64 + 32 * NUM_EPI_WARPS;
 // The dt Proj (softplus output ops) has two K blocks per tile and about ten instructions plus two special-function
 // operations per output element: its time is its epilogue's, so it runs sixteen epilogue warps instead of eight.
 __host__ __device__ constexpr int epi_warps_of(int mode) { return (mode == EPI_SOFTPLUS || mode == EPI_SOFTPLUS_ROWS) ? 16 : NUM_EPI_WARPS_C; }
@@ -46,13 +45,17 @@ __host__ __device__ constexpr bool f32_out(int mode) { return mode == EPI_SOFTPL
 // The x Proj (a narrow B tile, one wave of row tiles, time set by how many bytes of A are in flight) runs six
 // smaller stages: its B tile is at most XPROJ_BLOCK_N rows.
 constexpr int XPROJ_BLOCK_N = 160;
-__host__ __device__ constexpr int stage_bytes_of(int mode) {
+// CG = 2 (CTA pairs): each CTA stages its own 128 rows of A and its half, 128 rows, of a 256-wide B tile.
+__host__ __device__ constexpr int stage_bytes_of(int mode, int cg = 1) {
+  if (cg == 2) return 2 * A_STAGE_BYTES;
   return mode == EPI_XPROJ ? A_STAGE_BYTES + XPROJ_BLOCK_N * BLOCK_K * 2 : STAGE_BYTES;
 }
-__host__ __device__ constexpr int stages_of(int mode) { return f32_out(mode) ? 3 : mode == EPI_XPROJ ? 6 : MAX_STAGES; }
+__host__ __device__ constexpr int stages_of(int mode, int cg = 1) {
+  return cg == 2 ? (f32_out(mode) ? 5 : 6) : f32_out(mode) ? 3 : mode == EPI_XPROJ ? 6 : MAX_STAGES;
+}
 __host__ __device__ constexpr int out_stage_bytes_of(int mode) { return f32_out(mode) ? epi_warps_of(mode) * 32 * 32 * 4 : 0; }
-__host__ __device__ constexpr int smem_bytes_of(int mode) {
-  return stages_of(mode) * stage_bytes_of(mode) + 1024 /*alignment slack*/ + 256 /*barriers*/ + out_stage_bytes_of(mode);
+__host__ __device__ constexpr int smem_bytes_of(int mode, int cg = 1) {
+  return stages_of(mode, cg) * stage_bytes_of(mode, cg) + 1024 /*alignment slack*/ + 256 /*barriers*/ + out_stage_bytes_of(mode);
 }
 
 // Bias of the 32 columns [n0, n0+32) (EPI_SOFTPLUS only), requested before the accumulator chunk is waited for.
@@ -162,15 +165,16 @@ __device__ __forceinline__ void epi_softplus32(const Epilogue& ep, float* sw, in
   __syncwarp();
 }
 
-template <int MODE>
+template <int MODE, int CG>
 __global__ void __launch_bounds__(threads_of(MODE), 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
                int M_max, int N, int Kd, int block_n, uint32_t idesc,
                const int32_t* __restrict__ tile_expert, const int32_t* __restrict__ num_m_tiles_dev,
                Epilogue ep, int32_t* __restrict__ status, uint32_t wait_limit, int withhold_kb,
-               const int32_t* __restrict__ k_seg, int n_seg, int a_mn, int b_mn) {
-  constexpr int STAGES = stages_of(MODE);
-  constexpr int SB = stage_bytes_of(MODE);          // bytes per operand stage (multiple of 1024)
+               const int32_t* __restrict__ k_seg, int n_seg, int a_mn, int b_mn,
+               const int32_t* __restrict__ pad_offsets, int n_experts) {
+  constexpr int STAGES = stages_of(MODE, CG);
+  constexpr int SB = stage_bytes_of(MODE, CG);      // bytes per operand stage (multiple of 1024)
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;               // 128B-swizzled tiles need 1024-byte alignment
@@ -186,6 +190,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   float* out_stage = reinterpret_cast<float*>(smem + STAGES * SB + 256);        // [8 warps][32][32] (softplus only)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // CTA pairs: the pair shares one 256 x 256 tile; CTA r owns rows [128 r, 128 r + 128) of it and stages half of B.  An expert with
+  // an odd number of 128-row tiles ends in a pair whose second CTA works on a copy of the first one's rows and stores nothing.
+  const uint32_t rank = CG == 2 ? cluster_rank() : 0;
+  const int worker = CG == 2 ? (int)blockIdx.x / 2 : (int)blockIdx.x, n_workers = CG == 2 ? (int)gridDim.x / 2 : (int)gridDim.x;
+  __shared__ int pair_off[CG == 2 ? kMaxE + 1 : 1], tile_off[CG == 2 ? kMaxE + 1 : 1];      // pairs / 128-row tiles before each expert
 
   int num_m_tiles = (M_max + BLOCK_M - 1) / BLOCK_M;
   if (num_m_tiles_dev) num_m_tiles = min(num_m_tiles, *num_m_tiles_dev);
@@ -195,12 +204,25 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   // Weight-gradient mode (k_seg != nullptr): n_seg independent problems share A and B; problem s contracts the K range
   // [k_seg[s], k_seg[s+1]) (multiples of BLOCK_K; an expert's padded row segment) and writes rows [s M_max, (s+1) M_max) of C.
   // Split-K mode (k_seg == nullptr, n_seg > 1): the K range is cut into n_seg equal pieces whose partial sums add up in C.
-  const int seg_tiles = num_m_tiles * n_tiles;
+  if (CG == 2 && pad_offsets) {
+    if (threadIdx.x == 0) {
+      int o = 0;
+      for (int e = 0; e <= n_experts; ++e) {
+        tile_off[e] = pad_offsets[e] / BLOCK_M;
+        pair_off[e] = o;
+        if (e < n_experts) o += ((pad_offsets[e + 1] - pad_offsets[e]) / BLOCK_M + 1) / 2;
+      }
+    }
+    __syncthreads();
+  }
+  const int m_units = CG == 1 ? num_m_tiles : pad_offsets ? pair_off[n_experts] : (num_m_tiles + 1) / 2;
+  const int seg_tiles = m_units * n_tiles;
   const int total_tiles = n_seg * seg_tiles;
   const int num_kb = (Kd + BLOCK_K - 1) / BLOCK_K;
   const int split_kb = (num_kb + n_seg - 1) / n_seg;
-  auto decode = [&](int tile, int& m_tile, int& n_tile, int& seg, int& kb0, int& nkb) {
-    seg = 0; kb0 = 0; nkb = num_kb;
+  // m_tile: this CTA's 128-row tile; own: it exists (false: the missing half of a pair)
+  auto decode = [&](int tile, int& m_tile, int& n_tile, int& seg, int& kb0, int& nkb, bool& own, int& e) {
+    seg = 0; kb0 = 0; nkb = num_kb; own = true;
     int lt = tile;
     if (n_seg > 1 || k_seg) {
       seg = tile / seg_tiles;
@@ -215,24 +237,47 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     }
     m_tile = lt / n_tiles;
     n_tile = lt - m_tile * n_tiles;
+    if (CG == 1) {
+      e = tile_expert ? tile_expert[m_tile] : 0;
+    } else if (pad_offsets) {
+      const int u = m_tile;
+      int lo = 0, hi = n_experts - 1;                // last expert with pair_off <= u
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (pair_off[mid] <= u) lo = mid; else hi = mid - 1;
+      }
+      e = lo;
+      m_tile = tile_off[e] + 2 * (u - pair_off[e]) + (int)rank;
+      own = m_tile < tile_off[e + 1];
+      if (!own) --m_tile;
+    } else {
+      e = 0;
+      m_tile = 2 * m_tile + (int)rank;               // (rows past the end are filled with zeros and not stored)
+    }
   };
   const int b_boxes = b_mn ? (block_n + 63) / 64 : 1;
-  const uint32_t stage_tx = A_STAGE_BYTES + (b_mn ? (uint32_t)b_boxes * MN_BOX_BYTES : (uint32_t)block_n * BLOCK_K * 2);
+  const uint32_t stage_tx = CG == 2 ? 2 * SB : A_STAGE_BYTES + (b_mn ? (uint32_t)b_boxes * MN_BOX_BYTES : (uint32_t)block_n * BLOCK_K * 2);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
-    for (int a = 0; a < ACC_STAGES; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), epi_warps_of(MODE)); }
+    for (int a = 0; a < ACC_STAGES; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), CG * epi_warps_of(MODE)); }
     mbar_init(drain_bar, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)), "r"(TMEM_COLS) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if constexpr (CG == 2) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)), "r"(TMEM_COLS) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)), "r"(TMEM_COLS) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
   }
   tc_fence_before();
   __syncthreads();
+  if (CG == 2) cluster_sync();                      // both CTAs' barriers and tensor memory exist before either is used
   tc_fence_after();
   const uint32_t tmem_base = *tmem_holder;
 
@@ -242,19 +287,40 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       int stage = 0; uint32_t phase = 0;
       int issued = 0;
       bool ok = true;
-      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-        int m_tile, n_tile, seg, kb0, nkb;
-        decode(tile, m_tile, n_tile, seg, kb0, nkb);
-        const int e = tile_expert ? tile_expert[m_tile] : 0;
+      for (int tile = worker; tile < total_tiles && ok; tile += n_workers) {
+        int m_tile, n_tile, seg, kb0, nkb, e;
+        bool own;
+        decode(tile, m_tile, n_tile, seg, kb0, nkb, own, e);
         const int b_row = MODE == EPI_SWIGLU ? e * 2 * N + n_tile * 128 : e * N + n_tile * block_n;
         for (int kq = 0; kq < nkb; ++kq) {
           const int kb = kb0 + kq;
           if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, wait_limit)) { ok = false; break; }
-          mbar_expect_tx(full_bar(stage), stage_tx);
           const uint32_t sa = base + stage * SB;
+          if constexpr (CG == 2) {
+            // both CTAs' copies count on the leader's barrier, which alone expects them
+            if (rank == 0) mbar_expect_tx(full_bar(stage), stage_tx);
+            const uint32_t fb = map_rank(full_bar(stage), 0);
+            if (a_mn) {
+              tma_load_2d_pair(sa, &tmap_a, fb, m_tile * BLOCK_M, kb * BLOCK_K);
+              tma_load_2d_pair(sa + MN_BOX_BYTES, &tmap_a, fb, m_tile * BLOCK_M + 64, kb * BLOCK_K);
+            } else {
+              tma_load_2d_pair(sa, &tmap_a, fb, kb * BLOCK_K, m_tile * BLOCK_M);
+            }
+            if (b_mn) {
+              const int n0 = n_tile * block_n + 128 * (int)rank;
+              tma_load_2d_pair(sa + A_STAGE_BYTES, &tmap_b, fb, n0, e * Kd + kb * BLOCK_K);
+              tma_load_2d_pair(sa + A_STAGE_BYTES + MN_BOX_BYTES, &tmap_b, fb, n0 + 64, e * Kd + kb * BLOCK_K);
+            } else {      // rows 128 .. 255 of the B tile: the next columns, or (SWIGLU) the up rows of the same hidden units
+              tma_load_2d_pair(sa + A_STAGE_BYTES, &tmap_b, fb, kb * BLOCK_K, b_row + (int)rank * (MODE == EPI_SWIGLU ? N : 128));
+            }
+            ++issued;
+            if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+            continue;
+          }
+          mbar_expect_tx(full_bar(stage), stage_tx);
           // fault injection (tests only): the copies of K block `withhold_kb` of this CTA's first tile are never issued,
           // so the stage never fills and the waits downstream run out
-          if (!(withhold_kb >= 0 && tile == (int)blockIdx.x && kq == withhold_kb)) {
+          if (!(withhold_kb >= 0 && tile == worker && kq == withhold_kb)) {
             if (a_mn) {
               tma_load_2d(sa, &tmap_a, full_bar(stage), m_tile * BLOCK_M, kb * BLOCK_K);
               tma_load_2d(sa + MN_BOX_BYTES, &tmap_a, full_bar(stage), m_tile * BLOCK_M + 64, kb * BLOCK_K);
@@ -290,18 +356,23 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    if (lane == 0 && rank == 0) {
       int stage = 0; uint32_t phase = 0;
       int acc = 0; uint32_t acc_phase = 0;
       bool ok = true, issued_any = false;
-      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-        if (!mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag, wait_limit)) { ok = false; break; }
+      auto commit = [&](uint32_t bar) { if constexpr (CG == 2) umma_commit_pair(bar); else umma_commit(bar); };
+      auto wait = [&](uint32_t bar, uint32_t ph) {
+        return CG == 2 ? mbar_wait_cluster(bar, ph, abort_flag, wait_limit) : mbar_wait(bar, ph, abort_flag, wait_limit);
+      };
+      for (int tile = worker; tile < total_tiles && ok; tile += n_workers) {
+        if (!wait(tempty_bar(acc), acc_phase ^ 1u)) { ok = false; break; }
         tc_fence_after();
         const uint32_t tmem_d = tmem_base + (uint32_t)acc * MAX_BLOCK_N;
-        int m_tile_, n_tile_, seg_, kb0_, nkb;
-        decode(tile, m_tile_, n_tile_, seg_, kb0_, nkb);
+        int m_tile_, n_tile_, seg_, kb0_, nkb, e_;
+        bool own_;
+        decode(tile, m_tile_, n_tile_, seg_, kb0_, nkb, own_, e_);
         for (int kb = 0; kb < nkb; ++kb) {
-          if (!mbar_wait(full_bar(stage), phase, abort_flag, wait_limit)) { ok = false; break; }
+          if (!wait(full_bar(stage), phase)) { ok = false; break; }
           tc_fence_after();
           const uint32_t sa = base + stage * SB;
           const uint64_t adesc = a_mn ? make_smem_desc_mn(sa) : make_smem_desc(sa);
@@ -309,14 +380,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
           // K-major: 16 elements = 32 bytes along K inside the swizzled row, +2 in the address field
           const uint32_t astep = a_mn ? MN_KSTEP : 2u, bstep = b_mn ? MN_KSTEP : 2u;
 #pragma unroll
-          for (int k = 0; k < BLOCK_K / UMMA_K; ++k)
-            umma_bf16(tmem_d, adesc + (uint64_t)(astep * k), bdesc + (uint64_t)(bstep * k), idesc, (kb | k) != 0 ? 1u : 0u);
-          umma_commit(empty_bar(stage));
+          for (int k = 0; k < BLOCK_K / UMMA_K; ++k) {
+            if constexpr (CG == 2) umma_bf16_pair(tmem_d, adesc + (uint64_t)(astep * k), bdesc + (uint64_t)(bstep * k), idesc, (kb | k) != 0 ? 1u : 0u);
+            else umma_bf16(tmem_d, adesc + (uint64_t)(astep * k), bdesc + (uint64_t)(bstep * k), idesc, (kb | k) != 0 ? 1u : 0u);
+          }
+          commit(empty_bar(stage));
           issued_any = true;
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
-        umma_commit(tfull_bar(acc));
+        commit(tfull_bar(acc));
         if (++acc == ACC_STAGES) { acc = 0; acc_phase ^= 1u; }
       }
       if (!ok) {
@@ -326,7 +399,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       if (*abort_flag && issued_any) {
         // the MMAs already issued may still read shared memory and write tensor memory: one more commit tracks them
         // all; wait for it (bounded) before the CTA frees its tensor memory
-        umma_commit(drain_bar);
+        commit(drain_bar);
         for (uint32_t it = 0; it < (wait_limit >> 2); ++it)
           if (mbar_try_wait(drain_bar, 0)) break;
       }
@@ -339,14 +412,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     const int n_chunks = block_n >> 5;
     int acc = 0; uint32_t acc_phase = 0;
     bool ok = true;
-    for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-      int m_tile, n_tile, seg, kb0_, nkb;
-      decode(tile, m_tile, n_tile, seg, kb0_, nkb);
+    for (int tile = worker; tile < total_tiles && ok; tile += n_workers) {
+      int m_tile, n_tile, seg, kb0_, nkb, e_;
+      bool own;
+      decode(tile, m_tile, n_tile, seg, kb0_, nkb, own, e_);
       // warp-uniform outcome: the tensor-memory loads below need the whole warp
       if (!__all_sync(0xffffffffu, mbar_wait(tfull_bar(acc), acc_phase, abort_flag, wait_limit))) { ok = false; break; }
       tc_fence_after();
       const int row = m_tile * BLOCK_M + quarter * 32 + lane;
-      bool row_ok = row < M_valid;
+      bool row_ok = row < M_valid && own;
       size_t out_row = (size_t)row;
       float scale = 1.0f;
       size_t tok_row = (size_t)row;
@@ -426,7 +500,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
 #pragma unroll
           for (int i = 0; i < 32; ++i) ra[i] = 0u;
         }
-        if (f32_out(MODE)) epi_softplus32<MODE>(epl, out_stage + (warp - 2) * 1024, m_tile * BLOCK_M + quarter * 32, M_valid, n_base + ch * 32, N, ra, bq, lane);
+        if (f32_out(MODE)) epi_softplus32<MODE>(epl, out_stage + (warp - 2) * 1024, m_tile * BLOCK_M + quarter * 32, own ? M_valid : 0, n_base + ch * 32, N, ra, bq, lane);
         else if (row_ok) epi_store32<MODE>(ep, out_row, tok_row, n_base + ch * 32, N, ra, scale, bq);
         ch += EWQ;
         if (ch >= n_chunks) break;
@@ -437,13 +511,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
 #pragma unroll
           for (int i = 0; i < 32; ++i) rb[i] = 0u;
         }
-        if (f32_out(MODE)) epi_softplus32<MODE>(epl, out_stage + (warp - 2) * 1024, m_tile * BLOCK_M + quarter * 32, M_valid, n_base + ch * 32, N, rb, bq, lane);
+        if (f32_out(MODE)) epi_softplus32<MODE>(epl, out_stage + (warp - 2) * 1024, m_tile * BLOCK_M + quarter * 32, own ? M_valid : 0, n_base + ch * 32, N, rb, bq, lane);
         else if (row_ok) epi_store32<MODE>(ep, out_row, tok_row, n_base + ch * 32, N, rb, scale, bq);
         ch += EWQ;
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(tempty_bar(acc));
+      if (lane == 0) { if (CG == 2) mbar_arrive_cluster(map_rank(tempty_bar(acc), 0)); else mbar_arrive(tempty_bar(acc)); }
       if (++acc == ACC_STAGES) { acc = 0; acc_phase ^= 1u; }
     }
     if (!ok && lane == 0) {
@@ -454,9 +528,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
 
   tc_fence_before();
   __syncthreads();
+  if (CG == 2) cluster_sync();                      // neither CTA leaves while the other may still signal it or read its operands
   if (warp == 1) {
+    __syncwarp();
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
+    if constexpr (CG == 2) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
+    else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
   }
 }
 
@@ -464,45 +541,68 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
 
 namespace {
 // instruction descriptor: D = f32, A = B = bf16, operand majorness (1 = MN-major) at bits 15 / 16, N >> 3 at bit 17, M >> 4 at bit 24
-uint32_t make_idesc(int block_n, bool a_mn, bool b_mn) {
+uint32_t make_idesc(int block_n, bool a_mn, bool b_mn, int block_m = BLOCK_M) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a_mn << 15) | ((uint32_t)b_mn << 16) | ((uint32_t)(block_n >> 3) << 17) |
-         ((uint32_t)(BLOCK_M >> 4) << 24);
+         ((uint32_t)(block_m >> 4) << 24);
+}
+
+// One persistent CTA pair per two SMs (a cluster of two), or one CTA per SM.
+template <typename... P, typename... Args>
+cudaError_t launch_workers(void (*kern)(P...), int cg, long long tiles, int num_sms, int threads, int smem, cudaStream_t st, Args... args) {
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  const long long slots = num_sms / cg;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(cg * (tiles < slots ? tiles : slots)));
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = cg; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = cg > 1 ? 1 : 0;
+  count_launch();
+  return cudaLaunchKernelEx(&cfg, kern, P(args)...);
 }
 }  // namespace
 
 cudaError_t launch_gemm_tc(const void* A, int lda, const void* Bw, int ldb, int n_experts, int M_max, int N, int Kd,
                            const int32_t* tile_expert, const int32_t* num_m_tiles_dev, const Epilogue& epi,
-                           int32_t* status, cudaStream_t st, bool test_stall, bool b_mn) {
+                           int32_t* status, cudaStream_t st, bool test_stall, bool b_mn, const int32_t* pad_offsets) {
   // N tile: a multiple of 32 (epilogue column groups) and of 16 (UMMA N for M = 128), at most 256
   const bool swiglu = epi.mode == EPI_SWIGLU;      // N output columns from 2N rows of B per expert, loaded as two boxes of 128 rows
   if (swiglu && (N % 128 != 0 || MAX_BLOCK_N != 256 || b_mn)) return cudaErrorInvalidValue;
   if (b_mn && n_experts > 1 && Kd % BLOCK_K != 0) return cudaErrorInvalidValue;      // a K block must not run into the next expert
   int block_n = (swiglu || N >= MAX_BLOCK_N) ? MAX_BLOCK_N : (N + 31) / 32 * 32;
   if (epi.mode == EPI_XPROJ && block_n > XPROJ_BLOCK_N) block_n = XPROJ_BLOCK_N;
-  CUtensorMap ta, tb;
-  if (!make_tmap(&ta, A, (uint64_t)M_max, (uint64_t)Kd, (uint64_t)lda, BLOCK_M)) return cudaErrorInvalidValue;
-  const bool ok = b_mn ? make_tmap(&tb, Bw, (uint64_t)n_experts * Kd, (uint64_t)N, (uint64_t)ldb, BLOCK_K)
-                       : make_tmap(&tb, Bw, (uint64_t)n_experts * (swiglu ? 2 * N : N), (uint64_t)Kd, (uint64_t)ldb, swiglu ? 128u : (uint32_t)block_n);
-  if (!ok) return cudaErrorInvalidValue;
-  const uint32_t idesc = make_idesc(block_n, false, b_mn);
   int num_sms = 0;
   cudaError_t e = current_device_sm_count(&num_sms);
   if (e != cudaSuccess) return e;
-  auto kern = epi.mode == EPI_STORE ? gemm_tc_kernel<EPI_STORE> : epi.mode == EPI_XPROJ ? gemm_tc_kernel<EPI_XPROJ>
-              : epi.mode == EPI_INPROJ ? gemm_tc_kernel<EPI_INPROJ> : epi.mode == EPI_OUTPROJ ? gemm_tc_kernel<EPI_OUTPROJ>
-              : epi.mode == EPI_F32 ? gemm_tc_kernel<EPI_F32> : epi.mode == EPI_SWIGLU ? gemm_tc_kernel<EPI_SWIGLU>
-              : epi.mode == EPI_SOFTPLUS_ROWS ? gemm_tc_kernel<EPI_SOFTPLUS_ROWS>
-              : gemm_tc_kernel<EPI_SOFTPLUS>;
-  const int smem_bytes = smem_bytes_of(epi.mode);
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-  if (e != cudaSuccess) return e;
+  // CTA pairs for the large grouped products: a pair fetches each B tile once for 256 rows (per CTA 32 KB a stage instead of 48).
+  // An expert's last pair is half empty every other time: from eight 128-row tiles per expert on, that costs at most 6 %.
+  const bool pair_mode = epi.mode == EPI_STORE || epi.mode == EPI_INPROJ || epi.mode == EPI_OUTPROJ || swiglu;
+  const int cg = pair_mode && pad_offsets && !test_stall && block_n == MAX_BLOCK_N && Kd >= 512 && M_max >= n_experts * 9 * BLOCK_M ? 2 : 1;
+  CUtensorMap ta, tb;
+  if (!make_tmap(&ta, A, (uint64_t)M_max, (uint64_t)Kd, (uint64_t)lda, BLOCK_M)) return cudaErrorInvalidValue;
+  const bool ok = b_mn ? make_tmap(&tb, Bw, (uint64_t)n_experts * Kd, (uint64_t)N, (uint64_t)ldb, BLOCK_K)
+                       : make_tmap(&tb, Bw, (uint64_t)n_experts * (swiglu ? 2 * N : N), (uint64_t)Kd, (uint64_t)ldb,
+                                   swiglu || cg == 2 ? 128u : (uint32_t)block_n);
+  if (!ok) return cudaErrorInvalidValue;
   const int n_tiles = swiglu ? N / 128 : (N + block_n - 1) / block_n;
-  const long long max_tiles = (long long)((M_max + BLOCK_M - 1) / BLOCK_M) * n_tiles;
-  const int grid = (int)(max_tiles < num_sms ? max_tiles : num_sms);
-  kern<<<grid, threads_of(epi.mode), smem_bytes, st>>>(ta, tb, M_max, N, Kd, block_n, idesc, tile_expert, num_m_tiles_dev, epi, status,
-                                                            test_stall ? WAIT_LIMIT_TEST : WAIT_LIMIT, test_stall ? 1 : -1, nullptr, 1, 0, b_mn ? 1 : 0);
-  count_launch();
-  return cudaGetLastError();
+  const int m_tiles = (M_max + BLOCK_M - 1) / BLOCK_M;
+  auto go = [&](auto kern) {
+    return launch_workers(kern, cg, (long long)(cg == 2 ? (m_tiles + n_experts) / 2 : m_tiles) * n_tiles, num_sms, threads_of(epi.mode),
+                          smem_bytes_of(epi.mode, cg), st, ta, tb, M_max, N, Kd, block_n, make_idesc(block_n, false, b_mn, cg * BLOCK_M), tile_expert,
+                          num_m_tiles_dev, epi, status, test_stall ? WAIT_LIMIT_TEST : WAIT_LIMIT, test_stall ? 1 : -1, nullptr, 1, 0, b_mn ? 1 : 0,
+                          pad_offsets, n_experts);
+  };
+  if (cg == 2) return go(epi.mode == EPI_STORE ? gemm_tc_kernel<EPI_STORE, 2> : epi.mode == EPI_INPROJ ? gemm_tc_kernel<EPI_INPROJ, 2>
+                         : epi.mode == EPI_OUTPROJ ? gemm_tc_kernel<EPI_OUTPROJ, 2> : gemm_tc_kernel<EPI_SWIGLU, 2>);
+  return go(epi.mode == EPI_STORE ? gemm_tc_kernel<EPI_STORE, 1> : epi.mode == EPI_XPROJ ? gemm_tc_kernel<EPI_XPROJ, 1>
+            : epi.mode == EPI_INPROJ ? gemm_tc_kernel<EPI_INPROJ, 1> : epi.mode == EPI_OUTPROJ ? gemm_tc_kernel<EPI_OUTPROJ, 1>
+            : epi.mode == EPI_F32 ? gemm_tc_kernel<EPI_F32, 1> : epi.mode == EPI_SWIGLU ? gemm_tc_kernel<EPI_SWIGLU, 1>
+            : epi.mode == EPI_SOFTPLUS_ROWS ? gemm_tc_kernel<EPI_SOFTPLUS_ROWS, 1> : gemm_tc_kernel<EPI_SOFTPLUS, 1>);
 }
 
 // Weight gradient on the tensor cores: C[s][P, Q] (fp32) = sum over the rows r of segment s of X[r, p] Y[r, q], X [rows, P] and
@@ -519,9 +619,6 @@ cudaError_t launch_gemm_tc_wgrad(const void* X, const void* Y, int rows, const i
   int num_sms = 0;
   cudaError_t e = current_device_sm_count(&num_sms);
   if (e != cudaSuccess) return e;
-  const int smem_bytes = smem_bytes_of(EPI_F32);
-  e = cudaFuncSetAttribute(gemm_tc_kernel<EPI_F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-  if (e != cudaSuccess) return e;
   const long long tiles = (long long)((P + BLOCK_M - 1) / BLOCK_M) * ((Q + block_n - 1) / block_n);
   Epilogue epi{EPI_F32, C, Q, nullptr, nullptr, nullptr, 0, 0, nullptr, nullptr};
   if (!seg) {
@@ -536,12 +633,11 @@ cudaError_t launch_gemm_tc_wgrad(const void* X, const void* Y, int rows, const i
       if ((e = cudaMemsetAsync(C, 0, sizeof(float) * (size_t)P * Q, st)) != cudaSuccess) return e;
     }
   }
-  const long long max_tiles = (long long)n_seg * tiles;
-  const int grid = (int)(max_tiles < num_sms ? max_tiles : num_sms);
-  gemm_tc_kernel<EPI_F32><<<grid, threads_of(EPI_F32), smem_bytes, st>>>(ta, tb, P, Q, rows, block_n, make_idesc(block_n, true, true), nullptr, nullptr, epi,
-                                                                        status, WAIT_LIMIT, -1, seg, n_seg, 1, 1);
-  count_launch();
-  return cudaGetLastError();
+  const int cg = seg && block_n == MAX_BLOCK_N && P >= 2 * BLOCK_M ? 2 : 1;
+  const long long units = (long long)n_seg * ((P + cg * BLOCK_M - 1) / (cg * BLOCK_M)) * ((Q + block_n - 1) / block_n);
+  return launch_workers(cg == 2 ? gemm_tc_kernel<EPI_F32, 2> : gemm_tc_kernel<EPI_F32, 1>, cg, units, num_sms, threads_of(EPI_F32), smem_bytes_of(EPI_F32, cg), st,
+                        ta, tb, P, Q, rows, block_n, make_idesc(block_n, true, true, cg * BLOCK_M), nullptr, nullptr, epi, status, WAIT_LIMIT, -1, seg, n_seg, 1, 1,
+                        nullptr, 0);
 }
 
 }  // namespace rom

@@ -156,7 +156,8 @@ cudaError_t launch_gemm_skinny(int dtype, const void* A, int lda, const void* Bw
 // on the weights as stored).
 cudaError_t launch_gemm_tc(const void* A, int lda, const void* Bw, int ldb, int n_experts,
                            int M_max, int N, int Kd, const int32_t* tile_expert, const int32_t* num_m_tiles_dev,
-                           const Epilogue& epi, int32_t* status, cudaStream_t st, bool test_stall = false, bool b_mn = false);
+                           const Epilogue& epi, int32_t* status, cudaStream_t st, bool test_stall = false, bool b_mn = false,
+                           const int32_t* pad_offsets = nullptr /* grouped: the padded segment offsets (n_experts + 1); allows CTA pairs */);
 
 // Weight gradient on the tensor cores (bf16): C[s][P, Q] fp32 = sum over rows r of segment s of X[r, p] Y[r, q]; X [rows, P],
 // Y [rows, Q]; seg: n_seg + 1 device row offsets, multiples of 64, or nullptr = one sum over all rows.

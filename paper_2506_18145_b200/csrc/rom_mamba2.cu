@@ -313,7 +313,8 @@ int rom_mamba2_layer_forward(const rom_config* cfg, int32_t headdim, const rom_m
   const int32_t* row_of_assign = reinterpret_cast<const int32_t*>(W + lay.row_of_assign);
   float* gates = gates_out ? gates_out : reinterpret_cast<float*>(W + lay.gates);
   auto gemm = [&](const void* A_, int lda, const void* B_, int ldb, int64_t bstride, int Nn, int Kd, const Epilogue& ep) -> cudaError_t {
-    if (tc) return launch_gemm_tc(A_, lda, B_, ldb, c.E, rows, Nn, Kd, tile_expert, num_m_tiles, ep, status, st);
+    if (tc) return launch_gemm_tc(A_, lda, B_, ldb, c.E, rows, Nn, Kd, tile_expert, num_m_tiles, ep, status, st, false, false,
+                                  reinterpret_cast<const int32_t*>(W + lay.pad_offsets));
     return launch_gemm_simt(c.dtype, A_, lda, B_, ldb, bstride, rows, Nn, Kd, tile_expert, num_m_tiles, ep, st);
   };
 
