@@ -44,8 +44,29 @@ inline int scan_chunks(int B, int De, int L) {
   }
   return best;
 }
+// Chunks per sequence of the warp kernel (rom_scan_warp.cu): the count with the smallest time by its measured pace.  A 128-channel
+// block takes 139 / 192 / 272 ns a step with one / two / three blocks on an SM (three fit), 115 / 161 / 230 ns state-only; more than
+// one chunk costs the state-only launch and about 12 us for the chain and the extra launches.  Chunks of at least 48 steps.  A
+// function of the problem sizes only (148 SMs assumed), so that workspace sizing and the launch agree.
+inline int scan_warp_chunks(int B, int De, int L) {
+  const long long blocks1 = (long long)B * ((De + 127) / 128);
+  auto pace = [](long long blocks, const double (&ns)[3]) {
+    const long long k = (blocks + 147) / 148;
+    return k <= 3 ? ns[k - 1] : ns[2] * (double)k / 3.0;
+  };
+  const double full[3] = {139.0, 192.0, 272.0}, state[3] = {115.0, 161.0, 230.0};
+  int best = 1;
+  double best_t = (double)L * pace(blocks1, full);
+  for (int n = 2; n <= 64 && L >= 48 * n; ++n) {
+    const long long blocks = blocks1 * (n - 1);
+    if (blocks > 148 * 12) break;
+    const double t = (double)L / (n - 0.3) * (pace(blocks, full) + pace(blocks, state)) + 12000.0;
+    if (t < best_t) { best_t = t; best = n; }
+  }
+  return best;
+}
 inline size_t scan_ws_floats(int B, int De, int L) {
-  const int nch = scan_chunks(B, De, L);
+  const int a = scan_chunks(B, De, L), b = scan_warp_chunks(B, De, L), nch = a > b ? a : b;
   return nch == 1 ? 0 : (size_t)B * nch * De * (2 * 16 + 1);
 }
 

@@ -33,7 +33,7 @@
 
 #include <cmath>
 
-#include "rom_internal.cuh"
+#include "rom_scan_args.cuh"
 
 namespace rom {
 namespace {
@@ -116,30 +116,12 @@ struct Tile {
   float4 bc[Geo<NC, NS>::TS][NST / 2];           // (B_n, B_n+1, C_n, C_n+1) per state pair
 };
 
-struct ScanArgs {
-  const void* u; const void* delta; const float* A; const float* Bm; const float* Cm; const float* D;
-  const void* z; int ldz; const int32_t* z_row; const float* h0; void* y; float* h_last; const int32_t* y_rows;
-  int K, L, De;
-  int Lc, nch;          // chunk length and chunks per sequence (nch == 1: Lc == L); blockIdx.z = chunk
-  int L0;               // length of chunk 0; chunk j >= 1 covers steps [L0 + (j-1) Lc, L0 + j Lc)
-  float* sum_delta;     // state-only blocks: [B*nch, De] sum of Delta over the chunk
-  int gate_activated;   // z already holds SiLU(gate pre-activation): multiply only
-  int chunk_off;        // chunk of blockIdx.z == 0
-  float* ckpt;          // MODE 3..5: [B, nck, De, 16] state at the start of every kScanCkpt steps (nck per sequence)
-  int nck;
-  int scalar_a;         // A[c, :] is one value per channel (scalar-per-head decay of a Mamba2-style block): one exponential
-                        // per channel and step instead of one per state (only with B-bar = Delta B)
-};
 // TD: type Delta is stored in: float (the rom_scan entry point, the fp32 layer) or the storage type (bf16 layer).
 
 // PRECISE: libm-accurate exp / expm1 (fp32 configuration, 1e-4 tolerance); otherwise one ex2.approx per
 // state update (bf16 configurations, 2e-2 tolerance).
 // ZOH: zero-order-hold B-bar (disc_mode 0); otherwise B-bar = Delta B.
-// MODE 0: full scan.  MODE 1: state only (no outputs, only h_last and sum_delta of every chunk).  MODE 3: state only
-// from the given chunk-start states, storing the state at the start of every kScanCkpt steps (backward pass).  MODE 4 and 5:
-// MODE 0 and 2 with those stores beside the outputs (the layer backward's recomputed forward).  MODE 2: first
-// launch of the chunked scan: chunk 0 runs the full scan from the caller's initial state (h0 indexed by
-// sequence), the other chunks run state-only from a zero state.
+// MODE: a ScanMode.
 template <typename T, typename TD, int NC, int NS, bool PRECISE, bool ZOH, int MODE>
 __global__ void __launch_bounds__(BLOCK, NS >= 8 ? 2 : 1)
 scan_kernel(const ScanArgs p) {
@@ -557,11 +539,11 @@ cudaError_t launch_shape(int shape, const ScanArgs& a, int B, cudaStream_t st) {
   }
 }
 
-// CKPT: also store the checkpoints of the backward pass (MODE 4 / 5 instead of 0 / 2).
+// CKPT: also store the checkpoints of the backward pass.
 template <typename T, typename TD, bool PRECISE, bool CKPT = false>
 cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const float* h0, float* h_last,
                           float* chunk_ws, int num_sms, cudaStream_t st) {
-  constexpr int FULL = CKPT ? 4 : 0, FIRST = CKPT ? 5 : 2;
+  constexpr ScanMode FULL = CKPT ? SCAN_FULL_CKPT : SCAN_FULL, FIRST = CKPT ? SCAN_FIRST_CKPT : SCAN_FIRST;
   const bool zoh = c.disc_mode == 0;
   if (!CKPT && c.L == 1) {
     a.h0 = h0; a.h_last = h_last;
@@ -571,28 +553,45 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
     count_launch();
     return cudaGetLastError();
   }
-  const int nch = chunk_ws ? scan_chunks(c.B, c.d_inner, c.L) : 1;
+  // bf16 storage, A per channel and state: the warp kernel, unless there is neither a workspace for chunks nor one of its warps
+  // per SM sub-partition (fewer states per thread then spread the work further)
+  const bool warp_kernel = !PRECISE && !a.scalar_a && (CKPT || chunk_ws || (long long)c.B * (c.d_inner / 32) >= 4LL * num_sms);
+  const int nch = !chunk_ws ? 1 : warp_kernel ? scan_warp_chunks(c.B, c.d_inner, c.L) : scan_chunks(c.B, c.d_inner, c.L);
+  // one launch over `grid_z` chunks with 8 states per thread (chunked) or the warp kernel
+  auto chunks = [&](const ScanArgs& x, int grid_z, auto mode) -> cudaError_t {
+    constexpr ScanMode M = decltype(mode)::value;
+    if constexpr (!PRECISE) { if (warp_kernel) return launch_scan_warp(x, c.B, grid_z, zoh, sizeof(TD) == 4, M, st); }
+    if constexpr (CKPT && !PRECISE) return cudaErrorInvalidValue;      // (the warp kernel has been taken)
+    else return zoh ? launch_one<T, TD, 1, 8, PRECISE, true, M>(x, c.B, grid_z, st) : launch_one<T, TD, 1, 8, PRECISE, false, M>(x, c.B, grid_z, st);
+  };
+  typedef std::integral_constant<ScanMode, FULL> FullTag;
+  typedef std::integral_constant<ScanMode, FIRST> FirstTag;
   if (nch == 1) {
     a.Lc = c.L; a.L0 = c.L; a.nch = 1;
-    const int shape = pick_thread_shape(c.B, c.d_inner, num_sms);
-    return zoh ? launch_shape<T, TD, PRECISE, true, FULL>(shape, a, c.B, st) : launch_shape<T, TD, PRECISE, false, FULL>(shape, a, c.B, st);
+    if (warp_kernel) return chunks(a, 1, FullTag{});
+    if constexpr (!(CKPT && !PRECISE)) {
+      const int shape = pick_thread_shape(c.B, c.d_inner, num_sms);
+      return zoh ? launch_shape<T, TD, PRECISE, true, FULL>(shape, a, c.B, st) : launch_shape<T, TD, PRECISE, false, FULL>(shape, a, c.B, st);
+    }
+    return cudaErrorInvalidValue;
   }
-  // chunked, two launches, 8 states per thread.  Launch A: chunk 0 in full from the caller's state, chunks
-  // 1..n_end-1 state-only from zero; chain; launch B: chunks 1..nch-1 in full from their true initial states.
+  // chunked, two launches.  Launch A: chunk 0 in full from the caller's state, chunks 1..n_end-1 state-only from zero; chain;
+  // launch B: chunks 1..nch-1 in full from their true initial states.
   const size_t n_state = (size_t)c.B * nch * c.d_inner * NST;
   float* h_end = chunk_ws;
   float* h_in = chunk_ws + n_state;
   float* sum_delta = chunk_ws + 2 * n_state;
   // Chunk 0 runs in full inside the first launch, next to state-only chunks that cost less per step: it is made
   // shorter by kFirstChunkRatio so that its blocks do not outlast the others.
+  const int align = warp_kernel ? 16 : 64;
   const double x = (double)c.L / ((double)(nch - 1) + kFirstChunkRatio);
-  a.Lc = (int)align_up((size_t)ceil(x), 64);
-  a.L0 = (int)align_up((size_t)ceil(kFirstChunkRatio * x), 64);
+  a.Lc = (int)align_up((size_t)ceil(x), align);
+  a.L0 = (int)align_up((size_t)ceil(kFirstChunkRatio * x), align);
   a.nch = nch;
   const int n_end = h_last ? nch : nch - 1;       // the last chunk's end state is only needed for h_last
   ScanArgs pa = a;
   pa.h_last = h_end; pa.sum_delta = sum_delta; pa.chunk_off = 0;
-  cudaError_t e = zoh ? launch_one<T, TD, 1, 8, PRECISE, true, FIRST>(pa, c.B, n_end, st) : launch_one<T, TD, 1, 8, PRECISE, false, FIRST>(pa, c.B, n_end, st);
+  cudaError_t e = chunks(pa, n_end, FirstTag{});
   if (e != cudaSuccess) return e;
   const long long n_thr = (long long)c.B * c.d_inner * NST;
   chain_chunk_states<<<(unsigned)((n_thr + 255) / 256), 256, 0, st>>>(A, h_end, sum_delta, h_in, h_last, c.B, c.d_inner, nch, n_end);
@@ -600,7 +599,7 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   a.h0 = h_in; a.h_last = nullptr; a.chunk_off = 1;
-  return zoh ? launch_one<T, TD, 1, 8, PRECISE, true, FULL>(a, c.B, nch - 1, st) : launch_one<T, TD, 1, 8, PRECISE, false, FULL>(a, c.B, nch - 1, st);
+  return chunks(a, nch - 1, FullTag{});
 }
 
 }  // namespace
@@ -640,11 +639,11 @@ cudaError_t launch_scan_states(const rom_config& c, const void* u, const float* 
   if (ckpt == nullptr) {
     a.h0 = nullptr;
     if (c.dtype != ROM_BF16) return zoh ? launch_one<float, float, 1, 8, true, true, 1>(a, c.B, ncc, st) : launch_one<float, float, 1, 8, true, false, 1>(a, c.B, ncc, st);
-    return zoh ? launch_one<__nv_bfloat16, float, 1, 8, false, true, 1>(a, c.B, ncc, st) : launch_one<__nv_bfloat16, float, 1, 8, false, false, 1>(a, c.B, ncc, st);
+    return launch_scan_warp(a, c.B, ncc, zoh, true, SCAN_STATE, st);
   }
   a.h_last = nullptr;
   if (c.dtype != ROM_BF16) return zoh ? launch_one<float, float, 1, 8, true, true, 3>(a, c.B, ncc, st) : launch_one<float, float, 1, 8, true, false, 3>(a, c.B, ncc, st);
-  return zoh ? launch_one<__nv_bfloat16, float, 1, 8, false, true, 3>(a, c.B, ncc, st) : launch_one<__nv_bfloat16, float, 1, 8, false, false, 3>(a, c.B, ncc, st);
+  return launch_scan_warp(a, c.B, ncc, zoh, true, SCAN_CKPT, st);
 }
 
 }  // namespace rom

@@ -59,6 +59,10 @@ struct BwdArgs {
   float* q_start; float* sum_delta;         // pre-pass outputs: [B, ncc, De, 16] and [B, ncc, De]
 };
 
+// slot of lane l's partial sums of step r: conflict-free both for a quarter-warp of writers (eight lanes, one step) and of readers
+// (lanes l = 8 g + const, two steps)
+__device__ __forceinline__ int ysw(int l, int r) { return l ^ (2 * (l >> 3) + (r & 1)); }
+
 // 8 consecutive elements of a row, as loaded
 template <typename T> struct Raw8;
 template <> struct Raw8<__nv_bfloat16> {
@@ -126,8 +130,9 @@ scan_bwd_kernel(const BwdArgs p) {
     g[i][0] = make_float2(gv.x, gv.y); g[i][1] = make_float2(gv.z, gv.w);
     dA[i][0] = make_float2(0.0f, 0.0f); dA[i][1] = dA[i][0];
   }
-  // ---- loader / output role: step lt of every checkpoint interval, channels lc .. lc+7
-  const int lt = lane & 7, l8 = lane >> 3, lc = c_warp + 8 * l8;
+  // ---- loader / output role: step lt of every checkpoint interval, channels lc .. lc+7 (four lanes per row: a load's quarter-warp
+  // touches two rows of global memory, not eight)
+  const int lt = lane >> 2, l8 = lane & 3, lc = c_warp + 8 * l8;
   float Dv[8], dDacc[8], dbacc[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) { Dv[i] = p.D ? p.D[lc + i] : 0.0f; dDacc[i] = 0.0f; dbacc[i] = 0.0f; }
@@ -265,9 +270,9 @@ scan_bwd_kernel(const BwdArgs p) {
       }
       // partial sums over this lane's states, into the slot of the state that every lane has now consumed
       __syncwarp();
-      s.h[r][0][lane ^ r] = make_float4(ddv[0], ddv[1], ddv[2], ddv[3]);
-      s.h[r][1][lane ^ r] = make_float4(duv[0], duv[1], duv[2], duv[3]);
-      s.h[r][2][lane ^ r] = make_float4(yv[0], yv[1], yv[2], yv[3]);
+      s.h[r][0][ysw(lane, r)] = make_float4(ddv[0], ddv[1], ddv[2], ddv[3]);
+      s.h[r][1][ysw(lane, r)] = make_float4(duv[0], duv[1], duv[2], duv[3]);
+      s.h[r][2][ysw(lane, r)] = make_float4(yv[0], yv[1], yv[2], yv[3]);
       // sums over the warp's channels: 8 values (4 dB, 4 dC of the lane's states) over the 8 channel groups; three exchange
       // steps halve the values a lane keeps while adding its partner's, so every lane ends with ONE fully reduced value
       {
@@ -302,7 +307,7 @@ scan_bwd_kernel(const BwdArgs p) {
         float4 acc[3];
 #pragma unroll
         for (int v = 0; v < 3; ++v) {
-          const float4 x0 = s.h[lt][v][(grp * 4) ^ lt], x1 = s.h[lt][v][(grp * 4 + 1) ^ lt], x2 = s.h[lt][v][(grp * 4 + 2) ^ lt], x3 = s.h[lt][v][(grp * 4 + 3) ^ lt];
+          const float4 x0 = s.h[lt][v][ysw(grp * 4, lt)], x1 = s.h[lt][v][ysw(grp * 4 + 1, lt)], x2 = s.h[lt][v][ysw(grp * 4 + 2, lt)], x3 = s.h[lt][v][ysw(grp * 4 + 3, lt)];
           acc[v] = make_float4((x0.x + x1.x) + (x2.x + x3.x), (x0.y + x1.y) + (x2.y + x3.y), (x0.z + x1.z) + (x2.z + x3.z), (x0.w + x1.w) + (x2.w + x3.w));
         }
         dd[4 * hf] = acc[0].x; dd[4 * hf + 1] = acc[0].y; dd[4 * hf + 2] = acc[0].z; dd[4 * hf + 3] = acc[0].w;
@@ -356,7 +361,7 @@ scan_bwd_kernel(const BwdArgs p) {
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
 #pragma unroll
-    for (int o = 1; o < 8; o <<= 1) { dDacc[i] += __shfl_xor_sync(0xffffffffu, dDacc[i], o); dbacc[i] += __shfl_xor_sync(0xffffffffu, dbacc[i], o); }
+    for (int o = 4; o < 32; o <<= 1) { dDacc[i] += __shfl_xor_sync(0xffffffffu, dDacc[i], o); dbacc[i] += __shfl_xor_sync(0xffffffffu, dbacc[i], o); }
     if (lt == 0 && p.dD) atomicAdd(p.dD + lc + i, dDacc[i]);
     if (lt == 0 && p.dpre) atomicAdd(p.db_dt + lc + i, dbacc[i]);
   }

@@ -1,0 +1,261 @@
+// Selective scan for bf16 storage (same arithmetic and arguments as rom_scan.cu): one warp owns 32 channels of one chunk of one
+// sequence, a lane 4 states of 4 adjacent channels.
+//
+// What bounds it: per state update one exponential on the special-function unit (16 per clock and SM), six fp32 lane operations
+// (128 per clock and SM) and the bytes that shared memory returns to registers (128 per clock and SM, one copy per lane).  With
+// 8 states of one channel per lane the B and C of every step cost 8 bytes per update -- as much time as the exponential -- and the
+// sums over states a shuffle and its selects.  Here the 16 updates of a lane and step share 16 bytes of B, 16 of C and 32 of
+// (Delta, u): 4 bytes per update; packed pairs run along the channels, so Delta and u need no duplication and the sums over a
+// lane's states no horizontal add; the four lanes of a channel leave their partial sums in shared memory, where the lane that
+// writes the output adds them (1 byte per update each way, no shuffles).  A warp is self-contained (no block barrier), eight steps
+// are staged at a time while the next eight are in flight in registers, and sixteen warps fit an SM.
+#include <type_traits>
+
+#include "rom_scan_args.cuh"
+
+namespace rom {
+namespace {
+
+typedef __nv_bfloat16 bf16;
+constexpr int NST = 16;
+constexpr int CK = kScanCkpt;     // steps per tile
+constexpr int WCH = 32;           // channels per warp
+constexpr int WPB = 4;            // warps per block
+constexpr int BT = WPB * 32;
+constexpr float kLog2e = 1.4426950408889634f;
+
+struct WarpTile {
+  float4 dl[CK][8], u[CK][8];     // Delta, u of 4 channels; group g of step r sits at g ^ r
+  float4 b[CK][4], c[CK][4];
+  float4 y[CK][32];               // partial sums of 4 channels over one lane's states; lane l of step r at ysw(l, r)
+};
+
+// conflict-free both for a quarter-warp of writers (eight lanes, one step) and of readers (lanes l = 8 g + const, two steps)
+__device__ __forceinline__ int ysw(int l, int r) { return l ^ (2 * (l >> 3) + (r & 1)); }
+
+// 8 consecutive elements of a row, as loaded
+template <typename T> struct Raw8;
+template <> struct Raw8<bf16> {
+  V16<bf16> q;
+  __device__ __forceinline__ void load(const bf16* p) { q.load(p); }
+  __device__ __forceinline__ void zero() { q.zero(); }
+  __device__ __forceinline__ void get(float (&v)[8]) const { q.get(v); }
+};
+template <> struct Raw8<float> {
+  float4 a, b;
+  __device__ __forceinline__ void load(const float* p) { a = __ldg(reinterpret_cast<const float4*>(p)); b = __ldg(reinterpret_cast<const float4*>(p) + 1); }
+  __device__ __forceinline__ void zero() { a = make_float4(0.0f, 0.0f, 0.0f, 0.0f); b = a; }
+  __device__ __forceinline__ void get(float (&v)[8]) const { v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w; }
+};
+__device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
+
+template <typename TD, bool ZOH, int MODE>
+__global__ void __launch_bounds__(BT, 3)
+scan_warp_kernel(const ScanArgs p) {
+  constexpr bool FIRST = MODE == SCAN_FIRST || MODE == SCAN_FIRST_CKPT;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  WarpTile& s = reinterpret_cast<WarpTile*>(smem_raw)[warp];
+  const int De = p.De;
+  const int c_warp = blockIdx.x * BT + warp * WCH;
+  if (c_warp >= De) return;       // d_inner is a multiple of 64: a warp's 32 channels are all in or all out
+  const int chunk = blockIdx.z + p.chunk_off;
+  const bool so = MODE == SCAN_STATE || MODE == SCAN_CKPT || (FIRST && chunk != 0);      // this block only produces states
+  const int t_first = chunk == 0 ? 0 : p.L0 + (chunk - 1) * p.Lc;
+  const int L = min(chunk == 0 ? p.L0 : p.Lc, p.L - t_first);      // steps of this chunk (<= 0: an empty chunk)
+  const size_t sc = (size_t)blockIdx.y * p.nch + chunk;            // index of the (sequence, chunk) state
+  const size_t tok0 = (size_t)blockIdx.y * p.L + (size_t)t_first;
+
+  // ---- compute role: channels c0 .. c0+3 (pairs), states 4q .. 4q+3
+  const int q = lane & 3, cg = lane >> 2;
+  const int c0 = c_warp + 4 * cg;
+  float2 a2[4][2], kin[4][2], h[4][2], sdel[2];
+  {
+    float av[4][4], hv[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float4 a4 = __ldg(reinterpret_cast<const float4*>(p.A + (size_t)(c0 + i) * NST) + q);
+      float4 h4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if (p.h0 && !(FIRST && so)) h4 = reinterpret_cast<const float4*>(p.h0 + ((FIRST ? (size_t)blockIdx.y : sc) * De + c0 + i) * NST)[q];
+      av[i][0] = a4.x; av[i][1] = a4.y; av[i][2] = a4.z; av[i][3] = a4.w;
+      hv[i][0] = h4.x; hv[i][1] = h4.y; hv[i][2] = h4.z; hv[i][3] = h4.w;
+    }
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        a2[n][j] = make_float2(av[2 * j][n] * kLog2e, av[2 * j + 1][n] * kLog2e);
+        kin[n][j] = make_float2(-1.0f / av[2 * j][n], -1.0f / av[2 * j + 1][n]);
+        h[n][j] = make_float2(hv[2 * j][n], hv[2 * j + 1][n]);
+      }
+    sdel[0] = make_float2(0.0f, 0.0f); sdel[1] = sdel[0];
+  }
+  auto put_state = [&](float* dst) {      // [De, 16] state array of one (sequence, chunk or checkpoint)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      *reinterpret_cast<float4*>(dst + (size_t)(c0 + 2 * j) * NST + 4 * q) = make_float4(h[0][j].x, h[1][j].x, h[2][j].x, h[3][j].x);
+      *reinterpret_cast<float4*>(dst + (size_t)(c0 + 2 * j + 1) * NST + 4 * q) = make_float4(h[0][j].y, h[1][j].y, h[2][j].y, h[3][j].y);
+    }
+  };
+  // ---- loader / output role: step lt of every tile, channels lc .. lc+7
+  // (four lanes per row: a load's quarter-warp touches two rows of global memory, not eight)
+  const int lt = lane >> 2, l8 = lane & 3, lc = c_warp + 8 * l8;
+  const bf16* __restrict__ zp = so ? nullptr : static_cast<const bf16*>(p.z);
+  const TD* dptr = static_cast<const TD*>(p.delta) + (tok0 + lt) * De + lc;
+  const bf16* uptr = static_cast<const bf16*>(p.u) + (tok0 + lt) * De + lc;
+  const float4* bptr = reinterpret_cast<const float4*>(p.Bm + tok0 * NST) + lane;
+  const float4* cptr = reinterpret_cast<const float4*>(p.Cm + tok0 * NST) + lane;
+
+  Raw8<TD> r_d;
+  Raw8<bf16> r_u, r_z, cur_u, cur_z;
+  float4 r_b, r_c;
+  int r_row = 0, cur_row = 0;      // first output row of this lane's step
+  auto fetch = [&](int t0) {
+    const int t = t0 + lt;
+    const float4 zero4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (t < L) {
+      r_d.load(dptr); r_u.load(uptr);
+      if (!so) {
+        if (zp) r_z.load(zp + (p.z_row ? (size_t)__ldg(p.z_row + tok0 + t) : tok0 + t) * p.ldz + lc);
+        r_row = p.y_rows ? __ldg(p.y_rows + (tok0 + t) * p.K) : (int)(tok0 + t);
+      }
+    } else {                       // steps past the end change nothing
+      r_d.zero(); r_u.zero();
+    }
+    dptr += (size_t)CK * De; uptr += (size_t)CK * De;
+    const bool in = t0 + (lane >> 2) < L;
+    r_b = in ? __ldg(bptr) : zero4;
+    if (!so) r_c = in ? __ldg(cptr) : zero4;
+    bptr += CK * 4; cptr += CK * 4;
+  };
+
+  auto run = [&](auto so_tag) {
+    constexpr bool SO = decltype(so_tag)::value;
+    constexpr bool CKPT = MODE == SCAN_CKPT || MODE == SCAN_FULL_CKPT || (MODE == SCAN_FIRST_CKPT && !SO);
+    fetch(0);
+    for (int t0 = 0; t0 < L; t0 += CK) {
+      {
+        float d[8], uu[8];
+        r_d.get(d); r_u.get(uu);
+        if (!ZOH) {                // B-bar = Delta B: the input enters as Delta u
+#pragma unroll
+          for (int i = 0; i < 8; ++i) uu[i] *= d[i];
+        }
+        s.dl[lt][(2 * l8) ^ lt] = make_float4(d[0], d[1], d[2], d[3]);
+        s.dl[lt][(2 * l8 + 1) ^ lt] = make_float4(d[4], d[5], d[6], d[7]);
+        s.u[lt][(2 * l8) ^ lt] = make_float4(uu[0], uu[1], uu[2], uu[3]);
+        s.u[lt][(2 * l8 + 1) ^ lt] = make_float4(uu[4], uu[5], uu[6], uu[7]);
+        reinterpret_cast<float4*>(s.b)[lane] = r_b;
+        if (!SO) { reinterpret_cast<float4*>(s.c)[lane] = r_c; cur_u = r_u; cur_z = r_z; cur_row = r_row; }
+      }
+      __syncwarp();
+      if (t0 + CK < L) fetch(t0 + CK);
+      if constexpr (CKPT) put_state(p.ckpt + ((size_t)blockIdx.y * p.nck + (size_t)((t_first + t0) / CK)) * De * NST);
+      // the next step's operands are requested before this step's arithmetic: a load issued behind a step's exponentials waits
+      // for all of them in the queue that both share
+      float4 nd = s.dl[0][cg], nu = s.u[0][cg], nb = s.b[0][q], nc = SO ? make_float4(0.0f, 0.0f, 0.0f, 0.0f) : s.c[0][q];
+      constexpr int UF = SO ? 4 : CK;      // (state-only: nothing orders the steps, and eight at once are slower)
+#pragma unroll UF
+      for (int r = 0; r < CK; ++r) {
+        const float4 d4 = nd, u4 = nu, b4 = nb, c4 = nc;
+        if (r + 1 < CK) {
+          nd = s.dl[r + 1][cg ^ (r + 1)]; nu = s.u[r + 1][cg ^ (r + 1)]; nb = s.b[r + 1][q];
+          if (!SO) nc = s.c[r + 1][q];
+        }
+        const float2 dl[2] = {make_float2(d4.x, d4.y), make_float2(d4.z, d4.w)}, uu[2] = {make_float2(u4.x, u4.y), make_float2(u4.z, u4.w)};
+        const float bb[4] = {b4.x, b4.y, b4.z, b4.w}, cc[4] = {c4.x, c4.y, c4.z, c4.w};
+        float2 acc[2];
+#pragma unroll
+        for (int n = 0; n < 4; ++n)
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const float2 x = __fmul2_rn(dl[j], a2[n][j]);
+            const float2 a = make_float2(ex2_ftz(x.x), ex2_ftz(x.y));
+            const float2 uB = __fmul2_rn(uu[j], dup(bb[n]));
+            if (ZOH) {             // w = -B u / A, h <- a (h - w) + w
+              const float2 w = __fmul2_rn(uB, kin[n][j]);
+              h[n][j] = __ffma2_rn(a, __ffma2_rn(w, dup(-1.0f), h[n][j]), w);
+            } else {
+              h[n][j] = __ffma2_rn(a, h[n][j], uB);
+            }
+            if (!SO) acc[j] = n == 0 ? __fmul2_rn(dup(cc[n]), h[n][j]) : __ffma2_rn(dup(cc[n]), h[n][j], acc[j]);
+          }
+        if (SO) { sdel[0] = __fadd2_rn(sdel[0], dl[0]); sdel[1] = __fadd2_rn(sdel[1], dl[1]); }
+        else s.y[r][ysw(lane, r)] = make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y);
+      }
+      __syncwarp();
+      if (!SO) {
+        // y = (sum over the four lanes + D u) * gate, rounded, written to the K rows of the token
+        const int t = t0 + lt;
+        if (t < L) {
+          float o[8], uu[8], zz[8];
+          cur_u.get(uu);
+          if (zp) {
+            cur_z.get(zz);
+            if (!p.gate_activated) {
+#pragma unroll
+              for (int i = 0; i < 8; ++i) zz[i] = silu_fast(zz[i]);
+            }
+          }
+#pragma unroll
+          for (int hf = 0; hf < 2; ++hf) {
+            const int g4 = 8 * l8 + 4 * hf;
+            const float4 x0 = s.y[lt][ysw(g4, lt)], x1 = s.y[lt][ysw(g4 + 1, lt)], x2 = s.y[lt][ysw(g4 + 2, lt)], x3 = s.y[lt][ysw(g4 + 3, lt)];
+            const float4 D4 = p.D ? __ldg(reinterpret_cast<const float4*>(p.D + lc) + hf) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            float2 v0 = __fadd2_rn(__fadd2_rn(make_float2(x0.x, x0.y), make_float2(x1.x, x1.y)), __fadd2_rn(make_float2(x2.x, x2.y), make_float2(x3.x, x3.y)));
+            float2 v1 = __fadd2_rn(__fadd2_rn(make_float2(x0.z, x0.w), make_float2(x1.z, x1.w)), __fadd2_rn(make_float2(x2.z, x2.w), make_float2(x3.z, x3.w)));
+            v0 = __ffma2_rn(make_float2(D4.x, D4.y), make_float2(uu[4 * hf], uu[4 * hf + 1]), v0);
+            v1 = __ffma2_rn(make_float2(D4.z, D4.w), make_float2(uu[4 * hf + 2], uu[4 * hf + 3]), v1);
+            if (zp) {
+              v0 = __fmul2_rn(v0, make_float2(zz[4 * hf], zz[4 * hf + 1]));
+              v1 = __fmul2_rn(v1, make_float2(zz[4 * hf + 2], zz[4 * hf + 3]));
+            }
+            o[4 * hf] = v0.x; o[4 * hf + 1] = v0.y; o[4 * hf + 2] = v1.x; o[4 * hf + 3] = v1.y;
+          }
+          bf16* y = static_cast<bf16*>(p.y) + lc;
+          V16<bf16>::store(y + (size_t)cur_row * De, o);
+          if (p.y_rows)
+            for (int k = 1; k < p.K; ++k) V16<bf16>::store(y + (size_t)__ldg(p.y_rows + (tok0 + t) * p.K + k) * De, o);
+        }
+        __syncwarp();
+      }
+    }
+  };
+  if constexpr (MODE == SCAN_STATE || MODE == SCAN_CKPT) run(std::true_type{});
+  else if constexpr (FIRST) { if (so) run(std::true_type{}); else run(std::false_type{}); }
+  else run(std::false_type{});
+
+  if (p.h_last) {
+    put_state(p.h_last + sc * De * NST);
+    if (so && q == 0 && p.sum_delta) *reinterpret_cast<float4*>(p.sum_delta + sc * De + c0) = make_float4(sdel[0].x, sdel[0].y, sdel[1].x, sdel[1].y);
+  }
+}
+
+template <typename TD, bool ZOH, int MODE>
+cudaError_t launch_mode(const ScanArgs& a, int B, int grid_z, cudaStream_t st) {
+  constexpr int smem = WPB * (int)sizeof(WarpTile);
+  scan_warp_kernel<TD, ZOH, MODE><<<dim3((a.De + BT - 1) / BT, B, grid_z), BT, smem, st>>>(a);
+  count_launch();
+  return cudaGetLastError();
+}
+template <typename TD, bool ZOH>
+cudaError_t launch_any(const ScanArgs& a, int B, int grid_z, ScanMode mode, cudaStream_t st) {
+  switch (mode) {
+    case SCAN_FULL: return launch_mode<TD, ZOH, SCAN_FULL>(a, B, grid_z, st);
+    case SCAN_STATE: return launch_mode<TD, ZOH, SCAN_STATE>(a, B, grid_z, st);
+    case SCAN_FIRST: return launch_mode<TD, ZOH, SCAN_FIRST>(a, B, grid_z, st);
+    case SCAN_CKPT: return launch_mode<TD, ZOH, SCAN_CKPT>(a, B, grid_z, st);
+    case SCAN_FULL_CKPT: return launch_mode<TD, ZOH, SCAN_FULL_CKPT>(a, B, grid_z, st);
+    case SCAN_FIRST_CKPT: return launch_mode<TD, ZOH, SCAN_FIRST_CKPT>(a, B, grid_z, st);
+  }
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace
+
+cudaError_t launch_scan_warp(const ScanArgs& a, int B, int grid_z, bool zoh, bool delta_fp32, ScanMode mode, cudaStream_t st) {
+  if (delta_fp32) return zoh ? launch_any<float, true>(a, B, grid_z, mode, st) : launch_any<float, false>(a, B, grid_z, mode, st);
+  return zoh ? launch_any<bf16, true>(a, B, grid_z, mode, st) : launch_any<bf16, false>(a, B, grid_z, mode, st);
+}
+
+}  // namespace rom
