@@ -321,7 +321,7 @@ int layer_forward_impl(const rom_config* cfg, const rom_weights* w, const void* 
     if (tc) return launch_gemm_tc(A_, lda, B_, ldb, n_experts, M_max, Nn, Kd, te, nmt, ep, status, st,
                                   (c.flags & ROM_FLAG_TEST_STALL) != 0 && (ep.mode == EPI_INPROJ || (ep.mode == EPI_STORE && Nn == 2 * De)), false,
                                   te ? reinterpret_cast<const int32_t*>(W + lay.pad_offsets) : nullptr);
-    return launch_gemm_simt(c.dtype, A_, lda, B_, ldb, bstride, M_max, Nn, Kd, te, nmt, ep, st);
+    return launch_gemm_simt(c.dtype, A_, lda, B_, ldb, bstride, M_max, Nn, Kd, te, nmt, ep, st, te ? reinterpret_cast<const int32_t*>(W + lay.assign_of_row) : nullptr);
   };
 
   // S3: grouped [Conv Proj | Gate Proj]

@@ -1,6 +1,6 @@
 // Plain fp32-FMA tiled GEMM, C[M,N] = A[M,Kd] * B[e][N,Kd]^T with fp32 accumulation.
-// It is the projection path of the fp32 configuration (a tf32 tensor path would not hold the 1e-4
-// tolerance) and, under ROM_FLAG_SIMT_GEMM, a bisecting aid for the bf16 tensor path.
+// gemm_f32 is the projection path of the fp32 configuration (a tf32 tensor path would not hold the 1e-4 tolerance); gemm_simt, under
+// ROM_FLAG_SIMT_GEMM, a bisecting aid for the bf16 tensor path.
 #include "rom_internal.cuh"
 
 namespace rom {
@@ -112,6 +112,106 @@ gemm_simt(const T* __restrict__ A, int lda, const T* __restrict__ Bw, int ldb, i
   }
 }
 
+// fp32 storage: C[M,N] = A[M,Kd] * B[e][N,Kd]^T on cp.async stages.  Operand rows lie in shared memory as in global (contracted
+// index innermost, pitch padded so that eight rows fall into different banks); a thread owns TM x TN outputs on rows and columns
+// (BM / TM) and (BN / TN) apart and takes four contracted elements of each per step.
+//   <128, 128, 8, 8, 1, 16>: shared-memory reads and FMAs in balance; for grids that fill the GPU.
+//   <32, 32, 4, 4, 4, 64>: the contracted index of a stage is split over four thread groups, so that a small product has four
+//     times the blocks' worth of threads in flight and a quarter of the serial steps (256 rows x 1024 columns x 256: the 64 x 64
+//     register-staged kernel took 28 us, waiting for one 16-wide stage after another).
+template <int BM, int BN, int TM, int TN, int KS, int BKF>
+__global__ void __launch_bounds__(BM / TM * (BN / TN) * KS)
+gemm_f32(const float* __restrict__ A, int lda, const float* __restrict__ Bw, int ldb, int64_t b_expert_stride, int M_max, int N, int Kd,
+         const int32_t* __restrict__ tile_expert, const int32_t* __restrict__ num_m_tiles_dev, const int32_t* __restrict__ assign_of_row, Epilogue ep) {
+  constexpr int TY = BM / TM, TX = BN / TN, GT = TY * TX, NT = GT * KS, PITCH = BKF + 4, STAGES = 3, KG = BKF / KS;
+  extern __shared__ __align__(16) float smf[];
+  const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
+  int M = M_max;
+  if (num_m_tiles_dev) M = min(M_max, *num_m_tiles_dev * kTileM);
+  if (m0 >= M) return;
+  const float* Bp = Bw;
+  if (tile_expert) {
+    const int e = tile_expert[m0 / kTileM];
+    if (e < 0) return;
+    Bp = Bw + (size_t)e * b_expert_stride;
+    if (assign_of_row && assign_of_row[m0] < 0) return;      // a segment's padding is at its end: nothing but padding here, nobody reads it
+  }
+  const int tid = threadIdx.x, kg = tid / GT, tx = tid % GT % TX, ty = tid % GT / TX;
+  auto fetch = [&](int k0, int stage) {
+    float* as = smf + stage * (BM + BN) * PITCH;
+    float* bs = as + BM * PITCH;
+    constexpr int VR = BKF / 4;
+#pragma unroll
+    for (int i = tid; i < (BM + BN) * VR; i += NT) {
+      const int r = i / VR, k = (i - r * VR) * 4;
+      const bool isA = r < BM;
+      const int row = isA ? m0 + r : n0 + r - BM;
+      const bool ok = (isA ? row < M : row < N) && k0 + k < Kd;
+      const float* src = ok ? (isA ? A + (size_t)row * lda : Bp + (size_t)row * ldb) + k0 + k : A;
+      const uint32_t dst = (uint32_t)__cvta_generic_to_shared((isA ? as + r * PITCH : bs + (r - BM) * PITCH) + k);
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  const int n_k = (Kd + BKF - 1) / BKF;
+#pragma unroll
+  for (int s = 0; s < STAGES - 1; ++s) {
+    if (s < n_k) fetch(s * BKF, s);
+    else asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  float acc[TM][TN] = {};
+  for (int kb = 0; kb < n_k; ++kb) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+    __syncthreads();
+    if (kb + STAGES - 1 < n_k) fetch((kb + STAGES - 1) * BKF, (kb + STAGES - 1) % STAGES);
+    else asm volatile("cp.async.commit_group;" ::: "memory");
+    const float* as = smf + (kb % STAGES) * (BM + BN) * PITCH + kg * KG;
+    const float* bs = as + BM * PITCH;
+#pragma unroll
+    for (int k = 0; k < KG; k += 4) {
+      float4 a[TM], b[TN];
+#pragma unroll
+      for (int i = 0; i < TM; ++i) a[i] = *reinterpret_cast<const float4*>(as + (ty + i * TY) * PITCH + k);
+#pragma unroll
+      for (int j = 0; j < TN; ++j) b[j] = *reinterpret_cast<const float4*>(bs + (tx + j * TX) * PITCH + k);
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+          acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
+          acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+          acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
+          acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
+        }
+    }
+  }
+  if (KS > 1) {
+    // the groups' partial sums, added in group order
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < TN; ++j) smf[(kg * BM + ty + i * TY) * (BN + 1) + tx + j * TX] = acc[i][j];
+    __syncthreads();
+    for (int i = tid; i < BM * BN; i += NT) {
+      const int r = i / BN, c = i % BN;
+      float v = 0.0f;
+#pragma unroll
+      for (int g = 0; g < KS; ++g) v += smf[(g * BM + r) * (BN + 1) + c];
+      if (m0 + r < M && n0 + c < N) epi_store_scalar<float>(ep, m0 + r, n0 + c, v);
+    }
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; ++j) {
+      const int m = m0 + ty + i * TY, n = n0 + tx + j * TX;
+      if (m < M && n < N) epi_store_scalar<float>(ep, m, n, acc[i][j]);
+    }
+}
+
 // Few rows, long K (the x Proj of a single-token step): C[M,N] = A[M,Kd] * B[N,Kd]^T with the K dimension split over
 // all 256 threads of a block.  A block owns 2 rows x 4 columns, so a handful of rows still spreads over
 // (M/2) x (N/4) blocks and every thread has only Kd / (256 V) rounds of loads in flight behind one another
@@ -166,16 +266,33 @@ gemm_skinny(const T* __restrict__ A, int lda, const T* __restrict__ Bw, int ldb,
 
 }  // namespace
 
+template <int BM_, int BN_, int TM, int TN, int KS, int BKF>
+static cudaError_t launch_f32(const float* A, int lda, const float* B, int ldb, int64_t stride, int M, int N, int Kd, const int32_t* te, const int32_t* nmt,
+                              const int32_t* assign_of_row, const Epilogue& ep, cudaStream_t st) {
+  constexpr int smem = 3 * (BM_ + BN_) * (BKF + 4) * (int)sizeof(float);
+  static_assert(smem >= KS * BM_ * (BN_ + 1) * (int)sizeof(float) || KS == 1, "partial sums reuse the stages");
+  auto kern = gemm_f32<BM_, BN_, TM, TN, KS, BKF>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  kern<<<dim3((M + BM_ - 1) / BM_, (N + BN_ - 1) / BN_), BM_ / TM * (BN_ / TN) * KS, smem, st>>>(A, lda, B, ldb, stride, M, N, Kd, te, nmt, assign_of_row, ep);
+  count_launch();
+  return cudaGetLastError();
+}
+
 cudaError_t launch_gemm_simt(int dtype, const void* A, int lda, const void* Bw, int ldb, int64_t b_expert_stride,
                              int M_max, int N, int Kd, const int32_t* tile_expert, const int32_t* num_m_tiles_dev,
-                             const Epilogue& epi, cudaStream_t st) {
+                             const Epilogue& epi, cudaStream_t st, const int32_t* assign_of_row) {
+  if (dtype == ROM_F32) {
+    const float* a = (const float*)A;
+    const float* b = (const float*)Bw;
+    // large tiles once they give every SM a block
+    if ((long long)((M_max + 127) / 128) * ((N + 127) / 128) >= 148)
+      return launch_f32<128, 128, 8, 8, 1, 16>(a, lda, b, ldb, b_expert_stride, M_max, N, Kd, tile_expert, num_m_tiles_dev, assign_of_row, epi, st);
+    return launch_f32<32, 32, 4, 4, 4, 64>(a, lda, b, ldb, b_expert_stride, M_max, N, Kd, tile_expert, num_m_tiles_dev, assign_of_row, epi, st);
+  }
   dim3 grid((M_max + BM - 1) / BM, (N + BN - 1) / BN);
-  if (dtype == ROM_BF16)
-    gemm_simt<__nv_bfloat16><<<grid, 256, 0, st>>>((const __nv_bfloat16*)A, lda, (const __nv_bfloat16*)Bw, ldb, b_expert_stride,
-                                                  M_max, N, Kd, tile_expert, num_m_tiles_dev, epi);
-  else
-    gemm_simt<float><<<grid, 256, 0, st>>>((const float*)A, lda, (const float*)Bw, ldb, b_expert_stride, M_max, N, Kd,
-                                          tile_expert, num_m_tiles_dev, epi);
+  gemm_simt<__nv_bfloat16><<<grid, 256, 0, st>>>((const __nv_bfloat16*)A, lda, (const __nv_bfloat16*)Bw, ldb, b_expert_stride,
+                                                M_max, N, Kd, tile_expert, num_m_tiles_dev, epi);
   count_launch();
   return cudaGetLastError();
 }

@@ -65,8 +65,20 @@ inline int scan_warp_chunks(int B, int De, int L) {
   }
   return best;
 }
+// Chunks per sequence of the fp32 scan: accurate exp / expm1 make a step of two states per thread (32 channels a block) cost about
+// 150 ns whatever the occupancy, so a short sequence is cut until those blocks fill the SMs once, into chunks of at least 32 steps.
+inline int scan_f32_chunks(int B, int De, int L) {
+  const long long blocks1 = (long long)B * ((De + 31) / 32);
+  long long n = (148 + blocks1 - 1) / blocks1 + 1;
+  if (n > L / 32) n = L / 32;
+  if (n > 24) n = 24;
+  const int old = scan_chunks(B, De, L);
+  return n < 3 ? old : n > old ? (int)n : old;
+}
 inline size_t scan_ws_floats(int B, int De, int L) {
-  const int a = scan_chunks(B, De, L), b = scan_warp_chunks(B, De, L), nch = a > b ? a : b;
+  int nch = scan_chunks(B, De, L);
+  if (scan_warp_chunks(B, De, L) > nch) nch = scan_warp_chunks(B, De, L);
+  if (scan_f32_chunks(B, De, L) > nch) nch = scan_f32_chunks(B, De, L);
   return nch == 1 ? 0 : (size_t)B * nch * De * (2 * 16 + 1);
 }
 
@@ -166,7 +178,8 @@ cudaError_t launch_small_combine(const rom_config& c, const float* Bp, const flo
 // i (kTileM rows) uses expert tile_expert[i]; the number of valid row tiles is *num_m_tiles_dev.
 cudaError_t launch_gemm_simt(int dtype, const void* A, int lda, const void* Bw, int ldb, int64_t b_expert_stride,
                              int M_max, int N, int Kd, const int32_t* tile_expert, const int32_t* num_m_tiles_dev,
-                             const Epilogue& epi, cudaStream_t st);
+                             const Epilogue& epi, cudaStream_t st,
+                             const int32_t* assign_of_row = nullptr /* grouped: row tiles that are all padding may be skipped */);
 
 // Ungrouped GEMM for a few rows and a long K (M <= 128, Kd a multiple of 2048 for bf16 / 1024 for fp32): K split over
 // the threads of a block.

@@ -530,13 +530,13 @@ int pick_thread_shape(int B, int De, int num_sms) {
 }
 
 template <typename T, typename TD, bool PRECISE, bool ZOH, int MODE>
-cudaError_t launch_shape(int shape, const ScanArgs& a, int B, cudaStream_t st) {
-  switch (shape) {
-    case 108: return launch_one<T, TD, 1, 8, PRECISE, ZOH, MODE>(a, B, a.nch, st);
-    case 104: return launch_one<T, TD, 1, 4, PRECISE, ZOH, MODE>(a, B, a.nch, st);
-    case 102: return launch_one<T, TD, 1, 2, PRECISE, ZOH, MODE>(a, B, a.nch, st);
-    default: return cudaErrorInvalidValue;
+cudaError_t launch_shape(int shape, const ScanArgs& a, int B, int grid_z, cudaStream_t st) {
+  if (shape == 108) return launch_one<T, TD, 1, 8, PRECISE, ZOH, MODE>(a, B, grid_z, st);
+  if constexpr (PRECISE || MODE == SCAN_FULL) {      // (bf16 chunks always run 8 states per thread)
+    if (shape == 104) return launch_one<T, TD, 1, 4, PRECISE, ZOH, MODE>(a, B, grid_z, st);
+    if (shape == 102) return launch_one<T, TD, 1, 2, PRECISE, ZOH, MODE>(a, B, grid_z, st);
   }
+  return cudaErrorInvalidValue;
 }
 
 // CKPT: also store the checkpoints of the backward pass.
@@ -556,13 +556,17 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
   // bf16 storage, A per channel and state: the warp kernel, unless there is neither a workspace for chunks nor one of its warps
   // per SM sub-partition (fewer states per thread then spread the work further)
   const bool warp_kernel = !PRECISE && !a.scalar_a && (CKPT || chunk_ws || (long long)c.B * (c.d_inner / 32) >= 4LL * num_sms);
-  const int nch = !chunk_ws ? 1 : warp_kernel ? scan_warp_chunks(c.B, c.d_inner, c.L) : scan_chunks(c.B, c.d_inner, c.L);
+  const int nch = !chunk_ws ? 1 : warp_kernel ? scan_warp_chunks(c.B, c.d_inner, c.L) : PRECISE ? scan_f32_chunks(c.B, c.d_inner, c.L) : scan_chunks(c.B, c.d_inner, c.L);
   // one launch over `grid_z` chunks with 8 states per thread (chunked) or the warp kernel
   auto chunks = [&](const ScanArgs& x, int grid_z, auto mode) -> cudaError_t {
     constexpr ScanMode M = decltype(mode)::value;
     if constexpr (!PRECISE) { if (warp_kernel) return launch_scan_warp(x, c.B, grid_z, zoh, sizeof(TD) == 4, M, st); }
     if constexpr (CKPT && !PRECISE) return cudaErrorInvalidValue;      // (the warp kernel has been taken)
-    else return zoh ? launch_one<T, TD, 1, 8, PRECISE, true, M>(x, c.B, grid_z, st) : launch_one<T, TD, 1, 8, PRECISE, false, M>(x, c.B, grid_z, st);
+    else {
+      // fp32 storage with few channels: fewer states per thread, so that the chunks together still spread over the SMs
+      const int shape = PRECISE ? pick_thread_shape(c.B * grid_z, c.d_inner, num_sms) : 108;
+      return zoh ? launch_shape<T, TD, PRECISE, true, M>(shape, x, c.B, grid_z, st) : launch_shape<T, TD, PRECISE, false, M>(shape, x, c.B, grid_z, st);
+    }
   };
   typedef std::integral_constant<ScanMode, FULL> FullTag;
   typedef std::integral_constant<ScanMode, FIRST> FirstTag;
@@ -571,7 +575,7 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
     if (warp_kernel) return chunks(a, 1, FullTag{});
     if constexpr (!(CKPT && !PRECISE)) {
       const int shape = pick_thread_shape(c.B, c.d_inner, num_sms);
-      return zoh ? launch_shape<T, TD, PRECISE, true, FULL>(shape, a, c.B, st) : launch_shape<T, TD, PRECISE, false, FULL>(shape, a, c.B, st);
+      return zoh ? launch_shape<T, TD, PRECISE, true, FULL>(shape, a, c.B, 1, st) : launch_shape<T, TD, PRECISE, false, FULL>(shape, a, c.B, 1, st);
     }
     return cudaErrorInvalidValue;
   }
@@ -583,7 +587,7 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
   float* sum_delta = chunk_ws + 2 * n_state;
   // Chunk 0 runs in full inside the first launch, next to state-only chunks that cost less per step: it is made
   // shorter by kFirstChunkRatio so that its blocks do not outlast the others.
-  const int align = warp_kernel ? 16 : 64;
+  const int align = warp_kernel || PRECISE ? 16 : 64;
   const double x = (double)c.L / ((double)(nch - 1) + kFirstChunkRatio);
   a.Lc = (int)align_up((size_t)ceil(x), align);
   a.L0 = (int)align_up((size_t)ceil(kFirstChunkRatio * x), align);
