@@ -246,8 +246,12 @@ int rom_scan_backward(const rom_config* cfg, const void* dy, const void* u, cons
   if (ws_bytes < scan_bwd_ws_bytes(cfg->B, cfg->d_inner, cfg->L)) return ROM_ERR_WORKSPACE;
   if ((rc = check_device()) != ROM_OK) return rc;
   LaunchCounter::count = 0;
-  ROM_CUDA(launch_scan_backward(*cfg, ScanBwd{dy, u, delta, true, A, Bm, Cm, D, z, h0, dh_last, nullptr, 1, du, ddelta, dA, dBm, dCm, dD, dz, dh0, nullptr, nullptr,
-                                              static_cast<float*>(ws), false, cfg->d_inner}, static_cast<cudaStream_t>(stream)));
+  const ScanBwd sb{dy, u, delta, true, A, Bm, Cm, D, z, h0, dh_last, nullptr, 1, du, ddelta, dA, dBm, dCm, dD, dz, dh0, nullptr, nullptr,
+                   static_cast<float*>(ws), false, cfg->d_inner};
+  ZeroList zl{};
+  scan_bwd_zero(*cfg, sb, zl);
+  ROM_CUDA(launch_zero(zl, static_cast<cudaStream_t>(stream)));
+  ROM_CUDA(launch_scan_backward(*cfg, sb, static_cast<cudaStream_t>(stream)));
   return ROM_OK;
 }
 
@@ -520,8 +524,30 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
     return launch_gemm_simt(c.dtype, A_, lda, scratch, Kd, (int64_t)Nn * Kd, M_max, Nn, Kd, te, nmt, ep, st);
   };
 
+  float* dBm = reinterpret_cast<float*>(W + bl.dBm);
+  float* dCm = reinterpret_cast<float*>(W + bl.dCm);
+  const char* zraw = W + bl.HZs + (size_t)De * esz;
+  const ScanBwd sb{W + bl.dYg, W + lay.U, W + lay.Delta, c.dtype != ROM_BF16, w->A, Bm, Cm, w->D, zraw, nullptr, nullptr, row_of_assign, c.K,
+                   W + bl.dU1, nullptr, g->dA, dBm, dCm, g->dD, W + bl.dHZp + (size_t)De * esz, nullptr, W + bl.dpre, g->db_dt,
+                   reinterpret_cast<float*>(W + bl.ckpt), true, 2 * De};
+  // everything that later kernels add into, and the status word, zeroed in one launch
+  float* rowscale = tc ? nullptr : reinterpret_cast<float*>(W + bl.rowscale);
+  {
+    ZeroList z{};
+    auto add = [&](void* p, size_t n) { if (p) { z.p[z.count] = static_cast<float*>(p); z.n[z.count++] = (long long)n; } };
+    add(status, kStatusInts);
+    scan_bwd_zero(c, sb, z);
+    add(g->dw_conv, (size_t)c.d_conv * De);
+    add(g->db_conv, De);
+    add(g->dW_r, (size_t)c.E * Dm);
+    add(g->db_r, c.E);
+    add(rowscale, rows);
+    if (tc && gemm_tc_wgrad_adds(T, De, R)) add(g->dW_dt, (size_t)De * R);
+    if (tc && gemm_tc_wgrad_adds(T, R + 2 * N, De)) add(g->dW_x, (size_t)(R + 2 * N) * De);
+    ROM_CUDA(launch_zero(z, st));
+  }
+
   // ---- forward, recomputed with the raw Gate Proj rows kept (the forward proper stores them activated at top-1)
-  ROM_CUDA(cudaMemsetAsync(status, 0, sizeof(int32_t) * kStatusInts, st));
   float* probs = reinterpret_cast<float*>(W + bl.probs);
   ROM_CUDA(launch_route_gather(c, x, w->W_r, w->b_r, nullptr, gates, nullptr, W, lay, st, probs));
   if (tc && c.K == 1) {
@@ -541,7 +567,6 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
   ROM_CUDA(gemm(W + lay.delta_r, R, w->W_dt, R, 1, 0, T, De, R, nullptr, nullptr, e_dt));
   // gated scan output in expert order (operand of the Out Proj weight gradient); padding rows must be zero
   ROM_CUDA(launch_zero_padding(c, W + lay.Ygp, De, W, lay, st));
-  const char* zraw = W + bl.HZs + (size_t)De * esz;
   ROM_CUDA(launch_scan(c, W + lay.U, W + lay.Delta, false, w->A, Bm, Cm, w->D, zraw, 2 * De, nullptr, nullptr, W + lay.Ygp, nullptr,
                        row_of_assign, c.K, reinterpret_cast<float*>(W + lay.scan_ws), false, st, false, reinterpret_cast<float*>(W + bl.ckpt)));
 
@@ -549,9 +574,7 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
   ROM_CUDA(launch_gather_rows_to(c, dout, W + bl.dOp, Dm, W, lay, st));
   ROM_CUDA(gemm_dgrad(W + bl.dOp, Dm, w->W_out, c.E, rows, De, Dm, tile_expert, num_m_tiles, W + bl.WoT, store_to(W + bl.dYgu, De)));
   // the weight gradient takes gate * Yg: scaled in place on the tensor path, a per-row factor of the plain-FMA kernel otherwise
-  float* rowscale = tc ? nullptr : reinterpret_cast<float*>(W + bl.rowscale);
   float* dgate = reinterpret_cast<float*>(W + bl.dgate);
-  if (rowscale) ROM_CUDA(cudaMemsetAsync(rowscale, 0, sizeof(float) * rows, st));
   ROM_CUDA(launch_combine_bwd(c.dtype, W + bl.dYgu, W + lay.Ygp, row_of_assign, gates, W + bl.dYg, dgate, rowscale, T, De, c.K, st));
   // weight gradients: sums over each expert's row segment (seg) or over all rows
   auto wgrad = [&](const void* X, int P, const void* Y, int Q, const float* scale, const int32_t* seg, int n_rows, float* C) -> cudaError_t {
@@ -563,11 +586,7 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
 
   // ---- gate, scan and softplus, reversed
   ROM_CUDA(launch_zero_padding(c, W + bl.dHZp, 2 * De, W, lay, st));
-  float* dBm = reinterpret_cast<float*>(W + bl.dBm);
-  float* dCm = reinterpret_cast<float*>(W + bl.dCm);
-  ROM_CUDA(launch_scan_backward(c, ScanBwd{W + bl.dYg, W + lay.U, W + lay.Delta, c.dtype != ROM_BF16, w->A, Bm, Cm, w->D, zraw, nullptr, nullptr, row_of_assign, c.K,
-                                           W + bl.dU1, nullptr, g->dA, dBm, dCm, g->dD, W + bl.dHZp + (size_t)De * esz, nullptr, W + bl.dpre, g->db_dt,
-                                           reinterpret_cast<float*>(W + bl.ckpt), true, 2 * De}, st));
+  ROM_CUDA(launch_scan_backward(c, sb, st));
 
   // ---- dt Proj and x Proj, reversed
   ROM_CUDA(gemm_dgrad(W + bl.dpre, De, w->W_dt, 1, T, R, De, nullptr, nullptr, W + bl.WdtT, store_to(W + bl.dxdbl, R + 2 * N)));      // d(delta) into columns [0, R)
@@ -577,8 +596,6 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
   ROM_CUDA(wgrad(W + bl.dxdbl, R + 2 * N, W + lay.U, De, nullptr, nullptr, T, g->dW_x));
 
   // ---- conv, reversed (dU = scan part + x Proj part)
-  ROM_CUDA(cudaMemsetAsync(g->dw_conv, 0, sizeof(float) * (size_t)c.d_conv * De, st));
-  ROM_CUDA(cudaMemsetAsync(g->db_conv, 0, sizeof(float) * De, st));
   ROM_CUDA(launch_conv_bwd(c, W + bl.HZs, w->w_conv, w->b_conv, W + bl.dU1, W + bl.dU2, W + bl.dHZp, row_of_assign, g->dw_conv, g->db_conv, st));
 
   // ---- Conv Proj | Gate Proj, reversed: every selected expert of a token receives the token's (dH, dZ), written above to its rows
@@ -587,8 +604,6 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
 
   // ---- router, reversed (through the gate values only), and dx
   float* dlogit = reinterpret_cast<float*>(W + bl.dlogit);
-  ROM_CUDA(cudaMemsetAsync(g->dW_r, 0, sizeof(float) * (size_t)c.E * Dm, st));
-  if (g->db_r) ROM_CUDA(cudaMemsetAsync(g->db_r, 0, sizeof(float) * c.E, st));
   ROM_CUDA(launch_router_bwd(c, x, probs, reinterpret_cast<const int32_t*>(W + lay.topk_idx), gates, dgate, dlogit, g->db_r, g->dW_r, st));
   ROM_CUDA(launch_dx(c, W + bl.dxp, row_of_assign, dlogit, w->W_r, dx, st));
   return ROM_OK;

@@ -36,6 +36,7 @@ __device__ __forceinline__ void stv(float* p, const float (&v)[4]) { *reinterpre
 template <typename T>
 __global__ void __launch_bounds__(256)
 transpose_kernel(const T* __restrict__ in, T* __restrict__ out, int R, int C) {
+  pdl_sync();
   __shared__ T tile[32][33];
   const size_t base = (size_t)blockIdx.z * R * C;
   const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
@@ -50,10 +51,18 @@ transpose_kernel(const T* __restrict__ in, T* __restrict__ out, int R, int C) {
   }
 }
 
+__global__ void __launch_bounds__(256)
+zero_kernel(const ZeroList z) {
+  pdl_sync();
+  float* p = z.p[blockIdx.y];
+  for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < z.n[blockIdx.y]; i += (long long)gridDim.x * 256) p[i] = 0.0f;
+}
+
 // dst[t, :] = sum_k src[row_of_assign[t*K + k], :]  (ascending k, fp32 accumulation), rows `width` wide
 template <typename T>
 __global__ void __launch_bounds__(256)
 slot_sum_kernel(const T* __restrict__ src, const int32_t* __restrict__ row_of_assign, T* __restrict__ dst, int width, int K, long long total_vec) {
+  pdl_sync();
   constexpr int V = VecN<T>::N;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= total_vec) return;
@@ -80,6 +89,7 @@ __global__ void __launch_bounds__(128)
 combine_bwd_kernel(const T* __restrict__ dYgu, T* Ygp, const int32_t* __restrict__ row_of_assign,
                    const float* __restrict__ gates, T* __restrict__ dYg, float* __restrict__ dgate, float* __restrict__ rowscale,
                    int De, int K) {
+  pdl_sync();
   __shared__ float red[kMaxK][4];
   const size_t t = blockIdx.x;
   int rows[kMaxK]; float g[kMaxK], part[kMaxK];
@@ -129,6 +139,7 @@ combine_bwd_kernel(const T* __restrict__ dYgu, T* Ygp, const int32_t* __restrict
 template <typename T>
 __global__ void __launch_bounds__(256)
 pack_bc_kernel(const float* __restrict__ dBm, const float* __restrict__ dCm, T* __restrict__ dxdbl, long long Tn, int R, int N) {
+  pdl_sync();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= Tn * 2 * N) return;
   const long long t = i / (2 * N);
@@ -176,6 +187,7 @@ __global__ void __launch_bounds__(128)
 conv_bwd_kernel(const T* __restrict__ HZ, const T* __restrict__ w_conv, const float* __restrict__ b_conv, const T* __restrict__ dU1,
                 const T* __restrict__ dU2, T* __restrict__ dHZ, const int32_t* __restrict__ row_of_assign, float* __restrict__ dw,
                 float* __restrict__ db, int L, int De, int K, int seg) {
+  pdl_sync();
   constexpr bool PRECISE = sizeof(T) == 4;
   constexpr int G = 4;
   const int c = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
@@ -267,6 +279,7 @@ conv_bwd_kernel(const T* __restrict__ HZ, const T* __restrict__ w_conv, const fl
 __global__ void __launch_bounds__(128)
 router_bwd_kernel(const float* __restrict__ P, const int32_t* __restrict__ idx, const float* __restrict__ gates, const float* __restrict__ dgate,
                   float* __restrict__ dlogit, float* __restrict__ db_r, long long Tn, int E, int K, int gate_mode) {
+  pdl_sync();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const bool in = t < Tn;
   const float* p = P + (in ? t : 0) * E;
@@ -297,6 +310,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 dx_kernel(const T* __restrict__ dxp, const int32_t* __restrict__ row_of_assign, const float* __restrict__ dlogit, const T* __restrict__ W_r,
           T* __restrict__ dx, int Dm, int E, int K, long long total_vec) {
+  pdl_sync();
   constexpr int V = VecN<T>::N;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= total_vec) return;
@@ -328,6 +342,7 @@ constexpr int RSLAB = 64;
 template <typename T>
 __global__ void __launch_bounds__(128)
 router_wgrad_kernel(const float* __restrict__ dlogit, const T* __restrict__ x, float* __restrict__ dW_r, long long Tn, int Dm, int E) {
+  pdl_sync();
   __shared__ float dl[RSLAB][8];
   const int e0 = blockIdx.y * 8;
   const long long t0 = (long long)blockIdx.z * RSLAB;
@@ -372,6 +387,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 wgrad_kernel(const T* __restrict__ X, int ldx, const T* __restrict__ Y, int ldy, const float* __restrict__ scale,
              const int32_t* __restrict__ seg, int rows_total, int P, int Q, float* __restrict__ C) {
+  pdl_sync();
   __shared__ float Xs[16][64 + 4];
   __shared__ float Ys[16][64 + 4];
   const int s = blockIdx.z;
@@ -421,8 +437,14 @@ wgrad_kernel(const T* __restrict__ X, int ldx, const T* __restrict__ Y, int ldy,
 
 cudaError_t launch_transpose(int dtype, const void* in, void* out, int batch, int R, int C, cudaStream_t st) {
   const dim3 grid((C + 31) / 32, (R + 31) / 32, batch), block(32, 8);
-  if (dtype == ROM_BF16) transpose_kernel<__nv_bfloat16><<<grid, block, 0, st>>>((const __nv_bfloat16*)in, (__nv_bfloat16*)out, R, C);
-  else transpose_kernel<float><<<grid, block, 0, st>>>((const float*)in, (float*)out, R, C);
+  if (dtype == ROM_BF16) launch_k(transpose_kernel<__nv_bfloat16>, grid, block, 0, st, (const __nv_bfloat16*)in, (__nv_bfloat16*)out, R, C);
+  else launch_k(transpose_kernel<float>, grid, block, 0, st, (const float*)in, (float*)out, R, C);
+  count_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t launch_zero(const ZeroList& z, cudaStream_t st) {
+  launch_k(zero_kernel, dim3(64, z.count), 256, 0, st, z);
   count_launch();
   return cudaGetLastError();
 }
@@ -430,8 +452,8 @@ cudaError_t launch_transpose(int dtype, const void* in, void* out, int batch, in
 cudaError_t launch_slot_sum(int dtype, const void* src, const int32_t* row_of_assign, void* dst, long long Tn, int width, int K, cudaStream_t st) {
   const long long total = Tn * (width / (dtype == ROM_BF16 ? 8 : 4));
   const unsigned blocks = (unsigned)((total + 255) / 256);
-  if (dtype == ROM_BF16) slot_sum_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>((const __nv_bfloat16*)src, row_of_assign, (__nv_bfloat16*)dst, width, K, total);
-  else slot_sum_kernel<float><<<blocks, 256, 0, st>>>((const float*)src, row_of_assign, (float*)dst, width, K, total);
+  if (dtype == ROM_BF16) launch_k(slot_sum_kernel<__nv_bfloat16>, blocks, 256, 0, st, (const __nv_bfloat16*)src, row_of_assign, (__nv_bfloat16*)dst, width, K, total);
+  else launch_k(slot_sum_kernel<float>, blocks, 256, 0, st, (const float*)src, row_of_assign, (float*)dst, width, K, total);
   count_launch();
   return cudaGetLastError();
 }
@@ -439,10 +461,10 @@ cudaError_t launch_slot_sum(int dtype, const void* src, const int32_t* row_of_as
 cudaError_t launch_combine_bwd(int dtype, const void* dYgu, void* Ygp, const int32_t* row_of_assign, const float* gates, void* dYg,
                                float* dgate, float* rowscale, long long Tn, int De, int K, cudaStream_t st) {
   if (dtype == ROM_BF16)
-    combine_bwd_kernel<__nv_bfloat16><<<(unsigned)Tn, 128, 0, st>>>((const __nv_bfloat16*)dYgu, (__nv_bfloat16*)Ygp, row_of_assign, gates,
+    launch_k(combine_bwd_kernel<__nv_bfloat16>, (unsigned)Tn, 128, 0, st, (const __nv_bfloat16*)dYgu, (__nv_bfloat16*)Ygp, row_of_assign, gates,
                                                                   (__nv_bfloat16*)dYg, dgate, rowscale, De, K);
   else
-    combine_bwd_kernel<float><<<(unsigned)Tn, 128, 0, st>>>((const float*)dYgu, (float*)Ygp, row_of_assign, gates, (float*)dYg, dgate,
+    launch_k(combine_bwd_kernel<float>, (unsigned)Tn, 128, 0, st, (const float*)dYgu, (float*)Ygp, row_of_assign, gates, (float*)dYg, dgate,
                                                           rowscale, De, K);
   count_launch();
   return cudaGetLastError();
@@ -450,8 +472,8 @@ cudaError_t launch_combine_bwd(int dtype, const void* dYgu, void* Ygp, const int
 
 cudaError_t launch_pack_bc(int dtype, const float* dBm, const float* dCm, void* dxdbl, long long Tn, int R, int N, cudaStream_t st) {
   const unsigned blocks = (unsigned)((Tn * 2 * N + 255) / 256);
-  if (dtype == ROM_BF16) pack_bc_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(dBm, dCm, (__nv_bfloat16*)dxdbl, Tn, R, N);
-  else pack_bc_kernel<float><<<blocks, 256, 0, st>>>(dBm, dCm, (float*)dxdbl, Tn, R, N);
+  if (dtype == ROM_BF16) launch_k(pack_bc_kernel<__nv_bfloat16>, blocks, 256, 0, st, dBm, dCm, (__nv_bfloat16*)dxdbl, Tn, R, N);
+  else launch_k(pack_bc_kernel<float>, blocks, 256, 0, st, dBm, dCm, (float*)dxdbl, Tn, R, N);
   count_launch();
   return cudaGetLastError();
 }
@@ -464,7 +486,7 @@ static void launch_conv_bwd_t(const rom_config& c, const void* HZ, const void* w
   const int seg = (long long)gx * c.B * ((c.L + 63) / 64) >= 4 * 148 ? 64 : 32;
   const dim3 grid(gx, (c.L + seg - 1) / seg, c.B);
   auto go = [&](auto kern) {
-    kern<<<grid, 128, 0, st>>>((const T*)HZ, (const T*)w_conv, b_conv, (const T*)dU1, (const T*)dU2, (T*)dHZ, row_of_assign, dw, db, c.L, c.d_inner, c.K, seg);
+    launch_k(kern, grid, 128, 0, st, (const T*)HZ, (const T*)w_conv, b_conv, (const T*)dU1, (const T*)dU2, (T*)dHZ, row_of_assign, dw, db, c.L, c.d_inner, c.K, seg);
   };
   if (c.d_conv == 4) go(conv_bwd_kernel<T, 4>);
   else if (c.d_conv == 3) go(conv_bwd_kernel<T, 3>);
@@ -481,11 +503,11 @@ cudaError_t launch_conv_bwd(const rom_config& c, const void* HZ, const void* w_c
 cudaError_t launch_router_bwd(const rom_config& c, const void* x, const float* probs, const int32_t* idx, const float* gates, const float* dgate,
                               float* dlogit, float* db_r, float* dW_r, cudaStream_t st) {
   const long long Tn = (long long)c.B * c.L;
-  router_bwd_kernel<<<(unsigned)((Tn + 127) / 128), 128, 0, st>>>(probs, idx, gates, dgate, dlogit, db_r, Tn, c.E, c.K, c.gate_mode);
+  launch_k(router_bwd_kernel, (unsigned)((Tn + 127) / 128), 128, 0, st, probs, idx, gates, dgate, dlogit, db_r, Tn, c.E, c.K, c.gate_mode);
   count_launch();
   const dim3 wgrid((c.d_model / 4 + 127) / 128, (c.E + 7) / 8, (unsigned)((Tn + RSLAB - 1) / RSLAB));
-  if (c.dtype == ROM_BF16) router_wgrad_kernel<__nv_bfloat16><<<wgrid, 128, 0, st>>>(dlogit, (const __nv_bfloat16*)x, dW_r, Tn, c.d_model, c.E);
-  else router_wgrad_kernel<float><<<wgrid, 128, 0, st>>>(dlogit, (const float*)x, dW_r, Tn, c.d_model, c.E);
+  if (c.dtype == ROM_BF16) launch_k(router_wgrad_kernel<__nv_bfloat16>, wgrid, 128, 0, st, dlogit, (const __nv_bfloat16*)x, dW_r, Tn, c.d_model, c.E);
+  else launch_k(router_wgrad_kernel<float>, wgrid, 128, 0, st, dlogit, (const float*)x, dW_r, Tn, c.d_model, c.E);
   count_launch();
   return cudaGetLastError();
 }
@@ -495,10 +517,10 @@ cudaError_t launch_dx(const rom_config& c, const void* dxp, const int32_t* row_o
   const long long total = (long long)c.B * c.L * (c.d_model / (c.dtype == ROM_BF16 ? 8 : 4));
   const unsigned blocks = (unsigned)((total + 255) / 256);
   if (c.dtype == ROM_BF16)
-    dx_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>((const __nv_bfloat16*)dxp, row_of_assign, dlogit, (const __nv_bfloat16*)W_r, (__nv_bfloat16*)dx,
+    launch_k(dx_kernel<__nv_bfloat16>, blocks, 256, 0, st, (const __nv_bfloat16*)dxp, row_of_assign, dlogit, (const __nv_bfloat16*)W_r, (__nv_bfloat16*)dx,
                                                    c.d_model, c.E, c.K, total);
   else
-    dx_kernel<float><<<blocks, 256, 0, st>>>((const float*)dxp, row_of_assign, dlogit, (const float*)W_r, (float*)dx, c.d_model, c.E, c.K, total);
+    launch_k(dx_kernel<float>, blocks, 256, 0, st, (const float*)dxp, row_of_assign, dlogit, (const float*)W_r, (float*)dx, c.d_model, c.E, c.K, total);
   count_launch();
   return cudaGetLastError();
 }
@@ -507,9 +529,9 @@ cudaError_t launch_wgrad(int dtype, const void* X, int ldx, const void* Y, int l
                          int rows_total, int P, int Q, float* C, cudaStream_t st) {
   const dim3 grid((Q + 63) / 64, (P + 63) / 64, n_seg);
   if (dtype == ROM_BF16)
-    wgrad_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>((const __nv_bfloat16*)X, ldx, (const __nv_bfloat16*)Y, ldy, scale, seg, rows_total, P, Q, C);
+    launch_k(wgrad_kernel<__nv_bfloat16>, grid, 256, 0, st, (const __nv_bfloat16*)X, ldx, (const __nv_bfloat16*)Y, ldy, scale, seg, rows_total, P, Q, C);
   else
-    wgrad_kernel<float><<<grid, 256, 0, st>>>((const float*)X, ldx, (const float*)Y, ldy, scale, seg, rows_total, P, Q, C);
+    launch_k(wgrad_kernel<float>, grid, 256, 0, st, (const float*)X, ldx, (const float*)Y, ldy, scale, seg, rows_total, P, Q, C);
   count_launch();
   return cudaGetLastError();
 }

@@ -90,6 +90,7 @@ template <typename T, int KT>
 __global__ void __launch_bounds__(128)
 conv_silu_kernel(const T* __restrict__ XZp, const int32_t* __restrict__ row_of_assign, const T* __restrict__ w_conv,
                  const float* __restrict__ b_conv, T* __restrict__ U, T* __restrict__ Zs, int L, int De, int K, int dconv) {
+  pdl_sync();
   constexpr int V = Vec<T>::N;
   const int c0 = (blockIdx.x * blockDim.x + threadIdx.x) * V;
   if (c0 >= De) return;
@@ -224,6 +225,7 @@ __global__ void __launch_bounds__(128)
 conv_step_kernel(const T* __restrict__ XZp, const int32_t* __restrict__ row_of_assign, const T* __restrict__ w_conv,
                  const float* __restrict__ b_conv, float* __restrict__ conv_state, T* __restrict__ U, T* __restrict__ Zs,
                  int De, int K, int dconv) {
+  pdl_sync();
   constexpr int V = Vec<T>::N;
   const int c0 = (blockIdx.x * blockDim.x + threadIdx.x) * V;
   if (c0 >= De) return;
@@ -276,6 +278,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 combine_kernel(const T* __restrict__ Op, const int32_t* __restrict__ row_of_assign, const float* __restrict__ gates,
                T* __restrict__ out, int Dm, int K, long long total_vec) {
+  pdl_sync();
   constexpr int V = Vec<T>::N;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= total_vec) return;
@@ -303,6 +306,7 @@ __global__ void __launch_bounds__(256)
 small_combine_kernel(const float* __restrict__ Bp, const float* __restrict__ Cp, const float* __restrict__ Dpre,
                      const int32_t* __restrict__ row_of_assign, const float* __restrict__ b_dt, float* __restrict__ Bm,
                      float* __restrict__ Cm, T* __restrict__ Delta, int De, int N, int K, long long total_vec) {
+  pdl_sync();
   constexpr bool PRECISE = sizeof(T) == 4;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= total_vec) return;
@@ -339,7 +343,7 @@ cudaError_t launch_conv_t(const rom_config& c, const void* XZp, const int32_t* r
   const int threads = 128;
   dim3 grid((c.d_inner / V + threads - 1) / threads, (c.L + TCH - 1) / TCH, c.B);
   auto args = [&](auto kern) {
-    kern<<<grid, threads, 0, st>>>((const T*)XZp, row_of_assign, (const T*)w_conv, b_conv, (T*)U, (T*)Zs, c.L, c.d_inner, c.K, c.d_conv);
+    launch_k(kern, grid, threads, 0, st, (const T*)XZp, row_of_assign, (const T*)w_conv, b_conv, (T*)U, (T*)Zs, c.L, c.d_inner, c.K, c.d_conv);
   };
   if (c.K == 1) args(conv_silu_kernel<T, 1>);
   else if (c.K == 2) args(conv_silu_kernel<T, 2>);
@@ -364,10 +368,10 @@ cudaError_t launch_combine(const rom_config& c, const void* Op, const int32_t* r
   const int threads = 256;
   const unsigned blocks = (unsigned)((total + threads - 1) / threads);
   if (bf)
-    combine_kernel<__nv_bfloat16><<<blocks, threads, 0, st>>>((const __nv_bfloat16*)Op, row_of_assign, gates, (__nv_bfloat16*)out,
+    launch_k(combine_kernel<__nv_bfloat16>, blocks, threads, 0, st, (const __nv_bfloat16*)Op, row_of_assign, gates, (__nv_bfloat16*)out,
                                                              c.d_model, c.K, total);
   else
-    combine_kernel<float><<<blocks, threads, 0, st>>>((const float*)Op, row_of_assign, gates, (float*)out, c.d_model, c.K, total);
+    launch_k(combine_kernel<float>, blocks, threads, 0, st, (const float*)Op, row_of_assign, gates, (float*)out, c.d_model, c.K, total);
   count_launch();
   return cudaGetLastError();
 }
@@ -378,9 +382,9 @@ cudaError_t launch_small_combine(const rom_config& c, const float* Bp, const flo
   const long long total = (long long)c.B * c.L * ((c.d_inner + 2 * c.d_state) / 4);
   const unsigned blocks = (unsigned)((total + 255) / 256);
   if (c.dtype == ROM_F32)
-    small_combine_kernel<float><<<blocks, 256, 0, st>>>(Bp, Cp, Dpre, row_of_assign, b_dt, Bm, Cm, (float*)Delta, c.d_inner, c.d_state, c.K, total);
+    launch_k(small_combine_kernel<float>, blocks, 256, 0, st, Bp, Cp, Dpre, row_of_assign, b_dt, Bm, Cm, (float*)Delta, c.d_inner, c.d_state, c.K, total);
   else
-    small_combine_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(Bp, Cp, Dpre, row_of_assign, b_dt, Bm, Cm, (__nv_bfloat16*)Delta, c.d_inner, c.d_state, c.K, total);
+    launch_k(small_combine_kernel<__nv_bfloat16>, blocks, 256, 0, st, Bp, Cp, Dpre, row_of_assign, b_dt, Bm, Cm, (__nv_bfloat16*)Delta, c.d_inner, c.d_state, c.K, total);
   count_launch();
   return cudaGetLastError();
 }
@@ -392,10 +396,10 @@ cudaError_t launch_conv_step(const rom_config& c, const void* XZp, const int32_t
   const int threads = 128;
   dim3 grid((c.d_inner / V + threads - 1) / threads, c.B);
   if (bf)
-    conv_step_kernel<__nv_bfloat16><<<grid, threads, 0, st>>>((const __nv_bfloat16*)XZp, row_of_assign, (const __nv_bfloat16*)w_conv, b_conv,
+    launch_k(conv_step_kernel<__nv_bfloat16>, grid, threads, 0, st, (const __nv_bfloat16*)XZp, row_of_assign, (const __nv_bfloat16*)w_conv, b_conv,
                                                             conv_state, (__nv_bfloat16*)U, (__nv_bfloat16*)Zs, c.d_inner, c.K, c.d_conv);
   else
-    conv_step_kernel<float><<<grid, threads, 0, st>>>((const float*)XZp, row_of_assign, (const float*)w_conv, b_conv, conv_state,
+    launch_k(conv_step_kernel<float>, grid, threads, 0, st, (const float*)XZp, row_of_assign, (const float*)w_conv, b_conv, conv_state,
                                                      (float*)U, (float*)Zs, c.d_inner, c.K, c.d_conv);
   count_launch();
   return cudaGetLastError();

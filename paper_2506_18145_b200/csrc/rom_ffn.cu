@@ -58,6 +58,7 @@ int check_ffn(const rom_config* c, int d_ff) {
 template <typename T>
 __global__ void __launch_bounds__(256)
 swiglu_rows(const T* __restrict__ GU, T* __restrict__ H, const int32_t* __restrict__ pad_offsets, int E, int d_ff, long long total) {
+  pdl_sync();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= total) return;
   const long long r = i / d_ff;
@@ -140,9 +141,9 @@ int rom_ffn_moe_forward(const rom_config* cfg, int32_t d_ff, const void* W_gu, c
     const unsigned blocks = (unsigned)((total + 255) / 256);
     const int32_t* pad_offsets = reinterpret_cast<const int32_t*>(W + lay.pad_offsets);
     if (c.dtype == ROM_BF16)
-      swiglu_rows<__nv_bfloat16><<<blocks, 256, 0, st>>>((const __nv_bfloat16*)(W + lay.XZp), (__nv_bfloat16*)(W + lay.Ygp), pad_offsets, c.E, d_ff, total);
+      launch_k(swiglu_rows<__nv_bfloat16>, blocks, 256, 0, st, (const __nv_bfloat16*)(W + lay.XZp), (__nv_bfloat16*)(W + lay.Ygp), pad_offsets, c.E, d_ff, total);
     else
-      swiglu_rows<float><<<blocks, 256, 0, st>>>((const float*)(W + lay.XZp), (float*)(W + lay.Ygp), pad_offsets, c.E, d_ff, total);
+      launch_k(swiglu_rows<float>, blocks, 256, 0, st, (const float*)(W + lay.XZp), (float*)(W + lay.Ygp), pad_offsets, c.E, d_ff, total);
     count_launch();
     ROM_CUDA(cudaGetLastError());
     Epilogue e_dn{EPI_STORE, W + lay.Op, Dm, nullptr, nullptr, nullptr, 0, 0, nullptr, nullptr};

@@ -50,6 +50,7 @@ __global__ void __launch_bounds__(256)
 gemm_simt(const T* __restrict__ A, int lda, const T* __restrict__ Bw, int ldb, int64_t b_expert_stride,
           int M_max, int N, int Kd, const int32_t* __restrict__ tile_expert, const int32_t* __restrict__ num_m_tiles_dev,
           Epilogue ep) {
+  pdl_sync();
   __shared__ float As[BK][BM + 1];
   __shared__ float Bs[BK][BN + 1];
   const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
@@ -123,6 +124,7 @@ template <int BM, int BN, int TM, int TN, int KS, int BKF>
 __global__ void __launch_bounds__(BM / TM * (BN / TN) * KS)
 gemm_f32(const float* __restrict__ A, int lda, const float* __restrict__ Bw, int ldb, int64_t b_expert_stride, int M_max, int N, int Kd,
          const int32_t* __restrict__ tile_expert, const int32_t* __restrict__ num_m_tiles_dev, const int32_t* __restrict__ assign_of_row, Epilogue ep) {
+  pdl_sync();
   constexpr int TY = BM / TM, TX = BN / TN, GT = TY * TX, NT = GT * KS, PITCH = BKF + 4, STAGES = 3, KG = BKF / KS;
   extern __shared__ __align__(16) float smf[];
   const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
@@ -219,6 +221,7 @@ gemm_f32(const float* __restrict__ A, int lda, const float* __restrict__ Bw, int
 template <typename T>
 __global__ void __launch_bounds__(256)
 gemm_skinny(const T* __restrict__ A, int lda, const T* __restrict__ Bw, int ldb, int M, int N, int Kd, Epilogue ep) {
+  pdl_sync();
   constexpr int V = 16 / sizeof(T);
   __shared__ float part[8][8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -274,7 +277,7 @@ static cudaError_t launch_f32(const float* A, int lda, const float* B, int ldb, 
   auto kern = gemm_f32<BM_, BN_, TM, TN, KS, BKF>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  kern<<<dim3((M + BM_ - 1) / BM_, (N + BN_ - 1) / BN_), BM_ / TM * (BN_ / TN) * KS, smem, st>>>(A, lda, B, ldb, stride, M, N, Kd, te, nmt, assign_of_row, ep);
+  launch_k(kern, dim3((M + BM_ - 1) / BM_, (N + BN_ - 1) / BN_), BM_ / TM * (BN_ / TN) * KS, smem, st, A, lda, B, ldb, stride, M, N, Kd, te, nmt, assign_of_row, ep);
   count_launch();
   return cudaGetLastError();
 }
@@ -291,7 +294,7 @@ cudaError_t launch_gemm_simt(int dtype, const void* A, int lda, const void* Bw, 
     return launch_f32<32, 32, 4, 4, 4, 64>(a, lda, b, ldb, b_expert_stride, M_max, N, Kd, tile_expert, num_m_tiles_dev, assign_of_row, epi, st);
   }
   dim3 grid((M_max + BM - 1) / BM, (N + BN - 1) / BN);
-  gemm_simt<__nv_bfloat16><<<grid, 256, 0, st>>>((const __nv_bfloat16*)A, lda, (const __nv_bfloat16*)Bw, ldb, b_expert_stride,
+  launch_k(gemm_simt<__nv_bfloat16>, grid, 256, 0, st, (const __nv_bfloat16*)A, lda, (const __nv_bfloat16*)Bw, ldb, b_expert_stride,
                                                 M_max, N, Kd, tile_expert, num_m_tiles_dev, epi);
   count_launch();
   return cudaGetLastError();
@@ -301,9 +304,9 @@ cudaError_t launch_gemm_skinny(int dtype, const void* A, int lda, const void* Bw
                                const Epilogue& epi, cudaStream_t st) {
   dim3 grid((N + 3) / 4, (M + 1) / 2);
   if (dtype == ROM_BF16)
-    gemm_skinny<__nv_bfloat16><<<grid, 256, 0, st>>>((const __nv_bfloat16*)A, lda, (const __nv_bfloat16*)Bw, ldb, M, N, Kd, epi);
+    launch_k(gemm_skinny<__nv_bfloat16>, grid, 256, 0, st, (const __nv_bfloat16*)A, lda, (const __nv_bfloat16*)Bw, ldb, M, N, Kd, epi);
   else
-    gemm_skinny<float><<<grid, 256, 0, st>>>((const float*)A, lda, (const float*)Bw, ldb, M, N, Kd, epi);
+    launch_k(gemm_skinny<float>, grid, 256, 0, st, (const float*)A, lda, (const float*)Bw, ldb, M, N, Kd, epi);
   count_launch();
   return cudaGetLastError();
 }

@@ -190,6 +190,25 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   float* out_stage = reinterpret_cast<float*>(smem + STAGES * SB + 256);        // [8 warps][32][32] (softplus only)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
+    for (int a = 0; a < ACC_STAGES; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), CG * epi_warps_of(MODE)); }
+    mbar_init(drain_bar, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {
+    if constexpr (CG == 2) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)), "r"(TMEM_COLS) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)), "r"(TMEM_COLS) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+  }
+  pdl_sync();                                       // (nothing above reads or writes memory of an earlier kernel)
+
   // CTA pairs: the pair shares one 256 x 256 tile; CTA r owns rows [128 r, 128 r + 128) of it and stages half of B.  An expert with
   // an odd number of 128-row tiles ends in a pair whose second CTA works on a copy of the first one's rows and stores nothing.
   const uint32_t rank = CG == 2 ? cluster_rank() : 0;
@@ -258,23 +277,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   const int b_boxes = b_mn ? (block_n + 63) / 64 : 1;
   const uint32_t stage_tx = CG == 2 ? 2 * SB : A_STAGE_BYTES + (b_mn ? (uint32_t)b_boxes * MN_BOX_BYTES : (uint32_t)block_n * BLOCK_K * 2);
 
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
-    for (int a = 0; a < ACC_STAGES; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), CG * epi_warps_of(MODE)); }
-    mbar_init(drain_bar, 1);
-    *abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
-  if (warp == 1) {
-    if constexpr (CG == 2) {
-      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)), "r"(TMEM_COLS) : "memory");
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-    } else {
-      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)), "r"(TMEM_COLS) : "memory");
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-  }
   tc_fence_before();
   __syncthreads();
   if (CG == 2) cluster_sync();                      // both CTAs' barriers and tensor memory exist before either is used
@@ -557,11 +559,13 @@ cudaError_t launch_workers(void (*kern)(P...), int cg, long long tiles, int num_
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = cg; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = cg > 1 ? 1 : 0;
+  cudaLaunchAttribute at[2]{};
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = cg; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = cg > 1 ? 2 : 1;
   count_launch();
   return cudaLaunchKernelEx(&cfg, kern, P(args)...);
 }
@@ -605,6 +609,26 @@ cudaError_t launch_gemm_tc(const void* A, int lda, const void* Bw, int ldb, int 
             : epi.mode == EPI_SOFTPLUS_ROWS ? gemm_tc_kernel<EPI_SOFTPLUS_ROWS, 1> : gemm_tc_kernel<EPI_SOFTPLUS, 1>);
 }
 
+namespace {
+// pieces of at least eight K blocks, as many as keep one tile per SM, none of them empty
+int wgrad_pieces(int rows, long long tiles, int num_sms) {
+  const int num_kb = (rows + BLOCK_K - 1) / BLOCK_K;
+  int n = 1;
+  while ((n + 1) * tiles <= num_sms && num_kb / (n + 1) >= 8) ++n;
+  const int per = (num_kb + n - 1) / n;
+  return (num_kb + per - 1) / per;
+}
+long long wgrad_tiles(int P, int Q) {
+  const int block_n = Q >= MAX_BLOCK_N ? MAX_BLOCK_N : (Q + 31) / 32 * 32;
+  return (long long)((P + BLOCK_M - 1) / BLOCK_M) * ((Q + block_n - 1) / block_n);
+}
+}  // namespace
+
+bool gemm_tc_wgrad_adds(int rows, int P, int Q) {
+  int num_sms = 0;
+  return current_device_sm_count(&num_sms) == cudaSuccess && wgrad_pieces(rows, wgrad_tiles(P, Q), num_sms) > 1;
+}
+
 // Weight gradient on the tensor cores: C[s][P, Q] (fp32) = sum over the rows r of segment s of X[r, p] Y[r, q], X [rows, P] and
 // Y [rows, Q] bf16 as the layer holds them (token rows outermost): both operands are MN-major tiles, nothing is transposed in
 // memory.  seg: n_seg + 1 device offsets, multiples of 64 (the padded expert segments; rows outside are never read).
@@ -619,19 +643,11 @@ cudaError_t launch_gemm_tc_wgrad(const void* X, const void* Y, int rows, const i
   int num_sms = 0;
   cudaError_t e = current_device_sm_count(&num_sms);
   if (e != cudaSuccess) return e;
-  const long long tiles = (long long)((P + BLOCK_M - 1) / BLOCK_M) * ((Q + block_n - 1) / block_n);
+  const long long tiles = wgrad_tiles(P, Q);
   Epilogue epi{EPI_F32, C, Q, nullptr, nullptr, nullptr, 0, 0, nullptr, nullptr};
   if (!seg) {
-    // pieces of at least eight K blocks, as many as keep one tile per SM
-    const int num_kb = (rows + BLOCK_K - 1) / BLOCK_K;
-    n_seg = 1;
-    while ((n_seg + 1) * tiles <= num_sms && num_kb / (n_seg + 1) >= 8) ++n_seg;
-    if (n_seg > 1) {
-      const int per = (num_kb + n_seg - 1) / n_seg;
-      n_seg = (num_kb + per - 1) / per;            // no empty piece
-      epi.accumulate = 1;
-      if ((e = cudaMemsetAsync(C, 0, sizeof(float) * (size_t)P * Q, st)) != cudaSuccess) return e;
-    }
+    n_seg = wgrad_pieces(rows, tiles, num_sms);
+    epi.accumulate = n_seg > 1;                      // (C was zeroed by the caller)
   }
   const int cg = seg && block_n == MAX_BLOCK_N && P >= 2 * BLOCK_M ? 2 : 1;
   const long long units = (long long)n_seg * ((P + cg * BLOCK_M - 1) / (cg * BLOCK_M)) * ((Q + block_n - 1) / block_n);

@@ -86,6 +86,7 @@ template <typename T>
 __global__ void __launch_bounds__(128)
 m2_conv_kernel(const T* __restrict__ ZXs, const T* __restrict__ w_conv, const float* __restrict__ b_conv, T* __restrict__ xc,
                float* __restrict__ Bm, float* __restrict__ Cm, int L, int De, int N, int W, int k) {
+  pdl_sync();
   constexpr int V = V16<T>::N;
   const int Cs = De + 2 * N;
   const int c0 = (blockIdx.x * blockDim.x + threadIdx.x) * V;
@@ -146,6 +147,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 m2_dt_kernel(const T* __restrict__ ZXs, const float* __restrict__ dt_bias, const float* __restrict__ A, const float* __restrict__ D,
              float* __restrict__ D32, float* __restrict__ A_exp, float* __restrict__ D_exp, int De, int N, int W, int headdim, long long Tn) {
+  pdl_sync();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < (long long)De) {
     const int h = (int)i / headdim;
@@ -168,6 +170,7 @@ template <typename T, int NV>
 __global__ void __launch_bounds__(256)
 m2_norm_kernel(const T* __restrict__ Yt, const float* __restrict__ w_norm, const int32_t* __restrict__ row_of_assign, T* __restrict__ Ygp,
                int De, int K, float eps, long long Tn) {
+  pdl_sync();
   constexpr int V = V16<T>::N;
   __shared__ float red[2][8];
   const int nvec = De / V, tid = threadIdx.x;
@@ -220,6 +223,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 m2_norm_wide_kernel(const T* __restrict__ Yt, const float* __restrict__ w_norm, const int32_t* __restrict__ row_of_assign, T* __restrict__ Ygp,
                int De, int K, float eps) {
+  pdl_sync();
   constexpr int V = V16<T>::N;
   __shared__ float red[8];
   const size_t t = blockIdx.x;
@@ -251,13 +255,13 @@ m2_norm_wide_kernel(const T* __restrict__ Yt, const float* __restrict__ w_norm, 
 template <typename T>
 cudaError_t launch_norm(const void* Yt, const float* w_norm, const int32_t* rows, void* Ygp, int De, int K, long long Tn, cudaStream_t st) {
   const int nv = (De / V16<T>::N + 255) / 256;
-  auto go = [&](auto kern) { kern<<<(unsigned)((Tn + M2_NT - 1) / M2_NT), 256, 0, st>>>((const T*)Yt, w_norm, rows, (T*)Ygp, De, K, 1e-5f, Tn); };
+  auto go = [&](auto kern) { launch_k(kern, (unsigned)((Tn + M2_NT - 1) / M2_NT), 256, 0, st, (const T*)Yt, w_norm, rows, (T*)Ygp, De, K, 1e-5f, Tn); };
   if (nv <= 1) go(m2_norm_kernel<T, 1>);
   else if (nv <= 2) go(m2_norm_kernel<T, 2>);
   else if (nv <= 4) go(m2_norm_kernel<T, 4>);
   else if (nv <= 8) go(m2_norm_kernel<T, 8>);
   else if (nv <= 16) go(m2_norm_kernel<T, 16>);
-  else m2_norm_wide_kernel<T><<<(unsigned)Tn, 256, 0, st>>>((const T*)Yt, w_norm, rows, (T*)Ygp, De, K, 1e-5f);
+  else launch_k(m2_norm_wide_kernel<T>, (unsigned)Tn, 256, 0, st, (const T*)Yt, w_norm, rows, (T*)Ygp, De, K, 1e-5f);
   count_launch();
   return cudaGetLastError();
 }
@@ -337,9 +341,9 @@ int rom_mamba2_layer_forward(const rom_config* cfg, int32_t headdim, const rom_m
     dim3 cgrid((Cs / vec + 127) / 128, (c.L + M2_TCH - 1) / M2_TCH, c.B);
     float* Bm = reinterpret_cast<float*>(W + m.Bm);
     float* Cm = reinterpret_cast<float*>(W + m.Cm);
-    if (bf) m2_conv_kernel<__nv_bfloat16><<<cgrid, 128, 0, st>>>((const __nv_bfloat16*)(W + m.ZXs), (const __nv_bfloat16*)w->w_conv, w->b_conv,
+    if (bf) launch_k(m2_conv_kernel<__nv_bfloat16>, cgrid, 128, 0, st, (const __nv_bfloat16*)(W + m.ZXs), (const __nv_bfloat16*)w->w_conv, w->b_conv,
                                                                 (__nv_bfloat16*)(W + m.xc), Bm, Cm, c.L, De, N, Wd, c.d_conv);
-    else m2_conv_kernel<float><<<cgrid, 128, 0, st>>>((const float*)(W + m.ZXs), (const float*)w->w_conv, w->b_conv, (float*)(W + m.xc), Bm, Cm,
+    else launch_k(m2_conv_kernel<float>, cgrid, 128, 0, st, (const float*)(W + m.ZXs), (const float*)w->w_conv, w->b_conv, (float*)(W + m.xc), Bm, Cm,
                                                     c.L, De, N, Wd, c.d_conv);
     count_launch();
     ROM_CUDA(cudaGetLastError());
@@ -351,9 +355,9 @@ int rom_mamba2_layer_forward(const rom_config* cfg, int32_t headdim, const rom_m
     float* D32 = reinterpret_cast<float*>(W + m.D32);
     float* A_exp = reinterpret_cast<float*>(W + m.A_exp);
     float* D_exp = reinterpret_cast<float*>(W + m.D_exp);
-    if (bf) m2_dt_kernel<__nv_bfloat16><<<blocks2, 256, 0, st>>>((const __nv_bfloat16*)(W + m.ZXs), w->dt_bias, w->A, w->D, D32, A_exp, D_exp, De, N, Wd,
+    if (bf) launch_k(m2_dt_kernel<__nv_bfloat16>, blocks2, 256, 0, st, (const __nv_bfloat16*)(W + m.ZXs), w->dt_bias, w->A, w->D, D32, A_exp, D_exp, De, N, Wd,
                                                                 headdim, T);
-    else m2_dt_kernel<float><<<blocks2, 256, 0, st>>>((const float*)(W + m.ZXs), w->dt_bias, w->A, w->D, D32, A_exp, D_exp, De, N, Wd, headdim, T);
+    else launch_k(m2_dt_kernel<float>, blocks2, 256, 0, st, (const float*)(W + m.ZXs), w->dt_bias, w->A, w->D, D32, A_exp, D_exp, De, N, Wd, headdim, T);
     count_launch();
     ROM_CUDA(cudaGetLastError());
     // the scalar-per-head recurrence as a special case of the selective scan (B-bar = Delta B), gate SiLU(z) applied there

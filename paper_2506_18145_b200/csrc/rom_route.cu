@@ -119,6 +119,7 @@ struct OffsetsArgs {
 
 __global__ void __launch_bounds__(1024)
 route_offsets(int32_t* __restrict__ chunk_counts, int n_chunks, int E, const OffsetsArgs o) {
+  pdl_sync();
   __shared__ int32_t cnt[kMaxE];
   __shared__ int32_t off[kMaxE + 1];
   __shared__ int32_t poff[kMaxE + 1];
@@ -138,6 +139,7 @@ route_logits_topk(const T* __restrict__ x, const T* __restrict__ W_r, const floa
                   int T_tokens, int Dm, int E, int K, int gate_mode,
                   int32_t* __restrict__ topk_idx, float* __restrict__ gates,
                   int32_t* __restrict__ chunk_counts, double* __restrict__ chunk_prob, float* __restrict__ probs, int n_chunks, const OffsetsArgs oa) {
+  pdl_sync();
   extern __shared__ __align__(16) unsigned char smem[];
   const int Epad = (E + NT8 - 1) / NT8 * NT8;
   const int n_wtiles = Epad / NT8;
@@ -345,6 +347,7 @@ route_scatter(const int32_t* __restrict__ topk_idx, const int32_t* __restrict__ 
               int T_tokens, int E, int K, int n_chunks,
               int32_t* __restrict__ perm, int32_t* __restrict__ inv_perm,
               int32_t* __restrict__ row_of_assign, int32_t* __restrict__ assign_of_row) {
+  pdl_sync();
   const int lane = threadIdx.x & 31;
   const int chunk = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (chunk >= n_chunks) return;
@@ -362,6 +365,7 @@ route_scatter_gather(const int32_t* __restrict__ topk_idx, const int32_t* __rest
                      int32_t* __restrict__ perm, int32_t* __restrict__ inv_perm,
                      int32_t* __restrict__ row_of_assign, int32_t* __restrict__ assign_of_row,
                      const uint4* __restrict__ x, uint4* __restrict__ x_perm, int vec_per_row) {
+  pdl_sync();
   __shared__ int32_t rows_s[kChunkTokens * kMaxK];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int chunk = blockIdx.x;
@@ -408,6 +412,7 @@ route_scatter_gather(const int32_t* __restrict__ topk_idx, const int32_t* __rest
 __global__ void __launch_bounds__(256)
 idx_chunk_histogram(const int32_t* __restrict__ topk_idx, int32_t* __restrict__ idx_ws, int T_tokens, int E, int K, int n_chunks,
                     int32_t* __restrict__ chunk_counts, int32_t* __restrict__ status) {
+  pdl_sync();
   const int lane = threadIdx.x & 31;
   const int chunk = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (chunk >= n_chunks) return;
@@ -435,6 +440,7 @@ idx_chunk_histogram(const int32_t* __restrict__ topk_idx, int32_t* __restrict__ 
 __global__ void __launch_bounds__(256)
 gather_rows(const uint4* __restrict__ x, uint4* __restrict__ x_perm, const int32_t* __restrict__ assign_of_row,
             const int32_t* __restrict__ pad_offsets, int E, int K, int vec_per_row, int rows_max) {
+  pdl_sync();
   const int lane = threadIdx.x & 31;
   const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (row >= rows_max || row >= pad_offsets[E]) return;
@@ -451,6 +457,7 @@ gather_rows(const uint4* __restrict__ x, uint4* __restrict__ x_perm, const int32
 // Padding rows of every expert segment set to zero (sixteen blocks share an expert's at most kTileM - 1 rows).
 __global__ void __launch_bounds__(256)
 zero_padding(uint4* __restrict__ buf, const int32_t* __restrict__ offsets, const int32_t* __restrict__ pad_offsets, int vec_per_row) {
+  pdl_sync();
   const int e = blockIdx.x;
   const int first = pad_offsets[e] + (offsets[e + 1] - offsets[e]), last = pad_offsets[e + 1];
   for (int r = first + blockIdx.y; r < last; r += gridDim.y)
@@ -460,7 +467,7 @@ zero_padding(uint4* __restrict__ buf, const int32_t* __restrict__ offsets, const
 }  // namespace
 
 cudaError_t launch_zero_padding(const rom_config& c, void* buf, int width, char* ws, const WsLayout& lay, cudaStream_t st) {
-  zero_padding<<<dim3(c.E, 16), 256, 0, st>>>(reinterpret_cast<uint4*>(buf), reinterpret_cast<const int32_t*>(ws + lay.offsets),
+  launch_k(zero_padding, dim3(c.E, 16), 256, 0, st, reinterpret_cast<uint4*>(buf), reinterpret_cast<const int32_t*>(ws + lay.offsets),
                                              reinterpret_cast<const int32_t*>(ws + lay.pad_offsets), (int)((size_t)width * lay.esz / 16));
   count_launch();
   return cudaGetLastError();
@@ -483,6 +490,7 @@ cudaError_t launch_route_gather(const rom_config& c, const void* x, const void* 
 __global__ void __launch_bounds__(64)
 balance_finish(const double* __restrict__ chunk_prob, const int32_t* __restrict__ counts, int n_chunks, int E, int T_tokens,
                float alpha, float* __restrict__ F, float* __restrict__ Pbar, float* __restrict__ loss) {
+  pdl_sync();
   __shared__ double term[kMaxE];
   const int e = threadIdx.x;
   if (e < E) {
@@ -506,7 +514,7 @@ cudaError_t launch_balance(const rom_config& c, const void* x, const void* W_r, 
   double* chunk_prob = reinterpret_cast<double*>(ws + lay.chunk_prob);
   cudaError_t err = launch_route_stats(c, x, W_r, b_r, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, ws, lay, chunk_prob, st, false);
   if (err != cudaSuccess) return err;
-  balance_finish<<<1, 64, 0, st>>>(chunk_prob, reinterpret_cast<const int32_t*>(ws + lay.counts), (int)lay.n_chunks, c.E, (int)lay.T,
+  launch_k(balance_finish, 1, 64, 0, st, chunk_prob, reinterpret_cast<const int32_t*>(ws + lay.counts), (int)lay.n_chunks, c.E, (int)lay.T,
                                   alpha, F, Pbar, loss);
   count_launch();
   return cudaGetLastError();
@@ -542,11 +550,11 @@ cudaError_t launch_route_stats(const rom_config& c, const void* x, const void* W
   const int idx_ints = RT * c.K > 3 * kMaxE + 2 ? RT * c.K : 3 * kMaxE + 2;
   const size_t smem = sizeof(double) * (size_t)(dsplit > 2 ? dsplit : 2) * RT * Epad8 + sizeof(int32_t) * idx_ints;
   if (bf)
-    route_logits_topk<__nv_bfloat16><<<blocks, threads, smem, st>>>(
+    launch_k(route_logits_topk<__nv_bfloat16>, blocks, threads, smem, st, 
         (const __nv_bfloat16*)x, (const __nv_bfloat16*)W_r, b_r, T, c.d_model, c.E, c.K, c.gate_mode, idx_ws, gates, chunk_counts,
         chunk_prob, probs, (int)lay.n_chunks, oa);
   else
-    route_logits_topk<float><<<blocks, threads, smem, st>>>(
+    launch_k(route_logits_topk<float>, blocks, threads, smem, st, 
         (const float*)x, (const float*)W_r, b_r, T, c.d_model, c.E, c.K, c.gate_mode, idx_ws, gates, chunk_counts, chunk_prob, probs,
         (int)lay.n_chunks, oa);
   count_launch();
@@ -568,12 +576,12 @@ static cudaError_t launch_scatter(const rom_config& c, const int32_t* idx_ws, in
     const cudaError_t e = current_device_sm_count(&num_sms);
     if (e != cudaSuccess) return e;
     const int grid = (int)lay.n_chunks > num_sms ? (int)lay.n_chunks : num_sms;
-    route_scatter_gather<<<grid, 256, 0, st>>>(idx_ws, chunk_base, offs, poffs, (int)lay.T, c.E, c.K, (int)lay.n_chunks, perm, inv_perm, roa, aor,
+    launch_k(route_scatter_gather, grid, 256, 0, st, idx_ws, chunk_base, offs, poffs, (int)lay.T, c.E, c.K, (int)lay.n_chunks, perm, inv_perm, roa, aor,
                                                            reinterpret_cast<const uint4*>(x), reinterpret_cast<uint4*>(ws + lay.x_perm),
                                                            (int)((size_t)c.d_model * lay.esz / 16));
   } else {
     const int wpb = 8;
-    route_scatter<<<((int)lay.n_chunks + wpb - 1) / wpb, wpb * 32, 0, st>>>(idx_ws, chunk_base, offs, poffs, (int)lay.T, c.E, c.K,
+    launch_k(route_scatter, ((int)lay.n_chunks + wpb - 1) / wpb, wpb * 32, 0, st, idx_ws, chunk_base, offs, poffs, (int)lay.T, c.E, c.K,
                                                                           (int)lay.n_chunks, perm, inv_perm, roa, aor);
   }
   count_launch();
@@ -586,7 +594,7 @@ static cudaError_t launch_perm_tables(const rom_config& c, const int32_t* idx_ws
   const OffsetsArgs oa{reinterpret_cast<int32_t*>(ws + lay.counts), reinterpret_cast<int32_t*>(ws + lay.offsets),
                        reinterpret_cast<int32_t*>(ws + lay.pad_offsets), reinterpret_cast<int32_t*>(ws + lay.num_m_tiles),
                        reinterpret_cast<int32_t*>(ws + lay.tile_expert), (int)lay.max_m_tiles, counts, offsets, nullptr, 0, nullptr};
-  route_offsets<<<1, 1024, 0, st>>>(reinterpret_cast<int32_t*>(ws + lay.chunk_counts), (int)lay.n_chunks, c.E, oa);
+  launch_k(route_offsets, 1, 1024, 0, st, reinterpret_cast<int32_t*>(ws + lay.chunk_counts), (int)lay.n_chunks, c.E, oa);
   count_launch();
   return launch_scatter(c, idx_ws, perm, inv_perm, ws, lay, nullptr, st);
 }
@@ -600,7 +608,7 @@ cudaError_t launch_gather_rows_to(const rom_config& c, const void* src, void* ds
   const int vec_per_row = (int)((size_t)width * lay.esz / 16);
   const int wpb = 8;
   const int blocks = (int)((lay.rows_max + wpb - 1) / wpb);
-  gather_rows<<<blocks, wpb * 32, 0, st>>>(reinterpret_cast<const uint4*>(src), reinterpret_cast<uint4*>(dst),
+  launch_k(gather_rows, blocks, wpb * 32, 0, st, reinterpret_cast<const uint4*>(src), reinterpret_cast<uint4*>(dst),
                                           reinterpret_cast<const int32_t*>(ws + lay.assign_of_row),
                                           reinterpret_cast<const int32_t*>(ws + lay.pad_offsets), c.E, c.K, vec_per_row,
                                           (int)lay.rows_max);
@@ -614,7 +622,7 @@ cudaError_t launch_perm_from_idx(const rom_config& c, const int32_t* topk_idx, i
   cudaError_t err = cudaMemsetAsync(ws + lay.assign_of_row, 0xff, sizeof(int32_t) * lay.rows_max, st);
   if (err != cudaSuccess) return err;
   const int wpb = 8;
-  idx_chunk_histogram<<<((int)lay.n_chunks + wpb - 1) / wpb, wpb * 32, 0, st>>>(
+  launch_k(idx_chunk_histogram, ((int)lay.n_chunks + wpb - 1) / wpb, wpb * 32, 0, st, 
       topk_idx, idx_ws, (int)lay.T, c.E, c.K, (int)lay.n_chunks, reinterpret_cast<int32_t*>(ws + lay.chunk_counts),
       reinterpret_cast<int32_t*>(ws + lay.status));
   count_launch();

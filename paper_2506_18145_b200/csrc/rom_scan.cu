@@ -125,6 +125,7 @@ struct Tile {
 template <typename T, typename TD, int NC, int NS, bool PRECISE, bool ZOH, int MODE>
 __global__ void __launch_bounds__(BLOCK, NS >= 8 ? 2 : 1)
 scan_kernel(const ScanArgs p) {
+  pdl_sync();
   using G = Geo<NC, NS>;
   using TileT = Tile<NC, NS>;
   constexpr int S = G::S, NP = G::NP, CH = G::CH, TS = G::TS, YP = G::YP;
@@ -429,6 +430,7 @@ scan_kernel(const ScanArgs p) {
 template <typename T, typename TD, bool PRECISE, bool ZOH>
 __global__ void __launch_bounds__(BLOCK)
 scan_step_kernel(const ScanArgs p) {
+  pdl_sync();
   const int c = blockIdx.x * BLOCK + threadIdx.x;
   const size_t b = blockIdx.y;
   if (c >= p.De) return;
@@ -487,6 +489,7 @@ scan_step_kernel(const ScanArgs p) {
 __global__ void __launch_bounds__(256)
 chain_chunk_states(const float* __restrict__ A, const float* __restrict__ h_end, const float* __restrict__ sum_delta,
                    float* __restrict__ h_in, float* __restrict__ h_last, int B, int De, int nch, int n_end) {
+  pdl_sync();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (long long)B * De * NST) return;
   const int n = (int)(i % NST);
@@ -509,7 +512,7 @@ cudaError_t launch_one(const ScanArgs& a, int B, int grid_z, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(scan_kernel<T, TD, NC, NS, PRECISE, ZOH, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   dim3 grid((a.De + G::CH - 1) / G::CH, B, grid_z);
-  scan_kernel<T, TD, NC, NS, PRECISE, ZOH, MODE><<<grid, BLOCK, smem, st>>>(a);
+  launch_k(scan_kernel<T, TD, NC, NS, PRECISE, ZOH, MODE>, grid, BLOCK, smem, st, a);
   count_launch();
   return cudaGetLastError();
 }
@@ -548,8 +551,8 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
   if (!CKPT && c.L == 1) {
     a.h0 = h0; a.h_last = h_last;
     dim3 grid((c.d_inner + BLOCK - 1) / BLOCK, c.B);
-    if (zoh) scan_step_kernel<T, TD, PRECISE, true><<<grid, BLOCK, 0, st>>>(a);
-    else scan_step_kernel<T, TD, PRECISE, false><<<grid, BLOCK, 0, st>>>(a);
+    if (zoh) launch_k(scan_step_kernel<T, TD, PRECISE, true>, grid, BLOCK, 0, st, a);
+    else launch_k(scan_step_kernel<T, TD, PRECISE, false>, grid, BLOCK, 0, st, a);
     count_launch();
     return cudaGetLastError();
   }
@@ -598,7 +601,7 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
   cudaError_t e = chunks(pa, n_end, FirstTag{});
   if (e != cudaSuccess) return e;
   const long long n_thr = (long long)c.B * c.d_inner * NST;
-  chain_chunk_states<<<(unsigned)((n_thr + 255) / 256), 256, 0, st>>>(A, h_end, sum_delta, h_in, h_last, c.B, c.d_inner, nch, n_end);
+  launch_k(chain_chunk_states, (unsigned)((n_thr + 255) / 256), 256, 0, st, A, h_end, sum_delta, h_in, h_last, c.B, c.d_inner, nch, n_end);
   count_launch();
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;

@@ -103,6 +103,7 @@ template <bool PRECISE> __device__ __forceinline__ float2 exp_pair(float2 x) {
 template <typename T, typename TD, bool ZOH>
 __global__ void __launch_bounds__(BT, BLOCKS_PER_SM)
 scan_bwd_kernel(const BwdArgs p) {
+  pdl_sync();
   constexpr bool PRECISE = sizeof(T) == 4;
   extern __shared__ __align__(16) unsigned char bwd_smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -375,6 +376,7 @@ struct PreSmem { float2 de[CK][32]; float4 c[CK][4]; };
 template <typename T, typename TD>
 __global__ void __launch_bounds__(BT)
 scan_bwd_prepass_kernel(const BwdArgs p) {
+  pdl_sync();
   constexpr bool PRECISE = sizeof(T) == 4;
   __shared__ PreSmem sm[WPB];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -457,6 +459,7 @@ scan_bwd_prepass_kernel(const BwdArgs p) {
 __global__ void __launch_bounds__(256)
 scan_bwd_chain_kernel(const float* __restrict__ A, const float* __restrict__ dh_last, const float* __restrict__ q_start,
                       const float* __restrict__ sum_delta, float* __restrict__ g_in, int B, int De, int ncc) {
+  pdl_sync();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (long long)B * De * NST) return;
   const int n = (int)(i % NST);
@@ -474,6 +477,7 @@ scan_bwd_chain_kernel(const float* __restrict__ A, const float* __restrict__ dh_
 __global__ void __launch_bounds__(256)
 scan_bwd_chain_states_kernel(const float* __restrict__ A, const float* __restrict__ h0, const float* __restrict__ h_end,
                              const float* __restrict__ sum_delta, float* __restrict__ h_in, int B, int De, int ncc) {
+  pdl_sync();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (long long)B * De * NST) return;
   const int n = (int)(i % NST);
@@ -520,6 +524,15 @@ size_t scan_bwd_ws_bytes(int B, int De, int L) {
   return align_up(sizeof(float) * floats, 256);
 }
 
+void scan_bwd_zero(const rom_config& c, const ScanBwd& s, ZeroList& z) {
+  auto add = [&](float* p, long long n) { if (p) { z.p[z.count] = p; z.n[z.count++] = n; } };
+  add(s.dA, (long long)c.d_inner * NST);
+  add(s.dBm, (long long)c.B * c.L * NST);
+  add(s.dCm, (long long)c.B * c.L * NST);
+  add(s.dD, c.d_inner);
+  add(s.dpre ? s.db_dt : nullptr, c.d_inner);
+}
+
 cudaError_t launch_scan_backward(const rom_config& c, const ScanBwd& s, cudaStream_t st) {
   const int nck = (c.L + CK - 1) / CK;
   int Lc = 0;
@@ -533,12 +546,7 @@ cudaError_t launch_scan_backward(const rom_config& c, const ScanBwd& s, cudaStre
   float* sum_delta_h = sum_delta + (size_t)c.B * ncc * c.d_inner;
   const BwdArgs a{s.dy, s.u, s.delta, s.A, s.Bm, s.Cm, s.D, s.z, s.dh_last, s.du, s.ddelta, s.dA, s.dBm, s.dCm, s.dD, s.dz, s.dh0, s.dpre, s.db_dt,
                   s.ckpt, c.L, c.d_inner, nck, s.ldz, s.dz_rows, s.K, Lc, ncc, g_in, q_start, sum_delta};
-  cudaError_t e = cudaMemsetAsync(s.dA, 0, sizeof(float) * (size_t)c.d_inner * NST, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(s.dBm, 0, sizeof(float) * (size_t)c.B * c.L * NST, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(s.dCm, 0, sizeof(float) * (size_t)c.B * c.L * NST, st);
-  if (e == cudaSuccess && s.dD) e = cudaMemsetAsync(s.dD, 0, sizeof(float) * (size_t)c.d_inner, st);
-  if (e == cudaSuccess && s.dpre) e = cudaMemsetAsync(s.db_dt, 0, sizeof(float) * (size_t)c.d_inner, st);
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
   const bool zoh = c.disc_mode == 0, bf = c.dtype == ROM_BF16;
   const long long n_thr = (long long)c.B * c.d_inner * NST;
   const unsigned chain_blocks = (unsigned)((n_thr + 255) / 256);
@@ -549,7 +557,7 @@ cudaError_t launch_scan_backward(const rom_config& c, const ScanBwd& s, cudaStre
     const float* h_start = s.h0;
     if (ncc > 1) {
       if ((e = launch_scan_states(c, s.u, delta, s.A, s.Bm, Lc, ncc, nullptr, h_end, sum_delta_h, nullptr, 0, st)) != cudaSuccess) return e;
-      scan_bwd_chain_states_kernel<<<chain_blocks, 256, 0, st>>>(s.A, s.h0, h_end, sum_delta_h, h_in, c.B, c.d_inner, ncc);
+      launch_k(scan_bwd_chain_states_kernel, chain_blocks, 256, 0, st, s.A, s.h0, h_end, sum_delta_h, h_in, c.B, c.d_inner, ncc);
       count_launch();
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       h_start = h_in;
@@ -559,12 +567,12 @@ cudaError_t launch_scan_backward(const rom_config& c, const ScanBwd& s, cudaStre
   const dim3 grid((c.d_inner + BCH - 1) / BCH, c.B, ncc);
   if (ncc > 1) {
     const dim3 pgrid(grid.x, grid.y, ncc - 1);
-    if (!bf) scan_bwd_prepass_kernel<float, float><<<pgrid, BT, 0, st>>>(a);
-    else if (s.delta_fp32) scan_bwd_prepass_kernel<__nv_bfloat16, float><<<pgrid, BT, 0, st>>>(a);
-    else scan_bwd_prepass_kernel<__nv_bfloat16, __nv_bfloat16><<<pgrid, BT, 0, st>>>(a);
+    if (!bf) launch_k(scan_bwd_prepass_kernel<float, float>, pgrid, BT, 0, st, a);
+    else if (s.delta_fp32) launch_k(scan_bwd_prepass_kernel<__nv_bfloat16, float>, pgrid, BT, 0, st, a);
+    else launch_k(scan_bwd_prepass_kernel<__nv_bfloat16, __nv_bfloat16>, pgrid, BT, 0, st, a);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    scan_bwd_chain_kernel<<<chain_blocks, 256, 0, st>>>(s.A, s.dh_last, q_start, sum_delta, g_in, c.B, c.d_inner, ncc);
+    launch_k(scan_bwd_chain_kernel, chain_blocks, 256, 0, st, s.A, s.dh_last, q_start, sum_delta, g_in, c.B, c.d_inner, ncc);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
@@ -572,7 +580,7 @@ cudaError_t launch_scan_backward(const rom_config& c, const ScanBwd& s, cudaStre
               : s.delta_fp32 ? (zoh ? scan_bwd_kernel<__nv_bfloat16, float, true> : scan_bwd_kernel<__nv_bfloat16, float, false>)
                              : (zoh ? scan_bwd_kernel<__nv_bfloat16, __nv_bfloat16, true> : scan_bwd_kernel<__nv_bfloat16, __nv_bfloat16, false>);
   if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, BWD_SMEM)) != cudaSuccess) return e;
-  kern<<<grid, BT, BWD_SMEM, st>>>(a);
+  launch_k(kern, grid, BT, BWD_SMEM, st, a);
   count_launch();
   return cudaGetLastError();
 }

@@ -74,6 +74,7 @@ __device__ __forceinline__ float raw_f32(__nv_bfloat16 v) { return __bfloat162fl
 template <typename TD, bool ZOH, int GATE, bool ROWS>
 __global__ void __launch_bounds__(Q_WARPS * 32, 1)
 scan_seq_kernel(const SeqArgs p) {
+  pdl_sync();
   using Stage = SeqStage<TD>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -301,7 +302,7 @@ cudaError_t launch_seq_k(const SeqArgs& a, int B, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   dim3 grid((a.De + Q_WARPS * Q_CH - 1) / (Q_WARPS * Q_CH), B);
-  kern<<<grid, Q_WARPS * 32, smem, st>>>(a);
+  launch_k(kern, grid, Q_WARPS * 32, smem, st, a);
   count_launch();
   return cudaGetLastError();
 }

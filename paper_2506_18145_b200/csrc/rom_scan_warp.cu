@@ -52,6 +52,7 @@ __device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
 template <typename TD, bool ZOH, int MODE>
 __global__ void __launch_bounds__(BT, 3)
 scan_warp_kernel(const ScanArgs p) {
+  pdl_sync();
   constexpr bool FIRST = MODE == SCAN_FIRST || MODE == SCAN_FIRST_CKPT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -234,7 +235,7 @@ scan_warp_kernel(const ScanArgs p) {
 template <typename TD, bool ZOH, int MODE>
 cudaError_t launch_mode(const ScanArgs& a, int B, int grid_z, cudaStream_t st) {
   constexpr int smem = WPB * (int)sizeof(WarpTile);
-  scan_warp_kernel<TD, ZOH, MODE><<<dim3((a.De + BT - 1) / BT, B, grid_z), BT, smem, st>>>(a);
+  launch_k(scan_warp_kernel<TD, ZOH, MODE>, dim3((a.De + BT - 1) / BT, B, grid_z), BT, smem, st, a);
   count_launch();
   return cudaGetLastError();
 }

@@ -79,6 +79,7 @@ __device__ __forceinline__ void split3(float v0, float v1, uint32_t& hi, uint32_
 template <bool STATE>
 __global__ void __launch_bounds__(BT, 1)
 ssd_kernel(const SsdArgs p) {
+  pdl_sync();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   using Smem = typename std::conditional<STATE, SsdStateSmem, SsdSmem>::type;
   Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
@@ -322,6 +323,7 @@ ssd_kernel(const SsdArgs p) {
 // Start state of every segment, in place over the end states: h_in[0] = 0, h_in[j + 1] = 2^s_seg[j] h_in[j] + h_end[j].
 __global__ void __launch_bounds__(256)
 ssd_chain(float* __restrict__ h_seg, const float* __restrict__ s_seg, int H, int nseg, long long total) {
+  pdl_sync();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;      // (sequence, head, element)
   if (i >= total) return;
   const int el = (int)(i & 1023);
@@ -387,16 +389,16 @@ cudaError_t launch_ssd(const rom_config& c, const void* xc, const float* Bm, con
   cudaError_t e;
   if (nseg > 1) {
     if ((e = cudaFuncSetAttribute(ssd_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SsdStateSmem))) != cudaSuccess) return e;
-    ssd_kernel<true><<<dim3(H / HPB, nseg - 1, c.B), BT, sizeof(SsdStateSmem), st>>>(a);
+    launch_k(ssd_kernel<true>, dim3(H / HPB, nseg - 1, c.B), BT, sizeof(SsdStateSmem), st, a);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const long long total = (long long)c.B * H * 1024;
-    ssd_chain<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(a.h_seg, a.s_seg, H, nseg, total);
+    launch_k(ssd_chain, (unsigned)((total + 255) / 256), 256, 0, st, a.h_seg, a.s_seg, H, nseg, total);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if ((e = cudaFuncSetAttribute(ssd_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SsdSmem))) != cudaSuccess) return e;
-  ssd_kernel<false><<<dim3(H / HPB, nseg, c.B), BT, sizeof(SsdSmem), st>>>(a);
+  launch_k(ssd_kernel<false>, dim3(H / HPB, nseg, c.B), BT, sizeof(SsdSmem), st, a);
   count_launch();
   return cudaGetLastError();
 }
