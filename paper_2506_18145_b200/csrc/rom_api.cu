@@ -42,7 +42,7 @@ WsLayout make_layout(const rom_config& c) {
   l.x_perm = take(l.esz * (size_t)l.rows_max * c.d_model);
   l.XZp = take(l.esz * (size_t)l.rows_max * 2 * c.d_inner);
   l.U = take(l.esz * (size_t)l.T * c.d_inner);
-  l.Zs = take(c.K > 1 ? l.esz * (size_t)l.T * c.d_inner : 0);   // gate rows summed over the K slots
+  l.Zs = take(c.K > 1 && !scan_sums_gate(c) ? l.esz * (size_t)l.T * c.d_inner : 0);   // gate rows summed over the K slots
   l.delta_r = take(l.esz * (size_t)l.T * R);
   l.Bm = take(sizeof(float) * (size_t)l.T * N);
   l.Cm = take(sizeof(float) * (size_t)l.T * N);
@@ -352,7 +352,8 @@ int layer_forward_impl(const rom_config* cfg, const rom_weights* w, const void* 
     ROM_CUDA(launch_conv_step(c, W + lay.XZp, in_token_order ? nullptr : row_of_assign, w->w_conv, w->b_conv, conv_state, W + lay.U,
                               c.K > 1 ? W + lay.Zs : nullptr, st));
   else
-    ROM_CUDA(launch_conv(c, W + lay.XZp, in_token_order ? nullptr : row_of_assign, w->w_conv, w->b_conv, W + lay.U, c.K > 1 ? W + lay.Zs : nullptr, st));
+    ROM_CUDA(launch_conv(c, W + lay.XZp, in_token_order ? nullptr : row_of_assign, w->w_conv, w->b_conv, W + lay.U,
+                         c.K > 1 && !scan_sums_gate(c) ? W + lay.Zs : nullptr, st));
   ROM_STAGE_DONE();
   if (c.small_proj_experts <= 1) {
     // S5: x Proj -> delta_r | B | C  (shared by all experts)
@@ -391,11 +392,14 @@ int layer_forward_impl(const rom_config* cfg, const rom_weights* w, const void* 
   }
   }      // !fused_small
   // S7 + S8 + S9: scan, gate, re-permute
-  // K = 1: the gate row of a token is its Gate Proj row in expert order; K > 1: the summed rows from S4
-  const char* zbase = c.K == 1 ? W + lay.XZp + (size_t)De * lay.esz : W + lay.Zs;
+  // K = 1: the gate row of a token is its Gate Proj row in expert order, activated; K > 1: the Gate Proj rows of its slots, summed and
+  // activated by the scan (bf16) or by S4 (rows of Zs)
+  const bool slots = scan_sums_gate(c);
+  const char* zbase = c.K == 1 || slots ? W + lay.XZp + (size_t)De * lay.esz : W + lay.Zs;
   ROM_CUDA(launch_scan(c, W + lay.U, W + lay.Delta, false, w->A, reinterpret_cast<float*>(W + lay.Bm),
-                       reinterpret_cast<float*>(W + lay.Cm), w->D, zbase, c.K == 1 ? 2 * De : De, (c.K == 1 && !in_token_order) ? row_of_assign : nullptr,
-                       ssm_state, W + lay.Ygp, ssm_state, row_of_assign, c.K, reinterpret_cast<float*>(W + lay.scan_ws), true, st));
+                       reinterpret_cast<float*>(W + lay.Cm), w->D, zbase, c.K == 1 || slots ? 2 * De : De,
+                       slots || (c.K == 1 && !in_token_order) ? row_of_assign : nullptr, ssm_state, W + lay.Ygp, ssm_state, row_of_assign, c.K,
+                       reinterpret_cast<float*>(W + lay.scan_ws), !slots, st));
   ROM_STAGE_DONE();
   // S10 + S11.  Tensor path with one expert per token: the epilogue of the grouped Out Proj scales each row by
   // its gate and writes it at its token's position (no intermediate rows, no combine pass).  Otherwise: grouped

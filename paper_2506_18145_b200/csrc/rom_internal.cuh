@@ -119,8 +119,10 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_sync() { pdl_wait(); pdl_trigger(); }
 
+// early == false: an ordinary launch, for grids of few blocks per SM whose balance matters: let in early, they would pile up on the
+// first SMs to drain (a scan of 256 blocks, three to an SM, took 40 % longer).
 template <typename... P, typename... Args>
-cudaError_t launch_k(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+cudaError_t launch_k(bool early, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -130,8 +132,12 @@ cudaError_t launch_k(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cud
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = early ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+template <typename... P, typename... Args>
+cudaError_t launch_k(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+  return launch_k(true, kern, grid, block, smem, st, args...);
 }
 
 // Zero up to 16 buffers (4-byte elements) in one launch.
@@ -249,7 +255,10 @@ bool step_small_applicable(const rom_config& c);
 cudaError_t launch_step_small(const rom_config& c, const rom_weights& w, const void* x, float* conv_state, float* ssm_state, void* out,
                               int32_t* topk_idx_out, float* gates, char* W, const WsLayout& lay, cudaStream_t st);
 
-// Scan.  z is a [rows, ldz] matrix; the gate row of token t is z_row[t] (z_row == nullptr: row t).
+// Whether launch_scan on a layer's activations (chunk workspace given) sums the K gate rows of a token itself: z_row [T, K].
+inline bool scan_sums_gate(const rom_config& c) { return c.dtype == ROM_BF16 && c.K > 1 && c.L > 1; }
+// Scan.  z is a [rows, ldz] matrix; the gate row of token t is z_row[t] (z_row == nullptr: row t).  With K > 1 and
+// scan_sums_gate: z_row is [T, K] and the gate is SiLU of the sum of those rows.
 // y_rows == nullptr: y is [T, d_inner]; otherwise the output row of token t is written K times, to rows
 // y_rows[t*K + k].
 // gate_activated: z already holds SiLU of the gate pre-activation (the producer applied it).

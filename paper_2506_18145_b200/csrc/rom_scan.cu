@@ -512,7 +512,7 @@ cudaError_t launch_one(const ScanArgs& a, int B, int grid_z, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(scan_kernel<T, TD, NC, NS, PRECISE, ZOH, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   dim3 grid((a.De + G::CH - 1) / G::CH, B, grid_z);
-  launch_k(scan_kernel<T, TD, NC, NS, PRECISE, ZOH, MODE>, grid, BLOCK, smem, st, a);
+  launch_k((long long)grid.x * grid.y * grid.z <= 148, scan_kernel<T, TD, NC, NS, PRECISE, ZOH, MODE>, grid, BLOCK, smem, st, a);
   count_launch();
   return cudaGetLastError();
 }

@@ -7,7 +7,7 @@ namespace rom {
 
 struct ScanArgs {
   const void* u; const void* delta; const float* A; const float* Bm; const float* Cm; const float* D;
-  const void* z; int ldz; const int32_t* z_row; const float* h0; void* y; float* h_last; const int32_t* y_rows;
+  const void* z; int ldz; const int32_t* z_row /* [T] or, warp kernel with K > 1, [T, K]: rows summed */; const float* h0; void* y; float* h_last; const int32_t* y_rows;
   int K, L, De;
   int Lc, nch;          // chunk length and chunks per sequence (nch == 1: Lc == L); blockIdx.z = chunk
   int L0;               // length of chunk 0; chunk j >= 1 covers steps [L0 + (j-1) Lc, L0 + j Lc)

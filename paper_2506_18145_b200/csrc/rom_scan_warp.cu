@@ -49,7 +49,8 @@ template <> struct Raw8<float> {
 };
 __device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
 
-template <typename TD, bool ZOH, int MODE>
+// SLOTS: the gate of a token is SiLU of the sum of its K >= 2 rows z_row[t K + k], which are also its output rows (y_rows).
+template <typename TD, bool ZOH, int MODE, bool SLOTS>
 __global__ void __launch_bounds__(BT, 3)
 scan_warp_kernel(const ScanArgs p) {
   pdl_sync();
@@ -108,17 +109,31 @@ scan_warp_kernel(const ScanArgs p) {
   const float4* cptr = reinterpret_cast<const float4*>(p.Cm + tok0 * NST) + lane;
 
   Raw8<TD> r_d;
-  Raw8<bf16> r_u, r_z, cur_u, cur_z;
+  Raw8<bf16> r_u, r_z, r_z2, cur_u, cur_z, cur_z2;
   float4 r_b, r_c;
-  int r_row = 0, cur_row = 0;      // first output row of this lane's step
+  int r_row = 0, cur_row = 0, r_row2 = 0, cur_row2 = 0;      // first output rows of this lane's step
+  int z_i0 = 0, z_i1 = 0;          // SLOTS: rows of the next tile to fetch: their indices are a tile ahead, so that nothing waits for them
+  auto fetch_rows = [&](int t0) {
+    if (SLOTS && t0 + lt < L) {
+      const int32_t* zr = p.z_row + (tok0 + t0 + lt) * p.K;
+      z_i0 = __ldg(zr);
+      z_i1 = __ldg(zr + 1);
+    }
+  };
   auto fetch = [&](int t0) {
     const int t = t0 + lt;
     const float4 zero4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (t < L) {
       r_d.load(dptr); r_u.load(uptr);
       if (!so) {
-        if (zp) r_z.load(zp + (p.z_row ? (size_t)__ldg(p.z_row + tok0 + t) : tok0 + t) * p.ldz + lc);
-        r_row = p.y_rows ? __ldg(p.y_rows + (tok0 + t) * p.K) : (int)(tok0 + t);
+        if constexpr (SLOTS) {     // gate rows by slot; the third and later ones are fetched where they are added
+          r_row = z_i0; r_row2 = z_i1;
+          r_z.load(zp + (size_t)z_i0 * p.ldz + lc);
+          r_z2.load(zp + (size_t)z_i1 * p.ldz + lc);
+        } else {
+          r_row = p.y_rows ? __ldg(p.y_rows + (tok0 + t) * p.K) : (int)(tok0 + t);
+          if (zp) r_z.load(zp + (p.z_row ? (size_t)__ldg(p.z_row + tok0 + t) : tok0 + t) * p.ldz + lc);
+        }
       }
     } else {                       // steps past the end change nothing
       r_d.zero(); r_u.zero();
@@ -128,11 +143,13 @@ scan_warp_kernel(const ScanArgs p) {
     r_b = in ? __ldg(bptr) : zero4;
     if (!so) r_c = in ? __ldg(cptr) : zero4;
     bptr += CK * 4; cptr += CK * 4;
+    if (SLOTS && !so) fetch_rows(t0 + CK);
   };
 
   auto run = [&](auto so_tag) {
     constexpr bool SO = decltype(so_tag)::value;
     constexpr bool CKPT = MODE == SCAN_CKPT || MODE == SCAN_FULL_CKPT || (MODE == SCAN_FIRST_CKPT && !SO);
+    if (SLOTS && !SO) fetch_rows(0);
     fetch(0);
     for (int t0 = 0; t0 < L; t0 += CK) {
       {
@@ -147,7 +164,7 @@ scan_warp_kernel(const ScanArgs p) {
         s.u[lt][(2 * l8) ^ lt] = make_float4(uu[0], uu[1], uu[2], uu[3]);
         s.u[lt][(2 * l8 + 1) ^ lt] = make_float4(uu[4], uu[5], uu[6], uu[7]);
         reinterpret_cast<float4*>(s.b)[lane] = r_b;
-        if (!SO) { reinterpret_cast<float4*>(s.c)[lane] = r_c; cur_u = r_u; cur_z = r_z; cur_row = r_row; }
+        if (!SO) { reinterpret_cast<float4*>(s.c)[lane] = r_c; cur_u = r_u; cur_z = r_z; cur_row = r_row; if (SLOTS) { cur_z2 = r_z2; cur_row2 = r_row2; } }
       }
       __syncwarp();
       if (t0 + CK < L) fetch(t0 + CK);
@@ -193,7 +210,20 @@ scan_warp_kernel(const ScanArgs p) {
           cur_u.get(uu);
           if (zp) {
             cur_z.get(zz);
-            if (!p.gate_activated) {
+            if (SLOTS) {
+              float z2[8];
+              cur_z2.get(z2);
+#pragma unroll
+              for (int i = 0; i < 8; ++i) zz[i] += z2[i];
+              for (int k = 2; k < p.K; ++k) {
+                V16<bf16> zk;
+                zk.load(zp + (size_t)__ldg(p.z_row + (tok0 + t) * p.K + k) * p.ldz + lc);
+                zk.get(z2);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) zz[i] += z2[i];
+              }
+            }
+            if (SLOTS || !p.gate_activated) {
 #pragma unroll
               for (int i = 0; i < 8; ++i) zz[i] = silu_fast(zz[i]);
             }
@@ -215,8 +245,9 @@ scan_warp_kernel(const ScanArgs p) {
           }
           bf16* y = static_cast<bf16*>(p.y) + lc;
           V16<bf16>::store(y + (size_t)cur_row * De, o);
+          if (SLOTS) V16<bf16>::store(y + (size_t)cur_row2 * De, o);
           if (p.y_rows)
-            for (int k = 1; k < p.K; ++k) V16<bf16>::store(y + (size_t)__ldg(p.y_rows + (tok0 + t) * p.K + k) * De, o);
+            for (int k = SLOTS ? 2 : 1; k < p.K; ++k) V16<bf16>::store(y + (size_t)__ldg(p.y_rows + (tok0 + t) * p.K + k) * De, o);
         }
         __syncwarp();
       }
@@ -235,7 +266,13 @@ scan_warp_kernel(const ScanArgs p) {
 template <typename TD, bool ZOH, int MODE>
 cudaError_t launch_mode(const ScanArgs& a, int B, int grid_z, cudaStream_t st) {
   constexpr int smem = WPB * (int)sizeof(WarpTile);
-  launch_k(scan_warp_kernel<TD, ZOH, MODE>, dim3((a.De + BT - 1) / BT, B, grid_z), BT, smem, st, a);
+  const dim3 grid((a.De + BT - 1) / BT, B, grid_z);
+  if (a.z_row && a.K > 1) {
+    if constexpr (sizeof(TD) == 2 && (MODE == SCAN_FULL || MODE == SCAN_FIRST)) launch_k(false, scan_warp_kernel<TD, ZOH, MODE, true>, grid, BT, smem, st, a);
+    else return cudaErrorInvalidValue;
+  } else {
+    launch_k(false, scan_warp_kernel<TD, ZOH, MODE, false>, grid, BT, smem, st, a);
+  }
   count_launch();
   return cudaGetLastError();
 }
