@@ -165,14 +165,17 @@ __device__ __forceinline__ void epi_softplus32(const Epilogue& ep, float* sw, in
   __syncwarp();
 }
 
-template <int MODE, int CG>
+// MN: which operands are MN-major tiles: MN_NONE, MN_B (data gradient on the weights as stored) or MN_BOTH (weight gradient).
+enum : int { MN_NONE = 0, MN_B = 1, MN_BOTH = 2 };
+template <int MODE, int CG, int MN>
 __global__ void __launch_bounds__(threads_of(MODE), 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
                int M_max, int N, int Kd, int block_n, uint32_t idesc,
                const int32_t* __restrict__ tile_expert, const int32_t* __restrict__ num_m_tiles_dev,
                Epilogue ep, int32_t* __restrict__ status, uint32_t wait_limit, int withhold_kb,
-               const int32_t* __restrict__ k_seg, int n_seg, int a_mn, int b_mn,
+               const int32_t* __restrict__ k_seg, int n_seg,
                const int32_t* __restrict__ pad_offsets, int n_experts) {
+  constexpr bool a_mn = MN == MN_BOTH, b_mn = MN != MN_NONE;
   constexpr int STAGES = stages_of(MODE, CG);
   constexpr int SB = stage_bytes_of(MODE, CG);      // bytes per operand stage (multiple of 1024)
   extern __shared__ unsigned char smem_raw[];
@@ -380,7 +383,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
           const uint64_t adesc = a_mn ? make_smem_desc_mn(sa) : make_smem_desc(sa);
           const uint64_t bdesc = b_mn ? make_smem_desc_mn(sa + A_STAGE_BYTES) : make_smem_desc(sa + A_STAGE_BYTES);
           // K-major: 16 elements = 32 bytes along K inside the swizzled row, +2 in the address field
-          const uint32_t astep = a_mn ? MN_KSTEP : 2u, bstep = b_mn ? MN_KSTEP : 2u;
+          constexpr uint32_t astep = a_mn ? MN_KSTEP : 2u, bstep = b_mn ? MN_KSTEP : 2u;
 #pragma unroll
           for (int k = 0; k < BLOCK_K / UMMA_K; ++k) {
             if constexpr (CG == 2) umma_bf16_pair(tmem_d, adesc + (uint64_t)(astep * k), bdesc + (uint64_t)(bstep * k), idesc, (kb | k) != 0 ? 1u : 0u);
@@ -583,10 +586,12 @@ cudaError_t launch_gemm_tc(const void* A, int lda, const void* Bw, int ldb, int 
   int num_sms = 0;
   cudaError_t e = current_device_sm_count(&num_sms);
   if (e != cudaSuccess) return e;
-  // CTA pairs for the large grouped products: a pair fetches each B tile once for 256 rows (per CTA 32 KB a stage instead of 48).
-  // An expert's last pair is half empty every other time: from eight 128-row tiles per expert on, that costs at most 6 %.
+  // CTA pairs: a pair fetches each B tile once for 256 rows (per CTA 32 KB a stage instead of 48).  An expert with an odd number of row
+  // tiles ends in a pair that is half empty; measured from 1 to 16 row tiles an expert, pairs are faster all the same (4300 tokens
+  // over 8 experts: 2-3 % of the layer) as long as the experts average a full tile; below that single CTAs spread over more SMs.
+  // (The dt Proj, two K blocks a tile, is slower on pairs: 69 us against 58 at 16384 x 4096.)
   const bool pair_mode = epi.mode == EPI_STORE || epi.mode == EPI_INPROJ || epi.mode == EPI_OUTPROJ || swiglu;
-  const int cg = pair_mode && pad_offsets && !test_stall && block_n == MAX_BLOCK_N && Kd >= 512 && M_max >= n_experts * 9 * BLOCK_M ? 2 : 1;
+  const int cg = pair_mode && pad_offsets && M_max >= n_experts * 2 * BLOCK_M && !test_stall && block_n == MAX_BLOCK_N ? 2 : 1;
   CUtensorMap ta, tb;
   if (!make_tmap(&ta, A, (uint64_t)M_max, (uint64_t)Kd, (uint64_t)lda, BLOCK_M)) return cudaErrorInvalidValue;
   const bool ok = b_mn ? make_tmap(&tb, Bw, (uint64_t)n_experts * Kd, (uint64_t)N, (uint64_t)ldb, BLOCK_K)
@@ -598,15 +603,20 @@ cudaError_t launch_gemm_tc(const void* A, int lda, const void* Bw, int ldb, int 
   auto go = [&](auto kern) {
     return launch_workers(kern, cg, (long long)(cg == 2 ? (m_tiles + n_experts) / 2 : m_tiles) * n_tiles, num_sms, threads_of(epi.mode),
                           smem_bytes_of(epi.mode, cg), st, ta, tb, M_max, N, Kd, block_n, make_idesc(block_n, false, b_mn, cg * BLOCK_M), tile_expert,
-                          num_m_tiles_dev, epi, status, test_stall ? WAIT_LIMIT_TEST : WAIT_LIMIT, test_stall ? 1 : -1, nullptr, 1, 0, b_mn ? 1 : 0,
+                          num_m_tiles_dev, epi, status, test_stall ? WAIT_LIMIT_TEST : WAIT_LIMIT, test_stall ? 1 : -1, nullptr, 1,
                           pad_offsets, n_experts);
   };
-  if (cg == 2) return go(epi.mode == EPI_STORE ? gemm_tc_kernel<EPI_STORE, 2> : epi.mode == EPI_INPROJ ? gemm_tc_kernel<EPI_INPROJ, 2>
-                         : epi.mode == EPI_OUTPROJ ? gemm_tc_kernel<EPI_OUTPROJ, 2> : gemm_tc_kernel<EPI_SWIGLU, 2>);
-  return go(epi.mode == EPI_STORE ? gemm_tc_kernel<EPI_STORE, 1> : epi.mode == EPI_XPROJ ? gemm_tc_kernel<EPI_XPROJ, 1>
-            : epi.mode == EPI_INPROJ ? gemm_tc_kernel<EPI_INPROJ, 1> : epi.mode == EPI_OUTPROJ ? gemm_tc_kernel<EPI_OUTPROJ, 1>
-            : epi.mode == EPI_F32 ? gemm_tc_kernel<EPI_F32, 1> : epi.mode == EPI_SWIGLU ? gemm_tc_kernel<EPI_SWIGLU, 1>
-            : epi.mode == EPI_SOFTPLUS_ROWS ? gemm_tc_kernel<EPI_SOFTPLUS_ROWS, 1> : gemm_tc_kernel<EPI_SOFTPLUS, 1>);
+  if (b_mn) {
+    if (epi.mode != EPI_STORE) return cudaErrorInvalidValue;      // data gradients leave as they are
+    return cg == 2 ? go(gemm_tc_kernel<EPI_STORE, 2, MN_B>) : go(gemm_tc_kernel<EPI_STORE, 1, MN_B>);
+  }
+  constexpr int NO = MN_NONE;
+  if (cg == 2) return go(epi.mode == EPI_STORE ? gemm_tc_kernel<EPI_STORE, 2, NO> : epi.mode == EPI_INPROJ ? gemm_tc_kernel<EPI_INPROJ, 2, NO>
+                         : epi.mode == EPI_OUTPROJ ? gemm_tc_kernel<EPI_OUTPROJ, 2, NO> : gemm_tc_kernel<EPI_SWIGLU, 2, NO>);
+  return go(epi.mode == EPI_STORE ? gemm_tc_kernel<EPI_STORE, 1, NO> : epi.mode == EPI_XPROJ ? gemm_tc_kernel<EPI_XPROJ, 1, NO>
+            : epi.mode == EPI_INPROJ ? gemm_tc_kernel<EPI_INPROJ, 1, NO> : epi.mode == EPI_OUTPROJ ? gemm_tc_kernel<EPI_OUTPROJ, 1, NO>
+            : epi.mode == EPI_F32 ? gemm_tc_kernel<EPI_F32, 1, NO> : epi.mode == EPI_SWIGLU ? gemm_tc_kernel<EPI_SWIGLU, 1, NO>
+            : epi.mode == EPI_SOFTPLUS_ROWS ? gemm_tc_kernel<EPI_SOFTPLUS_ROWS, 1, NO> : gemm_tc_kernel<EPI_SOFTPLUS, 1, NO>);
 }
 
 namespace {
@@ -651,8 +661,8 @@ cudaError_t launch_gemm_tc_wgrad(const void* X, const void* Y, int rows, const i
   }
   const int cg = seg && block_n == MAX_BLOCK_N && P >= 2 * BLOCK_M ? 2 : 1;
   const long long units = (long long)n_seg * ((P + cg * BLOCK_M - 1) / (cg * BLOCK_M)) * ((Q + block_n - 1) / block_n);
-  return launch_workers(cg == 2 ? gemm_tc_kernel<EPI_F32, 2> : gemm_tc_kernel<EPI_F32, 1>, cg, units, num_sms, threads_of(EPI_F32), smem_bytes_of(EPI_F32, cg), st,
-                        ta, tb, P, Q, rows, block_n, make_idesc(block_n, true, true, cg * BLOCK_M), nullptr, nullptr, epi, status, WAIT_LIMIT, -1, seg, n_seg, 1, 1,
+  return launch_workers(cg == 2 ? gemm_tc_kernel<EPI_F32, 2, MN_BOTH> : gemm_tc_kernel<EPI_F32, 1, MN_BOTH>, cg, units, num_sms, threads_of(EPI_F32), smem_bytes_of(EPI_F32, cg), st,
+                        ta, tb, P, Q, rows, block_n, make_idesc(block_n, true, true, cg * BLOCK_M), nullptr, nullptr, epi, status, WAIT_LIMIT, -1, seg, n_seg,
                         nullptr, 0);
 }
 
