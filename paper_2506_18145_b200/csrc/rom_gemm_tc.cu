@@ -19,7 +19,12 @@
 // the status word, waits (bounded) for its own copies and for the MMAs it already issued, frees its
 // TMEM and returns.
 //
-// Every TMA load here is a plain single-CTA load (no thread-block clusters).
+// CG = 2: a cluster of two CTAs (cta_group::2) works on one 256 x 256 tile, each staging its own 128 rows of A and half of B; the copies
+// of both count on the leader's barriers, the leader issues the MMAs, and each CTA drains its own half of the accumulator.  No load is
+// multicast.  What bounds it: the tensor pipe at the clock the power limit leaves (1430 TFLOP/s at 16384 x 8192 x 2048 in a cool
+// call, 0.86 of the measured cuBLAS burst; about the sustained cuBLAS rate in a loop), then the 3 to 12 % of padding rows.  One CTA
+// per tile took 433 us there, pairs 385 (415 before the issuing thread's descriptor steps were compile-time constants: with four
+// MMAs of 128 cycles a block it has 500 cycles for its wait, descriptors and commit).
 #include "rom_tc_ptx.cuh"
 
 namespace rom {

@@ -2,6 +2,9 @@
 // fused with the output gate y * SiLU(z) and with the re-permutation of the gated rows into expert
 // order (the routing decision of the Gate/Conv projections is reused for Out Proj, Section 4.2).
 //
+// This is the kernel of fp32 storage, of the scalar-decay block, and of a few bf16 channels without a workspace; bf16 otherwise runs
+// rom_scan_warp.cu.  The launch logic of all of them (chunks, chain, checkpoints) is here.
+//
 // State and arithmetic are fp32.  The recurrence is sequential in t, so the parallelism is
 // (sequence, channel, state).  One thread owns NS of the 16 states of NC adjacent channels
 // (registers, packed pairs); the S = 16/NS lanes of a channel group are adjacent.  Per state and step

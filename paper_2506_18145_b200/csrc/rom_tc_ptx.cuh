@@ -1,6 +1,6 @@
 // PTX wrappers and host helpers shared by the tcgen05 kernels (grouped GEMM, fused conv + x Proj + dt Proj):
-// mbarrier with bounded waits, TMA tile loads (plain single-CTA loads), tcgen05 MMA / commit / tensor-memory loads,
-// shared-memory matrix descriptors for 128-byte-swizzled K-major bf16 tiles, tensor-map encoding.
+// mbarrier with bounded waits, TMA tile loads (for one CTA or one of a CTA pair), tcgen05 MMA / commit / tensor-memory loads,
+// shared-memory matrix descriptors for 128-byte-swizzled bf16 tiles (K-major or MN-major), tensor-map encoding.
 #pragma once
 
 #include <cuda.h>
