@@ -46,7 +46,7 @@ inline int scan_chunks(int B, int De, int L) {
 }
 // Chunks per sequence of the warp kernel (rom_scan_warp.cu): the count with the smallest time by its measured pace.  A 128-channel
 // block takes 139 / 192 / 272 ns a step with one / two / three blocks on an SM (three fit), 115 / 161 / 230 ns state-only; more than
-// one chunk costs the state-only launch and about 12 us for the chain and the extra launches.  Chunks of at least 48 steps.  A
+// one chunk costs the state-only launch and about 7 us for the chained states and the extra launch.  Chunks of at least 48 steps.  A
 // function of the problem sizes only (148 SMs assumed), so that workspace sizing and the launch agree.
 inline int scan_warp_chunks(int B, int De, int L) {
   const long long blocks1 = (long long)B * ((De + 127) / 128);
@@ -60,7 +60,7 @@ inline int scan_warp_chunks(int B, int De, int L) {
   for (int n = 2; n <= 64 && L >= 48 * n; ++n) {
     const long long blocks = blocks1 * (n - 1);
     if (blocks > 148 * 12) break;
-    const double t = (double)L / (n - 0.3) * (pace(blocks, full) + pace(blocks, state)) + 12000.0;
+    const double t = (double)L / (n - 0.3) * (pace(blocks, full) + pace(blocks, state)) + 7000.0;
     if (t < best_t) { best_t = t; best = n; }
   }
   return best;

@@ -585,7 +585,8 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
     }
     return cudaErrorInvalidValue;
   }
-  // chunked, two launches.  Launch A: chunk 0 in full from the caller's state, chunks 1..n_end-1 state-only from zero; chain;
+  // chunked, two launches.  Launch A: chunk 0 in full from the caller's state, chunks 1..n_end-1 state-only from zero; chain (a kernel,
+  // or the prologue of launch B);
   // launch B: chunks 1..nch-1 in full from their true initial states.
   const size_t n_state = (size_t)c.B * nch * c.d_inner * NST;
   float* h_end = chunk_ws;
@@ -598,17 +599,23 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
   a.Lc = (int)align_up((size_t)ceil(x), align);
   a.L0 = (int)align_up((size_t)ceil(kFirstChunkRatio * x), align);
   a.nch = nch;
-  const int n_end = h_last ? nch : nch - 1;       // the last chunk's end state is only needed for h_last
+  // the last chunk's end state is only needed for h_last, which the warp kernel's second launch writes itself
+  const int n_end = h_last && !warp_kernel ? nch : nch - 1;
   ScanArgs pa = a;
   pa.h_last = h_end; pa.sum_delta = sum_delta; pa.chunk_off = 0;
   cudaError_t e = chunks(pa, n_end, FirstTag{});
   if (e != cudaSuccess) return e;
+  a.h0 = h_in; a.h_last = nullptr; a.chunk_off = 1;
+  if (warp_kernel) {      // its blocks chain the states before them on their own: 5 us less than the launch (4 x 2048 steps of 2048 channels)
+    a.h0 = nullptr; a.h_last = h_last; a.chain_end = h_end; a.chain_sum = sum_delta;
+    return chunks(a, nch - 1, FullTag{});
+  }
+  // (the general kernel's blocks, 2 states to a thread, would take 3 us longer for it than the launch, which overlaps its neighbours)
   const long long n_thr = (long long)c.B * c.d_inner * NST;
   launch_k(chain_chunk_states, (unsigned)((n_thr + 255) / 256), 256, 0, st, A, h_end, sum_delta, h_in, h_last, c.B, c.d_inner, nch, n_end);
   count_launch();
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  a.h0 = h_in; a.h_last = nullptr; a.chunk_off = 1;
   return chunks(a, nch - 1, FullTag{});
 }
 

@@ -18,6 +18,11 @@ struct ScanArgs {
   int nck;
   int scalar_a;         // A[c, :] is one value per channel (scalar-per-head decay of a Mamba2-style block): one exponential
                         // per channel and step instead of one per state (only with B-bar = Delta B)
+  // second launch of the chunked scan (SCAN_FULL, SCAN_FULL_CKPT): [B, nch, De, 16] end states of the chunks before (chunk 0: true;
+  // others: from a zero state) and their [B, nch, De] sums of Delta, from which a block chains its own initial state; h_last is then
+  // [B, De, 16], written by the last chunk
+  const float* chain_end;
+  const float* chain_sum;
 };
 
 // What a scan launch does.  SCAN_FULL: outputs.  SCAN_STATE: state only (h_last and sum_delta of every chunk).  SCAN_FIRST: first

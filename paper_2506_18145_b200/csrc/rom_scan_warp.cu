@@ -74,6 +74,7 @@ scan_warp_kernel(const ScanArgs p) {
   // ---- compute role: channels c0 .. c0+3 (pairs), states 4q .. 4q+3
   const int q = lane & 3, cg = lane >> 2;
   const int c0 = c_warp + 4 * cg;
+  constexpr bool SECOND = MODE == SCAN_FULL || MODE == SCAN_FULL_CKPT;      // may be the second launch of the chunked scan
   float2 a2[4][2], kin[4][2], h[4][2], sdel[2];
   {
     float av[4][4], hv[4][4];
@@ -84,6 +85,32 @@ scan_warp_kernel(const ScanArgs p) {
       if (p.h0 && !(FIRST && so)) h4 = reinterpret_cast<const float4*>(p.h0 + ((FIRST ? (size_t)blockIdx.y : sc) * De + c0 + i) * NST)[q];
       av[i][0] = a4.x; av[i][1] = a4.y; av[i][2] = a4.z; av[i][3] = a4.w;
       hv[i][0] = h4.x; hv[i][1] = h4.y; hv[i][2] = h4.z; hv[i][3] = h4.w;
+    }
+    if (SECOND && p.chain_end) {      // the state this chunk starts from: h <- exp(A sum Delta_j) h + h_end[j] over the chunks before
+      const size_t s0 = sc - chunk;
+      const float4 zero4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      for (int k0 = 0; k0 < chunk; k0 += 4) {      // four chunks' loads in flight; past the last one: the identity
+        float4 d4[4], e4[4][4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const size_t sk = s0 + k0 + k;
+          const bool in = k0 + k < chunk;
+          // (chunk 0's end state is the true one and nothing precedes it: its sum is not kept)
+          d4[k] = in && k0 + k > 0 ? __ldg(reinterpret_cast<const float4*>(p.chain_sum + sk * De + c0)) : zero4;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) e4[k][i] = in ? __ldg(reinterpret_cast<const float4*>(p.chain_end + (sk * De + c0 + i) * NST) + q) : zero4;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float dk[4] = {d4[k].x, d4[k].y, d4[k].z, d4[k].w};
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float ev[4] = {e4[k][i].x, e4[k][i].y, e4[k][i].z, e4[k][i].w};
+#pragma unroll
+            for (int n = 0; n < 4; ++n) hv[i][n] = fmaf(expf(av[i][n] * dk[i]), hv[i][n], ev[n]);
+          }
+        }
+      }
     }
 #pragma unroll
     for (int n = 0; n < 4; ++n)
@@ -260,8 +287,9 @@ scan_warp_kernel(const ScanArgs p) {
   else if constexpr (FIRST) { if (so) run(std::true_type{}); else run(std::false_type{}); }
   else run(std::false_type{});
 
-  if (p.h_last) {
-    put_state(p.h_last + sc * De * NST);
+  const bool chained = SECOND && p.chain_end;
+  if (p.h_last && (!chained || chunk == p.nch - 1)) {
+    put_state(p.h_last + (chained ? (size_t)blockIdx.y : sc) * De * NST);
     if (so && q == 0 && p.sum_delta) *reinterpret_cast<float4*>(p.sum_delta + sc * De + c0) = make_float4(sdel[0].x, sdel[0].y, sdel[1].x, sdel[1].y);
   }
 }

@@ -18,3 +18,9 @@ pytestmark = pytest.mark.gpu
 ])
 def test_scan_warp_chunked(disc_mode, B, L, De, with_z, with_h0, with_D):
     run_scan(B, L, De, "bf16", disc_mode, with_z, with_h0, with_D, seed=8800 + L, use_ws=True)
+
+
+@pytest.mark.parametrize("L", [200, 250, 300, 340, 390])
+def test_scan_warp_chained_states(L):
+    """Three to seven chunks after the first: every block chains the states before it, four at a time; h_last leaves with the last."""
+    run_scan(2, L, 64, "bf16", 0, True, True, True, seed=8900 + L, use_ws=True)
