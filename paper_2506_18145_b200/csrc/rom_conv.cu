@@ -217,6 +217,101 @@ conv_silu_kernel(const T* __restrict__ XZp, const int32_t* __restrict__ row_of_a
   }
 }
 
+// The same for many tokens and K = 1 or 2 in bf16, without the gate: a thread walks seg steps with the last four rows of H in registers
+// as packed fp32 pairs, and the next four rows are in flight while four are used (their indices four rows earlier still).  HBM-bound
+// (two or three 16-byte vectors per output vector); in the kernel above a thread loads 11 rows for 8 steps, computes, and ends, so that
+// loads and arithmetic overlap only between blocks and every row is widened for each of its four taps.  K = 2, 64 x 1024 steps of 3072
+// channels: 317 -> 239 us (5.1 TB/s), 8 x 4096 of 4096: 211 -> 163; K = 1, 16384 of 4096: 70 -> 61.  More blocks per SM (96 and 128
+// registers) spill and are slower than the kernel above.
+template <int KT>
+__global__ void __launch_bounds__(128, KT == 1 ? 4 : 3)
+conv_silu_roll_kernel(const __nv_bfloat16* __restrict__ XZp, const int32_t* __restrict__ row_of_assign, const __nv_bfloat16* __restrict__ w_conv,
+                      const float* __restrict__ b_conv, __nv_bfloat16* __restrict__ U, int L, int De, int dconv, int seg) {
+  typedef __nv_bfloat16 T;
+  pdl_sync();
+  const int c0 = (blockIdx.x * blockDim.x + threadIdx.x) * 8;
+  if (c0 >= De) return;
+  const int tb = blockIdx.y * seg, te = min(tb + seg, L);
+  const int ld = 2 * De;
+  const size_t tok0 = (size_t)blockIdx.z * L;
+  const T* __restrict__ H = XZp + c0;
+
+  auto index = [&](int t, int k) -> int32_t {      // rows outside the sequence: -1 (zeros)
+    if (t < 0 || t >= te) return -1;
+    return row_of_assign ? __ldg(row_of_assign + (tok0 + t) * KT + k) : (int32_t)(tok0 + t);
+  };
+  auto fetch = [&](RawVec<T>& r, int32_t ix) {
+    if (ix >= 0) r.load(H + (size_t)ix * ld);
+    else r.zero();
+  };
+  auto widen = [&](const RawVec<T> (&r)[KT], float2 (&h)[4]) {
+    float v[8];
+    r[0].get(v);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) h[i] = make_float2(v[2 * i], v[2 * i + 1]);
+    if constexpr (KT == 2) {
+      r[1].get(v);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) h[i] = __fadd2_rn(h[i], make_float2(v[2 * i], v[2 * i + 1]));
+    }
+  };
+
+  RawVec<T> nxt[4][KT], halo[3][KT];
+  int32_t ix[4][KT];
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+#pragma unroll
+    for (int k = 0; k < KT; ++k) fetch(halo[r][k], index(tb - 3 + r, k));
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int k = 0; k < KT; ++k) { fetch(nxt[r][k], index(tb + r, k)); ix[r][k] = index(tb + 4 + r, k); }
+
+  // taps right-aligned into 4 slots: slot 3 multiplies the current token
+  float2 w[4][4], bias[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int src = j - (4 - dconv);
+    float v[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    if (src >= 0) load_vec(w_conv + (size_t)src * De + c0, v);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[j][i] = make_float2(v[2 * i], v[2 * i + 1]);
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) bias[i] = b_conv ? __ldg(reinterpret_cast<const float2*>(b_conv + c0) + i) : make_float2(0.0f, 0.0f);
+
+  float2 h[4][4];      // row t of H in slot t & 3 (tb is a multiple of four)
+#pragma unroll
+  for (int r = 0; r < 3; ++r) widen(halo[r], h[r + 1]);
+  T* out = U + (tok0 + tb) * De + c0;
+  for (int t0 = tb; t0 < te; t0 += 4) {
+    RawVec<T> cur[4][KT];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int k = 0; k < KT; ++k) {
+        cur[r][k] = nxt[r][k];
+        fetch(nxt[r][k], ix[r][k]);
+        ix[r][k] = index(t0 + 8 + r, k);
+      }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      widen(cur[r], h[r]);
+      float u[8];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        float2 pre = bias[i];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) pre = __ffma2_rn(w[j][i], h[(r + 1 + j) & 3][i], pre);
+        u[2 * i] = silu_fast(pre.x);
+        u[2 * i + 1] = silu_fast(pre.y);
+      }
+      if (t0 + r < te) store_vec(out, u);
+      out += De;
+    }
+  }
+}
+
 // Single-token step of the short convolution: one thread = one 16-byte vector of channels of one sequence.
 // conv_state [B, dconv-1, De] fp32 holds H of the previous dconv-1 tokens, oldest first; it is shifted by one and
 // the new H appended.  Taps are applied in the same order as in conv_silu_kernel (right-aligned into 4 slots).
@@ -345,6 +440,19 @@ cudaError_t launch_conv_t(const rom_config& c, const void* XZp, const int32_t* r
   auto args = [&](auto kern) {
     launch_k(kern, grid, threads, 0, st, (const T*)XZp, row_of_assign, (const T*)w_conv, b_conv, (T*)U, (T*)Zs, c.L, c.d_inner, c.K, c.d_conv);
   };
+  if constexpr (sizeof(T) == 2) {
+    // 64 steps to a thread once that leaves three waves of four blocks per SM, else 32 (4 x 2048 steps of 2048 channels: 20 us, 22.6
+    // with 64); the short walk of the kernel above where even those do not give every SM a block
+    const long long cols = (long long)grid.x * c.B;
+    const int seg = cols * ((c.L + 63) / 64) >= 148 * 12 ? 64 : 32;
+    const dim3 g2(grid.x, (c.L + seg - 1) / seg, c.B);
+    if (c.K <= 2 && Zs == nullptr && cols * g2.y >= 148) {
+      launch_k(c.K == 1 ? conv_silu_roll_kernel<1> : conv_silu_roll_kernel<2>, g2, threads, 0, st, (const T*)XZp, row_of_assign,
+               (const T*)w_conv, b_conv, (T*)U, c.L, c.d_inner, c.d_conv, seg);
+      count_launch();
+      return cudaGetLastError();
+    }
+  }
   if (c.K == 1) args(conv_silu_kernel<T, 1>);
   else if (c.K == 2) args(conv_silu_kernel<T, 2>);
   else args(conv_silu_kernel<T, 0>);
