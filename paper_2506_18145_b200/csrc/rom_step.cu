@@ -68,7 +68,10 @@ step_route(const bf16* __restrict__ x, const bf16* __restrict__ W_r, const float
     for (int d = (warp * 32 + lane) * 8; d < Dm; d += 2048) {
       V16<bf16> q;
       float xv[8];
+      double xd[8];                     // widened before the product, as in the forward's router: exact whatever the operands' exponents
       q.load(x + (size_t)t * Dm + d); q.get(xv);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) xd[i] = (double)xv[i];
       V16<bf16> wq[8];
 #pragma unroll
       for (int e = 0; e < 8; ++e) wq[e].load(W_r + (size_t)min(e0 + e, E - 1) * Dm + d);
@@ -77,7 +80,7 @@ step_route(const bf16* __restrict__ x, const bf16* __restrict__ W_r, const float
         float wv[8];
         wq[e].get(wv);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) acc[e] += (double)(xv[i] * wv[i]);      // bf16 products are exact in fp32
+        for (int i = 0; i < 8; ++i) acc[e] = fma(xd[i], (double)wv[i], acc[e]);
       }
     }
     // transposed sums over the lanes: 8 values -> lane keeps value (lane & 7) after three exchanges, then two plain ones

@@ -1,8 +1,15 @@
 """Edges of the bf16 single-token step's own kernels (few tokens per expert) against the CPU oracle: the register-fed and the
 streamed projections on both sides of their dispatch line, one to several passes of 64 token columns, 16 / 32 / 64 columns, a K
 range that leaves half a stage, weight tiles cut short, dt ranks off the 32- and 128-wide blocks, every conv width."""
+import numpy as np
 import pytest
+import torch
 
+from oracle import rom_oracle as O
+from paper_2506_18145_b200 import binding as rb
+from paper_2506_18145_b200 import synth
+
+from rom_testlib import np64
 from test_gpu_parity import run_steps, small_shape
 
 pytestmark = pytest.mark.gpu
@@ -20,3 +27,31 @@ pytestmark = pytest.mark.gpu
 ])
 def test_step_small_parity(kw):
     run_steps(small_shape(**{**dict(L=4, dtype="bf16"), **kw}), 3)
+
+
+def one_step(s, p, B, flags=0):
+    """One token for the first B sequences of p from seeded states; (out, conv_state, ssm_state, idx, gates, workspace)."""
+    cfg = rb.config_from_shape(s.replace(B=B, L=1), flags=flags)
+    dev = {k: (None if v is None else v.cuda().contiguous()) for k, v in p.items()}
+    conv = synth._randn(771, (s.B, s.d_conv - 1, s.d_inner))[:B].cuda()
+    ssm = synth._randn(772, (s.B, s.d_inner, s.d_state), 0.3)[:B].cuda()
+    out = torch.empty((B, s.d_model), dtype=synth.torch_dtype(s), device="cuda")
+    idx = torch.empty((B, s.K), dtype=torch.int32, device="cuda")
+    gates = torch.empty((B, s.K), dtype=torch.float32, device="cuda")
+    ws = rb.alloc_workspace(cfg, "cuda")
+    rb.rom_layer_step(cfg, rb.make_weights(dev), dev["x"][:B, 0].contiguous(), conv, ssm, out, idx, gates, ws)
+    torch.cuda.synchronize()
+    return out, conv, ssm, idx, gates, ws
+
+
+@pytest.mark.parametrize("scale", [2.0 ** -80, 2.0 ** -68, 2.0 ** 70])
+@pytest.mark.parametrize("B", [2, 9])
+def test_step_route_products_outside_fp32(B, scale):
+    """Router products below and above the range of fp32: logits are fp64 sums of exact products, so the routing is the oracle's."""
+    s = small_shape(B=B, L=1, E=8, K=2, d_model=320, dtype="bf16")
+    p = synth.make_inputs(s, recipe="unit")
+    p["x"], p["W_r"], p["W_inz"] = p["x"] * scale, p["W_r"] * scale, torch.zeros_like(p["W_inz"])
+    _, _, _, idx, gates, _ = one_step(s, p, B)
+    ref_idx, ref_gate, _, _ = O.route(np64(p["x"]).reshape(B, s.d_model), np64(p["W_r"]), None, s.K, 0)
+    np.testing.assert_array_equal(idx.cpu().numpy(), ref_idx)
+    np.testing.assert_allclose(gates.cpu().numpy(), ref_gate, rtol=2e-6, atol=1e-30)
