@@ -265,6 +265,9 @@ ROM_API int rom_layer_forward_host(const rom_config *cfg, const rom_weights *w, 
  *   ssm_state  : [B, d_inner, d_state] fp32, in/out: h_{t-1}; zeros at the start of a sequence
  * Feeding a sequence token by token from zero states reproduces rom_layer_forward on the whole sequence
  * (up to the rounding of the storage dtype).  topk_idx_out [B,K], gates_out [B,K] may be NULL.
+ * bf16 (small_proj_experts <= 1, no flags, d_r a multiple of 16, B <= 512, B*K <= 2048): a sequence's result does not depend on the
+ * other sequences of the batch, to the last bit, among all calls of fewer than four assignments (B*K) and among all calls of
+ * four and more; the two differ by fp32 rounding order.
  * ws: rom_workspace_size(cfg) bytes.                                                               */
 ROM_API int rom_layer_step(const rom_config *cfg, const rom_weights *w, const void *x, float *conv_state,
                    float *ssm_state, void *out, int32_t *topk_idx_out, float *gates_out,

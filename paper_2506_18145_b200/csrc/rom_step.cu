@@ -366,9 +366,10 @@ step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_
   const int tpe = (p.n_rows + p.tile_rows - 1) / p.tile_rows;      // weight tiles per expert
   const int total = n_act_s * tpe;
   const int num_kb = (p.Kd + 2 * BLOCK_K - 1) / (2 * BLOCK_K);      // stages of 128; d_model may leave half of the last one
-  // every CTA starts at its own K block: in step they would all read the same 128-byte column of rows that are a power of two apart
-  const int rot = (blockIdx.x * 5) % num_kb;
-  auto k_of = [&](int kb) { return (kb + rot < num_kb ? kb + rot : kb + rot - num_kb) * 2 * BLOCK_K; };
+  // every weight tile starts at its own K block: in step the CTAs would all read the same 128-byte column of rows that are a power of two
+  // apart.  The start depends on the tile's rows alone, so a token's sums do not depend on the CTA, i.e. on the batch around it.
+  auto rot_of = [&](int w) { return (w % tpe * 5) % num_kb; };
+  auto k_of = [&](int kb, int rot) { return (kb + rot < num_kb ? kb + rot : kb + rot - num_kb) * 2 * BLOCK_K; };
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer of the weights (nothing here depends on the launch before)
@@ -376,11 +377,11 @@ step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_
     int stage = 0, issued = 0; uint32_t phase = 0;
     bool ok = true;
     for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
-      const int e = act[w / tpe], row = e * p.n_rows + (w % tpe) * p.tile_rows;
+      const int e = act[w / tpe], row = e * p.n_rows + (w % tpe) * p.tile_rows, rot = rot_of(w);
       for (int n0 = 0; n0 < cnt[e] && ok; n0 += TC_N)
         for (int kb = 0; kb < num_kb; ++kb) {
           if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, WAIT_LIMIT)) { ok = false; break; }
-          const int k0 = k_of(kb);
+          const int k0 = k_of(kb, rot);
           mbar_expect_tx(full_bar(stage), 2 * p.tile_rows * BLOCK_K * 2);
           tma_load_2d(base + stage * TC_STAGE, &tmap_w, full_bar(stage), k0, row);
           tma_load_2d(base + stage * TC_STAGE + TC_W_HALF, &tmap_w, full_bar(stage), k0 + BLOCK_K, row);
@@ -407,7 +408,7 @@ step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_
       int acc = 0; uint32_t acc_phase = 0;
       bool ok = true, issued_any = false;
       for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
-        const int e = act[w / tpe];
+        const int e = act[w / tpe], rot = rot_of(w);
         for (int n0 = 0; n0 < cnt[e] && ok; n0 += TC_N) {
           const int n16 = cols(min(cnt[e] - n0, TC_N));
           const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n16 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
@@ -416,7 +417,7 @@ step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_
           for (int kb = 0; kb < num_kb; ++kb) {
             if (!mbar_wait(full_bar(stage), phase, abort_flag, WAIT_LIMIT)) { ok = false; break; }
             tc_fence_after();
-            const int halves = k_of(kb) + BLOCK_K < p.Kd ? 2 : 1;
+            const int halves = k_of(kb, rot) + BLOCK_K < p.Kd ? 2 : 1;
             for (int hf = 0; hf < halves; ++hf) {
               const uint64_t adesc = make_smem_desc(base + stage * TC_STAGE + hf * TC_W_HALF);
               const uint64_t bdesc = make_smem_desc(base + stage * TC_STAGE + TC_A_BYTES + hf * TC_X_HALF);
@@ -457,7 +458,7 @@ step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_
       --pending;
     };
     for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
-      const int e = act[w / tpe];
+      const int e = act[w / tpe], rot = rot_of(w);
       for (int n0 = 0; n0 < cnt[e] && ok; n0 += TC_N) {
         const int m = min(cnt[e] - n0, TC_N), nq = cols(m) >> 4;      // 16-row groups: 1, 2 or 4 pieces per thread and stage
         const bf16* src[4];
@@ -467,7 +468,7 @@ step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_
           ok = __all_sync(0xffffffffu, mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, WAIT_LIMIT));
           if (!ok) break;
           const uint32_t dst = base + stage * TC_STAGE + TC_A_BYTES + lrow * 128 + ((chunk ^ (lrow & 7)) << 4);
-          const int k0 = k_of(kb);
+          const int k0 = k_of(kb, rot);
 #pragma unroll
           for (int q = 0; q < 4; ++q)
             if (q < nq) {
@@ -750,13 +751,14 @@ cudaError_t launch_step_tc(const StepGemmArgs& a, int num_sms, int32_t* status, 
   return launch_chained_smem(step_tc<MODE>, dim3(num_sms), TC_THREADS, TC_SMEM, st, true, tw, a, status);
 }
 
-// Rows per weight tile: the multiple of 16 in 96 .. 128 for which the CTAs' rounds x rows is smallest when every expert that can be
-// selected is (d_model 2048, 8 experts: 112 rows make the in_proj 4.0 rounds of tiles, where 128 need 4 rounds for 3.46).
-int pick_tile_rows(int slots, int n_rows, int num_sms) {
+// Rows per weight tile: the multiple of 16 in 96 .. 128 for which the CTAs' rounds x rows is smallest when every expert is selected
+// (d_model 2048, 8 experts: 112 rows make the in_proj 4.0 rounds of tiles, where 128 need 4 rounds for 3.46).  Not a function of the
+// batch, which would show in the last bits of every token's result.
+int pick_tile_rows(int E, int n_rows, int num_sms) {
   int best = 128;
   long long cost = -1;
   for (int h = 128; h >= 96; h -= 16) {
-    const long long tiles = (long long)slots * ((n_rows + h - 1) / h), c = (tiles + num_sms - 1) / num_sms * h;
+    const long long tiles = (long long)E * ((n_rows + h - 1) / h), c = (tiles + num_sms - 1) / num_sms * h;
     if (cost < 0 || c < cost) { cost = c; best = h; }
   }
   return best;
@@ -799,7 +801,7 @@ cudaError_t launch_step_small(const rom_config& c, const rom_weights& w, const v
   if ((e = current_device_sm_count(&num_sms)) != cudaSuccess) return e;
   int32_t* status = reinterpret_cast<int32_t*>(W + lay.status);
   const bool stream = B * K >= kStreamMin;
-  a.tile_rows = pick_tile_rows(slots, 2 * De, num_sms);
+  a.tile_rows = pick_tile_rows(c.E, 2 * De, num_sms);
   if (stream) e = launch_step_tc<STEP_IN>(a, num_sms, status, st);
   else e = launch_step_gemm<STEP_IN, 2, 8>(a, dim3(2 * De / 32, slots), st);
   if (e != cudaSuccess) return e;
@@ -814,7 +816,7 @@ cudaError_t launch_step_small(const rom_config& c, const rom_weights& w, const v
   StepGemmArgs ao{};
   ao.x = Yg; ao.ldx = De; ao.W = (const bf16*)w.W_out; ao.Kd = De; ao.n_rows = Dm; ao.idx = idx; ao.gates = gates; ao.B = B; ao.K = K; ao.E = c.E;
   ao.C = K == 1 ? (bf16*)out : Op; ao.ldc = Dm;
-  ao.tile_rows = pick_tile_rows(slots, Dm, num_sms);
+  ao.tile_rows = pick_tile_rows(c.E, Dm, num_sms);
   if (stream) e = launch_step_tc<STEP_OUT>(ao, num_sms, status, st);
   else e = launch_step_gemm<STEP_OUT, 1, 16>(ao, dim3(Dm / 16, slots), st);
   if (e != cudaSuccess) return e;

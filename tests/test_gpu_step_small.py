@@ -55,3 +55,15 @@ def test_step_route_products_outside_fp32(B, scale):
     ref_idx, ref_gate, _, _ = O.route(np64(p["x"]).reshape(B, s.d_model), np64(p["W_r"]), None, s.K, 0)
     np.testing.assert_array_equal(idx.cpu().numpy(), ref_idx)
     np.testing.assert_allclose(gates.cpu().numpy(), ref_gate, rtol=2e-6, atol=1e-30)
+
+
+@pytest.mark.parametrize("K,sizes", [(1, (4, 9, 70)), (2, (2, 7, 64))])
+def test_step_result_does_not_depend_on_the_batch(K, sizes):
+    """From four assignments on, a sequence's output and states are the same to the last bit whatever the batch around it."""
+    s = small_shape(B=sizes[-1], L=1, E=8, K=K, d_model=1024, d_inner=2048, dtype="bf16")
+    p = synth.make_inputs(s, recipe="unit")
+    ref = one_step(s, p, sizes[-1])
+    for B in sizes[:-1]:
+        got = one_step(s, p, B)
+        for name, a, b in zip(("out", "conv state", "ssm state", "idx", "gates"), got, ref):
+            assert torch.equal(a, b[:B]), f"{name}: {B} against {sizes[-1]} sequences"
