@@ -9,7 +9,10 @@
  *     library allocates no device memory and keeps no state on the device between calls.  The one
  *     exception is rom_route_noalloc: its scratch is an array resident in the library's device image, so
  *     overlapping calls of it on one GPU must be serialised by the caller (see its own comment).
- *   - All tensors are dense, row-major, channels-last; device pointers must be 16-byte aligned.
+ *   - All tensors are dense, row-major, channels-last; device pointers must be 16-byte aligned.  The
+ *     alignment of the elements (4 bytes) is enough for the fp32 vectors b_r, b_conv, dt_bias and D,
+ *     for b_dt on the fp32 and plain-FMA paths and in rom_layer_step with the shared dt Proj, for h0 and h_last of rom_scan,
+ *     for db_r and dD, and for routing outputs (topk_idx, gates, counts, offsets, perm, inv_perm, F, Pbar, loss).
  *   - "dtype" tensors are stored as ROM_F32 (float) or ROM_BF16 (bfloat16) as rom_config.dtype says.
  *   - Calls are asynchronous on `stream` (a cudaStream_t passed as void*; NULL = default stream);
  *     they neither synchronise the host nor copy device memory to the host.

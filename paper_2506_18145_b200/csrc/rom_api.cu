@@ -111,6 +111,19 @@ int check_config(const rom_config* c, int which) {
 namespace {
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+template <size_t N>
+bool all_aligned4(const void* const (&ptrs)[N]) {
+  for (const void* p : ptrs)
+    if (!aligned4(p)) return false;
+  return true;
+}
+// The vectors of a layer that need the alignment of their elements only, and b_dt, which the tensor path's output ops and the
+// slot sums of the per-expert small projections read 16 bytes at a time (small_step: the single-token step's own kernels do not).
+bool layer_vectors_ok(const rom_config& c, const rom_weights& w, bool small_step) {
+  const void* const ptrs[] = {w.b_r, w.b_conv, w.b_dt, w.D};
+  const bool wide_b_dt = !small_step && ((c.dtype == ROM_BF16 && !(c.flags & ROM_FLAG_SIMT_GEMM)) || c.small_proj_experts > 1);
+  return all_aligned4(ptrs) && (!wide_b_dt || aligned16(w.b_dt));
+}
 
 int check_device() {
   int dev = 0;
@@ -176,7 +189,8 @@ int rom_route(const rom_config* cfg, const void* x, const void* W_r, const float
   int rc = check_config(cfg, 1);
   if (rc != ROM_OK) return rc;
   if (!x || !W_r || !ws) return ROM_ERR_INVALID_ARG;
-  if (!aligned16(x) || !aligned16(W_r) || !aligned16(ws)) return ROM_ERR_INVALID_ARG;
+  const void* const small[] = {b_r, topk_idx, gates, counts, offsets, perm, inv_perm};
+  if (!aligned16(x) || !aligned16(W_r) || !aligned16(ws) || !all_aligned4(small)) return ROM_ERR_INVALID_ARG;
   const WsLayout lay = make_layout(*cfg);
   if (ws_bytes < lay.total) return ROM_ERR_WORKSPACE;
   if ((rc = check_device()) != ROM_OK) return rc;
@@ -192,7 +206,8 @@ int rom_route_balance(const rom_config* cfg, const void* x, const void* W_r, con
   int rc = check_config(cfg, 1);
   if (rc != ROM_OK) return rc;
   if (!x || !W_r || !ws) return ROM_ERR_INVALID_ARG;
-  if (!aligned16(x) || !aligned16(W_r) || !aligned16(ws)) return ROM_ERR_INVALID_ARG;
+  const void* const small[] = {b_r, F, Pbar, loss};
+  if (!aligned16(x) || !aligned16(W_r) || !aligned16(ws) || !all_aligned4(small)) return ROM_ERR_INVALID_ARG;
   const WsLayout lay = make_layout(*cfg);
   if (ws_bytes < lay.total) return ROM_ERR_WORKSPACE;
   if ((rc = check_device()) != ROM_OK) return rc;
@@ -208,7 +223,7 @@ int rom_scan(const rom_config* cfg, const void* u, const float* delta, const flo
   if (rc != ROM_OK) return rc;
   if (!u || !delta || !A || !Bm || !Cm || !y) return ROM_ERR_INVALID_ARG;
   if (!aligned16(u) || !aligned16(delta) || !aligned16(A) || !aligned16(Bm) || !aligned16(Cm) || !aligned16(y) ||
-      (z && !aligned16(z)))
+      (z && !aligned16(z)) || !aligned4(D) || !aligned4(h0) || !aligned4(h_last))
     return ROM_ERR_INVALID_ARG;
   if ((rc = check_device()) != ROM_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -243,6 +258,7 @@ int rom_scan_backward(const rom_config* cfg, const void* dy, const void* u, cons
   const void* ptrs[] = {dy, u, delta, A, Bm, Cm, du, ddelta, dA, dBm, dCm, ws, z, dz, h0, dh_last, dh0};
   for (const void* p : ptrs)
     if (p && !aligned16(p)) return ROM_ERR_INVALID_ARG;
+  if (!aligned4(D) || !aligned4(dD)) return ROM_ERR_INVALID_ARG;
   if (ws_bytes < scan_bwd_ws_bytes(cfg->B, cfg->d_inner, cfg->L)) return ROM_ERR_WORKSPACE;
   if ((rc = check_device()) != ROM_OK) return rc;
   LaunchCounter::count = 0;
@@ -278,6 +294,9 @@ int layer_forward_impl(const rom_config* cfg, const rom_weights* w, const void* 
   const void* ptrs[] = {x, out, ws, w->W_r, w->W_inz, w->w_conv, w->W_x, w->W_dt, w->A, w->W_out};
   for (const void* p : ptrs)
     if (!aligned16(p)) return ROM_ERR_INVALID_ARG;
+  const void* const small[] = {topk_idx_out, gates_out, counts_out};
+  const bool small_step = conv_state && !ev && step_small_applicable(*cfg);      // single-token step with its own short launch sequence
+  if (!all_aligned4(small) || !layer_vectors_ok(*cfg, *w, small_step)) return ROM_ERR_INVALID_ARG;
   const rom_config& c = *cfg;
   const WsLayout lay = make_layout(c);
   if (ws_bytes < lay.total) return ROM_ERR_WORKSPACE;
@@ -294,8 +313,7 @@ int layer_forward_impl(const rom_config* cfg, const rom_weights* w, const void* 
   int32_t* row_of_assign = reinterpret_cast<int32_t*>(W + lay.row_of_assign);
   float* gates = gates_out ? gates_out : reinterpret_cast<float*>(W + lay.gates);
 
-  // single-token step with few tokens per expert: its own short launch sequence
-  if (conv_state && !ev && step_small_applicable(c)) {
+  if (small_step) {
     ROM_CUDA(launch_step_small(c, *w, x, conv_state, ssm_state, out, topk_idx_out, gates, W, lay, st));
     return ROM_OK;
   }
@@ -492,6 +510,7 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
                         g->db_conv, g->dW_x, g->dW_dt, g->db_dt, g->dA, g->dW_out};
   for (const void* p : ptrs)
     if (!aligned16(p)) return ROM_ERR_INVALID_ARG;
+  if (!aligned4(g->db_r) || !aligned4(g->dD) || !layer_vectors_ok(*cfg, *w, false)) return ROM_ERR_INVALID_ARG;
   const rom_config& c = *cfg;
   const WsLayout lay = make_layout(c);
   const BwdLayout bl = make_bwd_layout(c, lay);

@@ -278,7 +278,7 @@ conv_silu_roll_kernel(const __nv_bfloat16* __restrict__ XZp, const int32_t* __re
     for (int i = 0; i < 4; ++i) w[j][i] = make_float2(v[2 * i], v[2 * i + 1]);
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) bias[i] = b_conv ? __ldg(reinterpret_cast<const float2*>(b_conv + c0) + i) : make_float2(0.0f, 0.0f);
+  for (int i = 0; i < 4; ++i) bias[i] = b_conv ? make_float2(__ldg(b_conv + c0 + 2 * i), __ldg(b_conv + c0 + 2 * i + 1)) : make_float2(0.0f, 0.0f);
 
   float2 h[4][4];      // row t of H in slot t & 3 (tb is a multiple of four)
 #pragma unroll

@@ -24,6 +24,8 @@ constexpr int kStatTicket = 8;     // router: blocks-done counter (zero between 
 constexpr int kMaxCanaries = 40;   // sub-buffers of the workspace (debug checks put a canary after each)
 constexpr int kCanaryBytes = 256;
 
+// The caller's fp32 vectors (b_r, b_conv, D), scan states and index / gate outputs need the alignment of their elements only.
+inline bool aligned4(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 3u) == 0; }
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // Chunks per sequence of the selective scan: 1 when batch x channels already gives the GPU about 2048 warps at
@@ -340,6 +342,16 @@ __device__ __forceinline__ float ex2_ftz(float x) { float y; asm("ex2.approx.ftz
 __device__ __forceinline__ float lg2_ftz(float x) { float y; asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 __device__ __forceinline__ float rcp_ftz(float x) { float y; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 __device__ __forceinline__ float silu_fast(float v) { return v * rcp_ftz(1.0f + ex2_ftz(-1.4426950408889634f * v)); }
+
+// four floats of a caller's array that may start at any of them
+__device__ __forceinline__ float4 load4_any(const float* p) {
+  if ((reinterpret_cast<uintptr_t>(p) & 15u) == 0) return *reinterpret_cast<const float4*>(p);
+  return make_float4(p[0], p[1], p[2], p[3]);
+}
+__device__ __forceinline__ void store4_any(float* p, float4 v) {
+  if ((reinterpret_cast<uintptr_t>(p) & 15u) == 0) *reinterpret_cast<float4*>(p) = v;
+  else { p[0] = v.x; p[1] = v.y; p[2] = v.z; p[3] = v.w; }
+}
 
 // 16 bytes of consecutive elements as floats
 template <typename T> struct V16;

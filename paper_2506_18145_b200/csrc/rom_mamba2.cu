@@ -296,6 +296,9 @@ int rom_mamba2_layer_forward(const rom_config* cfg, int32_t headdim, const rom_m
   const void* ptrs[] = {x, out, ws, w->W_r, w->W_in, w->w_conv, w->A, w->w_norm, w->W_out};
   for (const void* p : ptrs)
     if (!aligned16(p)) return ROM_ERR_INVALID_ARG;
+  const void* small[] = {w->b_r, w->b_conv, w->dt_bias, w->D, topk_idx_out, gates_out, counts_out};
+  for (const void* p : small)
+    if (!aligned4(p)) return ROM_ERR_INVALID_ARG;
   const rom_config& c = *cfg;
   const M2Layout m = make_m2_layout(c, headdim);
   const WsLayout& lay = m.t;

@@ -81,6 +81,9 @@ extern "C" int rom_route_noalloc(const rom_config* cfg, const void* x, const voi
   if (cfg_rc != ROM_OK) return cfg_rc;
   const rom_config& c = *cfg;
   if ((reinterpret_cast<uintptr_t>(x) & 15u) || (reinterpret_cast<uintptr_t>(W_r) & 15u)) return ROM_ERR_INVALID_ARG;
+  const void* small[] = {b_r, topk_idx, gates, counts, offsets, perm, inv_perm};
+  for (const void* p : small)
+    if (!aligned4(p)) return ROM_ERR_INVALID_ARG;
   // the built-in scratch has a fixed size: larger problems must use rom_route with a caller workspace
   if ((int64_t)c.B * c.L > kNoAllocMaxTokens || (int64_t)c.B * c.L * c.K > kNoAllocMaxAssign) return ROM_ERR_STATIC_SCRATCH;
   const WsLayout lay = make_route_only_layout(c);

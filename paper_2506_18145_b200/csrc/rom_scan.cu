@@ -443,13 +443,13 @@ scan_step_kernel(const ScanArgs p) {
   const float4* Bq = reinterpret_cast<const float4*>(p.Bm + b * NST);
   const float4* Cq = reinterpret_cast<const float4*>(p.Cm + b * NST);
   const float4* Aq = reinterpret_cast<const float4*>(p.A + (size_t)c * NST);
-  const float4* Hq = p.h0 ? reinterpret_cast<const float4*>(p.h0 + (b * p.De + c) * NST) : nullptr;
-  float4* Ho = p.h_last ? reinterpret_cast<float4*>(p.h_last + (b * p.De + c) * NST) : nullptr;
+  const float* Hq = p.h0 ? p.h0 + (b * p.De + c) * NST : nullptr;
+  float* Ho = p.h_last ? p.h_last + (b * p.De + c) * NST : nullptr;
   float y = 0.0f;
 #pragma unroll
   for (int q = 0; q < NST / 4; ++q) {
     const float4 a4 = __ldg(Aq + q), b4 = __ldg(Bq + q), c4 = __ldg(Cq + q);
-    const float4 h4 = Hq ? Hq[q] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    const float4 h4 = Hq ? load4_any(Hq + 4 * q) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     const float av[4] = {a4.x, a4.y, a4.z, a4.w}, bv[4] = {b4.x, b4.y, b4.z, b4.w}, cv[4] = {c4.x, c4.y, c4.z, c4.w};
     float hv[4] = {h4.x, h4.y, h4.z, h4.w};
 #pragma unroll
@@ -469,7 +469,7 @@ scan_step_kernel(const ScanArgs p) {
       }
       y = fmaf(cv[i], hv[i], y);
     }
-    if (Ho) Ho[q] = make_float4(hv[0], hv[1], hv[2], hv[3]);
+    if (Ho) store4_any(Ho + 4 * q, make_float4(hv[0], hv[1], hv[2], hv[3]));
   }
   if (p.D) y = fmaf(p.D[c], uu, y);
   if (p.z) {

@@ -290,8 +290,7 @@ scan_seq_kernel(const SeqArgs p) {
   }
 
   if (p.h_last) {
-    float4* dst = reinterpret_cast<float4*>(p.h_last + ((size_t)b * De + c) * NST + 4 * g);
-    *dst = make_float4(h[0].x, h[0].y, h[1].x, h[1].y);
+    store4_any(p.h_last + ((size_t)b * De + c) * NST + 4 * g, make_float4(h[0].x, h[0].y, h[1].x, h[1].y));
   }
 }
 

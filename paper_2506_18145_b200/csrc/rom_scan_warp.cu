@@ -30,6 +30,7 @@ constexpr float kLog2e = 1.4426950408889634f;
 struct WarpTile {
   float4 dl[CK][8], u[CK][8];     // Delta, u of 4 channels; group g of step r sits at g ^ r
   float4 b[CK][4], c[CK][4];
+  float D[WCH];                   // skip factors (zeros without)
   float4 y[CK][32];               // partial sums of 4 channels over one lane's states; lane l of step r at ysw(l, r)
 };
 
@@ -82,7 +83,7 @@ scan_warp_kernel(const ScanArgs p) {
     for (int i = 0; i < 4; ++i) {
       const float4 a4 = __ldg(reinterpret_cast<const float4*>(p.A + (size_t)(c0 + i) * NST) + q);
       float4 h4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      if (p.h0 && !(FIRST && so)) h4 = reinterpret_cast<const float4*>(p.h0 + ((FIRST ? (size_t)blockIdx.y : sc) * De + c0 + i) * NST)[q];
+      if (p.h0 && !(FIRST && so)) h4 = load4_any(p.h0 + ((FIRST ? (size_t)blockIdx.y : sc) * De + c0 + i) * NST + 4 * q);
       av[i][0] = a4.x; av[i][1] = a4.y; av[i][2] = a4.z; av[i][3] = a4.w;
       hv[i][0] = h4.x; hv[i][1] = h4.y; hv[i][2] = h4.z; hv[i][3] = h4.w;
     }
@@ -122,13 +123,15 @@ scan_warp_kernel(const ScanArgs p) {
       }
     sdel[0] = make_float2(0.0f, 0.0f); sdel[1] = sdel[0];
   }
-  auto put_state = [&](float* dst) {      // [De, 16] state array of one (sequence, chunk or checkpoint)
+  auto put_state = [&](float* dst, auto any_tag) {      // [De, 16] state array of one (sequence, chunk or checkpoint); any: the caller's
+    auto put = [&](float* at, float4 v) { if constexpr (decltype(any_tag)::value) store4_any(at, v); else *reinterpret_cast<float4*>(at) = v; };
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      *reinterpret_cast<float4*>(dst + (size_t)(c0 + 2 * j) * NST + 4 * q) = make_float4(h[0][j].x, h[1][j].x, h[2][j].x, h[3][j].x);
-      *reinterpret_cast<float4*>(dst + (size_t)(c0 + 2 * j + 1) * NST + 4 * q) = make_float4(h[0][j].y, h[1][j].y, h[2][j].y, h[3][j].y);
+      put(dst + (size_t)(c0 + 2 * j) * NST + 4 * q, make_float4(h[0][j].x, h[1][j].x, h[2][j].x, h[3][j].x));
+      put(dst + (size_t)(c0 + 2 * j + 1) * NST + 4 * q, make_float4(h[0][j].y, h[1][j].y, h[2][j].y, h[3][j].y));
     }
   };
+  s.D[lane] = p.D ? __ldg(p.D + c_warp + lane) : 0.0f;
   // ---- loader / output role: step lt of every tile, channels lc .. lc+7
   // (four lanes per row: a load's quarter-warp touches two rows of global memory, not eight)
   const int lt = lane >> 2, l8 = lane & 3, lc = c_warp + 8 * l8;
@@ -198,7 +201,7 @@ scan_warp_kernel(const ScanArgs p) {
       }
       __syncwarp();
       if (t0 + CK < L) fetch(t0 + CK);
-      if constexpr (CKPT) put_state(p.ckpt + ((size_t)blockIdx.y * p.nck + (size_t)((t_first + t0) / CK)) * De * NST);
+      if constexpr (CKPT) put_state(p.ckpt + ((size_t)blockIdx.y * p.nck + (size_t)((t_first + t0) / CK)) * De * NST, std::false_type{});
       // the next step's operands are requested before this step's arithmetic: a load issued behind a step's exponentials waits
       // for all of them in the queue that both share
       float4 nd = s.dl[0][cg], nu = s.u[0][cg], nb = s.b[0][q], nc = SO ? make_float4(0.0f, 0.0f, 0.0f, 0.0f) : s.c[0][q];
@@ -262,7 +265,7 @@ scan_warp_kernel(const ScanArgs p) {
           for (int hf = 0; hf < 2; ++hf) {
             const int g4 = 8 * l8 + 4 * hf;
             const float4 x0 = s.y[lt][ysw(g4, lt)], x1 = s.y[lt][ysw(g4 + 1, lt)], x2 = s.y[lt][ysw(g4 + 2, lt)], x3 = s.y[lt][ysw(g4 + 3, lt)];
-            const float4 D4 = p.D ? __ldg(reinterpret_cast<const float4*>(p.D + lc) + hf) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            const float4 D4 = reinterpret_cast<const float4*>(s.D)[2 * l8 + hf];
             float2 v0 = __fadd2_rn(__fadd2_rn(make_float2(x0.x, x0.y), make_float2(x1.x, x1.y)), __fadd2_rn(make_float2(x2.x, x2.y), make_float2(x3.x, x3.y)));
             float2 v1 = __fadd2_rn(__fadd2_rn(make_float2(x0.z, x0.w), make_float2(x1.z, x1.w)), __fadd2_rn(make_float2(x2.z, x2.w), make_float2(x3.z, x3.w)));
             v0 = __ffma2_rn(make_float2(D4.x, D4.y), make_float2(uu[4 * hf], uu[4 * hf + 1]), v0);
@@ -289,7 +292,7 @@ scan_warp_kernel(const ScanArgs p) {
 
   const bool chained = SECOND && p.chain_end;
   if (p.h_last && (!chained || chunk == p.nch - 1)) {
-    put_state(p.h_last + (chained ? (size_t)blockIdx.y : sc) * De * NST);
+    put_state(p.h_last + (chained ? (size_t)blockIdx.y : sc) * De * NST, std::true_type{});
     if (so && q == 0 && p.sum_delta) *reinterpret_cast<float4*>(p.sum_delta + sc * De + c0) = make_float4(sdel[0].x, sdel[0].y, sdel[1].x, sdel[1].y);
   }
 }

@@ -278,7 +278,7 @@ step_gemm(const StepGemmArgs p) {
           const __nv_bfloat162 hb = __floats2bfloat162_rn(v.x, v.y);
           const float2 h = __bfloat1622float2(hb);
           float* st = p.conv_state + (size_t)a * (p.dconv - 1) * p.De + row;
-          float2 u = p.b_conv ? *reinterpret_cast<const float2*>(p.b_conv + row) : make_float2(0.0f, 0.0f);
+          float2 u = p.b_conv ? make_float2(p.b_conv[row], p.b_conv[row + 1]) : make_float2(0.0f, 0.0f);
           float2 win[3];
           for (int q = 0; q < p.dconv - 1; ++q) win[q] = *reinterpret_cast<const float2*>(st + (size_t)q * p.De);
           for (int q = 0; q < p.dconv; ++q) {
@@ -590,7 +590,7 @@ step_conv(const bf16* __restrict__ XZ, int K, int De, const bf16* __restrict__ w
   float* st = conv_state + b * (size_t)(dconv - 1) * De + c;
   float2 win[3], w[4], u = make_float2(0.0f, 0.0f);
   if (in) {                                          // the window and the taps do not depend on the launch before
-    if (b_conv) u = *reinterpret_cast<const float2*>(b_conv + c);
+    if (b_conv) u = make_float2(b_conv[c], b_conv[c + 1]);
     for (int q = 0; q < dconv - 1; ++q) win[q] = *reinterpret_cast<const float2*>(st + (size_t)q * De);
     for (int q = 0; q < dconv; ++q) w[q] = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(w_conv + (size_t)q * De + c));
   }

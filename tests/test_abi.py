@@ -97,3 +97,47 @@ def test_no_device_means_an_error_not_a_fallback(L):
     need = rb.workspace_size(cfg)
     rc = L.rom_layer_forward(ctypes.byref(cfg), ctypes.byref(w), 4096, 4096, None, None, None, 4096, need, None)
     assert rc in (-4, -5)      # CUDA call failed / wrong device: never a silent CPU path
+
+
+def test_alignment_of_vectors_is_checked_on_the_host(L):
+    """Elements' alignment for b_r, b_conv, D and the routing outputs; 16 bytes for b_dt where the kernels read it so; what passes the
+    check fails here only for want of a device (with a device these made-up pointers must not get that far)."""
+    import torch
+    if torch.cuda.is_available():
+        pytest.skip("a GPU is present")
+    names = [n for n, _ in rb.RomWeights._fields_]
+
+    def forward(cfg, at=None, off=0, outs=(None, None, None), step=False):
+        w = rb.RomWeights(*([4096] * 11))
+        if at:
+            setattr(w, at, 4096 + off)
+        need = rb.workspace_size(cfg)
+        if step:
+            return L.rom_layer_step(ctypes.byref(cfg), ctypes.byref(w), 4096, 4096, 4096, 4096, outs[0], outs[1], 4096, need, None)
+        return L.rom_layer_forward(ctypes.byref(cfg), ctypes.byref(w), 4096, 4096, *outs, 4096, need, None)
+
+    assert set(("b_r", "b_conv", "b_dt", "D")) <= set(names)
+    bf, f32 = _cfg(), _cfg(dtype="f32")
+    for cfg in (bf, f32):
+        for n in ("b_r", "b_conv", "D"):
+            assert forward(cfg, n, 4) in (-4, -5), n
+            assert forward(cfg, n, 2) == -1, n
+        for i in range(3):
+            outs = [None, None, None]
+            outs[i] = 4100
+            assert forward(cfg, outs=outs) in (-4, -5)
+            outs[i] = 4097
+            assert forward(cfg, outs=outs) == -1
+    assert forward(bf, "b_dt", 4) == -1
+    assert forward(f32, "b_dt", 4) in (-4, -5)
+    assert forward(_cfg(flags=rb.ROM_FLAG_SIMT_GEMM), "b_dt", 4) in (-4, -5)
+    assert forward(_cfg(dtype="f32", small_proj_experts=4), "b_dt", 4) == -1
+    assert forward(_cfg(L=1), "b_dt", 4, step=True) in (-4, -5)
+    assert forward(_cfg(L=1, small_proj_experts=4), "b_dt", 4, step=True) == -1
+
+    def scan(D=4096, h0=4096, h_last=4096):
+        return L.rom_scan(ctypes.byref(bf), 4096, 4096, 4096, 4096, 4096, D, None, h0, 4096, h_last, None, 0, None)
+    for kw in (dict(D=4100), dict(h0=4100), dict(h_last=4104)):
+        assert scan(**kw) in (-4, -5)
+    for kw in (dict(D=4097), dict(h0=4098), dict(h_last=4099)):
+        assert scan(**kw) == -1
