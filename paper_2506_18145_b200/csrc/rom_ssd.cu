@@ -9,7 +9,11 @@
 //
 // Precision: x enters exactly; every other operand is computed in fp32 and fed as the sum of three bf16 terms (24 bits), products
 // accumulate in fp32 -- the tensor cores replace fp32 arithmetic, not its precision.  (Terms of the state product below 2^-24 of
-// the leading one are dropped: six of nine.)
+// the leading one are dropped: six of nine.)  S_t - S_s is a difference of running sums, and an fp32 sum would leave the decay
+// between two late steps with the rounding of all that came before (units of S, where the recurrence has those of S_t - S_s): S_t is
+// summed in fp64 and kept as two floats, the low one of s folded into dt_s.  Steps of a decay below 2^-256 count as 2^-256: a product
+// with one of them is 0 in fp32 either way, and |S| stays below 2^14.  (One more fp32 addition per table entry: recurrence 251 -> 254 us
+// at 16384 steps of 4096 channels.)
 //
 // A warp owns one head of one segment of the sequence and carries h (64 x 16, fp32) in accumulator registers; everything is kept
 // transposed (Y^T = X^T G^T, h^T) so that h^T is the A operand of the next chunk as it stands and G^T, C and B fragments are
@@ -34,12 +38,12 @@ struct SsdSmem {
   bf16 z[HPB][Q * P];
   float cb[Q * CBP];                                 // [t][s]
   float Bt[NST * NP], Ct[NST * NP];                  // [n][step]
-  float S[HPB][Q], dt[HPB][Q];                       // running sum of dt A log2(e); dt
+  float S[HPB][Q], Sl[HPB][Q], dt[HPB][Q];           // running sum of dt A log2(e), its low part; dt 2^-Sl
 };
 struct SsdStateSmem {
   bf16 x[HPB][2][Q * P];
   float Bt[NST * NP];
-  float S[HPB][Q], dt[HPB][Q];
+  float S[HPB][Q], Sl[HPB][Q], dt[HPB][Q];
 };
 
 struct SsdArgs {
@@ -136,20 +140,27 @@ ssd_kernel(const SsdArgs p) {
         if constexpr (!STATE) sm.Ct[(q4 + i) * NP + r] = cv[i];
       }
       // dt and the running sum of dt A (base-2 logarithm of the decay); steps past the end of the sequence do nothing
-      float d[2], s[2];
+      float d[2];
+      double s[2];
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         d[j] = c * Q + lane + 32 * j < p.L ? softplus_f(to_f32(rd[j]) + bias) : 0.0f;
-        s[j] = d[j] * a2;
+        const float x = d[j] * a2;
+        s[j] = x < -256.0f ? -256.0 : (double)x;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-          const float v = __shfl_up_sync(0xffffffffu, s[j], o);
+          const double v = __shfl_up_sync(0xffffffffu, s[j], o);
           if (lane >= o) s[j] += v;
         }
       }
       s[1] += __shfl_sync(0xffffffffu, s[0], 31);
-      sm.S[warp][lane] = s[0]; sm.S[warp][lane + 32] = s[1];
-      sm.dt[warp][lane] = d[0]; sm.dt[warp][lane + 32] = d[1];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const float hi = (float)s[j], lo = (float)(s[j] - (double)hi);
+        sm.S[warp][lane + 32 * j] = hi;
+        sm.Sl[warp][lane + 32 * j] = lo;
+        sm.dt[warp][lane + 32 * j] = d[j] * exp2f(-lo);
+      }
     }
     if (c + 1 < c_hi) fetch_small(c + 1);
     asm volatile("cp.async.wait_group 1;" ::: "memory");      // x of this chunk (committed an iteration ago)
@@ -227,9 +238,10 @@ ssd_kernel(const SsdArgs p) {
             const int jt = 4 * th + tj;
             if (jt < 2 * ks) continue;               // (warp-uniform) all of it is above the diagonal
             const int t = 8 * jt + g;
-            const float St = Sw[t];
+            const float St = Sw[t], Sl = sm.Sl[warp][t];
             const float2 q0 = *reinterpret_cast<const float2*>(sm.cb + t * CBP + s0), q1 = *reinterpret_cast<const float2*>(sm.cb + t * CBP + s0 + 8);
-            float v[4] = {q0.x * ex2_ftz(St - S0.x) * d0.x, q0.y * ex2_ftz(St - S0.y) * d0.y, q1.x * ex2_ftz(St - S1.x) * d1.x, q1.y * ex2_ftz(St - S1.y) * d1.y};
+            float v[4] = {q0.x * ex2_ftz((St - S0.x) + Sl) * d0.x, q0.y * ex2_ftz((St - S0.y) + Sl) * d0.y,
+                          q1.x * ex2_ftz((St - S1.x) + Sl) * d1.x, q1.y * ex2_ftz((St - S1.y) + Sl) * d1.y};
             if (jt < 2 * ks + 2) {                   // on the diagonal: later steps out, the skip term in
               const int sv[4] = {s0, s0 + 1, s0 + 8, s0 + 9};
 #pragma unroll
@@ -279,7 +291,7 @@ ssd_kernel(const SsdArgs p) {
     }
 
     // ---- the state after the chunk
-    const float S63 = Sw[Q - 1], dec = ex2_ftz(S63);
+    const float S63 = Sw[Q - 1], Sl63 = sm.Sl[warp][Q - 1], dec = ex2_ftz(S63);
     s_total += S63;
 #pragma unroll
     for (int m = 0; m < 4; ++m)
@@ -294,7 +306,8 @@ ssd_kernel(const SsdArgs p) {
       const int s0 = 16 * ks + 2 * t4;
       const float2 S0 = *reinterpret_cast<const float2*>(Sw + s0), S1 = *reinterpret_cast<const float2*>(Sw + s0 + 8);
       const float2 d0 = *reinterpret_cast<const float2*>(dw + s0), d1 = *reinterpret_cast<const float2*>(dw + s0 + 8);
-      const float f[4] = {ex2_ftz(S63 - S0.x) * d0.x, ex2_ftz(S63 - S0.y) * d0.y, ex2_ftz(S63 - S1.x) * d1.x, ex2_ftz(S63 - S1.y) * d1.y};
+      const float f[4] = {ex2_ftz((S63 - S0.x) + Sl63) * d0.x, ex2_ftz((S63 - S0.y) + Sl63) * d0.y,
+                          ex2_ftz((S63 - S1.x) + Sl63) * d1.x, ex2_ftz((S63 - S1.y) + Sl63) * d1.y};
 #pragma unroll
       for (int nt = 0; nt < 2; ++nt) {
         const float2 b0 = *reinterpret_cast<const float2*>(sm.Bt + (8 * nt + g) * NP + s0), b1 = *reinterpret_cast<const float2*>(sm.Bt + (8 * nt + g) * NP + s0 + 8);
