@@ -84,9 +84,10 @@ typedef struct {
                                  the SM) instead of three launches.  Same results up to rounding.  Off by default: as
                                  measured it is slower than the three launches (instruction-issue bound on one CTA per
                                  128 tokens); ignored where the sizes do not fit (d_r > 128, d_r + 2 D_s > 160)          */
-#define ROM_FLAG_TEST_STALL 4 /* fault injection for tests of the device-side timeout path (tensor path only): the
-                                 first grouped projection withholds the copies of one operand stage per CTA and
-                                 every device wait gives up after 2^14 polls instead of 2^22, so the call returns
+#define ROM_FLAG_TEST_STALL 4 /* fault injection for tests of the device-side timeout path (tensor path only; needs
+                                 d_model > 64, and > 128 for rom_layer_step of four assignments and more): the
+                                 first grouped projection withholds the copies of one operand stage per CTA (or CTA
+                                 pair) and every wait of it gives up after 2^14 polls instead of 2^22, so the call returns
                                  normally, produces no valid output, and rom_get_status reports
                                  ROM_ERR_DEVICE_TIMEOUT.  The workspace stays usable for the next call.          */
 

@@ -306,31 +306,34 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
           const int kb = kb0 + kq;
           if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, wait_limit)) { ok = false; break; }
           const uint32_t sa = base + stage * SB;
+          // fault injection (tests only): the copies of K block `withhold_kb` of this CTA's (pair's) first tile are never issued,
+          // so the stage never fills and the waits downstream run out
+          const bool withhold = withhold_kb >= 0 && tile == worker && kq == withhold_kb;
           if constexpr (CG == 2) {
             // both CTAs' copies count on the leader's barrier, which alone expects them
             if (rank == 0) mbar_expect_tx(full_bar(stage), stage_tx);
             const uint32_t fb = map_rank(full_bar(stage), 0);
-            if (a_mn) {
-              tma_load_2d_pair(sa, &tmap_a, fb, m_tile * BLOCK_M, kb * BLOCK_K);
-              tma_load_2d_pair(sa + MN_BOX_BYTES, &tmap_a, fb, m_tile * BLOCK_M + 64, kb * BLOCK_K);
-            } else {
-              tma_load_2d_pair(sa, &tmap_a, fb, kb * BLOCK_K, m_tile * BLOCK_M);
-            }
-            if (b_mn) {
-              const int n0 = n_tile * block_n + 128 * (int)rank;
-              tma_load_2d_pair(sa + A_STAGE_BYTES, &tmap_b, fb, n0, e * Kd + kb * BLOCK_K);
-              tma_load_2d_pair(sa + A_STAGE_BYTES + MN_BOX_BYTES, &tmap_b, fb, n0 + 64, e * Kd + kb * BLOCK_K);
-            } else {      // rows 128 .. 255 of the B tile: the next columns, or (SWIGLU) the up rows of the same hidden units
-              tma_load_2d_pair(sa + A_STAGE_BYTES, &tmap_b, fb, kb * BLOCK_K, b_row + (int)rank * (MODE == EPI_SWIGLU ? N : 128));
+            if (!withhold) {
+              if (a_mn) {
+                tma_load_2d_pair(sa, &tmap_a, fb, m_tile * BLOCK_M, kb * BLOCK_K);
+                tma_load_2d_pair(sa + MN_BOX_BYTES, &tmap_a, fb, m_tile * BLOCK_M + 64, kb * BLOCK_K);
+              } else {
+                tma_load_2d_pair(sa, &tmap_a, fb, kb * BLOCK_K, m_tile * BLOCK_M);
+              }
+              if (b_mn) {
+                const int n0 = n_tile * block_n + 128 * (int)rank;
+                tma_load_2d_pair(sa + A_STAGE_BYTES, &tmap_b, fb, n0, e * Kd + kb * BLOCK_K);
+                tma_load_2d_pair(sa + A_STAGE_BYTES + MN_BOX_BYTES, &tmap_b, fb, n0 + 64, e * Kd + kb * BLOCK_K);
+              } else {      // rows 128 .. 255 of the B tile: the next columns, or (SWIGLU) the up rows of the same hidden units
+                tma_load_2d_pair(sa + A_STAGE_BYTES, &tmap_b, fb, kb * BLOCK_K, b_row + (int)rank * (MODE == EPI_SWIGLU ? N : 128));
+              }
             }
             ++issued;
             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
             continue;
           }
           mbar_expect_tx(full_bar(stage), stage_tx);
-          // fault injection (tests only): the copies of K block `withhold_kb` of this CTA's first tile are never issued,
-          // so the stage never fills and the waits downstream run out
-          if (!(withhold_kb >= 0 && tile == worker && kq == withhold_kb)) {
+          if (!withhold) {
             if (a_mn) {
               tma_load_2d(sa, &tmap_a, full_bar(stage), m_tile * BLOCK_M, kb * BLOCK_K);
               tma_load_2d(sa + MN_BOX_BYTES, &tmap_a, full_bar(stage), m_tile * BLOCK_M + 64, kb * BLOCK_K);
@@ -596,7 +599,7 @@ cudaError_t launch_gemm_tc(const void* A, int lda, const void* Bw, int ldb, int 
   // over 8 experts: 2-3 % of the layer) as long as the experts average a full tile; below that single CTAs spread over more SMs.
   // (The dt Proj, two K blocks a tile, is slower on pairs: 69 us against 58 at 16384 x 4096.)
   const bool pair_mode = epi.mode == EPI_STORE || epi.mode == EPI_INPROJ || epi.mode == EPI_OUTPROJ || swiglu;
-  const int cg = pair_mode && pad_offsets && M_max >= n_experts * 2 * BLOCK_M && !test_stall && block_n == MAX_BLOCK_N ? 2 : 1;
+  const int cg = pair_mode && pad_offsets && M_max >= n_experts * 2 * BLOCK_M && block_n == MAX_BLOCK_N ? 2 : 1;
   CUtensorMap ta, tb;
   if (!make_tmap(&ta, A, (uint64_t)M_max, (uint64_t)Kd, (uint64_t)lda, BLOCK_M)) return cudaErrorInvalidValue;
   const bool ok = b_mn ? make_tmap(&tb, Bw, (uint64_t)n_experts * Kd, (uint64_t)N, (uint64_t)ldb, BLOCK_K)

@@ -313,7 +313,7 @@ constexpr int TC_THREADS = 320;
 
 template <int MODE>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_t* __restrict__ status) {
+step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_t* __restrict__ status, uint32_t wait_limit, int withhold_kb) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   __shared__ int cnt[kMaxE], off[kMaxE + 1], fill[kMaxE], act[kMaxE], n_act_s;
@@ -380,11 +380,13 @@ step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_
       const int e = act[w / tpe], row = e * p.n_rows + (w % tpe) * p.tile_rows, rot = rot_of(w);
       for (int n0 = 0; n0 < cnt[e] && ok; n0 += TC_N)
         for (int kb = 0; kb < num_kb; ++kb) {
-          if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, WAIT_LIMIT)) { ok = false; break; }
+          if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, wait_limit)) { ok = false; break; }
           const int k0 = k_of(kb, rot);
           mbar_expect_tx(full_bar(stage), 2 * p.tile_rows * BLOCK_K * 2);
-          tma_load_2d(base + stage * TC_STAGE, &tmap_w, full_bar(stage), k0, row);
-          tma_load_2d(base + stage * TC_STAGE + TC_W_HALF, &tmap_w, full_bar(stage), k0 + BLOCK_K, row);
+          if (!(kb == withhold_kb && w == (int)blockIdx.x && n0 == 0)) {      // (fault injection, tests only: the stage never fills)
+            tma_load_2d(base + stage * TC_STAGE, &tmap_w, full_bar(stage), k0, row);
+            tma_load_2d(base + stage * TC_STAGE + TC_W_HALF, &tmap_w, full_bar(stage), k0 + BLOCK_K, row);
+          }
           ++issued;
           if (++stage == TC_STAGES) { stage = 0; phase ^= 1u; }
         }
@@ -396,7 +398,7 @@ step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_
     if (*abort_flag) {                               // give the copies still in flight a bounded time to land before the CTA exits
       for (int i = 0; i < min(issued, TC_STAGES); ++i) {
         if (--stage < 0) { stage = TC_STAGES - 1; phase ^= 1u; }
-        for (uint32_t it = 0; it < (WAIT_LIMIT >> 2); ++it)
+        for (uint32_t it = 0; it < (wait_limit >> 2); ++it)
           if (mbar_try_wait(full_bar(stage), phase)) break;
       }
     }
@@ -412,10 +414,10 @@ step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_
         for (int n0 = 0; n0 < cnt[e] && ok; n0 += TC_N) {
           const int n16 = cols(min(cnt[e] - n0, TC_N));
           const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n16 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-          if (!mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag, WAIT_LIMIT)) { ok = false; break; }
+          if (!mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag, wait_limit)) { ok = false; break; }
           tc_fence_after();
           for (int kb = 0; kb < num_kb; ++kb) {
-            if (!mbar_wait(full_bar(stage), phase, abort_flag, WAIT_LIMIT)) { ok = false; break; }
+            if (!mbar_wait(full_bar(stage), phase, abort_flag, wait_limit)) { ok = false; break; }
             tc_fence_after();
             const int halves = k_of(kb, rot) + BLOCK_K < p.Kd ? 2 : 1;
             for (int hf = 0; hf < halves; ++hf) {
@@ -440,7 +442,7 @@ step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_
       }
       if (*abort_flag && issued_any) {
         umma_commit(drain_bar);
-        for (uint32_t it = 0; it < (WAIT_LIMIT >> 2); ++it)
+        for (uint32_t it = 0; it < (wait_limit >> 2); ++it)
           if (mbar_try_wait(drain_bar, 0)) break;
       }
     }
@@ -465,7 +467,7 @@ step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_
 #pragma unroll
         for (int q = 0; q < 4; ++q) src[q] = p.x + (size_t)tok[off[e] + n0 + min(lrow + 16 * q, m - 1)] * p.ldx + chunk * 8;      // (rows past the last token repeat it)
         for (int kb = 0; kb < num_kb; ++kb) {
-          ok = __all_sync(0xffffffffu, mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, WAIT_LIMIT));
+          ok = __all_sync(0xffffffffu, mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, wait_limit));
           if (!ok) break;
           const uint32_t dst = base + stage * TC_STAGE + TC_A_BYTES + lrow * 128 + ((chunk ^ (lrow & 7)) << 4);
           const int k0 = k_of(kb, rot);
@@ -510,7 +512,7 @@ step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_
       for (int n0 = 0; n0 < cnt[e] && ok; n0 += TC_N) {
         const int m = min(cnt[e] - n0, TC_N);
         const short* mine = list + off[e] + n0;
-        if (!__all_sync(0xffffffffu, mbar_wait(tfull_bar(acc), acc_phase, abort_flag, WAIT_LIMIT))) { ok = false; break; }
+        if (!__all_sync(0xffffffffu, mbar_wait(tfull_bar(acc), acc_phase, abort_flag, wait_limit))) { ok = false; break; }
         tc_fence_after();
         const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)acc * TC_N;
         for (int c0 = 0; c0 < m; c0 += 32) {
@@ -743,12 +745,13 @@ cudaError_t launch_chained(void (*kern)(P...), dim3 grid, int threads, cudaStrea
 }
 
 template <int MODE>
-cudaError_t launch_step_tc(const StepGemmArgs& a, int num_sms, int32_t* status, cudaStream_t st) {
+cudaError_t launch_step_tc(const StepGemmArgs& a, int num_sms, int32_t* status, bool test_stall, cudaStream_t st) {
   CUtensorMap tw;
   if (!make_tmap(&tw, a.W, (uint64_t)a.E * a.n_rows, (uint64_t)a.Kd, (uint64_t)a.Kd, a.tile_rows)) return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(step_tc<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
   if (e != cudaSuccess) return e;
-  return launch_chained_smem(step_tc<MODE>, dim3(num_sms), TC_THREADS, TC_SMEM, st, true, tw, a, status);
+  return launch_chained_smem(step_tc<MODE>, dim3(num_sms), TC_THREADS, TC_SMEM, st, true, tw, a, status,
+                             test_stall ? WAIT_LIMIT_TEST : WAIT_LIMIT, test_stall ? 1 : -1);
 }
 
 // Rows per weight tile: the multiple of 16 in 96 .. 128 for which the CTAs' rounds x rows is smallest when every expert is selected
@@ -772,7 +775,9 @@ cudaError_t launch_step_gemm(const StepGemmArgs& a, dim3 grid, cudaStream_t st) 
 }  // namespace
 
 bool step_small_applicable(const rom_config& c) {
-  return c.dtype == ROM_BF16 && c.flags == 0 && c.small_proj_experts <= 1 && c.L == 1 && c.B <= kStepMaxTokens && c.B * c.K <= kStepMaxAssign &&
+  // (the fault injection needs a kernel with bounded waits: below kStreamMin the general sequence serves it)
+  const bool flags_ok = c.flags == 0 || (c.flags == ROM_FLAG_TEST_STALL && c.B * c.K >= kStreamMin);
+  return c.dtype == ROM_BF16 && flags_ok && c.small_proj_experts <= 1 && c.L == 1 && c.B <= kStepMaxTokens && c.B * c.K <= kStepMaxAssign &&
          c.dt_rank % 16 == 0;
 }
 
@@ -802,7 +807,7 @@ cudaError_t launch_step_small(const rom_config& c, const rom_weights& w, const v
   int32_t* status = reinterpret_cast<int32_t*>(W + lay.status);
   const bool stream = B * K >= kStreamMin;
   a.tile_rows = pick_tile_rows(c.E, 2 * De, num_sms);
-  if (stream) e = launch_step_tc<STEP_IN>(a, num_sms, status, st);
+  if (stream) e = launch_step_tc<STEP_IN>(a, num_sms, status, c.flags & ROM_FLAG_TEST_STALL, st);
   else e = launch_step_gemm<STEP_IN, 2, 8>(a, dim3(2 * De / 32, slots), st);
   if (e != cudaSuccess) return e;
   if (K > 1 && (e = launch_chained(step_conv, dim3((De / 2 + 127) / 128, B), 128, st, true, (const bf16*)XZ, K, De, (const bf16*)w.w_conv, w.b_conv, conv_state,
@@ -817,7 +822,7 @@ cudaError_t launch_step_small(const rom_config& c, const rom_weights& w, const v
   ao.x = Yg; ao.ldx = De; ao.W = (const bf16*)w.W_out; ao.Kd = De; ao.n_rows = Dm; ao.idx = idx; ao.gates = gates; ao.B = B; ao.K = K; ao.E = c.E;
   ao.C = K == 1 ? (bf16*)out : Op; ao.ldc = Dm;
   ao.tile_rows = pick_tile_rows(c.E, Dm, num_sms);
-  if (stream) e = launch_step_tc<STEP_OUT>(ao, num_sms, status, st);
+  if (stream) e = launch_step_tc<STEP_OUT>(ao, num_sms, status, false, st);
   else e = launch_step_gemm<STEP_OUT, 1, 16>(ao, dim3(Dm / 16, slots), st);
   if (e != cudaSuccess) return e;
   if (K > 1) return launch_chained(step_combine, dim3((Dm / 2 + 127) / 128, B), 128, st, true, (const bf16*)Op, (const float*)gates, (bf16*)out, Dm, K);
