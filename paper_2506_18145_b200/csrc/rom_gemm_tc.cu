@@ -38,7 +38,6 @@ constexpr int B_STAGE_BYTES = MAX_BLOCK_N * BLOCK_K * 2;      // 32 KB
 constexpr int STAGE_BYTES = A_STAGE_BYTES + B_STAGE_BYTES;
 constexpr int ACC_STAGES = 2;
 constexpr int TMEM_COLS = 512;
-constexpr int NUM_EPI_WARPS = NUM_EPI_WARPS_C;
 // The dt Proj (softplus output ops) has two K blocks per tile and about ten instructions plus two special-function
 // operations per output element: its time is its epilogue's, so it runs sixteen epilogue warps instead of eight.
 __host__ __device__ constexpr int epi_warps_of(int mode) { return (mode == EPI_SOFTPLUS || mode == EPI_SOFTPLUS_ROWS) ? 16 : NUM_EPI_WARPS_C; }

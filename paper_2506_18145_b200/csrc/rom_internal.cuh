@@ -283,9 +283,8 @@ cudaError_t launch_ssd(const rom_config& c, const void* xc, const float* Bm, con
 // One-pass scan for few long sequences (rom_scan_seq.cu): every exponential evaluated once, no workspace.  bf16 storage only.
 bool scan_seq_applicable(const rom_config& c, const void* u, const void* delta, bool delta_fp32, const float* Bm, const float* Cm,
                          const void* z, int ldz, const int32_t* z_row, const int32_t* y_rows, bool gate_activated, int num_sms);
-cudaError_t launch_scan_seq(const rom_config& c, const void* u, const void* delta, bool delta_fp32, const float* A, const float* Bm,
-                            const float* Cm, const float* D, const void* z, int ldz, const float* h0, void* y, float* h_last,
-                            const int32_t* y_rows, int K, bool gate_activated, cudaStream_t st);
+cudaError_t launch_scan_seq(const rom_config& c, const void* u, const float* delta, const float* A, const float* Bm, const float* Cm, const float* D,
+                            const void* z, int ldz, const float* h0, void* y, float* h_last, cudaStream_t st);
 
 // State recurrence alone over uniform chunks (rom_scan.cu; used by the backward pass): see the definition.
 cudaError_t launch_scan_states(const rom_config& c, const void* u, const float* delta, const float* A, const float* Bm, int Lc, int ncc,
@@ -380,6 +379,20 @@ template <> struct V16<float> {
   __device__ __forceinline__ void zero() { q = make_float4(0.0f, 0.0f, 0.0f, 0.0f); }
   __device__ __forceinline__ void get(float (&v)[4]) const { v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w; }
   static __device__ __forceinline__ void store(float* p, const float (&v)[4]) { *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]); }
+};
+
+// 8 consecutive elements of a row, as loaded until consumed
+template <typename T> struct Raw8;
+template <> struct Raw8<__nv_bfloat16> : V16<__nv_bfloat16> {};
+template <> struct Raw8<float> {
+  float4 a, b;
+  __device__ __forceinline__ void load(const float* p) { a = __ldg(reinterpret_cast<const float4*>(p)); b = __ldg(reinterpret_cast<const float4*>(p) + 1); }
+  __device__ __forceinline__ void zero() { a = make_float4(0.0f, 0.0f, 0.0f, 0.0f); b = a; }
+  __device__ __forceinline__ void get(float (&v)[8]) const { v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w; }
+  static __device__ __forceinline__ void store(float* p, const float (&v)[8]) {
+    reinterpret_cast<float4*>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
+    reinterpret_cast<float4*>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
+  }
 };
 
 // softplus for results that are rounded to bf16: max(v,0) + log1p(e), e = exp(-|v|) in (0, 1], with

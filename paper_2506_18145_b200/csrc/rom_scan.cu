@@ -52,47 +52,6 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
-// 8 consecutive elements of a row, kept raw (16-byte words) until consumed.
-template <typename T> struct Raw8;
-template <> struct Raw8<__nv_bfloat16> {
-  uint4 q;
-  __device__ __forceinline__ void load(const __nv_bfloat16* p) { q = __ldg(reinterpret_cast<const uint4*>(p)); }
-  __device__ __forceinline__ void zero() { q = make_uint4(0, 0, 0, 0); }
-  __device__ __forceinline__ void get(float (&v)[8]) const {
-    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      v[2 * i] = __uint_as_float(w[i] << 16);
-      v[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
-    }
-  }
-  static __device__ __forceinline__ void store(__nv_bfloat16* p, const float (&v)[8]) {
-    uint4 o;
-    uint32_t* w = reinterpret_cast<uint32_t*>(&o);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const __nv_bfloat162 hh = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-      w[i] = *reinterpret_cast<const uint32_t*>(&hh);
-    }
-    *reinterpret_cast<uint4*>(p) = o;
-  }
-};
-template <> struct Raw8<float> {
-  float4 a, b;
-  __device__ __forceinline__ void load(const float* p) {
-    a = __ldg(reinterpret_cast<const float4*>(p));
-    b = __ldg(reinterpret_cast<const float4*>(p) + 1);
-  }
-  __device__ __forceinline__ void zero() { a = make_float4(0.0f, 0.0f, 0.0f, 0.0f); b = a; }
-  __device__ __forceinline__ void get(float (&v)[8]) const {
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-  }
-  static __device__ __forceinline__ void store(float* p, const float (&v)[8]) {
-    reinterpret_cast<float4*>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
-    reinterpret_cast<float4*>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
-  }
-};
-
 template <int NC, int NS>
 struct Geo {
   static constexpr int S = NST / NS;                    // lanes per channel group
@@ -550,6 +509,7 @@ template <typename T, typename TD, bool PRECISE, bool CKPT = false>
 cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const float* h0, float* h_last,
                           float* chunk_ws, int num_sms, cudaStream_t st) {
   constexpr ScanMode FULL = CKPT ? SCAN_FULL_CKPT : SCAN_FULL, FIRST = CKPT ? SCAN_FIRST_CKPT : SCAN_FIRST;
+  constexpr bool GENERAL = sizeof(TD) == 4;      // bf16 Delta is the layer's, which always has a workspace: the warp kernel (and one step)
   const bool zoh = c.disc_mode == 0;
   if (!CKPT && c.L == 1) {
     a.h0 = h0; a.h_last = h_last;
@@ -567,7 +527,7 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
   auto chunks = [&](const ScanArgs& x, int grid_z, auto mode) -> cudaError_t {
     constexpr ScanMode M = decltype(mode)::value;
     if constexpr (!PRECISE) { if (warp_kernel) return launch_scan_warp(x, c.B, grid_z, zoh, sizeof(TD) == 4, M, st); }
-    if constexpr (CKPT && !PRECISE) return cudaErrorInvalidValue;      // (the warp kernel has been taken)
+    if constexpr (!GENERAL) return cudaErrorInvalidValue;
     else {
       // fp32 storage with few channels: fewer states per thread, so that the chunks together still spread over the SMs
       const int shape = PRECISE ? pick_thread_shape(c.B * grid_z, c.d_inner, num_sms) : 108;
@@ -579,7 +539,7 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
   if (nch == 1) {
     a.Lc = c.L; a.L0 = c.L; a.nch = 1;
     if (warp_kernel) return chunks(a, 1, FullTag{});
-    if constexpr (!(CKPT && !PRECISE)) {
+    if constexpr (GENERAL) {
       const int shape = pick_thread_shape(c.B, c.d_inner, num_sms);
       return zoh ? launch_shape<T, TD, PRECISE, true, FULL>(shape, a, c.B, 1, st) : launch_shape<T, TD, PRECISE, false, FULL>(shape, a, c.B, 1, st);
     }
@@ -632,7 +592,7 @@ cudaError_t launch_scan(const rom_config& c, const void* u, const void* delta, b
   // 0.74 ms against 1.04 ms for one 16384-step sequence of 4096 channels).  With a workspace the two chunked launches
   // below are faster (0.67 ms), so they stay the path of the layer.
   if (chunk_ws == nullptr && !scalar_A && ckpt == nullptr && scan_seq_applicable(c, u, delta, delta_fp32, Bm, Cm, z, ldz, z_row, y_rows, gate_activated, num_sms))
-    return launch_scan_seq(c, u, delta, delta_fp32, A, Bm, Cm, D, z, ldz, h0, y, h_last, y_rows, K, gate_activated, st);
+    return launch_scan_seq(c, u, static_cast<const float*>(delta), A, Bm, Cm, D, z, ldz, h0, y, h_last, st);
   const ScanArgs a{u, delta, A, Bm, Cm, D, z, ldz, z_row, h0, y, h_last, y_rows, K, c.L, c.d_inner, c.L, 1, c.L, nullptr, gate_activated ? 1 : 0, 0,
                    ckpt, (c.L + kScanCkpt - 1) / kScanCkpt, (scalar_A && c.disc_mode == 1) ? 1 : 0};
   if (ckpt != nullptr) {      // the layer backward's recomputed forward: Delta in the storage type

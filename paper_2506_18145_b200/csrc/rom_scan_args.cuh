@@ -1,4 +1,4 @@
-// Arguments shared by the selective-scan kernels (rom_scan.cu, rom_scan_warp.cu).
+// Arguments and helpers shared by the selective-scan kernels (rom_scan.cu, rom_scan_warp.cu, rom_scan_bwd.cu).
 #pragma once
 
 #include "rom_internal.cuh"
@@ -24,6 +24,11 @@ struct ScanArgs {
   const float* chain_end;
   const float* chain_sum;
 };
+
+__device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
+// Slot of lane l's partial sums of step r: conflict-free both for a quarter-warp of writers (eight lanes, one step) and of readers
+// (lanes l = 8 g + const, two steps).
+__device__ __forceinline__ int ysw(int l, int r) { return l ^ (2 * (l >> 3) + (r & 1)); }
 
 // What a scan launch does.  SCAN_FULL: outputs.  SCAN_STATE: state only (h_last and sum_delta of every chunk).  SCAN_FIRST: first
 // launch of the chunked scan: chunk 0 in full from the caller's initial state (h0 indexed by sequence), the others state-only

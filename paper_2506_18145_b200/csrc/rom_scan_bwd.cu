@@ -24,7 +24,7 @@
 // warps) allows two blocks per SM, and the 16 independent updates per thread and step hide the latencies.
 // All arithmetic is fp32; the fp32 configuration uses the accurate exp / expm1, the bf16 one a single ex2.approx per state
 // and step (exp(x) - 1 by subtraction: with Delta A down to -5e-4 that is still good to a few 1e-4 relative).
-#include "rom_internal.cuh"
+#include "rom_scan_args.cuh"
 
 namespace rom {
 namespace {
@@ -59,30 +59,6 @@ struct BwdArgs {
   float* q_start; float* sum_delta;         // pre-pass outputs: [B, ncc, De, 16] and [B, ncc, De]
 };
 
-// slot of lane l's partial sums of step r: conflict-free both for a quarter-warp of writers (eight lanes, one step) and of readers
-// (lanes l = 8 g + const, two steps)
-__device__ __forceinline__ int ysw(int l, int r) { return l ^ (2 * (l >> 3) + (r & 1)); }
-
-// 8 consecutive elements of a row, as loaded
-template <typename T> struct Raw8;
-template <> struct Raw8<__nv_bfloat16> {
-  V16<__nv_bfloat16> q;
-  __device__ __forceinline__ void load(const __nv_bfloat16* p) { q.load(p); }
-  __device__ __forceinline__ void zero() { q.zero(); }
-  __device__ __forceinline__ void get(float (&v)[8]) const { q.get(v); }
-};
-template <> struct Raw8<float> {
-  float4 a, b;
-  __device__ __forceinline__ void load(const float* p) { a = __ldg(reinterpret_cast<const float4*>(p)); b = __ldg(reinterpret_cast<const float4*>(p) + 1); }
-  __device__ __forceinline__ void zero() { a = make_float4(0.0f, 0.0f, 0.0f, 0.0f); b = a; }
-  __device__ __forceinline__ void get(float (&v)[8]) const { v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w; }
-};
-__device__ __forceinline__ void store8(__nv_bfloat16* p, const float (&v)[8]) { V16<__nv_bfloat16>::store(p, v); }
-__device__ __forceinline__ void store8(float* p, const float (&v)[8]) {
-  reinterpret_cast<float4*>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
-  reinterpret_cast<float4*>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
-}
-
 template <bool PRECISE> __device__ __forceinline__ float sigmoid_f(float v) {
   return PRECISE ? 1.0f / (1.0f + expf(-v)) : rcp_ftz(1.0f + ex2_ftz(-kLog2e * v));
 }
@@ -93,7 +69,6 @@ template <bool PRECISE> __device__ __forceinline__ float one_minus_exp(float x) 
   const float s = x * fmaf(x, -fmaf(x, -fmaf(x, -fmaf(x, -1.0f / 120.0f, 1.0f / 24.0f), 1.0f / 6.0f), 0.5f), 1.0f);
   return x < 0.25f ? s : 1.0f - ex2_ftz(-kLog2e * x);
 }
-__device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }      // a - b
 // exp(Delta A) of a pair of states, and exp - 1; a2 holds A log2(e) (A itself when PRECISE)
 template <bool PRECISE> __device__ __forceinline__ float2 exp_pair(float2 x) {
@@ -324,7 +299,7 @@ scan_bwd_kernel(const BwdArgs p) {
         const size_t row = b * L + t;
 #pragma unroll
         for (int i = 0; i < 8; ++i) { du[i] = fmaf(Dv[i], ee[i], du[i]); dDacc[i] = fmaf(ee[i], uu[i], dDacc[i]); }
-        store8(static_cast<T*>(p.du) + row * De + lc, du);
+        Raw8<T>::store(static_cast<T*>(p.du) + row * De + lc, du);
         if (zp) {
           float zz[8], dy[8], o[8];
           cur_z.get(zz); cur_dy.get(dy);
@@ -333,16 +308,16 @@ scan_bwd_kernel(const BwdArgs p) {
             const float sg = sigmoid_f<PRECISE>(zz[i]);
             o[i] = dy[i] * fmaf(Dv[i], uu[i], yy[i]) * sg * (1.0f + zz[i] * (1.0f - sg));
           }
-          store8(static_cast<T*>(p.dz) + (size_t)cur_row * p.ldz + lc, o);
+          Raw8<T>::store(static_cast<T*>(p.dz) + (size_t)cur_row * p.ldz + lc, o);
           if (p.dz_rows)
-            for (int kk = 1; kk < p.K; ++kk) store8(static_cast<T*>(p.dz) + (size_t)__ldg(p.dz_rows + row * p.K + kk) * p.ldz + lc, o);
+            for (int kk = 1; kk < p.K; ++kk) Raw8<T>::store(static_cast<T*>(p.dz) + (size_t)__ldg(p.dz_rows + row * p.K + kk) * p.ldz + lc, o);
         }
         if (p.dpre) {
 #pragma unroll
           for (int i = 0; i < 8; ++i) { dd[i] *= one_minus_exp<PRECISE>(dl[i]); dbacc[i] += dd[i]; }
-          store8(static_cast<T*>(p.dpre) + row * De + lc, dd);
+          Raw8<T>::store(static_cast<T*>(p.dpre) + row * De + lc, dd);
         } else {
-          store8(p.ddelta + row * De + lc, dd);
+          Raw8<float>::store(p.ddelta + row * De + lc, dd);
         }
       }
     }

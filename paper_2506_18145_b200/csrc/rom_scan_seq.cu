@@ -37,45 +37,32 @@ constexpr int Q_TT = 32;         // steps per tile
 constexpr int Q_STAGES = 4;      // tiles in the ring of a warp
 constexpr float kLog2e = 1.4426950408889634f;
 
-template <typename TD>
 struct __align__(16) SeqStage {
-  TD delta[Q_TT][Q_CH];
+  float delta[Q_TT][Q_CH];
   __nv_bfloat16 u[Q_TT][Q_CH];
   __nv_bfloat16 z[Q_TT][Q_CH];
   float Bm[Q_TT][NST];
   float Cm[Q_TT][NST];
-  int32_t rows[Q_TT];              // output row of each step (only when the caller scatters the rows)
 };
 
 struct SeqArgs {
-  const void* u; const void* delta; const float* A; const float* Bm; const float* Cm; const float* D;
-  const void* z; int ldz; const float* h0; void* y; float* h_last; const int32_t* y_rows;
-  int K, L, De, gate_activated;
+  const void* u; const float* delta; const float* A; const float* Bm; const float* Cm; const float* D;
+  const void* z; int ldz; const float* h0; void* y; float* h_last;
+  int L, De;
 };
 
-__device__ __forceinline__ float ex2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-__device__ __forceinline__ float raw_f32(float v) { return v; }
-__device__ __forceinline__ float raw_f32(__nv_bfloat16 v) { return __bfloat162float(v); }
-
-// GATE: 0 no gate, 1 z holds SiLU(gate) already, 2 z holds the raw gate.  ROWS: outputs go to the rows listed in y_rows.
-template <typename TD, bool ZOH, int GATE, bool ROWS>
+// GATE: z holds the gate pre-activation.
+template <bool ZOH, bool GATE>
 __global__ void __launch_bounds__(Q_WARPS * 32, 1)
 scan_seq_kernel(const SeqArgs p) {
   pdl_sync();
-  using Stage = SeqStage<TD>;
+  using Stage = SeqStage;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   Stage* stages = reinterpret_cast<Stage*>(smem_raw) + warp * Q_STAGES;
@@ -87,7 +74,7 @@ scan_seq_kernel(const SeqArgs p) {
   const int c = c0 + ch;
   const size_t tok0 = (size_t)b * L;
 
-  const TD* __restrict__ gd = static_cast<const TD*>(p.delta) + tok0 * De + c0;
+  const float* __restrict__ gd = p.delta + tok0 * De + c0;
   const __nv_bfloat16* __restrict__ gu = static_cast<const __nv_bfloat16*>(p.u) + tok0 * De + c0;
   const __nv_bfloat16* __restrict__ gz = GATE ? static_cast<const __nv_bfloat16*>(p.z) + tok0 * p.ldz + c0 : nullptr;
   const float* __restrict__ gB = p.Bm + tok0 * NST;
@@ -101,10 +88,9 @@ scan_seq_kernel(const SeqArgs p) {
     if (t < L) {
       const char* src = reinterpret_cast<const char*>(gd + (size_t)t * De);
 #pragma unroll
-      for (int k = 0; k < (int)(sizeof(TD) * Q_CH / 16); ++k) cp_async16(reinterpret_cast<char*>(&s.delta[lane][0]) + 16 * k, src + 16 * k);
+      for (int k = 0; k < (int)(sizeof(float) * Q_CH / 16); ++k) cp_async16(reinterpret_cast<char*>(&s.delta[lane][0]) + 16 * k, src + 16 * k);
       cp_async16(&s.u[lane][0], gu + (size_t)t * De);
       if (GATE) cp_async16(&s.z[lane][0], gz + (size_t)t * p.ldz);
-      if (ROWS) cp_async4(&s.rows[lane], p.y_rows + tok0 + t);
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -137,17 +123,16 @@ scan_seq_kernel(const SeqArgs p) {
   //   S1 raw operand loads;  S2 conversions, exponentials, input terms w;  S3 the recurrence and the partial sums C h;
   //   S4, S5 the two steps of the exchange that finishes the sums;  S6 skip term, gate, rounding, store.
   struct Raw {
-    TD d[4];
+    float d[4];
     __nv_bfloat16 u[4];
     float4 B4[4], C4[4];
     __nv_bfloat16 ue, ze;    // u and gate of the step this lane finishes (step g of the group)
-    int row;                 // its output row
   };
   struct Ops {
     float2 a[4][2], w[4][2];
     float4 C4[4];
   };
-  struct Meta { float ue, ze; int row; };
+  struct Meta { float ue, ze; };
   struct X1 { float k0, k1, r0, r1; Meta m; };       // kept partial sums and what the partner sent (first exchange)
   struct X2 { float k, r; Meta m; };                 // the same for the second exchange
 
@@ -163,13 +148,12 @@ scan_seq_kernel(const SeqArgs p) {
     }
     o.ue = s.u[r0 + g][ch];
     if (GATE) o.ze = s.z[r0 + g][ch];
-    if (ROWS) o.row = s.rows[r0 + g];
   };
   auto S2 = [&](const Raw& in, Ops& o, Meta& m) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const float dl = raw_f32(in.d[j]);
-      const float uu = raw_f32(in.u[j]);
+      const float dl = in.d[j];
+      const float uu = to_f32(in.u[j]);
       const float vv = ZOH ? uu : dl * uu;
       const float2 dl2 = make_float2(dl, dl), vv2 = make_float2(vv, vv);
       o.C4[j] = in.C4[j];
@@ -177,14 +161,13 @@ scan_seq_kernel(const SeqArgs p) {
       for (int q = 0; q < 2; ++q) {
         const float2 Bv = q ? make_float2(in.B4[j].z, in.B4[j].w) : make_float2(in.B4[j].x, in.B4[j].y);
         const float2 x = __fmul2_rn(dl2, a2[q]);
-        o.a[j][q] = make_float2(ex2_approx(x.x), ex2_approx(x.y));
+        o.a[j][q] = make_float2(ex2_ftz(x.x), ex2_ftz(x.y));
         // zero-order hold: w = -B u / A (h <- a (h - w) + w); otherwise w = (Delta u) B (h <- a h + w)
         o.w[j][q] = ZOH ? __fmul2_rn(__fmul2_rn(vv2, kin[q]), Bv) : __fmul2_rn(vv2, Bv);
       }
     }
-    m.ue = raw_f32(in.ue);
-    m.ze = GATE ? raw_f32(in.ze) : 1.0f;
-    m.row = ROWS ? in.row : 0;
+    m.ue = to_f32(in.ue);
+    m.ze = GATE ? to_f32(in.ze) : 1.0f;
   };
   auto S3 = [&](const Ops& o, float (&part)[4], auto fast_tag, int nvalid) {
     constexpr bool FAST = decltype(fast_tag)::value;      // every step of the group is inside the sequence
@@ -224,10 +207,8 @@ scan_seq_kernel(const SeqArgs p) {
     const int t = grp * 4 + g;
     if (FAST || (grp >= 0 && t < L)) {
       float o = fmaf(Dc, in.m.ue, in.k + in.r);
-      if (GATE == 1) o *= in.m.ze;
-      if (GATE == 2) o *= silu_fast(in.m.ze);
-      const size_t orow = ROWS ? (size_t)in.m.row : tok0 + (size_t)t;
-      y[orow * De + c] = __float2bfloat16_rn(o);
+      if (GATE) o *= silu_fast(in.m.ze);
+      y[(tok0 + (size_t)t) * De + c] = __float2bfloat16_rn(o);
     }
   };
 
@@ -294,10 +275,10 @@ scan_seq_kernel(const SeqArgs p) {
   }
 }
 
-template <typename TD, bool ZOH, int GATE, bool ROWS>
+template <bool ZOH, bool GATE>
 cudaError_t launch_seq_k(const SeqArgs& a, int B, cudaStream_t st) {
-  const size_t smem = sizeof(SeqStage<TD>) * Q_STAGES * Q_WARPS;
-  auto kern = scan_seq_kernel<TD, ZOH, GATE, ROWS>;
+  const size_t smem = sizeof(SeqStage) * Q_STAGES * Q_WARPS;
+  auto kern = scan_seq_kernel<ZOH, GATE>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   dim3 grid((a.De + Q_WARPS * Q_CH - 1) / (Q_WARPS * Q_CH), B);
@@ -305,10 +286,9 @@ cudaError_t launch_seq_k(const SeqArgs& a, int B, cudaStream_t st) {
   count_launch();
   return cudaGetLastError();
 }
-template <typename TD, bool ZOH>
+template <bool ZOH>
 cudaError_t launch_seq_t(const SeqArgs& a, int B, cudaStream_t st) {
-  // the entry point that reaches this kernel passes the raw gate (or none) and writes rows in token order
-  return a.z == nullptr ? launch_seq_k<TD, ZOH, 0, false>(a, B, st) : launch_seq_k<TD, ZOH, 2, false>(a, B, st);
+  return a.z == nullptr ? launch_seq_k<ZOH, false>(a, B, st) : launch_seq_k<ZOH, true>(a, B, st);
 }
 
 bool aligned16p(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -317,23 +297,19 @@ bool aligned16p(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) =
 
 bool scan_seq_applicable(const rom_config& c, const void* u, const void* delta, bool delta_fp32, const float* Bm, const float* Cm,
                          const void* z, int ldz, const int32_t* z_row, const int32_t* y_rows, bool gate_activated, int num_sms) {
-  if (y_rows != nullptr || (z != nullptr && gate_activated)) return false;      // only the plain forms are instantiated
+  if (!delta_fp32 || y_rows != nullptr || (z != nullptr && gate_activated)) return false;      // fp32 Delta, the raw gate or none, rows in token order
   if (c.dtype != ROM_BF16 || c.d_state != NST || c.L < 2 || z_row != nullptr) return false;
   if (c.d_inner % Q_CH != 0 || (z && ldz % Q_CH != 0)) return false;
   if (!aligned16p(u) || !aligned16p(delta) || !aligned16p(Bm) || !aligned16p(Cm) || (z && !aligned16p(z))) return false;
-  (void)delta_fp32;
   // few independent recurrences: at most two warps of this kernel per SM sub-partition
   const long long warps = (long long)c.B * ((c.d_inner + Q_CH - 1) / Q_CH);
   return warps <= 2LL * 4 * num_sms;
 }
 
-cudaError_t launch_scan_seq(const rom_config& c, const void* u, const void* delta, bool delta_fp32, const float* A, const float* Bm,
-                            const float* Cm, const float* D, const void* z, int ldz, const float* h0, void* y, float* h_last,
-                            const int32_t* y_rows, int K, bool gate_activated, cudaStream_t st) {
-  const SeqArgs a{u, delta, A, Bm, Cm, D, z, ldz, h0, y, h_last, y_rows, K, c.L, c.d_inner, gate_activated ? 1 : 0};
-  const bool zoh = c.disc_mode == 0;
-  if (delta_fp32) return zoh ? launch_seq_t<float, true>(a, c.B, st) : launch_seq_t<float, false>(a, c.B, st);
-  return zoh ? launch_seq_t<__nv_bfloat16, true>(a, c.B, st) : launch_seq_t<__nv_bfloat16, false>(a, c.B, st);
+cudaError_t launch_scan_seq(const rom_config& c, const void* u, const float* delta, const float* A, const float* Bm, const float* Cm, const float* D,
+                            const void* z, int ldz, const float* h0, void* y, float* h_last, cudaStream_t st) {
+  const SeqArgs a{u, delta, A, Bm, Cm, D, z, ldz, h0, y, h_last, c.L, c.d_inner};
+  return c.disc_mode == 0 ? launch_seq_t<true>(a, c.B, st) : launch_seq_t<false>(a, c.B, st);
 }
 
 }  // namespace rom

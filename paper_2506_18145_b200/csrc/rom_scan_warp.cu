@@ -34,25 +34,6 @@ struct WarpTile {
   float4 y[CK][32];               // partial sums of 4 channels over one lane's states; lane l of step r at ysw(l, r)
 };
 
-// conflict-free both for a quarter-warp of writers (eight lanes, one step) and of readers (lanes l = 8 g + const, two steps)
-__device__ __forceinline__ int ysw(int l, int r) { return l ^ (2 * (l >> 3) + (r & 1)); }
-
-// 8 consecutive elements of a row, as loaded
-template <typename T> struct Raw8;
-template <> struct Raw8<bf16> {
-  V16<bf16> q;
-  __device__ __forceinline__ void load(const bf16* p) { q.load(p); }
-  __device__ __forceinline__ void zero() { q.zero(); }
-  __device__ __forceinline__ void get(float (&v)[8]) const { q.get(v); }
-};
-template <> struct Raw8<float> {
-  float4 a, b;
-  __device__ __forceinline__ void load(const float* p) { a = __ldg(reinterpret_cast<const float4*>(p)); b = __ldg(reinterpret_cast<const float4*>(p) + 1); }
-  __device__ __forceinline__ void zero() { a = make_float4(0.0f, 0.0f, 0.0f, 0.0f); b = a; }
-  __device__ __forceinline__ void get(float (&v)[8]) const { v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w; }
-};
-__device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
-
 // SLOTS: the gate of a token is SiLU of the sum of its K >= 2 rows z_row[t K + k], which are also its output rows (y_rows).
 template <typename TD, bool ZOH, int MODE, bool SLOTS>
 __global__ void __launch_bounds__(BT, 3)
@@ -310,15 +291,17 @@ cudaError_t launch_mode(const ScanArgs& a, int B, int grid_z, cudaStream_t st) {
   count_launch();
   return cudaGetLastError();
 }
+// fp32 Delta: rom_scan and the state passes of rom_scan_backward; bf16 Delta: the layer, whose backward takes checkpoints from the full scan.
 template <typename TD, bool ZOH>
 cudaError_t launch_any(const ScanArgs& a, int B, int grid_z, ScanMode mode, cudaStream_t st) {
-  switch (mode) {
-    case SCAN_FULL: return launch_mode<TD, ZOH, SCAN_FULL>(a, B, grid_z, st);
-    case SCAN_STATE: return launch_mode<TD, ZOH, SCAN_STATE>(a, B, grid_z, st);
-    case SCAN_FIRST: return launch_mode<TD, ZOH, SCAN_FIRST>(a, B, grid_z, st);
-    case SCAN_CKPT: return launch_mode<TD, ZOH, SCAN_CKPT>(a, B, grid_z, st);
-    case SCAN_FULL_CKPT: return launch_mode<TD, ZOH, SCAN_FULL_CKPT>(a, B, grid_z, st);
-    case SCAN_FIRST_CKPT: return launch_mode<TD, ZOH, SCAN_FIRST_CKPT>(a, B, grid_z, st);
+  if (mode == SCAN_FULL) return launch_mode<TD, ZOH, SCAN_FULL>(a, B, grid_z, st);
+  if (mode == SCAN_FIRST) return launch_mode<TD, ZOH, SCAN_FIRST>(a, B, grid_z, st);
+  if constexpr (sizeof(TD) == 4) {
+    if (mode == SCAN_STATE) return launch_mode<TD, ZOH, SCAN_STATE>(a, B, grid_z, st);
+    if (mode == SCAN_CKPT) return launch_mode<TD, ZOH, SCAN_CKPT>(a, B, grid_z, st);
+  } else {
+    if (mode == SCAN_FULL_CKPT) return launch_mode<TD, ZOH, SCAN_FULL_CKPT>(a, B, grid_z, st);
+    if (mode == SCAN_FIRST_CKPT) return launch_mode<TD, ZOH, SCAN_FIRST_CKPT>(a, B, grid_z, st);
   }
   return cudaErrorInvalidValue;
 }

@@ -159,10 +159,10 @@ struct StepGemmArgs {
   int tile_rows;                        // step_tc: rows per weight tile
 };
 
-template <int MODE, int RT, int NT, int WARPS>
+template <int MODE, int RT, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32)
 step_gemm(const StepGemmArgs p) {
-  constexpr int ROWS = RT * 16, COLS = NT * 8, PITCH = ROWS + 4;
+  constexpr int ROWS = RT * 16, COLS = 8, PITCH = ROWS + 4;
   constexpr int U = RT == 2 ? 4 : 8;                 // 32-wide blocks in flight per warp
   __shared__ __align__(16) float red[WARPS][COLS][PITCH];
   __shared__ int list[kStepMaxTokens];               // assignments of this block's expert
@@ -204,15 +204,9 @@ step_gemm(const StepGemmArgs p) {
 
   bool waited = MODE == STEP_IN;
   for (int n0 = 0; n0 < m; n0 += COLS) {
-    const int nt_used = (min(m - n0, COLS) + 7) / 8;
-    const bf16* xrow[NT];
-#pragma unroll
-    for (int n = 0; n < NT; ++n) {
-      const int j = n0 + n * 8 + g;
-      const int tok = j < m ? (MODE == STEP_X ? (int)blockIdx.y * COLS + j : list[j] / p.K) : -1;
-      xrow[n] = tok >= 0 ? p.x + (size_t)tok * p.ldx + 8 * t4 : nullptr;
-    }
-    float acc[RT][NT][4] = {};
+    const int tok_g = n0 + g < m ? (MODE == STEP_X ? (int)blockIdx.y * COLS + n0 + g : list[n0 + g] / p.K) : -1;
+    const bf16* xrow = tok_g >= 0 ? p.x + (size_t)tok_g * p.ldx + 8 * t4 : nullptr;
+    float acc[RT][4] = {};
     for (int kb0 = warp; kb0 < nkb; kb0 += WARPS * U) {
       uint4 wq[U][RT][2];
 #pragma unroll
@@ -225,27 +219,20 @@ step_gemm(const StepGemmArgs p) {
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int kb = kb0 + u * WARPS;
+        const uint4 xq = (xrow && kb < nkb) ? ld_act(xrow + kb * 32) : make_uint4(0, 0, 0, 0);
 #pragma unroll
-        for (int n = 0; n < NT; ++n) {
-          if (n >= nt_used) break;
-          const uint4 xq = (xrow[n] && kb < nkb) ? ld_act(xrow[n] + kb * 32) : make_uint4(0, 0, 0, 0);
-#pragma unroll
-          for (int r = 0; r < RT; ++r) mma_block(acc[r][n], wq[u][r][0], wq[u][r][1], xq);
-        }
+        for (int r = 0; r < RT; ++r) mma_block(acc[r], wq[u][r][0], wq[u][r][1], xq);
       }
     }
     if (!waited) { pdl_wait(); pdl_trigger(); waited = true; }
     if (n0 > 0) __syncthreads();                     // the previous group's sums have been read
 #pragma unroll
-    for (int r = 0; r < RT; ++r)
-#pragma unroll
-      for (int n = 0; n < NT; ++n) {
-        if (n >= nt_used) break;
-        red[warp][n * 8 + 2 * t4][r * 16 + g] = acc[r][n][0];
-        red[warp][n * 8 + 2 * t4 + 1][r * 16 + g] = acc[r][n][1];
-        red[warp][n * 8 + 2 * t4][r * 16 + g + 8] = acc[r][n][2];
-        red[warp][n * 8 + 2 * t4 + 1][r * 16 + g + 8] = acc[r][n][3];
-      }
+    for (int r = 0; r < RT; ++r) {
+      red[warp][2 * t4][r * 16 + g] = acc[r][0];
+      red[warp][2 * t4 + 1][r * 16 + g] = acc[r][1];
+      red[warp][2 * t4][r * 16 + g + 8] = acc[r][2];
+      red[warp][2 * t4 + 1][r * 16 + g + 8] = acc[r][3];
+    }
     __syncthreads();
     // sums over the warps, output op on two adjacent rows of one token
     constexpr int PAIRS = ROWS / 2;
@@ -769,7 +756,7 @@ int pick_tile_rows(int E, int n_rows, int num_sms) {
 
 template <int MODE, int RT, int WARPS>
 cudaError_t launch_step_gemm(const StepGemmArgs& a, dim3 grid, cudaStream_t st) {
-  return launch_chained(step_gemm<MODE, RT, 1, WARPS>, grid, WARPS * 32, st, true, a);
+  return launch_chained(step_gemm<MODE, RT, WARPS>, grid, WARPS * 32, st, true, a);
 }
 
 }  // namespace
