@@ -21,6 +21,7 @@ constexpr int kStatCode = 0;       // 0 or the rom_status a kernel latched (a wa
 constexpr int kStatWhere = 1;      // which wait gave up / which debug check failed (debug aid)
 constexpr int kStatIndex = 2;      // debug checks: the offending index
 constexpr int kStatTicket = 8;     // router: blocks-done counter (zero between calls)
+constexpr int kStatNonFinite = 9;  // Mamba2-style block: some x after the conv is not finite
 constexpr int kMaxCanaries = 40;   // sub-buffers of the workspace (debug checks put a canary after each)
 constexpr int kCanaryBytes = 256;
 
@@ -278,7 +279,7 @@ cudaError_t launch_scan(const rom_config& c, const void* u, const void* delta, b
 bool ssd_applicable(const rom_config& c, int headdim);
 size_t ssd_ws_floats(const rom_config& c);
 cudaError_t launch_ssd(const rom_config& c, const void* xc, const float* Bm, const float* Cm, const void* zx, int W, int dt_col, const float* dt_bias,
-                       const float* A, const float* D, void* y, float* ws, cudaStream_t st);
+                       const float* A, const float* D, void* y, float* ws, const int32_t* nonfinite /* device flag: some xc is not finite */, cudaStream_t st);
 
 // One-pass scan for few long sequences (rom_scan_seq.cu): every exponential evaluated once, no workspace.  bf16 storage only.
 bool scan_seq_applicable(const rom_config& c, const void* u, const void* delta, bool delta_fp32, const float* Bm, const float* Cm,

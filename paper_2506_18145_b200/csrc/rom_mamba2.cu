@@ -80,12 +80,13 @@ int check_m2(const rom_config* c, int headdim) {
 constexpr int M2_TCH = 16;      // tokens per thread of the conv kernel
 
 // SiLU(conv) over the x | B | C slab of the token-order projection rows.  A thread owns one 16-byte group of channels
-// and M2_TCH consecutive tokens of one sequence: the M2_TCH + 3 rows it needs are requested at once.
+// and M2_TCH consecutive tokens of one sequence: the M2_TCH + 3 rows it needs are requested at once.  bf16: *nonfinite is set when an x is not
+// finite (zeroed by the caller).
 //   ZXs [T, W]: columns [De, 2De + 2N) are the slab; x part -> xc [T, De] (dtype), B, C parts -> Bm, Cm [T, N] (fp32).
 template <typename T>
 __global__ void __launch_bounds__(128)
 m2_conv_kernel(const T* __restrict__ ZXs, const T* __restrict__ w_conv, const float* __restrict__ b_conv, T* __restrict__ xc,
-               float* __restrict__ Bm, float* __restrict__ Cm, int L, int De, int N, int W, int k) {
+               float* __restrict__ Bm, float* __restrict__ Cm, int L, int De, int N, int W, int k, int32_t* __restrict__ nonfinite) {
   pdl_sync();
   constexpr int V = V16<T>::N;
   const int Cs = De + 2 * N;
@@ -114,6 +115,7 @@ m2_conv_kernel(const T* __restrict__ ZXs, const T* __restrict__ w_conv, const fl
   }
 #pragma unroll
   for (int i = 0; i < V; ++i) bias[i] = b_conv ? b_conv[c0 + i] : 0.0f;
+  uint32_t emax = 0u;                                // largest exponent field of the x written (bf16: both halves)
 #pragma unroll
   for (int r = 0; r < M2_TCH; ++r) {
     const int t = tb + r;
@@ -133,12 +135,20 @@ m2_conv_kernel(const T* __restrict__ ZXs, const T* __restrict__ w_conv, const fl
     const size_t tok = tok0 + t;
     if (c0 < De) {
       V16<T>::store(xc + tok * De + c0, acc);
+      if constexpr (sizeof(T) == 2) {
+#pragma unroll
+        for (int i = 0; i < V; i += 2) {
+          const __nv_bfloat162 h = __floats2bfloat162_rn(acc[i], acc[i + 1]);
+          emax = __vmaxu2(emax, *reinterpret_cast<const uint32_t*>(&h) & 0x7f807f80u);
+        }
+      }
     } else {
       float* dst = c0 < De + N ? Bm + tok * N + (c0 - De) : Cm + tok * N + (c0 - De - N);
 #pragma unroll
       for (int i = 0; i < V; i += 4) *reinterpret_cast<float4*>(dst + i) = make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
     }
   }
+  if ((emax >> 16) == 0x7f80u || (emax & 0xffffu) == 0x7f80u) *nonfinite = 1;      // (every writer stores the same)
 }
 
 // Delta[t, c] = softplus(dt_raw[t, head(c)] + dt_bias[head(c)]) expanded over the head's channels (fp32), four channels
@@ -345,13 +355,14 @@ int rom_mamba2_layer_forward(const rom_config* cfg, int32_t headdim, const rom_m
     float* Bm = reinterpret_cast<float*>(W + m.Bm);
     float* Cm = reinterpret_cast<float*>(W + m.Cm);
     if (bf) launch_k(m2_conv_kernel<__nv_bfloat16>, cgrid, 128, 0, st, (const __nv_bfloat16*)(W + m.ZXs), (const __nv_bfloat16*)w->w_conv, w->b_conv,
-                                                                (__nv_bfloat16*)(W + m.xc), Bm, Cm, c.L, De, N, Wd, c.d_conv);
+                                                                (__nv_bfloat16*)(W + m.xc), Bm, Cm, c.L, De, N, Wd, c.d_conv, status + kStatNonFinite);
     else launch_k(m2_conv_kernel<float>, cgrid, 128, 0, st, (const float*)(W + m.ZXs), (const float*)w->w_conv, w->b_conv, (float*)(W + m.xc), Bm, Cm,
-                                                    c.L, De, N, Wd, c.d_conv);
+                                                    c.L, De, N, Wd, c.d_conv, status + kStatNonFinite);
     count_launch();
     ROM_CUDA(cudaGetLastError());
     if (ssd_applicable(c, headdim)) {
-      ROM_CUDA(launch_ssd(c, W + m.xc, Bm, Cm, W + m.ZXs, Wd, 2 * De + 2 * N, w->dt_bias, w->A, w->D, W + m.Yt, reinterpret_cast<float*>(W + m.scan_ws), st));
+      ROM_CUDA(launch_ssd(c, W + m.xc, Bm, Cm, W + m.ZXs, Wd, 2 * De + 2 * N, w->dt_bias, w->A, w->D, W + m.Yt, reinterpret_cast<float*>(W + m.scan_ws),
+                          status + kStatNonFinite, st));
     } else {
     const long long total2 = max((long long)T * (De / 4), (long long)De);
     const unsigned blocks2 = (unsigned)((total2 + 255) / 256);

@@ -52,6 +52,7 @@ struct SsdArgs {
   const float* dt_bias; const float* A; const float* D;
   bf16* y; int L, De, H;
   int seg_chunks, nseg;                              // chunks per segment
+  const int32_t* nonfinite;                          // set when some x is not finite
   float* h_seg; float* s_seg;                        // [B, nseg, H, 1024] states in fragment order; [B, nseg, H] log2 decay of the segment
 };
 
@@ -80,10 +81,14 @@ __device__ __forceinline__ void split3(float v0, float v1, uint32_t& hi, uint32_
 }
 
 // STATE: only the segment's end state from zero and its total decay (the chunks after the last segment boundary are not needed).
-template <bool STATE>
+// CHECK: the outputs again, for a call whose conv has seen an x that is not finite (otherwise the launch ends at once): in a block on the
+// diagonal the zero weights of the steps before such an x must not meet it.  A launch of its own, since the test inside the loops costs
+// every call: 8 us of 202 where it looks x over, 5 to 15 where a flag skips that.  With this launch the layer takes 1149 us as without.
+template <bool STATE, bool CHECK>
 __global__ void __launch_bounds__(BT, 1)
 ssd_kernel(const SsdArgs p) {
   pdl_sync();
+  if (CHECK && *p.nonfinite == 0) return;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   using Smem = typename std::conditional<STATE, SsdStateSmem, SsdSmem>::type;
   Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
@@ -230,6 +235,15 @@ ssd_kernel(const SsdArgs p) {
         for (int ks = 0; ks < 2 * th + 2; ++ks) {
           uint32_t xa[4][4];
           load_x(ks, xa);
+          bool bad = false;
+          if (CHECK && ks >= 2 * th) {
+            uint32_t mx = 0u;
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+#pragma unroll
+              for (int i = 0; i < 4; ++i) mx = __vmaxu2(mx, xa[m][i] & 0x7f807f80u);
+            bad = __any_sync(0xffffffffu, (mx >> 16) == 0x7f80u || (mx & 0xffffu) == 0x7f80u);
+          }
           const int s0 = 16 * ks + 2 * t4;
           const float2 S0 = *reinterpret_cast<const float2*>(Sw + s0), S1 = *reinterpret_cast<const float2*>(Sw + s0 + 8);
           const float2 d0 = *reinterpret_cast<const float2*>(dw + s0), d1 = *reinterpret_cast<const float2*>(dw + s0 + 8);
@@ -250,6 +264,24 @@ ssd_kernel(const SsdArgs p) {
             uint32_t gb[3][2];
             split3(v[0], v[1], gb[0][0], gb[1][0], gb[2][0]);
             split3(v[2], v[3], gb[0][1], gb[1][1], gb[2][1]);
+            if (CHECK && bad && jt < 2 * ks + 2) {            // one step s of the block at a time, kept by the steps t >= s
+#pragma unroll 1
+              for (int i = 0; i < 16; ++i) {
+                const uint32_t keep = t4 == ((i & 7) >> 1) ? ((i & 1) ? 0xffff0000u : 0x0000ffffu) : 0u;
+                const uint32_t k0 = i < 8 ? keep : 0u, k1 = i < 8 ? 0u : keep;
+                const bool in0 = 8 * jt + 2 * t4 >= 16 * ks + i, in1 = 8 * jt + 2 * t4 + 1 >= 16 * ks + i;
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                  const uint32_t xi[4] = {xa[m][0] & k0, xa[m][1] & k0, xa[m][2] & k1, xa[m][3] & k1};
+                  float d[4] = {acc[m][tj][0], acc[m][tj][1], acc[m][tj][2], acc[m][tj][3]};
+#pragma unroll
+                  for (int u = 2; u >= 0; --u) mma(d, xi, gb[u][0] & k0, gb[u][1] & k1);
+                  if (in0) { acc[m][tj][0] = d[0]; acc[m][tj][2] = d[2]; }
+                  if (in1) { acc[m][tj][1] = d[1]; acc[m][tj][3] = d[3]; }
+                }
+              }
+              continue;
+            }
 #pragma unroll
             for (int u = 2; u >= 0; --u)
 #pragma unroll
@@ -395,14 +427,14 @@ size_t ssd_ws_floats(const rom_config& c) {
 }
 
 cudaError_t launch_ssd(const rom_config& c, const void* xc, const float* Bm, const float* Cm, const void* zx, int W, int dt_col, const float* dt_bias,
-                       const float* A, const float* D, void* y, float* ws, cudaStream_t st) {
+                       const float* A, const float* D, void* y, float* ws, const int32_t* nonfinite, cudaStream_t st) {
   const int H = c.d_inner / P, per = segment_chunks(c.B, H, c.L), nseg = ((c.L + Q - 1) / Q + per - 1) / per;
   const SsdArgs a{(const bf16*)xc, Bm, Cm, (const bf16*)zx, W, dt_col, dt_bias, A, D, (bf16*)y, c.L, c.d_inner, H, per, nseg,
-                  ws, ws + (size_t)c.B * nseg * H * 1024};
+                  nonfinite, ws, ws + (size_t)c.B * nseg * H * 1024};
   cudaError_t e;
   if (nseg > 1) {
-    if ((e = cudaFuncSetAttribute(ssd_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SsdStateSmem))) != cudaSuccess) return e;
-    launch_k(ssd_kernel<true>, dim3(H / HPB, nseg - 1, c.B), BT, sizeof(SsdStateSmem), st, a);
+    if ((e = cudaFuncSetAttribute(ssd_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SsdStateSmem))) != cudaSuccess) return e;
+    launch_k(ssd_kernel<true, false>, dim3(H / HPB, nseg - 1, c.B), BT, sizeof(SsdStateSmem), st, a);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const long long total = (long long)c.B * H * 1024;
@@ -410,10 +442,13 @@ cudaError_t launch_ssd(const rom_config& c, const void* xc, const float* Bm, con
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  if ((e = cudaFuncSetAttribute(ssd_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SsdSmem))) != cudaSuccess) return e;
-  launch_k(ssd_kernel<false>, dim3(H / HPB, nseg, c.B), BT, sizeof(SsdSmem), st, a);
-  count_launch();
-  return cudaGetLastError();
+  for (auto kern : {ssd_kernel<false, false>, ssd_kernel<false, true>}) {
+    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SsdSmem))) != cudaSuccess) return e;
+    launch_k(kern, dim3(H / HPB, nseg, c.B), BT, sizeof(SsdSmem), st, a);
+    count_launch();
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 }  // namespace rom

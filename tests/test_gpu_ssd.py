@@ -5,8 +5,10 @@ import math
 import pytest
 import torch
 
+from paper_2506_18145_b200 import binding as rb
 from paper_2506_18145_b200 import synth
 
+from rom_testlib import assert_close, np64
 from test_gpu_mamba2 import m2shape, run_mamba2
 
 pytestmark = pytest.mark.gpu
@@ -41,3 +43,29 @@ def test_ssd_decay_between_late_steps_after_large_ones(monkeypatch, big):
     p["D"] = None
     monkeypatch.setattr(synth, "make_mamba2_inputs", lambda shape, headdim: p)
     run_mamba2(s, 64)
+
+
+@pytest.mark.parametrize("at", [5, 31, 38, 100])
+def test_ssd_steps_before_one_that_is_not_finite(at):
+    """A token whose channels overflow leaves every earlier token's output as it is: the recurrence is causal.  The steps of its own
+    block of 16 are summed in another order, which may move the roundings to bf16 behind it by one unit (2^-8 of a value)."""
+    s = m2shape(B=1, L=140, E=4, K=1, d_inner=512)
+    p = synth.make_mamba2_inputs(s, 64)
+    p["W_in"][:, s.d_inner + 3:2 * s.d_inner:64, 0] = 4      # one channel of every head follows x[t, 0]
+    p["W_r"][:, 0] = 0
+    p["x"][:, :, 0] = 0
+    cfg = rb.config_from_shape(s)
+    outs = []
+    for v in (0.0, 3e38):
+        p["x"][0, at, 0] = v
+        dev = {k: (None if t is None else t.cuda().contiguous()) for k, t in p.items()}
+        ws = torch.empty(rb.mamba2_workspace_size(cfg, 64), dtype=torch.uint8, device="cuda")
+        out = torch.empty_like(dev["x"])
+        rb.rom_mamba2_layer_forward(cfg, 64, rb.make_mamba2_weights(dev), dev["x"], out, None, None, None, ws)
+        torch.cuda.synchronize()
+        outs.append(out[0])
+    assert torch.isfinite(outs[0]).all() and not torch.isfinite(outs[1][at]).all()
+    block = at // 16 * 16
+    assert torch.equal(outs[0][:block], outs[1][:block])
+    assert torch.isfinite(outs[1][:at]).all()
+    assert_close(np64(outs[1][block:at]), np64(outs[0][block:at]), 2.0 ** -7, "the steps before")
