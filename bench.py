@@ -203,7 +203,7 @@ def run_stage(args, s):
         nbytes = s.T * (4 * s.d_inner * esz + 8 * s.d_state)        # u, Delta, z, y at storage width; B, C fp32
         extra = {"exps": s.T * s.d_inner * s.d_state}
     elif args.stage == "backward":
-        # the whole layer's backward pass (forward activations recomputed inside the call); first, untuned version
+        # the whole layer's backward pass (forward activations recomputed inside the call)
         p = synth.make_inputs(s)
         d = {k: (None if v is None else v.to(dev)) for k, v in p.items()}
         weights = rb.make_weights(d)
@@ -218,8 +218,7 @@ def run_stage(args, s):
         # forward recompute (in_proj) + data and weight gradients of the two grouped projections
         extra = {"flops": 2.0 * s.T * s.K * s.d_model * s.d_inner * (2 + 2 * 3), "d_ff": None}
     elif args.stage == "mamba2":
-        # RoM on a Mamba2-style block at the workload's widths, headdim 64 (first version: the scalar-per-head recurrence runs
-        # on the selective-scan kernel as a special case)
+        # RoM on a Mamba2-style block at the workload's widths, headdim 64
         headdim = 64
         p = synth.make_mamba2_inputs(s, headdim)
         d = {k: (None if v is None else v.to(dev)) for k, v in p.items()}

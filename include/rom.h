@@ -192,7 +192,7 @@ ROM_API int rom_scan(const rom_config *cfg, const void *u, const float *delta, c
  *   dBm, dCm [B, L, d_state], dD [d_inner] (NULL exactly when D is) fp32, each the sum over everything that shares the
  *   parameter (dA and dD over sequences and steps; dBm, dCm over channels) -- accumulated with floating-point atomics,
  *   so their last bits vary from run to run;  dh0 [B, d_inner, d_state] fp32 or NULL.
- * ws: rom_scan_backward_workspace_size(cfg) bytes (the state at the start of every 16 steps, plus the chunk states of the chunk-parallel form).  All arithmetic fp32.
+ * ws: rom_scan_backward_workspace_size(cfg) bytes (the state at the start of every 8 steps, plus the chunk states of the chunk-parallel form).  All arithmetic fp32.
  * Uses cfg->B, L, d_inner, d_state, dtype, disc_mode.                                                              */
 ROM_API int rom_scan_backward_workspace_size(const rom_config *cfg, size_t *bytes);
 ROM_API int rom_scan_backward(const rom_config *cfg, const void *dy, const void *u, const float *delta, const float *A,
@@ -226,8 +226,8 @@ ROM_API int rom_layer_forward(const rom_config *cfg, const rom_weights *w, const
  * training-time estimators and are not part of this call.  Only the shared x Proj / dt Proj wiring (Section 4.3) is
  * differentiated: cfg->small_proj_experts == E returns ROM_ERR_UNSUPPORTED.
  * The call recomputes the forward activations it needs from x (it does not read a forward workspace), then walks the
- * steps backwards: data gradients of the projections are the forward grouped GEMMs on transposed weights; weight
- * gradients are sums over the tokens of each expert's segment.
+ * steps backwards: data gradients of the projections are grouped GEMMs on the weights as stored (the plain-FMA path
+ * makes transposed copies of them in the workspace); weight gradients are sums over the tokens of each expert's segment.
  *   x, dout, dx : [B, L, d_model] dtype.
  *   g           : device pointers, fp32, fully overwritten: the shapes of the corresponding rom_weights fields;
  *                 db_r may be NULL (not produced); dD is NULL exactly when w->D is.
@@ -339,7 +339,10 @@ ROM_API const char *rom_stage_name(int i);
  * arithmetic; for tests and debugging).  Names: "U" [T,D_e] dtype, "delta_r" [T,d_r] dtype,
  * "Bm","Cm" [T,D_s] f32, "Delta" [T,D_e] dtype, "row_of_assign" [T*K] i32 (padded row of each
  * assignment), "XZp" [rows,2*D_e] dtype, "Ygp" [rows,D_e] dtype, "pad_offsets" [E+1] i32.
- * Returns ROM_ERR_INVALID_ARG for an unknown name.                                                */
+ * Returns ROM_ERR_INVALID_ARG for an unknown name.
+ * After rom_layer_step on its own kernels (bf16, see there) "U", "delta_r", "Bm" and "Cm" hold the step's rows, and
+ * "Ygp" its gated rows in token order ([B,D_e]); "row_of_assign", "pad_offsets", "Delta" and (top-1) the Conv half of
+ * "XZp" are not filled: that path needs no permutation and keeps Delta in registers.               */
 ROM_API int rom_workspace_find(const rom_config *cfg, const char *name, size_t *offset, size_t *bytes);
 
 /* Re-run the checks of ROM_FLAG_DEBUG_CHECKS on a workspace that the last rom_layer_forward / rom_layer_step call

@@ -1,6 +1,7 @@
-// Kernels of the layer's backward pass other than the scan's (rom_scan_bwd.cu) and the projections' data gradients
-// (the forward grouped GEMMs run on transposed weights): transposes, the sum over a token's slots, the reverse of the
-// gate-weighted combine, softplus / conv / router reverses and the weight gradients (sums over tokens).
+// Kernels of the layer's backward pass other than the scan's (rom_scan_bwd.cu) and, on the tensor path, the projections' data and
+// weight gradients (rom_gemm_tc.cu, on weights and activations as stored): the sum over a token's slots, the reverse of the gate-weighted
+// combine, conv / router reverses; for the plain-FMA path transposed weights (its data gradients are the forward's grouped GEMMs on
+// them) and the weight gradients (sums over tokens).
 //
 // Section 5.1 trains the layer end to end and Appendix A.3 trains the router through the gate values; the equations
 // differentiated are those of Sections 3.1 and 4.2 (forward: rom_api.cu).  All

@@ -7,9 +7,10 @@
 //   per head h:  H_t = exp(dt A_h) H_{t-1} + dt x_t (x) B_t,  y_t = C_t H_t + D_h x_t;
 //   y^ = RMSNorm(y * SiLU(z)) * w_norm;  O_t = sum_i R_i y^_t W_out,i.
 // Launch sequence: the RoM layer's router / permutation / gather, the grouped GEMM (rows back in token order at top-1 on
-// the tensor path, otherwise a sum over the slots), a conv over the x|B|C slab, a per-head dt expansion, the selective-scan kernel (the scalar-per-head recurrence is its special case
-// A[c, n] = A_head(c), Delta[t, c] = dt[t, head(c)], B-bar = Delta B), a row-wise gated RMS norm that writes the rows in
-// expert order, the grouped output GEMM and the gate-weighted combine.
+// the tensor path, otherwise a sum over the slots), a conv over the x|B|C slab, the recurrence (bf16 with 64 channels per head: chunked
+// matrix products, rom_ssd.cu; otherwise a per-head dt expansion and the selective-scan kernel, whose special case A[c, n] = A_head(c),
+// Delta[t, c] = dt[t, head(c)], B-bar = Delta B it is), a row-wise gated RMS norm that writes the rows in expert order, the grouped
+// output GEMM and the gate-weighted combine.
 #include "rom_internal.cuh"
 
 namespace rom {

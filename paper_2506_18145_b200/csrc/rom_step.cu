@@ -23,7 +23,10 @@ namespace {
 
 constexpr int NST = 16;
 constexpr int kStepMaxTokens = 512, kStepMaxAssign = 2048;
-constexpr int kStreamMin = 4;          // assignments from which the weights are streamed (step_tc)
+// Assignments from which the weights are streamed (step_tc).  us a step, register-fed / streamed, 2048 channels, 8 experts, top-1:
+// 1: 28.4 / 43.7, 2: 41.7 / 49.4, 3: 54.5 / 54.3, 4: 63.3 / 60.3, 5: 69.0 / 64.8, 8: 91.9 / 75.2, 16: 121.6 / 88.7; 16 experts 3: 52.9 / 59.8,
+// 4: 68.1 / 63.3; 1024 channels, 8 experts 3: 30.2 / 32.9, 4: 31.7 / 33.5, 5: 35.6 / 35.3, 8: 43.7 / 38.8.
+constexpr int kStreamMin = 4;
 constexpr float kLog2e = 1.4426950408889634f;
 typedef __nv_bfloat16 bf16;
 
