@@ -83,7 +83,8 @@ typedef struct {
                                  dt Proj + softplus as ONE tcgen05 kernel (U written once and never re-read, delta kept on
                                  the SM) instead of three launches.  Same results up to rounding.  Off by default: as
                                  measured it is slower than the three launches (instruction-issue bound on one CTA per
-                                 128 tokens); ignored where the sizes do not fit (d_r > 128, d_r + 2 D_s > 160)          */
+                                 128 tokens); ignored where the sizes do not fit (d_r > 128, d_r + 2 D_s > 160) or b_conv
+                                 is off a 16-byte boundary                                                      */
 #define ROM_FLAG_TEST_STALL 4 /* fault injection for tests of the device-side timeout path (tensor path only; needs
                                  d_model > 64, and > 128 for rom_layer_step of four assignments and more): the
                                  first grouped projection withholds the copies of one operand stage per CTA (or CTA

@@ -355,9 +355,10 @@ int layer_forward_impl(const rom_config* cfg, const rom_weights* w, const void* 
                 in_token_order ? reinterpret_cast<const int32_t*>(W + lay.assign_of_row) : nullptr, nullptr};
   ROM_CUDA(gemm(W + lay.x_perm, Dm, w->W_inz, Dm, c.E, (int64_t)2 * De * Dm, (int)lay.rows_max, 2 * De, Dm, tile_expert, num_m_tiles, e_in));
   ROM_STAGE_DONE();
-  // S4 + S5 + S6 as one kernel (opt-in): tensor path, top-1 (rows already in token order), shared x Proj / dt Proj
+  // S4 + S5 + S6 as one kernel (opt-in): tensor path, top-1 (rows already in token order), shared x Proj / dt Proj.  It reads b_conv 16
+  // bytes at a time, for every block of channels and token (a test of the address in there takes 0.158 ms to 0.162 at 16384 x 4096).
   const bool fused_small = in_token_order && !conv_state && c.small_proj_experts <= 1 && (c.flags & ROM_FLAG_FUSED_SMALL) &&
-                           fused_conv_xdt_supported(c);
+                           fused_conv_xdt_supported(c) && aligned16(w->b_conv);
   if (fused_small) {
     ROM_CUDA(launch_fused_conv_xdt(c, W + lay.XZp, 2 * De, w->w_conv, w->b_conv, w->W_x, w->W_dt, w->b_dt, W + lay.U, W + lay.delta_r,
                                    reinterpret_cast<float*>(W + lay.Bm), reinterpret_cast<float*>(W + lay.Cm), W + lay.Delta, status, st));

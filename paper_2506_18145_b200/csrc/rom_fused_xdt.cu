@@ -249,7 +249,7 @@ fused_conv_xdt_kernel(const __grid_constant__ CUtensorMap tmap_h, const __grid_c
         for (int j = 0; j < KCONV; ++j) unpack8(__ldg(reinterpret_cast<const uint4*>(p.w_conv + (size_t)j * p.De + c0)), wv[j]);
         float acc[2][8];
         if (p.b_conv) {
-          const float4 b0 = load4_any(p.b_conv + c0), b1 = load4_any(p.b_conv + c0 + 4);
+          const float4 b0 = __ldg(reinterpret_cast<const float4*>(p.b_conv + c0)), b1 = __ldg(reinterpret_cast<const float4*>(p.b_conv + c0) + 1);
           const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
           for (int i = 0; i < 8; ++i) { acc[0][i] = bb[i]; acc[1][i] = bb[i]; }
