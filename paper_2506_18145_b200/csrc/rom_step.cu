@@ -765,8 +765,9 @@ cudaError_t launch_step_gemm(const StepGemmArgs& a, dim3 grid, cudaStream_t st) 
 }  // namespace
 
 bool step_small_applicable(const rom_config& c) {
-  // (the fault injection needs a kernel with bounded waits: below kStreamMin the general sequence serves it)
-  const bool flags_ok = c.flags == 0 || (c.flags == ROM_FLAG_TEST_STALL && c.B * c.K >= kStreamMin);
+  // (the fault injection withholds the second operand stage of a kernel with bounded waits: the general sequence serves it below
+  // kStreamMin, where there is no such kernel here, and up to 128 columns, which are one stage)
+  const bool flags_ok = c.flags == 0 || (c.flags == ROM_FLAG_TEST_STALL && c.B * c.K >= kStreamMin && c.d_model > 2 * BLOCK_K);
   return c.dtype == ROM_BF16 && flags_ok && c.small_proj_experts <= 1 && c.L == 1 && c.B <= kStepMaxTokens && c.B * c.K <= kStepMaxAssign &&
          c.dt_rank % 16 == 0;
 }

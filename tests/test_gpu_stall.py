@@ -37,14 +37,15 @@ def test_stalled_projection_is_reported(kw):
     assert_close(np64(out), ref, TOL["bf16"], "out after a timed-out call")
 
 
-@pytest.mark.parametrize("B,E,K,where", [
-    (3, 8, 1, (1, 2, 3)),                                # no bounded wait in the step's own kernels: the general sequence
-    (4, 8, 1, (4, 5, 6, 7)),
-    (70, 1, 1, (4, 5, 6, 7)),                            # two passes of columns
-    (33, 8, 2, (4, 5, 6, 7)),
+@pytest.mark.parametrize("B,E,K,d_model,where", [
+    (3, 8, 1, 1024, (1, 2, 3)),                          # no bounded wait in the step's own kernels: the general sequence
+    (9, 8, 1, 128, (1, 2, 3)),                           # one operand stage: the same
+    (4, 8, 1, 1024, (4, 5, 6, 7)),
+    (70, 1, 1, 192, (4, 5, 6, 7)),                       # two passes of columns
+    (33, 8, 2, 1024, (4, 5, 6, 7)),
 ])
-def test_stalled_step_is_reported(B, E, K, where):
-    s = small_shape(B=B, L=1, E=E, K=K, d_model=1024, d_inner=1024, dtype="bf16")
+def test_stalled_step_is_reported(B, E, K, d_model, where):
+    s = small_shape(B=B, L=1, E=E, K=K, d_model=d_model, d_inner=1024, dtype="bf16")
     p = synth.make_inputs(s, recipe="unit")
     ref = one_step(s, p, B)
     ws = one_step(s, p, B, flags=rb.ROM_FLAG_TEST_STALL)[-1]
