@@ -530,8 +530,12 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
     if constexpr (!GENERAL) return cudaErrorInvalidValue;
     else {
       // fp32 storage with few channels: fewer states per thread, so that the chunks together still spread over the SMs
-      const int shape = PRECISE ? pick_thread_shape(c.B * grid_z, c.d_inner, num_sms) : 108;
-      return zoh ? launch_shape<T, TD, PRECISE, true, M>(shape, x, c.B, grid_z, st) : launch_shape<T, TD, PRECISE, false, M>(shape, x, c.B, grid_z, st);
+      if constexpr (PRECISE) {
+        const int shape = pick_thread_shape(c.B * grid_z, c.d_inner, num_sms);
+        return zoh ? launch_shape<T, TD, PRECISE, true, M>(shape, x, c.B, grid_z, st) : launch_shape<T, TD, PRECISE, false, M>(shape, x, c.B, grid_z, st);
+      } else {      // the scalar-decay block, whose B-bar is Delta B
+        return zoh ? cudaErrorInvalidValue : launch_shape<T, TD, PRECISE, false, M>(108, x, c.B, grid_z, st);
+      }
     }
   };
   typedef std::integral_constant<ScanMode, FULL> FullTag;
