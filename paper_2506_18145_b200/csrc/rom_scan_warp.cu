@@ -58,6 +58,7 @@ scan_warp_kernel(const ScanArgs p) {
   const int c0 = c_warp + 4 * cg;
   constexpr bool SECOND = MODE == SCAN_FULL || MODE == SCAN_FULL_CKPT;      // may be the second launch of the chunked scan
   float2 a2[4][2], kin[4][2], h[4][2], sdel[2];
+  const float d_skip = !so && p.D ? __ldg(p.D + c_warp + lane) : 0.0f;      // (in flight with A: put down below)
   {
     float av[4][4], hv[4][4];
 #pragma unroll
@@ -112,7 +113,7 @@ scan_warp_kernel(const ScanArgs p) {
       put(dst + (size_t)(c0 + 2 * j + 1) * NST + 4 * q, make_float4(h[0][j].y, h[1][j].y, h[2][j].y, h[3][j].y));
     }
   };
-  s.D[lane] = p.D ? __ldg(p.D + c_warp + lane) : 0.0f;
+  if (!so) s.D[lane] = d_skip;
   // ---- loader / output role: step lt of every tile, channels lc .. lc+7
   // (four lanes per row: a load's quarter-warp touches two rows of global memory, not eight)
   const int lt = lane >> 2, l8 = lane & 3, lc = c_warp + 8 * l8;
