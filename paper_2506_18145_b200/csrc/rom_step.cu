@@ -303,7 +303,7 @@ constexpr int TC_THREADS = 320;
 
 template <int MODE>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_t* __restrict__ status, uint32_t wait_limit, int withhold_kb) {
+step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_t* __restrict__ status, uint32_t wait_limit, bool stall) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   __shared__ int cnt[kMaxE], off[kMaxE + 1], fill[kMaxE], act[kMaxE], n_act_s;
@@ -366,17 +366,19 @@ step_tc(const __grid_constant__ CUtensorMap tmap_w, const StepGemmArgs p, int32_
     if (lane == 0) {
     int stage = 0, issued = 0; uint32_t phase = 0;
     bool ok = true;
+    // fault injection (tests only): from the second stage on 16 bytes are expected that never come
+    uint32_t tx = 2 * p.tile_rows * BLOCK_K * 2;
+    const uint32_t tx_later = tx + (stall ? 16u : 0u);
     for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
       const int e = act[w / tpe], row = e * p.n_rows + (w % tpe) * p.tile_rows, rot = rot_of(w);
       for (int n0 = 0; n0 < cnt[e] && ok; n0 += TC_N)
         for (int kb = 0; kb < num_kb; ++kb) {
           if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, wait_limit)) { ok = false; break; }
           const int k0 = k_of(kb, rot);
-          mbar_expect_tx(full_bar(stage), 2 * p.tile_rows * BLOCK_K * 2);
-          if (!(kb == withhold_kb && w == (int)blockIdx.x && n0 == 0)) {      // (fault injection, tests only: the stage never fills)
-            tma_load_2d(base + stage * TC_STAGE, &tmap_w, full_bar(stage), k0, row);
-            tma_load_2d(base + stage * TC_STAGE + TC_W_HALF, &tmap_w, full_bar(stage), k0 + BLOCK_K, row);
-          }
+          mbar_expect_tx(full_bar(stage), tx);
+          tx = tx_later;
+          tma_load_2d(base + stage * TC_STAGE, &tmap_w, full_bar(stage), k0, row);
+          tma_load_2d(base + stage * TC_STAGE + TC_W_HALF, &tmap_w, full_bar(stage), k0 + BLOCK_K, row);
           ++issued;
           if (++stage == TC_STAGES) { stage = 0; phase ^= 1u; }
         }
@@ -741,7 +743,7 @@ cudaError_t launch_step_tc(const StepGemmArgs& a, int num_sms, int32_t* status, 
   cudaError_t e = cudaFuncSetAttribute(step_tc<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
   if (e != cudaSuccess) return e;
   return launch_chained_smem(step_tc<MODE>, dim3(num_sms), TC_THREADS, TC_SMEM, st, true, tw, a, status,
-                             test_stall ? WAIT_LIMIT_TEST : WAIT_LIMIT, test_stall ? 1 : -1);
+                             test_stall ? WAIT_LIMIT_TEST : WAIT_LIMIT, test_stall);
 }
 
 // Rows per weight tile: the multiple of 16 in 96 .. 128 for which the CTAs' rounds x rows is smallest when every expert is selected
@@ -765,7 +767,7 @@ cudaError_t launch_step_gemm(const StepGemmArgs& a, dim3 grid, cudaStream_t st) 
 }  // namespace
 
 bool step_small_applicable(const rom_config& c) {
-  // (the fault injection withholds the second operand stage of a kernel with bounded waits: the general sequence serves it below
+  // (the fault injection stalls the second operand stage of a kernel with bounded waits: the general sequence serves it below
   // kStreamMin, where there is no such kernel here, and up to 128 columns, which are one stage)
   const bool flags_ok = c.flags == 0 || (c.flags == ROM_FLAG_TEST_STALL && c.B * c.K >= kStreamMin && c.d_model > 2 * BLOCK_K);
   return c.dtype == ROM_BF16 && flags_ok && c.small_proj_experts <= 1 && c.L == 1 && c.B <= kStepMaxTokens && c.B * c.K <= kStepMaxAssign &&
