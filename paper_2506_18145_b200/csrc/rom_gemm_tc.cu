@@ -38,12 +38,11 @@ constexpr int B_STAGE_BYTES = MAX_BLOCK_N * BLOCK_K * 2;      // 32 KB
 constexpr int STAGE_BYTES = A_STAGE_BYTES + B_STAGE_BYTES;
 constexpr int ACC_STAGES = 2;
 constexpr int TMEM_COLS = 512;
-// The dt Proj (softplus output ops) has two K blocks per tile and about ten instructions plus two special-function
-// operations per output element: its time is its epilogue's, so it runs sixteen epilogue warps instead of eight.
+// The softplus output ops (per-expert dt Proj; the shared one where its rank exceeds 128, otherwise rom_dt_proj.cu) have few K blocks
+// per tile: their time is their epilogue's, so they run sixteen epilogue warps instead of eight.
 __host__ __device__ constexpr int epi_warps_of(int mode) { return (mode == EPI_SOFTPLUS || mode == EPI_SOFTPLUS_ROWS) ? 16 : NUM_EPI_WARPS_C; }
 __host__ __device__ constexpr int threads_of(int mode) { return 64 + 32 * epi_warps_of(mode); }
-// Operand stages and epilogue staging per output op.  The softplus epilogue (dt Proj: only two K blocks per tile,
-// and the one GEMM here whose time is its fp32 output) gives up one operand stage for a 32 x 32 fp32 staging
+// Operand stages and epilogue staging per output op.  The softplus epilogue gives up one operand stage for a 32 x 32 fp32 staging
 // square per epilogue warp, through which its stores become whole 128-byte row segments.
 __host__ __device__ constexpr bool f32_out(int mode) { return mode == EPI_SOFTPLUS || mode == EPI_F32 || mode == EPI_SOFTPLUS_ROWS; }
 // The x Proj (a narrow B tile, one wave of row tiles, time set by how many bytes of A are in flight) runs six
@@ -589,6 +588,8 @@ cudaError_t launch_gemm_tc(const void* A, int lda, const void* Bw, int ldb, int 
   // N tile: a multiple of 32 (epilogue column groups) and of 16 (UMMA N for M = 128), at most 256
   const bool swiglu = epi.mode == EPI_SWIGLU;      // N output columns from 2N rows of B per expert, loaded as two boxes of 128 rows
   if (swiglu && (N % 128 != 0 || MAX_BLOCK_N != 256 || b_mn)) return cudaErrorInvalidValue;
+  if (epi.mode == EPI_SOFTPLUS && lda == Kd && ldb == Kd && epi.ldc == N && dt_proj_applicable(N, Kd))
+    return launch_dt_proj(A, Bw, M_max, N, Kd, epi, status, st);
   if (b_mn && n_experts > 1 && Kd % BLOCK_K != 0) return cudaErrorInvalidValue;      // a K block must not run into the next expert
   int block_n = (swiglu || N >= MAX_BLOCK_N) ? MAX_BLOCK_N : (N + 31) / 32 * 32;
   if (epi.mode == EPI_XPROJ && block_n > XPROJ_BLOCK_N) block_n = XPROJ_BLOCK_N;
@@ -598,7 +599,7 @@ cudaError_t launch_gemm_tc(const void* A, int lda, const void* Bw, int ldb, int 
   // CTA pairs: a pair fetches each B tile once for 256 rows (per CTA 32 KB a stage instead of 48).  An expert with an odd number of row
   // tiles ends in a pair that is half empty; measured from 1 to 16 row tiles an expert, pairs are faster all the same (4300 tokens
   // over 8 experts: 2-3 % of the layer) as long as the experts average a full tile; below that single CTAs spread over more SMs.
-  // (The dt Proj, two K blocks a tile, is slower on pairs: 69 us against 58 at 16384 x 4096.)
+  // (The softplus output ops, few K blocks a tile, are slower on pairs: 69 us against 58 at 16384 x 4096 x 128.)
   const bool pair_mode = epi.mode == EPI_STORE || epi.mode == EPI_INPROJ || epi.mode == EPI_OUTPROJ || swiglu;
   const int cg = pair_mode && pad_offsets && M_max >= n_experts * 2 * BLOCK_M && block_n == MAX_BLOCK_N ? 2 : 1;
   CUtensorMap ta, tb;

@@ -230,6 +230,10 @@ cudaError_t launch_gemm_tc(const void* A, int lda, const void* Bw, int ldb, int 
                            const Epilogue& epi, int32_t* status, cudaStream_t st, bool test_stall = false, bool b_mn = false,
                            const int32_t* pad_offsets = nullptr /* grouped: the padded segment offsets (n_experts + 1); allows CTA pairs */);
 
+// dt Proj with a short contraction (rom_dt_proj.cu): C[M, N] = softplus(A[M, Kd] Bw[N, Kd]^T + bias), rows contiguous; bf16.
+bool dt_proj_applicable(int N, int Kd);
+cudaError_t launch_dt_proj(const void* A, const void* Bw, int M, int N, int Kd, const Epilogue& epi, int32_t* status, cudaStream_t st);
+
 // Weight gradient on the tensor cores (bf16): C[s][P, Q] fp32 = sum over rows r of segment s of X[r, p] Y[r, q]; X [rows, P],
 // Y [rows, Q]; seg: n_seg + 1 device row offsets, multiples of 64, or nullptr = one sum over all rows.
 cudaError_t launch_gemm_tc_wgrad(const void* X, const void* Y, int rows, const int32_t* seg, int n_seg, int P, int Q, float* C,
