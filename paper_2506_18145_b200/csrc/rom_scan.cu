@@ -2,8 +2,8 @@
 // fused with the output gate y * SiLU(z) and with the re-permutation of the gated rows into expert
 // order (the routing decision of the Gate/Conv projections is reused for Out Proj, Section 4.2).
 //
-// This is the kernel of fp32 storage, of the scalar-decay block, and of a few bf16 channels without a workspace; bf16 otherwise runs
-// rom_scan_warp.cu.  The launch logic of all of them (chunks, chain, checkpoints) is here.
+// This is the kernel of fp32 storage with many channels (few: rom_scan_f32.cu), of the scalar-decay block, and of a few bf16 channels
+// without a workspace; bf16 otherwise runs rom_scan_warp.cu.  The launch logic of all of them (chunks, chain, checkpoints) is here.
 //
 // State and arithmetic are fp32.  The recurrence is sequential in t, so the parallelism is
 // (sequence, channel, state).  One thread owns NS of the 16 states of NC adjacent channels
@@ -497,7 +497,8 @@ int pick_thread_shape(int B, int De, int num_sms) {
 template <typename T, typename TD, bool PRECISE, bool ZOH, int MODE>
 cudaError_t launch_shape(int shape, const ScanArgs& a, int B, int grid_z, cudaStream_t st) {
   if (shape == 108) return launch_one<T, TD, 1, 8, PRECISE, ZOH, MODE>(a, B, grid_z, st);
-  if constexpr (PRECISE || MODE == SCAN_FULL) {      // (bf16 chunks always run 8 states per thread)
+  // (fp32: many channels, or the scalar decay of a Mamba2-style block; bf16 chunks always run 8 states per thread)
+  if constexpr (PRECISE ? !ZOH && (MODE == SCAN_FULL || MODE == SCAN_FIRST) : MODE == SCAN_FULL) {
     if (shape == 104) return launch_one<T, TD, 1, 4, PRECISE, ZOH, MODE>(a, B, grid_z, st);
     if (shape == 102) return launch_one<T, TD, 1, 2, PRECISE, ZOH, MODE>(a, B, grid_z, st);
   }
@@ -521,21 +522,23 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
   }
   // bf16 storage, A per channel and state: the warp kernel, unless there is neither a workspace for chunks nor one of its warps
   // per SM sub-partition (fewer states per thread then spread the work further)
+  if (PRECISE && !a.scalar_a && scan_f32_applicable(c.B, c.d_inner)) {
+    a.h0 = h0; a.h_last = h_last;
+    return launch_scan_f32(a, c.B, zoh, CKPT, st);
+  }
   const bool warp_kernel = !PRECISE && !a.scalar_a && (CKPT || chunk_ws || (long long)c.B * (c.d_inner / 32) >= 4LL * num_sms);
-  const int nch = !chunk_ws ? 1 : warp_kernel ? scan_warp_chunks(c.B, c.d_inner, c.L) : PRECISE ? scan_f32_chunks(c.B, c.d_inner, c.L) : scan_chunks(c.B, c.d_inner, c.L);
+  const int nch = !chunk_ws ? 1 : warp_kernel ? scan_warp_chunks(c.B, c.d_inner, c.L) : PRECISE ? (a.scalar_a ? scan_f32_chunks(c.B, c.d_inner, c.L) : 1) : scan_chunks(c.B, c.d_inner, c.L);
   // one launch over `grid_z` chunks with 8 states per thread (chunked) or the warp kernel
   auto chunks = [&](const ScanArgs& x, int grid_z, auto mode) -> cudaError_t {
-    constexpr ScanMode M = decltype(mode)::value;
+    [[maybe_unused]] constexpr ScanMode M = decltype(mode)::value;
     if constexpr (!PRECISE) { if (warp_kernel) return launch_scan_warp(x, c.B, grid_z, zoh, sizeof(TD) == 4, M, st); }
     if constexpr (!GENERAL) return cudaErrorInvalidValue;
     else {
-      // fp32 storage with few channels: fewer states per thread, so that the chunks together still spread over the SMs
-      if constexpr (PRECISE) {
-        const int shape = pick_thread_shape(c.B * grid_z, c.d_inner, num_sms);
-        return zoh ? launch_shape<T, TD, PRECISE, true, M>(shape, x, c.B, grid_z, st) : launch_shape<T, TD, PRECISE, false, M>(shape, x, c.B, grid_z, st);
-      } else {      // the scalar-decay block, whose B-bar is Delta B
-        return zoh ? cudaErrorInvalidValue : launch_shape<T, TD, PRECISE, false, M>(108, x, c.B, grid_z, st);
-      }
+      // the scalar-decay block, whose B-bar is Delta B; fp32 storage with few channels: fewer states per thread, so that the chunks
+      // together still spread over the SMs
+      if constexpr (CKPT) return cudaErrorInvalidValue;
+      else return zoh ? cudaErrorInvalidValue
+                      : launch_shape<T, TD, PRECISE, false, M>(PRECISE ? pick_thread_shape(c.B * grid_z, c.d_inner, num_sms) : 108, x, c.B, grid_z, st);
     }
   };
   typedef std::integral_constant<ScanMode, FULL> FullTag;

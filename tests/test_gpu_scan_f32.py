@@ -1,0 +1,45 @@
+"""The one-launch fp32 scan against the fp64 recurrence: lengths around the 16 steps of a segment and the 256, 128 and 64 steps of a
+round (by the number of blocks), several rounds, both sides of the channel count where the general kernel takes over, without a
+workspace as well; and causality next to values that are not finite."""
+import pytest
+import torch
+
+from paper_2506_18145_b200 import binding as rb
+from test_gpu_parity import run_scan
+from rom_testlib import TOL, assert_close
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("disc_mode", [0, 1])
+@pytest.mark.parametrize("B,L,De,use_ws", [
+    (1, 2, 64, True), (1, 15, 64, False), (1, 16, 128, True), (2, 17, 64, True), (1, 255, 512, True), (1, 257, 192, False),
+    (1, 600, 64, True), (1, 129, 1024, True), (2, 300, 512, False), (3, 65, 1024, True), (5, 130, 1024, True),
+    (15, 33, 2176, True), (16, 33, 2048, True),
+])
+def test_scan_f32(disc_mode, B, L, De, use_ws):
+    y, Y, hl, HL = run_scan(B, L, De, "f32", disc_mode, True, True, True, seed=7100 + L + De, use_ws=use_ws)
+    assert_close(y, Y, TOL["f32"], "y")
+    assert_close(hl, HL, TOL["f32"], "h_last")
+
+
+@pytest.mark.parametrize("what", ["u", "B"])
+def test_scan_f32_not_finite_stays_where_it_is(what):
+    B, L, De, t_bad, c_bad = 1, 200, 64, 100, 5
+    g = torch.Generator(device="cuda").manual_seed(3)
+    r = lambda *s: torch.randn(*s, device="cuda", generator=g)      # noqa: E731
+    u, d, A = r(B, L, De), torch.rand(B, L, De, device="cuda", generator=g) * 0.1, -torch.rand(De, 16, device="cuda", generator=g) * 15 - 0.5
+    Bm, Cm = r(B, L, 16), r(B, L, 16)
+    cfg = rb.make_config(B, L, De // 2, De, 16, 4, 16, 1, 1, "f32")
+    ref, y = torch.empty_like(u), torch.empty_like(u)
+    rb.rom_scan(cfg, u, d, A, Bm, Cm, None, None, None, ref, None)
+    if what == "u":
+        u[0, t_bad, c_bad] = float("inf")
+    else:
+        Bm[0, t_bad, 7] = float("nan")
+    rb.rom_scan(cfg, u, d, A, Bm, Cm, None, None, None, y, None)
+    torch.cuda.synchronize()
+    assert torch.equal(y[:, :t_bad], ref[:, :t_bad])
+    keep = [c for c in range(De) if c != c_bad] if what == "u" else []
+    assert torch.equal(y[:, :, keep], ref[:, :, keep])
+    assert not torch.isfinite(y[0, t_bad, c_bad])
