@@ -2,6 +2,7 @@
 // dependent launch, against the eight of the general sequence.
 //
 //   step_route    : one block per token: logits in fp64 (exact products, the same order for every expert), softmax, top-K
+//                   (one or two tokens: inside the In Proj, four launches)
 //   step_gemm<IN> : grouped [Conv Proj | Gate Proj] of the selected experts; at top-1 its output op also runs the short conv
 //                   on the caller's window of H (step_conv does both for K > 1, where H is a sum over experts)
 //   step_gemm<X>  : x Proj -> delta_r | B | C
@@ -24,8 +25,9 @@ namespace {
 constexpr int NST = 16;
 constexpr int kStepMaxTokens = 512, kStepMaxAssign = 2048;
 // Assignments from which the weights are streamed (step_tc).  us a step, register-fed / streamed, 2048 channels, 8 experts, top-1:
-// 1: 28.4 / 43.7, 2: 41.7 / 49.4, 3: 54.5 / 54.3, 4: 63.3 / 60.3, 5: 69.0 / 64.8, 8: 91.9 / 75.2, 16: 121.6 / 88.7; 16 experts 3: 52.9 / 59.8,
-// 4: 68.1 / 63.3; 1024 channels, 8 experts 3: 30.2 / 32.9, 4: 31.7 / 33.5, 5: 35.6 / 35.3, 8: 43.7 / 38.8.
+// 1: 23.1 / 43.7, 2: 33.3 / 49.4, 3: 44.1 / 54.3, 4: 55.4 / 61.5, 5: 59.7 / 65.8, 8: 77.8 / 77.5, 16: 121.6 / 91.0; 16 experts 3: 49.4 / 59.8,
+// 4: 60.0 / 64.6; 1024 channels, 8 experts 4: 30.7 / 37.0, 5: 33.3 / 38.5, 8: 39.1 / 42.1.  By these times the line would lie at eight; it
+// stays at four because the two kernels add in different orders and a sequence's result is the same in every batch from four on.
 constexpr int kStreamMin = 4;
 constexpr float kLog2e = 1.4426950408889634f;
 typedef __nv_bfloat16 bf16;
@@ -54,30 +56,30 @@ __device__ __forceinline__ uint4 ld_act(const bf16* p) {
 }
 
 // ---------------------------------------------------------------------------------------------- router
-__global__ void __launch_bounds__(256)
-step_route(const bf16* __restrict__ x, const bf16* __restrict__ W_r, const float* __restrict__ b_r, int Dm, int E, int K, int gate_mode,
-           int32_t* __restrict__ idx_ws, float* __restrict__ gates_ws, int32_t* __restrict__ idx_out, int32_t* __restrict__ status) {
-  __shared__ double part[8][kMaxE];
-  __shared__ double lg[kMaxE], pr[kMaxE];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int t = blockIdx.x;
-  pdl_trigger();                        // the first kernel of the chain: nothing before it is pending
-  if (t == 0 && threadIdx.x < kStatusInts) status[threadIdx.x] = 0;
-  // warp w takes the 8-element groups w * 32 + lane, ...: every expert sums in the same order
+constexpr int kRouteWarps = 8;
+struct RouteArgs { const bf16* x; const bf16* W_r; const float* b_r; int Dm, E, K, gate_mode; int32_t* idx_ws; float* gates_ws; int32_t* idx_out; int32_t* status; };
+struct RouteSmem { double part[kRouteWarps][kMaxE], lg[kMaxE], pr[kMaxE]; };
+
+// logits of one token in lg, by a block of eight warps: products widened before they are multiplied (exact whatever the operands'
+// exponents, as in the forward's router), every expert summed in the same order
+__device__ __forceinline__ void route_logits(const RouteArgs& p, int t, RouteSmem& s) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, E = p.E;
+  // warp w takes the 8-element groups w * 32 + lane, ...
   for (int e0 = 0; e0 < E; e0 += 8) {
     double acc[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[e] = 0.0;
-    for (int d = (warp * 32 + lane) * 8; d < Dm; d += 2048) {
+    for (int d = (warp * 32 + lane) * 8; d < p.Dm; d += 2048) {
       V16<bf16> q;
       float xv[8];
-      double xd[8];                     // widened before the product, as in the forward's router: exact whatever the operands' exponents
-      q.load(x + (size_t)t * Dm + d); q.get(xv);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) xd[i] = (double)xv[i];
+      double xd[8];
+      q.load(p.x + (size_t)t * p.Dm + d);
       V16<bf16> wq[8];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) wq[e].load(W_r + (size_t)min(e0 + e, E - 1) * Dm + d);
+      for (int e = 0; e < 8; ++e) wq[e].load(p.W_r + (size_t)min(e0 + e, E - 1) * p.Dm + d);
+      q.get(xv);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) xd[i] = (double)xv[i];
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         float wv[8];
@@ -104,48 +106,64 @@ step_route(const bf16* __restrict__ x, const bf16* __restrict__ W_r, const float
       a1 = keep + __shfl_xor_sync(0xffffffffu, send, 1);
       a1 += __shfl_xor_sync(0xffffffffu, a1, 8);
       a1 += __shfl_xor_sync(0xffffffffu, a1, 16);
-      if (lane < 8 && e0 + lane < kMaxE) part[warp][e0 + lane] = a1;
+      if (lane < 8 && e0 + lane < kMaxE) s.part[warp][e0 + lane] = a1;
     }
   }
   __syncthreads();
   if (threadIdx.x < E) {
     const int e = threadIdx.x;
-    double v = b_r ? (double)b_r[e] : 0.0;
+    double v = p.b_r ? (double)p.b_r[e] : 0.0;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) v += part[w][e];
-    lg[e] = v;
+    for (int w = 0; w < kRouteWarps; ++w) v += s.part[w][e];
+    s.lg[e] = v;
   }
   __syncthreads();
+}
+// the k-th expert: largest logit not taken yet, ties to the lowest id, NaN below everything
+__device__ __forceinline__ int route_pick(const double* lg, int E, unsigned long long& taken) {
+  int best = -1; double bestv = -INFINITY;
+  for (int e = 0; e < E; ++e) {
+    if ((taken >> e) & 1ull) continue;
+    double v = lg[e];
+    if (v != v) v = -INFINITY;
+    if (best < 0 || v > bestv) { best = e; bestv = v; }
+  }
+  taken |= 1ull << best;
+  return best;
+}
+// logits, softmax, top-K and gates of one token, written out
+__device__ __forceinline__ void route_token(const RouteArgs& p, int t, RouteSmem& s) {
+  const int E = p.E, K = p.K;
+  route_logits(p, t, s);
   if (threadIdx.x < E) {
     double m = -INFINITY;
-    for (int j = 0; j < E; ++j) { const double v = lg[j]; if (v > m) m = v; }      // NaN never raises m
-    pr[threadIdx.x] = exp(lg[threadIdx.x] - m);
+    for (int j = 0; j < E; ++j) { const double v = s.lg[j]; if (v > m) m = v; }      // NaN never raises m
+    s.pr[threadIdx.x] = exp(s.lg[threadIdx.x] - m);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
     double denom = 0.0, gsum = 0.0, gsel[kMaxK];
-    for (int e = 0; e < E; ++e) denom += pr[e];
+    for (int e = 0; e < E; ++e) denom += s.pr[e];
     unsigned long long taken = 0ull;
     int isel[kMaxK];
     for (int k = 0; k < K; ++k) {
-      int best = -1; double bestv = -INFINITY;
-      for (int e = 0; e < E; ++e) {
-        if ((taken >> e) & 1ull) continue;
-        double v = lg[e];
-        if (v != v) v = -INFINITY;
-        if (best < 0 || v > bestv) { best = e; bestv = v; }
-      }
-      taken |= 1ull << best;
-      isel[k] = best;
-      gsel[k] = pr[best] / denom;
+      isel[k] = route_pick(s.lg, E, taken);
+      gsel[k] = s.pr[isel[k]] / denom;
       gsum += gsel[k];
     }
     for (int k = 0; k < K; ++k) {
-      idx_ws[t * K + k] = isel[k];
-      if (idx_out) idx_out[t * K + k] = isel[k];
-      gates_ws[t * K + k] = (float)(gate_mode == 1 ? gsel[k] / gsum : gsel[k]);
+      p.idx_ws[t * K + k] = isel[k];
+      if (p.idx_out) p.idx_out[t * K + k] = isel[k];
+      p.gates_ws[t * K + k] = (float)(p.gate_mode == 1 ? gsel[k] / gsum : gsel[k]);
     }
   }
+}
+__global__ void __launch_bounds__(kRouteWarps * 32)
+step_route(const RouteArgs p) {
+  __shared__ RouteSmem s;
+  pdl_trigger();                        // the first kernel of the chain: nothing before it is pending
+  if (blockIdx.x == 0 && threadIdx.x < kStatusInts) p.status[threadIdx.x] = 0;
+  route_token(p, blockIdx.x, s);
 }
 
 // ---------------------------------------------------------------------------------------------- projections
@@ -162,13 +180,21 @@ struct StepGemmArgs {
   int tile_rows;                        // step_tc: rows per weight tile
 };
 
-template <int MODE, int RT, int WARPS>
-__global__ void __launch_bounds__(WARPS * 32)
-step_gemm(const StepGemmArgs p) {
-  constexpr int ROWS = RT * 16, COLS = 8, PITCH = ROWS + 4;
+// ROUTE (the In Proj of one or two tokens, while all its blocks are resident at once): every block finds the experts itself, 32 KB of
+// router weights from the L2, which takes less than a launch and the tables in between; one more block writes the routing out for the
+// kernels to come.  With the window, taps and gate of a thread's output requested beside the weights and the first token's operands of
+// step_dt_scan beside delta_r: one token of 2048 channels 28.1 -> 23.1 us, of 1280 23.6 -> 20.0, top-2 of 16 experts 45.4 -> 41.6, two
+// tokens 37.0 -> 33.3 (routing inside without the limit on the blocks: 37.7 and 45.5 for the last two, second waves route again).
+constexpr int kRouteInside = 2;
+template <int MODE, int RT, int WARPS, bool ROUTE = false>
+__global__ void __launch_bounds__(WARPS * 32, MODE == STEP_IN ? 2 : MODE == STEP_OUT ? 1 : 0)
+step_gemm(const StepGemmArgs p, const RouteArgs rt) {
+  constexpr int ROWS = RT * 16, COLS = 8, PITCH = ROWS + 4, PAIRS = ROWS / 2;
   constexpr int U = RT == 2 ? 4 : 8;                 // 32-wide blocks in flight per warp
+  static_assert(kStreamMin <= COLS + 1 && COLS * PAIRS <= WARPS * 32, "an expert's tokens are one group, an output pair a thread");
+  static_assert(!ROUTE || (MODE == STEP_IN && WARPS == kRouteWarps), "");
   __shared__ __align__(16) float red[WARPS][COLS][PITCH];
-  __shared__ int list[kStepMaxTokens];               // assignments of this block's expert
+  __shared__ int list[kStreamMin];                   // assignments of this block's expert
   __shared__ unsigned long long mask;
   __shared__ int count;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t4 = lane & 3;
@@ -177,13 +203,33 @@ step_gemm(const StepGemmArgs p) {
 
   int e = 0;
   int m;                                             // tokens of this block
-  if (MODE == STEP_IN) { pdl_wait(); pdl_trigger(); }      // (OUT: the routing tables are two kernels back, complete already)
+  if (ROUTE) pdl_trigger();                          // the first kernel of the chain
+  else if (MODE == STEP_IN) { pdl_wait(); pdl_trigger(); }      // (OUT: the routing tables are two kernels back, complete already)
   if (MODE != STEP_X) {
     // the blockIdx.y-th selected expert and its assignments (in whatever order: a token's column does not matter)
+    const int A = p.B * p.K;
+    int mine = -1;                                   // thread a < A: the expert of assignment a
+    if constexpr (ROUTE) {
+      __shared__ RouteSmem rs;
+      if (blockIdx.x == gridDim.x - 1) {
+        if (blockIdx.y) return;
+        if (threadIdx.x < kStatusInts) rt.status[threadIdx.x] = 0;
+        for (int t = 0; t < p.B; ++t) { route_token(rt, t, rs); __syncthreads(); }
+        return;
+      }
+      for (int t = 0; t < p.B; ++t) {
+        route_logits(rt, t, rs);
+        const int k = (int)threadIdx.x - t * p.K;    // thread t K + k walks the picks up to its own
+        unsigned long long taken = 0ull;
+        if (k >= 0 && k < p.K)
+          for (int q = 0; q <= k; ++q) mine = route_pick(rs.lg, p.E, taken);
+      }
+    } else if (threadIdx.x < A) {
+      mine = p.idx[threadIdx.x];
+    }
     if (threadIdx.x == 0) { mask = 0ull; count = 0; }
     __syncthreads();
-    const int A = p.B * p.K;
-    for (int a = threadIdx.x; a < A; a += WARPS * 32) atomicOr(&mask, 1ull << p.idx[a]);
+    if (mine >= 0) atomicOr(&mask, 1ull << mine);
     __syncthreads();
     unsigned long long mk = mask;
     for (int i = 0; i < (int)blockIdx.y && mk; ++i) mk &= mk - 1;
@@ -192,8 +238,7 @@ step_gemm(const StepGemmArgs p) {
       return;
     }
     e = __ffsll(mk) - 1;
-    for (int a = threadIdx.x; a < A; a += WARPS * 32)
-      if (p.idx[a] == e) list[atomicAdd(&count, 1)] = a;
+    if (mine == e) list[atomicAdd(&count, 1)] = threadIdx.x;
     __syncthreads();
     m = count;
   } else {
@@ -205,85 +250,97 @@ step_gemm(const StepGemmArgs p) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) wrow[r][h] = p.W + ((size_t)e * p.n_rows + row0 + r * 16 + h * 8 + g) * p.Kd + 8 * t4;
 
+  // output of this thread: two adjacent rows of one token, and what it takes besides the products, requested with the weights
+  const int j_out = threadIdx.x / PAIRS, row_out = row0 + (threadIdx.x % PAIRS) * 2;
+  const bool has_out = j_out < m;
+  const int a_out = MODE != STEP_X && has_out ? list[j_out] : 0;
+  const bool conv = MODE == STEP_IN && p.U != nullptr && has_out && row_out < p.De;
+  float2 win[3], taps[4], ub = make_float2(0.0f, 0.0f);
+  float gate = 1.0f;
+  float* const st = p.conv_state + (size_t)a_out * (p.dconv - 1) * p.De + row_out;
+  auto fetch_out = [&]() {
+    if (conv) {
+      if (p.b_conv) ub = make_float2(p.b_conv[row_out], p.b_conv[row_out + 1]);
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+        if (q < p.dconv - 1) win[q] = *reinterpret_cast<const float2*>(st + (size_t)q * p.De);
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (q < p.dconv) taps[q] = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p.w_conv + (size_t)q * p.De + row_out));
+    }
+    if (MODE == STEP_OUT && has_out && p.K == 1) gate = p.gates[a_out];
+  };
+
   bool waited = MODE == STEP_IN;
-  for (int n0 = 0; n0 < m; n0 += COLS) {
-    const int tok_g = n0 + g < m ? (MODE == STEP_X ? (int)blockIdx.y * COLS + n0 + g : list[n0 + g] / p.K) : -1;
-    const bf16* xrow = tok_g >= 0 ? p.x + (size_t)tok_g * p.ldx + 8 * t4 : nullptr;
-    float acc[RT][4] = {};
-    for (int kb0 = warp; kb0 < nkb; kb0 += WARPS * U) {
-      uint4 wq[U][RT][2];
+  const int tok_g = g < m ? (MODE == STEP_X ? (int)blockIdx.y * COLS + g : list[g] / p.K) : -1;
+  const bf16* xrow = tok_g >= 0 ? p.x + (size_t)tok_g * p.ldx + 8 * t4 : nullptr;
+  float acc[RT][4] = {};
+  for (int kb0 = warp; kb0 < nkb; kb0 += WARPS * U) {
+    uint4 wq[U][RT][2];
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int kb = min(kb0 + u * WARPS, nkb - 1);      // past the end: the last block again, against zero activations
+    for (int u = 0; u < U; ++u) {
+      const int kb = min(kb0 + u * WARPS, nkb - 1);      // past the end: the last block again, against zero activations
 #pragma unroll
-        for (int r = 0; r < RT; ++r) { wq[u][r][0] = ld_stream(wrow[r][0] + kb * 32); wq[u][r][1] = ld_stream(wrow[r][1] + kb * 32); }
-      }
-      if (!waited) { pdl_wait(); pdl_trigger(); waited = true; }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int kb = kb0 + u * WARPS;
-        const uint4 xq = (xrow && kb < nkb) ? ld_act(xrow + kb * 32) : make_uint4(0, 0, 0, 0);
-#pragma unroll
-        for (int r = 0; r < RT; ++r) mma_block(acc[r], wq[u][r][0], wq[u][r][1], xq);
-      }
+      for (int r = 0; r < RT; ++r) { wq[u][r][0] = ld_stream(wrow[r][0] + kb * 32); wq[u][r][1] = ld_stream(wrow[r][1] + kb * 32); }
     }
+    if (kb0 == warp) fetch_out();
     if (!waited) { pdl_wait(); pdl_trigger(); waited = true; }
-    if (n0 > 0) __syncthreads();                     // the previous group's sums have been read
 #pragma unroll
-    for (int r = 0; r < RT; ++r) {
-      red[warp][2 * t4][r * 16 + g] = acc[r][0];
-      red[warp][2 * t4 + 1][r * 16 + g] = acc[r][1];
-      red[warp][2 * t4][r * 16 + g + 8] = acc[r][2];
-      red[warp][2 * t4 + 1][r * 16 + g + 8] = acc[r][3];
-    }
-    __syncthreads();
-    // sums over the warps, output op on two adjacent rows of one token
-    constexpr int PAIRS = ROWS / 2;
-    for (int i = threadIdx.x; i < min(m - n0, COLS) * PAIRS; i += WARPS * 32) {
-      const int j = i / PAIRS, r = (i % PAIRS) * 2;
-      float2 v = make_float2(0.0f, 0.0f);
+    for (int u = 0; u < U; ++u) {
+      const int kb = kb0 + u * WARPS;
+      const uint4 xq = (xrow && kb < nkb) ? ld_act(xrow + kb * 32) : make_uint4(0, 0, 0, 0);
 #pragma unroll
-      for (int w = 0; w < WARPS; ++w) {
-        const float2 q = *reinterpret_cast<const float2*>(&red[w][j][r]);
-        v.x += q.x; v.y += q.y;
-      }
-      const int row = row0 + r;
-      if (MODE == STEP_X) {
-        const size_t tok = blockIdx.y * COLS + j;
-        if (row < p.R) *reinterpret_cast<__nv_bfloat162*>(p.C + tok * p.R + row) = __floats2bfloat162_rn(v.x, v.y);
-        else if (row < p.R + NST) *reinterpret_cast<float2*>(p.Bm + tok * NST + row - p.R) = v;
-        else *reinterpret_cast<float2*>(p.Cm + tok * NST + row - p.R - NST) = v;
-      } else if (MODE == STEP_OUT) {
-        const int a = list[n0 + j];
-        const float gt = p.K == 1 ? p.gates[a] : 1.0f;
-        *reinterpret_cast<__nv_bfloat162*>(p.C + (size_t)a * p.ldc + row) = __floats2bfloat162_rn(v.x * gt, v.y * gt);
-      } else {
-        const int a = list[n0 + j];
-        if (p.U == nullptr) {                        // K > 1: rows of the assignment, summed over the slots by step_conv
-          *reinterpret_cast<__nv_bfloat162*>(p.C + (size_t)a * p.ldc + row) = __floats2bfloat162_rn(v.x, v.y);
-        } else if (row >= p.De) {                    // Gate Proj row, activated
-          *reinterpret_cast<__nv_bfloat162*>(p.C + (size_t)a * p.ldc + row) = __floats2bfloat162_rn(silu_fast(v.x), silu_fast(v.y));
-        } else {
-          // Conv Proj row: H (rounded to the storage type), the conv over the caller's window, and the window moved on
-          const __nv_bfloat162 hb = __floats2bfloat162_rn(v.x, v.y);
-          const float2 h = __bfloat1622float2(hb);
-          float* st = p.conv_state + (size_t)a * (p.dconv - 1) * p.De + row;
-          float2 u = p.b_conv ? make_float2(p.b_conv[row], p.b_conv[row + 1]) : make_float2(0.0f, 0.0f);
-          float2 win[3];
-          for (int q = 0; q < p.dconv - 1; ++q) win[q] = *reinterpret_cast<const float2*>(st + (size_t)q * p.De);
-          for (int q = 0; q < p.dconv; ++q) {
-            const float2 w = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p.w_conv + (size_t)q * p.De + row));
-            const float2 hv = q < p.dconv - 1 ? win[q] : h;
-            u.x = fmaf(w.x, hv.x, u.x); u.y = fmaf(w.y, hv.y, u.y);
-          }
-          *reinterpret_cast<__nv_bfloat162*>(p.U + (size_t)a * p.De + row) = __floats2bfloat162_rn(silu_fast(u.x), silu_fast(u.y));
-          for (int q = 0; q + 1 < p.dconv - 1; ++q) *reinterpret_cast<float2*>(st + (size_t)q * p.De) = win[q + 1];
-          *reinterpret_cast<float2*>(st + (size_t)(p.dconv - 2) * p.De) = h;
-        }
-      }
+      for (int r = 0; r < RT; ++r) mma_block(acc[r], wq[u][r][0], wq[u][r][1], xq);
     }
   }
+  if (warp >= nkb) fetch_out();                      // (a warp without a block of the contracted index)
   if (!waited) { pdl_wait(); pdl_trigger(); }
+#pragma unroll
+  for (int r = 0; r < RT; ++r) {
+    red[warp][2 * t4][r * 16 + g] = acc[r][0];
+    red[warp][2 * t4 + 1][r * 16 + g] = acc[r][1];
+    red[warp][2 * t4][r * 16 + g + 8] = acc[r][2];
+    red[warp][2 * t4 + 1][r * 16 + g + 8] = acc[r][3];
+  }
+  __syncthreads();
+  if (!has_out) return;
+  // sums over the warps, output op
+  float2 v = make_float2(0.0f, 0.0f);
+#pragma unroll
+  for (int w = 0; w < WARPS; ++w) {
+    const float2 q = *reinterpret_cast<const float2*>(&red[w][j_out][row_out - row0]);
+    v.x += q.x; v.y += q.y;
+  }
+  const size_t a = a_out;
+  const int row = row_out;
+  if (MODE == STEP_X) {
+    const size_t tok = blockIdx.y * COLS + j_out;
+    if (row < p.R) *reinterpret_cast<__nv_bfloat162*>(p.C + tok * p.R + row) = __floats2bfloat162_rn(v.x, v.y);
+    else if (row < p.R + NST) *reinterpret_cast<float2*>(p.Bm + tok * NST + row - p.R) = v;
+    else *reinterpret_cast<float2*>(p.Cm + tok * NST + row - p.R - NST) = v;
+  } else if (MODE == STEP_OUT) {
+    *reinterpret_cast<__nv_bfloat162*>(p.C + a * p.ldc + row) = __floats2bfloat162_rn(v.x * gate, v.y * gate);
+  } else if (p.U == nullptr) {                       // K > 1: rows of the assignment, summed over the slots by step_conv
+    *reinterpret_cast<__nv_bfloat162*>(p.C + a * p.ldc + row) = __floats2bfloat162_rn(v.x, v.y);
+  } else if (row >= p.De) {                          // Gate Proj row, activated
+    *reinterpret_cast<__nv_bfloat162*>(p.C + a * p.ldc + row) = __floats2bfloat162_rn(silu_fast(v.x), silu_fast(v.y));
+  } else {
+    // Conv Proj row: H (rounded to the storage type), the conv over the caller's window, and the window moved on
+    const __nv_bfloat162 hb = __floats2bfloat162_rn(v.x, v.y);
+    const float2 h = __bfloat1622float2(hb);
+    float2 u = ub;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (q < p.dconv) {
+        const float2 hv = q < p.dconv - 1 ? win[q < 3 ? q : 2] : h;
+        u.x = fmaf(taps[q].x, hv.x, u.x); u.y = fmaf(taps[q].y, hv.y, u.y);
+      }
+    *reinterpret_cast<__nv_bfloat162*>(p.U + a * p.De + row) = __floats2bfloat162_rn(silu_fast(u.x), silu_fast(u.y));
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      if (q + 1 < p.dconv - 1) *reinterpret_cast<float2*>(st + (size_t)q * p.De) = win[q + 1];
+    *reinterpret_cast<float2*>(st + (size_t)(p.dconv - 2) * p.De) = h;
+  }
 }
 
 // The same for more assignments, where the weights of most experts are walked and streaming them is all that counts: tcgen05 with
@@ -608,23 +665,25 @@ step_conv(const bf16* __restrict__ XZ, int K, int De, const bf16* __restrict__ w
 }
 
 // ---------------------------------------------------------------------------------------------- dt Proj + recurrence
-// A warp takes 16 channels x 8 tokens: Delta by MMA, then one (channel half, token) at a time with four lanes per channel (four
+// A warp takes 16 channels x TPW tokens: Delta by MMA, then one (channel half, token) at a time with four lanes per channel (four
 // states each), so that states move as whole 512-byte rows.  The states (the traffic that counts: 8 KB in and out per warp), A and
 // the dt weights are requested before the wait.
-template <bool ZOH>
+// TPW: tokens per warp at most.  With four the registers also take the first token's B, C, u and gate before they are needed (with
+// eight that spills: 105.3 us a step of 64 sequences instead of 104.0).
+template <bool ZOH, int TPW>
 __global__ void __launch_bounds__(128, 4)
 step_dt_scan(const bf16* __restrict__ delta_r, const bf16* __restrict__ W_dt, const float* __restrict__ b_dt, int R,
              const float* __restrict__ A, const float* __restrict__ Bm, const float* __restrict__ Cm, const float* __restrict__ D,
              const bf16* __restrict__ U, const bf16* __restrict__ Z, int ldz, float* __restrict__ ssm_state, bf16* __restrict__ Yg, int B, int De) {
-  __shared__ float dls[4][8][17], ys[4][8][17];
+  __shared__ float dls[4][TPW][17], ys[4][TPW][17];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t4 = lane & 3;
   const int c0 = (blockIdx.x * 4 + warp) * 16;
-  const int tb = blockIdx.y * 8, nt = min(8, B - tb);
+  const int tb = blockIdx.y * TPW, nt = min(TPW, B - tb);
   const uint4 zero4 = make_uint4(0, 0, 0, 0);
   float4* hp = reinterpret_cast<float4*>(ssm_state) + ((size_t)tb * De + c0 + g) * 4 + t4;      // token tl, half hf: + (tl De + 8 hf) 4
-  float4 h[8][2];
+  float4 h[TPW][2];
 #pragma unroll
-  for (int tl = 0; tl < 8; ++tl)
+  for (int tl = 0; tl < TPW; ++tl)
 #pragma unroll
     for (int hf = 0; hf < 2; ++hf) h[tl][hf] = tl < nt ? hp[((size_t)tl * De + 8 * hf) * 4] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   uint4 wq[4][2];                                    // the first 128 columns of the dt weights
@@ -639,6 +698,14 @@ step_dt_scan(const bf16* __restrict__ delta_r, const bf16* __restrict__ W_dt, co
   const float bias[2] = {b_dt ? b_dt[c0 + g] : 0.0f, b_dt ? b_dt[c0 + 8 + g] : 0.0f}, Dc[2] = {D ? D[c0 + g] : 0.0f, D ? D[c0 + 8 + g] : 0.0f};
   pdl_wait();
   pdl_trigger();
+  constexpr bool AHEAD = TPW < 8;
+  float4 b4_0, c4_0;
+  bf16 u_0[2], z_0[2];
+  if (AHEAD) {
+    b4_0 = reinterpret_cast<const float4*>(Bm + (size_t)tb * NST)[t4]; c4_0 = reinterpret_cast<const float4*>(Cm + (size_t)tb * NST)[t4];
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) { u_0[hf] = U[(size_t)tb * De + c0 + 8 * hf + g]; z_0[hf] = Z[(size_t)tb * ldz + c0 + 8 * hf + g]; }
+  }
   float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
   const bool tok_ok = g < nt;
   const bf16* dr = delta_r + (size_t)(tb + g) * R + 8 * t4;
@@ -654,7 +721,8 @@ step_dt_scan(const bf16* __restrict__ delta_r, const bf16* __restrict__ W_dt, co
     mma_block(acc, q0, q1, (tok_ok && in) ? ld_act(dr + kb * 32) : zero4);
   }
 #pragma unroll
-  for (int j = 0; j < 4; ++j) dls[warp][2 * t4 + (j & 1)][g + 8 * (j >> 1)] = softplus_fast(acc[j] + bias[j >> 1]);
+  for (int j = 0; j < 4; ++j)
+    if (TPW == 8 || 2 * t4 + (j & 1) < TPW) dls[warp][2 * t4 + (j & 1)][g + 8 * (j >> 1)] = softplus_fast(acc[j] + bias[j >> 1]);
   __syncwarp();
   float a2[2][4], nk[2][4];
 #pragma unroll
@@ -662,15 +730,15 @@ step_dt_scan(const bf16* __restrict__ delta_r, const bf16* __restrict__ W_dt, co
 #pragma unroll
     for (int i = 0; i < 4; ++i) { a2[hf][i] = av[hf][i] * kLog2e; nk[hf][i] = -1.0f / av[hf][i]; }
 #pragma unroll
-  for (int tl = 0; tl < 8; ++tl) {
+  for (int tl = 0; tl < TPW; ++tl) {
     if (tl >= nt) break;
     const size_t t = tb + tl;
-    const float4 b4 = reinterpret_cast<const float4*>(Bm + t * NST)[t4], c4 = reinterpret_cast<const float4*>(Cm + t * NST)[t4];
+    const float4 b4 = AHEAD && tl == 0 ? b4_0 : reinterpret_cast<const float4*>(Bm + t * NST)[t4], c4 = AHEAD && tl == 0 ? c4_0 : reinterpret_cast<const float4*>(Cm + t * NST)[t4];
     const float bb[4] = {b4.x, b4.y, b4.z, b4.w}, cc[4] = {c4.x, c4.y, c4.z, c4.w};
 #pragma unroll
     for (int hf = 0; hf < 2; ++hf) {
       const int c = c0 + 8 * hf + g;
-      const float uu = to_f32(U[t * De + c]), dl = dls[warp][tl][8 * hf + g];
+      const float uu = to_f32(AHEAD && tl == 0 ? u_0[hf] : U[t * De + c]), dl = dls[warp][tl][8 * hf + g];
       float hv[4] = {h[tl][hf].x, h[tl][hf].y, h[tl][hf].z, h[tl][hf].w};
       float y = 0.0f;
 #pragma unroll
@@ -687,7 +755,7 @@ step_dt_scan(const bf16* __restrict__ delta_r, const bf16* __restrict__ W_dt, co
       hp[((size_t)tl * De + 8 * hf) * 4] = make_float4(hv[0], hv[1], hv[2], hv[3]);
       y += __shfl_xor_sync(0xffffffffu, y, 1);
       y += __shfl_xor_sync(0xffffffffu, y, 2);
-      if (t4 == 0) ys[warp][tl][8 * hf + g] = fmaf(Dc[hf], uu, y) * to_f32(Z[t * ldz + c]);
+      if (t4 == 0) ys[warp][tl][8 * hf + g] = fmaf(Dc[hf], uu, y) * to_f32(AHEAD && tl == 0 ? z_0[hf] : Z[t * ldz + c]);
     }
   }
   __syncwarp();
@@ -761,7 +829,7 @@ int pick_tile_rows(int E, int n_rows, int num_sms) {
 
 template <int MODE, int RT, int WARPS>
 cudaError_t launch_step_gemm(const StepGemmArgs& a, dim3 grid, cudaStream_t st) {
-  return launch_chained(step_gemm<MODE, RT, WARPS>, grid, WARPS * 32, st, true, a);
+  return launch_chained(step_gemm<MODE, RT, WARPS>, grid, WARPS * 32, st, true, a, RouteArgs{});
 }
 
 }  // namespace
@@ -786,21 +854,22 @@ cudaError_t launch_step_small(const rom_config& c, const rom_weights& w, const v
   bf16* Op = reinterpret_cast<bf16*>(W + lay.Op);
   float* Bm = reinterpret_cast<float*>(W + lay.Bm);
   float* Cm = reinterpret_cast<float*>(W + lay.Cm);
-  cudaError_t e = launch_chained(step_route, dim3(B), 256, st, false, (const bf16*)x, (const bf16*)w.W_r, w.b_r, Dm, c.E, K, c.gate_mode, idx, gates,
-                                 topk_idx_out, reinterpret_cast<int32_t*>(W + lay.status));
+  const RouteArgs rt{(const bf16*)x, (const bf16*)w.W_r, w.b_r, Dm, c.E, K, c.gate_mode, idx, gates, topk_idx_out, reinterpret_cast<int32_t*>(W + lay.status)};
+  int num_sms = 0;
+  cudaError_t e = current_device_sm_count(&num_sms);
   if (e != cudaSuccess) return e;
   const int slots = B * K < c.E ? B * K : c.E;      // selected experts at most
+  // few assignments: latency counts, the register-fed kernel spreads them over more blocks; more: stream the weights
+  const bool stream = B * K >= kStreamMin, route_inside = !stream && B <= kRouteInside && (2 * De / 32 + 1) * slots <= 2 * num_sms;
+  if (!route_inside && (e = launch_chained(step_route, dim3(B), kRouteWarps * 32, st, false, rt)) != cudaSuccess) return e;
   StepGemmArgs a{};
   a.x = (const bf16*)x; a.ldx = Dm; a.W = (const bf16*)w.W_inz; a.Kd = Dm; a.n_rows = 2 * De;
   a.idx = idx; a.gates = gates; a.B = B; a.K = K; a.E = c.E; a.C = XZ; a.ldc = 2 * De; a.De = De;
   if (K == 1) { a.w_conv = (const bf16*)w.w_conv; a.b_conv = w.b_conv; a.conv_state = conv_state; a.dconv = c.d_conv; a.U = U; }
-  // few assignments: latency counts, the register-fed kernel spreads them over more blocks; more: stream the weights
-  int num_sms = 0;
-  if ((e = current_device_sm_count(&num_sms)) != cudaSuccess) return e;
   int32_t* status = reinterpret_cast<int32_t*>(W + lay.status);
-  const bool stream = B * K >= kStreamMin;
   a.tile_rows = pick_tile_rows(c.E, 2 * De, num_sms);
   if (stream) e = launch_step_tc<STEP_IN>(a, num_sms, status, c.flags & ROM_FLAG_TEST_STALL, st);
+  else if (route_inside) e = launch_chained(step_gemm<STEP_IN, 2, 8, true>, dim3(2 * De / 32 + 1, slots), 256, st, false, a, rt);
   else e = launch_step_gemm<STEP_IN, 2, 8>(a, dim3(2 * De / 32, slots), st);
   if (e != cudaSuccess) return e;
   if (K > 1 && (e = launch_chained(step_conv, dim3((De / 2 + 127) / 128, B), 128, st, true, (const bf16*)XZ, K, De, (const bf16*)w.w_conv, w.b_conv, conv_state,
@@ -808,8 +877,9 @@ cudaError_t launch_step_small(const rom_config& c, const rom_weights& w, const v
   StepGemmArgs ax{};
   ax.x = U; ax.ldx = De; ax.W = (const bf16*)w.W_x; ax.Kd = De; ax.n_rows = R + 2 * NST; ax.B = B; ax.K = K; ax.C = dr; ax.ldc = R; ax.Bm = Bm; ax.Cm = Cm; ax.R = R;
   if ((e = launch_step_gemm<STEP_X, 1, 16>(ax, dim3((R + 2 * NST) / 16, (B + 7) / 8), st)) != cudaSuccess) return e;
-  auto scan = c.disc_mode == 0 ? step_dt_scan<true> : step_dt_scan<false>;
-  if ((e = launch_chained(scan, dim3(De / 64, (B + 7) / 8), 128, st, true, (const bf16*)dr, (const bf16*)w.W_dt, w.b_dt, R, w.A, (const float*)Bm, (const float*)Cm, w.D,
+  const int tpw = B <= 4 ? 4 : 8;
+  auto scan = tpw == 4 ? (c.disc_mode == 0 ? step_dt_scan<true, 4> : step_dt_scan<false, 4>) : c.disc_mode == 0 ? step_dt_scan<true, 8> : step_dt_scan<false, 8>;
+  if ((e = launch_chained(scan, dim3(De / 64, (B + tpw - 1) / tpw), 128, st, true, (const bf16*)dr, (const bf16*)w.W_dt, w.b_dt, R, w.A, (const float*)Bm, (const float*)Cm, w.D,
                           (const bf16*)U, (const bf16*)(K == 1 ? XZ + De : Zs), K == 1 ? 2 * De : De, ssm_state, Yg, B, De)) != cudaSuccess) return e;
   StepGemmArgs ao{};
   ao.x = Yg; ao.ldx = De; ao.W = (const bf16*)w.W_out; ao.Kd = De; ao.n_rows = Dm; ao.idx = idx; ao.gates = gates; ao.B = B; ao.K = K; ao.E = c.E;

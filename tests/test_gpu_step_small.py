@@ -29,6 +29,17 @@ def test_step_small_parity(kw):
     run_steps(small_shape(**{**dict(L=4, dtype="bf16"), **kw}), 3)
 
 
+@pytest.mark.parametrize("kw", [
+    dict(B=1, E=64, K=3, d_model=192, d_inner=128),                            # three picks of one token, most expert groups full
+    dict(B=1, E=9, K=1, d_model=2112, d_inner=192, router_bias_scale=1.0),     # a second round of the contracted index, a lone ninth expert
+    dict(B=2, E=8, K=1, d_model=256, d_inner=2304, d_conv=2),                  # two tokens, two experts: the most blocks that route themselves
+    dict(B=2, E=8, K=1, d_model=256, d_inner=2368),                            # more: a launch of its own routes
+    dict(B=4, E=1, K=1, d_model=64, d_inner=128), dict(B=5, E=1, K=1, d_model=64, d_inner=128),      # four and eight tokens a warp
+])
+def test_step_route_inside_the_projection(kw):
+    run_steps(small_shape(**{**dict(L=4, dtype="bf16"), **kw}), 3)
+
+
 def one_step(s, p, B, flags=0):
     """One token for the first B sequences of p from seeded states; (out, conv_state, ssm_state, idx, gates, workspace)."""
     cfg = rb.config_from_shape(s.replace(B=B, L=1), flags=flags)
@@ -45,7 +56,7 @@ def one_step(s, p, B, flags=0):
 
 
 @pytest.mark.parametrize("scale", [2.0 ** -80, 2.0 ** -68, 2.0 ** 70])
-@pytest.mark.parametrize("B", [2, 9])
+@pytest.mark.parametrize("B", [1, 2, 9])
 def test_step_route_products_outside_fp32(B, scale):
     """Router products below and above the range of fp32: logits are fp64 sums of exact products, so the routing is the oracle's."""
     s = small_shape(B=B, L=1, E=8, K=2, d_model=320, dtype="bf16")
