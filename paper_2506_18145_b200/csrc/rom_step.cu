@@ -182,7 +182,7 @@ struct StepGemmArgs {
 
 // ROUTE (the In Proj of one or two tokens, while all its blocks are resident at once): every block finds the experts itself, 32 KB of
 // router weights from the L2, which takes less than a launch and the tables in between; one more block writes the routing out for the
-// kernels to come.  With the window, taps and gate of a thread's output requested beside the weights and the first token's operands of
+// kernels to come.  With the window, taps and gate of a thread's output requested beside the weights and the tokens' operands of
 // step_dt_scan beside delta_r: one token of 2048 channels 28.1 -> 23.1 us, of 1280 23.6 -> 20.0, top-2 of 16 experts 45.4 -> 41.6, two
 // tokens 37.0 -> 33.3 (routing inside without the limit on the blocks: 37.7 and 45.5 for the last two, second waves route again).
 constexpr int kRouteInside = 2;
@@ -665,25 +665,26 @@ step_conv(const bf16* __restrict__ XZ, int K, int De, const bf16* __restrict__ w
 }
 
 // ---------------------------------------------------------------------------------------------- dt Proj + recurrence
-// A warp takes 16 channels x TPW tokens: Delta by MMA, then one (channel half, token) at a time with four lanes per channel (four
+// A warp takes 16 channels x 8 tokens: Delta by MMA, then one (channel half, token) at a time with four lanes per channel (four
 // states each), so that states move as whole 512-byte rows.  The states (the traffic that counts: 8 KB in and out per warp), A and
-// the dt weights are requested before the wait.
-// TPW: tokens per warp at most.  With four the registers also take the first token's B, C, u and gate before they are needed (with
-// eight that spills: 105.3 us a step of 64 sequences instead of 104.0).
-template <bool ZOH, int TPW>
+// the dt weights are requested before the wait; B, C, u and the gate of the block's tokens right after it, into shared memory (read
+// token by token each was waited for: 64 sequences 104.1 -> 101.6 us a step, 200: 158.1 -> 147.6).
+template <bool ZOH>
 __global__ void __launch_bounds__(128, 4)
 step_dt_scan(const bf16* __restrict__ delta_r, const bf16* __restrict__ W_dt, const float* __restrict__ b_dt, int R,
              const float* __restrict__ A, const float* __restrict__ Bm, const float* __restrict__ Cm, const float* __restrict__ D,
              const bf16* __restrict__ U, const bf16* __restrict__ Z, int ldz, float* __restrict__ ssm_state, bf16* __restrict__ Yg, int B, int De) {
-  __shared__ float dls[4][TPW][17], ys[4][TPW][17];
+  __shared__ float dls[4][8][17], ys[4][8][17];
+  __shared__ __align__(16) float bcs[8][2 * NST];
+  __shared__ __align__(16) bf16 us[8][64], zs[8][64];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t4 = lane & 3;
   const int c0 = (blockIdx.x * 4 + warp) * 16;
-  const int tb = blockIdx.y * TPW, nt = min(TPW, B - tb);
+  const int tb = blockIdx.y * 8, nt = min(8, B - tb);
   const uint4 zero4 = make_uint4(0, 0, 0, 0);
   float4* hp = reinterpret_cast<float4*>(ssm_state) + ((size_t)tb * De + c0 + g) * 4 + t4;      // token tl, half hf: + (tl De + 8 hf) 4
-  float4 h[TPW][2];
+  float4 h[8][2];
 #pragma unroll
-  for (int tl = 0; tl < TPW; ++tl)
+  for (int tl = 0; tl < 8; ++tl)
 #pragma unroll
     for (int hf = 0; hf < 2; ++hf) h[tl][hf] = tl < nt ? hp[((size_t)tl * De + 8 * hf) * 4] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   uint4 wq[4][2];                                    // the first 128 columns of the dt weights
@@ -698,13 +699,14 @@ step_dt_scan(const bf16* __restrict__ delta_r, const bf16* __restrict__ W_dt, co
   const float bias[2] = {b_dt ? b_dt[c0 + g] : 0.0f, b_dt ? b_dt[c0 + 8 + g] : 0.0f}, Dc[2] = {D ? D[c0 + g] : 0.0f, D ? D[c0 + 8 + g] : 0.0f};
   pdl_wait();
   pdl_trigger();
-  constexpr bool AHEAD = TPW < 8;
-  float4 b4_0, c4_0;
-  bf16 u_0[2], z_0[2];
-  if (AHEAD) {
-    b4_0 = reinterpret_cast<const float4*>(Bm + (size_t)tb * NST)[t4]; c4_0 = reinterpret_cast<const float4*>(Cm + (size_t)tb * NST)[t4];
-#pragma unroll
-    for (int hf = 0; hf < 2; ++hf) { u_0[hf] = U[(size_t)tb * De + c0 + 8 * hf + g]; z_0[hf] = Z[(size_t)tb * ldz + c0 + 8 * hf + g]; }
+  // what the tokens need besides, in flight with delta_r: token by token these loads would be waited for one after another
+  const int tid = threadIdx.x, pt = tid >> 3, pc = tid & 7;      // threads 0..63: eight 16-byte pieces a token
+  uint4 q_bc = zero4, q_uz = zero4;
+  if ((pt & 7) < nt) {
+    const size_t t = tb + (pt & 7);
+    if (pt < 8) q_bc = reinterpret_cast<const uint4*>((pc < 4 ? Bm : Cm) + t * NST)[pc & 3];
+    const int cb = blockIdx.x * 64 + 8 * pc;
+    q_uz = *reinterpret_cast<const uint4*>(pt < 8 ? U + t * De + cb : Z + t * ldz + cb);
   }
   float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
   const bool tok_ok = g < nt;
@@ -720,25 +722,25 @@ step_dt_scan(const bf16* __restrict__ delta_r, const bf16* __restrict__ W_dt, co
     const uint4 q1 = in ? ld_stream(W_dt + (size_t)(c0 + g + 8) * R + kb * 32 + 8 * t4) : zero4;
     mma_block(acc, q0, q1, (tok_ok && in) ? ld_act(dr + kb * 32) : zero4);
   }
+  if (pt < 8) { *reinterpret_cast<uint4*>(&bcs[pt][4 * pc]) = q_bc; *reinterpret_cast<uint4*>(&us[pt][8 * pc]) = q_uz; }
+  else *reinterpret_cast<uint4*>(&zs[pt - 8][8 * pc]) = q_uz;
 #pragma unroll
-  for (int j = 0; j < 4; ++j)
-    if (TPW == 8 || 2 * t4 + (j & 1) < TPW) dls[warp][2 * t4 + (j & 1)][g + 8 * (j >> 1)] = softplus_fast(acc[j] + bias[j >> 1]);
-  __syncwarp();
+  for (int j = 0; j < 4; ++j) dls[warp][2 * t4 + (j & 1)][g + 8 * (j >> 1)] = softplus_fast(acc[j] + bias[j >> 1]);
+  __syncthreads();
   float a2[2][4], nk[2][4];
 #pragma unroll
   for (int hf = 0; hf < 2; ++hf)
 #pragma unroll
     for (int i = 0; i < 4; ++i) { a2[hf][i] = av[hf][i] * kLog2e; nk[hf][i] = -1.0f / av[hf][i]; }
 #pragma unroll
-  for (int tl = 0; tl < TPW; ++tl) {
+  for (int tl = 0; tl < 8; ++tl) {
     if (tl >= nt) break;
-    const size_t t = tb + tl;
-    const float4 b4 = AHEAD && tl == 0 ? b4_0 : reinterpret_cast<const float4*>(Bm + t * NST)[t4], c4 = AHEAD && tl == 0 ? c4_0 : reinterpret_cast<const float4*>(Cm + t * NST)[t4];
+    const float4 b4 = *reinterpret_cast<const float4*>(&bcs[tl][4 * t4]), c4 = *reinterpret_cast<const float4*>(&bcs[tl][NST + 4 * t4]);
     const float bb[4] = {b4.x, b4.y, b4.z, b4.w}, cc[4] = {c4.x, c4.y, c4.z, c4.w};
 #pragma unroll
     for (int hf = 0; hf < 2; ++hf) {
-      const int c = c0 + 8 * hf + g;
-      const float uu = to_f32(AHEAD && tl == 0 ? u_0[hf] : U[t * De + c]), dl = dls[warp][tl][8 * hf + g];
+      const int cl = warp * 16 + 8 * hf + g;
+      const float uu = to_f32(us[tl][cl]), dl = dls[warp][tl][8 * hf + g];
       float hv[4] = {h[tl][hf].x, h[tl][hf].y, h[tl][hf].z, h[tl][hf].w};
       float y = 0.0f;
 #pragma unroll
@@ -755,7 +757,7 @@ step_dt_scan(const bf16* __restrict__ delta_r, const bf16* __restrict__ W_dt, co
       hp[((size_t)tl * De + 8 * hf) * 4] = make_float4(hv[0], hv[1], hv[2], hv[3]);
       y += __shfl_xor_sync(0xffffffffu, y, 1);
       y += __shfl_xor_sync(0xffffffffu, y, 2);
-      if (t4 == 0) ys[warp][tl][8 * hf + g] = fmaf(Dc[hf], uu, y) * to_f32(AHEAD && tl == 0 ? z_0[hf] : Z[t * ldz + c]);
+      if (t4 == 0) ys[warp][tl][8 * hf + g] = fmaf(Dc[hf], uu, y) * to_f32(zs[tl][cl]);
     }
   }
   __syncwarp();
@@ -877,9 +879,8 @@ cudaError_t launch_step_small(const rom_config& c, const rom_weights& w, const v
   StepGemmArgs ax{};
   ax.x = U; ax.ldx = De; ax.W = (const bf16*)w.W_x; ax.Kd = De; ax.n_rows = R + 2 * NST; ax.B = B; ax.K = K; ax.C = dr; ax.ldc = R; ax.Bm = Bm; ax.Cm = Cm; ax.R = R;
   if ((e = launch_step_gemm<STEP_X, 1, 16>(ax, dim3((R + 2 * NST) / 16, (B + 7) / 8), st)) != cudaSuccess) return e;
-  const int tpw = B <= 4 ? 4 : 8;
-  auto scan = tpw == 4 ? (c.disc_mode == 0 ? step_dt_scan<true, 4> : step_dt_scan<false, 4>) : c.disc_mode == 0 ? step_dt_scan<true, 8> : step_dt_scan<false, 8>;
-  if ((e = launch_chained(scan, dim3(De / 64, (B + tpw - 1) / tpw), 128, st, true, (const bf16*)dr, (const bf16*)w.W_dt, w.b_dt, R, w.A, (const float*)Bm, (const float*)Cm, w.D,
+  auto scan = c.disc_mode == 0 ? step_dt_scan<true> : step_dt_scan<false>;
+  if ((e = launch_chained(scan, dim3(De / 64, (B + 7) / 8), 128, st, true, (const bf16*)dr, (const bf16*)w.W_dt, w.b_dt, R, w.A, (const float*)Bm, (const float*)Cm, w.D,
                           (const bf16*)U, (const bf16*)(K == 1 ? XZ + De : Zs), K == 1 ? 2 * De : De, ssm_state, Yg, B, De)) != cudaSuccess) return e;
   StepGemmArgs ao{};
   ao.x = Yg; ao.ldx = De; ao.W = (const bf16*)w.W_out; ao.Kd = De; ao.n_rows = Dm; ao.idx = idx; ao.gates = gates; ao.B = B; ao.K = K; ao.E = c.E;

@@ -34,7 +34,6 @@ def test_step_small_parity(kw):
     dict(B=1, E=9, K=1, d_model=2112, d_inner=192, router_bias_scale=1.0),     # a second round of the contracted index, a lone ninth expert
     dict(B=2, E=8, K=1, d_model=256, d_inner=2304, d_conv=2),                  # two tokens, two experts: the most blocks that route themselves
     dict(B=2, E=8, K=1, d_model=256, d_inner=2368),                            # more: a launch of its own routes
-    dict(B=4, E=1, K=1, d_model=64, d_inner=128), dict(B=5, E=1, K=1, d_model=64, d_inner=128),      # four and eight tokens a warp
 ])
 def test_step_route_inside_the_projection(kw):
     run_steps(small_shape(**{**dict(L=4, dtype="bf16"), **kw}), 3)
