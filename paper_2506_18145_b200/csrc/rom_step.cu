@@ -5,7 +5,7 @@
 //                   (one or two tokens: inside the In Proj, four launches)
 //   step_gemm<IN> : grouped [Conv Proj | Gate Proj] of the selected experts; at top-1 its output op also runs the short conv
 //                   on the caller's window of H (step_conv does both for K > 1, where H is a sum over experts)
-//   step_gemm<X>  : x Proj -> delta_r | B | C
+//   step_xproj    : x Proj -> delta_r | B | C, clusters of eight CTAs that share the contracted index
 //   step_dt_scan  : dt Proj + softplus, one step of the recurrence on the caller's state, skip, gate
 //   step_gemm<OUT>: grouped Out Proj, times the gate (K > 1: rows summed by step_combine)
 //
@@ -167,16 +167,14 @@ step_route(const RouteArgs p) {
 }
 
 // ---------------------------------------------------------------------------------------------- projections
-enum StepGemm { STEP_IN = 0, STEP_X = 1, STEP_OUT = 2 };
+enum StepGemm { STEP_IN = 0, STEP_OUT = 1 };
 struct StepGemmArgs {
-  const bf16* x; int ldx;               // activation rows: IN: x [B, Dm]; X: U [B, De]; OUT: Yg [B, De]
-  const bf16* W; int Kd, n_rows;        // weights [E or 1, n_rows, Kd]
+  const bf16* x; int ldx;               // activation rows: IN: x [B, Dm]; OUT: Yg [B, De]
+  const bf16* W; int Kd, n_rows;        // weights [E, n_rows, Kd]
   const int32_t* idx; const float* gates; int B, K, E;
-  bf16* C; int ldc;                     // IN: XZ [B K, 2 De]; X: delta_r [B, R]; OUT: out [B, Dm] (K == 1) or Op [B K, Dm]
+  bf16* C; int ldc;                     // IN: XZ [B K, 2 De]; OUT: out [B, Dm] (K == 1) or Op [B K, Dm]
   // IN at top-1: the short conv
   int De; const bf16* w_conv; const float* b_conv; float* conv_state; int dconv; bf16* U;
-  // X
-  float* Bm; float* Cm; int R;
   int tile_rows;                        // step_tc: rows per weight tile
 };
 
@@ -187,7 +185,7 @@ struct StepGemmArgs {
 // tokens 37.0 -> 33.3 (routing inside without the limit on the blocks: 37.7 and 45.5 for the last two, second waves route again).
 constexpr int kRouteInside = 2;
 template <int MODE, int RT, int WARPS, bool ROUTE = false>
-__global__ void __launch_bounds__(WARPS * 32, MODE == STEP_IN ? 2 : MODE == STEP_OUT ? 1 : 0)
+__global__ void __launch_bounds__(WARPS * 32, MODE == STEP_IN ? 2 : 1)
 step_gemm(const StepGemmArgs p, const RouteArgs rt) {
   constexpr int ROWS = RT * 16, COLS = 8, PITCH = ROWS + 4, PAIRS = ROWS / 2;
   constexpr int U = RT == 2 ? 4 : 8;                 // 32-wide blocks in flight per warp
@@ -201,49 +199,43 @@ step_gemm(const StepGemmArgs p, const RouteArgs rt) {
   const int row0 = blockIdx.x * ROWS;
   const int nkb = p.Kd / 32;
 
-  int e = 0;
-  int m;                                             // tokens of this block
   if (ROUTE) pdl_trigger();                          // the first kernel of the chain
   else if (MODE == STEP_IN) { pdl_wait(); pdl_trigger(); }      // (OUT: the routing tables are two kernels back, complete already)
-  if (MODE != STEP_X) {
-    // the blockIdx.y-th selected expert and its assignments (in whatever order: a token's column does not matter)
-    const int A = p.B * p.K;
-    int mine = -1;                                   // thread a < A: the expert of assignment a
-    if constexpr (ROUTE) {
-      __shared__ RouteSmem rs;
-      if (blockIdx.x == gridDim.x - 1) {
-        if (blockIdx.y) return;
-        if (threadIdx.x < kStatusInts) rt.status[threadIdx.x] = 0;
-        for (int t = 0; t < p.B; ++t) { route_token(rt, t, rs); __syncthreads(); }
-        return;
-      }
-      for (int t = 0; t < p.B; ++t) {
-        route_logits(rt, t, rs);
-        const int k = (int)threadIdx.x - t * p.K;    // thread t K + k walks the picks up to its own
-        unsigned long long taken = 0ull;
-        if (k >= 0 && k < p.K)
-          for (int q = 0; q <= k; ++q) mine = route_pick(rs.lg, p.E, taken);
-      }
-    } else if (threadIdx.x < A) {
-      mine = p.idx[threadIdx.x];
-    }
-    if (threadIdx.x == 0) { mask = 0ull; count = 0; }
-    __syncthreads();
-    if (mine >= 0) atomicOr(&mask, 1ull << mine);
-    __syncthreads();
-    unsigned long long mk = mask;
-    for (int i = 0; i < (int)blockIdx.y && mk; ++i) mk &= mk - 1;
-    if (!mk) {
-      if (MODE == STEP_OUT) { pdl_wait(); pdl_trigger(); }
+  // the blockIdx.y-th selected expert and its assignments (in whatever order: a token's column does not matter)
+  const int A = p.B * p.K;
+  int mine = -1;                                     // thread a < A: the expert of assignment a
+  if constexpr (ROUTE) {
+    __shared__ RouteSmem rs;
+    if (blockIdx.x == gridDim.x - 1) {
+      if (blockIdx.y) return;
+      if (threadIdx.x < kStatusInts) rt.status[threadIdx.x] = 0;
+      for (int t = 0; t < p.B; ++t) { route_token(rt, t, rs); __syncthreads(); }
       return;
     }
-    e = __ffsll(mk) - 1;
-    if (mine == e) list[atomicAdd(&count, 1)] = threadIdx.x;
-    __syncthreads();
-    m = count;
-  } else {
-    m = min(COLS, p.B - (int)blockIdx.y * COLS);
+    for (int t = 0; t < p.B; ++t) {
+      route_logits(rt, t, rs);
+      const int k = (int)threadIdx.x - t * p.K;      // thread t K + k walks the picks up to its own
+      unsigned long long taken = 0ull;
+      if (k >= 0 && k < p.K)
+        for (int q = 0; q <= k; ++q) mine = route_pick(rs.lg, p.E, taken);
+    }
+  } else if (threadIdx.x < A) {
+    mine = p.idx[threadIdx.x];
   }
+  if (threadIdx.x == 0) { mask = 0ull; count = 0; }
+  __syncthreads();
+  if (mine >= 0) atomicOr(&mask, 1ull << mine);
+  __syncthreads();
+  unsigned long long mk = mask;
+  for (int i = 0; i < (int)blockIdx.y && mk; ++i) mk &= mk - 1;
+  if (!mk) {
+    if (MODE == STEP_OUT) { pdl_wait(); pdl_trigger(); }
+    return;
+  }
+  const int e = __ffsll(mk) - 1;
+  if (mine == e) list[atomicAdd(&count, 1)] = threadIdx.x;
+  __syncthreads();
+  const int m = count;                               // tokens of this block
   const bf16* wrow[RT][2];
 #pragma unroll
   for (int r = 0; r < RT; ++r)
@@ -253,7 +245,7 @@ step_gemm(const StepGemmArgs p, const RouteArgs rt) {
   // output of this thread: two adjacent rows of one token, and what it takes besides the products, requested with the weights
   const int j_out = threadIdx.x / PAIRS, row_out = row0 + (threadIdx.x % PAIRS) * 2;
   const bool has_out = j_out < m;
-  const int a_out = MODE != STEP_X && has_out ? list[j_out] : 0;
+  const int a_out = has_out ? list[j_out] : 0;
   const bool conv = MODE == STEP_IN && p.U != nullptr && has_out && row_out < p.De;
   float2 win[3], taps[4], ub = make_float2(0.0f, 0.0f);
   float gate = 1.0f;
@@ -272,7 +264,7 @@ step_gemm(const StepGemmArgs p, const RouteArgs rt) {
   };
 
   bool waited = MODE == STEP_IN;
-  const int tok_g = g < m ? (MODE == STEP_X ? (int)blockIdx.y * COLS + g : list[g] / p.K) : -1;
+  const int tok_g = g < m ? list[g] / p.K : -1;
   const bf16* xrow = tok_g >= 0 ? p.x + (size_t)tok_g * p.ldx + 8 * t4 : nullptr;
   float acc[RT][4] = {};
   for (int kb0 = warp; kb0 < nkb; kb0 += WARPS * U) {
@@ -313,12 +305,7 @@ step_gemm(const StepGemmArgs p, const RouteArgs rt) {
   }
   const size_t a = a_out;
   const int row = row_out;
-  if (MODE == STEP_X) {
-    const size_t tok = blockIdx.y * COLS + j_out;
-    if (row < p.R) *reinterpret_cast<__nv_bfloat162*>(p.C + tok * p.R + row) = __floats2bfloat162_rn(v.x, v.y);
-    else if (row < p.R + NST) *reinterpret_cast<float2*>(p.Bm + tok * NST + row - p.R) = v;
-    else *reinterpret_cast<float2*>(p.Cm + tok * NST + row - p.R - NST) = v;
-  } else if (MODE == STEP_OUT) {
+  if (MODE == STEP_OUT) {
     *reinterpret_cast<__nv_bfloat162*>(p.C + a * p.ldc + row) = __floats2bfloat162_rn(v.x * gate, v.y * gate);
   } else if (p.U == nullptr) {                       // K > 1: rows of the assignment, summed over the slots by step_conv
     *reinterpret_cast<__nv_bfloat162*>(p.C + a * p.ldc + row) = __floats2bfloat162_rn(v.x, v.y);
@@ -664,6 +651,82 @@ step_conv(const bf16* __restrict__ XZ, int K, int De, const bf16* __restrict__ w
   *reinterpret_cast<float2*>(st + (size_t)(dconv - 2) * De) = h;
 }
 
+// ---------------------------------------------------------------------------------------------- x Proj
+// 16 weight rows and up to 16 tokens a cluster of eight CTAs, which share the contracted index: its 32-wide blocks are dealt out to the
+// CTAs and their warps, the partial sums meet in shared memory (warps, in order) and across the cluster (CTAs, in order; the order is
+// the same for every batch).  What bounds it: latency; a row is 2 De bytes, and one block per 16 rows and 8 tokens, as before, took
+// 131 KB of weights through one SM (7.8 us from the end of the In Proj at 64 tokens).  us a step, before / 64, 32, 16, 8 tokens a
+// cluster: 64 tokens of 2048 channels 101.9 / 101.7, 103.6, 100.1, 103.3; 8 tokens 74.3 / 71.5, 71.9, 71.1, 71.5; 1 token 23.6 / -, -,
+// 23.2, -; 4 of 1024 35.1 / -, -, 33.2, -.
+constexpr int XC = 8, X_TOK = 16, X_WARPS = 8;
+__global__ void __launch_bounds__(X_WARPS * 32)
+step_xproj(const bf16* __restrict__ U, const bf16* __restrict__ W, int De, int R, bf16* __restrict__ delta_r, float* __restrict__ Bm,
+           float* __restrict__ Cm, int B) {
+  constexpr int ROWS = 16, NG = X_TOK / 8, KB = 2;      // KB: blocks of a warp in flight
+  __shared__ __align__(16) float red[X_WARPS][X_TOK][ROWS + 1];
+  __shared__ float part[X_TOK][ROWS];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t4 = lane & 3;
+  const int rank = (int)cluster_rank(), row0 = blockIdx.y * ROWS, tb = blockIdx.z * X_TOK, nt = min(X_TOK, B - tb);
+  const int nkb = De / 32, lo = nkb * rank / XC, hi = nkb * (rank + 1) / XC;
+  const bf16* w0 = W + (size_t)(row0 + g) * De + 8 * t4;
+  const bf16* w1 = w0 + (size_t)8 * De;
+  const uint4 zero4 = make_uint4(0, 0, 0, 0);
+  float acc[NG][4] = {};
+  bool waited = false;
+  for (int kb0 = lo + warp; kb0 < hi; kb0 += X_WARPS * KB) {
+    uint4 q0[KB], q1[KB];
+#pragma unroll
+    for (int k = 0; k < KB; ++k) {
+      const int kb = kb0 + k * X_WARPS;
+      q0[k] = kb < hi ? ld_stream(w0 + kb * 32) : zero4;
+      q1[k] = kb < hi ? ld_stream(w1 + kb * 32) : zero4;
+    }
+    if (!waited) { pdl_wait(); pdl_trigger(); waited = true; }
+    uint4 xq[NG][KB];                  // (all of them requested before the first is used)
+#pragma unroll
+    for (int n = 0; n < NG; ++n)
+#pragma unroll
+      for (int k = 0; k < KB; ++k) {
+        const int kb = kb0 + k * X_WARPS;
+        xq[n][k] = n * 8 + g < nt && kb < hi ? ld_act(U + (size_t)(tb + n * 8 + g) * De + 8 * t4 + kb * 32) : zero4;
+      }
+#pragma unroll
+    for (int n = 0; n < NG; ++n)
+#pragma unroll
+      for (int k = 0; k < KB; ++k) mma_block(acc[n], q0[k], q1[k], xq[n][k]);
+  }
+  if (!waited) { pdl_wait(); pdl_trigger(); }
+#pragma unroll
+  for (int n = 0; n < NG; ++n) {
+    if (n * 8 >= nt) break;
+    float (*r)[ROWS + 1] = red[warp] + n * 8 + 2 * t4;
+    r[0][g] = acc[n][0]; r[1][g] = acc[n][1]; r[0][g + 8] = acc[n][2]; r[1][g + 8] = acc[n][3];
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < nt * ROWS; i += X_WARPS * 32) {
+    float v = 0.0f;
+#pragma unroll
+    for (int w = 0; w < X_WARPS; ++w) v += red[w][i / ROWS][i % ROWS];
+    part[i / ROWS][i % ROWS] = v;
+  }
+  cluster_sync();
+  // CTA q finishes tokens q, q + 8, ...
+  for (int i = threadIdx.x; i < X_TOK / XC * ROWS; i += X_WARPS * 32) {
+    const int t = (i / ROWS) * XC + rank, r = i % ROWS, row = row0 + r;
+    if (t >= nt) continue;
+    float q[XC], v = 0.0f;
+#pragma unroll
+    for (int c = 0; c < XC; ++c) asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(q[c]) : "r"(map_rank(smem_u32(&part[t][r]), c)) : "memory");
+#pragma unroll
+    for (int c = 0; c < XC; ++c) v += q[c];
+    const size_t tok = tb + t;
+    if (row < R) delta_r[tok * R + row] = __float2bfloat16_rn(v);
+    else if (row < R + NST) Bm[tok * NST + row - R] = v;
+    else Cm[tok * NST + row - R - NST] = v;
+  }
+  cluster_sync();                      // nobody leaves while its sums may still be read
+}
+
 // ---------------------------------------------------------------------------------------------- dt Proj + recurrence
 // A warp takes 16 channels x 8 tokens: Delta by MMA, then one (channel half, token) at a time with four lanes per channel (four
 // states each), so that states move as whole 512-byte rows.  The states (the traffic that counts: 8 KB in and out per warp), A and
@@ -876,9 +939,21 @@ cudaError_t launch_step_small(const rom_config& c, const rom_weights& w, const v
   if (e != cudaSuccess) return e;
   if (K > 1 && (e = launch_chained(step_conv, dim3((De / 2 + 127) / 128, B), 128, st, true, (const bf16*)XZ, K, De, (const bf16*)w.w_conv, w.b_conv, conv_state,
                                    c.d_conv, U, Zs)) != cudaSuccess) return e;
-  StepGemmArgs ax{};
-  ax.x = U; ax.ldx = De; ax.W = (const bf16*)w.W_x; ax.Kd = De; ax.n_rows = R + 2 * NST; ax.B = B; ax.K = K; ax.C = dr; ax.ldc = R; ax.Bm = Bm; ax.Cm = Cm; ax.R = R;
-  if ((e = launch_step_gemm<STEP_X, 1, 16>(ax, dim3((R + 2 * NST) / 16, (B + 7) / 8), st)) != cudaSuccess) return e;
+  {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(XC, (R + 2 * NST) / 16, (B + X_TOK - 1) / X_TOK);
+    cfg.blockDim = dim3(X_WARPS * 32);
+    cfg.stream = st;
+    cudaLaunchAttribute at[2]{};
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = XC; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    count_launch();
+    if ((e = cudaLaunchKernelEx(&cfg, step_xproj, (const bf16*)U, (const bf16*)w.W_x, De, R, dr, Bm, Cm, B)) != cudaSuccess) return e;
+  }
   auto scan = c.disc_mode == 0 ? step_dt_scan<true> : step_dt_scan<false>;
   if ((e = launch_chained(scan, dim3(De / 64, (B + 7) / 8), 128, st, true, (const bf16*)dr, (const bf16*)w.W_dt, w.b_dt, R, w.A, (const float*)Bm, (const float*)Cm, w.D,
                           (const bf16*)U, (const bf16*)(K == 1 ? XZ + De : Zs), K == 1 ? 2 * De : De, ssm_state, Yg, B, De)) != cudaSuccess) return e;
