@@ -152,6 +152,91 @@ m2_conv_kernel(const T* __restrict__ ZXs, const T* __restrict__ w_conv, const fl
   if ((emax >> 16) == 0x7f80u || (emax & 0xffffu) == 0x7f80u) *nonfinite = 1;      // (every writer stores the same)
 }
 
+// The same in bf16 for many tokens: a thread walks seg steps of its 8 channels with the last four rows in registers as packed fp32 pairs
+// and the next four in flight, as the layer's conv does (rom_conv.cu).  HBM-bound; above, a thread loads 19 rows, computes and ends, so
+// that loads and arithmetic overlap only between blocks and every row is widened for each of its four taps.  (Channel groups and
+// segments share one index: 516 groups of 4096 channels would leave the last of five blocks nearly empty.)  16384 steps of 4096 channels:
+// 87 -> 69 us, whatever the steps to a thread (16, 32, 64) and with three blocks an SM as with four; used once its blocks give every
+// SM one.
+__global__ void __launch_bounds__(128, 4)
+m2_conv_roll_kernel(const __nv_bfloat16* __restrict__ ZXs, const __nv_bfloat16* __restrict__ w_conv, const float* __restrict__ b_conv,
+                    __nv_bfloat16* __restrict__ xc, float* __restrict__ Bm, float* __restrict__ Cm, int L, int De, int N, int W, int k,
+                    int seg, int32_t* __restrict__ nonfinite) {
+  pdl_sync();
+  typedef V16<__nv_bfloat16> Vec;
+  const int Cs = De + 2 * N, nv = Cs / 8;
+  const long long id = (long long)blockIdx.x * 128 + threadIdx.x;
+  const int c0 = (int)(id % nv) * 8;
+  const long long sg = id / nv;
+  if (sg * seg >= L) return;
+  const int tb = (int)sg * seg, te = min(tb + seg, L);
+  const size_t tok0 = (size_t)blockIdx.y * L;
+  const __nv_bfloat16* src = ZXs + tok0 * W + De + c0;
+  Vec nxt[4], halo[3];
+  auto fetch = [&](Vec& r, int t) { if (t >= 0 && t < te) r.load(src + (size_t)t * W); else r.zero(); };
+#pragma unroll
+  for (int r = 0; r < 3; ++r) fetch(halo[r], tb - 3 + r);
+#pragma unroll
+  for (int r = 0; r < 4; ++r) fetch(nxt[r], tb + r);
+  float2 w[4][4], bias[4];             // taps right-aligned into 4 slots: slot 3 multiplies the current token
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int q = j - (4 - k);
+    float v[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    if (q >= 0) { Vec t; t.load(w_conv + (size_t)q * Cs + c0); t.get(v); }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[j][i] = make_float2(v[2 * i], v[2 * i + 1]);
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) bias[i] = b_conv ? make_float2(__ldg(b_conv + c0 + 2 * i), __ldg(b_conv + c0 + 2 * i + 1)) : make_float2(0.0f, 0.0f);
+  float2 h[4][4];                      // row t in slot t & 3 (tb is a multiple of four)
+  auto widen = [&](const Vec& r, float2 (&o)[4]) {
+    float v[8];
+    r.get(v);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) o[i] = make_float2(v[2 * i], v[2 * i + 1]);
+  };
+#pragma unroll
+  for (int r = 0; r < 3; ++r) widen(halo[r], h[r + 1]);
+  uint32_t emax = 0u;                  // largest exponent field of the x written (both halves)
+  for (int t0 = tb; t0 < te; t0 += 4) {
+    Vec cur[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) { cur[r] = nxt[r]; fetch(nxt[r], t0 + 4 + r); }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      widen(cur[r], h[r]);
+      float u[8];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        float2 pre = bias[i];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) pre = __ffma2_rn(w[j][i], h[(r + 1 + j) & 3][i], pre);
+        u[2 * i] = silu_fast(pre.x);
+        u[2 * i + 1] = silu_fast(pre.y);
+      }
+      if (t0 + r >= te) break;
+      const size_t tok = tok0 + t0 + r;
+      if (c0 < De) {
+        uint4 o;
+        uint32_t* ow = reinterpret_cast<uint32_t*>(&o);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const __nv_bfloat162 b = __floats2bfloat162_rn(u[2 * i], u[2 * i + 1]);
+          ow[i] = *reinterpret_cast<const uint32_t*>(&b);
+          emax = __vmaxu2(emax, ow[i] & 0x7f807f80u);
+        }
+        *reinterpret_cast<uint4*>(xc + tok * De + c0) = o;
+      } else {
+        float* dst = c0 < De + N ? Bm + tok * N + (c0 - De) : Cm + tok * N + (c0 - De - N);
+        *reinterpret_cast<float4*>(dst) = make_float4(u[0], u[1], u[2], u[3]);
+        *reinterpret_cast<float4*>(dst + 4) = make_float4(u[4], u[5], u[6], u[7]);
+      }
+    }
+  }
+  if ((emax >> 16) == 0x7f80u || (emax & 0xffffu) == 0x7f80u) *nonfinite = 1;      // (every writer stores the same)
+}
+
 // Delta[t, c] = softplus(dt_raw[t, head(c)] + dt_bias[head(c)]) expanded over the head's channels (fp32), four channels
 // per thread; the first threads also expand A_h, D_h to the per-(channel, state) / per-channel arrays the scan kernel reads.
 template <typename T>
@@ -355,7 +440,13 @@ int rom_mamba2_layer_forward(const rom_config* cfg, int32_t headdim, const rom_m
     dim3 cgrid((Cs / vec + 127) / 128, (c.L + M2_TCH - 1) / M2_TCH, c.B);
     float* Bm = reinterpret_cast<float*>(W + m.Bm);
     float* Cm = reinterpret_cast<float*>(W + m.Cm);
-    if (bf) launch_k(m2_conv_kernel<__nv_bfloat16>, cgrid, 128, 0, st, (const __nv_bfloat16*)(W + m.ZXs), (const __nv_bfloat16*)w->w_conv, w->b_conv,
+    const long long nv = Cs / vec;
+    const int seg = nv * c.B * ((c.L + 63) / 64) >= 148LL * 12 * 128 ? 64 : 32;
+    const long long walk_blocks = (nv * ((c.L + seg - 1) / seg) + 127) / 128;
+    if (bf && walk_blocks * c.B >= 148)
+      launch_k(m2_conv_roll_kernel, dim3((unsigned)walk_blocks, c.B), 128, 0, st, (const __nv_bfloat16*)(W + m.ZXs), (const __nv_bfloat16*)w->w_conv, w->b_conv,
+                                                                              (__nv_bfloat16*)(W + m.xc), Bm, Cm, c.L, De, N, Wd, c.d_conv, seg, status + kStatNonFinite);
+    else if (bf) launch_k(m2_conv_kernel<__nv_bfloat16>, cgrid, 128, 0, st, (const __nv_bfloat16*)(W + m.ZXs), (const __nv_bfloat16*)w->w_conv, w->b_conv,
                                                                 (__nv_bfloat16*)(W + m.xc), Bm, Cm, c.L, De, N, Wd, c.d_conv, status + kStatNonFinite);
     else launch_k(m2_conv_kernel<float>, cgrid, 128, 0, st, (const float*)(W + m.ZXs), (const float*)w->w_conv, w->b_conv, (float*)(W + m.xc), Bm, Cm,
                                                     c.L, De, N, Wd, c.d_conv, status + kStatNonFinite);
