@@ -136,6 +136,63 @@ combine_bwd_kernel(const T* __restrict__ dYgu, T* Ygp, const int32_t* __restrict
   }
 }
 
+// The same in bf16 for top-1 and top-2, the scaled rows written: a warp per token, four 16-byte pieces of every row in flight and no
+// block barrier.  HBM-bound (2 K + 2 rows a token); with the experts of a token in a loop of unknown length and one block per token,
+// 16384 tokens of 4096 channels took 123 us, here 90 (82 at the copy bandwidth); 4113 of 2048 at top-2 22 -> 16.
+template <int KT>
+__global__ void __launch_bounds__(128)
+combine_bwd_warp_kernel(const __nv_bfloat16* __restrict__ dYgu, __nv_bfloat16* Ygp, const int32_t* __restrict__ row_of_assign,
+                        const float* __restrict__ gates, __nv_bfloat16* __restrict__ dYg, float* __restrict__ dgate, int De, long long Tn) {
+  pdl_sync();
+  typedef V16<__nv_bfloat16> Vec;
+  const int lane = threadIdx.x & 31;
+  const long long t = (long long)blockIdx.x * 4 + (threadIdx.x >> 5);
+  if (t >= Tn) return;
+  size_t rows[KT];
+  float g[KT], part[KT];
+#pragma unroll
+  for (int k = 0; k < KT; ++k) { rows[k] = (size_t)__ldg(row_of_assign + t * KT + k); g[k] = __ldg(gates + t * KT + k); part[k] = 0.0f; }
+  const int nv = De / 8;
+  constexpr int G = 4;
+  for (int v0 = lane; v0 < nv; v0 += 32 * G) {
+    Vec y[G], b[G][KT];
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+      const int v = min(v0 + 32 * i, nv - 1);      // (past the end: loaded and not used)
+      y[i].q = *reinterpret_cast<const uint4*>(Ygp + rows[0] * De + (size_t)v * 8);      // the K rows of a token hold the same gated scan output
+#pragma unroll
+      for (int k = 0; k < KT; ++k) b[i][k].load(dYgu + rows[k] * De + (size_t)v * 8);
+    }
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+      if (v0 + 32 * i >= nv) break;
+      float yv[8], acc[8];
+      y[i].get(yv);
+#pragma unroll
+      for (int k = 0; k < KT; ++k) {
+        float bv[8];
+        b[i][k].get(bv);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) { acc[j] = fmaf(g[k], bv[j], k == 0 ? 0.0f : acc[j]); part[k] = fmaf(bv[j], yv[j], part[k]); }
+      }
+      Vec::store(dYg + t * De + (size_t)(v0 + 32 * i) * 8, acc);
+#pragma unroll
+      for (int k = 0; k < KT; ++k) {
+        float sv[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) sv[j] = g[k] * yv[j];
+        Vec::store(Ygp + rows[k] * De + (size_t)(v0 + 32 * i) * 8, sv);
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < KT; ++k) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) part[k] += __shfl_xor_sync(0xffffffffu, part[k], o);
+    if (lane == 0) dgate[t * KT + k] = part[k];
+  }
+}
+
 // dxdbl[t, R + j] = dB[t, j] (j < N) or dC[t, j - N]: the B | C part of the gradient of (delta, B, C) = U W_x
 template <typename T>
 __global__ void __launch_bounds__(256)
@@ -337,6 +394,90 @@ dx_kernel(const T* __restrict__ dxp, const int32_t* __restrict__ row_of_assign, 
   stv(dx + t * Dm + c0, acc);
 }
 
+// The same in bf16 for 4, 8 or 16 experts at top-1 and top-2: a thread keeps its 8 columns of W_r and walks seg tokens, four in flight
+// (their row indices four tokens earlier still).  Above, every vector of dx reads and widens all E of W_r, about 170 instructions: 16384
+// tokens of 2048 channels with 8 experts 58 us, here 38 (20 at the copy bandwidth), 4113 of 1024 at top-2 11.6 -> 8.9.  Eight tokens to a
+// thread: with 16 and 32 the former takes 36 and 35, the latter 11.6 and 19.9 (too few threads).
+template <int NE, int KT>
+__global__ void __launch_bounds__(128, NE <= 8 ? 4 : 2)
+dx_walk_kernel(const __nv_bfloat16* __restrict__ dxp, const int32_t* __restrict__ row_of_assign, const float* __restrict__ dlogit,
+               const __nv_bfloat16* __restrict__ W_r, __nv_bfloat16* __restrict__ dx, int Dm, int seg, long long Tn) {
+  pdl_sync();
+  typedef V16<__nv_bfloat16> Vec;
+  constexpr int G = 4;
+  constexpr bool WIDE = NE <= 8;       // W_r widened once; 16 experts stay as stored
+  const int nv = Dm / 8;
+  const long long id = (long long)blockIdx.x * 128 + threadIdx.x;
+  const int c0 = (int)(id % nv) * 8;
+  const long long tb = id / nv * seg, te = min(tb + seg, Tn);
+  if (tb >= Tn) return;
+  Vec wr[NE];
+  float2 w[WIDE ? NE : 1][4];
+#pragma unroll
+  for (int e = 0; e < NE; ++e) wr[e].load(W_r + (size_t)e * Dm + c0);
+  auto pairs = [](const Vec& q, float2 (&o)[4]) {
+    float v[8];
+    q.get(v);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) o[i] = make_float2(v[2 * i], v[2 * i + 1]);
+  };
+  if constexpr (WIDE) {
+#pragma unroll
+    for (int e = 0; e < NE; ++e) pairs(wr[e], w[e]);
+  }
+  int32_t ix[G][KT];
+  Vec nxt[G][KT];
+  auto index = [&](long long t0) {
+#pragma unroll
+    for (int i = 0; i < G; ++i)
+#pragma unroll
+      for (int k = 0; k < KT; ++k) ix[i][k] = __ldg(row_of_assign + min(t0 + i, te - 1) * KT + k);      // (past the end: the last token again)
+  };
+  auto fetch = [&]() {
+#pragma unroll
+    for (int i = 0; i < G; ++i)
+#pragma unroll
+      for (int k = 0; k < KT; ++k) nxt[i][k].load(dxp + (size_t)ix[i][k] * Dm + c0);
+  };
+  index(tb);
+  fetch();
+  index(tb + G);
+  for (long long t0 = tb; t0 < te; t0 += G) {
+    Vec cur[G][KT];
+#pragma unroll
+    for (int i = 0; i < G; ++i)
+#pragma unroll
+      for (int k = 0; k < KT; ++k) cur[i][k] = nxt[i][k];
+    fetch();
+    index(t0 + 2 * G);
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+      const long long t = min(t0 + i, te - 1);
+      float4 dl[NE / 4];
+#pragma unroll
+      for (int q = 0; q < NE / 4; ++q) dl[q] = __ldg(reinterpret_cast<const float4*>(dlogit + t * NE) + q);
+      float2 acc[4], v[4];
+      pairs(cur[i][0], acc);
+      if constexpr (KT == 2) {
+        pairs(cur[i][1], v);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[j] = __fadd2_rn(acc[j], v[j]);
+      }
+#pragma unroll
+      for (int e = 0; e < NE; ++e) {
+        const float f = (e & 3) == 0 ? dl[e / 4].x : (e & 3) == 1 ? dl[e / 4].y : (e & 3) == 2 ? dl[e / 4].z : dl[e / 4].w;
+        if constexpr (!WIDE) pairs(wr[e], v);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[j] = __ffma2_rn(make_float2(f, f), WIDE ? w[WIDE ? e : 0][j] : v[j], acc[j]);
+      }
+      if (t0 + i < te) {
+        const float o[8] = {acc[0].x, acc[0].y, acc[1].x, acc[1].y, acc[2].x, acc[2].y, acc[3].x, acc[3].y};
+        Vec::store(dx + t * Dm + c0, o);
+      }
+    }
+  }
+}
+
 // dW_r[e, d] = sum_t dlogit[t, e] x[t, d]: a thread owns four columns of x and eight experts over a slab of tokens (x is read
 // once per eight experts; the slab's dlogit values sit in shared memory), one 16-byte atomic per slab, expert and four columns.
 constexpr int RSLAB = 64;
@@ -461,7 +602,10 @@ cudaError_t launch_slot_sum(int dtype, const void* src, const int32_t* row_of_as
 
 cudaError_t launch_combine_bwd(int dtype, const void* dYgu, void* Ygp, const int32_t* row_of_assign, const float* gates, void* dYg,
                                float* dgate, float* rowscale, long long Tn, int De, int K, cudaStream_t st) {
-  if (dtype == ROM_BF16)
+  if (dtype == ROM_BF16 && !rowscale && K <= 2)
+    launch_k(K == 1 ? combine_bwd_warp_kernel<1> : combine_bwd_warp_kernel<2>, (unsigned)((Tn + 3) / 4), 128, 0, st, (const __nv_bfloat16*)dYgu,
+             (__nv_bfloat16*)Ygp, row_of_assign, gates, (__nv_bfloat16*)dYg, dgate, De, Tn);
+  else if (dtype == ROM_BF16)
     launch_k(combine_bwd_kernel<__nv_bfloat16>, (unsigned)Tn, 128, 0, st, (const __nv_bfloat16*)dYgu, (__nv_bfloat16*)Ygp, row_of_assign, gates,
                                                                   (__nv_bfloat16*)dYg, dgate, rowscale, De, K);
   else
@@ -517,7 +661,14 @@ cudaError_t launch_dx(const rom_config& c, const void* dxp, const int32_t* row_o
                       cudaStream_t st) {
   const long long total = (long long)c.B * c.L * (c.d_model / (c.dtype == ROM_BF16 ? 8 : 4));
   const unsigned blocks = (unsigned)((total + 255) / 256);
-  if (c.dtype == ROM_BF16)
+  if (c.dtype == ROM_BF16 && c.K <= 2 && (c.E == 4 || c.E == 8 || c.E == 16)) {
+    const long long Tn = (long long)c.B * c.L, nv = c.d_model / 8;
+    const int seg = 8;
+    const unsigned wb = (unsigned)((nv * ((Tn + seg - 1) / seg) + 127) / 128);
+    auto go = [&](auto kern) { launch_k(kern, wb, 128, 0, st, (const __nv_bfloat16*)dxp, row_of_assign, dlogit, (const __nv_bfloat16*)W_r, (__nv_bfloat16*)dx, c.d_model, seg, Tn); };
+    if (c.K == 1) go(c.E == 4 ? dx_walk_kernel<4, 1> : c.E == 8 ? dx_walk_kernel<8, 1> : dx_walk_kernel<16, 1>);
+    else go(c.E == 4 ? dx_walk_kernel<4, 2> : c.E == 8 ? dx_walk_kernel<8, 2> : dx_walk_kernel<16, 2>);
+  } else if (c.dtype == ROM_BF16)
     launch_k(dx_kernel<__nv_bfloat16>, blocks, 256, 0, st, (const __nv_bfloat16*)dxp, row_of_assign, dlogit, (const __nv_bfloat16*)W_r, (__nv_bfloat16*)dx,
                                                    c.d_model, c.E, c.K, total);
   else
