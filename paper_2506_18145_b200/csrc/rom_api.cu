@@ -418,7 +418,8 @@ int layer_forward_impl(const rom_config* cfg, const rom_weights* w, const void* 
   ROM_CUDA(launch_scan(c, W + lay.U, W + lay.Delta, false, w->A, reinterpret_cast<float*>(W + lay.Bm),
                        reinterpret_cast<float*>(W + lay.Cm), w->D, zbase, c.K == 1 || slots ? 2 * De : De,
                        slots || (c.K == 1 && !in_token_order) ? row_of_assign : nullptr, ssm_state, W + lay.Ygp, ssm_state, row_of_assign, c.K,
-                       reinterpret_cast<float*>(W + lay.scan_ws), !slots, st));
+                       reinterpret_cast<float*>(W + lay.scan_ws), !slots, st, false, nullptr,
+                       tc && !fused_small && c.small_proj_experts <= 1 && dt_proj_applicable(De, R)));
   ROM_STAGE_DONE();
   // S10 + S11.  Tensor path with one expert per token: the epilogue of the grouped Out Proj scales each row by
   // its gate and writes it at its token's position (no intermediate rows, no combine pass).  Otherwise: grouped
@@ -587,12 +588,13 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
   ROM_CUDA(launch_conv(c1, W + bl.HZs, nullptr, w->w_conv, w->b_conv, W + lay.U, nullptr, st));
   Epilogue e_x{EPI_XPROJ, W + lay.delta_r, R, Bm, Cm, nullptr, R, N, nullptr, nullptr};
   ROM_CUDA(gemm(W + lay.U, De, w->W_x, De, 1, 0, T, R + 2 * N, De, nullptr, nullptr, e_x));
-  Epilogue e_dt{EPI_SOFTPLUS, W + lay.Delta, De, nullptr, nullptr, w->b_dt, 0, 0, nullptr, nullptr};
-  ROM_CUDA(gemm(W + lay.delta_r, R, w->W_dt, R, 1, 0, T, De, R, nullptr, nullptr, e_dt));
   // gated scan output in expert order (operand of the Out Proj weight gradient); padding rows must be zero
   ROM_CUDA(launch_zero_padding(c, W + lay.Ygp, De, W, lay, st));
+  Epilogue e_dt{EPI_SOFTPLUS, W + lay.Delta, De, nullptr, nullptr, w->b_dt, 0, 0, nullptr, nullptr};
+  ROM_CUDA(gemm(W + lay.delta_r, R, w->W_dt, R, 1, 0, T, De, R, nullptr, nullptr, e_dt));
   ROM_CUDA(launch_scan(c, W + lay.U, W + lay.Delta, false, w->A, Bm, Cm, w->D, zraw, 2 * De, nullptr, nullptr, W + lay.Ygp, nullptr,
-                       row_of_assign, c.K, reinterpret_cast<float*>(W + lay.scan_ws), false, st, false, reinterpret_cast<float*>(W + bl.ckpt)));
+                       row_of_assign, c.K, reinterpret_cast<float*>(W + lay.scan_ws), false, st, false, reinterpret_cast<float*>(W + bl.ckpt),
+                       tc && dt_proj_applicable(De, R)));
 
   // ---- Out Proj and combine, reversed: back_k = dO_t W_out,k; dYg, dgate; dW_out
   ROM_CUDA(launch_gather_rows_to(c, dout, W + bl.dOp, Dm, W, lay, st));

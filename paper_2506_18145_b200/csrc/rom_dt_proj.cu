@@ -79,7 +79,7 @@ dt_proj_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   for (int i = threadIdx.x; i < DT_N; i += DT_THREADS) bias_s[i] = bias && n_tile * block_n + i < N ? __ldg(bias + n_tile * block_n + i) : 0.0f;
-  pdl_sync();
+  pdl_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();

@@ -230,7 +230,8 @@ cudaError_t launch_gemm_tc(const void* A, int lda, const void* Bw, int ldb, int 
                            const Epilogue& epi, int32_t* status, cudaStream_t st, bool test_stall = false, bool b_mn = false,
                            const int32_t* pad_offsets = nullptr /* grouped: the padded segment offsets (n_experts + 1); allows CTA pairs */);
 
-// dt Proj with a short contraction (rom_dt_proj.cu): C[M, N] = softplus(A[M, Kd] Bw[N, Kd]^T + bias), rows contiguous; bf16.
+// dt Proj with a short contraction (rom_dt_proj.cu): C[M, N] = softplus(A[M, Kd] Bw[N, Kd]^T + bias), rows contiguous; bf16.  Its kernel lets
+// the next one in only as its blocks end (a scan's blocks must not pile up).
 bool dt_proj_applicable(int N, int Kd);
 cudaError_t launch_dt_proj(const void* A, const void* Bw, int M, int N, int Kd, const Epilogue& epi, int32_t* status, cudaStream_t st);
 
@@ -276,7 +277,8 @@ cudaError_t launch_scan(const rom_config& c, const void* u, const void* delta, b
                         const float* Cm, const float* D, const void* z, int ldz, const int32_t* z_row, const float* h0,
                         void* y, float* h_last, const int32_t* y_rows, int K, float* chunk_ws, bool gate_activated, cudaStream_t st,
                         bool scalar_A = false /* A[c, :] constant per channel and disc_mode 1: one exponential per channel and step */,
-                        float* ckpt = nullptr /* also store the state at the start of every kScanCkpt steps, [B, ceil(L / kScanCkpt), De, 16] */);
+                        float* ckpt = nullptr /* also store the state at the start of every kScanCkpt steps, [B, ceil(L / kScanCkpt), De, 16] */,
+                        bool after_dt_proj = false /* the launch before is launch_dt_proj's */);
 
 // Scalar-decay recurrence of the Mamba2-style block as chunked matrix products (rom_ssd.cu): bf16, 64 channels per head.  zx: the
 // projection rows [T, W] (gate pre-activation in column 0.., dt pre-activation of head h in column dt_col + h); y: gated rows [T, De].

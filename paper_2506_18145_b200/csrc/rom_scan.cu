@@ -574,7 +574,7 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
   if (e != cudaSuccess) return e;
   a.h0 = h_in; a.h_last = nullptr; a.chunk_off = 1;
   if (warp_kernel) {      // its blocks chain the states before them on their own: 5 us less than the launch (4 x 2048 steps of 2048 channels)
-    a.h0 = nullptr; a.h_last = h_last; a.chain_end = h_end; a.chain_sum = sum_delta;
+    a.h0 = nullptr; a.h_last = h_last; a.chain_end = h_end; a.chain_sum = sum_delta; a.early = 1;
     return chunks(a, nch - 1, FullTag{});
   }
   // (the general kernel's blocks, 2 states to a thread, would take 3 us longer for it than the launch, which overlaps its neighbours)
@@ -591,7 +591,7 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
 cudaError_t launch_scan(const rom_config& c, const void* u, const void* delta, bool delta_fp32, const float* A, const float* Bm,
                         const float* Cm, const float* D, const void* z, int ldz, const int32_t* z_row, const float* h0,
                         void* y, float* h_last, const int32_t* y_rows, int K, float* chunk_ws, bool gate_activated, cudaStream_t st,
-                        bool scalar_A, float* ckpt) {
+                        bool scalar_A, float* ckpt, bool after_dt_proj) {
   int num_sms = 0;
   const cudaError_t e = current_device_sm_count(&num_sms);
   if (e != cudaSuccess) return e;
@@ -601,7 +601,7 @@ cudaError_t launch_scan(const rom_config& c, const void* u, const void* delta, b
   if (chunk_ws == nullptr && !scalar_A && ckpt == nullptr && scan_seq_applicable(c, u, delta, delta_fp32, Bm, Cm, z, ldz, z_row, y_rows, gate_activated, num_sms))
     return launch_scan_seq(c, u, static_cast<const float*>(delta), A, Bm, Cm, D, z, ldz, h0, y, h_last, st);
   const ScanArgs a{u, delta, A, Bm, Cm, D, z, ldz, z_row, h0, y, h_last, y_rows, K, c.L, c.d_inner, c.L, 1, c.L, nullptr, gate_activated ? 1 : 0, 0,
-                   ckpt, (c.L + kScanCkpt - 1) / kScanCkpt, (scalar_A && c.disc_mode == 1) ? 1 : 0};
+                   ckpt, (c.L + kScanCkpt - 1) / kScanCkpt, (scalar_A && c.disc_mode == 1) ? 1 : 0, nullptr, nullptr, after_dt_proj ? 1 : 0};
   if (ckpt != nullptr) {      // the layer backward's recomputed forward: Delta in the storage type
     if (c.dtype != ROM_BF16) return launch_scan_t<float, float, true, true>(c, a, A, h0, h_last, chunk_ws, num_sms, st);
     return delta_fp32 ? cudaErrorInvalidValue : launch_scan_t<__nv_bfloat16, __nv_bfloat16, false, true>(c, a, A, h0, h_last, chunk_ws, num_sms, st);

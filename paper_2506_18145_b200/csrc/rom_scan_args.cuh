@@ -23,6 +23,7 @@ struct ScanArgs {
   // [B, De, 16], written by the last chunk
   const float* chain_end;
   const float* chain_sum;
+  int early;            // warp kernel: the kernel before lets nobody in before its blocks end
 };
 
 __device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }

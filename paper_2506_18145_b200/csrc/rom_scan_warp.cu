@@ -38,8 +38,9 @@ struct WarpTile {
 template <typename TD, bool ZOH, int MODE, bool SLOTS>
 __global__ void __launch_bounds__(BT, 3)
 scan_warp_kernel(const ScanArgs p) {
-  pdl_sync();
   constexpr bool FIRST = MODE == SCAN_FIRST || MODE == SCAN_FIRST_CKPT;
+  pdl_wait();
+  if (!FIRST) pdl_trigger();      // (the second launch comes in as the blocks of the first end: see launch_mode)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   WarpTile& s = reinterpret_cast<WarpTile*>(smem_raw)[warp];
@@ -279,15 +280,18 @@ scan_warp_kernel(const ScanArgs p) {
   }
 }
 
+// A scan is launched early only behind a kernel that lets nobody in before its blocks end: let in while they run, few blocks per SM
+// pile up on the first SMs to drain (+40 % at 256 blocks).  Behind such a kernel (the dt Proj; the first launch of a chunked scan) the
+// launch itself is hidden: 4 x 2048 steps of 2048 channels 5 us less for the two.
 template <typename TD, bool ZOH, int MODE>
 cudaError_t launch_mode(const ScanArgs& a, int B, int grid_z, cudaStream_t st) {
   constexpr int smem = WPB * (int)sizeof(WarpTile);
   const dim3 grid((a.De + BT - 1) / BT, B, grid_z);
   if (a.z_row && a.K > 1) {
-    if constexpr (sizeof(TD) == 2 && (MODE == SCAN_FULL || MODE == SCAN_FIRST)) launch_k(false, scan_warp_kernel<TD, ZOH, MODE, true>, grid, BT, smem, st, a);
+    if constexpr (sizeof(TD) == 2 && (MODE == SCAN_FULL || MODE == SCAN_FIRST)) launch_k(a.early != 0, scan_warp_kernel<TD, ZOH, MODE, true>, grid, BT, smem, st, a);
     else return cudaErrorInvalidValue;
   } else {
-    launch_k(false, scan_warp_kernel<TD, ZOH, MODE, false>, grid, BT, smem, st, a);
+    launch_k(a.early != 0, scan_warp_kernel<TD, ZOH, MODE, false>, grid, BT, smem, st, a);
   }
   count_launch();
   return cudaGetLastError();
