@@ -196,7 +196,7 @@ int rom_route(const rom_config* cfg, const void* x, const void* W_r, const float
   if ((rc = check_device()) != ROM_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   LaunchCounter::count = 0;
-  ROM_CUDA(cudaMemsetAsync(static_cast<char*>(ws) + lay.status, 0, sizeof(int32_t) * kStatusInts, st));
+  ROM_CUDA(launch_init_status(reinterpret_cast<int32_t*>(static_cast<char*>(ws) + lay.status), st));
   ROM_CUDA(launch_route(*cfg, x, W_r, b_r, topk_idx, gates, counts, offsets, perm, inv_perm, static_cast<char*>(ws), lay, st));
   return ROM_OK;
 }
@@ -212,7 +212,7 @@ int rom_route_balance(const rom_config* cfg, const void* x, const void* W_r, con
   if (ws_bytes < lay.total) return ROM_ERR_WORKSPACE;
   if ((rc = check_device()) != ROM_OK) return rc;
   LaunchCounter::count = 0;
-  ROM_CUDA(cudaMemsetAsync(static_cast<char*>(ws) + lay.status, 0, sizeof(int32_t) * kStatusInts, static_cast<cudaStream_t>(stream)));
+  ROM_CUDA(launch_init_status(reinterpret_cast<int32_t*>(static_cast<char*>(ws) + lay.status), static_cast<cudaStream_t>(stream)));
   ROM_CUDA(launch_balance(*cfg, x, W_r, b_r, alpha, F, Pbar, loss, static_cast<char*>(ws), lay, static_cast<cudaStream_t>(stream)));
   return ROM_OK;
 }
@@ -324,7 +324,7 @@ int layer_forward_impl(const rom_config* cfg, const rom_weights* w, const void* 
     if (ev) ROM_CUDA(cudaEventRecord(ev[++stage], st));        \
   } while (0)
   if (ev) ROM_CUDA(cudaEventRecord(ev[0], st));
-  ROM_CUDA(cudaMemsetAsync(status, 0, sizeof(int32_t) * kStatusInts, st));
+  ROM_CUDA(launch_init_status(status, st));
   const bool debug_checks = (c.flags & ROM_FLAG_DEBUG_CHECKS) != 0;
   if (debug_checks) ROM_CUDA(launch_canaries(W, lay, false, st));
   // S1 + S2: router, top-K, permutation tables

@@ -117,7 +117,6 @@ int rom_ffn_moe_forward(const rom_config* cfg, int32_t d_ff, const void* W_gu, c
   const int32_t* row_of_assign = reinterpret_cast<const int32_t*>(W + lay.row_of_assign);
   const int32_t* assign_of_row = reinterpret_cast<const int32_t*>(W + lay.assign_of_row);
 
-  ROM_CUDA(cudaMemsetAsync(status, 0, sizeof(int32_t) * kStatusInts, st));
   // the shared routing decision -> this call's own permutation tables
   ROM_CUDA(launch_perm_from_idx(c, topk_idx, nullptr, nullptr, nullptr, nullptr, W, lay, st));
   ROM_CUDA(launch_gather_rows(c, x, W, lay, st));

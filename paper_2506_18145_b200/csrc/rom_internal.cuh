@@ -194,8 +194,10 @@ cudaError_t launch_route_gather(const rom_config& c, const void* x, const void* 
 cudaError_t launch_balance(const rom_config& c, const void* x, const void* W_r, const float* b_r, float alpha,
                            float* F, float* Pbar, float* loss, char* ws, const WsLayout& lay, cudaStream_t st);
 
+// Status block of a call to zero.
+cudaError_t launch_init_status(int32_t* status, cudaStream_t st);
 // Permutation tables from a routing decision made elsewhere: topk_idx [T, K] (device) -> the same tables launch_route
-// leaves in the workspace (counts, offsets, padded offsets, row tiles, row <-> assignment maps).
+// leaves in the workspace (counts, offsets, padded offsets, row tiles, row <-> assignment maps).  Zeroes the status block first.
 cudaError_t launch_perm_from_idx(const rom_config& c, const int32_t* topk_idx, int32_t* counts, int32_t* offsets, int32_t* perm,
                                  int32_t* inv_perm, char* ws, const WsLayout& lay, cudaStream_t st);
 

@@ -464,7 +464,22 @@ zero_padding(uint4* __restrict__ buf, const int32_t* __restrict__ offsets, const
     for (int v = threadIdx.x; v < vec_per_row; v += blockDim.x) buf[(size_t)r * vec_per_row + v] = make_uint4(0, 0, 0, 0);
 }
 
+// Status block zero; table (may be null): -1 everywhere.  A kernel and not a memset: it chains with the launches around it (a layer of
+// 256 tokens 75.2 -> 72.2 us, 8192 tokens 335.5 -> 333.2).
+__global__ void __launch_bounds__(256)
+init_tables(int32_t* __restrict__ status, int32_t* __restrict__ table, int n) {
+  pdl_sync();
+  if (blockIdx.x == 0 && threadIdx.x < kStatusInts) status[threadIdx.x] = 0;
+  for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) table[i] = -1;
+}
+
 }  // namespace
+
+cudaError_t launch_init_status(int32_t* status, cudaStream_t st) {
+  launch_k(init_tables, 1, 256, 0, st, status, nullptr, 0);
+  count_launch();
+  return cudaGetLastError();
+}
 
 cudaError_t launch_zero_padding(const rom_config& c, void* buf, int width, char* ws, const WsLayout& lay, cudaStream_t st) {
   launch_k(zero_padding, dim3(c.E, 16), 256, 0, st, reinterpret_cast<uint4*>(buf), reinterpret_cast<const int32_t*>(ws + lay.offsets),
@@ -619,7 +634,10 @@ cudaError_t launch_gather_rows_to(const rom_config& c, const void* src, void* ds
 cudaError_t launch_perm_from_idx(const rom_config& c, const int32_t* topk_idx, int32_t* counts, int32_t* offsets, int32_t* perm,
                                  int32_t* inv_perm, char* ws, const WsLayout& lay, cudaStream_t st) {
   int32_t* idx_ws = reinterpret_cast<int32_t*>(ws + lay.topk_idx);
-  cudaError_t err = cudaMemsetAsync(ws + lay.assign_of_row, 0xff, sizeof(int32_t) * lay.rows_max, st);
+  const int rows = (int)lay.rows_max;
+  launch_k(init_tables, (rows + 1023) / 1024, 256, 0, st, reinterpret_cast<int32_t*>(ws + lay.status), reinterpret_cast<int32_t*>(ws + lay.assign_of_row), rows);
+  count_launch();
+  const cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) return err;
   const int wpb = 8;
   launch_k(idx_chunk_histogram, ((int)lay.n_chunks + wpb - 1) / wpb, wpb * 32, 0, st, 
