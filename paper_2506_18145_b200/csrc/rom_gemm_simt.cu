@@ -119,7 +119,8 @@ gemm_simt(const T* __restrict__ A, int lda, const T* __restrict__ Bw, int ldb, i
 //   <128, 128, 8, 8, 1, 16>: shared-memory reads and FMAs in balance; for grids that fill the GPU.
 //   <32, 32, 4, 4, 4, 64>: the contracted index of a stage is split over four thread groups, so that a small product has four
 //     times the blocks' worth of threads in flight and a quarter of the serial steps (256 rows x 1024 columns x 256: the 64 x 64
-//     register-staged kernel took 28 us, waiting for one 16-wide stage after another).
+//     register-staged kernel took 28 us, waiting for one 16-wide stage after another).  <32, 32, 4, 4, 8, 128>, <16, 16, 2, 4, 8, 128>: see
+//     launch_gemm_simt.
 template <int BM, int BN, int TM, int TN, int KS, int BKF>
 __global__ void __launch_bounds__(BM / TM * (BN / TN) * KS)
 gemm_f32(const float* __restrict__ A, int lda, const float* __restrict__ Bw, int ldb, int64_t b_expert_stride, int M_max, int N, int Kd,
@@ -128,20 +129,16 @@ gemm_f32(const float* __restrict__ A, int lda, const float* __restrict__ Bw, int
   constexpr int TY = BM / TM, TX = BN / TN, GT = TY * TX, NT = GT * KS, PITCH = BKF + 4, STAGES = 3, KG = BKF / KS;
   extern __shared__ __align__(16) float smf[];
   const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
-  int M = M_max;
-  if (num_m_tiles_dev) M = min(M_max, *num_m_tiles_dev * kTileM);
-  if (m0 >= M) return;
-  const float* Bp = Bw;
-  if (tile_expert) {
-    const int e = tile_expert[m0 / kTileM];
-    if (e < 0) return;
-    Bp = Bw + (size_t)e * b_expert_stride;
-    if (assign_of_row && assign_of_row[m0] < 0) return;      // a segment's padding is at its end: nothing but padding here, nobody reads it
-  }
+  // (requested together: one after another they cost a small product three trips to the L2 before its first operand)
+  const int nmt = num_m_tiles_dev ? __ldcg(num_m_tiles_dev) : 0, e = tile_expert ? __ldcg(tile_expert + m0 / kTileM) : 0;
+  const int as = tile_expert && assign_of_row ? __ldcg(assign_of_row + m0) : 0;
+  const int M = num_m_tiles_dev ? min(M_max, nmt * kTileM) : M_max;
+  if (m0 >= M || e < 0 || as < 0) return;      // a segment's padding is at its end: nothing but padding here, nobody reads it
+  const float* Bp = Bw + (size_t)e * b_expert_stride;
   const int tid = threadIdx.x, kg = tid / GT, tx = tid % GT % TX, ty = tid % GT / TX;
   auto fetch = [&](int k0, int stage) {
-    float* as = smf + stage * (BM + BN) * PITCH;
-    float* bs = as + BM * PITCH;
+    float* sa = smf + stage * (BM + BN) * PITCH;
+    float* sb = sa + BM * PITCH;
     constexpr int VR = BKF / 4;
 #pragma unroll
     for (int i = tid; i < (BM + BN) * VR; i += NT) {
@@ -150,7 +147,7 @@ gemm_f32(const float* __restrict__ A, int lda, const float* __restrict__ Bw, int
       const int row = isA ? m0 + r : n0 + r - BM;
       const bool ok = (isA ? row < M : row < N) && k0 + k < Kd;
       const float* src = ok ? (isA ? A + (size_t)row * lda : Bp + (size_t)row * ldb) + k0 + k : A;
-      const uint32_t dst = (uint32_t)__cvta_generic_to_shared((isA ? as + r * PITCH : bs + (r - BM) * PITCH) + k);
+      const uint32_t dst = (uint32_t)__cvta_generic_to_shared((isA ? sa + r * PITCH : sb + (r - BM) * PITCH) + k);
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -167,15 +164,15 @@ gemm_f32(const float* __restrict__ A, int lda, const float* __restrict__ Bw, int
     __syncthreads();
     if (kb + STAGES - 1 < n_k) fetch((kb + STAGES - 1) * BKF, (kb + STAGES - 1) % STAGES);
     else asm volatile("cp.async.commit_group;" ::: "memory");
-    const float* as = smf + (kb % STAGES) * (BM + BN) * PITCH + kg * KG;
-    const float* bs = as + BM * PITCH;
+    const float* sa = smf + (kb % STAGES) * (BM + BN) * PITCH + kg * KG;
+    const float* sb = sa + BM * PITCH;
 #pragma unroll
     for (int k = 0; k < KG; k += 4) {
       float4 a[TM], b[TN];
 #pragma unroll
-      for (int i = 0; i < TM; ++i) a[i] = *reinterpret_cast<const float4*>(as + (ty + i * TY) * PITCH + k);
+      for (int i = 0; i < TM; ++i) a[i] = *reinterpret_cast<const float4*>(sa + (ty + i * TY) * PITCH + k);
 #pragma unroll
-      for (int j = 0; j < TN; ++j) b[j] = *reinterpret_cast<const float4*>(bs + (tx + j * TX) * PITCH + k);
+      for (int j = 0; j < TN; ++j) b[j] = *reinterpret_cast<const float4*>(sb + (tx + j * TX) * PITCH + k);
 #pragma unroll
       for (int i = 0; i < TM; ++i)
 #pragma unroll
@@ -291,6 +288,12 @@ cudaError_t launch_gemm_simt(int dtype, const void* A, int lda, const void* Bw, 
     // large tiles once they give every SM a block
     if ((long long)((M_max + 127) / 128) * ((N + 127) / 128) >= 148)
       return launch_f32<128, 128, 8, 8, 1, 16>(a, lda, b, ldb, b_expert_stride, M_max, N, Kd, tile_expert, num_m_tiles_dev, assign_of_row, epi, st);
+    // Longer contractions in stages of 128 over eight groups, half as many serial steps (256 rows x 256 columns x 512: 17.8 us -> 12; 256
+    // columns and less are two to four stages either way and faster with four groups: 256 x 1024 x 256 12.4 us against 14.9), in 16 x 16
+    // tiles where 32 x 32 leave most SMs idle (the x Proj of a short sequence, 256 x 48 x 512: 8 -> 7).
+    if (!tile_expert && (long long)((M_max + 31) / 32) * ((N + 31) / 32) <= 74 && Kd >= 256)
+      return launch_f32<16, 16, 2, 4, 8, 128>(a, lda, b, ldb, b_expert_stride, M_max, N, Kd, tile_expert, num_m_tiles_dev, assign_of_row, epi, st);
+    if (Kd > 256) return launch_f32<32, 32, 4, 4, 8, 128>(a, lda, b, ldb, b_expert_stride, M_max, N, Kd, tile_expert, num_m_tiles_dev, assign_of_row, epi, st);
     return launch_f32<32, 32, 4, 4, 4, 64>(a, lda, b, ldb, b_expert_stride, M_max, N, Kd, tile_expert, num_m_tiles_dev, assign_of_row, epi, st);
   }
   dim3 grid((M_max + BM - 1) / BM, (N + BN - 1) / BN);
