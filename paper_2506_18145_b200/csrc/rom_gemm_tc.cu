@@ -56,7 +56,9 @@ __host__ __device__ constexpr int stage_bytes_of(int mode, int cg = 1) {
 __host__ __device__ constexpr int stages_of(int mode, int cg = 1) {
   return cg == 2 ? (f32_out(mode) ? 5 : 6) : f32_out(mode) ? 3 : mode == EPI_XPROJ ? 6 : MAX_STAGES;
 }
-__host__ __device__ constexpr int out_stage_bytes_of(int mode) { return f32_out(mode) ? epi_warps_of(mode) * 32 * 32 * 4 : 0; }
+// bf16 rows of a grouped product leave through 32 rows x 64 columns a warp (row_out).
+__host__ __device__ constexpr bool row_out(int mode) { return mode == EPI_STORE || mode == EPI_INPROJ || mode == EPI_OUTPROJ || mode == EPI_SWIGLU; }
+__host__ __device__ constexpr int out_stage_bytes_of(int mode) { return f32_out(mode) || row_out(mode) ? epi_warps_of(mode) * 32 * 32 * 4 : 0; }
 __host__ __device__ constexpr int smem_bytes_of(int mode, int cg = 1) {
   return stages_of(mode, cg) * stage_bytes_of(mode, cg) + 1024 /*alignment slack*/ + 256 /*barriers*/ + out_stage_bytes_of(mode);
 }
@@ -71,12 +73,9 @@ __device__ __forceinline__ void load_bias(const Epilogue& ep, int n0, int N, flo
   }
 }
 
-// Fused output op on 32 consecutive accumulator columns [n0, n0+32) of row m (n0 % 32 == 0); columns at
-// or beyond N are skipped in groups of 8 (N % 8 == 0).
-// m: output row; m_tok (EPI_XPROJ with row_token only): row of the B / C parts, the token of this expert-order row.
-template <int MODE>
-__device__ __forceinline__ void epi_store32(const Epilogue& ep, size_t m, size_t m_tok, int n0, int N, const uint32_t (&r)[32],
-                                            float scale, const float4 (&bq)[8]) {
+// x Proj output op on 32 consecutive accumulator columns [n0, n0+32) of row m (n0 % 32 == 0); columns at or beyond N are skipped in groups
+// of 8 (N % 8 == 0).  m: output row; m_tok (with row_token): row of the B / C parts, the token of this expert-order row.
+__device__ __forceinline__ void epi_xproj32(const Epilogue& ep, size_t m, size_t m_tok, int n0, int N, const uint32_t (&r)[32]) {
 #pragma unroll
   for (int j = 0; j < 32; j += 8) {
     const int n = n0 + j;
@@ -84,16 +83,7 @@ __device__ __forceinline__ void epi_store32(const Epilogue& ep, size_t m, size_t
     float v[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[j + i]);
-    if (MODE == EPI_INPROJ && n >= ep.R) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = silu_fast(v[i]);
-    }
-    if (MODE == EPI_OUTPROJ) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] *= scale;
-    }
-    if (MODE == EPI_STORE || MODE == EPI_INPROJ || MODE == EPI_OUTPROJ || (MODE == EPI_XPROJ && n < ep.R)) {
-      const int ld = MODE == EPI_XPROJ ? ep.R : ep.ldc;
+    if (n < ep.R) {
       uint4 q;
       uint32_t* w = reinterpret_cast<uint32_t*>(&q);
 #pragma unroll
@@ -101,14 +91,50 @@ __device__ __forceinline__ void epi_store32(const Epilogue& ep, size_t m, size_t
         __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
         w[i] = *reinterpret_cast<uint32_t*>(&h);
       }
-      *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(ep.C) + m * ld + n) = q;
-    } else if (MODE == EPI_XPROJ) {
+      *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(ep.C) + m * ep.R + n) = q;
+    } else {
       float* dst = (n < ep.R + ep.N) ? ep.Bm + m_tok * ep.N + (n - ep.R) : ep.Cm + m_tok * ep.N + (n - ep.R - ep.N);
       *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
       *reinterpret_cast<float4*>(dst + 4) = make_float4(v[4], v[5], v[6], v[7]);
-    } else {
-      // (softplus and plain-fp32 output go through epi_softplus32; nothing reaches this branch)
     }
+  }
+}
+
+// Row-store output ops: a lane puts 32 columns of its row into the warp's staging rows (128 bytes each, 16-byte pieces swizzled), and the
+// warp writes two adjacent chunks as whole 128-byte row segments, four rows a store instruction.  Straight from the accumulator's lanes a
+// store touched 32 rows with 16 bytes each: 32 half-filled sectors, eight times the requests of the LSU and twice the write sectors of
+// the L2, which together with the activation took longer than the 16 K blocks of a 1024-wide contraction (tensor pipe 53 %).
+// 8192 x 4096 x 1024: 72 -> 63 us; 6102 x 6144 x 1536 106 -> 102; 16384 x 8192 x 2048 385 -> 378.
+template <int MODE>
+__device__ __forceinline__ void stage_rows32(uint4* stage, int cc, const uint32_t (&r)[32], const uint32_t (&up)[32], bool silu, float scale, int lane) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    uint4 q;
+    uint32_t* w = reinterpret_cast<uint32_t*>(&q);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float2 v = make_float2(__uint_as_float(r[8 * j + 2 * i]), __uint_as_float(r[8 * j + 2 * i + 1]));
+      if (MODE == EPI_SWIGLU || (MODE == EPI_INPROJ && silu)) {      // SiLU, the operations of silu_fast two at a time
+        const float2 t = __fmul2_rn(v, make_float2(-1.4426950408889634f, -1.4426950408889634f));
+        const float2 d = __fadd2_rn(make_float2(ex2_ftz(t.x), ex2_ftz(t.y)), make_float2(1.0f, 1.0f));
+        v = __fmul2_rn(v, make_float2(rcp_ftz(d.x), rcp_ftz(d.y)));
+      }
+      if (MODE == EPI_SWIGLU) v = __fmul2_rn(v, make_float2(__uint_as_float(up[8 * j + 2 * i]), __uint_as_float(up[8 * j + 2 * i + 1])));
+      if (MODE == EPI_OUTPROJ) v = __fmul2_rn(v, make_float2(scale, scale));
+      const __nv_bfloat162 h = __float22bfloat162_rn(v);
+      w[i] = *reinterpret_cast<const uint32_t*>(&h);
+    }
+    stage[lane * 8 + ((4 * cc + j) ^ (lane & 7))] = q;
+  }
+}
+// orow: output row of this lane's accumulator row, -1: not stored
+__device__ __forceinline__ void flush_rows64(const Epilogue& ep, const uint4* stage, int orow, int n0, int N, int lane) {
+  const int p = lane & 7, n = n0 + 8 * p;
+#pragma unroll
+  for (int r4 = 0; r4 < 8; ++r4) {
+    const int R = r4 * 4 + (lane >> 3), to = __shfl_sync(0xffffffffu, orow, R);
+    const uint4 q = stage[R * 8 + (p ^ (R & 7))];
+    if (to >= 0 && n < N) *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(ep.C) + (size_t)to * ep.ldc + n) = q;
   }
 }
 
@@ -193,7 +219,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   const uint32_t drain_bar = bars + 8u * (2 * STAGES + 2 * ACC_STAGES);      // abort path only: completion of the MMAs already issued
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + STAGES * SB + 8 * (2 * STAGES + 2 * ACC_STAGES + 1));
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
-  float* out_stage = reinterpret_cast<float*>(smem + STAGES * SB + 256);        // [8 warps][32][32] (softplus only)
+  float* out_stage = reinterpret_cast<float*>(smem + STAGES * SB + 256);        // [epilogue warps] staging of the rows that leave
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -455,28 +481,39 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       const int n_base = n_tile * block_n;
       uint32_t ra[32], rb[32];
       float4 bq[8];
-      if constexpr (MODE == EPI_SWIGLU) {
-        // accumulator columns [0,128) = gate, [128,256) = up; this warp takes 32-column groups half and half + 2
-        for (int c = half; c < 4; c += 2) {
-          tmem_ld32_issue(taddr + c * 32, ra);
-          tmem_ld32_issue(taddr + 128 + c * 32, rb);
-          tmem_ld_wait(ra);
-          tmem_ld_wait(rb);
-          if (row_ok) {
-            __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(ep.C) + out_row * ep.ldc + n_tile * 128 + c * 32;
-#pragma unroll
-            for (int j = 0; j < 32; j += 8) {
-              uint4 q;
-              uint32_t* w = reinterpret_cast<uint32_t*>(&q);
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                const float v0 = silu_fast(__uint_as_float(ra[j + 2 * i])) * __uint_as_float(rb[j + 2 * i]);
-                const float v1 = silu_fast(__uint_as_float(ra[j + 2 * i + 1])) * __uint_as_float(rb[j + 2 * i + 1]);
-                __nv_bfloat162 hh = __floats2bfloat162_rn(v0, v1);
-                w[i] = *reinterpret_cast<uint32_t*>(&hh);
-              }
-              *reinterpret_cast<uint4*>(dst + j) = q;
+      if constexpr (row_out(MODE)) {
+        uint4* stage = reinterpret_cast<uint4*>(out_stage + (warp - 2) * 1024);
+        const int orow = row_ok ? (int)out_row : -1;
+        if constexpr (MODE == EPI_SWIGLU) {
+          // accumulator columns [0,128) = gate, [128,256) = up; this warp takes the 32-column groups 2 half and 2 half + 1
+          for (int cc = 0; cc < 2; ++cc) {
+            tmem_ld32_issue(taddr + (2 * half + cc) * 32, ra);
+            tmem_ld32_issue(taddr + 128 + (2 * half + cc) * 32, rb);
+            tmem_ld_wait(ra);
+            tmem_ld_wait(rb);
+            stage_rows32<MODE>(stage, cc, ra, rb, true, 1.0f, lane);
+          }
+          __syncwarp();
+          flush_rows64(ep, stage, orow, n_tile * 128 + half * 64, N, lane);
+          __syncwarp();
+        } else {
+          // pairs of adjacent chunks 2 half, 2 half + 4; the next chunk's load is in flight while one is staged
+          int ch = 2 * half;
+          if (ch < n_chunks) tmem_ld32_issue(taddr + ch * 32, ra);
+          while (ch < n_chunks) {
+            const bool act = MODE == EPI_INPROJ && n_base + ch * 32 >= ep.R;      // (the boundary is a multiple of 64)
+            tmem_ld_wait(ra);
+            if (ch + 1 < n_chunks) tmem_ld32_issue(taddr + (ch + 1) * 32, rb);
+            stage_rows32<MODE>(stage, 0, ra, ra, act, scale, lane);
+            if (ch + 1 < n_chunks) {
+              tmem_ld_wait(rb);
+              if (ch + 4 < n_chunks) tmem_ld32_issue(taddr + (ch + 4) * 32, ra);
+              stage_rows32<MODE>(stage, 1, rb, rb, act, scale, lane);
             }
+            __syncwarp();
+            flush_rows64(ep, stage, orow, n_base + ch * 32, min(N, n_base + min(ch + 2, n_chunks) * 32), lane);
+            __syncwarp();
+            ch += 4;
           }
         }
       }
@@ -502,7 +539,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       Epilogue epl = ep;
       if (MODE == EPI_F32 && k_seg) epl.C = reinterpret_cast<float*>(ep.C) + (size_t)seg * M_max * ep.ldc;
       const bool zero_acc = MODE == EPI_F32 && nkb <= 0;
-      int ch = (MODE == EPI_SWIGLU || EWQ == 4) ? n_chunks : half;
+      int ch = (row_out(MODE) || EWQ == 4) ? n_chunks : half;
       if (ch < n_chunks) tmem_ld32_issue(taddr + ch * 32, ra);
       // two register buffers: while one chunk is processed the next chunk's tensor-memory load is in flight
       while (ch < n_chunks) {
@@ -514,7 +551,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
           for (int i = 0; i < 32; ++i) ra[i] = 0u;
         }
         if (f32_out(MODE)) epi_softplus32<MODE>(epl, out_stage + (warp - 2) * 1024, m_tile * BLOCK_M + quarter * 32, own ? M_valid : 0, n_base + ch * 32, N, ra, bq, lane);
-        else if (row_ok) epi_store32<MODE>(ep, out_row, tok_row, n_base + ch * 32, N, ra, scale, bq);
+        else if (row_ok) epi_xproj32(ep, out_row, tok_row, n_base + ch * 32, N, ra);
         ch += EWQ;
         if (ch >= n_chunks) break;
         load_bias<MODE>(ep, n_base + ch * 32, N, bq);
@@ -525,7 +562,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
           for (int i = 0; i < 32; ++i) rb[i] = 0u;
         }
         if (f32_out(MODE)) epi_softplus32<MODE>(epl, out_stage + (warp - 2) * 1024, m_tile * BLOCK_M + quarter * 32, own ? M_valid : 0, n_base + ch * 32, N, rb, bq, lane);
-        else if (row_ok) epi_store32<MODE>(ep, out_row, tok_row, n_base + ch * 32, N, rb, scale, bq);
+        else if (row_ok) epi_xproj32(ep, out_row, tok_row, n_base + ch * 32, N, rb);
         ch += EWQ;
       }
       tc_fence_before();
