@@ -232,6 +232,10 @@ cudaError_t launch_gemm_tc(const void* A, int lda, const void* Bw, int ldb, int 
                            const Epilogue& epi, int32_t* status, cudaStream_t st, bool test_stall = false, bool b_mn = false,
                            const int32_t* pad_offsets = nullptr /* grouped: the padded segment offsets (n_experts + 1); allows CTA pairs */);
 
+// x Proj of few tokens, the contracted index shared by a cluster (rom_x_proj.cu): C = A[M, Kd] Bw[N, Kd]^T split into delta | B | C; bf16.
+bool x_proj_applicable(int M, int N, int Kd);
+cudaError_t launch_x_proj(const void* A, const void* Bw, int M, int N, int Kd, const Epilogue& epi, int32_t* status, cudaStream_t st);
+
 // dt Proj with a short contraction (rom_dt_proj.cu): C[M, N] = softplus(A[M, Kd] Bw[N, Kd]^T + bias), rows contiguous; bf16.  Its kernel lets
 // the next one in only as its blocks end (a scan's blocks must not pile up).
 bool dt_proj_applicable(int N, int Kd);
