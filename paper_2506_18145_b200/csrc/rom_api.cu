@@ -324,7 +324,6 @@ int layer_forward_impl(const rom_config* cfg, const rom_weights* w, const void* 
     if (ev) ROM_CUDA(cudaEventRecord(ev[++stage], st));        \
   } while (0)
   if (ev) ROM_CUDA(cudaEventRecord(ev[0], st));
-  ROM_CUDA(launch_init_status(status, st));
   const bool debug_checks = (c.flags & ROM_FLAG_DEBUG_CHECKS) != 0;
   if (debug_checks) ROM_CUDA(launch_canaries(W, lay, false, st));
   // S1 + S2: router, top-K, permutation tables
@@ -574,7 +573,7 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
 
   // ---- forward, recomputed with the raw Gate Proj rows kept (the forward proper stores them activated at top-1)
   float* probs = reinterpret_cast<float*>(W + bl.probs);
-  ROM_CUDA(launch_route_gather(c, x, w->W_r, w->b_r, nullptr, gates, nullptr, W, lay, st, probs));
+  ROM_CUDA(launch_route_gather(c, x, w->W_r, w->b_r, nullptr, gates, nullptr, W, lay, st, probs, true));
   if (tc && c.K == 1) {
     // one expert per token: the output op writes every row at its token's position (no activation: R = width)
     Epilogue e_in{EPI_INPROJ, W + bl.HZs, 2 * De, nullptr, nullptr, nullptr, 2 * De, 0, reinterpret_cast<const int32_t*>(W + lay.assign_of_row), nullptr};

@@ -186,10 +186,10 @@ cudaError_t launch_route_stats(const rom_config& c, const void* x, const void* W
                                int32_t* topk_idx, float* gates, int32_t* counts, int32_t* offsets,
                                int32_t* perm, int32_t* inv_perm, char* ws, const WsLayout& lay, double* chunk_prob, cudaStream_t st,
                                bool gather_x, float* probs = nullptr /* [T, E] Softmax(X W_r) */);
-// Router + tables + x_perm in two launches (the layer's path).
+// Router + tables + x_perm in two launches (the layer's path), the status block zeroed first (status_zeroed: the caller has).
 cudaError_t launch_route_gather(const rom_config& c, const void* x, const void* W_r, const float* b_r,
                                 int32_t* topk_idx, float* gates, int32_t* counts, char* ws, const WsLayout& lay, cudaStream_t st,
-                                float* probs = nullptr);
+                                float* probs = nullptr, bool status_zeroed = false);
 // Router + load-balance statistic: F[E], Pbar[E], loss[1] (device fp32, each may be null).
 cudaError_t launch_balance(const rom_config& c, const void* x, const void* W_r, const float* b_r, float alpha,
                            float* F, float* Pbar, float* loss, char* ws, const WsLayout& lay, cudaStream_t st);

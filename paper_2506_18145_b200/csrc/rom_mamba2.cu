@@ -421,7 +421,6 @@ int rom_mamba2_layer_forward(const rom_config* cfg, int32_t headdim, const rom_m
     return launch_gemm_simt(c.dtype, A_, lda, B_, ldb, bstride, rows, Nn, Kd, tile_expert, num_m_tiles, ep, st);
   };
 
-  ROM_CUDA(launch_init_status(status, st));
   ROM_CUDA(launch_route_gather(c, x, w->W_r, w->b_r, topk_idx_out, gates, counts_out, W, lay, st));
   // fused input projection of the selected experts, then the sum over a token's slots (indicator only)
   if (tc && c.K == 1) {

@@ -5,12 +5,13 @@
 //   route_logits_topk : logits in fp64 on the tensor cores (products of bf16 or fp32 inputs are exact in
 //                       fp64; every expert's sum is taken in the same order, so ties stay ties), softmax,
 //                       top-K with ties to the lowest expert id, per-chunk histogram; clears the
-//                       row -> assignment table; the block that finishes last (an atomic ticket, no
-//                       waiting) turns the chunk histograms into expert offsets, offsets padded to the
-//                       GEMM row tile and the row-tile -> expert map.
+//                       row -> assignment table; with many chunks the block that finishes last (an
+//                       atomic ticket, no waiting) turns the chunk histograms into expert offsets,
+//                       offsets padded to the GEMM row tile and the row-tile -> expert map.
 //   route_scatter     : stable rank of every assignment inside its chunk by warp ballots; writes
 //                       perm / inv_perm and the padded-row tables and, when asked, copies each token's
-//                       row to its padded row (x_perm, zero rows in the padding) while x is still in L2.
+//                       row to its padded row (x_perm, zero rows in the padding) while x is still in L2;
+//                       with few chunks every block adds up the histograms itself.
 //   route_offsets, idx_chunk_histogram, gather_rows : the same steps as separate kernels, for tables
 //                       built from a routing decision made elsewhere and for other row gathers.
 #include "rom_internal.cuh"
@@ -43,12 +44,79 @@ template <> struct RawX4<float> {
   __device__ __forceinline__ void get(double (&xd)[4]) const { xd[0] = v.x; xd[1] = v.y; xd[2] = v.z; xd[3] = v.w; }
 };
 
+struct OffsetsArgs {
+  int32_t* counts_ws; int32_t* offsets_ws; int32_t* pad_offsets; int32_t* num_m_tiles; int32_t* tile_expert; int max_m_tiles;
+  int32_t* counts_out; int32_t* offsets_out;
+  int32_t* assign_of_row; int rows_max;      // cleared to -1 by the grid
+  int32_t* ticket;                           // zero on entry; left zero on exit (null: the offsets are formed later)
+  int32_t* status;                           // by_expert: the status block, zeroed here
+  bool by_expert;                            // histograms as [E, n_chunks] instead of [n_chunks, E]
+};
+
+// offsets and the row-tile -> expert map from the shared copies, by one block
+__device__ void write_offsets(int E, const OffsetsArgs& o, const int32_t* cnt, const int32_t* off, const int32_t* poff) {
+  for (int e = threadIdx.x; e <= E; e += blockDim.x) {
+    o.offsets_ws[e] = off[e];
+    o.pad_offsets[e] = poff[e];
+    if (o.offsets_out) o.offsets_out[e] = off[e];
+    if (e < E) {
+      o.counts_ws[e] = cnt[e];
+      if (o.counts_out) o.counts_out[e] = cnt[e];
+    }
+  }
+  const int ntiles = poff[E] / kTileM;
+  if (threadIdx.x == 0) *o.num_m_tiles = ntiles;
+  for (int i = threadIdx.x; i < o.max_m_tiles; i += blockDim.x) {
+    int ex = -1;
+    if (i < ntiles) {
+      const int row = i * kTileM;
+      for (int e = 0; e < E; ++e)
+        if (row >= poff[e] && row < poff[e + 1]) ex = e;
+    }
+    o.tile_expert[i] = ex;
+  }
+}
+
+// From the histograms by expert ([E, n_chunks]), by every block for itself: assignments of each expert in all chunks (cnt) and in those
+// before this one (base), offsets and offsets padded to the row tile.
+__device__ __forceinline__ void bases_from_histograms(const int32_t* __restrict__ counts, int n_chunks, int E, int chunk,
+                                                      int32_t* base, int32_t* cnt, int32_t* off, int32_t* poff) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+  for (int e = warp; e < E; e += nwarps) {
+    int all = 0, before = 0;
+#pragma unroll 8
+    for (int c = lane; c < n_chunks; c += 32) {
+      const int v = __ldg(counts + (size_t)e * n_chunks + c);
+      all += v;
+      if (c < chunk) before += v;
+    }
+    all = __reduce_add_sync(0xffffffffu, all);
+    before = __reduce_add_sync(0xffffffffu, before);
+    if (lane == 0) { cnt[e] = all; base[e] = before; }
+  }
+  __syncthreads();
+  if (warp == 0) {
+    int o0 = 0, p0 = 0;
+    for (int e0 = 0; e0 < E; e0 += 32) {
+      const int e = e0 + lane, c = e < E ? cnt[e] : 0, pc = (c + kTileM - 1) / kTileM * kTileM;
+      int o = c, p = pc;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int on = __shfl_up_sync(0xffffffffu, o, d), pn = __shfl_up_sync(0xffffffffu, p, d);
+        if (lane >= d) { o += on; p += pn; }
+      }
+      if (e < E) { off[e] = o0 + o - c; poff[e] = p0 + p - pc; }
+      o0 += __shfl_sync(0xffffffffu, o, 31);
+      p0 += __shfl_sync(0xffffffffu, p, 31);
+    }
+    if (lane == 0) { off[E] = o0; poff[E] = p0; }
+  }
+  __syncthreads();
+}
+
 // Run by one block: warp w scans the chunk histogram of experts w, w + nwarps, ... over all chunks (exclusive bases
 // written back in place), then expert offsets, offsets padded to the row tile, tile count and row-tile -> expert map.
-__device__ void offsets_from_histograms(int32_t* __restrict__ chunk_counts, int n_chunks, int E,
-                                        int32_t* __restrict__ counts_ws, int32_t* __restrict__ offsets_ws, int32_t* __restrict__ pad_offsets,
-                                        int32_t* __restrict__ num_m_tiles, int32_t* __restrict__ tile_expert, int max_m_tiles,
-                                        int32_t* __restrict__ counts_out, int32_t* __restrict__ offsets_out,
+__device__ void offsets_from_histograms(int32_t* __restrict__ chunk_counts, int n_chunks, int E, const OffsetsArgs& o,
                                         int32_t* cnt, int32_t* off, int32_t* poff /* shared: kMaxE, kMaxE+1, kMaxE+1 */) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
   for (int e = warp; e < E; e += nwarps) {
@@ -79,43 +147,17 @@ __device__ void offsets_from_histograms(int32_t* __restrict__ chunk_counts, int 
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    int o = 0, p = 0;
+    int n = 0, p = 0;
     for (int e = 0; e < E; ++e) {
-      off[e] = o; poff[e] = p;
-      o += cnt[e];
+      off[e] = n; poff[e] = p;
+      n += cnt[e];
       p += (cnt[e] + kTileM - 1) / kTileM * kTileM;
     }
-    off[E] = o; poff[E] = p;
-    *num_m_tiles = p / kTileM;
+    off[E] = n; poff[E] = p;
   }
   __syncthreads();
-  for (int e = threadIdx.x; e <= E; e += blockDim.x) {
-    offsets_ws[e] = off[e];
-    pad_offsets[e] = poff[e];
-    if (offsets_out) offsets_out[e] = off[e];
-    if (e < E) {
-      counts_ws[e] = cnt[e];
-      if (counts_out) counts_out[e] = cnt[e];
-    }
-  }
-  const int ntiles = poff[E] / kTileM;
-  for (int i = threadIdx.x; i < max_m_tiles; i += blockDim.x) {
-    int ex = -1;
-    if (i < ntiles) {
-      const int row = i * kTileM;
-      for (int e = 0; e < E; ++e)
-        if (row >= poff[e] && row < poff[e + 1]) ex = e;
-    }
-    tile_expert[i] = ex;
-  }
+  write_offsets(E, o, cnt, off, poff);
 }
-
-struct OffsetsArgs {
-  int32_t* counts_ws; int32_t* offsets_ws; int32_t* pad_offsets; int32_t* num_m_tiles; int32_t* tile_expert; int max_m_tiles;
-  int32_t* counts_out; int32_t* offsets_out;
-  int32_t* assign_of_row; int rows_max;      // cleared to -1 by the grid
-  int32_t* ticket;                           // zero on entry; left zero on exit
-};
 
 __global__ void __launch_bounds__(1024)
 route_offsets(int32_t* __restrict__ chunk_counts, int n_chunks, int E, const OffsetsArgs o) {
@@ -123,8 +165,7 @@ route_offsets(int32_t* __restrict__ chunk_counts, int n_chunks, int E, const Off
   __shared__ int32_t cnt[kMaxE];
   __shared__ int32_t off[kMaxE + 1];
   __shared__ int32_t poff[kMaxE + 1];
-  offsets_from_histograms(chunk_counts, n_chunks, E, o.counts_ws, o.offsets_ws, o.pad_offsets, o.num_m_tiles, o.tile_expert,
-                          o.max_m_tiles, o.counts_out, o.offsets_out, cnt, off, poff);
+  offsets_from_histograms(chunk_counts, n_chunks, E, o, cnt, off, poff);
 }
 
 // One block = 32 tokens (one routing chunk); warp w computes the logits of experts [8w, 8w+8) for them with
@@ -172,6 +213,7 @@ route_logits_topk(const T* __restrict__ x, const T* __restrict__ W_r, const floa
   const bool w_ok = w * NT8 + gq < E;
   const T* wrow = W_r + (size_t)min(w * NT8 + gq, E - 1) * Dm + 4 * t4;
 
+  if (oa.by_expert && blockIdx.x == 0 && tid < kStatusInts) oa.status[tid] = 0;
   // the row -> assignment table starts at -1 everywhere (padding rows keep it); the whole grid clears it
   for (int i = blockIdx.x * blockDim.x + tid; i < oa.rows_max; i += gridDim.x * blockDim.x) oa.assign_of_row[i] = -1;
 
@@ -283,7 +325,7 @@ route_logits_topk(const T* __restrict__ x, const T* __restrict__ W_r, const floa
     for (int e = 0; e < E; ++e) {
       int c = 0;
       for (int k = 0; k < K; ++k) c += __popc(__ballot_sync(0xffffffffu, idx_s[tid * K + k] == e));
-      if (tid == 0) chunk_counts[(size_t)blockIdx.x * E + e] = c;
+      if (tid == 0) chunk_counts[oa.by_expert ? (size_t)e * n_chunks + blockIdx.x : (size_t)blockIdx.x * E + e] = c;
     }
   }
 
@@ -299,14 +341,13 @@ route_logits_topk(const T* __restrict__ x, const T* __restrict__ W_r, const floa
   __threadfence();
   if (tid == 0) *oa.ticket = 0;                  // ready for the next call on this workspace
   int32_t* cnt = idx_s;                          // the top-K scratch is free now: kMaxE + 2 (kMaxE + 1) ints (sized by the launcher)
-  offsets_from_histograms(chunk_counts, n_chunks, E, oa.counts_ws, oa.offsets_ws, oa.pad_offsets, oa.num_m_tiles, oa.tile_expert,
-                          oa.max_m_tiles, oa.counts_out, oa.offsets_out, cnt, cnt + kMaxE, cnt + 2 * kMaxE + 1);
+  offsets_from_histograms(chunk_counts, n_chunks, E, oa, cnt, cnt + kMaxE, cnt + 2 * kMaxE + 1);
 }
 
 // Stable rank of the chunk's assignments by warp ballots, then the table entries; called by one full warp.
-// my_row[k] receives the padded row of (token, slot k), -1 past the end.
-__device__ __forceinline__ void scatter_chunk(const int32_t* __restrict__ topk_idx, const int32_t* __restrict__ chunk_base,
-                                              const int32_t* __restrict__ offsets, const int32_t* __restrict__ pad_offsets,
+// my_row[k] receives the padded row of (token, slot k), -1 past the end.  chunk_base: assignments of every expert before this chunk.
+__device__ __forceinline__ void scatter_chunk(const int32_t* __restrict__ topk_idx, const int32_t* chunk_base,
+                                              const int32_t* offsets, const int32_t* pad_offsets,
                                               int T_tokens, int E, int K, int chunk, int lane,
                                               int32_t* __restrict__ perm, int32_t* __restrict__ inv_perm,
                                               int32_t* __restrict__ row_of_assign, int32_t* __restrict__ assign_of_row,
@@ -329,7 +370,7 @@ __device__ __forceinline__ void scatter_chunk(const int32_t* __restrict__ topk_i
   for (int k = 0; k < K; ++k) {
     const int e = my_e[k];
     const int a = t * K + k;
-    const int within = chunk_base[(size_t)chunk * E + e] + my_rank[k];
+    const int within = chunk_base[e] + my_rank[k];
     const int r = offsets[e] + within;
     const int pr = pad_offsets[e] + within;
     if (perm) perm[r] = a;
@@ -352,40 +393,51 @@ route_scatter(const int32_t* __restrict__ topk_idx, const int32_t* __restrict__ 
   const int chunk = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (chunk >= n_chunks) return;
   int my_row[kMaxK];
-  scatter_chunk(topk_idx, chunk_base, offsets, pad_offsets, T_tokens, E, K, chunk, lane, perm, inv_perm, row_of_assign, assign_of_row, my_row);
+  scatter_chunk(topk_idx, chunk_base + (size_t)chunk * E, offsets, pad_offsets, T_tokens, E, K, chunk, lane, perm, inv_perm, row_of_assign, assign_of_row, my_row);
 }
 
 // One block of 8 warps per chunk of 32 tokens: warp 0 builds the chunk's table entries, then every warp copies the rows
 // of four of the chunk's tokens to their padded rows (x_perm, the operand of the grouped Conv/Gate projection; x was read
 // by the router a moment ago and is still in L2), and the grid zero-fills the padding rows of every expert segment.
+// OWN: every block adds up the histograms (by expert) itself and the last one writes the offsets out for the kernels to come: no ticket,
+// no tail of one block between the two routing launches, and no launch before them to zero it.
+template <bool OWN>
 __global__ void __launch_bounds__(256)
-route_scatter_gather(const int32_t* __restrict__ topk_idx, const int32_t* __restrict__ chunk_base,
-                     const int32_t* __restrict__ offsets, const int32_t* __restrict__ pad_offsets,
-                     int T_tokens, int E, int K, int n_chunks,
-                     int32_t* __restrict__ perm, int32_t* __restrict__ inv_perm,
-                     int32_t* __restrict__ row_of_assign, int32_t* __restrict__ assign_of_row,
-                     const uint4* __restrict__ x, uint4* __restrict__ x_perm, int vec_per_row) {
+route_scatter_gather(const int32_t* __restrict__ topk_idx, const int32_t* __restrict__ chunk_counts,
+                     const OffsetsArgs o, int T_tokens, int E, int K, int n_chunks,
+                     int32_t* __restrict__ row_of_assign, const uint4* __restrict__ x, uint4* __restrict__ x_perm, int vec_per_row) {
   pdl_sync();
   __shared__ int32_t rows_s[kChunkTokens * kMaxK];
+  __shared__ int32_t base_s[OWN ? kMaxE : 1], cnt_s[OWN ? kMaxE : 1], off_s[OWN ? kMaxE + 1 : 1], poff_s[OWN ? kMaxE + 1 : 1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int chunk = blockIdx.x;
+  const int n_tok = chunk < n_chunks ? min(kChunkTokens, T_tokens - chunk * kChunkTokens) : 0;
+  uint4 buf[8];
+  auto fetch = [&](int j, int v0) {
+    const uint4* src = x + (size_t)(chunk * kChunkTokens + j) * vec_per_row;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int v = v0 + 32 * i + lane;
+      if (v < vec_per_row) buf[i] = __ldg(src + v);
+    }
+  };
+  if (warp < n_tok) fetch(warp, 0);      // (the first row does not depend on the tables)
+  const int32_t *chunk_base = chunk_counts + (size_t)chunk * E, *offsets = o.offsets_ws, *pad_offsets = o.pad_offsets;
+  if constexpr (OWN) {
+    bases_from_histograms(chunk_counts, n_chunks, E, chunk, base_s, cnt_s, off_s, poff_s);
+    chunk_base = base_s; offsets = off_s; pad_offsets = poff_s;
+    if (blockIdx.x == gridDim.x - 1) write_offsets(E, o, cnt_s, off_s, poff_s);
+  }
   // blocks beyond the last chunk (the grid never drops below one block per SM) only help with the padding rows
   if (chunk < n_chunks && warp == 0) {
     int my_row[kMaxK];
-    scatter_chunk(topk_idx, chunk_base, offsets, pad_offsets, T_tokens, E, K, chunk, lane, perm, inv_perm, row_of_assign, assign_of_row, my_row);
+    scatter_chunk(topk_idx, chunk_base, offsets, pad_offsets, T_tokens, E, K, chunk, lane, nullptr, nullptr, row_of_assign, o.assign_of_row, my_row);
     for (int k = 0; k < K; ++k) rows_s[lane * K + k] = my_row[k];
   }
   __syncthreads();
-  const int n_tok = chunk < n_chunks ? min(kChunkTokens, T_tokens - chunk * kChunkTokens) : 0;
   for (int j = warp; j < n_tok; j += 8) {
-    const uint4* src = x + (size_t)(chunk * kChunkTokens + j) * vec_per_row;
     for (int v0 = 0; v0 < vec_per_row; v0 += 32 * 8) {
-      uint4 buf[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int v = v0 + 32 * i + lane;
-        if (v < vec_per_row) buf[i] = __ldg(src + v);
-      }
+      if (j != warp || v0) fetch(j, v0);
       for (int k = 0; k < K; ++k) {
         uint4* dst = x_perm + (size_t)rows_s[j * K + k] * vec_per_row;
 #pragma unroll
@@ -475,6 +527,12 @@ init_tables(int32_t* __restrict__ status, int32_t* __restrict__ table, int n) {
 
 }  // namespace
 
+// Blocks of the scatter add up the histograms themselves (OWN) up to one chunk per SM.  us of a call, ticket / own: 256 tokens in fp32
+// 59.0 / 56.1, 700 tokens 128.1 / 122.1, 3051 tokens 314.2 / 312.6, backward of 4113 tokens 784.7 / 780.1.  Beyond, the logits kernel must
+// not be let in early behind the call before (8192 tokens: its blocks pile up on the first SMs to drain, 318.0 / 326.3), and without that
+// it is even (318.2 / 317.7; 24576 tokens 760 / 758; 32768 tokens 3794 / 3919).
+static bool route_own_bases(const WsLayout& lay) { return lay.n_chunks <= 148; }
+
 cudaError_t launch_init_status(int32_t* status, cudaStream_t st) {
   launch_k(init_tables, 1, 256, 0, st, status, nullptr, 0);
   count_launch();
@@ -496,7 +554,11 @@ cudaError_t launch_route(const rom_config& c, const void* x, const void* W_r, co
 
 cudaError_t launch_route_gather(const rom_config& c, const void* x, const void* W_r, const float* b_r,
                                 int32_t* topk_idx, float* gates, int32_t* counts, char* ws, const WsLayout& lay, cudaStream_t st,
-                                float* probs) {
+                                float* probs, bool status_zeroed) {
+  if (!status_zeroed && !route_own_bases(lay)) {
+    const cudaError_t e = launch_init_status(reinterpret_cast<int32_t*>(ws + lay.status), st);
+    if (e != cudaSuccess) return e;
+  }
   return launch_route_stats(c, x, W_r, b_r, topk_idx, gates, counts, nullptr, nullptr, nullptr, ws, lay, nullptr, st, true, probs);
 }
 
@@ -538,7 +600,7 @@ cudaError_t launch_balance(const rom_config& c, const void* x, const void* W_r, 
 static cudaError_t launch_perm_tables(const rom_config& c, const int32_t* idx_ws, int32_t* counts, int32_t* offsets, int32_t* perm,
                                       int32_t* inv_perm, char* ws, const WsLayout& lay, cudaStream_t st);
 static cudaError_t launch_scatter(const rom_config& c, const int32_t* idx_ws, int32_t* perm, int32_t* inv_perm, char* ws,
-                                  const WsLayout& lay, const void* x, cudaStream_t st);
+                                  const WsLayout& lay, const void* x, const OffsetsArgs& oa, cudaStream_t st);
 
 cudaError_t launch_route_stats(const rom_config& c, const void* x, const void* W_r, const float* b_r,
                                int32_t* topk_idx, float* gates, int32_t* counts, int32_t* offsets,
@@ -558,10 +620,12 @@ cudaError_t launch_route_stats(const rom_config& c, const void* x, const void* W
   while (dsplit > 1 && (n_wtiles * dsplit > 16 || c.d_model / 16 < 4 * dsplit)) dsplit >>= 1;
   const int threads = 32 * n_wtiles * dsplit;
   const bool bf = c.dtype == ROM_BF16;
+  int32_t* status = reinterpret_cast<int32_t*>(ws + lay.status);
+  const bool own = gather_x && route_own_bases(lay);
   const OffsetsArgs oa{reinterpret_cast<int32_t*>(ws + lay.counts), reinterpret_cast<int32_t*>(ws + lay.offsets),
                        reinterpret_cast<int32_t*>(ws + lay.pad_offsets), reinterpret_cast<int32_t*>(ws + lay.num_m_tiles),
                        reinterpret_cast<int32_t*>(ws + lay.tile_expert), (int)lay.max_m_tiles, counts, offsets,
-                       assign_of_row, (int)lay.rows_max, reinterpret_cast<int32_t*>(ws + lay.status) + kStatTicket};
+                       assign_of_row, (int)lay.rows_max, own ? nullptr : status + kStatTicket, status, own};
   const int idx_ints = RT * c.K > 3 * kMaxE + 2 ? RT * c.K : 3 * kMaxE + 2;
   const size_t smem = sizeof(double) * (size_t)(dsplit > 2 ? dsplit : 2) * RT * Epad8 + sizeof(int32_t) * idx_ints;
   if (bf)
@@ -575,12 +639,12 @@ cudaError_t launch_route_stats(const rom_config& c, const void* x, const void* W
   count_launch();
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) return err;
-  return launch_scatter(c, idx_ws, perm, inv_perm, ws, lay, gather_x ? x : nullptr, st);
+  return launch_scatter(c, idx_ws, perm, inv_perm, ws, lay, gather_x ? x : nullptr, oa, st);
 }
 
 // the permutation (and, with x, the gathered rows) from the indices, the per-chunk bases and the offsets
 static cudaError_t launch_scatter(const rom_config& c, const int32_t* idx_ws, int32_t* perm, int32_t* inv_perm, char* ws,
-                                  const WsLayout& lay, const void* x, cudaStream_t st) {
+                                  const WsLayout& lay, const void* x, const OffsetsArgs& oa, cudaStream_t st) {
   const int32_t* chunk_base = reinterpret_cast<int32_t*>(ws + lay.chunk_counts);
   const int32_t* offs = reinterpret_cast<int32_t*>(ws + lay.offsets);
   const int32_t* poffs = reinterpret_cast<int32_t*>(ws + lay.pad_offsets);
@@ -591,9 +655,8 @@ static cudaError_t launch_scatter(const rom_config& c, const int32_t* idx_ws, in
     const cudaError_t e = current_device_sm_count(&num_sms);
     if (e != cudaSuccess) return e;
     const int grid = (int)lay.n_chunks > num_sms ? (int)lay.n_chunks : num_sms;
-    launch_k(route_scatter_gather, grid, 256, 0, st, idx_ws, chunk_base, offs, poffs, (int)lay.T, c.E, c.K, (int)lay.n_chunks, perm, inv_perm, roa, aor,
-                                                           reinterpret_cast<const uint4*>(x), reinterpret_cast<uint4*>(ws + lay.x_perm),
-                                                           (int)((size_t)c.d_model * lay.esz / 16));
+    launch_k(oa.by_expert ? route_scatter_gather<true> : route_scatter_gather<false>, grid, 256, 0, st, idx_ws, chunk_base, oa, (int)lay.T, c.E, c.K,
+             (int)lay.n_chunks, roa, reinterpret_cast<const uint4*>(x), reinterpret_cast<uint4*>(ws + lay.x_perm), (int)((size_t)c.d_model * lay.esz / 16));
   } else {
     const int wpb = 8;
     launch_k(route_scatter, ((int)lay.n_chunks + wpb - 1) / wpb, wpb * 32, 0, st, idx_ws, chunk_base, offs, poffs, (int)lay.T, c.E, c.K,
@@ -608,10 +671,11 @@ static cudaError_t launch_perm_tables(const rom_config& c, const int32_t* idx_ws
                                       int32_t* inv_perm, char* ws, const WsLayout& lay, cudaStream_t st) {
   const OffsetsArgs oa{reinterpret_cast<int32_t*>(ws + lay.counts), reinterpret_cast<int32_t*>(ws + lay.offsets),
                        reinterpret_cast<int32_t*>(ws + lay.pad_offsets), reinterpret_cast<int32_t*>(ws + lay.num_m_tiles),
-                       reinterpret_cast<int32_t*>(ws + lay.tile_expert), (int)lay.max_m_tiles, counts, offsets, nullptr, 0, nullptr};
+                       reinterpret_cast<int32_t*>(ws + lay.tile_expert), (int)lay.max_m_tiles, counts, offsets,
+                       reinterpret_cast<int32_t*>(ws + lay.assign_of_row), 0, nullptr, nullptr, false};
   launch_k(route_offsets, 1, 1024, 0, st, reinterpret_cast<int32_t*>(ws + lay.chunk_counts), (int)lay.n_chunks, c.E, oa);
   count_launch();
-  return launch_scatter(c, idx_ws, perm, inv_perm, ws, lay, nullptr, st);
+  return launch_scatter(c, idx_ws, perm, inv_perm, ws, lay, nullptr, oa, st);
 }
 
 cudaError_t launch_gather_rows(const rom_config& c, const void* x, char* ws, const WsLayout& lay, cudaStream_t st) {
