@@ -56,7 +56,8 @@ struct BwdArgs {
   const int32_t* dz_rows; int K;  // rows of dz that take token t: dz_rows[t K + k]; nullptr: row t
   int Lc, ncc;                    // coarse chunks (blockIdx.z): chunk j covers steps [j Lc, (j+1) Lc); Lc is a multiple of 16
   float* g_in;                    // [B, ncc, De, 16] state gradient at the end of every coarse chunk (ncc > 1)
-  float* q_start; float* sum_delta;         // pre-pass outputs: [B, ncc, De, 16] and [B, ncc, De]
+  int Lp, mp;                     // pre-pass: every coarse chunk in mp pieces of Lp steps (the last ones shorter or empty)
+  float* q_start; float* sum_delta;         // pre-pass outputs: [B, ncc, mp, De, 16] and [B, ncc, mp, De]
 };
 
 template <bool PRECISE> __device__ __forceinline__ float sigmoid_f(float v) {
@@ -343,8 +344,8 @@ scan_bwd_kernel(const BwdArgs p) {
   }
 }
 
-// Pre-pass of the chunk-parallel form, one coarse chunk per blockIdx.z: from a zero gradient, the gradient that leaves the
-// chunk's start (g <- a_t (g + C_t e_t), t descending) and the sum of Delta over the chunk.  A lane owns all 16 states of one
+// Pre-pass of the chunk-parallel form, one piece of a coarse chunk per blockIdx.z: from a zero gradient, the gradient that leaves the
+// piece's start (g <- a_t (g + C_t e_t), t descending) and the sum of Delta over it.  A lane owns all 16 states of one
 // channel, a warp 32 channels; eight steps are staged at a time, the next eight in flight.  Bound by the special-function unit
 // (one exponential per state and step against three fp32 operations).
 struct PreSmem { float2 de[CK][32]; float4 c[CK][4]; };
@@ -360,8 +361,8 @@ scan_bwd_prepass_kernel(const BwdArgs p) {
   const int c_warp = blockIdx.x * BCH + warp * WCH;
   if (c_warp >= De) return;
   const size_t b = blockIdx.y;
-  const int cj = blockIdx.z + 1;                  // chunk 0's start gradient is nobody's input
-  const int t_lo = cj * p.Lc, t_hi = min(t_lo + p.Lc, p.L);
+  const int cj = blockIdx.z / p.mp + 1, piece = blockIdx.z % p.mp;      // chunk 0's start gradient is nobody's input
+  const int c_hi = min((cj + 1) * p.Lc, p.L), t_lo = min(cj * p.Lc + piece * p.Lp, c_hi), t_hi = min(t_lo + p.Lp, c_hi);
   const int c = c_warp + lane;
   const int lt = lane & 7, l8 = lane >> 3, lc = c_warp + 8 * l8;
   float2 a2[8], g[8];
@@ -388,7 +389,7 @@ scan_bwd_prepass_kernel(const BwdArgs p) {
     }
     r_c = t0 + (lane >> 2) < t_hi ? __ldg(reinterpret_cast<const float4*>(p.Cm + (b * p.L + t0) * NST) + lane) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   };
-  int t0 = t_lo + (t_hi - t_lo - 1) / CK * CK;
+  int t0 = t_lo + (t_hi - t_lo - 1) / CK * CK;      // (an empty piece: t_lo, every step past the end)
   fetch(t0);
   for (; t0 >= t_lo; t0 -= CK) {
     {
@@ -422,18 +423,18 @@ scan_bwd_prepass_kernel(const BwdArgs p) {
     }
     __syncwarp();
   }
-  const size_t o = (b * p.ncc + cj) * De + c;
+  const size_t o = ((b * p.ncc + cj) * p.mp + piece) * De + c;
 #pragma unroll
   for (int i = 0; i < 4; ++i)
     *reinterpret_cast<float4*>(p.q_start + o * NST + 4 * i) = make_float4(g[2 * i].x, g[2 * i].y, g[2 * i + 1].x, g[2 * i + 1].y);
   p.sum_delta[o] = sd;
 }
 
-// Composes the gradient over the coarse chunks (the recurrence is linear): with P_j = exp(A sum_delta_j),
-//   g_in[ncc-1] = dh_last,  g_in[j-1] = P_j g_in[j] + q_start[j].
+// Composes the gradient over the pieces of the coarse chunks (the recurrence is linear): with P_s = exp(A sum_delta_s), from dh_last,
+//   g <- P_s g + q_start[s]  for s = ncc mp - 1 down to mp;  what stands before a coarse chunk's last piece is its g_in.
 __global__ void __launch_bounds__(256)
 scan_bwd_chain_kernel(const float* __restrict__ A, const float* __restrict__ dh_last, const float* __restrict__ q_start,
-                      const float* __restrict__ sum_delta, float* __restrict__ g_in, int B, int De, int ncc) {
+                      const float* __restrict__ sum_delta, float* __restrict__ g_in, int B, int De, int ncc, int mp) {
   pdl_sync();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (long long)B * De * NST) return;
@@ -442,11 +443,24 @@ scan_bwd_chain_kernel(const float* __restrict__ A, const float* __restrict__ dh_
   const size_t b = (size_t)(i / ((long long)NST * De));
   const float a = A[(size_t)c * NST + n];
   float g = dh_last ? dh_last[i] : 0.0f;
-  for (int j = ncc - 1; j >= 0; --j) {
-    const size_t sq = b * ncc + j;
-    g_in[(sq * De + c) * NST + n] = g;
-    if (j > 0) g = fmaf(expf(a * sum_delta[sq * De + c]), g, q_start[(sq * De + c) * NST + n]);
+  constexpr int G = 8;             // pieces whose loads are in flight together
+  for (int s0 = ncc * mp - 1; s0 >= mp; s0 -= G) {
+    float qv[G], sv[G];
+#pragma unroll
+    for (int k = 0; k < G; ++k) {
+      const size_t sq = b * ncc * mp + max(s0 - k, mp);
+      sv[k] = __ldg(sum_delta + sq * De + c);
+      qv[k] = __ldg(q_start + (sq * De + c) * NST + n);
+    }
+#pragma unroll
+    for (int k = 0; k < G; ++k) {
+      const int s = s0 - k;
+      if (s < mp) break;
+      if ((s + 1) % mp == 0) g_in[((b * ncc + s / mp) * De + c) * NST + n] = g;
+      g = fmaf(expf(a * sv[k]), g, qv[k]);
+    }
   }
+  g_in[(b * ncc * De + c) * NST + n] = g;
 }
 // The same for the states (rom_scan_backward, where no forward scan has left checkpoints): h_in[0] = h0, h_in[j+1] = P_j h_in[j] + h_end[j].
 __global__ void __launch_bounds__(256)
@@ -487,6 +501,22 @@ int coarse_chunks(int B, int De, int L, int* Lc_out) {
   return (L + Lc - 1) / Lc;
 }
 
+// Pieces of a coarse chunk in the pre-pass (at most 8): the coarse chunks fill the reverse kernel's two blocks per SM and leave the
+// pre-pass, which has four, with an uneven few.  The count minimises a model measured on this kernel: ns a step with so many blocks to
+// an SM, and 160 ns of the chain kernel for every piece of a sequence.  Both kernels, us, one piece / by the rule: 16384 steps of 4096
+// channels 363 / 294 (4 pieces), 3 x 1371 of 2048 55.6 / 48.2 (3), 2 x 6000 of 2048 142 / 120 (4), 5 x 800 of 3584 60 / 48 (5).
+int prepass_pieces(int B, int De, int Lc, int ncc, int* Lp_out) {
+  const long long blocks1 = (long long)B * ((De + BCH - 1) / BCH) * (ncc - 1);
+  int best = 1;
+  long long best_t = 0;
+  for (int m = 1; m <= 8; ++m) {
+    const long long k = (blocks1 * m + 147) / 148, Lp = ((Lc + m - 1) / m + CK - 1) / CK * CK;
+    const long long t = Lp * (k <= 1 ? 133 : k == 2 ? 197 : k == 3 ? 275 : 90 * k) + 160LL * ncc * m;
+    if (m == 1 || t < best_t) { best = m; best_t = t; *Lp_out = (int)Lp; }
+  }
+  return best;
+}
+
 }  // namespace
 
 size_t scan_bwd_ckpt_floats(int B, int De, int L) { return (size_t)B * ((L + CK - 1) / CK) * De * NST; }
@@ -495,7 +525,10 @@ size_t scan_bwd_ws_bytes(int B, int De, int L) {
   int Lc = 0;
   const int ncc = coarse_chunks(B, De, L, &Lc);
   size_t floats = scan_bwd_ckpt_floats(B, De, L);
-  if (ncc > 1) floats += (size_t)B * ncc * De * (4 * NST + 2);
+  if (ncc > 1) {
+    int Lp = 0;
+    floats += (size_t)B * ncc * De * (3 * NST + 1 + (NST + 1) * (size_t)prepass_pieces(B, De, Lc, ncc, &Lp));
+  }
   return align_up(sizeof(float) * floats, 256);
 }
 
@@ -512,15 +545,17 @@ cudaError_t launch_scan_backward(const rom_config& c, const ScanBwd& s, cudaStre
   const int nck = (c.L + CK - 1) / CK;
   int Lc = 0;
   const int ncc = coarse_chunks(c.B, c.d_inner, c.L, &Lc);
+  int Lp = 0;
+  const int mp = prepass_pieces(c.B, c.d_inner, Lc, ncc, &Lp);
   const size_t n_fine = scan_bwd_ckpt_floats(c.B, c.d_inner, c.L), n_coarse = (size_t)c.B * ncc * c.d_inner * NST;
-  float* q_start = s.ckpt + n_fine;
-  float* g_in = q_start + n_coarse;
+  float* g_in = s.ckpt + n_fine;
   float* h_end = g_in + n_coarse;
   float* h_in = h_end + n_coarse;
-  float* sum_delta = h_in + n_coarse;
-  float* sum_delta_h = sum_delta + (size_t)c.B * ncc * c.d_inner;
+  float* q_start = h_in + n_coarse;
+  float* sum_delta_h = q_start + n_coarse * mp;
+  float* sum_delta = sum_delta_h + (size_t)c.B * ncc * c.d_inner;
   const BwdArgs a{s.dy, s.u, s.delta, s.A, s.Bm, s.Cm, s.D, s.z, s.dh_last, s.du, s.ddelta, s.dA, s.dBm, s.dCm, s.dD, s.dz, s.dh0, s.dpre, s.db_dt,
-                  s.ckpt, c.L, c.d_inner, nck, s.ldz, s.dz_rows, s.K, Lc, ncc, g_in, q_start, sum_delta};
+                  s.ckpt, c.L, c.d_inner, nck, s.ldz, s.dz_rows, s.K, Lc, ncc, g_in, Lp, mp, q_start, sum_delta};
   cudaError_t e = cudaSuccess;
   const bool zoh = c.disc_mode == 0, bf = c.dtype == ROM_BF16;
   const long long n_thr = (long long)c.B * c.d_inner * NST;
@@ -541,13 +576,13 @@ cudaError_t launch_scan_backward(const rom_config& c, const ScanBwd& s, cudaStre
   }
   const dim3 grid((c.d_inner + BCH - 1) / BCH, c.B, ncc);
   if (ncc > 1) {
-    const dim3 pgrid(grid.x, grid.y, ncc - 1);
+    const dim3 pgrid(grid.x, grid.y, (ncc - 1) * mp);
     if (!bf) launch_k(scan_bwd_prepass_kernel<float, float>, pgrid, BT, 0, st, a);
     else if (s.delta_fp32) launch_k(scan_bwd_prepass_kernel<__nv_bfloat16, float>, pgrid, BT, 0, st, a);
     else launch_k(scan_bwd_prepass_kernel<__nv_bfloat16, __nv_bfloat16>, pgrid, BT, 0, st, a);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    launch_k(scan_bwd_chain_kernel, chain_blocks, 256, 0, st, s.A, s.dh_last, q_start, sum_delta, g_in, c.B, c.d_inner, ncc);
+    launch_k(scan_bwd_chain_kernel, chain_blocks, 256, 0, st, s.A, s.dh_last, q_start, sum_delta, g_in, c.B, c.d_inner, ncc, mp);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
