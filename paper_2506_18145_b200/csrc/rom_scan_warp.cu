@@ -165,6 +165,9 @@ scan_warp_kernel(const ScanArgs p) {
   auto run = [&](auto so_tag) {
     constexpr bool SO = decltype(so_tag)::value;
     constexpr bool CKPT = MODE == SCAN_CKPT || MODE == SCAN_FULL_CKPT || (MODE == SCAN_FIRST_CKPT && !SO);
+    // from a zero state and with nothing read before the end, the state is carried times -A: one product less an update (16384 steps of
+    // 4096 channels 280 -> 272 us for the first launch, 4 x 2048 of 2048 75.4 -> 73.8)
+    constexpr bool SCALED = ZOH && SO && !CKPT;
     if (SLOTS && !SO) fetch_rows(0);
     fetch(0);
     for (int t0 = 0; t0 < L; t0 += CK) {
@@ -206,7 +209,9 @@ scan_warp_kernel(const ScanArgs p) {
             const float2 x = __fmul2_rn(dl[j], a2[n][j]);
             const float2 a = make_float2(ex2_ftz(x.x), ex2_ftz(x.y));
             const float2 uB = __fmul2_rn(uu[j], dup(bb[n]));
-            if (ZOH) {             // w = -B u / A, h <- a (h - w) + w
+            if (SCALED) {
+              h[n][j] = __ffma2_rn(a, __ffma2_rn(uB, dup(-1.0f), h[n][j]), uB);
+            } else if (ZOH) {      // w = -B u / A, h <- a (h - w) + w
               const float2 w = __fmul2_rn(uB, kin[n][j]);
               h[n][j] = __ffma2_rn(a, __ffma2_rn(w, dup(-1.0f), h[n][j]), w);
             } else {
@@ -268,6 +273,11 @@ scan_warp_kernel(const ScanArgs p) {
         __syncwarp();
       }
     }
+    if constexpr (SCALED)
+#pragma unroll
+      for (int n = 0; n < 4; ++n)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) h[n][j] = __fmul2_rn(h[n][j], kin[n][j]);
   };
   if constexpr (MODE == SCAN_STATE || MODE == SCAN_CKPT) run(std::true_type{});
   else if constexpr (FIRST) { if (so) run(std::true_type{}); else run(std::false_type{}); }
