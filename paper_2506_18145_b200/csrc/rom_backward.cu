@@ -212,7 +212,8 @@ pack_bc_kernel(const float* __restrict__ dBm, const float* __restrict__ dCm, T* 
 // A thread walks `seg` steps of four channels (two packed pairs) with a window of the last k-1 rows of H and of the k-1 rows of
 // dH still being collected; three rows of four steps are in flight while four are used.  Bound by HBM (24 bytes per token and
 // four channels at bf16) at one walk per element: one channel per thread with two-byte loads took 0.96 ms at 16384 x 4096
-// channels (0.56 TB/s), bound by its load and exponential instructions.
+// channels (0.56 TB/s), bound by its load and exponential instructions.  bf16: four blocks to an SM by register limit (158 otherwise), so
+// that 516 blocks are one wave: 4113 tokens of 2048 channels 30.9 -> 24.7 us, 16384 of 4096 135.6 -> 133.8.
 template <typename T> struct Raw4;
 template <> struct Raw4<__nv_bfloat16> {
   uint2 q;
@@ -241,7 +242,7 @@ template <bool PRECISE> __device__ __forceinline__ float dsilu(float v) {
 }
 
 template <typename T, int KC>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, sizeof(T) == 2 ? 4 : 2)
 conv_bwd_kernel(const T* __restrict__ HZ, const T* __restrict__ w_conv, const float* __restrict__ b_conv, const T* __restrict__ dU1,
                 const T* __restrict__ dU2, T* __restrict__ dHZ, const int32_t* __restrict__ row_of_assign, float* __restrict__ dw,
                 float* __restrict__ db, int L, int De, int K, int seg) {
