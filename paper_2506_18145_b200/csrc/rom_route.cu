@@ -48,9 +48,8 @@ struct OffsetsArgs {
   int32_t* counts_ws; int32_t* offsets_ws; int32_t* pad_offsets; int32_t* num_m_tiles; int32_t* tile_expert; int max_m_tiles;
   int32_t* counts_out; int32_t* offsets_out;
   int32_t* assign_of_row; int rows_max;      // cleared to -1 by the grid
-  int32_t* ticket;                           // zero on entry; left zero on exit (null: the offsets are formed later)
-  int32_t* status;                           // by_expert: the status block, zeroed here
-  bool by_expert;                            // histograms as [E, n_chunks] instead of [n_chunks, E]
+  int32_t* ticket;                           // zero on entry; left zero on exit
+  int32_t* status;                           // OWN: the status block, zeroed by the logits kernel
 };
 
 // offsets and the row-tile -> expert map from the shared copies, by one block
@@ -174,7 +173,8 @@ route_offsets(int32_t* __restrict__ chunk_counts, int n_chunks, int E, const Off
 // d_model a lane reads 4 consecutive elements of one token row per 8-token tile (32-byte sectors, straight
 // from global memory) and 4 consecutive fp64 weights of one expert (L1/L2-resident copy); MMA j of the step
 // contracts elements {j, 4+j, 8+j, 12+j} of the 16.  No shared memory until the logits meet for the top-K.
-template <typename T>
+// OWN: for route_scatter_gather<true> (no ticket).
+template <typename T, bool OWN>
 __global__ void __launch_bounds__(512)
 route_logits_topk(const T* __restrict__ x, const T* __restrict__ W_r, const float* __restrict__ b_r,
                   int T_tokens, int Dm, int E, int K, int gate_mode,
@@ -213,7 +213,7 @@ route_logits_topk(const T* __restrict__ x, const T* __restrict__ W_r, const floa
   const bool w_ok = w * NT8 + gq < E;
   const T* wrow = W_r + (size_t)min(w * NT8 + gq, E - 1) * Dm + 4 * t4;
 
-  if (oa.by_expert && blockIdx.x == 0 && tid < kStatusInts) oa.status[tid] = 0;
+  if (OWN && blockIdx.x == 0 && tid < kStatusInts) oa.status[tid] = 0;
   // the row -> assignment table starts at -1 everywhere (padding rows keep it); the whole grid clears it
   for (int i = blockIdx.x * blockDim.x + tid; i < oa.rows_max; i += gridDim.x * blockDim.x) oa.assign_of_row[i] = -1;
 
@@ -325,13 +325,13 @@ route_logits_topk(const T* __restrict__ x, const T* __restrict__ W_r, const floa
     for (int e = 0; e < E; ++e) {
       int c = 0;
       for (int k = 0; k < K; ++k) c += __popc(__ballot_sync(0xffffffffu, idx_s[tid * K + k] == e));
-      if (tid == 0) chunk_counts[oa.by_expert ? (size_t)e * n_chunks + blockIdx.x : (size_t)blockIdx.x * E + e] = c;
+      if (tid == 0) chunk_counts[OWN ? (size_t)e * n_chunks + blockIdx.x : (size_t)blockIdx.x * E + e] = c;
     }
   }
 
   // The block that finishes last builds the offsets from all the histograms: every block publishes its writes
   // (histogram, cleared table slice) and takes a ticket; nobody waits for anybody.
-  if (oa.ticket == nullptr) return;
+  if (OWN) return;
   __shared__ int s_last;
   __threadfence();
   __syncthreads();
@@ -600,7 +600,7 @@ cudaError_t launch_balance(const rom_config& c, const void* x, const void* W_r, 
 static cudaError_t launch_perm_tables(const rom_config& c, const int32_t* idx_ws, int32_t* counts, int32_t* offsets, int32_t* perm,
                                       int32_t* inv_perm, char* ws, const WsLayout& lay, cudaStream_t st);
 static cudaError_t launch_scatter(const rom_config& c, const int32_t* idx_ws, int32_t* perm, int32_t* inv_perm, char* ws,
-                                  const WsLayout& lay, const void* x, const OffsetsArgs& oa, cudaStream_t st);
+                                  const WsLayout& lay, const void* x, const OffsetsArgs& oa, bool own, cudaStream_t st);
 
 cudaError_t launch_route_stats(const rom_config& c, const void* x, const void* W_r, const float* b_r,
                                int32_t* topk_idx, float* gates, int32_t* counts, int32_t* offsets,
@@ -625,26 +625,26 @@ cudaError_t launch_route_stats(const rom_config& c, const void* x, const void* W
   const OffsetsArgs oa{reinterpret_cast<int32_t*>(ws + lay.counts), reinterpret_cast<int32_t*>(ws + lay.offsets),
                        reinterpret_cast<int32_t*>(ws + lay.pad_offsets), reinterpret_cast<int32_t*>(ws + lay.num_m_tiles),
                        reinterpret_cast<int32_t*>(ws + lay.tile_expert), (int)lay.max_m_tiles, counts, offsets,
-                       assign_of_row, (int)lay.rows_max, own ? nullptr : status + kStatTicket, status, own};
+                       assign_of_row, (int)lay.rows_max, status + kStatTicket, status};
   const int idx_ints = RT * c.K > 3 * kMaxE + 2 ? RT * c.K : 3 * kMaxE + 2;
   const size_t smem = sizeof(double) * (size_t)(dsplit > 2 ? dsplit : 2) * RT * Epad8 + sizeof(int32_t) * idx_ints;
   if (bf)
-    launch_k(route_logits_topk<__nv_bfloat16>, blocks, threads, smem, st, 
+    launch_k(own ? route_logits_topk<__nv_bfloat16, true> : route_logits_topk<__nv_bfloat16, false>, blocks, threads, smem, st, 
         (const __nv_bfloat16*)x, (const __nv_bfloat16*)W_r, b_r, T, c.d_model, c.E, c.K, c.gate_mode, idx_ws, gates, chunk_counts,
         chunk_prob, probs, (int)lay.n_chunks, oa);
   else
-    launch_k(route_logits_topk<float>, blocks, threads, smem, st, 
+    launch_k(own ? route_logits_topk<float, true> : route_logits_topk<float, false>, blocks, threads, smem, st, 
         (const float*)x, (const float*)W_r, b_r, T, c.d_model, c.E, c.K, c.gate_mode, idx_ws, gates, chunk_counts, chunk_prob, probs,
         (int)lay.n_chunks, oa);
   count_launch();
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) return err;
-  return launch_scatter(c, idx_ws, perm, inv_perm, ws, lay, gather_x ? x : nullptr, oa, st);
+  return launch_scatter(c, idx_ws, perm, inv_perm, ws, lay, gather_x ? x : nullptr, oa, own, st);
 }
 
 // the permutation (and, with x, the gathered rows) from the indices, the per-chunk bases and the offsets
 static cudaError_t launch_scatter(const rom_config& c, const int32_t* idx_ws, int32_t* perm, int32_t* inv_perm, char* ws,
-                                  const WsLayout& lay, const void* x, const OffsetsArgs& oa, cudaStream_t st) {
+                                  const WsLayout& lay, const void* x, const OffsetsArgs& oa, bool own, cudaStream_t st) {
   const int32_t* chunk_base = reinterpret_cast<int32_t*>(ws + lay.chunk_counts);
   const int32_t* offs = reinterpret_cast<int32_t*>(ws + lay.offsets);
   const int32_t* poffs = reinterpret_cast<int32_t*>(ws + lay.pad_offsets);
@@ -655,7 +655,7 @@ static cudaError_t launch_scatter(const rom_config& c, const int32_t* idx_ws, in
     const cudaError_t e = current_device_sm_count(&num_sms);
     if (e != cudaSuccess) return e;
     const int grid = (int)lay.n_chunks > num_sms ? (int)lay.n_chunks : num_sms;
-    launch_k(oa.by_expert ? route_scatter_gather<true> : route_scatter_gather<false>, grid, 256, 0, st, idx_ws, chunk_base, oa, (int)lay.T, c.E, c.K,
+    launch_k(own ? route_scatter_gather<true> : route_scatter_gather<false>, grid, 256, 0, st, idx_ws, chunk_base, oa, (int)lay.T, c.E, c.K,
              (int)lay.n_chunks, roa, reinterpret_cast<const uint4*>(x), reinterpret_cast<uint4*>(ws + lay.x_perm), (int)((size_t)c.d_model * lay.esz / 16));
   } else {
     const int wpb = 8;
@@ -672,10 +672,10 @@ static cudaError_t launch_perm_tables(const rom_config& c, const int32_t* idx_ws
   const OffsetsArgs oa{reinterpret_cast<int32_t*>(ws + lay.counts), reinterpret_cast<int32_t*>(ws + lay.offsets),
                        reinterpret_cast<int32_t*>(ws + lay.pad_offsets), reinterpret_cast<int32_t*>(ws + lay.num_m_tiles),
                        reinterpret_cast<int32_t*>(ws + lay.tile_expert), (int)lay.max_m_tiles, counts, offsets,
-                       reinterpret_cast<int32_t*>(ws + lay.assign_of_row), 0, nullptr, nullptr, false};
+                       reinterpret_cast<int32_t*>(ws + lay.assign_of_row), 0, nullptr, nullptr};
   launch_k(route_offsets, 1, 1024, 0, st, reinterpret_cast<int32_t*>(ws + lay.chunk_counts), (int)lay.n_chunks, c.E, oa);
   count_launch();
-  return launch_scatter(c, idx_ws, perm, inv_perm, ws, lay, nullptr, oa, st);
+  return launch_scatter(c, idx_ws, perm, inv_perm, ws, lay, nullptr, oa, false, st);
 }
 
 cudaError_t launch_gather_rows(const rom_config& c, const void* x, char* ws, const WsLayout& lay, cudaStream_t st) {
