@@ -86,9 +86,10 @@ typedef struct {
                                  128 tokens); ignored where the sizes do not fit (d_r > 128, d_r + 2 D_s > 160) or b_conv
                                  is off a 16-byte boundary                                                      */
 #define ROM_FLAG_TEST_STALL 4 /* fault injection for tests of the device-side timeout path (tensor path only, d_model > 64): the
-                                 first grouped projection withholds the copies of one operand stage per CTA (or, on CTA pairs and
-                                 in rom_layer_step, waits for more bytes than are copied) and every wait of it gives up after 2^14 polls instead of 2^22, so the call returns
-                                 normally, produces no valid output, and rom_get_status reports
+                                 first grouped projection, and the shared x Proj and dt Proj after it, withhold the copies of one
+                                 operand stage per CTA (or, on CTA pairs, in the x Proj and dt Proj kernels and
+                                 in rom_layer_step, wait for more bytes than are copied) and every wait of them gives up after 2^14 polls
+                                 instead of 2^22, so the call returns normally, produces no valid output, and rom_get_status reports
                                  ROM_ERR_DEVICE_TIMEOUT.  The workspace stays usable for the next call.          */
 
 typedef struct {                /* all read-only device pointers                                   */

@@ -340,7 +340,8 @@ int layer_forward_impl(const rom_config* cfg, const rom_weights* w, const void* 
     if (!te && M_max <= 128 && Kd >= 1024 && Kd % 2048 == 0 && ep.mode == EPI_XPROJ)
       return launch_gemm_skinny(c.dtype, A_, lda, B_, ldb, M_max, Nn, Kd, ep, st);
     if (tc) return launch_gemm_tc(A_, lda, B_, ldb, n_experts, M_max, Nn, Kd, te, nmt, ep, status, st,
-                                  (c.flags & ROM_FLAG_TEST_STALL) != 0 && (ep.mode == EPI_INPROJ || (ep.mode == EPI_STORE && Nn == 2 * De)), false,
+                                  (c.flags & ROM_FLAG_TEST_STALL) != 0 && (ep.mode == EPI_INPROJ || (ep.mode == EPI_STORE && Nn == 2 * De) ||
+                                                                           (!te && (ep.mode == EPI_XPROJ || ep.mode == EPI_SOFTPLUS))), false,
                                   te ? reinterpret_cast<const int32_t*>(W + lay.pad_offsets) : nullptr);
     return launch_gemm_simt(c.dtype, A_, lda, B_, ldb, bstride, M_max, Nn, Kd, te, nmt, ep, st, te ? reinterpret_cast<const int32_t*>(W + lay.assign_of_row) : nullptr);
   };

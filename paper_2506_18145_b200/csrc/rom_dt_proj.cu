@@ -41,7 +41,8 @@ __device__ __forceinline__ float2 softplus2_bf16(float2 v) {
 template <int NKB>
 __global__ void __launch_bounds__(DT_THREADS, 1)
 dt_proj_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b, const __grid_constant__ CUtensorMap tmap_c,
-               const float* __restrict__ bias, int M, int N, int block_n, uint32_t idesc, int n_tiles, int32_t* __restrict__ status) {
+               const float* __restrict__ bias, int M, int N, int block_n, uint32_t idesc, int n_tiles, int32_t* __restrict__ status,
+               uint32_t wait_limit, uint32_t stall) {
   constexpr int STAGES = dt_stages(NKB), SA = NKB * A_KB;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw), base = (raw + 1023u) & ~1023u;      // 128B-swizzled tiles need 1024-byte alignment
@@ -70,7 +71,7 @@ dt_proj_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     // the weights: not written by the kernel before this one, and everything before that one is complete
-    mbar_expect_tx(w_bar, (uint32_t)(NKB * block_n * BLOCK_K * 2));
+    mbar_expect_tx(w_bar, (uint32_t)(NKB * block_n * BLOCK_K * 2) + stall);      // (fault injection: 16 bytes that never come)
 #pragma unroll
     for (int kb = 0; kb < NKB; ++kb) tma_load_2d(sb + kb * B_KB, &tmap_b, w_bar, kb * BLOCK_K, n_tile * block_n);
   }
@@ -91,7 +92,7 @@ dt_proj_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     if (lane == 0) {
       int stage = 0, issued = 0; uint32_t phase = 0;
       for (int m = m_first; m < m_tiles; m += m_step) {
-        if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, WAIT_LIMIT)) { ok = false; break; }
+        if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, wait_limit)) { ok = false; break; }
         mbar_expect_tx(full_bar(stage), (uint32_t)SA);
 #pragma unroll
         for (int kb = 0; kb < NKB; ++kb) tma_load_2d(sa0 + stage * SA + kb * A_KB, &tmap_a, full_bar(stage), kb * BLOCK_K, m * BLOCK_M);
@@ -99,28 +100,26 @@ dt_proj_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
         if (++stage == STAGES) { stage = 0; phase ^= 1u; }
       }
       if (!ok) {
-        if (!*abort_flag) { atomicExch(status + kStatCode, ROM_ERR_DEVICE_TIMEOUT); atomicExch(status + kStatWhere, 31); }
+        if (!*abort_flag) latch_timeout(status, 31);
         *abort_flag = 1;
       }
-      if (*abort_flag) {      // the copies in flight get a bounded time to land before the CTA exits
-        int s = stage; uint32_t ph = phase;
-        for (int i = 0; i < min(issued, STAGES); ++i) {
-          if (--s < 0) { s = STAGES - 1; ph ^= 1u; }
-          for (uint32_t it = 0; it < (WAIT_LIMIT >> 2); ++it)
-            if (mbar_try_wait(full_bar(s), ph)) break;
-        }
-        for (uint32_t it = 0; it < (WAIT_LIMIT >> 2); ++it)
-          if (mbar_try_wait(w_bar, 0)) break;
+      // the CTA does not exit before its copies have landed, or had a bounded time to (another role may give up after the last was issued)
+      for (int i = 0; i < min(issued, STAGES); ++i) {
+        if (--stage < 0) { stage = STAGES - 1; phase ^= 1u; }
+        for (uint32_t it = 0; it < (wait_limit >> 2); ++it)
+          if (mbar_try_wait(full_bar(stage), phase)) break;
       }
+      for (uint32_t it = 0; it < (wait_limit >> 2); ++it)
+        if (mbar_try_wait(w_bar, 0)) break;
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     if (lane == 0) {
       int stage = 0, acc = 0; uint32_t phase = 0, acc_phase = 0;
       bool issued_any = false;
-      ok = mbar_wait(w_bar, 0, abort_flag, WAIT_LIMIT);
+      ok = mbar_wait(w_bar, 0, abort_flag, wait_limit);
       for (int m = m_first; m < m_tiles && ok; m += m_step) {
-        if (!mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag, WAIT_LIMIT) || !mbar_wait(full_bar(stage), phase, abort_flag, WAIT_LIMIT)) { ok = false; break; }
+        if (!mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag, wait_limit) || !mbar_wait(full_bar(stage), phase, abort_flag, wait_limit)) { ok = false; break; }
         tc_fence_after();
 #pragma unroll
         for (int kb = 0; kb < NKB; ++kb) {
@@ -135,12 +134,12 @@ dt_proj_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
         if (++acc == DT_ACC) { acc = 0; acc_phase ^= 1u; }
       }
       if (!ok) {
-        if (!*abort_flag) { atomicExch(status + kStatCode, ROM_ERR_DEVICE_TIMEOUT); atomicExch(status + kStatWhere, 32); }
+        if (!*abort_flag) latch_timeout(status, 32);
         *abort_flag = 1;
       }
       if (*abort_flag && issued_any) {
         umma_commit(drain_bar);
-        for (uint32_t it = 0; it < (WAIT_LIMIT >> 2); ++it)
+        for (uint32_t it = 0; it < (wait_limit >> 2); ++it)
           if (mbar_try_wait(drain_bar, 0)) break;
       }
     }
@@ -152,7 +151,7 @@ dt_proj_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     int acc = 0; uint32_t acc_phase = 0;
     for (int m = m_first; m < m_tiles; m += m_step) {
       // warp-uniform outcome: the tensor-memory loads below need the whole warp
-      if (!__all_sync(0xffffffffu, mbar_wait(tfull_bar(acc), acc_phase, abort_flag, WAIT_LIMIT))) { ok = false; break; }
+      if (!__all_sync(0xffffffffu, mbar_wait(tfull_bar(acc), acc_phase, abort_flag, wait_limit))) { ok = false; break; }
       tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)acc * DT_N;
       for (int cc = 0; cc < n_chunks; ++cc) {
@@ -195,7 +194,7 @@ dt_proj_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     }
     if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     if (!ok && lane == 0) {
-      if (!*abort_flag) { atomicExch(status + kStatCode, ROM_ERR_DEVICE_TIMEOUT); atomicExch(status + kStatWhere, 33); }
+      if (!*abort_flag) latch_timeout(status, 33);
       *abort_flag = 1;
     }
   }
@@ -214,7 +213,7 @@ bool dt_proj_applicable(int N, int Kd) {
   return Kd <= 2 * BLOCK_K && current_device_sm_count(&num_sms) == cudaSuccess && (N + DT_N - 1) / DT_N <= num_sms;
 }
 
-cudaError_t launch_dt_proj(const void* A, const void* Bw, int M, int N, int Kd, const Epilogue& epi, int32_t* status, cudaStream_t st) {
+cudaError_t launch_dt_proj(const void* A, const void* Bw, int M, int N, int Kd, const Epilogue& epi, int32_t* status, cudaStream_t st, bool test_stall) {
   int num_sms = 0;
   cudaError_t e = current_device_sm_count(&num_sms);
   if (e != cudaSuccess) return e;
@@ -230,7 +229,8 @@ cudaError_t launch_dt_proj(const void* A, const void* Bw, int M, int N, int Kd, 
     const cudaError_t e2 = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e2 != cudaSuccess) return e2;
     count_launch();
-    return launch_k(kern, dim3((unsigned)(n_tiles * (m_tiles < rows ? m_tiles : rows))), DT_THREADS, smem, st, ta, tb, tc, epi.bias, M, N, block_n, idesc, n_tiles, status);
+    return launch_k(kern, dim3((unsigned)(n_tiles * (m_tiles < rows ? m_tiles : rows))), DT_THREADS, smem, st, ta, tb, tc, epi.bias, M, N, block_n, idesc, n_tiles, status,
+                    test_stall ? WAIT_LIMIT_TEST : WAIT_LIMIT, test_stall ? 16u : 0u);
   };
   return Kd <= BLOCK_K ? go(dt_proj_kernel<1>, dt_smem(1)) : go(dt_proj_kernel<2>, dt_smem(2));
 }

@@ -626,9 +626,9 @@ cudaError_t launch_gemm_tc(const void* A, int lda, const void* Bw, int ldb, int 
   const bool swiglu = epi.mode == EPI_SWIGLU;      // N output columns from 2N rows of B per expert, loaded as two boxes of 128 rows
   if (swiglu && (N % 128 != 0 || MAX_BLOCK_N != 256 || b_mn)) return cudaErrorInvalidValue;
   if (epi.mode == EPI_XPROJ && !tile_expert && !epi.row_token && lda == Kd && ldb == Kd && x_proj_applicable(M_max, N, Kd))
-    return launch_x_proj(A, Bw, M_max, N, Kd, epi, status, st);
+    return launch_x_proj(A, Bw, M_max, N, Kd, epi, status, st, test_stall);
   if (epi.mode == EPI_SOFTPLUS && lda == Kd && ldb == Kd && epi.ldc == N && dt_proj_applicable(N, Kd))
-    return launch_dt_proj(A, Bw, M_max, N, Kd, epi, status, st);
+    return launch_dt_proj(A, Bw, M_max, N, Kd, epi, status, st, test_stall);
   if (b_mn && n_experts > 1 && Kd % BLOCK_K != 0) return cudaErrorInvalidValue;      // a K block must not run into the next expert
   int block_n = (swiglu || N >= MAX_BLOCK_N) ? MAX_BLOCK_N : (N + 31) / 32 * 32;
   if (epi.mode == EPI_XPROJ && block_n > XPROJ_BLOCK_N) block_n = XPROJ_BLOCK_N;

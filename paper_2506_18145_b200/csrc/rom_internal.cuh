@@ -20,6 +20,7 @@ constexpr int kStatusInts = 64;    // status block at the head of the workspace
 constexpr int kStatCode = 0;       // 0 or the rom_status a kernel latched (a wait that expired, an index out of range)
 constexpr int kStatWhere = 1;      // which wait gave up / which debug check failed (debug aid)
 constexpr int kStatIndex = 2;      // debug checks: the offending index
+constexpr int kStatWaits = 3;      // x Proj / dt Proj kernels: bit i set when their wait 31 + i gave up (what gave up first is in kStatWhere)
 constexpr int kStatTicket = 8;     // router: blocks-done counter (zero between calls)
 constexpr int kStatNonFinite = 9;  // Mamba2-style block: some x after the conv is not finite
 constexpr int kMaxCanaries = 40;   // sub-buffers of the workspace (debug checks put a canary after each)
@@ -234,12 +235,12 @@ cudaError_t launch_gemm_tc(const void* A, int lda, const void* Bw, int ldb, int 
 
 // x Proj of few tokens, the contracted index shared by a cluster (rom_x_proj.cu): C = A[M, Kd] Bw[N, Kd]^T split into delta | B | C; bf16.
 bool x_proj_applicable(int M, int N, int Kd);
-cudaError_t launch_x_proj(const void* A, const void* Bw, int M, int N, int Kd, const Epilogue& epi, int32_t* status, cudaStream_t st);
+cudaError_t launch_x_proj(const void* A, const void* Bw, int M, int N, int Kd, const Epilogue& epi, int32_t* status, cudaStream_t st, bool test_stall);
 
 // dt Proj with a short contraction (rom_dt_proj.cu): C[M, N] = softplus(A[M, Kd] Bw[N, Kd]^T + bias), rows contiguous; bf16.  Its kernel lets
 // the next one in only as its blocks end (a scan's blocks must not pile up).
 bool dt_proj_applicable(int N, int Kd);
-cudaError_t launch_dt_proj(const void* A, const void* Bw, int M, int N, int Kd, const Epilogue& epi, int32_t* status, cudaStream_t st);
+cudaError_t launch_dt_proj(const void* A, const void* Bw, int M, int N, int Kd, const Epilogue& epi, int32_t* status, cudaStream_t st, bool test_stall);
 
 // Weight gradient on the tensor cores (bf16): C[s][P, Q] fp32 = sum over rows r of segment s of X[r, p] Y[r, q]; X [rows, P],
 // Y [rows, Q]; seg: n_seg + 1 device row offsets, multiples of 64, or nullptr = one sum over all rows.

@@ -44,6 +44,12 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
   return false;
 }
+// A wait of the x Proj or dt Proj kernel (31..33, 41..43) gave up.
+__device__ __forceinline__ void latch_timeout(int32_t* status, int where) {
+  atomicExch(status + kStatCode, ROM_ERR_DEVICE_TIMEOUT);
+  atomicCAS(status + kStatWhere, 0, where);
+  atomicOr(status + kStatWaits, 1 << (where - 31));
+}
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"

@@ -29,7 +29,7 @@ __device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
 template <int S>
 __global__ void __launch_bounds__(X_THREADS, 1)
 x_proj_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b, int M, int N, int num_kb,
-              int block_n, uint32_t idesc, Epilogue ep, int32_t* __restrict__ status) {
+              int block_n, uint32_t idesc, Epilogue ep, int32_t* __restrict__ status, uint32_t wait_limit, uint32_t stall) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw), base = (raw + 1023u) & ~1023u;      // 128B-swizzled tiles need 1024-byte alignment
   unsigned char* smem = smem_raw + (base - raw);
@@ -58,7 +58,7 @@ x_proj_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant_
   const uint32_t stage_tx = (uint32_t)(BLOCK_M + block_n) * BLOCK_K * 2;
   if (tid == 0) {
     for (int s = 0; s < n_ahead; ++s) {
-      mbar_expect_tx(full_bar(s), stage_tx);
+      mbar_expect_tx(full_bar(s), stage_tx + (s == 0 ? stall : 0u));      // (fault injection: 16 bytes that never come)
       tma_load_2d(base + s * X_STAGE + BLOCK_M * BLOCK_K * 2, &tmap_b, full_bar(s), (kb0 + s) * BLOCK_K, 0);
     }
   }
@@ -76,7 +76,7 @@ x_proj_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant_
       for (int kb = kb0; kb < kb1; ++kb) {
         const uint32_t sa = base + stage * X_STAGE;
         if (kb - kb0 >= n_ahead) {
-          if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, WAIT_LIMIT)) { ok = false; break; }
+          if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, wait_limit)) { ok = false; break; }
           mbar_expect_tx(full_bar(stage), stage_tx);
           tma_load_2d(sa + BLOCK_M * BLOCK_K * 2, &tmap_b, full_bar(stage), kb * BLOCK_K, 0);
         }
@@ -85,15 +85,14 @@ x_proj_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant_
         if (++stage == X_STAGES) { stage = 0; phase ^= 1u; }
       }
       if (!ok) {
-        if (!*abort_flag) { atomicExch(status + kStatCode, ROM_ERR_DEVICE_TIMEOUT); atomicExch(status + kStatWhere, 41); }
+        if (!*abort_flag) latch_timeout(status, 41);
         *abort_flag = 1;
       }
-      if (*abort_flag) {      // the copies in flight get a bounded time to land before the CTA goes on
-        for (int i = 0; i < min(issued, X_STAGES); ++i) {
-          if (--stage < 0) { stage = X_STAGES - 1; phase ^= 1u; }
-          for (uint32_t it = 0; it < (WAIT_LIMIT >> 2); ++it)
-            if (mbar_try_wait(full_bar(stage), phase)) break;
-        }
+      // the CTA does not go on before its copies have landed, or had a bounded time to (another role may give up after the last was issued)
+      for (int i = 0; i < min(issued, X_STAGES); ++i) {
+        if (--stage < 0) { stage = X_STAGES - 1; phase ^= 1u; }
+        for (uint32_t it = 0; it < (wait_limit >> 2); ++it)
+          if (mbar_try_wait(full_bar(stage), phase)) break;
       }
     }
   } else if (warp == 1) {
@@ -101,7 +100,7 @@ x_proj_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant_
     if (lane == 0) {
       int stage = 0; uint32_t phase = 0;
       for (int kb = kb0; kb < kb1; ++kb) {
-        if (!mbar_wait(full_bar(stage), phase, abort_flag, WAIT_LIMIT)) { ok = false; break; }
+        if (!mbar_wait(full_bar(stage), phase, abort_flag, wait_limit)) { ok = false; break; }
         tc_fence_after();
         const uint64_t ad = make_smem_desc(base + stage * X_STAGE), bd = make_smem_desc(base + stage * X_STAGE + BLOCK_M * BLOCK_K * 2);
 #pragma unroll
@@ -110,7 +109,7 @@ x_proj_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant_
         if (++stage == X_STAGES) { stage = 0; phase ^= 1u; }
       }
       if (!ok) {
-        if (!*abort_flag) { atomicExch(status + kStatCode, ROM_ERR_DEVICE_TIMEOUT); atomicExch(status + kStatWhere, 42); }
+        if (!*abort_flag) latch_timeout(status, 42);
         *abort_flag = 1;
       }
       umma_commit(done_bar);      // (after a wait that ran out too: what has been issued is waited for below)
@@ -119,13 +118,13 @@ x_proj_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant_
   // every product of this CTA is complete: its operands have been read and its sums lie in tensor memory.  (No other wait in the
   // kernel needs the outcome: all threads go on to the barriers, and after a timeout write rows that the status disowns.)
   if (warp >= 2) {
-    ok = __all_sync(0xffffffffu, mbar_wait(done_bar, 0, abort_flag, WAIT_LIMIT));
+    ok = __all_sync(0xffffffffu, mbar_wait(done_bar, 0, abort_flag, wait_limit));
     if (!ok && lane == 0) {
-      if (!*abort_flag) { atomicExch(status + kStatCode, ROM_ERR_DEVICE_TIMEOUT); atomicExch(status + kStatWhere, 43); }
+      if (!*abort_flag) latch_timeout(status, 43);
       *abort_flag = 1;
     }
     if (*abort_flag)              // give the products in flight a bounded time all the same: the stages are about to be written
-      for (uint32_t it = 0; it < (WAIT_LIMIT >> 2); ++it)
+      for (uint32_t it = 0; it < (wait_limit >> 2); ++it)
         if (mbar_try_wait(done_bar, 0)) break;
     __syncwarp();
     tc_fence_after();
@@ -198,7 +197,7 @@ int x_proj_split(int M, int Kd) {
 
 bool x_proj_applicable(int M, int N, int Kd) { return N <= X_N && N % 8 == 0 && x_proj_split(M, Kd) > 1; }
 
-cudaError_t launch_x_proj(const void* A, const void* Bw, int M, int N, int Kd, const Epilogue& epi, int32_t* status, cudaStream_t st) {
+cudaError_t launch_x_proj(const void* A, const void* Bw, int M, int N, int Kd, const Epilogue& epi, int32_t* status, cudaStream_t st, bool test_stall) {
   const int S = x_proj_split(M, Kd), block_n = (N + 31) / 32 * 32;
   CUtensorMap ta, tb;
   if (!make_tmap(&ta, A, (uint64_t)M, (uint64_t)Kd, (uint64_t)Kd, BLOCK_M)) return cudaErrorInvalidValue;
@@ -220,7 +219,8 @@ cudaError_t launch_x_proj(const void* A, const void* Bw, int M, int N, int Kd, c
   cfg.attrs = at;
   cfg.numAttrs = 2;
   count_launch();
-  return cudaLaunchKernelEx(&cfg, kern, ta, tb, M, N, (Kd + BLOCK_K - 1) / BLOCK_K, block_n, idesc, epi, status);
+  return cudaLaunchKernelEx(&cfg, kern, ta, tb, M, N, (Kd + BLOCK_K - 1) / BLOCK_K, block_n, idesc, epi, status, test_stall ? WAIT_LIMIT_TEST : WAIT_LIMIT,
+                            test_stall ? 16u : 0u);
 }
 
 }  // namespace rom

@@ -1,5 +1,5 @@
-"""The device-side timeout path of every kernel with bounded waits that the first grouped projection can run on: one CTA per tile, CTA
-pairs, and the streamed projections of the single-token step.  The host asks for the fault injection; the call must return, report the
+"""The device-side timeout path of every kernel with bounded waits that the first grouped projection can run on (one CTA per tile, CTA
+pairs, the streamed projections of the single-token step) and of the x Proj and dt Proj kernels.  The host asks for the fault injection; the call must return, report the
 wait that ran out, and leave the workspace usable."""
 import numpy as np
 import pytest
@@ -35,6 +35,27 @@ def test_stalled_projection_is_reported(kw):
     ref, im = oracle_layer(s, p)
     np.testing.assert_array_equal(good.idx.cpu().numpy(), im["idx"])
     assert_close(np64(out), ref, TOL["bf16"], "out after a timed-out call")
+
+
+@pytest.mark.parametrize("L,d_inner,dt_rank", [
+    (200, 2048, 128),                                    # clusters of eight, four K blocks a CTA; two K blocks and one row tile of the dt Proj
+    (300, 1088, 48),                                     # four, uneven shares
+    (4300, 2048, 16),                                    # two, more K blocks than stages; more row tiles than stages of the dt Proj
+])
+def test_stalled_small_projections_are_reported(L, d_inner, dt_rank):
+    s = synth.RomShape("stall", 1, L, 128, d_inner, 16, 4, dt_rank, 2, 1, "bf16", 3100 + L)
+    p = synth.make_inputs(s, recipe="unit")
+    good = GpuLayer(s, p)
+    ref = good.forward().clone()
+    g = GpuLayer(s, p, flags=rb.ROM_FLAG_TEST_STALL)
+    rb.rom_layer_forward(g.cfg, g.weights, g.dev["x"], g.out, g.idx, g.gates, g.counts, g.ws)
+    torch.cuda.synchronize()
+    waits = int(g.ws[:16].view(torch.int32).cpu()[3])    # bit i: wait 31 + i gave up
+    assert waits & 0b111, "dt Proj"
+    assert waits & (0b111 << 10), "x Proj"
+    assert rb.rom_get_status(g.ws) == -6
+    good.ws = g.ws
+    assert torch.equal(good.forward(), ref)
 
 
 @pytest.mark.parametrize("B,E,K,d_model,where", [
