@@ -69,7 +69,7 @@ inline int scan_warp_chunks(int B, int De, int L) {
   }
   return best;
 }
-// Chunks per sequence of the fp32 scan with a scalar decay (Mamba2-style block): accurate exp / expm1 make a step of two states per thread (32 channels a block) cost about
+// Chunks per sequence of the fp32 scan: accurate exp / expm1 make a step of two states per thread (32 channels a block) cost about
 // 150 ns whatever the occupancy, so a short sequence is cut until those blocks fill the SMs once, into chunks of at least 32 steps.
 inline int scan_f32_chunks(int B, int De, int L) {
   const long long blocks1 = (long long)B * ((De + 31) / 32);

@@ -2,8 +2,8 @@
 // fused with the output gate y * SiLU(z) and with the re-permutation of the gated rows into expert
 // order (the routing decision of the Gate/Conv projections is reused for Out Proj, Section 4.2).
 //
-// This is the kernel of fp32 storage with many channels (few: rom_scan_f32.cu), of the scalar-decay block, and of a few bf16 channels
-// without a workspace; bf16 otherwise runs rom_scan_warp.cu.  The launch logic of all of them (chunks, chain, checkpoints) is here.
+// This is the kernel of fp32 storage (with rom_scan_f32.cu where that is the faster one: f32_one_launch), of the scalar-decay block, and of
+// a few bf16 channels without a workspace; bf16 otherwise runs rom_scan_warp.cu.  The launch logic of all of them (chunks, chain, checkpoints) is here.
 //
 // State and arithmetic are fp32.  The recurrence is sequential in t, so the parallelism is
 // (sequence, channel, state).  One thread owns NS of the 16 states of NC adjacent channels
@@ -497,12 +497,44 @@ int pick_thread_shape(int B, int De, int num_sms) {
 template <typename T, typename TD, bool PRECISE, bool ZOH, int MODE>
 cudaError_t launch_shape(int shape, const ScanArgs& a, int B, int grid_z, cudaStream_t st) {
   if (shape == 108) return launch_one<T, TD, 1, 8, PRECISE, ZOH, MODE>(a, B, grid_z, st);
-  // (fp32: many channels, or the scalar decay of a Mamba2-style block; bf16 chunks always run 8 states per thread)
-  if constexpr (PRECISE ? !ZOH && (MODE == SCAN_FULL || MODE == SCAN_FIRST) : MODE == SCAN_FULL) {
+  if constexpr (PRECISE || MODE == SCAN_FULL) {      // (bf16 chunks always run 8 states per thread)
     if (shape == 104) return launch_one<T, TD, 1, 4, PRECISE, ZOH, MODE>(a, B, grid_z, st);
     if (shape == 102) return launch_one<T, TD, 1, 2, PRECISE, ZOH, MODE>(a, B, grid_z, st);
   }
   return cudaErrorInvalidValue;
+}
+
+// Whether the one-launch form (rom_scan_f32.cu) takes an fp32 scan with A per channel and state: by the time of the two forms in a model of
+// their measured paces.  nch: chunks per sequence that the general form would use.
+//   one launch: 21.2 ns a step for every block (4 channels) on an SM with the zero-order hold, 14.7 with Delta B (20 and 13.2 beyond four
+//     blocks), whole rounds of a block's segments;
+//   general: ns a step [zoh][NS = 2, 4, 8] of a launch in full and of one with state-only chunks, with one and with two blocks on an SM
+//     (two fit; the mean for a few more than one), whole tiles of 64, 32 and 16 steps, 8.5 or 9.5 us for the launches of a chunked scan.
+// At 724 measured sizes of 64 to 30720 channels and 32 to 16384 steps, with and without a workspace, it names the faster form but for six,
+// where the two differ by 1 to 5 %.  us, general / one launch: one sequence of 16384 x 64
+// 190 / 345, 16384 x 256 327 / 345, 4096 x 512 153 / 88, 256 x 512 25 / 7; Delta B: 4096 x 128 37 / 60, 4096 x 512 68 / 61,
+// 24 x 2048 x 1024 802 / 1118.  The one-launch form was timed below 32768 channels in all.
+bool f32_one_launch(int B, int De, int L, int nch, bool zoh, int num_sms) {
+  if ((long long)B * De >= 32768) return false;
+  constexpr double full[2][3][2] = {{{80, 111}, {200, 314}, {180, 355}}, {{148, 240}, {360, 560}, {460, 915}}};
+  constexpr double state[2][3][2] = {{{60, 82}, {80, 153}, {110, 263}}, {{110, 217}, {250, 412}, {300, 835}}};
+  auto launch = [&](const double (&pace)[2][3][2], int grid_z, int steps) {
+    const int NS = pick_thread_shape(B * grid_z, De, num_sms) % 100, ch = BLOCK / (NST / NS), tile = 128 / NS;
+    const double* t = pace[zoh ? 1 : 0][NS == 2 ? 0 : NS == 4 ? 1 : 2];
+    const int blocks = B * grid_z * ((De + ch - 1) / ch), rest = blocks % 296;
+    const double last = rest == 0 ? 0.0 : rest <= 148 ? t[0] : rest <= 160 ? 0.5 * (t[0] + t[1]) : t[1];
+    return ((blocks / 296) * t[1] + last) * ((steps + tile - 1) / tile * tile);
+  };
+  double general;
+  if (nch == 1) {
+    general = 2000.0 + launch(full, 1, L);
+  } else {
+    const int Lc = (int)align_up((size_t)ceil(L / (nch - 1 + kFirstChunkRatio)), 16);
+    general = (zoh ? 9500.0 : 8500.0) + launch(state, nch, Lc) + launch(full, nch - 1, Lc);
+  }
+  const long long blocks = (long long)B * (De / 4), k = (blocks + 147) / 148;
+  const int seg = blocks <= 148 ? 16 : blocks <= 296 ? 8 : 4, segs = (L + 15) / 16, round = 16 * (segs < seg ? segs : seg);
+  return 1500.0 + (double)align_up((size_t)L, round) * k * (zoh ? (k <= 4 ? 21.2 : 20.0) : (k <= 4 ? 14.7 : 13.2)) <= general;
 }
 
 // CKPT: also store the checkpoints of the backward pass.
@@ -522,23 +554,25 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
   }
   // bf16 storage, A per channel and state: the warp kernel, unless there is neither a workspace for chunks nor one of its warps
   // per SM sub-partition (fewer states per thread then spread the work further)
-  if (PRECISE && !a.scalar_a && scan_f32_applicable(c.B, c.d_inner)) {
+  const bool warp_kernel = !PRECISE && !a.scalar_a && (CKPT || chunk_ws || (long long)c.B * (c.d_inner / 32) >= 4LL * num_sms);
+  const int nch = !chunk_ws ? 1 : warp_kernel ? scan_warp_chunks(c.B, c.d_inner, c.L) : PRECISE ? scan_f32_chunks(c.B, c.d_inner, c.L) : scan_chunks(c.B, c.d_inner, c.L);
+  if (PRECISE && !a.scalar_a && f32_one_launch(c.B, c.d_inner, c.L, nch, zoh, num_sms)) {
     a.h0 = h0; a.h_last = h_last;
     return launch_scan_f32(a, c.B, zoh, CKPT, st);
   }
-  const bool warp_kernel = !PRECISE && !a.scalar_a && (CKPT || chunk_ws || (long long)c.B * (c.d_inner / 32) >= 4LL * num_sms);
-  const int nch = !chunk_ws ? 1 : warp_kernel ? scan_warp_chunks(c.B, c.d_inner, c.L) : PRECISE ? (a.scalar_a ? scan_f32_chunks(c.B, c.d_inner, c.L) : 1) : scan_chunks(c.B, c.d_inner, c.L);
   // one launch over `grid_z` chunks with 8 states per thread (chunked) or the warp kernel
   auto chunks = [&](const ScanArgs& x, int grid_z, auto mode) -> cudaError_t {
-    [[maybe_unused]] constexpr ScanMode M = decltype(mode)::value;
+    constexpr ScanMode M = decltype(mode)::value;
     if constexpr (!PRECISE) { if (warp_kernel) return launch_scan_warp(x, c.B, grid_z, zoh, sizeof(TD) == 4, M, st); }
     if constexpr (!GENERAL) return cudaErrorInvalidValue;
     else {
-      // the scalar-decay block, whose B-bar is Delta B; fp32 storage with few channels: fewer states per thread, so that the chunks
-      // together still spread over the SMs
-      if constexpr (CKPT) return cudaErrorInvalidValue;
-      else return zoh ? cudaErrorInvalidValue
-                      : launch_shape<T, TD, PRECISE, false, M>(PRECISE ? pick_thread_shape(c.B * grid_z, c.d_inner, num_sms) : 108, x, c.B, grid_z, st);
+      // fp32 storage with few channels: fewer states per thread, so that the chunks together still spread over the SMs
+      if constexpr (PRECISE) {
+        const int shape = pick_thread_shape(c.B * grid_z, c.d_inner, num_sms);
+        return zoh ? launch_shape<T, TD, PRECISE, true, M>(shape, x, c.B, grid_z, st) : launch_shape<T, TD, PRECISE, false, M>(shape, x, c.B, grid_z, st);
+      } else {      // the scalar-decay block, whose B-bar is Delta B
+        return zoh ? cudaErrorInvalidValue : launch_shape<T, TD, PRECISE, false, M>(108, x, c.B, grid_z, st);
+      }
     }
   };
   typedef std::integral_constant<ScanMode, FULL> FullTag;

@@ -1,4 +1,4 @@
-// Selective scan for fp32 storage, A per channel and state (same arithmetic and arguments as rom_scan.cu), of few channels: one launch,
+// Selective scan for fp32 storage, A per channel and state (same arithmetic and arguments as rom_scan.cu), below 32768 channels: one launch,
 // every exponential evaluated once.
 //
 // What bounds it: the accurate expf and expm1f of an update (about 45 instructions with the rest of it), and for short sequences the
@@ -7,8 +7,8 @@
 // keeps the decays and inputs of 16 steps of one state in registers and what they do to a state, h -> P h + E, meets in shared memory;
 // every thread composes the segments before its own, sweeps its 16 steps and the 16 lanes of a channel exchange their products with C
 // until each holds one output.  256 steps of 512 channels: 26.7 -> 10 us (one launch of 128 blocks); 2 x 2048 of 1024: 293 -> 175;
-// 24 x 1024 of 1024: 1112 -> 828.  From 32768 channels on the general kernel needs no chunks and is the faster one (512 steps:
-// 469 us against 556; 24576 channels: 1112 against 828).
+// 24 x 1024 of 1024: 1112 -> 828.  It is not the faster one everywhere: long sequences of few channels (the general kernel's chunks fill
+// the SMs), many channels with B-bar = Delta B, and counts that fill the general kernel's blocks evenly (f32_one_launch, rom_scan.cu).
 #include "rom_scan_args.cuh"
 
 namespace rom {
@@ -137,8 +137,6 @@ cudaError_t launch_segs(const ScanArgs& a, int B, cudaStream_t st) {
 }
 
 }  // namespace
-
-bool scan_f32_applicable(int B, int De) { return (long long)B * De < 32768; }
 
 cudaError_t launch_scan_f32(const ScanArgs& a, int B, bool zoh, bool ckpt, cudaStream_t st) {
   if (ckpt) return zoh ? launch_segs<true, true>(a, B, st) : launch_segs<false, true>(a, B, st);
