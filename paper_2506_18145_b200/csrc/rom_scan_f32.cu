@@ -76,6 +76,12 @@ scan_f32_kernel(const ScanArgs p) {
       E = fmaf(a[i], E, b[i]);
       P *= a[i];
     }
+    if (__any_sync(0xffffffffu, P == 0.0f)) {      // none of the decays zero, but their product: an infinite state stays infinite, as step by step
+      bool zero = false;
+#pragma unroll
+      for (int i = 0; i < TS; ++i) zero |= a[i] == 0.0f;
+      if (P == 0.0f && !zero) P = __int_as_float(1);
+    }
     s.map[seg][pr] = make_float2(P, E);
     __syncthreads();
     float h = s.carry[pr];

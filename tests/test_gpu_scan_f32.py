@@ -47,6 +47,21 @@ def test_scan_f32_not_finite_stays_where_it_is(what):
     assert not torch.isfinite(y[0, t_bad, c_bad])
 
 
+@pytest.mark.parametrize("B,L,De", [(1, 1, 64), (1, 200, 64), (1, 3000, 64), (1, 700, 640)])
+def test_scan_f32_infinite_state_stays_infinite(B, L, De):
+    # every decay is above zero, their product over a segment (0.5 * 15 * 16 steps) is not: step by step the state is infinite from then on
+    t_bad, c_bad = L // 3, 5
+    u, d = torch.ones(B, L, De, device="cuda"), torch.full((B, L, De), 0.5, device="cuda")
+    A, Bm = torch.full((De, 16), -15.0, device="cuda"), torch.ones(B, L, 16, device="cuda")
+    cfg = rb.make_config(B, L, De // 2, De, 16, 4, 16, 1, 1, "f32")
+    y, h_last = torch.empty_like(u), torch.empty(B, De, 16, device="cuda")
+    u[0, t_bad, c_bad] = float("inf")
+    rb.rom_scan(cfg, u, d, A, Bm, Bm, torch.ones(De, device="cuda"), None, None, y, h_last)
+    torch.cuda.synchronize()
+    assert torch.isposinf(y[0, t_bad:, c_bad]).all() and torch.isposinf(h_last[0, c_bad]).all()
+    assert torch.isfinite(y[0, :t_bad]).all() and torch.isfinite(y[:, :, [c for c in range(De) if c != c_bad]]).all()
+
+
 @pytest.mark.parametrize("B,L,De,disc_mode,launches", [
     (1, 256, 512, 0, 1), (1, 4096, 512, 0, 1), (1, 2048, 64, 1, 3), (1, 16384, 64, 0, 3), (1, 4096, 192, 0, 3), (1, 512, 64, 1, 1),
     (24, 1024, 1024, 1, 3), (24, 1024, 1024, 0, 1),
