@@ -343,7 +343,7 @@ int layer_forward_impl(const rom_config* cfg, const rom_weights* w, const void* 
                                   (c.flags & ROM_FLAG_TEST_STALL) != 0 && (ep.mode == EPI_INPROJ || (ep.mode == EPI_STORE && Nn == 2 * De) ||
                                                                            (!te && (ep.mode == EPI_XPROJ || ep.mode == EPI_SOFTPLUS))), false,
                                   te ? reinterpret_cast<const int32_t*>(W + lay.pad_offsets) : nullptr);
-    return launch_gemm_simt(c.dtype, A_, lda, B_, ldb, bstride, M_max, Nn, Kd, te, nmt, ep, st, te ? reinterpret_cast<const int32_t*>(W + lay.assign_of_row) : nullptr);
+    return launch_gemm_simt(c.dtype, A_, lda, B_, ldb, bstride, M_max, Nn, Kd, te, nmt, ep, st, te ? reinterpret_cast<const int32_t*>(W + lay.assign_of_row) : nullptr, (int)lay.A);
   };
 
   // S3: grouped [Conv Proj | Gate Proj]
@@ -536,7 +536,7 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
   auto gemm = [&](const void* A_, int lda, const void* B_, int ldb, int n_experts, int64_t bstride, int M_max, int Nn, int Kd,
                   const int32_t* te, const int32_t* nmt, const Epilogue& ep) -> cudaError_t {
     if (tc) return launch_gemm_tc(A_, lda, B_, ldb, n_experts, M_max, Nn, Kd, te, nmt, ep, status, st, false, false, te ? pad_offsets : nullptr);
-    return launch_gemm_simt(c.dtype, A_, lda, B_, ldb, bstride, M_max, Nn, Kd, te, nmt, ep, st);
+    return launch_gemm_simt(c.dtype, A_, lda, B_, ldb, bstride, M_max, Nn, Kd, te, nmt, ep, st, nullptr, (int)lay.A);
   };
   auto store_to = [&](void* C_, int ldc) { return Epilogue{EPI_STORE, C_, ldc, nullptr, nullptr, nullptr, 0, 0, nullptr, nullptr}; };
   // data gradient C[M, Nn] = A[M, Kd] W[e], W [n_experts, Kd, Nn] as the layer holds it: the tensor path reads it MN-major, the
@@ -546,7 +546,7 @@ int rom_layer_backward(const rom_config* cfg, const rom_weights* w, const void* 
     if (tc) return launch_gemm_tc(A_, lda, Wt, Nn, n_experts, M_max, Nn, Kd, te, nmt, ep, status, st, false, true, te ? pad_offsets : nullptr);
     const cudaError_t e = launch_transpose(c.dtype, Wt, scratch, n_experts, Kd, Nn, st);
     if (e != cudaSuccess) return e;
-    return launch_gemm_simt(c.dtype, A_, lda, scratch, Kd, (int64_t)Nn * Kd, M_max, Nn, Kd, te, nmt, ep, st);
+    return launch_gemm_simt(c.dtype, A_, lda, scratch, Kd, (int64_t)Nn * Kd, M_max, Nn, Kd, te, nmt, ep, st, nullptr, (int)lay.A);
   };
 
   float* dBm = reinterpret_cast<float*>(W + bl.dBm);

@@ -135,7 +135,7 @@ int rom_ffn_moe_forward(const rom_config* cfg, int32_t d_ff, const void* W_gu, c
   } else {
     Epilogue e_up{EPI_STORE, W + lay.XZp, 2 * d_ff, nullptr, nullptr, nullptr, 0, 0, nullptr, nullptr};
     ROM_CUDA(launch_gemm_simt(c.dtype, W + lay.x_perm, Dm, W_gu, Dm, (int64_t)2 * d_ff * Dm, (int)lay.rows_max, 2 * d_ff, Dm,
-                              tile_expert, num_m_tiles, e_up, st));
+                              tile_expert, num_m_tiles, e_up, st, nullptr, (int)lay.A));
     const long long total = (long long)lay.rows_max * d_ff;
     const unsigned blocks = (unsigned)((total + 255) / 256);
     const int32_t* pad_offsets = reinterpret_cast<const int32_t*>(W + lay.pad_offsets);
@@ -147,7 +147,7 @@ int rom_ffn_moe_forward(const rom_config* cfg, int32_t d_ff, const void* W_gu, c
     ROM_CUDA(cudaGetLastError());
     Epilogue e_dn{EPI_STORE, W + lay.Op, Dm, nullptr, nullptr, nullptr, 0, 0, nullptr, nullptr};
     ROM_CUDA(launch_gemm_simt(c.dtype, W + lay.Ygp, d_ff, W_down, d_ff, (int64_t)Dm * d_ff, (int)lay.rows_max, Dm, d_ff, tile_expert,
-                              num_m_tiles, e_dn, st));
+                              num_m_tiles, e_dn, st, nullptr, (int)lay.A));
   }
   ROM_CUDA(launch_combine(c, W + lay.Op, row_of_assign, gates, out, st));
   return ROM_OK;

@@ -281,19 +281,32 @@ static cudaError_t launch_f32(const float* A, int lda, const float* B, int ldb, 
 
 cudaError_t launch_gemm_simt(int dtype, const void* A, int lda, const void* Bw, int ldb, int64_t b_expert_stride,
                              int M_max, int N, int Kd, const int32_t* tile_expert, const int32_t* num_m_tiles_dev,
-                             const Epilogue& epi, cudaStream_t st, const int32_t* assign_of_row) {
+                             const Epilogue& epi, cudaStream_t st, const int32_t* assign_of_row, int n_rows) {
   if (dtype == ROM_F32) {
     const float* a = (const float*)A;
     const float* b = (const float*)Bw;
     // large tiles once they give every SM a block
     if ((long long)((M_max + 127) / 128) * ((N + 127) / 128) >= 148)
       return launch_f32<128, 128, 8, 8, 1, 16>(a, lda, b, ldb, b_expert_stride, M_max, N, Kd, tile_expert, num_m_tiles_dev, assign_of_row, epi, st);
-    // Longer contractions in stages of 128 over eight groups, half as many serial steps (256 rows x 256 columns x 512: 17.8 us -> 12; 256
-    // columns and less are two to four stages either way and faster with four groups: 256 x 1024 x 256 12.4 us against 14.9), in 16 x 16
-    // tiles where 32 x 32 leave most SMs idle (the x Proj of a short sequence, 256 x 48 x 512: 8 -> 7).
-    if (!tile_expert && (long long)((M_max + 31) / 32) * ((N + 31) / 32) <= 74 && Kd >= 256)
+    // Blocks of 32 x 32 that have work.  Grouped, M_max counts a row tile of padding for every expert; half of that is there on average,
+    // and half a block of 32 rows an expert where blocks that are all padding leave at once.
+    long long rows = M_max;
+    if (tile_expert && n_rows > 0) {
+      const int experts = (M_max - (int)align_up((size_t)n_rows, kTileM)) / kTileM;
+      const int least = (experts < n_rows ? experts : n_rows) * kTileM, mean = n_rows + experts * kTileM / 2;
+      rows = assign_of_row ? n_rows + experts * 16 : mean > least ? mean : least;
+    }
+    const long long blocks = (rows + 31) / 32 * ((N + 31) / 32);
+    // Longer contractions whose last stage is not mostly empty in stages of 128 over eight groups, half as many serial steps, as long as all
+    // blocks are resident at once (two an SM); in 16 x 16 tiles where 32 x 32 leave most SMs idle.  us, stages of 64 / 128 / 16 x 16 tiles:
+    // 32 blocks, K = 512: 8.2 / 7.9 / 4.1; 64, 512: 8.2 / 8.0 / 7.7; 64, 320: 5.8 / 6.3 / 6.2; 256, 1024: 43.5 / 37.5 / 38; 512, 1024: 44 / 54 / 54;
+    // 2048, 512: 76 / 102 / 112.  Grouped (whole calls): 96 blocks, K = 512: 67.8 / 59.2; 200, 512: 85.6 / 83.2; 288, 1024: 140.6 / 137.4; 320, 1024:
+    // 177.3 / 185.4.  Between 150 and 220 blocks of one product, where some SMs have two and most one, stages of 64: 200, 1024: 1 / 1.2 / 1.08.
+    const bool whole = Kd > 256 && 10 * Kd >= 9 * ((Kd + 127) / 128 * 128);
+    if (!tile_expert && Kd >= 256 && (blocks <= 48 || (whole && blocks <= 74)))
       return launch_f32<16, 16, 2, 4, 8, 128>(a, lda, b, ldb, b_expert_stride, M_max, N, Kd, tile_expert, num_m_tiles_dev, assign_of_row, epi, st);
-    if (Kd > 256) return launch_f32<32, 32, 4, 4, 8, 128>(a, lda, b, ldb, b_expert_stride, M_max, N, Kd, tile_expert, num_m_tiles_dev, assign_of_row, epi, st);
+    if (whole && blocks <= 290 && (tile_expert || blocks <= 148 || blocks >= 225))
+      return launch_f32<32, 32, 4, 4, 8, 128>(a, lda, b, ldb, b_expert_stride, M_max, N, Kd, tile_expert, num_m_tiles_dev, assign_of_row, epi, st);
     return launch_f32<32, 32, 4, 4, 4, 64>(a, lda, b, ldb, b_expert_stride, M_max, N, Kd, tile_expert, num_m_tiles_dev, assign_of_row, epi, st);
   }
   dim3 grid((M_max + BM - 1) / BM, (N + BN - 1) / BN);

@@ -219,7 +219,8 @@ cudaError_t launch_small_combine(const rom_config& c, const float* Bp, const flo
 cudaError_t launch_gemm_simt(int dtype, const void* A, int lda, const void* Bw, int ldb, int64_t b_expert_stride,
                              int M_max, int N, int Kd, const int32_t* tile_expert, const int32_t* num_m_tiles_dev,
                              const Epilogue& epi, cudaStream_t st,
-                             const int32_t* assign_of_row = nullptr /* grouped: row tiles that are all padding may be skipped */);
+                             const int32_t* assign_of_row = nullptr /* grouped: row tiles that are all padding may be skipped */,
+                             int n_rows = 0 /* grouped: rows that are not padding, of the M_max */);
 
 // Ungrouped GEMM for a few rows and a long K (M <= 128, Kd a multiple of 2048 for bf16 / 1024 for fp32): K split over
 // the threads of a block.

@@ -418,7 +418,7 @@ int rom_mamba2_layer_forward(const rom_config* cfg, int32_t headdim, const rom_m
   auto gemm = [&](const void* A_, int lda, const void* B_, int ldb, int64_t bstride, int Nn, int Kd, const Epilogue& ep) -> cudaError_t {
     if (tc) return launch_gemm_tc(A_, lda, B_, ldb, c.E, rows, Nn, Kd, tile_expert, num_m_tiles, ep, status, st, false, false,
                                   reinterpret_cast<const int32_t*>(W + lay.pad_offsets));
-    return launch_gemm_simt(c.dtype, A_, lda, B_, ldb, bstride, rows, Nn, Kd, tile_expert, num_m_tiles, ep, st);
+    return launch_gemm_simt(c.dtype, A_, lda, B_, ldb, bstride, rows, Nn, Kd, tile_expert, num_m_tiles, ep, st, nullptr, (int)lay.A);
   };
 
   ROM_CUDA(launch_route_gather(c, x, w->W_r, w->b_r, topk_idx_out, gates, counts_out, W, lay, st));
