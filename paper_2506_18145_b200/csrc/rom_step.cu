@@ -178,12 +178,19 @@ struct StepGemmArgs {
   int tile_rows;                        // step_tc: rows per weight tile
 };
 
-// ROUTE (the In Proj of one or two tokens, while all its blocks are resident at once): every block finds the experts itself, 32 KB of
-// router weights from the L2, which takes less than a launch and the tables in between; one more block writes the routing out for the
-// kernels to come.  With the window, taps and gate of a thread's output requested beside the weights and the tokens' operands of
+// ROUTE (the In Proj of one or two tokens, while all its blocks are resident at once and there are few logits): every block finds the
+// experts itself, 32 KB of router weights from the L2 with 8 experts, which takes less than a launch and the tables in between; one more
+// block writes the routing out for the kernels to come.  With the window, taps and gate of a thread's output requested beside the weights and the tokens' operands of
 // step_dt_scan beside delta_r: one token of 2048 channels 28.1 -> 23.1 us, of 1280 23.6 -> 20.0, top-2 of 16 experts 45.4 -> 41.6, two
 // tokens 37.0 -> 33.3 (routing inside without the limit on the blocks: 37.7 and 45.5 for the last two, second waves route again).
-constexpr int kRouteInside = 2;
+// Every block reads all E rows of the router for every token: us a step, launch of its own / inside: one token, 8 experts of 2048 channels
+// 21.0 / 19.4, 16 20.3 / 20.0, 24 21.8 / 22.0, 64 33.4 / 35.0; 64 of 1024 (one block an SM) 24.2 / 21.1, 64 of 1280 29.2 / 27.1, 64 of 1536 26.9 / 29.5; two
+// tokens, 4 of 1024 16.2 / 15.6, 8 of 512 13.2 / 13.1, 8 of 1024 15.4 / 15.6, 16 of 1024 18.2 / 19.2, 64 of 1024 25.2 / 34.4.
+bool route_inside_pays(int B, int K, int E, int Dm, int De, int num_sms) {
+  const int slots = B * K < E ? B * K : E;
+  if (B > 2 || (2 * De / 32 + 1) * slots > 2 * num_sms) return false;
+  return B == 1 ? Dm <= 1280 || E * Dm <= 24 * 1536 : E * Dm <= 4096;
+}
 template <int MODE, int RT, int WARPS, bool ROUTE = false>
 __global__ void __launch_bounds__(WARPS * 32, MODE == STEP_IN ? 2 : 1)
 step_gemm(const StepGemmArgs p, const RouteArgs rt) {
@@ -925,7 +932,7 @@ cudaError_t launch_step_small(const rom_config& c, const rom_weights& w, const v
   if (e != cudaSuccess) return e;
   const int slots = B * K < c.E ? B * K : c.E;      // selected experts at most
   // few assignments: latency counts, the register-fed kernel spreads them over more blocks; more: stream the weights
-  const bool stream = B * K >= kStreamMin, route_inside = !stream && B <= kRouteInside && (2 * De / 32 + 1) * slots <= 2 * num_sms;
+  const bool stream = B * K >= kStreamMin, route_inside = !stream && route_inside_pays(B, K, c.E, Dm, De, num_sms);
   if (!route_inside && (e = launch_chained(step_route, dim3(B), kRouteWarps * 32, st, false, rt)) != cudaSuccess) return e;
   StepGemmArgs a{};
   a.x = (const bf16*)x; a.ldx = Dm; a.W = (const bf16*)w.W_inz; a.Kd = Dm; a.n_rows = 2 * De;

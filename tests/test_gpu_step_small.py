@@ -39,6 +39,19 @@ def test_step_route_inside_the_projection(kw):
     run_steps(small_shape(**{**dict(L=4, dtype="bf16"), **kw}), 3)
 
 
+@pytest.mark.parametrize("B,E,K,d_model,launches", [
+    (1, 8, 1, 2048, 4), (1, 64, 1, 1280, 4), (1, 64, 1, 1344, 5), (1, 24, 1, 1600, 5), (2, 8, 1, 512, 4), (2, 8, 1, 576, 5), (2, 64, 1, 128, 5),
+])
+def test_step_routes_inside_only_few_logits(B, E, K, d_model, launches):
+    s = small_shape(B=B, L=1, E=E, K=K, d_model=d_model, d_inner=128, dtype="bf16")
+    p = synth.make_inputs(s, recipe="unit")
+    idx, gates = one_step(s, p, B)[3:5]
+    assert rb.last_launch_count() == launches
+    ref_idx, ref_gate, _, _ = O.route(np64(p["x"]).reshape(B, d_model), np64(p["W_r"]), np64(p["b_r"]), K, 0)
+    np.testing.assert_array_equal(idx.cpu().numpy(), ref_idx)
+    np.testing.assert_allclose(gates.cpu().numpy(), ref_gate, rtol=2e-6, atol=1e-30)
+
+
 def one_step(s, p, B, flags=0):
     """One token for the first B sequences of p from seeded states; (out, conv_state, ssm_state, idx, gates, workspace)."""
     cfg = rb.config_from_shape(s.replace(B=B, L=1), flags=flags)
