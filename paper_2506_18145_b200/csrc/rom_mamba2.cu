@@ -156,8 +156,10 @@ m2_conv_kernel(const T* __restrict__ ZXs, const T* __restrict__ w_conv, const fl
 // and the next four in flight, as the layer's conv does (rom_conv.cu).  HBM-bound; above, a thread loads 19 rows, computes and ends, so
 // that loads and arithmetic overlap only between blocks and every row is widened for each of its four taps.  (Channel groups and
 // segments share one index: 516 groups of 4096 channels would leave the last of five blocks nearly empty.)  16384 steps of 4096 channels:
-// 87 -> 69 us, whatever the steps to a thread (16, 32, 64) and with three blocks an SM as with four; used once its blocks give every
-// SM one.
+// 87 -> 69 us, whatever the steps to a thread (16, 32, 64) and with three blocks an SM as with four.  The line and the steps to a thread,
+// us of a layer (form above / 16 steps / 32): 136 blocks of 16 steps 84.6 / 87.8 / -, 264 124.6 / 126.4 / -, 320 92.3 / 87.3 / 95.4, 528
+// (264 of 32) 142.2 / 136.0 / 144.4, 1056 (528) 228.8 / 219.3 / 217.9: two blocks an SM at least, 32 steps (fewer rows read twice) once
+// that leaves three.
 __global__ void __launch_bounds__(128, 4)
 m2_conv_roll_kernel(const __nv_bfloat16* __restrict__ ZXs, const __nv_bfloat16* __restrict__ w_conv, const float* __restrict__ b_conv,
                     __nv_bfloat16* __restrict__ xc, float* __restrict__ Bm, float* __restrict__ Cm, int L, int De, int N, int W, int k,
@@ -440,9 +442,10 @@ int rom_mamba2_layer_forward(const rom_config* cfg, int32_t headdim, const rom_m
     float* Bm = reinterpret_cast<float*>(W + m.Bm);
     float* Cm = reinterpret_cast<float*>(W + m.Cm);
     const long long nv = Cs / vec;
-    const int seg = nv * c.B * ((c.L + 63) / 64) >= 148LL * 12 * 128 ? 64 : 32;
-    const long long walk_blocks = (nv * ((c.L + seg - 1) / seg) + 127) / 128;
-    if (bf && walk_blocks * c.B >= 148)
+    auto blocks_of = [&](int steps) { return (nv * ((c.L + steps - 1) / steps) + 127) / 128; };
+    const int seg = blocks_of(32) * c.B >= 3 * 148 ? 32 : 16;
+    const long long walk_blocks = blocks_of(seg);
+    if (bf && walk_blocks * c.B >= 2 * 148)
       launch_k(m2_conv_roll_kernel, dim3((unsigned)walk_blocks, c.B), 128, 0, st, (const __nv_bfloat16*)(W + m.ZXs), (const __nv_bfloat16*)w->w_conv, w->b_conv,
                                                                               (__nv_bfloat16*)(W + m.xc), Bm, Cm, c.L, De, N, Wd, c.d_conv, seg, status + kStatNonFinite);
     else if (bf) launch_k(m2_conv_kernel<__nv_bfloat16>, cgrid, 128, 0, st, (const __nv_bfloat16*)(W + m.ZXs), (const __nv_bfloat16*)w->w_conv, w->b_conv,

@@ -1,5 +1,5 @@
 """The walking form of the Mamba2-style block's conv (enough tokens that its threads fill the GPU), through the layer against the
-oracle: lengths that four and 32 steps do not divide, many sequences, every conv width; and its note of values that are not finite."""
+oracle: lengths that four, 16 and 32 steps do not divide, many sequences, every conv width, too few blocks for it; and its note of values that are not finite."""
 import pytest
 import torch
 
@@ -13,13 +13,15 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("kw,headdim", [
     (dict(B=1, L=9005, d_conv=3, K=1), 64), (dict(B=75, L=70, d_conv=2, K=2), 64), (dict(B=150, L=33, K=1), 32),
+    (dict(B=150, L=70, d_conv=2, K=2), 64), (dict(B=222, L=70, d_conv=3, K=1), 64),      # 450 blocks of 16 steps, 444 of 32
 ])
 def test_m2_conv_walk(kw, headdim):
     run_mamba2(m2shape(**{**dict(d_model=64, d_inner=512, E=2), **kw}), headdim)
 
 
-def test_m2_conv_walk_not_finite():
-    s = m2shape(B=75, L=70, d_model=64, d_inner=512, E=2, K=1)
+@pytest.mark.parametrize("B", [75, 150])
+def test_m2_conv_walk_not_finite(B):
+    s = m2shape(B=B, L=70, d_model=64, d_inner=512, E=2, K=1)
     b, at = 40, 38
     p = synth.make_mamba2_inputs(s, 64)
     p["W_in"][:, s.d_inner + 3:2 * s.d_inner:64, 0] = 4      # one channel of every head follows x[t, 0]
