@@ -184,12 +184,14 @@ x_proj_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant_
   }
 }
 
-// CTAs that share a tile: 8, 4 or 2 while all of them are resident together (clusters of up to eight CTAs fill 16 SMs of a GPC; 128 SMs
-// counted), 1: the general GEMM's kernel, whose tiles then have an SM each.
+// CTAs that share a tile: 8 up to 8 tiles, 4 up to 33, 2 up to 66, as long as each has four K blocks; 1: the general GEMM's kernel, whose tiles
+// then have an SM each.  us of a layer of 1024 channels, 8 / 4 / 2 / 1 CTAs: 4 tiles 97.9 / 98.4 / 99.7 / 102.6, 8 113.7 / 113.4 / 114.7 / 117.4,
+// 15 147.4 / 146.9 / 147.6 / 150.6, 16 (clusters of eight no longer all resident) 156.4 / 148.8 / 149.9 / 152.4, 33 - / 228.9 / 229.7 / 231.9,
+// 34 (nor those of four) - / 237.4 / 230.7 / 233.5, 66 - / - / 352.2 / 355.1.
 int x_proj_split(int M, int Kd) {
   const int tiles = (M + BLOCK_M - 1) / BLOCK_M, num_kb = (Kd + BLOCK_K - 1) / BLOCK_K;
   int S = 8;
-  while (S > 1 && (tiles * S > 132 || num_kb < 4 * S)) S >>= 1;
+  while (S > 1 && (tiles * S > (S == 8 ? 64 : 132) || num_kb < 4 * S)) S >>= 1;
   return S;
 }
 

@@ -1,5 +1,5 @@
 """x Proj of the tensor path against fp64 on the rows it was given: clusters of two, four and eight CTAs on both sides of their lines
-(16, 33 and 66 row tiles; 8, 16 and 32 K blocks), uneven shares of the contracted index, row and column counts that no tile divides, and
+(8, 33 and 66 row tiles; 8, 16 and 32 K blocks), uneven shares of the contracted index, row and column counts that no tile divides, and
 sizes that stay with the general GEMM."""
 import pytest
 import torch
@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("T,De,R", [
     (1, 2048, 16), (127, 2112, 128), (2048, 2048, 64), (2049, 1088, 48), (4200, 1024, 80), (4300, 512, 16), (8448, 576, 128), (8449, 576, 32),
-    (300, 448, 16), (130, 64, 16), (200, 1024, 144),
+    (300, 448, 16), (130, 64, 16), (200, 1024, 144), (1024, 2112, 48), (1025, 2048, 16),
 ])
 def test_x_proj(T, De, R):
     s = synth.RomShape("xp", 1, T, 64, De, 16, 4, R, 2, 1, "bf16", 8100 + De + R)
