@@ -405,7 +405,9 @@ dx_kernel(const T* __restrict__ dxp, const int32_t* __restrict__ row_of_assign, 
 // The same in bf16 for 4, 8 or 16 experts at top-1 and top-2: a thread keeps its 8 columns of W_r and walks seg tokens, four in flight
 // (their row indices four tokens earlier still).  Above, every vector of dx reads and widens all E of W_r, about 170 instructions: 16384
 // tokens of 2048 channels with 8 experts 58 us, here 38 (20 at the copy bandwidth), 4113 of 1024 at top-2 11.6 -> 8.9.  Eight tokens to a
-// thread: with 16 and 32 the former takes 36 and 35, the latter 11.6 and 19.9 (too few threads).
+// thread: with 16 and 32 the former takes 36 and 35, the latter 11.6 and 19.9 (too few threads).  Other counts in the next larger form, with
+// zero rows of W_r, gain nothing (whole backward of 8192 tokens of 768 channels, 6 experts: 831.5 us above, 831.2 padded; top-2 979 / 987; 12
+// experts 863 / 862): their dlogit rows are no longer 16-byte pieces.
 template <int NE, int KT>
 __global__ void __launch_bounds__(128, NE <= 8 ? 4 : 2)
 dx_walk_kernel(const __nv_bfloat16* __restrict__ dxp, const int32_t* __restrict__ row_of_assign, const float* __restrict__ dlogit,
