@@ -116,8 +116,10 @@ inline void count_launch() { LaunchCounter::count++; }
 
 // ---------------------------------------------------------------- launches
 // Programmatic dependent launch: a kernel launched by launch_k may become resident while the one before it on the stream drains; it
-// waits (pdl_wait: the predecessor is complete and its writes are visible) before it touches memory, and only then lets its own
-// successor in (pdl_trigger), so every earlier kernel is complete too.  About 1.5 us less between two launches (41 launches of a
+// waits (pdl_wait: the predecessor is complete and its writes are visible) before it reads what that one may write or writes anything,
+// and only then lets its own successor in (pdl_trigger), so every kernel before the predecessor is complete as it starts.  Some read before
+// they wait: the weights (and bias) of the x Proj and dt Proj kernels and of the single-token step, the step's states and gates; the
+// launch just before such a kernel must not write those.  About 1.5 us less between two launches (41 launches of a
 // small backward pass: 60 us of gaps).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -227,6 +229,8 @@ cudaError_t launch_gemm_simt(int dtype, const void* A, int lda, const void* Bw, 
 cudaError_t launch_gemm_skinny(int dtype, const void* A, int lda, const void* Bw, int ldb, int M, int N, int Kd,
                                const Epilogue& epi, cudaStream_t st);
 
+// EPI_XPROJ and EPI_SOFTPLUS products may go to the two kernels below, which read Bw and epi.bias before the launch just before them on the
+// stream has ended: that launch must not write them.
 // b_mn: B is [n_experts * Kd, N] with N contiguous (ldb its row pitch), i.e. C = A * B[e] instead of A * B[e]^T (a data gradient
 // on the weights as stored).
 cudaError_t launch_gemm_tc(const void* A, int lda, const void* Bw, int ldb, int n_experts,
@@ -235,11 +239,12 @@ cudaError_t launch_gemm_tc(const void* A, int lda, const void* Bw, int ldb, int 
                            const int32_t* pad_offsets = nullptr /* grouped: the padded segment offsets (n_experts + 1); allows CTA pairs */);
 
 // x Proj of few tokens, the contracted index shared by a cluster (rom_x_proj.cu): C = A[M, Kd] Bw[N, Kd]^T split into delta | B | C; bf16.
+// Bw: not written by the launch just before on the stream.
 bool x_proj_applicable(int M, int N, int Kd);
 cudaError_t launch_x_proj(const void* A, const void* Bw, int M, int N, int Kd, const Epilogue& epi, int32_t* status, cudaStream_t st, bool test_stall);
 
 // dt Proj with a short contraction (rom_dt_proj.cu): C[M, N] = softplus(A[M, Kd] Bw[N, Kd]^T + bias), rows contiguous; bf16.  Its kernel lets
-// the next one in only as its blocks end (a scan's blocks must not pile up).
+// the next one in only as its blocks end (a scan's blocks must not pile up).  Bw, bias: not written by the launch just before on the stream.
 bool dt_proj_applicable(int N, int Kd);
 cudaError_t launch_dt_proj(const void* A, const void* Bw, int M, int N, int Kd, const Epilogue& epi, int32_t* status, cudaStream_t st, bool test_stall);
 
