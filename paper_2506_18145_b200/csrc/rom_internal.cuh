@@ -52,19 +52,22 @@ inline int scan_chunks(int B, int De, int L) {
 // block takes 139 / 192 / 272 ns a step with one / two / three blocks on an SM (three fit), 115 / 161 / 230 ns state-only; more than
 // one chunk costs the state-only launch and about 7 us for the chained states and the extra launch.  Chunks of at least 48 steps.  A
 // function of the problem sizes only (148 SMs assumed), so that workspace sizing and the launch agree.
-inline int scan_warp_chunks(int B, int De, int L) {
+inline double scan_warp_time(int B, int De, int L, int n) {      // ns
   const long long blocks1 = (long long)B * ((De + 127) / 128);
   auto pace = [](long long blocks, const double (&ns)[3]) {
     const long long k = (blocks + 147) / 148;
     return k <= 3 ? ns[k - 1] : ns[2] * (double)k / 3.0;
   };
   const double full[3] = {139.0, 192.0, 272.0}, state[3] = {115.0, 161.0, 230.0};
+  if (n == 1) return (double)L * pace(blocks1, full);
+  return (double)L / (n - 0.3) * (pace(blocks1 * (n - 1), full) + pace(blocks1 * (n - 1), state)) + 7000.0;
+}
+inline int scan_warp_chunks(int B, int De, int L) {
   int best = 1;
-  double best_t = (double)L * pace(blocks1, full);
+  double best_t = scan_warp_time(B, De, L, 1);
   for (int n = 2; n <= 64 && L >= 48 * n; ++n) {
-    const long long blocks = blocks1 * (n - 1);
-    if (blocks > 148 * 12) break;
-    const double t = (double)L / (n - 0.3) * (pace(blocks, full) + pace(blocks, state)) + 7000.0;
+    if ((long long)B * ((De + 127) / 128) * (n - 1) > 148 * 12) break;
+    const double t = scan_warp_time(B, De, L, n);
     if (t < best_t) { best_t = t; best = n; }
   }
   return best;

@@ -537,6 +537,18 @@ bool f32_one_launch(int B, int De, int L, int nch, bool zoh, int num_sms) {
   return 1500.0 + (double)align_up((size_t)L, round) * k * (zoh ? (k <= 4 ? 21.2 : 20.0) : (k <= 4 ? 14.7 : 13.2)) <= general;
 }
 
+// Whether the one-launch form of the warp kernel (rom_scan_ring.cu) takes a scan that would be cut into nch chunks: by the time of the two in a
+// model of their measured paces.  One launch: rounds of 148 blocks of 32 channels, 35.8 ns a step (31.2 with B-bar = Delta B), 4.4 us a round
+// and 4.4 once; chunked: scan_warp_chunks' model, which leaves out what grows with the chunks (measured 5 to 33 us above it).  At 95 measured
+// sizes of 32 to 2048 blocks and 100 to 16384 steps it names the faster form but for those where the two differ by less than 1.5 %.
+// us, chunked / one launch: 128 blocks of 1000 steps 59 / 44, 4096 171 / 155, 16384 618 / 588; 256 of 2048 171 / 159; 288 of 4000 327 / 296;
+// 64 of 16384 335 / 587; 160 of 4096 196 / 304; 512 of 2048 282 / 313.  Delta B: 128 of 16384 597 / 512, 256 of 8192 582 / 520.
+bool scan_ring_pays(int B, int De, int L, int nch, bool zoh) {
+  const long long rounds = ((long long)B * (De / 32) + 147) / 148;
+  const double ring = (double)rounds * ((double)L * (zoh ? 35.8 : 31.2) + 4400.0) + 4400.0;
+  return ring <= (zoh ? 1.03 : 1.0) * scan_warp_time(B, De, L, nch) + 1000.0 + (nch < 11 ? 1200.0 * nch : 13000.0);
+}
+
 // CKPT: also store the checkpoints of the backward pass.
 template <typename T, typename TD, bool PRECISE, bool CKPT = false>
 cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const float* h0, float* h_last,
@@ -559,6 +571,12 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
   if (PRECISE && !a.scalar_a && f32_one_launch(c.B, c.d_inner, c.L, nch, zoh, num_sms)) {
     a.h0 = h0; a.h_last = h_last;
     return launch_scan_f32(a, c.B, zoh, CKPT, st);
+  }
+  if constexpr (!PRECISE) {
+    if (warp_kernel && nch > 1 && scan_ring_pays(c.B, c.d_inner, c.L, nch, zoh)) {
+      a.h0 = h0; a.h_last = h_last;
+      return launch_scan_ring(a, c.B, zoh, sizeof(TD) == 4, CKPT, st);
+    }
   }
   // one launch over `grid_z` chunks with 8 states per thread (chunked) or the warp kernel
   auto chunks = [&](const ScanArgs& x, int grid_z, auto mode) -> cudaError_t {

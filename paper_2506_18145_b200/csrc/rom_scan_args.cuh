@@ -40,6 +40,9 @@ enum ScanMode : int { SCAN_FULL = 0, SCAN_STATE = 1, SCAN_FIRST = 2, SCAN_CKPT =
 // rom_scan_warp.cu: bf16 storage, A per channel and state.  grid_z chunks per sequence from a.chunk_off on.
 cudaError_t launch_scan_warp(const ScanArgs& a, int B, int grid_z, bool zoh, bool delta_fp32, ScanMode mode, cudaStream_t st);
 
+// rom_scan_ring.cu: the whole scan in one launch; bf16 storage, A per channel and state.  ckpt: with checkpoints (delta in bf16).
+cudaError_t launch_scan_ring(const ScanArgs& a, int B, bool zoh, bool delta_fp32, bool ckpt, cudaStream_t st);
+
 // rom_scan_f32.cu: the whole scan in one launch; fp32 storage, A per channel and state.
 cudaError_t launch_scan_f32(const ScanArgs& a, int B, bool zoh, bool ckpt, cudaStream_t st);
 
