@@ -174,7 +174,8 @@ route_offsets(int32_t* __restrict__ chunk_counts, int n_chunks, int E, const Off
 // from global memory) and 4 consecutive fp64 weights of one expert (L1/L2-resident copy); MMA j of the step
 // contracts elements {j, 4+j, 8+j, 12+j} of the 16.  No shared memory until the logits meet for the top-K.
 // OWN: for route_scatter_gather<true> (no ticket).
-template <typename T, bool OWN>
+// NTW: 8-expert tiles to a warp, which widens an x row once for all of them (it is what a warp reads and converts most).
+template <typename T, bool OWN, int NTW>
 __global__ void __launch_bounds__(512)
 route_logits_topk(const T* __restrict__ x, const T* __restrict__ W_r, const float* __restrict__ b_r,
                   int T_tokens, int Dm, int E, int K, int gate_mode,
@@ -182,8 +183,9 @@ route_logits_topk(const T* __restrict__ x, const T* __restrict__ W_r, const floa
                   int32_t* __restrict__ chunk_counts, double* __restrict__ chunk_prob, float* __restrict__ probs, int n_chunks, const OffsetsArgs oa) {
   pdl_sync();
   extern __shared__ __align__(16) unsigned char smem[];
-  const int Epad = (E + NT8 - 1) / NT8 * NT8;
-  const int n_wtiles = Epad / NT8;
+  constexpr int WE = NTW * NT8;                                    // experts per warp
+  const int Epad = (E + WE - 1) / WE * WE;
+  const int n_wtiles = Epad / WE;
   const int dsplit = (blockDim.x >> 5) / n_wtiles;                 // warps that share one expert tile, each on its own d range
   double* lg = reinterpret_cast<double*>(smem);                    // [dsplit][RT][Epad] partial logits; [0] becomes the sum
   int32_t* idx_s = reinterpret_cast<int32_t*>(lg + max(dsplit, 2) * RT * Epad);   // [RT][K] (later: scratch of the offsets scan)
@@ -195,23 +197,30 @@ route_logits_topk(const T* __restrict__ x, const T* __restrict__ W_r, const floa
   const int gq = lane >> 2, t4 = lane & 3;                        // fragment row / column group of this lane
   const int t0 = blockIdx.x * RT;
 
-  // accumulators: 4 tiles of 8 tokens x this warp's 8 experts; lane holds (token 8*mt + gq, experts 2*t4, 2*t4+1)
-  double acc[4][2];
+  // accumulators: 4 tiles of 8 tokens x this warp's tiles of 8 experts; lane holds (token 8*mt + gq, experts 2*t4, 2*t4+1)
+  double acc[NTW][4][2];
 #pragma unroll
-  for (int mt = 0; mt < 4; ++mt) {
+  for (int n = 0; n < NTW; ++n)
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int ee = w * NT8 + 2 * t4 + i;
-      acc[mt][i] = (b_r != nullptr && ee < E && dq == 0) ? (double)b_r[ee] : 0.0;
-    }
-  }
+    for (int mt = 0; mt < 4; ++mt)
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int ee = w * WE + n * NT8 + 2 * t4 + i;
+        acc[n][mt][i] = (b_r != nullptr && ee < E && dq == 0) ? (double)b_r[ee] : 0.0;
+      }
   const T* xrow[4];
 #pragma unroll
   for (int mt = 0; mt < 4; ++mt) xrow[mt] = x + (size_t)min(t0 + 8 * mt + gq, T_tokens - 1) * Dm + 4 * t4;   // rows past the end repeat the last token
-  // weights: 4 consecutive d of expert 8w + gq, read in the storage type and widened on use (exact); experts beyond E
+  // weights: 4 consecutive d of an expert, read in the storage type and widened on use (exact); experts beyond E
   // (padding of the 8-expert tile) read expert E-1 and are zeroed
-  const bool w_ok = w * NT8 + gq < E;
-  const T* wrow = W_r + (size_t)min(w * NT8 + gq, E - 1) * Dm + 4 * t4;
+  bool w_ok[NTW];
+  const T* wrow[NTW];
+#pragma unroll
+  for (int n = 0; n < NTW; ++n) {
+    const int ee = w * WE + n * NT8 + gq;
+    w_ok[n] = ee < E;
+    wrow[n] = W_r + (size_t)min(ee, E - 1) * Dm + 4 * t4;
+  }
 
   if (OWN && blockIdx.x == 0 && tid < kStatusInts) oa.status[tid] = 0;
   // the row -> assignment table starts at -1 everywhere (padding rows keep it); the whole grid clears it
@@ -219,13 +228,14 @@ route_logits_topk(const T* __restrict__ x, const T* __restrict__ W_r, const floa
 
   // operands of the next PF-1 steps are in flight (raw, unconverted) while one step is contracted
   // (d_model is a multiple of 64, so there are at least PF steps)
-  constexpr int PF = 4;
+  constexpr int PF = NTW == 1 ? 4 : 3;
   RawX4<T> rx[PF][4];
-  RawX4<T> rw[PF];
-  auto fetch = [&](int d, RawX4<T> (&xo)[4], RawX4<T>& wo) {
+  RawX4<T> rw[PF][NTW];
+  auto fetch = [&](int d, RawX4<T> (&xo)[4], RawX4<T> (&wo)[NTW]) {
 #pragma unroll
     for (int mt = 0; mt < 4; ++mt) xo[mt].load(xrow[mt] + d);
-    wo.load(wrow + d);
+#pragma unroll
+    for (int n = 0; n < NTW; ++n) wo[n].load(wrow[n] + d);
   };
 #pragma unroll
   for (int i = 0; i < PF - 1; ++i)
@@ -236,24 +246,31 @@ route_logits_topk(const T* __restrict__ x, const T* __restrict__ W_r, const floa
       if (d0 + 16 * i >= d_hi) break;
       const int dn = d0 + 16 * (i + PF - 1);                              // step that enters the ring now
       if (dn < d_hi) fetch(dn, rx[(i + PF - 1) % PF], rw[(i + PF - 1) % PF]);
-      double wb[4];
-      rw[i].get(wb);
-      if (!w_ok) { wb[0] = 0.0; wb[1] = 0.0; wb[2] = 0.0; wb[3] = 0.0; }
+      double wb[NTW][4];
+#pragma unroll
+      for (int n = 0; n < NTW; ++n) {
+        rw[i][n].get(wb[n]);
+        if (!w_ok[n]) { wb[n][0] = 0.0; wb[n][1] = 0.0; wb[n][2] = 0.0; wb[n][3] = 0.0; }
+      }
       double xa[4][4];
 #pragma unroll
       for (int mt = 0; mt < 4; ++mt) rx[i][mt].get(xa[mt]);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
 #pragma unroll
-        for (int mt = 0; mt < 4; ++mt) dmma_m8n8k4(acc[mt], xa[mt][j], wb[j]);
+        for (int mt = 0; mt < 4; ++mt)
+#pragma unroll
+          for (int n = 0; n < NTW; ++n) dmma_m8n8k4(acc[n][mt], xa[mt][j], wb[n][j]);
       }
     }
   }
 #pragma unroll
-  for (int mt = 0; mt < 4; ++mt) {
-    lg[(dq * RT + 8 * mt + gq) * Epad + w * NT8 + 2 * t4] = acc[mt][0];
-    lg[(dq * RT + 8 * mt + gq) * Epad + w * NT8 + 2 * t4 + 1] = acc[mt][1];
-  }
+  for (int n = 0; n < NTW; ++n)
+#pragma unroll
+    for (int mt = 0; mt < 4; ++mt) {
+      lg[(dq * RT + 8 * mt + gq) * Epad + w * WE + n * NT8 + 2 * t4] = acc[n][mt][0];
+      lg[(dq * RT + 8 * mt + gq) * Epad + w * WE + n * NT8 + 2 * t4 + 1] = acc[n][mt][1];
+    }
   __syncthreads();
 
   // the d ranges are added in a fixed order, the same for every expert
@@ -611,15 +628,17 @@ cudaError_t launch_route_stats(const rom_config& c, const void* x, const void* W
   int32_t* chunk_counts = reinterpret_cast<int32_t*>(ws + lay.chunk_counts);
   int32_t* assign_of_row = reinterpret_cast<int32_t*>(ws + lay.assign_of_row);
 
-  const int n_wtiles = (c.E + NT8 - 1) / NT8;
-  const int Epad8 = n_wtiles * NT8;
-  // warps per chunk: one per 8-expert tile, times a split of d_model that puts more loads in flight: up to 4 ranges,
-  // up to 16 when there are too few chunks to fill the GPU (a handful of tokens: latency is all that matters)
-  const int blocks = (T + RT - 1) / RT;
-  int dsplit = blocks < 148 ? 16 : 4;
-  while (dsplit > 1 && (n_wtiles * dsplit > 16 || c.d_model / 16 < 4 * dsplit)) dsplit >>= 1;
-  const int threads = 32 * n_wtiles * dsplit;
   const bool bf = c.dtype == ROM_BF16;
+  // 8-expert tiles to a warp: 32768 tokens of 2048, 16 experts 131 -> 115 us (fp32 rows take twice the registers: one)
+  const int ntw = bf && c.E > NT8 ? 2 : 1;
+  const int n_wtiles = (c.E + ntw * NT8 - 1) / (ntw * NT8);
+  const int Epad8 = n_wtiles * ntw * NT8;
+  // warps per chunk: one per tile of experts, times a split of d_model that puts more loads in flight: up to 4 ranges, 8 while two blocks of
+  // that size an SM hold all of them (8192 tokens of 1024, 8 experts 18.3 -> 16.3 us), up to 16 when there are too few chunks to fill the GPU (a handful of tokens: latency is all that matters)
+  const int blocks = (T + RT - 1) / RT;
+  int dsplit = blocks < 148 ? 16 : blocks <= 296 ? 8 : 4;
+  while (dsplit > 1 && (n_wtiles * ntw * dsplit > 16 || c.d_model / 16 < 4 * dsplit)) dsplit >>= 1;
+  const int threads = 32 * n_wtiles * dsplit;
   int32_t* status = reinterpret_cast<int32_t*>(ws + lay.status);
   const bool own = gather_x && route_own_bases(lay);
   const OffsetsArgs oa{reinterpret_cast<int32_t*>(ws + lay.counts), reinterpret_cast<int32_t*>(ws + lay.offsets),
@@ -629,11 +648,12 @@ cudaError_t launch_route_stats(const rom_config& c, const void* x, const void* W
   const int idx_ints = RT * c.K > 3 * kMaxE + 2 ? RT * c.K : 3 * kMaxE + 2;
   const size_t smem = sizeof(double) * (size_t)(dsplit > 2 ? dsplit : 2) * RT * Epad8 + sizeof(int32_t) * idx_ints;
   if (bf)
-    launch_k(own ? route_logits_topk<__nv_bfloat16, true> : route_logits_topk<__nv_bfloat16, false>, blocks, threads, smem, st, 
+    launch_k(ntw == 1 ? (own ? route_logits_topk<__nv_bfloat16, true, 1> : route_logits_topk<__nv_bfloat16, false, 1>)
+                      : (own ? route_logits_topk<__nv_bfloat16, true, 2> : route_logits_topk<__nv_bfloat16, false, 2>), blocks, threads, smem, st,
         (const __nv_bfloat16*)x, (const __nv_bfloat16*)W_r, b_r, T, c.d_model, c.E, c.K, c.gate_mode, idx_ws, gates, chunk_counts,
         chunk_prob, probs, (int)lay.n_chunks, oa);
   else
-    launch_k(own ? route_logits_topk<float, true> : route_logits_topk<float, false>, blocks, threads, smem, st, 
+    launch_k(own ? route_logits_topk<float, true, 1> : route_logits_topk<float, false, 1>, blocks, threads, smem, st, 
         (const float*)x, (const float*)W_r, b_r, T, c.d_model, c.E, c.K, c.gate_mode, idx_ws, gates, chunk_counts, chunk_prob, probs,
         (int)lay.n_chunks, oa);
   count_launch();
