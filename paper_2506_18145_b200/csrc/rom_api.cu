@@ -421,10 +421,10 @@ int layer_forward_impl(const rom_config* cfg, const rom_weights* w, const void* 
                        reinterpret_cast<float*>(W + lay.scan_ws), !slots, st, false, nullptr,
                        tc && !fused_small && c.small_proj_experts <= 1 && dt_proj_applicable(De, R)));
   ROM_STAGE_DONE();
-  // S10 + S11.  Tensor path with one expert per token: the epilogue of the grouped Out Proj scales each row by
+  // S10 + S11.  Tensor path or fp32, one expert per token: the epilogue of the grouped Out Proj scales each row by
   // its gate and writes it at its token's position (no intermediate rows, no combine pass).  Otherwise: grouped
   // Out Proj into expert-order rows, then the gate-weighted sum over the K slots.
-  const bool fused_out = tc && c.K == 1;
+  const bool fused_out = (tc || c.dtype == ROM_F32) && c.K == 1;
   if (fused_out) {
     Epilogue e_out{EPI_OUTPROJ, out, Dm, nullptr, nullptr, nullptr, 0, 0, reinterpret_cast<const int32_t*>(W + lay.assign_of_row), gates};
     ROM_CUDA(gemm(W + lay.Ygp, De, w->W_out, De, c.E, (int64_t)Dm * De, (int)lay.rows_max, Dm, De, tile_expert, num_m_tiles, e_out));

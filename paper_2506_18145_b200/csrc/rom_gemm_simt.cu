@@ -36,6 +36,11 @@ __device__ __forceinline__ void epi_store_scalar(const Epilogue& ep, int m, int 
       else if (n < ep.R + ep.N) ep.Bm[(size_t)m * ep.N + (n - ep.R)] = v;
       else ep.Cm[(size_t)m * ep.N + (n - ep.R - ep.N)] = v;
       break;
+    case EPI_OUTPROJ: {      // (fp32, top-1: no pass for the combine)
+      const int t = __ldg(ep.row_token + m);
+      if (t >= 0) reinterpret_cast<T*>(ep.C)[(size_t)t * ep.ldc + n] = from_f32<T>(fmaf(__ldg(ep.row_scale + t), v, 0.0f));
+      break;
+    }
     case EPI_F32:
       reinterpret_cast<float*>(ep.C)[(size_t)m * ep.ldc + n] = v;
       break;

@@ -161,7 +161,7 @@ enum EpiMode : int {
   EPI_INPROJ = 3,     // C[m, n] = acc for n < R (Conv Proj), SiLU(acc) for n >= R (Gate Proj)   (dtype); with row_token
                       // (tensor path, top-1) row m is written at row row_token[m], i.e. back in token order
   EPI_OUTPROJ = 4,    // top-1 combine fused: C[row_token[m], n] = row_scale[row_token[m]] * acc; rows with
-                      // row_token[m] < 0 (segment padding) are skipped   (dtype; tensor path only)
+                      // row_token[m] < 0 (segment padding) are skipped   (dtype; tensor path and fp32)
   EPI_F32 = 5,        // C[m, n] = acc                          (fp32)
   EPI_SWIGLU = 6,     // C[m, j] = SiLU(acc[m, j]) * acc[m, N + j], j < N: B holds, per expert, N "gate" rows then N "up"
                       // rows; N % 128 == 0   (dtype; tensor path only)
