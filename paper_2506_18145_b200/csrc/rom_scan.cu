@@ -538,14 +538,14 @@ bool f32_one_launch(int B, int De, int L, int nch, bool zoh, int num_sms) {
 }
 
 // Whether the one-launch form of the warp kernel (rom_scan_ring.cu) takes a scan that would be cut into nch chunks: by the time of the two in a
-// model of their measured paces.  One launch: rounds of 148 blocks of 32 channels, 35.8 ns a step (31.2 with B-bar = Delta B), 4.4 us a round
+// model of their measured paces.  One launch: rounds of 148 blocks of 32 channels, 33.3 ns a step (31.2 with B-bar = Delta B), 4.4 us a round
 // and 4.4 once; chunked: scan_warp_chunks' model, which leaves out what grows with the chunks (measured 5 to 33 us above it).  At 95 measured
-// sizes of 32 to 2048 blocks and 100 to 16384 steps it names the faster form but for those where the two differ by less than 1.5 %.
-// us, chunked / one launch: 128 blocks of 1000 steps 59 / 44, 4096 171 / 155, 16384 618 / 588; 256 of 2048 171 / 159; 288 of 4000 327 / 296;
-// 64 of 16384 335 / 587; 160 of 4096 196 / 304; 512 of 2048 282 / 313.  Delta B: 128 of 16384 597 / 512, 256 of 8192 582 / 520.
+// sizes of 32 to 2048 blocks and 100 to 16384 steps it names the faster form but for those where the two differ by less than 3 %.
+// us, chunked / one launch: 128 blocks of 1000 steps 59 / 42, 4096 171 / 147, 16384 618 / 553; 256 of 2048 171 / 151; 288 of 4000 327 / 280;
+// 64 of 16384 335 / 547; 160 of 4096 196 / 285; 512 of 2048 282 / 295.  Delta B: 128 of 16384 597 / 508, 256 of 8192 582 / 515.
 bool scan_ring_pays(int B, int De, int L, int nch, bool zoh) {
   const long long rounds = ((long long)B * (De / 32) + 147) / 148;
-  const double ring = (double)rounds * ((double)L * (zoh ? 35.8 : 31.2) + 4400.0) + 4400.0;
+  const double ring = (double)rounds * ((double)L * (zoh ? 33.3 : 31.2) + 4400.0) + 4400.0;
   return ring <= (zoh ? 1.03 : 1.0) * scan_warp_time(B, De, L, nch) + 1000.0 + (nch < 11 ? 1200.0 * nch : 13000.0);
 }
 

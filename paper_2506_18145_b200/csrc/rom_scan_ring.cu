@@ -8,11 +8,12 @@
 // running product of the decays: 16 values a lane and step, which registers cannot hold for eight steps.  They go to tensor memory (128
 // columns a warp; no matrix instruction runs).  The state then comes from the warp before, P h + E goes on to the next warp at once, and
 // one multiply-add an update brings the outputs up to date; nothing of that depends on the step before.
-// Measured (layer's operands): 16384 steps of 4096 channels 593 -> 551 us, 4 x 2048 of 2048 170 -> 155, 3 x 1017 of 3072 (two Gate rows
-// a token) 103 -> 90.  What bounds it: issue (69 % where an SM has two blocks' work) and the fp32 pipe (nine operations an update).
-// Tried: decays and inputs both in tensor memory with eight warps of 255 registers (seven operations, but two warps a scheduler: 161 us
-// at 4 x 2048); that with the second sweep beside the next tile's first (200); decays alone in tensor memory and the inputs formed twice
-// with sixteen warps (163).
+// Measured in the layer: 4 x 2048 steps of 2048 channels 170 -> 152 us, 16384 of 4096 593 -> 545; as rom_scan 3 x 1017 of 3072 95 -> 82.  What
+// bounds it: issue (10.2 instructions an update at up to 69 %), the fp32 pipe (nine operations of an update) and latency: twelve warps an SM.
+// Tried (us of a layer of 4 x 2048 steps of 2048 channels; this form 300, in chunks 317): decays and inputs both in tensor memory with eight
+// warps of 255 registers (seven operations, but two warps a scheduler) 309, that with the second sweep beside the next tile's first 352;
+// decays alone and the inputs formed twice, sixteen warps 317; B and C twice in shared memory for the packed pairs 319; Delta and u staged
+// as bf16 307; the outputs from the zero state in tensor memory as well 315; the carry in the layout of the registers 309 (spills).
 #include <type_traits>
 
 #include "rom_scan_args.cuh"
@@ -195,7 +196,7 @@ scan_ring_kernel(const ScanArgs p) {
               E[k] = r == 0 ? uB : __ffma2_rn(a, E[k], uB);
             }
             P[k] = r == 0 ? a : __fmul2_rn(P[k], a);
-            cp[k] = __fmul2_rn(dup(cc[n]), P[k]);
+            cp[k] = make_float2(cc[n] * P[k].x, cc[n] * P[k].y);      // (single: a packed product takes two moves into the store's registers)
             acc[j] = n == 0 ? __fmul2_rn(dup(cc[n]), E[k]) : __ffma2_rn(dup(cc[n]), E[k], acc[j]);
           }
         s.y[r][ysw(lane, r)] = make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y);
@@ -254,11 +255,14 @@ scan_ring_kernel(const ScanArgs p) {
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
           const int r = 2 * r2 + i;
-          const float4 y4 = s.y[r][ysw(lane, r)];
-          float2 acc[2] = {make_float2(y4.x, y4.y), make_float2(y4.z, y4.w)};
+          float4 y4 = s.y[r][ysw(lane, r)];
+          const float* vr = v[r2 & 1] + 16 * i;
 #pragma unroll
-          for (int k = 0; k < 8; ++k) acc[k & 1] = __ffma2_rn(make_float2(v[r2 & 1][16 * i + 2 * k], v[r2 & 1][16 * i + 2 * k + 1]), h[k], acc[k & 1]);
-          s.y[r][ysw(lane, r)] = make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y);
+          for (int n = 0; n < 4; ++n) {      // (single, for the same reason)
+            y4.x = fmaf(vr[4 * n], h[2 * n].x, y4.x); y4.y = fmaf(vr[4 * n + 1], h[2 * n].y, y4.y);
+            y4.z = fmaf(vr[4 * n + 2], h[2 * n + 1].x, y4.z); y4.w = fmaf(vr[4 * n + 3], h[2 * n + 1].y, y4.w);
+          }
+          s.y[r][ysw(lane, r)] = y4;
         }
       }
     }
