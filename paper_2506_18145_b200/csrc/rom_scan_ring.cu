@@ -9,7 +9,7 @@
 // columns a warp; no matrix instruction runs).  The state then comes from the warp before, P h + E goes on to the next warp at once, and
 // one multiply-add an update brings the outputs up to date; nothing of that depends on the step before.
 // Measured in the layer: 4 x 2048 steps of 2048 channels 170 -> 152 us, 16384 of 4096 593 -> 545; as rom_scan 3 x 1017 of 3072 95 -> 82.  What
-// bounds it: issue (10.2 instructions an update at up to 69 %), the fp32 pipe (nine operations of an update) and latency: twelve warps an SM.
+// bounds it: issue (9.8 instructions an update at up to 69 %), the fp32 pipe (nine operations of an update) and latency: twelve warps an SM.
 // Tried (us of a layer of 4 x 2048 steps of 2048 channels; this form 300, in chunks 317): decays and inputs both in tensor memory with eight
 // warps of 255 registers (seven operations, but two warps a scheduler) 309, that with the second sweep beside the next tile's first 352;
 // decays alone and the inputs formed twice, sixteen warps 317; B and C twice in shared memory for the packed pairs 319; Delta and u staged
@@ -196,7 +196,7 @@ scan_ring_kernel(const ScanArgs p) {
               E[k] = r == 0 ? uB : __ffma2_rn(a, E[k], uB);
             }
             P[k] = r == 0 ? a : __fmul2_rn(P[k], a);
-            cp[k] = make_float2(cc[n] * P[k].x, cc[n] * P[k].y);      // (single: a packed product takes two moves into the store's registers)
+            cp[k] = __fmul2_rn(dup(cc[n]), P[k]);
             acc[j] = n == 0 ? __fmul2_rn(dup(cc[n]), E[k]) : __ffma2_rn(dup(cc[n]), E[k], acc[j]);
           }
         s.y[r][ysw(lane, r)] = make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y);
@@ -258,7 +258,7 @@ scan_ring_kernel(const ScanArgs p) {
           float4 y4 = s.y[r][ysw(lane, r)];
           const float* vr = v[r2 & 1] + 16 * i;
 #pragma unroll
-          for (int n = 0; n < 4; ++n) {      // (single, for the same reason)
+          for (int n = 0; n < 4; ++n) {      // (single: the values of the load take two moves into the pair of a packed sum)
             y4.x = fmaf(vr[4 * n], h[2 * n].x, y4.x); y4.y = fmaf(vr[4 * n + 1], h[2 * n].y, y4.y);
             y4.z = fmaf(vr[4 * n + 2], h[2 * n + 1].x, y4.z); y4.w = fmaf(vr[4 * n + 3], h[2 * n + 1].y, y4.w);
           }
