@@ -392,8 +392,7 @@ __device__ __forceinline__ void scatter_chunk(const int32_t* __restrict__ topk_i
     const int pr = pad_offsets[e] + within;
     if (perm) perm[r] = a;
     if (inv_perm) inv_perm[a] = r;
-    row_of_assign[a] = pr;
-    assign_of_row[pr] = a;
+    if (row_of_assign) { row_of_assign[a] = pr; assign_of_row[pr] = a; }
     my_row[k] = pr;
   }
 }
@@ -413,8 +412,8 @@ route_scatter(const int32_t* __restrict__ topk_idx, const int32_t* __restrict__ 
   scatter_chunk(topk_idx, chunk_base + (size_t)chunk * E, offsets, pad_offsets, T_tokens, E, K, chunk, lane, perm, inv_perm, row_of_assign, assign_of_row, my_row);
 }
 
-// One block of 8 warps per chunk of 32 tokens: warp 0 builds the chunk's table entries, then every warp copies the rows
-// of four of the chunk's tokens to their padded rows (x_perm, the operand of the grouped Conv/Gate projection; x was read
+// `parts` (1, 2 or 4) blocks of 8 warps per chunk of 32 tokens: warp 0 finds the chunk's table entries (the first block writes them), then every warp
+// copies the rows of four (two, one) of the chunk's tokens to their padded rows (x_perm, the operand of the grouped Conv/Gate projection; x was read
 // by the router a moment ago and is still in L2), and the grid zero-fills the padding rows of every expert segment.
 // OWN: every block adds up the histograms (by expert) itself and the last one writes the offsets out for the kernels to come: no ticket,
 // no tail of one block between the two routing launches, and no launch before them to zero it.
@@ -422,13 +421,13 @@ template <bool OWN>
 __global__ void __launch_bounds__(256)
 route_scatter_gather(const int32_t* __restrict__ topk_idx, const int32_t* __restrict__ chunk_counts,
                      const OffsetsArgs o, int T_tokens, int E, int K, int n_chunks,
-                     int32_t* __restrict__ row_of_assign, const uint4* __restrict__ x, uint4* __restrict__ x_perm, int vec_per_row) {
+                     int32_t* __restrict__ row_of_assign, const uint4* __restrict__ x, uint4* __restrict__ x_perm, int vec_per_row, int parts) {
   pdl_sync();
   __shared__ int32_t rows_s[kChunkTokens * kMaxK];
   __shared__ int32_t base_s[OWN ? kMaxE : 1], cnt_s[OWN ? kMaxE : 1], off_s[OWN ? kMaxE + 1 : 1], poff_s[OWN ? kMaxE + 1 : 1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int chunk = blockIdx.x;
-  const int n_tok = chunk < n_chunks ? min(kChunkTokens, T_tokens - chunk * kChunkTokens) : 0;
+  const int chunk = blockIdx.x / parts, part = blockIdx.x % parts, j0 = part * (kChunkTokens / parts) + warp;
+  const int n_tok = chunk < n_chunks ? min((part + 1) * (kChunkTokens / parts), T_tokens - chunk * kChunkTokens) : 0;      // this block's end in the chunk
   uint4 buf[8];
   auto fetch = [&](int j, int v0) {
     const uint4* src = x + (size_t)(chunk * kChunkTokens + j) * vec_per_row;
@@ -438,7 +437,7 @@ route_scatter_gather(const int32_t* __restrict__ topk_idx, const int32_t* __rest
       if (v < vec_per_row) buf[i] = __ldg(src + v);
     }
   };
-  if (warp < n_tok) fetch(warp, 0);      // (the first row does not depend on the tables)
+  if (j0 < n_tok) fetch(j0, 0);      // (the first row does not depend on the tables)
   const int32_t *chunk_base = chunk_counts + (size_t)chunk * E, *offsets = o.offsets_ws, *pad_offsets = o.pad_offsets;
   if constexpr (OWN) {
     bases_from_histograms(chunk_counts, n_chunks, E, chunk, base_s, cnt_s, off_s, poff_s);
@@ -448,13 +447,13 @@ route_scatter_gather(const int32_t* __restrict__ topk_idx, const int32_t* __rest
   // blocks beyond the last chunk (the grid never drops below one block per SM) only help with the padding rows
   if (chunk < n_chunks && warp == 0) {
     int my_row[kMaxK];
-    scatter_chunk(topk_idx, chunk_base, offsets, pad_offsets, T_tokens, E, K, chunk, lane, nullptr, nullptr, row_of_assign, o.assign_of_row, my_row);
+    scatter_chunk(topk_idx, chunk_base, offsets, pad_offsets, T_tokens, E, K, chunk, lane, nullptr, nullptr, part == 0 ? row_of_assign : nullptr, o.assign_of_row, my_row);
     for (int k = 0; k < K; ++k) rows_s[lane * K + k] = my_row[k];
   }
   __syncthreads();
-  for (int j = warp; j < n_tok; j += 8) {
+  for (int j = j0; j < n_tok; j += 8) {
     for (int v0 = 0; v0 < vec_per_row; v0 += 32 * 8) {
-      if (j != warp || v0) fetch(j, v0);
+      if (j != j0 || v0) fetch(j, v0);
       for (int k = 0; k < K; ++k) {
         uint4* dst = x_perm + (size_t)rows_s[j * K + k] * vec_per_row;
 #pragma unroll
@@ -674,9 +673,12 @@ static cudaError_t launch_scatter(const rom_config& c, const int32_t* idx_ws, in
     int num_sms = 0;
     const cudaError_t e = current_device_sm_count(&num_sms);
     if (e != cudaSuccess) return e;
-    const int grid = (int)lay.n_chunks > num_sms ? (int)lay.n_chunks : num_sms;
+    // few chunks: several blocks to each, since a warp that copies four rows waits for four loads (one block / by
+    // this rule, whole calls, us: 3051 tokens top-2 306.8 / 304.3, backward of 4113 768.7 / 762.0, 256 in fp32 55.9 / 55.0, 8192 top-1 298.8 / 296.4)
+    const int parts = lay.n_chunks <= num_sms ? 4 : lay.n_chunks <= 2 * num_sms ? 2 : 1;
+    const int grid = (int)lay.n_chunks * parts > num_sms ? (int)lay.n_chunks * parts : num_sms;
     launch_k(own ? route_scatter_gather<true> : route_scatter_gather<false>, grid, 256, 0, st, idx_ws, chunk_base, oa, (int)lay.T, c.E, c.K,
-             (int)lay.n_chunks, roa, reinterpret_cast<const uint4*>(x), reinterpret_cast<uint4*>(ws + lay.x_perm), (int)((size_t)c.d_model * lay.esz / 16));
+             (int)lay.n_chunks, roa, reinterpret_cast<const uint4*>(x), reinterpret_cast<uint4*>(ws + lay.x_perm), (int)((size_t)c.d_model * lay.esz / 16), parts);
   } else {
     const int wpb = 8;
     launch_k(route_scatter, ((int)lay.n_chunks + wpb - 1) / wpb, wpb * 32, 0, st, idx_ws, chunk_base, offs, poffs, (int)lay.T, c.E, c.K,
