@@ -287,7 +287,7 @@ inline bool scan_sums_gate(const rom_config& c) { return c.dtype == ROM_BF16 && 
 // y_rows[t*K + k].
 // gate_activated: z already holds SiLU of the gate pre-activation (the producer applied it).
 // chunk_ws == nullptr: one pass per sequence.  Otherwise a long sequence with too few channels to fill the GPU is cut into chunks scanned in
-// parallel in two launches (scan_warp_chunks, scan_f32_chunks or scan_chunks of them, by the kernel); chunk_ws holds scan_ws_floats() floats.
+// parallel in two launches, or by forms that take the whole sequence in one (scan_warp_chunks, scan_f32_chunks or scan_chunks of them, by the kernel); chunk_ws holds scan_ws_floats() floats.
 // delta: [B, L, d_inner], fp32 when delta_fp32, else in the storage dtype.
 cudaError_t launch_scan(const rom_config& c, const void* u, const void* delta, bool delta_fp32, const float* A, const float* Bm,
                         const float* Cm, const float* D, const void* z, int ldz, const int32_t* z_row, const float* h0,

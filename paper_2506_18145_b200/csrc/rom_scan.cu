@@ -3,7 +3,7 @@
 // order (the routing decision of the Gate/Conv projections is reused for Out Proj, Section 4.2).
 //
 // This is the kernel of fp32 storage (with rom_scan_f32.cu where that is the faster one: f32_one_launch), of the scalar-decay block, and of
-// a few bf16 channels without a workspace; bf16 otherwise runs rom_scan_warp.cu.  The launch logic of all of them (chunks, chain, checkpoints) is here.
+// a few bf16 channels without a workspace; bf16 otherwise runs rom_scan_warp.cu or rom_scan_ring.cu.  The launch logic of all of them (chunks, chain, checkpoints) is here.
 //
 // State and arithmetic are fp32.  The recurrence is sequential in t, so the parallelism is
 // (sequence, channel, state).  One thread owns NS of the 16 states of NC adjacent channels
@@ -648,8 +648,8 @@ cudaError_t launch_scan(const rom_config& c, const void* u, const void* delta, b
   const cudaError_t e = current_device_sm_count(&num_sms);
   if (e != cudaSuccess) return e;
   // Few long sequences and no workspace for the chunked scan: the one-pass low-occupancy kernel (every exponential once;
-  // 0.74 ms against 1.04 ms for one 16384-step sequence of 4096 channels).  With a workspace the two chunked launches
-  // below are faster (0.63 ms there, 0.60 in the layer), so they stay the path of the layer.
+  // 0.74 ms against 1.04 ms for one 16384-step sequence of 4096 channels).  With a workspace the forms
+  // below are faster (0.55 ms there, 0.53 in the layer), so they are the path of the layer.
   if (chunk_ws == nullptr && !scalar_A && ckpt == nullptr && scan_seq_applicable(c, u, delta, delta_fp32, Bm, Cm, z, ldz, z_row, y_rows, gate_activated, num_sms))
     return launch_scan_seq(c, u, static_cast<const float*>(delta), A, Bm, Cm, D, z, ldz, h0, y, h_last, st);
   const ScanArgs a{u, delta, A, Bm, Cm, D, z, ldz, z_row, h0, y, h_last, y_rows, K, c.L, c.d_inner, c.L, 1, c.L, nullptr, gate_activated ? 1 : 0, 0,
