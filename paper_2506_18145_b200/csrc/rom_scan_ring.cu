@@ -9,7 +9,7 @@
 // columns a warp; no matrix instruction runs).  The state then comes from the warp before, P h + E goes on to the next warp at once, and
 // one multiply-add an update brings the outputs up to date; nothing of that depends on the step before.  (A state that is infinite stays so step
 // by step; where the decays of a tile multiply to zero it is NaN from the next tile on, as from the next chunk on in the chunked form.)
-// Measured in the layer: 4 x 2048 steps of 2048 channels 170 -> 152 us, 16384 of 4096 593 -> 545; as rom_scan 3 x 1017 of 3072 95 -> 82.  What
+// Measured in the layer: 4 x 2048 steps of 2048 channels 164 -> 147 us, 16384 of 4096 593 -> 531; as rom_scan 3 x 1017 of 3072 95 -> 82.  What
 // bounds it: issue (9.8 instructions an update at up to 69 %), the fp32 pipe (nine operations of an update) and latency: twelve warps an SM.
 // Tried (us of a layer of 4 x 2048 steps of 2048 channels; this form 300, in chunks 317): decays and inputs both in tensor memory with eight
 // warps of 255 registers (seven operations, but two warps a scheduler) 309, that with the second sweep beside the next tile's first 352;
