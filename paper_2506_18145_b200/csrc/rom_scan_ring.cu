@@ -7,8 +7,9 @@
 // 4 states of 4 adjacent channels, as in rom_scan_warp.cu) and keeps what a state before the tile would add to the outputs, C times the
 // running product of the decays: 16 values a lane and step, which registers cannot hold for eight steps.  They go to tensor memory (128
 // columns a warp; no matrix instruction runs).  The state then comes from the warp before, P h + E goes on to the next warp at once, and
-// one multiply-add an update brings the outputs up to date; nothing of that depends on the step before.  (A state that is infinite stays so step
-// by step; where the decays of a tile multiply to zero it is NaN from the next tile on, as from the next chunk on in the chunked form.)
+// one multiply-add an update brings the outputs up to date; nothing of that depends on the step before.  A tile that a state or a C
+// that is not finite meets is run again step by step: where its decays multiply to zero, none of them zero, an infinite state stays infinite
+// (one vote a tile: 4 x 2048 steps of 2048 channels 296.9 -> 297.9 us in the layer, 16384 of 4096 1374 -> 1379).
 // Measured in the layer: 4 x 2048 steps of 2048 channels 164 -> 147 us, 16384 of 4096 593 -> 531; as rom_scan 3 x 1017 of 3072 95 -> 82.  What
 // bounds it: issue (9.8 instructions an update at up to 69 %), the fp32 pipe (nine operations of an update) and latency: twelve warps an SM.
 // Tried (us of a layer of 4 x 2048 steps of 2048 channels; this form 300, in chunks 317): decays and inputs both in tensor memory with eight
@@ -213,7 +214,8 @@ scan_ring_kernel(const ScanArgs p) {
       }
     }
     if (tile + W < NT) fetch(t0 + W * CK);
-    float2 h[8];
+    const float4 cq = reinterpret_cast<const float4*>(s.c)[lane];
+    float2 h[8], nf = make_float2(fmaf(cq.x, 0.0f, cq.y * 0.0f), fmaf(cq.z, 0.0f, cq.w * 0.0f));      // NaN: a value of the tile that is not finite
     // ---- the state before the tile arrives, the one behind it leaves
     if (tile > 0) bar_sync(warp);
 #pragma unroll
@@ -222,7 +224,38 @@ scan_ring_kernel(const ScanArgs p) {
       h[j] = make_float2(x.x, y.x); h[2 + j] = make_float2(x.y, y.y); h[4 + j] = make_float2(x.z, y.z); h[6 + j] = make_float2(x.w, y.w);
     }
 #pragma unroll
-    for (int k = 0; k < 8; ++k) E[k] = __ffma2_rn(P[k], h[k], E[k]);
+    for (int k = 0; k < 8; ++k) { E[k] = __ffma2_rn(P[k], h[k], E[k]); nf = __ffma2_rn(E[k], dup(0.0f), nf); }
+    // a state or a C that is not finite: products formed ahead of the state it meets are not what the steps give (0 where the decays
+    // underflow together and none of them alone, against an infinite state): the tile again, step by step
+    const bool stepwise = __any_sync(0xffffffffu, !(nf.x + nf.y == 0.0f));
+    if (stepwise) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) E[k] = h[k];
+#pragma unroll 1
+      for (int r = 0; r < CK; ++r) {
+        const float4 d4 = s.dl[r][cg ^ r], u4 = s.u[r][cg ^ r], b4 = s.b[r][q], c4 = s.c[r][q];
+        const float2 dl[2] = {make_float2(d4.x, d4.y), make_float2(d4.z, d4.w)}, uu[2] = {make_float2(u4.x, u4.y), make_float2(u4.z, u4.w)};
+        const float bb[4] = {b4.x, b4.y, b4.z, b4.w}, cc[4] = {c4.x, c4.y, c4.z, c4.w};
+        float2 acc[2];
+#pragma unroll
+        for (int n = 0; n < 4; ++n)
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const int k = 2 * n + j;
+            const float2 x = __fmul2_rn(dl[j], a2[k]);
+            const float2 a = make_float2(ex2_ftz(x.x), ex2_ftz(x.y));
+            const float2 uB = __fmul2_rn(uu[j], dup(bb[n]));
+            if (ZOH) {
+              const float2 w = __fmul2_rn(uB, kin[k]);
+              E[k] = __ffma2_rn(a, __ffma2_rn(w, dup(-1.0f), E[k]), w);
+            } else {
+              E[k] = __ffma2_rn(a, E[k], uB);
+            }
+            acc[j] = n == 0 ? __fmul2_rn(dup(cc[n]), E[k]) : __ffma2_rn(dup(cc[n]), E[k], acc[j]);
+          }
+        s.y[r][ysw(lane, r)] = make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y);
+      }
+    }
     {
       const float4 e[4] = {make_float4(E[0].x, E[2].x, E[4].x, E[6].x), make_float4(E[0].y, E[2].y, E[4].y, E[6].y),
                            make_float4(E[1].x, E[3].x, E[5].x, E[7].x), make_float4(E[1].y, E[3].y, E[5].y, E[7].y)};
@@ -245,8 +278,8 @@ scan_ring_kernel(const ScanArgs p) {
       }
     }
     // ---- what the state before the tile adds to the outputs
-    {
-      tm_store_wait();
+    tm_store_wait();
+    if (!stepwise) {
       float v[2][32];
       tm_load32(tm, v[0]);
 #pragma unroll

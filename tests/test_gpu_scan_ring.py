@@ -1,10 +1,11 @@
 """The one-launch bf16 scan against the CPU oracle: sequences around the eight steps of a tile and the twelve warps that take tiles in turn,
 one and two rounds of blocks, every gate / skip / initial state combination; in the layer with one to three Gate rows a token, and with the
-checkpoints of the backward pass."""
+checkpoints of the backward pass.  And values that are not finite: what they give step by step."""
 import pytest
+import torch
 
 from paper_2506_18145_b200 import binding as rb
-from rom_testlib import TOL, assert_close
+from rom_testlib import TOL, assert_close, launched_kernels
 from test_gpu_backward import bshape, run_layer_backward
 from test_gpu_parity import check_layer, run_scan, small_shape
 
@@ -35,3 +36,57 @@ def test_layer_forward_scan_ring(K):
 @pytest.mark.parametrize("disc_mode", [0, 1])
 def test_layer_backward_scan_ring(L, disc_mode):
     run_layer_backward(bshape(B=1, L=L, d_model=64, d_inner=4096, K=1), disc_mode=disc_mode)
+
+
+def ring_inputs(B, L, De, delta, A, disc_mode):
+    """Inputs of ones, an initial state of ones; the call that scans them, and y and the final state that it writes."""
+    one = lambda *shape: torch.ones(*shape, device="cuda")      # noqa: E731
+    q = dict(u=one(B, L, De).bfloat16(), delta=one(B, L, De) * delta, A=-one(De, 16) * A, Bm=one(B, L, 16), Cm=one(B, L, 16), D=one(De), h0=one(B, De, 16))
+    y, h_last = torch.empty_like(q["u"]), one(B, De, 16)
+    cfg = rb.make_config(B, L, 64, De, 16, 4, 16, 1, 1, "bf16", 0, disc_mode)
+    ws = torch.empty(rb.scan_workspace_size(cfg), dtype=torch.uint8, device="cuda")
+
+    def call():
+        rb.rom_scan(cfg, q["u"], q["delta"], q["A"], q["Bm"], q["Cm"], q["D"], None, q["h0"], y, h_last, ws)
+    call()
+    assert any("scan_ring_kernel" in n for n in launched_kernels(call))
+    return q, call, y, h_last
+
+
+@pytest.mark.parametrize("disc_mode", [0, 1])
+@pytest.mark.parametrize("L,De", [(160, 64), (203, 192)])
+def test_scan_ring_infinite_state_stays_infinite(L, De, disc_mode):
+    # every decay is above zero, their product over a tile (exp(-15)^8) is not: step by step the state is infinite from the first step on
+    q, call, y, h_last = ring_inputs(1, L, De, 1.0, 15.0, disc_mode)
+    c_bad = 37
+    q["h0"][0, c_bad] = float("inf")
+    call()
+    torch.cuda.synchronize()
+    rest = [c for c in range(De) if c != c_bad]
+    assert torch.isposinf(y[0, :, c_bad]).all() and torch.isposinf(h_last[0, c_bad]).all()
+    assert torch.isfinite(y[:, :, rest]).all() and torch.isfinite(h_last[:, rest]).all()
+
+
+def test_scan_ring_state_that_becomes_infinite():
+    # (with B-bar = Delta B: the zero-order hold takes the input from the state, infinite from infinite)
+    L, t_bad, c_bad = 203, 101, 5
+    q, call, y, h_last = ring_inputs(1, L, 64, 1.0, 15.0, 1)
+    q["u"][0, t_bad, c_bad] = float("inf")
+    call()
+    torch.cuda.synchronize()
+    rest = [c for c in range(64) if c != c_bad]
+    assert torch.isposinf(y[0, t_bad:, c_bad]).all() and torch.isposinf(h_last[0, c_bad]).all()
+    assert torch.isfinite(y[0, :t_bad]).all() and torch.isfinite(y[:, :, rest]).all()
+
+
+@pytest.mark.parametrize("disc_mode", [0, 1])
+def test_scan_ring_infinite_output_weight(disc_mode):
+    # no input in the tile, so that its outputs come from the state before it alone: infinite where C is
+    L, t_bad = 203, 101
+    q, call, y, h_last = ring_inputs(1, L, 64, 0.1, 0.5, disc_mode)
+    q["u"][0, 96:104] = 0
+    q["Cm"][0, t_bad, 7] = float("inf")
+    call()
+    torch.cuda.synchronize()
+    assert torch.isposinf(y[0, t_bad]).all()
+    assert torch.isfinite(y[0, [t for t in range(L) if t != t_bad]]).all() and torch.isfinite(h_last).all()
