@@ -78,7 +78,6 @@ template <typename TD, bool ZOH, bool CKPT, bool SLOTS>
 __global__ void __launch_bounds__(W * 32, 1)
 scan_ring_kernel(const ScanArgs p) {
   pdl_wait();
-  pdl_trigger();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   RingSmem& sm = *reinterpret_cast<RingSmem*>(smem_raw);
   const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
@@ -119,6 +118,7 @@ scan_ring_kernel(const ScanArgs p) {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  pdl_trigger();      // (only now: the product that follows takes its tensor memory before it waits for this kernel)
   const uint32_t tm = sm.tmem + ((uint32_t)(warp & 3) << 21) + (uint32_t)(warp >> 2) * 128;
 
   // ---- loader / output role: step lt of every tile, channels lc .. lc+7
