@@ -214,6 +214,7 @@ scan_ring_kernel(const ScanArgs p) {
       }
     }
     if (tile + W < NT) fetch(t0 + W * CK);
+    __syncwarp();                 // (the lanes part in a last tile cut short; the barrier and the waits below take the whole warp)
     const float4 cq = reinterpret_cast<const float4*>(s.c)[lane];
     float2 h[8], nf = make_float2(fmaf(cq.x, 0.0f, cq.y * 0.0f), fmaf(cq.z, 0.0f, cq.w * 0.0f));      // NaN: a value of the tile that is not finite
     // ---- the state before the tile arrives, the one behind it leaves

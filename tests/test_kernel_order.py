@@ -26,3 +26,18 @@ def test_tensor_memory_is_allocated_before_the_successor_comes_in(path):
         let_in = re.search(r"pdl_trigger\(\)|pdl_sync\(\)", body)
         if alloc >= 0 and let_in:
             assert alloc < let_in.start()
+
+
+# bar.sync, bar.arrive and the tensor-memory instructions (all of the .aligned kind) take a whole warp, converged: after a branch by lane the
+# warp is brought together by name.
+@pytest.mark.parametrize("before,after", [
+    (r"cur_z\.load", r"bar_sync\(warp\)"),                    # gate rows and the next tile's operands, up to the hand-over
+    (r"fetch_rows\(t0\)", r"tm_store16\("),                   # rows' indices, up to the first sweep
+    (r"V16<bf16>::store", r"tcgen05\.dealloc"),               # outputs of the last step, up to the end
+])
+def test_lanes_of_the_one_launch_scan_meet_before_aligned_instructions(before, after):
+    body, = kernels(os.path.join(rbuild.CSRC, "rom_scan_ring.cu"))
+    for m in re.finditer(before, body):
+        end = re.search(after, body[m.end():])
+        if end:
+            assert "__syncwarp();" in body[m.end():m.end() + end.start()]
