@@ -36,11 +36,6 @@ __device__ __forceinline__ void epi_store_scalar(const Epilogue& ep, int m, int 
       else if (n < ep.R + ep.N) ep.Bm[(size_t)m * ep.N + (n - ep.R)] = v;
       else ep.Cm[(size_t)m * ep.N + (n - ep.R - ep.N)] = v;
       break;
-    case EPI_OUTPROJ: {      // (fp32, top-1: no pass for the combine)
-      const int t = __ldg(ep.row_token + m);
-      if (t >= 0) reinterpret_cast<T*>(ep.C)[(size_t)t * ep.ldc + n] = from_f32<T>(fmaf(__ldg(ep.row_scale + t), v, 0.0f));
-      break;
-    }
     case EPI_F32:
       reinterpret_cast<float*>(ep.C)[(size_t)m * ep.ldc + n] = v;
       break;
@@ -126,7 +121,10 @@ gemm_simt(const T* __restrict__ A, int lda, const T* __restrict__ Bw, int ldb, i
 //     times the blocks' worth of threads in flight and a quarter of the serial steps (256 rows x 1024 columns x 256: the 64 x 64
 //     register-staged kernel took 28 us, waiting for one 16-wide stage after another).  <32, 32, 4, 4, 8, 128>, <16, 16, 2, 4, 8, 128>: see
 //     launch_gemm_simt.
-template <int BM, int BN, int TM, int TN, int KS, int BKF>
+// TO_TOKENS (EPI_OUTPROJ; top-1): a row leaves, times its gate, at its token's position (no pass for the combine: 256 tokens of 256 57.0 -> 54.9 us
+// a layer).  An instance of its own, its rows' tokens and gates read ahead of the stores: as one more output op of the stores above it
+// takes every product in 128 x 128 tiles a quarter longer (In Proj of 4000 tokens of 512: 288 -> 361 us; the layer 725 -> 804, now 711).
+template <int BM, int BN, int TM, int TN, int KS, int BKF, bool TO_TOKENS>
 __global__ void __launch_bounds__(BM / TM * (BN / TN) * KS)
 gemm_f32(const float* __restrict__ A, int lda, const float* __restrict__ Bw, int ldb, int64_t b_expert_stride, int M_max, int N, int Kd,
          const int32_t* __restrict__ tile_expert, const int32_t* __restrict__ num_m_tiles_dev, const int32_t* __restrict__ assign_of_row, Epilogue ep) {
@@ -203,17 +201,40 @@ gemm_f32(const float* __restrict__ A, int lda, const float* __restrict__ Bw, int
       float v = 0.0f;
 #pragma unroll
       for (int g = 0; g < KS; ++g) v += smf[(g * BM + r) * (BN + 1) + c];
-      if (m0 + r < M && n0 + c < N) epi_store_scalar<float>(ep, m0 + r, n0 + c, v);
+      if (m0 + r >= M || n0 + c >= N) continue;
+      if constexpr (TO_TOKENS) {
+        const int t = __ldg(ep.row_token + m0 + r);
+        if (t >= 0) reinterpret_cast<float*>(ep.C)[(size_t)t * ep.ldc + n0 + c] = fmaf(__ldg(ep.row_scale + t), v, 0.0f);
+      } else {
+        epi_store_scalar<float>(ep, m0 + r, n0 + c, v);
+      }
     }
     return;
   }
+  if constexpr (TO_TOKENS) {
+    int t[TM];
+    float g[TM];
 #pragma unroll
-  for (int i = 0; i < TM; ++i)
+    for (int i = 0; i < TM; ++i) t[i] = m0 + ty + i * TY < M ? __ldg(ep.row_token + m0 + ty + i * TY) : -1;
 #pragma unroll
-    for (int j = 0; j < TN; ++j) {
-      const int m = m0 + ty + i * TY, n = n0 + tx + j * TX;
-      if (m < M && n < N) epi_store_scalar<float>(ep, m, n, acc[i][j]);
+    for (int i = 0; i < TM; ++i) g[i] = t[i] >= 0 ? __ldg(ep.row_scale + t[i]) : 0.0f;
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+      if (t[i] < 0) continue;
+      float* row = reinterpret_cast<float*>(ep.C) + (size_t)t[i] * ep.ldc + n0 + tx;
+#pragma unroll
+      for (int j = 0; j < TN; ++j)
+        if (n0 + tx + j * TX < N) row[j * TX] = fmaf(g[i], acc[i][j], 0.0f);
     }
+  } else {
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < TN; ++j) {
+        const int m = m0 + ty + i * TY, n = n0 + tx + j * TX;
+        if (m < M && n < N) epi_store_scalar<float>(ep, m, n, acc[i][j]);
+      }
+  }
 }
 
 // Few rows, long K (the x Proj of a single-token step): C[M,N] = A[M,Kd] * B[N,Kd]^T with the K dimension split over
@@ -276,7 +297,7 @@ static cudaError_t launch_f32(const float* A, int lda, const float* B, int ldb, 
                               const int32_t* assign_of_row, const Epilogue& ep, cudaStream_t st) {
   constexpr int smem = 3 * (BM_ + BN_) * (BKF + 4) * (int)sizeof(float);
   static_assert(smem >= KS * BM_ * (BN_ + 1) * (int)sizeof(float) || KS == 1, "partial sums reuse the stages");
-  auto kern = gemm_f32<BM_, BN_, TM, TN, KS, BKF>;
+  auto kern = ep.mode == EPI_OUTPROJ ? gemm_f32<BM_, BN_, TM, TN, KS, BKF, true> : gemm_f32<BM_, BN_, TM, TN, KS, BKF, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   launch_k(kern, dim3((M + BM_ - 1) / BM_, (N + BN_ - 1) / BN_), BM_ / TM * (BN_ / TN) * KS, smem, st, A, lda, B, ldb, stride, M, N, Kd, te, nmt, assign_of_row, ep);
