@@ -167,7 +167,7 @@ route_offsets(int32_t* __restrict__ chunk_counts, int n_chunks, int E, const Off
   offsets_from_histograms(chunk_counts, n_chunks, E, o, cnt, off, poff);
 }
 
-// One block = 32 tokens (one routing chunk); warp w computes the logits of experts [8w, 8w+8) for them with
+// One block = 32 tokens (one routing chunk); a warp computes the logits of 8 or 16 experts over its range of d_model for them with
 // fp64 tensor-core MMAs (products of bf16/fp32 inputs are exact in fp64; every expert column is accumulated
 // in the same order, so equal weight rows give bit-equal logits and ties stay ties).  Per 16 elements of
 // d_model a lane reads 4 consecutive elements of one token row per 8-token tile (32-byte sectors, straight
@@ -628,15 +628,22 @@ cudaError_t launch_route_stats(const rom_config& c, const void* x, const void* W
   int32_t* assign_of_row = reinterpret_cast<int32_t*>(ws + lay.assign_of_row);
 
   const bool bf = c.dtype == ROM_BF16;
-  // 8-expert tiles to a warp: 32768 tokens of 2048, 16 experts 131 -> 115 us (fp32 rows take twice the registers: one)
-  const int ntw = bf && c.E > NT8 ? 2 : 1;
-  const int n_wtiles = (c.E + ntw * NT8 - 1) / (ntw * NT8);
+  // 8-expert tiles to a warp: two beyond 296 blocks where the tiles share out evenly, or nearly (from 49 experts on).  us of rom_route, one / two, each
+  // with its best split: 32768 tokens of 2048, 16 experts 125 / 121, 64 542 / 489, 40 295 / 400; fewer blocks only lose warps (1024 tokens
+  // of 2048, 17 experts 37 / 45).  fp32 rows take twice the registers: one.
+  const int blocks = (T + RT - 1) / RT, tiles = (c.E + NT8 - 1) / NT8;
+  const int ntw = bf && blocks > 296 && (tiles == 2 || tiles >= 7) ? 2 : 1;
+  const int n_wtiles = (tiles + ntw - 1) / ntw;
   const int Epad8 = n_wtiles * ntw * NT8;
-  // warps per chunk: one per tile of experts, times a split of d_model that puts more loads in flight: up to 4 ranges, 8 while two blocks of
-  // that size an SM hold all of them (8192 tokens of 1024, 8 experts 18.3 -> 16.3 us), up to 16 when there are too few chunks to fill the GPU (a handful of tokens: latency is all that matters)
-  const int blocks = (T + RT - 1) / RT;
-  int dsplit = blocks < 148 ? 16 : blocks <= 296 ? 8 : 4;
-  while (dsplit > 1 && (n_wtiles * ntw * dsplit > 16 || c.d_model / 16 < 4 * dsplit)) dsplit >>= 1;
+  // warps per chunk: one per tile of experts, times a split of d_model that puts more loads in flight: up to 16 ranges and 16 warps while every
+  // block has an SM to itself (latency is all that matters; 145 to 147 blocks do not get that, 148 do: 32 experts, d_model 1024, 16 / 8 warps,
+  // 4480 tokens 48 / 51, 4640 55 / 52, 4736 48 / 50), up to 8 ranges and ten warps while two blocks an SM hold them all, then 4 and eight.
+  // us by ranges: 6000 tokens of 1024, 8 experts 4: 22.0, 8: 20.3, 16: 27.4; 24 experts 1: 56, 2: 46, 4: 55; 16 in fp32 4: 34, 8: 43; 16384
+  // tokens, 24 experts 1: 72, 2: 85, 4: 100.
+  const bool own_sm = blocks <= 144 || blocks == 148;
+  const int most = own_sm ? 16 : blocks < 148 ? 12 : blocks <= 296 ? 10 : 8;
+  int dsplit = own_sm ? 16 : blocks <= 296 ? 8 : 4;
+  while (dsplit > 1 && (n_wtiles * ntw * dsplit > most || c.d_model / 16 < 4 * dsplit)) dsplit >>= 1;
   const int threads = 32 * n_wtiles * dsplit;
   int32_t* status = reinterpret_cast<int32_t*>(ws + lay.status);
   const bool own = gather_x && route_own_bases(lay);

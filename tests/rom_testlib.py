@@ -42,17 +42,18 @@ def oracle_layer(shape, p, gate_mode=0, disc_mode=0, intermediates=True):
 
 
 def launched_kernels(call):
-    """Mangled names of the kernels that a call launches, from its capture in a graph (the call has run before)."""
+    """(mangled name, threads a block) of the kernels that a call launches, from its capture in a graph (the call has run before)."""
     from cuda.bindings import driver
     graph = torch.cuda.CUDAGraph(keep_graph=True)
     with torch.cuda.graph(graph):
         call()
-    raw, names = graph.raw_cuda_graph(), []
+    raw, kernels = graph.raw_cuda_graph(), []
     nodes = driver.cuGraphGetNodes(raw, driver.cuGraphGetNodes(raw, 0)[2])[1]
     for node in nodes:
         if driver.cuGraphNodeGetType(node)[1] == driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
-            names.append(driver.cuFuncGetName(driver.cuGraphKernelNodeGetParams(node)[1].func)[1].decode())
-    return names
+            p = driver.cuGraphKernelNodeGetParams(node)[1]
+            kernels.append((driver.cuFuncGetName(p.func)[1].decode(), p.blockDimX * p.blockDimY * p.blockDimZ))
+    return kernels
 
 
 class GpuLayer:

@@ -32,7 +32,7 @@ def test_layer_fp32_top1_rows_leave_at_their_tokens(kw, tile):
     s = small_shape(K=1, dtype="f32", **kw)
     check_layer(s, "unit")
     g = GpuLayer(s, synth.make_inputs(s, recipe="unit"))
-    names = launched_kernels(lambda: rb.rom_layer_forward(g.cfg, g.weights, g.dev["x"], g.out, g.idx, g.gates, g.counts, g.ws))
+    names = [n for n, _ in launched_kernels(lambda: rb.rom_layer_forward(g.cfg, g.weights, g.dev["x"], g.out, g.idx, g.gates, g.counts, g.ws))]
     torch.cuda.synchronize()
     gemms = [n for n in names if "gemm_f32" in n]
     assert [n for n in gemms if "Lb1E" in n] == [n for n in gemms if tile + "Lb1E" in n] and sum("Lb1E" in n for n in gemms) == 1
