@@ -549,6 +549,11 @@ bool scan_ring_pays(int B, int De, int L, int nch, bool zoh) {
   return ring <= (zoh ? 1.03 : 1.0) * scan_warp_time(B, De, L, nch) + 1000.0 + (nch < 11 ? 1200.0 * nch : 13000.0);
 }
 
+inline bool disjoint(const void* p, size_t np, const void* q, size_t nq) {
+  const char *a = static_cast<const char*>(p), *b = static_cast<const char*>(q);
+  return a + np <= b || b + nq <= a;
+}
+
 // CKPT: also store the checkpoints of the backward pass.
 template <typename T, typename TD, bool PRECISE, bool CKPT = false>
 cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const float* h0, float* h_last,
@@ -573,7 +578,10 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
     return launch_scan_f32(a, c.B, zoh, CKPT, st);
   }
   if constexpr (!PRECISE) {
-    if (warp_kernel && nch > 1 && scan_ring_pays(c.B, c.d_inner, c.L, nch, zoh)) {
+    // (that form may go over a sequence twice: not with outputs in the place of an input)
+    const size_t n = (size_t)c.B * c.L * c.d_inner;
+    const bool apart = a.y_rows || (disjoint(a.y, n * 2, a.u, n * 2) && disjoint(a.y, n * 2, a.delta, n * sizeof(TD)) && (!a.z || disjoint(a.y, n * 2, a.z, n * 2)));
+    if (warp_kernel && nch > 1 && apart && scan_ring_pays(c.B, c.d_inner, c.L, nch, zoh)) {
       a.h0 = h0; a.h_last = h_last;
       return launch_scan_ring(a, c.B, zoh, sizeof(TD) == 4, CKPT, st);
     }

@@ -4,32 +4,26 @@
 // Few channels fill the SMs only when a sequence is cut along time, and the chunked form (rom_scan_warp.cu) then evaluates nearly every
 // exponential twice: 16 of the special-function unit's cycles a warp-wide update against ten of the fp32 pipe.  Here a block owns 32
 // channels of one sequence, and its twelve warps take tiles of eight steps in turn.  A warp runs its tile from a zero state (a lane holds
-// 4 states of 4 adjacent channels, as in rom_scan_warp.cu) and keeps what a state before the tile would add to the outputs, C times the
+// 4 states of 4 adjacent channels, as in rom_scan_warp.cuh) and keeps what a state before the tile would add to the outputs, C times the
 // running product of the decays: 16 values a lane and step, which registers cannot hold for eight steps.  They go to tensor memory (128
 // columns a warp; no matrix instruction runs).  The state then comes from the warp before, P h + E goes on to the next warp at once, and
-// one multiply-add an update brings the outputs up to date; nothing of that depends on the step before.  A tile that a state or a C
-// that is not finite meets is run again step by step: where its decays multiply to zero, none of them zero, an infinite state stays infinite
-// (one vote a tile: 4 x 2048 steps of 2048 channels 296.9 -> 297.9 us in the layer, 16384 of 4096 1374 -> 1379).
+// one multiply-add an update brings the outputs up to date; nothing of that depends on the step before.
+// Values that are not finite: where the decays of a tile multiply to zero, none of them zero, an infinite state would become NaN, and an
+// infinite C meets the two parts of a state one by one.  A state that is not finite is there to the end: the last tile looks at it, every
+// tile at its C, and a block that has seen one goes over its sequence again step by step.  (Looked at tile by tile the states cost 4 %.)
 // Measured in the layer: 4 x 2048 steps of 2048 channels 164 -> 147 us, 16384 of 4096 593 -> 531; as rom_scan 3 x 1017 of 3072 95 -> 82.  What
 // bounds it: issue (9.8 instructions an update at up to 69 %), the fp32 pipe (nine operations of an update) and latency: twelve warps an SM.
 // Tried (us of a layer of 4 x 2048 steps of 2048 channels; this form 300, in chunks 317): decays and inputs both in tensor memory with eight
 // warps of 255 registers (seven operations, but two warps a scheduler) 309, that with the second sweep beside the next tile's first 352;
 // decays alone and the inputs formed twice, sixteen warps 317; B and C twice in shared memory for the packed pairs 319; Delta and u staged
 // as bf16 307; the outputs from the zero state in tensor memory as well 315; the carry in the layout of the registers 309 (spills).
-#include <type_traits>
-
-#include "rom_scan_args.cuh"
+#include "rom_scan_warp.cuh"
 
 namespace rom {
 namespace {
 
-typedef __nv_bfloat16 bf16;
-constexpr int NST = 16;
-constexpr int CK = kScanCkpt;     // steps per tile
-constexpr int WCH = 32;           // channels per block
-constexpr int W = 12;             // warps per block
+constexpr int W = 12;             // warps per block (of WCH channels)
 constexpr int TM_COLS = 512;      // tensor memory columns (a power of two): 128 for each of a lane quarter's three warps
-constexpr float kLog2e = 1.4426950408889634f;
 
 struct RingTile {
   float4 dl[CK][8], u[CK][8];     // Delta, u of 4 channels; group g of step r sits at g ^ r
@@ -41,7 +35,7 @@ struct RingSmem {
   float4 carry[W][4][32];         // state before the tile of warp w
   float D[WCH];
   uint32_t tmem;
-  int ended;
+  int odd;                        // a state or a C that is not finite has turned up
 };
 
 __device__ __forceinline__ void tm_store16(uint32_t at, const float2 (&a)[8]) {
@@ -72,11 +66,18 @@ __device__ __forceinline__ void tm_load_wait(float (&r)[32]) {
                :: "memory");
 }
 __device__ __forceinline__ void bar_sync(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
+__device__ __forceinline__ void block_sync() { asm volatile("bar.sync %0, %1;" ::"n"(W), "n"(W * 32) : "memory"); }      // (0 .. W - 1: the warps')
 __device__ __forceinline__ void bar_arrive(int id) { asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory"); }
+
+// The block's channels again, step by step, by one warp.  (A function of its own, so that the kernel's registers do not feel it.)
+template <typename TD, bool ZOH, bool CKPT, bool SLOTS>
+__device__ __noinline__ void scan_stepwise(const ScanArgs& p, WarpTile& s) {
+  scan_warp_channels<TD, ZOH, CKPT ? SCAN_FULL_CKPT : SCAN_FULL, SLOTS>(p, s, blockIdx.x * WCH, blockIdx.y, 0);
+}
 
 template <typename TD, bool ZOH, bool CKPT, bool SLOTS>
 __global__ void __launch_bounds__(W * 32, 1)
-scan_ring_kernel(const ScanArgs p) {
+scan_ring_kernel(const __grid_constant__ ScanArgs p) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   RingSmem& sm = *reinterpret_cast<RingSmem*>(smem_raw);
@@ -112,7 +113,7 @@ scan_ring_kernel(const ScanArgs p) {
       }
   }
   if (warp == 0) {
-    if (lane == 0) sm.ended = 0;
+    if (lane == 0) sm.odd = 0;
     sm.D[lane] = p.D ? __ldg(p.D + c_warp + lane) : 0.0f;
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -170,6 +171,11 @@ scan_ring_kernel(const ScanArgs p) {
       cur_u = r_u;
     }
     fetch_rows(t0);
+    {      // (by vote or by lane, as the instance's registers like it: fp32 Delta with the hold 153 us by lane, 142 by vote, 4096 steps of 4096 channels)
+      constexpr bool VOTE = SLOTS || (ZOH && sizeof(TD) == 4);
+      const bool odd = !(fabsf((r_c.x + r_c.y) + (r_c.z + r_c.w)) < __int_as_float(0x7f800000));
+      if (VOTE ? __any_sync(0xffffffffu, odd) : odd) sm.odd = 1;
+    }
     __syncwarp();
     // ---- from a zero state: outputs, what a state before the tile adds to them (C times the running product of the decays, to tensor
     // memory) and what the tile does to it
@@ -215,8 +221,7 @@ scan_ring_kernel(const ScanArgs p) {
     }
     if (tile + W < NT) fetch(t0 + W * CK);
     __syncwarp();                 // (the lanes part in a last tile cut short; the barrier and the waits below take the whole warp)
-    const float4 cq = reinterpret_cast<const float4*>(s.c)[lane];
-    float2 h[8], nf = make_float2(fmaf(cq.x, 0.0f, cq.y * 0.0f), fmaf(cq.z, 0.0f, cq.w * 0.0f));      // NaN: a value of the tile that is not finite
+    float2 h[8];
     // ---- the state before the tile arrives, the one behind it leaves
     if (tile > 0) bar_sync(warp);
 #pragma unroll
@@ -225,38 +230,7 @@ scan_ring_kernel(const ScanArgs p) {
       h[j] = make_float2(x.x, y.x); h[2 + j] = make_float2(x.y, y.y); h[4 + j] = make_float2(x.z, y.z); h[6 + j] = make_float2(x.w, y.w);
     }
 #pragma unroll
-    for (int k = 0; k < 8; ++k) { E[k] = __ffma2_rn(P[k], h[k], E[k]); nf = __ffma2_rn(E[k], dup(0.0f), nf); }
-    // a state or a C that is not finite: products formed ahead of the state it meets are not what the steps give (0 where the decays
-    // underflow together and none of them alone, against an infinite state): the tile again, step by step
-    const bool stepwise = __any_sync(0xffffffffu, !(nf.x + nf.y == 0.0f));
-    if (stepwise) {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) E[k] = h[k];
-#pragma unroll 1
-      for (int r = 0; r < CK; ++r) {
-        const float4 d4 = s.dl[r][cg ^ r], u4 = s.u[r][cg ^ r], b4 = s.b[r][q], c4 = s.c[r][q];
-        const float2 dl[2] = {make_float2(d4.x, d4.y), make_float2(d4.z, d4.w)}, uu[2] = {make_float2(u4.x, u4.y), make_float2(u4.z, u4.w)};
-        const float bb[4] = {b4.x, b4.y, b4.z, b4.w}, cc[4] = {c4.x, c4.y, c4.z, c4.w};
-        float2 acc[2];
-#pragma unroll
-        for (int n = 0; n < 4; ++n)
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            const int k = 2 * n + j;
-            const float2 x = __fmul2_rn(dl[j], a2[k]);
-            const float2 a = make_float2(ex2_ftz(x.x), ex2_ftz(x.y));
-            const float2 uB = __fmul2_rn(uu[j], dup(bb[n]));
-            if (ZOH) {
-              const float2 w = __fmul2_rn(uB, kin[k]);
-              E[k] = __ffma2_rn(a, __ffma2_rn(w, dup(-1.0f), E[k]), w);
-            } else {
-              E[k] = __ffma2_rn(a, E[k], uB);
-            }
-            acc[j] = n == 0 ? __fmul2_rn(dup(cc[n]), E[k]) : __ffma2_rn(dup(cc[n]), E[k], acc[j]);
-          }
-        s.y[r][ysw(lane, r)] = make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y);
-      }
-    }
+    for (int k = 0; k < 8; ++k) E[k] = __ffma2_rn(P[k], h[k], E[k]);
     {
       const float4 e[4] = {make_float4(E[0].x, E[2].x, E[4].x, E[6].x), make_float4(E[0].y, E[2].y, E[4].y, E[6].y),
                            make_float4(E[1].x, E[3].x, E[5].x, E[7].x), make_float4(E[1].y, E[3].y, E[5].y, E[7].y)};
@@ -265,9 +239,14 @@ scan_ring_kernel(const ScanArgs p) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) sm.carry[nx][i][lane] = e[i];
         bar_arrive(nx);
-      } else if (p.h_last) {
+      } else {
+        float nf = 0.0f;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) store4_any(p.h_last + (b * De + c0 + i) * NST + 4 * q, e[i]);
+        for (int i = 0; i < 4; ++i) nf = fmaf(e[i].x, 0.0f, fmaf(e[i].y, 0.0f, fmaf(e[i].z, 0.0f, fmaf(e[i].w, 0.0f, nf))));
+        if (__any_sync(0xffffffffu, !(nf == 0.0f))) sm.odd = 1;
+        else if (p.h_last && !sm.odd)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) store4_any(p.h_last + (b * De + c0 + i) * NST + 4 * q, e[i]);
       }
     }
     if (CKPT) {
@@ -279,8 +258,8 @@ scan_ring_kernel(const ScanArgs p) {
       }
     }
     // ---- what the state before the tile adds to the outputs
-    tm_store_wait();
-    if (!stepwise) {
+    {
+      tm_store_wait();
       float v[2][32];
       tm_load32(tm, v[0]);
 #pragma unroll
@@ -350,14 +329,12 @@ scan_ring_kernel(const ScanArgs p) {
     }
     __syncwarp();
   }
-  // the last warp to end frees the tensor memory (no barrier: all sixteen may be in use between two warps)
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncwarp();
-  int ended = 0;
-  if (lane == 0) { __threadfence_block(); ended = atomicAdd(&sm.ended, 1); }
-  if (__shfl_sync(0xffffffffu, ended, 0) == W - 1) {
+  block_sync();
+  if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sm.tmem), "r"(TM_COLS));
+    if (sm.odd) scan_stepwise<TD, ZOH, CKPT, SLOTS>(p, *reinterpret_cast<WarpTile*>(sm.tile));
   }
 }
 

@@ -53,6 +53,29 @@ def ring_inputs(B, L, De, delta, A, disc_mode):
     return q, call, y, h_last
 
 
+@pytest.mark.parametrize("name", ["u", "z"])
+def test_scan_with_its_output_in_the_place_of_an_input(name):
+    # the one-launch form, which may go over a sequence twice, does not take it
+    B, L, De = 2, 201, 192
+    g = torch.Generator(device="cuda").manual_seed(11)
+    r = lambda *s: torch.randn(*s, device="cuda", generator=g)      # noqa: E731
+    q = dict(u=r(B, L, De).bfloat16(), z=r(B, L, De).bfloat16())
+    delta, A, Bm, Cm = 0.1 * r(B, L, De).abs(), -(0.5 + 15 * r(De, 16).abs()), r(B, L, 16), r(B, L, 16)
+    cfg = rb.make_config(B, L, 64, De, 16, 4, 16, 1, 1, "bf16")
+    ws = torch.empty(rb.scan_workspace_size(cfg), dtype=torch.uint8, device="cuda")
+    y = torch.empty_like(q["u"])
+
+    def call(t):
+        rb.rom_scan(cfg, t["u"], delta, A, Bm, Cm, None, t["z"], None, t.get("y", t[name]), None, ws)
+    call(dict(q, y=y))
+    again = {k: v.clone() for k, v in q.items()}
+    call(again)
+    torch.cuda.synchronize()
+    got = again[name].float()
+    assert (got - y.float()).norm() <= 2e-3 * y.float().norm()      # outputs rounded to bf16 from sums in two orders: an ulp here and there
+    assert [any("scan_ring_kernel" in n for n, _ in launched_kernels(lambda: call(t))) for t in (dict(q, y=y), again)] == [True, False]
+
+
 @pytest.mark.parametrize("disc_mode", [0, 1])
 @pytest.mark.parametrize("L,De", [(160, 64), (203, 192)])
 def test_scan_ring_infinite_state_stays_infinite(L, De, disc_mode):
