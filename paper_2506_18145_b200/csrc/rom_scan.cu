@@ -537,16 +537,18 @@ bool f32_one_launch(int B, int De, int L, int nch, bool zoh, int num_sms) {
   return 1500.0 + (double)align_up((size_t)L, round) * k * (zoh ? (k <= 4 ? 21.2 : 20.0) : (k <= 4 ? 14.7 : 13.2)) <= general;
 }
 
-// Whether the one-launch form of the warp kernel (rom_scan_ring.cu) takes a scan that would be cut into nch chunks: by the time of the two in a
-// model of their measured paces.  One launch: rounds of 148 blocks of 32 channels, 33.3 ns a step (31.2 with B-bar = Delta B), 4.4 us a round
-// and 4.4 once; chunked: scan_warp_chunks' model, which leaves out what grows with the chunks (measured 5 to 33 us above it).  At 95 measured
-// sizes of 32 to 2048 blocks and 100 to 16384 steps it names the faster form but for those where the two differ by less than 3 %.
-// us, chunked / one launch: 128 blocks of 1000 steps 59 / 42, 4096 171 / 147, 16384 618 / 553; 256 of 2048 171 / 151; 288 of 4000 327 / 280;
-// 64 of 16384 335 / 547; 160 of 4096 196 / 285; 512 of 2048 282 / 295.  Delta B: 128 of 16384 597 / 508, 256 of 8192 582 / 515.
+// Whether the one-launch form of the warp kernel (rom_scan_ring.cu) takes a scan that would be cut into nch > 1 chunks (from about 156 steps on): by
+// the time of the two in a model of their measured paces.  One launch: rounds of 148 blocks of 32 channels, 32.3 ns a step and 3.5 us a round
+// (30 and 4.2 with B-bar = Delta B), 5 us (5.4) once.  Chunked: scan_warp_chunks' model, and what that leaves out: 0.49 us (0.47) a chunk for the
+// states that a block chains, 1.7 us (1.55) for every 148 blocks of a launch beyond the first.  At 988 measured sizes of 2 to 896 blocks and
+// 160 to 16000 steps it names the faster form but for six, where the two differ by 2 to 8 %, and some that are nearer.
+// us, chunked / one launch: 2 blocks of 400 steps 22.9 / 19.7, 600 22.8 / 26.9; 48 of 800 25 / 33; 128 of 1000 58 / 40, 16000 603 / 530; 192 of
+// 224 23.7 / 25.1; 256 of 2200 180 / 156; 160 of 4500 219 / 308.  Delta B: 192 of 600 41 / 46, 256 of 600 54 / 47.
 bool scan_ring_pays(int B, int De, int L, int nch, bool zoh) {
-  const long long rounds = ((long long)B * (De / 32) + 147) / 148;
-  const double ring = (double)rounds * ((double)L * (zoh ? 33.3 : 31.2) + 4400.0) + 4400.0;
-  return ring <= (zoh ? 1.03 : 1.0) * scan_warp_time(B, De, L, nch) + 1000.0 + (nch < 11 ? 1200.0 * nch : 13000.0);
+  const double rounds = (double)(((long long)B * (De / 32) + 147) / 148), fill = (double)((long long)B * ((De + 127) / 128) * (nch - 1)) / 148.0 - 1.0;
+  const double more = fill > 0.0 ? fill : 0.0, chunked = scan_warp_time(B, De, L, nch);
+  return zoh ? rounds * (32.3 * L + 3500.0) + 5000.0 <= chunked + 490.0 * nch + 1700.0 * more
+             : rounds * (30.0 * L + 4200.0) + 5400.0 <= chunked + 470.0 * nch + 1550.0 * more;
 }
 
 inline bool disjoint(const void* p, size_t np, const void* q, size_t nq) {

@@ -113,3 +113,23 @@ def test_scan_ring_infinite_output_weight(disc_mode):
     torch.cuda.synchronize()
     assert torch.isposinf(y[0, t_bad]).all()
     assert torch.isfinite(y[0, [t for t in range(L) if t != t_bad]]).all() and torch.isfinite(h_last).all()
+
+
+@pytest.mark.parametrize("B,L,De,disc_mode,ring", [
+    (1, 400, 64, 0, True), (1, 600, 64, 0, False), (1, 800, 512, 1, False), (1, 16000, 2048, 0, False), (1, 2500, 3072, 0, True),
+    (1, 1000, 4096, 0, True), (3, 600, 2048, 1, False), (3, 224, 1600, 0, False), (4, 2048, 2048, 0, True), (3, 1371, 2048, 0, False),
+    (8, 600, 1024, 1, True), (3, 512, 4096, 0, False),
+])
+def test_scan_form(B, L, De, disc_mode, ring):
+    # the faster of the two forms, as measured
+    zeros = lambda *shape: torch.zeros(*shape, device="cuda")      # noqa: E731
+    u, y = zeros(B, L, De).bfloat16(), zeros(B, L, De).bfloat16()
+    cfg = rb.make_config(B, L, 64, De, 16, 4, 16, 1, 1, "bf16", 0, disc_mode)
+    ws = torch.empty(rb.scan_workspace_size(cfg), dtype=torch.uint8, device="cuda")
+    delta, A, Bm = zeros(B, L, De), zeros(De, 16) - 1, zeros(B, L, 16)
+
+    def call():
+        rb.rom_scan(cfg, u, delta, A, Bm, Bm, None, None, None, y, None, ws)
+    call()
+    names = [n for n, _ in launched_kernels(call)]
+    assert ["scan_ring_kernel" in n for n in names] == ([True] if ring else [False, False])
