@@ -2,6 +2,8 @@
 oracle on the same seeded inputs, compare.  (Test infrastructure; not part of the product.)"""
 from __future__ import annotations
 
+import contextlib
+
 import numpy as np
 import torch
 
@@ -54,6 +56,27 @@ def launched_kernels(call):
             p = driver.cuGraphKernelNodeGetParams(node)[1]
             kernels.append((driver.cuFuncGetName(p.func)[1].decode(), p.blockDimX * p.blockDimY * p.blockDimZ))
     return kernels
+
+
+@contextlib.contextmanager
+def recorded(name):
+    """Records the calls of a function of the binding, as callables that make them again."""
+    original, calls = getattr(rb, name), []
+
+    def record(*args, **kw):
+        calls.append(lambda: original(*args, **kw))
+        return original(*args, **kw)
+    setattr(rb, name, record)
+    try:
+        yield calls
+    finally:
+        setattr(rb, name, original)
+
+
+def scan_kernels(call):
+    """Those of a call's kernels that scan: "ring" (one launch), "warp" (one pass over whole sequences, or one of two over chunks) or others."""
+    names = [n for n, _ in launched_kernels(call)]
+    return ["ring" if "scan_ring_kernel" in n else "warp" if "scan_warp_kernel" in n else n for n in names if "scan" in n and "scan_bwd" not in n]
 
 
 class GpuLayer:
