@@ -363,12 +363,13 @@ route_logits_topk(const T* __restrict__ x, const T* __restrict__ W_r, const floa
 
 // Stable rank of the chunk's assignments by warp ballots, then the table entries; called by one full warp.
 // my_row[k] receives the padded row of (token, slot k), -1 past the end.  chunk_base: assignments of every expert before this chunk.
+// write_tables: one block of a chunk writes row_of_assign and assign_of_row, the others only want their rows.
 __device__ __forceinline__ void scatter_chunk(const int32_t* __restrict__ topk_idx, const int32_t* chunk_base,
                                               const int32_t* offsets, const int32_t* pad_offsets,
                                               int T_tokens, int E, int K, int chunk, int lane,
                                               int32_t* __restrict__ perm, int32_t* __restrict__ inv_perm,
                                               int32_t* __restrict__ row_of_assign, int32_t* __restrict__ assign_of_row,
-                                              int (&my_row)[kMaxK]) {
+                                              bool write_tables, int (&my_row)[kMaxK]) {
   const int t = chunk * kChunkTokens + lane;
   int my_e[kMaxK], my_rank[kMaxK];
   for (int k = 0; k < K; ++k) {
@@ -392,7 +393,7 @@ __device__ __forceinline__ void scatter_chunk(const int32_t* __restrict__ topk_i
     const int pr = pad_offsets[e] + within;
     if (perm) perm[r] = a;
     if (inv_perm) inv_perm[a] = r;
-    if (row_of_assign) { row_of_assign[a] = pr; assign_of_row[pr] = a; }
+    if (write_tables) { row_of_assign[a] = pr; assign_of_row[pr] = a; }
     my_row[k] = pr;
   }
 }
@@ -409,7 +410,7 @@ route_scatter(const int32_t* __restrict__ topk_idx, const int32_t* __restrict__ 
   const int chunk = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (chunk >= n_chunks) return;
   int my_row[kMaxK];
-  scatter_chunk(topk_idx, chunk_base + (size_t)chunk * E, offsets, pad_offsets, T_tokens, E, K, chunk, lane, perm, inv_perm, row_of_assign, assign_of_row, my_row);
+  scatter_chunk(topk_idx, chunk_base + (size_t)chunk * E, offsets, pad_offsets, T_tokens, E, K, chunk, lane, perm, inv_perm, row_of_assign, assign_of_row, true, my_row);
 }
 
 // `parts` (1, 2 or 4) blocks of 8 warps per chunk of 32 tokens: warp 0 finds the chunk's table entries (the first block writes them), then every warp
@@ -447,7 +448,7 @@ route_scatter_gather(const int32_t* __restrict__ topk_idx, const int32_t* __rest
   // blocks beyond the last chunk (the grid never drops below one block per SM) only help with the padding rows
   if (chunk < n_chunks && warp == 0) {
     int my_row[kMaxK];
-    scatter_chunk(topk_idx, chunk_base, offsets, pad_offsets, T_tokens, E, K, chunk, lane, nullptr, nullptr, part == 0 ? row_of_assign : nullptr, o.assign_of_row, my_row);
+    scatter_chunk(topk_idx, chunk_base, offsets, pad_offsets, T_tokens, E, K, chunk, lane, nullptr, nullptr, row_of_assign, o.assign_of_row, part == 0, my_row);
     for (int k = 0; k < K; ++k) rows_s[lane * K + k] = my_row[k];
   }
   __syncthreads();

@@ -18,6 +18,7 @@
 // decays alone and the inputs formed twice, sixteen warps 317; B and C twice in shared memory for the packed pairs 319; Delta and u staged
 // as bf16 307; the outputs from the zero state in tensor memory as well 315; the carry in the layout of the registers 309 (spills).
 #include "rom_scan_warp.cuh"
+#include "rom_tc_ptx.cuh"
 
 namespace rom {
 namespace {
@@ -46,25 +47,6 @@ __device__ __forceinline__ void tm_store16(uint32_t at, const float2 (&a)[8]) {
       : "memory");
 }
 __device__ __forceinline__ void tm_store_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tm_load32(uint32_t at, float (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]),
-        "=f"(r[8]), "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15]),
-        "=f"(r[16]), "=f"(r[17]), "=f"(r[18]), "=f"(r[19]), "=f"(r[20]), "=f"(r[21]), "=f"(r[22]), "=f"(r[23]),
-        "=f"(r[24]), "=f"(r[25]), "=f"(r[26]), "=f"(r[27]), "=f"(r[28]), "=f"(r[29]), "=f"(r[30]), "=f"(r[31])
-      : "r"(at));
-}
-__device__ __forceinline__ void tm_load_wait(float (&r)[32]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+f"(r[0]), "+f"(r[1]), "+f"(r[2]), "+f"(r[3]), "+f"(r[4]), "+f"(r[5]), "+f"(r[6]), "+f"(r[7]),
-                 "+f"(r[8]), "+f"(r[9]), "+f"(r[10]), "+f"(r[11]), "+f"(r[12]), "+f"(r[13]), "+f"(r[14]), "+f"(r[15]),
-                 "+f"(r[16]), "+f"(r[17]), "+f"(r[18]), "+f"(r[19]), "+f"(r[20]), "+f"(r[21]), "+f"(r[22]), "+f"(r[23]),
-                 "+f"(r[24]), "+f"(r[25]), "+f"(r[26]), "+f"(r[27]), "+f"(r[28]), "+f"(r[29]), "+f"(r[30]), "+f"(r[31])
-               :: "memory");
-}
 __device__ __forceinline__ void bar_sync(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
 __device__ __forceinline__ void block_sync() { asm volatile("bar.sync %0, %1;" ::"n"(W), "n"(W * 32) : "memory"); }      // (0 .. W - 1: the warps')
 __device__ __forceinline__ void bar_arrive(int id) { asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory"); }
@@ -84,7 +66,7 @@ scan_ring_kernel(const __grid_constant__ ScanArgs p) {
   const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
   RingTile& s = sm.tile[warp];
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(&sm.tmem)), "r"(TM_COLS) : "memory");
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sm.tmem)), "r"(TM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   const int De = p.De, L = p.L;
@@ -116,9 +98,9 @@ scan_ring_kernel(const __grid_constant__ ScanArgs p) {
     if (lane == 0) sm.odd = 0;
     sm.D[lane] = p.D ? __ldg(p.D + c_warp + lane) : 0.0f;
   }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  tc_fence_before();
   __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  tc_fence_after();
   pdl_trigger();      // (only now: the product that follows takes its tensor memory before it waits for this kernel)
   const uint32_t tm = sm.tmem + ((uint32_t)(warp & 3) << 21) + (uint32_t)(warp >> 2) * 128;
 
@@ -260,21 +242,21 @@ scan_ring_kernel(const __grid_constant__ ScanArgs p) {
     // ---- what the state before the tile adds to the outputs
     {
       tm_store_wait();
-      float v[2][32];
-      tm_load32(tm, v[0]);
+      uint32_t v[2][32];
+      tmem_ld32_issue(tm, v[0]);
 #pragma unroll
       for (int r2 = 0; r2 < CK / 2; ++r2) {
-        tm_load_wait(v[r2 & 1]);
-        if (r2 + 1 < CK / 2) tm_load32(tm + 32 * (r2 + 1), v[(r2 + 1) & 1]);
+        tmem_ld_wait(v[r2 & 1]);
+        if (r2 + 1 < CK / 2) tmem_ld32_issue(tm + 32 * (r2 + 1), v[(r2 + 1) & 1]);
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
           const int r = 2 * r2 + i;
           float4 y4 = s.y[r][ysw(lane, r)];
-          const float* vr = v[r2 & 1] + 16 * i;
+          const uint32_t* vr = v[r2 & 1] + 16 * i;
 #pragma unroll
           for (int n = 0; n < 4; ++n) {      // (single: the values of the load take two moves into the pair of a packed sum)
-            y4.x = fmaf(vr[4 * n], h[2 * n].x, y4.x); y4.y = fmaf(vr[4 * n + 1], h[2 * n].y, y4.y);
-            y4.z = fmaf(vr[4 * n + 2], h[2 * n + 1].x, y4.z); y4.w = fmaf(vr[4 * n + 3], h[2 * n + 1].y, y4.w);
+            y4.x = fmaf(__uint_as_float(vr[4 * n]), h[2 * n].x, y4.x); y4.y = fmaf(__uint_as_float(vr[4 * n + 1]), h[2 * n].y, y4.y);
+            y4.z = fmaf(__uint_as_float(vr[4 * n + 2]), h[2 * n + 1].x, y4.z); y4.w = fmaf(__uint_as_float(vr[4 * n + 3]), h[2 * n + 1].y, y4.w);
           }
           s.y[r][ysw(lane, r)] = y4;
         }
@@ -329,10 +311,10 @@ scan_ring_kernel(const __grid_constant__ ScanArgs p) {
     }
     __syncwarp();
   }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  tc_fence_before();
   block_sync();
   if (warp == 0) {
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sm.tmem), "r"(TM_COLS));
     if (sm.odd) scan_stepwise<TD, ZOH, CKPT, SLOTS>(p, *reinterpret_cast<WarpTile*>(sm.tile));
   }
