@@ -659,7 +659,7 @@ cudaError_t launch_scan(const rom_config& c, const void* u, const void* delta, b
   if (e != cudaSuccess) return e;
   // Few long sequences and no workspace for the chunked scan: the one-pass low-occupancy kernel (every exponential once;
   // 0.74 ms against 1.04 ms for one 16384-step sequence of 4096 channels).  With a workspace the forms
-  // below are faster (0.55 ms there, 0.53 in the layer), so they are the path of the layer.
+  // below are faster (0.54 ms there, 0.52 in the layer), so they are the path of the layer.
   if (chunk_ws == nullptr && !scalar_A && ckpt == nullptr && scan_seq_applicable(c, u, delta, delta_fp32, Bm, Cm, z, ldz, z_row, y_rows, gate_activated, num_sms))
     return launch_scan_seq(c, u, static_cast<const float*>(delta), A, Bm, Cm, D, z, ldz, h0, y, h_last, st);
   const ScanArgs a{u, delta, A, Bm, Cm, D, z, ldz, z_row, h0, y, h_last, y_rows, K, c.L, c.d_inner, c.L, 1, c.L, nullptr, gate_activated ? 1 : 0, 0,

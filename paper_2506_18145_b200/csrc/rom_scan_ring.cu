@@ -11,8 +11,9 @@
 // Values that are not finite: where the decays of a tile multiply to zero, none of them zero, an infinite state would become NaN, and an
 // infinite C meets the two parts of a state one by one.  A state that is not finite is there to the end: the last tile looks at it, every
 // tile at its C, and a block that has seen one goes over its sequence again step by step.  (Looked at tile by tile the states cost 4 %.)
-// Measured in the layer: 4 x 2048 steps of 2048 channels 164 -> 147 us, 16384 of 4096 593 -> 531; as rom_scan 3 x 1017 of 3072 95 -> 82.  What
-// bounds it: issue (9.8 instructions an update at up to 69 %), the fp32 pipe (nine operations of an update) and latency: twelve warps an SM.
+// Measured against the chunked form, in the layer: 4 x 2048 steps of 2048 channels 164 -> 146 us, 16384 of 4096 593 -> 524; as rom_scan 3 x 1017 of
+// 3072 95 -> 82.  What bounds it: issue (9.6 instructions an update at up to 72 %), the fp32 pipe (nine operations of an update) and latency: twelve
+// warps an SM.
 // Tried (us of a layer of 4 x 2048 steps of 2048 channels; this form 300, in chunks 317): decays and inputs both in tensor memory with eight
 // warps of 255 registers (seven operations, but two warps a scheduler) 309, that with the second sweep beside the next tile's first 352;
 // decays alone and the inputs formed twice, sixteen warps 317; B and C twice in shared memory for the packed pairs 319; Delta and u staged

@@ -17,7 +17,7 @@
 //     ends up with the sum of step g of the group, adds D u, applies the gate, rounds and stores that one value;
 //   * the loop is software-pipelined by hand over groups of four steps (six stages, see the kernel).
 // Measured on one 16384-step sequence of 4096 channels (fp32 Delta, raw gate): 0.74 ms (the general kernel without a
-// workspace: 1.04 ms; with a workspace, chunked: 0.63 ms).  What binds is not the special-function unit: with every shared-memory load,
+// workspace: 1.04 ms; with a workspace, rom_scan_ring.cu: 0.54 ms).  What binds is not the special-function unit: with every shared-memory load,
 // exponential and shuffle taken out the remaining fp32 / integer stream alone needs 0.48 ms, and two sequences take
 // 1.8 x the time of one, i.e. the fp32 pipes are the limit (a packed fp32 operation occupies them for two cycles:
 // 128 lanes per clock per SM, packed or not, as measured).

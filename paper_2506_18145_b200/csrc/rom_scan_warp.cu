@@ -1,5 +1,5 @@
 // Selective scan for bf16 storage (same arithmetic and arguments as rom_scan.cu): one warp owns 32 channels of one chunk of one
-// sequence, a lane 4 states of 4 adjacent channels.
+// sequence, a lane 4 states of 4 adjacent channels (rom_scan_warp.cuh).
 //
 // What bounds it: per state update one exponential on the special-function unit (16 per clock and SM), six fp32 lane operations
 // (128 per clock and SM) and the bytes that shared memory returns to registers (128 per clock and SM, one copy per lane).  With
