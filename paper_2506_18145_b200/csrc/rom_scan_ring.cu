@@ -10,9 +10,10 @@
 // one multiply-add an update brings the outputs up to date; nothing of that depends on the step before.
 // Values that are not finite: where the decays of a tile multiply to zero, none of them zero, an infinite state would become NaN, and an
 // infinite C meets the two parts of a state one by one.  A state that is not finite is there to the end: the last tile looks at it, every
-// tile at its C, and a block that has seen one goes over its sequence again step by step.  (Looked at tile by tile the states cost 4 %.)
+// tile at its C, and a block that has seen one goes over its sequence again step by step.  (Looked at tile by tile the states cost 4 %.  With a NaN
+// in every sequence 16384 steps of 4096 channels take 2.1 ms; all by one warp a block 3.1.)
 // Measured against the chunked form, in the layer: 4 x 2048 steps of 2048 channels 164 -> 146 us, 16384 of 4096 593 -> 524; as rom_scan 3 x 1017 of
-// 3072 95 -> 82.  What bounds it: issue (9.6 instructions an update at up to 72 %), the fp32 pipe (nine operations of an update) and latency: twelve
+// 3072 95 -> 82.  What bounds it: issue (9.5 instructions an update at up to 72 %), the fp32 pipe (nine operations of an update) and latency: twelve
 // warps an SM.
 // Tried (us of a layer of 4 x 2048 steps of 2048 channels; this form 300, in chunks 317): decays and inputs both in tensor memory with eight
 // warps of 255 registers (seven operations, but two warps a scheduler) 309, that with the second sweep beside the next tile's first 352;
@@ -52,10 +53,42 @@ __device__ __forceinline__ void bar_sync(int id) { asm volatile("bar.sync %0, 64
 __device__ __forceinline__ void block_sync() { asm volatile("bar.sync %0, %1;" ::"n"(W), "n"(W * 32) : "memory"); }      // (0 .. W - 1: the warps')
 __device__ __forceinline__ void bar_arrive(int id) { asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory"); }
 
-// The block's channels again, step by step, by one warp.  (A function of its own, so that the kernel's registers do not feel it.)
+// The block's channels again, step by step, the warps still in turns.  (A function of its own, so that the kernel's registers do not feel it.)
+struct StepSmem {
+  WarpTile tile[W];
+  float4 carry[W][4][32];
+};
+struct TilesInTurns {
+  StepSmem& sm;
+  const int warp, lane;
+  static constexpr int STRIDE = W * CK;
+  __device__ int first() const { return warp * CK; }
+  __device__ void take(float2 (&h)[4][2], int t0) const {
+    if (t0 == 0) return;
+    __syncwarp();
+    bar_sync(warp);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const float4 x = sm.carry[warp][2 * j][lane], y = sm.carry[warp][2 * j + 1][lane];
+      h[0][j] = make_float2(x.x, y.x); h[1][j] = make_float2(x.y, y.y); h[2][j] = make_float2(x.z, y.z); h[3][j] = make_float2(x.w, y.w);
+    }
+  }
+  __device__ void give(const float2 (&h)[4][2], int t0, int L) const {
+    if (t0 + CK >= L) return;
+    const int nx = warp + 1 == W ? 0 : warp + 1;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      sm.carry[nx][2 * j][lane] = make_float4(h[0][j].x, h[1][j].x, h[2][j].x, h[3][j].x);
+      sm.carry[nx][2 * j + 1][lane] = make_float4(h[0][j].y, h[1][j].y, h[2][j].y, h[3][j].y);
+    }
+    bar_arrive(nx);
+  }
+  __device__ bool has_last(int L) const { return (L - 1) / CK % W == warp; }
+};
 template <typename TD, bool ZOH, bool CKPT, bool SLOTS>
-__device__ __noinline__ void scan_stepwise(const ScanArgs& p, WarpTile& s) {
-  scan_warp_channels<TD, ZOH, CKPT ? SCAN_FULL_CKPT : SCAN_FULL, SLOTS>(p, s, blockIdx.x * WCH, blockIdx.y, 0);
+__device__ __noinline__ void scan_stepwise(const ScanArgs& p, StepSmem& sm) {
+  const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
+  scan_warp_channels<TD, ZOH, CKPT ? SCAN_FULL_CKPT : SCAN_FULL, SLOTS>(p, sm.tile[warp], blockIdx.x * WCH, blockIdx.y, 0, TilesInTurns{sm, warp, lane});
 }
 
 template <typename TD, bool ZOH, bool CKPT, bool SLOTS>
@@ -154,8 +187,8 @@ scan_ring_kernel(const __grid_constant__ ScanArgs p) {
       cur_u = r_u;
     }
     fetch_rows(t0);
-    {      // (by vote or by lane, as the instance's registers like it: fp32 Delta with the hold 153 us by lane, 142 by vote, 4096 steps of 4096 channels)
-      constexpr bool VOTE = SLOTS || (ZOH && sizeof(TD) == 4);
+    {      // (by vote or by lane, as the instance's registers like it: fp32 Delta with the hold 153 us by lane, 141 by vote, 4096 steps of 4096 channels)
+      constexpr bool VOTE = ZOH && sizeof(TD) == 4;
       const bool odd = !(fabsf((r_c.x + r_c.y) + (r_c.z + r_c.w)) < __int_as_float(0x7f800000));
       if (VOTE ? __any_sync(0xffffffffu, odd) : odd) sm.odd = 1;
     }
@@ -314,16 +347,20 @@ scan_ring_kernel(const __grid_constant__ ScanArgs p) {
   }
   tc_fence_before();
   block_sync();
+  const bool odd = sm.odd;
   if (warp == 0) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sm.tmem), "r"(TM_COLS));
-    if (sm.odd) scan_stepwise<TD, ZOH, CKPT, SLOTS>(p, *reinterpret_cast<WarpTile*>(sm.tile));
+  }
+  if (odd) {
+    block_sync();      // (everybody has read what lay there)
+    scan_stepwise<TD, ZOH, CKPT, SLOTS>(p, *reinterpret_cast<StepSmem*>(smem_raw));
   }
 }
 
 template <typename TD, bool ZOH, bool CKPT, bool SLOTS>
 cudaError_t launch_one(const ScanArgs& a, int B, cudaStream_t st) {
-  constexpr int smem = (int)sizeof(RingSmem);
+  constexpr int smem = (int)(sizeof(RingSmem) > sizeof(StepSmem) ? sizeof(RingSmem) : sizeof(StepSmem));
   const cudaError_t e = cudaFuncSetAttribute(scan_ring_kernel<TD, ZOH, CKPT, SLOTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   launch_k(a.early != 0, scan_ring_kernel<TD, ZOH, CKPT, SLOTS>, dim3(a.De / WCH, B), W * 32, smem, st, a);

@@ -22,9 +22,19 @@ struct WarpTile {
   float4 y[CK][32];               // partial sums of 4 channels over one lane's states; lane l of step r at ysw(l, r)
 };
 
+// Which tiles of its chunk a warp takes: all of them, the state staying with it.  (rom_scan_ring.cu: warps in turns, which hand it on.)
+struct AllTiles {
+  static constexpr int STRIDE = CK;
+  __device__ int first() const { return 0; }
+  __device__ void take(float2 (&)[4][2], int) const {}
+  __device__ void give(const float2 (&)[4][2], int, int) const {}
+  __device__ bool has_last(int) const { return true; }
+};
+
 // SLOTS: the gate of a token is SiLU of the sum of its K >= 2 rows z_row[t K + k], which are also its output rows (y_rows).
-template <typename TD, bool ZOH, int MODE, bool SLOTS>
-__device__ __forceinline__ void scan_warp_channels(const ScanArgs& p, WarpTile& s, const int c_warp, const int seq, const int chunk) {
+template <typename TD, bool ZOH, int MODE, bool SLOTS, typename Tiles = AllTiles>
+__device__ __forceinline__ void scan_warp_channels(const ScanArgs& p, WarpTile& s, const int c_warp, const int seq, const int chunk, const Tiles& tiles = {}) {
+  constexpr int STRIDE = Tiles::STRIDE;
   constexpr bool FIRST = MODE == SCAN_FIRST || MODE == SCAN_FIRST_CKPT;
   const int lane = threadIdx.x & 31, De = p.De;
   const bool so = MODE == SCAN_STATE || MODE == SCAN_CKPT || (FIRST && chunk != 0);      // this block only produces states
@@ -96,12 +106,12 @@ __device__ __forceinline__ void scan_warp_channels(const ScanArgs& p, WarpTile& 
   if (!so) s.D[lane] = d_skip;
   // ---- loader / output role: step lt of every tile, channels lc .. lc+7
   // (four lanes per row: a load's quarter-warp touches two rows of global memory, not eight)
-  const int lt = lane >> 2, l8 = lane & 3, lc = c_warp + 8 * l8;
+  const int lt = lane >> 2, l8 = lane & 3, lc = c_warp + 8 * l8, t_own = tiles.first();
   const bf16* __restrict__ zp = so ? nullptr : static_cast<const bf16*>(p.z);
-  const TD* dptr = static_cast<const TD*>(p.delta) + (tok0 + lt) * De + lc;
-  const bf16* uptr = static_cast<const bf16*>(p.u) + (tok0 + lt) * De + lc;
-  const float4* bptr = reinterpret_cast<const float4*>(p.Bm + tok0 * NST) + lane;
-  const float4* cptr = reinterpret_cast<const float4*>(p.Cm + tok0 * NST) + lane;
+  const TD* dptr = static_cast<const TD*>(p.delta) + (tok0 + t_own + lt) * De + lc;
+  const bf16* uptr = static_cast<const bf16*>(p.u) + (tok0 + t_own + lt) * De + lc;
+  const float4* bptr = reinterpret_cast<const float4*>(p.Bm + (tok0 + t_own) * NST) + lane;
+  const float4* cptr = reinterpret_cast<const float4*>(p.Cm + (tok0 + t_own) * NST) + lane;
 
   Raw8<TD> r_d;
   Raw8<bf16> r_u, r_z, r_z2, cur_u, cur_z, cur_z2;
@@ -133,12 +143,12 @@ __device__ __forceinline__ void scan_warp_channels(const ScanArgs& p, WarpTile& 
     } else {                       // steps past the end change nothing
       r_d.zero(); r_u.zero();
     }
-    dptr += (size_t)CK * De; uptr += (size_t)CK * De;
+    dptr += (size_t)STRIDE * De; uptr += (size_t)STRIDE * De;
     const bool in = t0 + (lane >> 2) < L;
     r_b = in ? __ldg(bptr) : zero4;
     if (!so) r_c = in ? __ldg(cptr) : zero4;
-    bptr += CK * 4; cptr += CK * 4;
-    if (SLOTS && !so) fetch_rows(t0 + CK);
+    bptr += STRIDE * 4; cptr += STRIDE * 4;
+    if (SLOTS && !so) fetch_rows(t0 + STRIDE);
   };
 
   auto run = [&](auto so_tag) {
@@ -147,9 +157,9 @@ __device__ __forceinline__ void scan_warp_channels(const ScanArgs& p, WarpTile& 
     // from a zero state and with nothing read before the end, the state is carried times -A: one product less an update (16384 steps of
     // 4096 channels 280 -> 272 us for the first launch, 4 x 2048 of 2048 75.4 -> 73.8)
     constexpr bool SCALED = ZOH && SO && !CKPT;
-    if (SLOTS && !SO) fetch_rows(0);
-    fetch(0);
-    for (int t0 = 0; t0 < L; t0 += CK) {
+    if (SLOTS && !SO) fetch_rows(t_own);
+    fetch(t_own);
+    for (int t0 = t_own; t0 < L; t0 += STRIDE) {
       {
         float d[8], uu[8];
         r_d.get(d); r_u.get(uu);
@@ -165,7 +175,8 @@ __device__ __forceinline__ void scan_warp_channels(const ScanArgs& p, WarpTile& 
         if (!SO) { reinterpret_cast<float4*>(s.c)[lane] = r_c; cur_u = r_u; cur_z = r_z; cur_row = r_row; if (SLOTS) { cur_z2 = r_z2; cur_row2 = r_row2; } }
       }
       __syncwarp();
-      if (t0 + CK < L) fetch(t0 + CK);
+      if (t0 + STRIDE < L) fetch(t0 + STRIDE);
+      tiles.take(h, t0);
       if constexpr (CKPT) put_state(p.ckpt + ((size_t)seq * p.nck + (size_t)((t_first + t0) / CK)) * De * NST, std::false_type{});
       // the next step's operands are requested before this step's arithmetic: a load issued behind a step's exponentials waits
       // for all of them in the queue that both share
@@ -201,6 +212,7 @@ __device__ __forceinline__ void scan_warp_channels(const ScanArgs& p, WarpTile& 
         if (SO) { sdel[0] = __fadd2_rn(sdel[0], dl[0]); sdel[1] = __fadd2_rn(sdel[1], dl[1]); }
         else s.y[r][ysw(lane, r)] = make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y);
       }
+      tiles.give(h, t0, L);
       __syncwarp();
       if (!SO) {
         // y = (sum over the four lanes + D u) * gate, rounded, written to the K rows of the token
@@ -263,7 +275,7 @@ __device__ __forceinline__ void scan_warp_channels(const ScanArgs& p, WarpTile& 
   else run(std::false_type{});
 
   const bool chained = SECOND && p.chain_end;
-  if (p.h_last && (!chained || chunk == p.nch - 1)) {
+  if (p.h_last && (!chained || chunk == p.nch - 1) && tiles.has_last(L)) {
     put_state(p.h_last + (chained ? (size_t)seq : sc) * De * NST, std::true_type{});
     if (so && q == 0 && p.sum_delta) *reinterpret_cast<float4*>(p.sum_delta + sc * De + c0) = make_float4(sdel[0].x, sdel[0].y, sdel[1].x, sdel[1].y);
   }
