@@ -538,17 +538,19 @@ bool f32_one_launch(int B, int De, int L, int nch, bool zoh, int num_sms) {
 }
 
 // Whether the one-launch form of the warp kernel (rom_scan_ring.cu) takes a scan that would be cut into nch > 1 chunks (from about 156 steps on): by
-// the time of the two in a model of their measured paces.  One launch: rounds of 148 blocks of 32 channels, 32.3 ns a step and 3.5 us a round
-// (30 and 4.2 with B-bar = Delta B), 5 us (5.4) once.  Chunked: scan_warp_chunks' model, and what that leaves out: 0.49 us (0.47) a chunk for the
-// states that a block chains, 1.7 us (1.55) for every 148 blocks of a launch beyond the first.  At 988 measured sizes of 2 to 896 blocks and
-// 160 to 16000 steps it names the faster form but for six, where the two differ by 2 to 8 %, and some that are nearer.
-// us, chunked / one launch: 2 blocks of 400 steps 22.9 / 19.7, 600 22.8 / 26.9; 48 of 800 25 / 33; 128 of 1000 58 / 40, 16000 603 / 530; 192 of
-// 224 23.7 / 25.1; 256 of 2200 180 / 156; 160 of 4500 219 / 308.  Delta B: 192 of 600 41 / 46, 256 of 600 54 / 47.
-bool scan_ring_pays(int B, int De, int L, int nch, bool zoh) {
+// the time of the two in a model of their measured paces.  One launch: `once`, and for every round of 148 blocks of 32 channels `round` and
+// `step` for each step.  Chunked: scan_warp_chunks' model, and what that leaves out: `chunk` for the states that a block chains, `more` for
+// every 148 blocks of a launch beyond the first.  At 988 measured sizes of rom_scan, 2 to 896 blocks and 160 to 16000 steps, it names the faster
+// form but for six, where the two differ by 2 to 8 %; at 665 sizes of the layer (forward and backward, top-1 to top-3; where the one launch hides
+// behind the dt Proj) but for nine that differ by more than 2 us, at most 8.
+// rom_scan, us, chunked / one launch: 2 blocks of 400 steps 22.9 / 19.7, 600 22.8 / 26.9; 48 of 800 25 / 33; 128 of 1000 58 / 40, 16000 603 / 530; 192
+// of 224 23.7 / 25.1; 256 of 2200 180 / 156; 160 of 4500 219 / 308.  Delta B: 192 of 600 41 / 46, 256 of 600 54 / 47.  Layers: 192 of 300 111.5 / 109.8,
+// 208 of 450 120.3 / 117.1, 208 of 1476 top-3 449 / 459.
+bool scan_ring_pays(int B, int De, int L, int nch, bool zoh, bool in_layer) {
+  struct Pace { double step, round, once, chunk, more; };      // ns
+  const Pace t = !zoh ? Pace{30.0, 4200.0, 5400.0, 470.0, 1550.0} : in_layer ? Pace{34.2, 2600.0, 1900.0, 320.0, 1360.0} : Pace{32.3, 3500.0, 5000.0, 490.0, 1700.0};
   const double rounds = (double)(((long long)B * (De / 32) + 147) / 148), fill = (double)((long long)B * ((De + 127) / 128) * (nch - 1)) / 148.0 - 1.0;
-  const double more = fill > 0.0 ? fill : 0.0, chunked = scan_warp_time(B, De, L, nch);
-  return zoh ? rounds * (32.3 * L + 3500.0) + 5000.0 <= chunked + 490.0 * nch + 1700.0 * more
-             : rounds * (30.0 * L + 4200.0) + 5400.0 <= chunked + 470.0 * nch + 1550.0 * more;
+  return rounds * (t.step * L + t.round) + t.once <= scan_warp_time(B, De, L, nch) + t.chunk * nch + t.more * (fill > 0.0 ? fill : 0.0);
 }
 
 inline bool disjoint(const void* p, size_t np, const void* q, size_t nq) {
@@ -583,7 +585,7 @@ cudaError_t launch_scan_t(const rom_config& c, ScanArgs a, const float* A, const
     // (that form may go over a sequence twice: not with outputs in the place of an input)
     const size_t n = (size_t)c.B * c.L * c.d_inner;
     const bool apart = a.y_rows || (disjoint(a.y, n * 2, a.u, n * 2) && disjoint(a.y, n * 2, a.delta, n * sizeof(TD)) && (!a.z || disjoint(a.y, n * 2, a.z, n * 2)));
-    if (warp_kernel && nch > 1 && apart && scan_ring_pays(c.B, c.d_inner, c.L, nch, zoh)) {
+    if (warp_kernel && nch > 1 && apart && scan_ring_pays(c.B, c.d_inner, c.L, nch, zoh, sizeof(TD) == 2)) {
       a.h0 = h0; a.h_last = h_last;
       return launch_scan_ring(a, c.B, zoh, sizeof(TD) == 4, CKPT, st);
     }

@@ -5,7 +5,8 @@ import pytest
 import torch
 
 from paper_2506_18145_b200 import binding as rb
-from rom_testlib import TOL, assert_close, recorded, scan_kernels
+from paper_2506_18145_b200 import synth
+from rom_testlib import TOL, GpuLayer, assert_close, recorded, scan_kernels
 from test_gpu_backward import bshape, run_layer_backward
 from test_gpu_parity import check_layer, run_scan, small_shape
 
@@ -141,4 +142,15 @@ def test_scan_form(B, L, De, disc_mode, ring):
     def call():
         rb.rom_scan(cfg, u, delta, A, Bm, Bm, None, None, None, y, None, ws)
     call()
+    assert scan_kernels(call) == (["ring"] if ring else ["warp", "warp"])
+
+
+@pytest.mark.parametrize("B,L,De,K,ring", [(3, 300, 2048, 1, True), (3, 300, 2048, 2, True), (3, 600, 2048, 1, False), (2, 600, 192, 1, False),
+                                           (2, 500, 192, 1, True), (4, 1476, 1664, 3, False)])
+def test_layer_scan_form(B, L, De, K, ring):
+    # (in the layer the line lies a little elsewhere)
+    s = small_shape(B=B, L=L, d_model=64, d_inner=De, E=4, K=K)
+    g = GpuLayer(s, synth.make_inputs(s, recipe="unit"))
+    g.forward()
+    call = lambda: rb.rom_layer_forward(g.cfg, g.weights, g.dev["x"], g.out, g.idx, g.gates, g.counts, g.ws)      # noqa: E731
     assert scan_kernels(call) == (["ring"] if ring else ["warp", "warp"])
